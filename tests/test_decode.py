@@ -83,3 +83,25 @@ def test_decode_step_rejects_bad_arguments():
     rc = libssd.lib().ssd_decode_step(ctypes.byref(shape), p(inp["x"]), p(inp["dt"]), p(inp["A"]), p(inp["Bm"]),
                                       p(inp["Cm"]), p(inp["D"]), p(h), p(inp["x"]), None)
     assert rc == libssd.SSD_EINVAL
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("N", [64, 128])
+@pytest.mark.parametrize("B,H,P", [(1, 4, 64), (5, 64, 64), (2, 3, 6), (2, 3, 5), (3, 148, 40)])
+def test_decode_step_rows_per_warp(B, H, P, N, dtype):
+    """Eight, two and one rows per warp (many rows; few or P even; P odd), a last CTA that is partly idle."""
+    from tests.parity_util import TOL, relerr
+
+    cfg = CONFIGS[0].scaled(dtype=dtype, B=B, L=1, H=H, P=P, N=N, h0_std=0.1)
+    inp = make_inputs(cfg, "cuda", seed=7)
+    d = to_f64_numpy(inp)
+    h = inp["h0"].clone()
+    y = libssd_decode(inp, h)
+    y_ref, h_ref = orc.decode_step(d["x"][:, 0], d["dt"][:, 0], d["A"], d["Bm"][:, 0], d["Cm"][:, 0], d["D"], d["h0"])
+    assert relerr(y[:, 0], y_ref) <= TOL[dtype] and relerr(h, h_ref) <= 1e-6
+
+
+def libssd_decode(inp, h):
+    from paper_2411_19460_b200 import libssd
+    return libssd.ssd_decode_step(inp["x"], inp["dt"], inp["A"], inp["Bm"], inp["Cm"], inp["D"], h)
