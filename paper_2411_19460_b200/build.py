@@ -1,15 +1,18 @@
 """Compile libssd (hand-written sm_100a CUDA + the C ABI of include/ssd.h) into
-paper_2411_19460_b200/lib/libssd.so with nvcc.  Works without a GPU (cross-compiles)."""
+paper_2411_19460_b200/lib/libssd.so with nvcc, and the CPython binding over it (csrc/binding.cpp) into
+paper_2411_19460_b200/_native.so.  Works without a GPU (cross-compiles)."""
 import concurrent.futures
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT = os.path.join(HERE, "lib", "libssd.so")
+BINDING = os.path.join(HERE, "_native.so")
 OBJ = os.path.join(HERE, "_build")
 
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -30,6 +33,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     deps = srcs + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(CSRC, "*.cuh")) + \
         glob.glob(os.path.join(ROOT, "include", "*.h"))
     if not force and os.path.exists(OUT) and os.path.getmtime(OUT) >= _newest(deps):
+        build_binding(force)
         return OUT
     os.makedirs(OBJ, exist_ok=True)
     os.makedirs(os.path.dirname(OUT), exist_ok=True)
@@ -57,7 +61,31 @@ def build(force: bool = False, verbose: bool = False) -> str:
     if r.returncode != 0:
         raise RuntimeError("link failed:\n" + r.stderr)
     os.replace(tmp, OUT)
+    build_binding(force)
     return OUT
+
+
+def build_binding(force: bool = False) -> str:
+    """The torch-facing marshalling layer; links the library next to it."""
+    src = os.path.join(CSRC, "binding.cpp")
+    deps = [src, os.path.join(ROOT, "include", "ssd.h")]
+    if not force and os.path.exists(BINDING) and os.path.getmtime(BINDING) >= _newest(deps):
+        return BINDING
+    import torch
+    tdir = os.path.dirname(torch.__file__)
+    inc = [os.path.join(tdir, "include"), os.path.join(tdir, "include", "torch", "csrc", "api", "include"),
+           os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include"), sysconfig.get_paths()["include"]]
+    tmp = BINDING + ".tmp.%d" % os.getpid()
+    cmd = ["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-I", os.path.join(ROOT, "include")]
+    for d in inc:
+        cmd += ["-isystem", d]
+    cmd += [src, "-o", tmp, "-L", os.path.dirname(OUT), "-lssd", "-L", os.path.join(tdir, "lib"), "-lc10", "-lc10_cuda", "-ltorch_cpu",
+            "-ltorch_python", "-Wl,-rpath,$ORIGIN/lib"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        raise RuntimeError("g++ failed for the binding:\n" + r.stderr)
+    os.replace(tmp, BINDING)
+    return BINDING
 
 
 if __name__ == "__main__":

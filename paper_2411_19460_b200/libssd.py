@@ -1,5 +1,6 @@
-"""ctypes binding of libssd (include/ssd.h).  Argument marshalling only: every step of the path
-runs in the library's CUDA kernels.  torch is used for device memory and streams, nothing else.
+"""Python binding of libssd (include/ssd.h).  Argument marshalling only: every step of the path
+runs in the library's CUDA kernels.  The calls that launch work go through the native module built from
+csrc/binding.cpp, queries and the rest through ctypes.  torch is used for device memory and streams, nothing else.
 There is no CPU fallback: if the shared library has not been built, loading raises.
 """
 import ctypes
@@ -114,6 +115,20 @@ def lib():
     return _lib
 
 
+_nat = None
+
+
+def _native():
+    """The binding of the calls that run kernels (csrc/binding.cpp): same checks and results as marshalling them here
+    with ctypes, at a fraction of the host time per call."""
+    global _nat
+    if _nat is None:
+        lib()                      # raises where nothing has been built
+        from . import _native as module
+        _nat = module
+    return _nat
+
+
 def _ptr(t):
     return None if t is None else ctypes.c_void_p(t.data_ptr())
 
@@ -197,18 +212,10 @@ def _check_inputs(x, dt, A, Bm, Cm, D):
 def ssd_fwd(x, dt, A, Bm, Cm, D, h0=None, *, chunk, seg=0, flags=0, y=None, h_final=None,
             ws=None, stream=None):
     """y, h_final = SSD forward (Eq. 1).  `seg` only sizes the scratch."""
-    _check_inputs(x, dt, A, Bm, Cm, D)
-    shape = make_shape(x, Bm, chunk, seg, flags)
-    B, L, H, P = x.shape
-    N = Bm.shape[3]
-    y = torch.empty_like(x) if y is None else y
-    h_final = torch.empty(B, H, P, N, dtype=torch.float32, device=x.device) if h_final is None else h_final
-    ws = alloc_workspace(shape, SSD_OP_FWD, x.device) if ws is None else ws
-    rc = lib().ssd_fwd(ctypes.byref(shape), _ptr(x), _ptr(dt), _ptr(A), _ptr(Bm), _ptr(Cm), _ptr(D),
-                       _ptr(h0), _ptr(y), _ptr(h_final), _ptr(ws), ws.numel(), _stream(stream))
-    if rc != SSD_OK:
-        raise SSDError(rc, "ssd_fwd")
-    return y, h_final
+    r = (_nat or _native()).fwd(x, dt, A, Bm, Cm, D, h0, chunk, seg, flags, y, h_final, False, ws, stream)
+    if r.__class__ is int:
+        raise SSDError(r, "ssd_fwd")
+    return r
 
 
 def ssd_fwd_static_ws(x, dt, A, Bm, Cm, D, h0=None, *, chunk, seg=0, flags=0, y, h_final, stream=None):
@@ -229,47 +236,26 @@ def ssd_fwd_segmented(x, dt, A, Bm, Cm, D, h0=None, *, chunk, seg, flags=0, y=No
                       boundary=None, ws=None, stream=None):
     """y, h_final, boundary = forward that also stores the state entering every segment
     (Algorithm 1, sequence axis)."""
-    _check_inputs(x, dt, A, Bm, Cm, D)
-    shape = make_shape(x, Bm, chunk, seg, flags)
-    B, L, H, P = x.shape
-    N = Bm.shape[3]
-    y = torch.empty_like(x) if y is None else y
-    h_final = torch.empty(B, H, P, N, dtype=torch.float32, device=x.device) if h_final is None else h_final
-    if boundary is None:
-        nb = boundary_bytes(shape)
-        if nb == 0:
-            raise SSDError(SSD_EINVAL, "ssd_boundary_bytes")
-        boundary = torch.empty(B, nb // (4 * B * H * P * N), H, P, N, dtype=torch.float32, device=x.device)
-    ws = alloc_workspace(shape, SSD_OP_FWD_SEG, x.device) if ws is None else ws
-    rc = lib().ssd_fwd_segmented(ctypes.byref(shape), _ptr(x), _ptr(dt), _ptr(A), _ptr(Bm), _ptr(Cm),
-                                 _ptr(D), _ptr(h0), _ptr(y), _ptr(h_final), _ptr(boundary), _ptr(ws),
-                                 ws.numel(), _stream(stream))
-    if rc != SSD_OK:
-        raise SSDError(rc, "ssd_fwd_segmented")
-    return y, h_final, boundary
+    r = (_nat or _native()).fwd(x, dt, A, Bm, Cm, D, h0, chunk, seg, flags, y, h_final, boundary, ws, stream)
+    if r.__class__ is int:
+        raise SSDError(r, "ssd_fwd_segmented")
+    return r
 
 
 def ssd_bwd_segmented(x, dt, A, Bm, Cm, D, boundary, dy, dh_final=None, *, chunk, seg, flags=0,
                       out=None, want_dh0=True, ws=None, stream=None):
     """Gradients of Loss = <y,dy> + <h_final,dh_final> by Algorithm 2 along the sequence axis.
     Returns dict(dx, ddt, dA, dB, dC, dD, dh0)."""
-    _check_inputs(x, dt, A, Bm, Cm, D)
-    shape = make_shape(x, Bm, chunk, seg, flags)
-    B, L, H, P = x.shape
-    N = Bm.shape[3]
-    dev = x.device
     if out is None:
+        B, _, H, P = x.shape
+        N, dev = Bm.shape[3], x.device
         out = dict(dx=torch.empty_like(x), ddt=torch.empty_like(dt),
                    dA=torch.empty(H, dtype=torch.float32, device=dev),
                    dB=torch.empty_like(Bm), dC=torch.empty_like(Cm),
                    dD=torch.empty(H, dtype=torch.float32, device=dev),
                    dh0=torch.empty(B, H, P, N, dtype=torch.float32, device=dev) if want_dh0 else None)
-    ws = alloc_workspace(shape, SSD_OP_BWD_SEG, dev) if ws is None else ws
-    rc = lib().ssd_bwd_segmented(ctypes.byref(shape), _ptr(x), _ptr(dt), _ptr(A), _ptr(Bm), _ptr(Cm),
-                                 _ptr(D), _ptr(boundary), _ptr(dy), _ptr(dh_final), _ptr(out["dx"]),
-                                 _ptr(out["ddt"]), _ptr(out["dA"]), _ptr(out["dB"]), _ptr(out["dC"]),
-                                 _ptr(out["dD"]), _ptr(out.get("dh0")), _ptr(ws), ws.numel(),
-                                 _stream(stream))
+    rc = (_nat or _native()).bwd(x, dt, A, Bm, Cm, D, boundary, dy, dh_final, chunk, seg, flags, out["dx"], out["ddt"], out["dA"],
+                                 out["dB"], out["dC"], out["dD"], out.get("dh0"), ws, stream)
     if rc != SSD_OK:
         raise SSDError(rc, "ssd_bwd_segmented")
     return out
@@ -278,114 +264,45 @@ def ssd_bwd_segmented(x, dt, A, Bm, Cm, D, boundary, dy, dh_final=None, *, chunk
 def ssd_decode_step(x, dt, A, Bm, Cm, D, h, y=None, stream=None):
     """One token of Eq. 1: h (fp32 [B,H,P,N]) is advanced in place, y [B,1,H,P] is returned.
     x [B,1,H,P], dt [B,1,H], Bm/Cm [B,1,G,N] may be one-token slices of longer tensors."""
-    if not (x.is_cuda and h.is_cuda):
-        raise ValueError("device tensors required")
-    B, L, H, P = x.shape
-    G, N = Bm.shape[2], Bm.shape[3]
-    if L != 1 or dt.shape != (B, 1, H) or Cm.shape != Bm.shape or Bm.shape[:2] != (B, 1):
-        raise ValueError("ssd_decode_step takes one token: x [B,1,H,P], dt [B,1,H], Bm/Cm [B,1,G,N]")
-    if h.shape != (B, H, P, N) or h.dtype != torch.float32 or not h.is_contiguous():
-        raise ValueError("h must be a contiguous float32 [B,H,P,N] tensor")
-    if x.dtype not in (torch.bfloat16, torch.float32) or Bm.dtype != x.dtype or Cm.dtype != x.dtype:
-        raise TypeError("x, Bm, Cm must share dtype float32 or bfloat16")
-    # one-token slices of longer tensors are made dense here (a few KB); the C call also takes batch strides
-    x, dt, Bm, Cm = x.contiguous(), dt.contiguous(), Bm.contiguous(), Cm.contiguous()
-    y = torch.empty(B, 1, H, P, dtype=x.dtype, device=x.device) if y is None else y
-    if not y.is_contiguous() or y.shape != x.shape or y.dtype != x.dtype:
-        raise ValueError("y must be a dense tensor like x")
-    code = SSD_DTYPE_BF16 if x.dtype == torch.bfloat16 else SSD_DTYPE_F32
-    shape = SSDShape(B, 1, H, P, N, G, 0, 0, code, 0, 0, 0, 0)
-    rc = lib().ssd_decode_step(ctypes.byref(shape), _ptr(x), _ptr(dt), _ptr(A), _ptr(Bm), _ptr(Cm), _ptr(D),
-                               _ptr(h), _ptr(y), _stream(stream))
-    if rc != SSD_OK:
-        raise SSDError(rc, "ssd_decode_step")
-    return y
-
-
-def _conv_args(u):
-    B, L, C = u.shape
-    if u.dtype == torch.bfloat16:
-        code = SSD_DTYPE_BF16
-    elif u.dtype == torch.float32:
-        code = SSD_DTYPE_F32
-    else:
-        raise TypeError("u must be float32 or bfloat16")
-    if not u.is_cuda or u.stride(2) != 1 or u.stride(1) != C:
-        raise ValueError("u must be a CUDA tensor [B, L, C] with contiguous rows")
-    return B, L, C, code, (u.stride(0) if B > 1 else 0)
+    r = (_nat or _native()).decode_step(x, dt, A, Bm, Cm, D, h, y, stream)
+    if r.__class__ is int:
+        raise SSDError(r, "ssd_decode_step")
+    return r
 
 
 def ssd_conv_fwd(u, w, bias, state_in=None, *, out=None, state_out=None, stream=None):
     """out, state_out = SiLU(depthwise causal conv4(u)); state_in / state_out [B,3,C] carry the three inputs across
     a segment cut."""
-    B, L, C, code, bs = _conv_args(u)
-    out = torch.empty_like(u) if out is None else out
-    state_out = torch.empty(B, 3, C, dtype=u.dtype, device=u.device) if state_out is None else state_out
-    rc = lib().ssd_conv_fwd(B, L, C, code, _ptr(u), bs, _ptr(w), _ptr(bias), _ptr(state_in), _ptr(out), _ptr(state_out),
-                            _stream(stream))
-    if rc != SSD_OK:
-        raise SSDError(rc, "ssd_conv_fwd")
-    return out, state_out
+    r = (_nat or _native()).conv_fwd(u, w, bias, state_in, out, state_out, stream)
+    if r.__class__ is int:
+        raise SSDError(r, "ssd_conv_fwd")
+    return r
 
 
 def ssd_conv_bwd(u, w, bias, state_in, dout, dtail=None, *, du=None, dstate=None, dw=None, dbias=None, accumulate=False,
                  ws=None, stream=None):
     """du, dstate, dw, dbias of one segment (Algorithm 2's order: the segment to the right first; its dstate is this
     call's dtail)."""
-    B, L, C, code, bs = _conv_args(u)
-    dev = u.device
-    du = torch.empty_like(u) if du is None else du
-    dstate = torch.empty(B, 3, C, dtype=torch.float32, device=dev) if dstate is None else dstate
-    dw = torch.zeros(C, 4, dtype=torch.float32, device=dev) if dw is None else dw
-    dbias = torch.zeros(C, dtype=torch.float32, device=dev) if dbias is None else dbias
-    nws = int(lib().ssd_conv_workspace_bytes(B, L, C))
-    ws = torch.empty(nws, dtype=torch.uint8, device=dev) if ws is None else ws
-    rc = lib().ssd_conv_bwd(B, L, C, code, _ptr(u), bs, _ptr(w), _ptr(bias), _ptr(state_in), _ptr(dout), _ptr(dtail),
-                            _ptr(du), _ptr(dstate), _ptr(dw), _ptr(dbias), 1 if accumulate else 0, _ptr(ws), ws.numel(),
-                            _stream(stream))
-    if rc != SSD_OK:
-        raise SSDError(rc, "ssd_conv_bwd")
-    return du, dstate, dw, dbias
-
-
-def _norm_args(y):
-    if y.dtype == torch.bfloat16:
-        code = SSD_DTYPE_BF16
-    elif y.dtype == torch.float32:
-        code = SSD_DTYPE_F32
-    else:
-        raise TypeError("y must be float32 or bfloat16")
-    if not y.is_cuda or not y.is_contiguous():
-        raise ValueError("y must be a contiguous CUDA tensor [..., D]")
-    D = y.shape[-1]
-    return y.numel() // D, D, code
+    r = (_nat or _native()).conv_bwd(u, w, bias, state_in, dout, dtail, du, dstate, dw, dbias, accumulate, ws, stream)
+    if r.__class__ is int:
+        raise SSDError(r, "ssd_conv_bwd")
+    return r
 
 
 def ssd_gated_norm_fwd(y, z, gamma, *, group=None, eps=1e-5, out=None, stream=None):
     """out = RMSNorm(y * silu(z)) * gamma over groups of `group` channels (default: the whole last dimension)."""
-    rows, D, code = _norm_args(y)
-    out = torch.empty_like(y) if out is None else out
-    rc = lib().ssd_gated_norm_fwd(rows, D, D if group is None else int(group), code, _ptr(y), _ptr(z), _ptr(gamma), float(eps),
-                                  _ptr(out), _stream(stream))
-    if rc != SSD_OK:
-        raise SSDError(rc, "ssd_gated_norm_fwd")
-    return out
+    r = (_nat or _native()).gated_norm_fwd(y, z, gamma, group, eps, out, stream)
+    if r.__class__ is int:
+        raise SSDError(r, "ssd_gated_norm_fwd")
+    return r
 
 
 def ssd_gated_norm_bwd(y, z, gamma, dout, *, group=None, eps=1e-5, dy=None, dz=None, dgamma=None, accumulate=False, ws=None,
                        stream=None):
-    rows, D, code = _norm_args(y)
-    dy = torch.empty_like(y) if dy is None else dy
-    dz = torch.empty_like(y) if dz is None else dz
-    dgamma = torch.zeros(D, dtype=torch.float32, device=y.device) if dgamma is None else dgamma
-    nws = int(lib().ssd_gated_norm_workspace_bytes(rows, D))
-    ws = torch.empty(nws, dtype=torch.uint8, device=y.device) if ws is None else ws
-    rc = lib().ssd_gated_norm_bwd(rows, D, D if group is None else int(group), code, _ptr(y), _ptr(z), _ptr(gamma), float(eps),
-                                  _ptr(dout), _ptr(dy), _ptr(dz), _ptr(dgamma), 1 if accumulate else 0, _ptr(ws), ws.numel(),
-                                  _stream(stream))
-    if rc != SSD_OK:
-        raise SSDError(rc, "ssd_gated_norm_bwd")
-    return dy, dz, dgamma
+    r = (_nat or _native()).gated_norm_bwd(y, z, gamma, dout, group, eps, dy, dz, dgamma, accumulate, ws, stream)
+    if r.__class__ is int:
+        raise SSDError(r, "ssd_gated_norm_bwd")
+    return r
 
 
 def _glue_shape(t):
@@ -403,7 +320,7 @@ def _glue_shape(t):
 
 def ssd_glue_fwd(x, y, W, x_next, stream=None):
     """x_next = W (y + x) per (batch, step, head): the hand-over between two stacked layers."""
-    rc = lib().ssd_glue_fwd(ctypes.byref(_glue_shape(x)), _ptr(x), _ptr(y), _ptr(W), _ptr(x_next), _stream(stream))
+    rc = (_nat or _native()).glue_fwd(x, y, W, x_next, stream)
     if rc != SSD_OK:
         raise SSDError(rc, "ssd_glue_fwd")
     return x_next
@@ -411,7 +328,7 @@ def ssd_glue_fwd(x, y, W, x_next, stream=None):
 
 def ssd_glue_bwd(g_next, W, dz, stream=None):
     """dz = W^T g_next: the gradient of the layer's output (its dy) and of the skip branch."""
-    rc = lib().ssd_glue_bwd(ctypes.byref(_glue_shape(g_next)), _ptr(g_next), _ptr(W), _ptr(dz), _stream(stream))
+    rc = (_nat or _native()).glue_bwd(g_next, W, dz, stream)
     if rc != SSD_OK:
         raise SSDError(rc, "ssd_glue_bwd")
     return dz
