@@ -44,15 +44,12 @@ static void prof_end(ProfEvent *ev, cudaStream_t st) {
     if (ev) cudaEventRecord(ev->b, st);
 }
 
+// Scratch regions of one call.  What the kernels of neighbouring segments touch at the same time exists twice on the
+// tensor-core path (copy k & 1 belongs to segment k).
 struct Layout {
-    size_t status, cs, dtT, Hst, Hbf, hcarry, Gst, Gbf, gcarry, ghdot, ddt_dir, rho, rho2, psi, psi2, pB, pC, dAp, dDp;
-    size_t rhob, psib;
-    // second copies (tensor-core path, more than one segment): the state chain of a segment runs on a helper
-    // stream while the large kernels of its neighbour still read the first copies
-    size_t cs_b, dtT_b, Hbf_b, Gbf_b, rho2_b, ghdot_b;
-    // and of what the large kernels of the backward leave for a segment's finishing kernels, so that the next
-    // segment's large kernels need not wait for those
-    size_t ddt_dir_b, rho_b, rhob_b, psi_b, psib_b, psi2_b, pB_b, pC_b;
+    size_t status, Hst, hcarry, Gst, gcarry, dAp, dDp;
+    size_t rec[2], cs[2], dtT[2], Hbf[2];
+    size_t Gbf[2], ghdot[2], ddt_dir[2], rho[2], rho2[2], rho2b[2], psi[2], psi2[2], pB[2], pC[2];
     size_t total;
 };
 
@@ -62,65 +59,25 @@ struct Layout {
 static const int kMinSegmentsForTwins = 4;
 
 struct Plan {
-    int B, L, H, P, N, G, Q, seg, nseg, ncs, nct, hpg, nsl, nslf, dtype;
+    int B, L, H, P, N, G, Q, seg, nseg, ncs, nct, hpg, nsl, dtype;   // Q: steps per chunk (CUDA cores) or block (tensor cores)
     bool use_tc, serial;
     int64_t x_bs, dt_bs, bc_bs;
     size_t esz;
 };
 
-// How many head ranges per group for the tensor-core kernels whose CTAs are (chunk, 128-row block,
-// head range).  Half of the CTAs do about 1.8 times the work of the other half (causal structure) and
-// are launched first; one CTA per SM, kNumSMs SMs.  The split that minimises the makespan of a greedy
-// schedule is taken (cost of a CTA: one head-time of set-up plus its heads).
-static int best_head_split(int nchunks, int groups, int batch, int hpg, int max_split) {
-    const int kNumSMs = 148;
-    // the driver asks once per segment: remember the last few answers
-    struct Memo { int nchunks, groups, batch, hpg, max_split, answer; };
-    static thread_local Memo memo[4] = {};
-    static thread_local int memo_next = 0;
-    for (const Memo &m : memo)
-        if (m.answer > 0 && m.nchunks == nchunks && m.groups == groups && m.batch == batch && m.hpg == hpg &&
-            m.max_split == max_split)
-            return m.answer;
+// Head ranges per group for the dB/dC kernel, whose CTAs are (block, head range), for a reference launch of 32 blocks: the
+// launch's share of the GPU (a part of a wave still takes the time of its slowest CTA; beyond one wave the kernels of
+// neighbouring segments fill each other's gaps) times the time of a CTA, eight head-times of set-up and output plus its
+// heads.  A function of H and G only, so the summation order of dB/dC does not depend on the segment length.
+static int bc_head_split(int groups, int hpg) {
     int best = 1;
-    double best_t = 1e300;
-    for (int ns = 1; ns <= max_split; ++ns) {
-        const int hps = (hpg + ns - 1) / ns;
-        if ((hpg + hps - 1) / hps != ns) continue;   // would leave an empty range
-        double sm[kNumSMs];
-        for (int i = 0; i < kNumSMs; ++i) sm[i] = 0.0;
-        double makespan = 0.0;
-        for (int pass = 0; pass < 2; ++pass)          // all long CTAs, then all short ones
-            for (int j = 0; j < nchunks * groups * batch; ++j)
-                for (int r = 0; r < ns; ++r) {
-                    const int heads = (r == ns - 1) ? hpg - hps * (ns - 1) : hps;
-                    const double cost = 1.0 + heads * (pass == 0 ? 1.0 : 0.55);
-                    int arg = 0;
-                    for (int i = 1; i < kNumSMs; ++i)
-                        if (sm[i] < sm[arg]) arg = i;
-                    sm[arg] += cost;
-                    if (sm[arg] > makespan) makespan = sm[arg];
-                }
-        if (makespan < best_t - 1e-9) { best_t = makespan; best = ns; }
-    }
-    memo[memo_next] = Memo{nchunks, groups, batch, hpg, max_split, best};
-    memo_next = (memo_next + 1) & 3;
-    return best;
-}
-
-// Head ranges per group for the fused dB/dC kernel, whose CTAs are (chunk, one of the three causal 128 x 128
-// tiles, head range), all of about the same cost: whole waves of 148 CTAs times (one head-time of set-up plus
-// the heads of a range), for a reference launch of 16 chunks.  A function of H and G only, so the summation
-// order of dB/dC does not depend on the segment length.
-static int fused_head_split(int groups, int hpg) {
-    int best = 1;
-    long best_t = -1;
+    double best_t = -1;
     const int max_split = hpg >= 4 ? hpg / 4 : 1;
     for (int ns = 1; ns <= max_split; ++ns) {
         const int hps = (hpg + ns - 1) / ns;
-        if ((hpg + hps - 1) / hps != ns) continue;
-        const long ctas = 16L * 3 * groups * ns;
-        const long t = ((ctas + 147) / 148) * (1 + hps);
+        if ((hpg + hps - 1) / hps != ns) continue;      // would leave an empty range
+        const double waves = 32.0 * groups * ns / kNumSMs;
+        const double t = (waves > 1 ? waves : 1) * (8 + hps);
         if (best_t < 0 || t < best_t) { best_t = t; best = ns; }
     }
     return best;
@@ -140,11 +97,13 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
     const int seg = s->seg == 0 ? s->L : (s->seg > s->L ? s->L : s->seg);
     if (seg % s->chunk) return SSD_EINVAL;
     if (s->x_bstride < 0 || s->dt_bstride < 0 || s->bc_bstride < 0) return SSD_EINVAL;
-    pl.B = s->B; pl.L = s->L; pl.H = s->H; pl.P = s->P; pl.N = s->N; pl.G = s->G; pl.Q = s->chunk;
+    pl.B = s->B; pl.L = s->L; pl.H = s->H; pl.P = s->P; pl.N = s->N; pl.G = s->G;
+    pl.use_tc = tc_supported(s->dtype, s->flags, s->P, s->N, s->chunk);
+    pl.Q = pl.use_tc ? kTcBlock : s->chunk;
     pl.seg = seg;
     pl.nseg = (s->L + seg - 1) / seg;
-    pl.ncs = seg / s->chunk;
-    pl.nct = s->L / s->chunk;
+    pl.ncs = seg / pl.Q;
+    pl.nct = s->L / pl.Q;
     pl.hpg = s->H / s->G;
     pl.dtype = s->dtype;
     pl.esz = s->dtype == SSD_DTYPE_BF16 ? 2 : 4;
@@ -158,18 +117,9 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
         ((size_t)pl.x_bs * pl.esz) % 16 || ((size_t)pl.bc_bs * pl.esz) % 16)
         return SSD_EALIGN;
     pl.serial = (s->flags & SSD_FLAG_SERIAL) != 0;
-    pl.use_tc = tc_supported(s->dtype, s->flags, s->P, s->N, s->chunk, pl.hpg);
-    // Partial slices of the dB/dC head sums.  CUDA-core kernels: one head per slice.  Tensor-core
-    // kernels: one slice per CTA head range, chosen for a reference launch of 16 chunks (at least 4
-    // heads per range).  A function of H and G only, so the summation order, and with it every bit
-    // of dB/dC, is the same for every segment length.
-    if (pl.use_tc) {
-        pl.nsl = best_head_split(16, pl.G, 1, pl.hpg, pl.hpg >= 4 ? pl.hpg / 4 : 1);
-        pl.nslf = fused_head_split(pl.G, pl.hpg);
-    } else {
-        pl.nsl = pl.hpg;
-        pl.nslf = 0;
-    }
+    // Partial slices of the dB/dC head sums.  CUDA-core kernels: one head per slice.  Tensor-core kernel: one slice per CTA
+    // head range.
+    pl.nsl = pl.use_tc ? bc_head_split(pl.G, pl.hpg) : pl.hpg;
     return SSD_OK;
 }
 
@@ -178,50 +128,47 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
 static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
     const size_t PN = (size_t)pl.P * pl.N, BH = (size_t)pl.B * pl.H;
     const size_t vec = BH * pl.ncs * pl.Q * sizeof(float);
-    const size_t st = (size_t)pl.B * (pl.ncs + 1) * pl.H * PN;
+    const size_t st = BH * (pl.ncs + 1) * PN * sizeof(float), stb = BH * pl.ncs * PN * 2;
     const bool bwd = (op == SSD_OP_BWD_SEG);
+    const bool twin = twins && pl.use_tc && pl.nseg >= kMinSegmentsForTwins;
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
+    auto take2 = [&](size_t (&r)[2], size_t bytes, bool two) {
+        r[0] = take(bytes);
+        r[1] = two ? take(bytes) : r[0];
+    };
     memset(&lo, 0, sizeof(lo));
     lo.status = take(256);
-    lo.cs = take(vec);
-    lo.dtT = take(vec);
-    lo.Hst = take(st * sizeof(float));
-    lo.Hbf = take(pl.use_tc ? st * 2 : 0);
     lo.hcarry = take(BH * PN * sizeof(float));
-    const bool twin = twins && pl.use_tc && pl.nseg >= kMinSegmentsForTwins;
-    lo.cs_b = take(twin ? vec : 0);
-    lo.dtT_b = take(twin ? vec : 0);
-    lo.Hbf_b = take(twin ? st * 2 : 0);
+    // the vectors and records (a fraction of the states) exist twice for any number of segments, so that the scratch is a function of
+    // the segment length that only rises
+    if (pl.use_tc) {
+        take2(lo.rec, BH * pl.ncs * REC_FLOATS * sizeof(float), twins);
+        take2(lo.Hbf, stb, twin);
+    } else {
+        take2(lo.cs, vec, false);
+        take2(lo.dtT, vec, false);
+        lo.Hst = take(st);
+    }
     if (bwd) {
-        lo.Gst = take(st * sizeof(float));
-        lo.Gbf = take(pl.use_tc ? st * 2 : 0);
         lo.gcarry = take(BH * PN * sizeof(float));
-        lo.ghdot = take(BH * pl.ncs * 16 * sizeof(float));
-        lo.ddt_dir = take(vec);
-        lo.rho = take(vec);
-        lo.rho2 = take(pl.use_tc ? vec : 0);
-        lo.psi = take(vec);
-        lo.psi2 = take(vec);
-        const int slots = (2 * pl.nslf > pl.nsl) ? 2 * pl.nslf : pl.nsl;   // fused kernel: two slots per head range
-        const size_t part = (size_t)pl.B * pl.seg * pl.G * slots * pl.N * sizeof(float);
-        lo.pB = take(part);
-        lo.pC = take(part);
+        if (pl.use_tc) take2(lo.Gbf, stb, twin);
+        else lo.Gst = take(st);
+        take2(lo.ghdot, BH * pl.ncs * 16 * sizeof(float), twin);
+        const bool vtwin = twins && pl.use_tc;
+        take2(lo.ddt_dir, vec, vtwin);
+        take2(lo.rho, vec, vtwin);
+        if (pl.use_tc) {
+            take2(lo.rho2, vec, vtwin);
+            take2(lo.rho2b, vec, vtwin);
+        }
+        take2(lo.psi, vec, vtwin);
+        take2(lo.psi2, vec, vtwin);
+        const size_t part = (size_t)pl.B * pl.seg * pl.G * pl.nsl * pl.N * sizeof(float);
+        take2(lo.pB, part, twin);
+        take2(lo.pC, part, twin);
         lo.dAp = take(BH * pl.nct * sizeof(float));
-        lo.dDp = take(BH * pl.nct * 16 * sizeof(float));
-        lo.Gbf_b = take(twin ? st * 2 : 0);
-        lo.rho2_b = take(twin ? vec : 0);
-        lo.ghdot_b = take(twin ? BH * pl.ncs * 16 * sizeof(float) : 0);
-        lo.rhob = take(pl.use_tc ? vec : 0);
-        lo.psib = take(pl.use_tc ? vec : 0);
-        lo.ddt_dir_b = take(twin ? vec : 0);
-        lo.rho_b = take(twin ? vec : 0);
-        lo.rhob_b = take(twin ? vec : 0);
-        lo.psi_b = take(twin ? vec : 0);
-        lo.psib_b = take(twin ? vec : 0);
-        lo.psi2_b = take(twin ? vec : 0);
-        lo.pB_b = take(twin ? part : 0);
-        lo.pC_b = take(twin ? part : 0);
+        lo.dDp = take(BH * pl.nct * 4 * sizeof(float));
     }
     lo.total = o;
 }
@@ -297,32 +244,43 @@ static SideStreams *side_streams() {
         }                                               \
     } while (0)
 
+// Points the kernels at copy 0 or 1 of the scratch regions that may exist twice.
+static void select_copy(const Layout &lo, void *ws, int k, SegParams &sp) {
+    char *w = (char *)ws;
+    auto f = [&](const size_t (&r)[2]) { return r[k] ? (float *)(w + r[k]) : nullptr; };
+    sp.rec = f(lo.rec);
+    sp.cs = f(lo.cs);
+    sp.dtT = sp.rec ? sp.rec + REC_DT : f(lo.dtT);
+    sp.dt_stride = sp.rec ? (int)REC_FLOATS : sp.Q;
+    sp.Hbf = (__nv_bfloat16 *)f(lo.Hbf);
+    sp.Gbf = (__nv_bfloat16 *)f(lo.Gbf);
+    sp.ghdot = f(lo.ghdot);
+    sp.ddt_dir = f(lo.ddt_dir);
+    sp.rho = f(lo.rho);
+    sp.rho2 = f(lo.rho2);
+    sp.rho2b = f(lo.rho2b);
+    sp.psi = f(lo.psi);
+    sp.psi2 = f(lo.psi2);
+    sp.pB = f(lo.pB);
+    sp.pC = f(lo.pC);
+}
+
 static void fill_params(const Plan &pl, const Layout &lo, void *ws, SegParams &sp) {
     memset(&sp, 0, sizeof(sp));
     sp.B = pl.B; sp.L = pl.L; sp.H = pl.H; sp.P = pl.P; sp.N = pl.N; sp.G = pl.G; sp.Q = pl.Q;
     sp.hpg = pl.hpg; sp.ncs = pl.ncs; sp.nct = pl.nct; sp.nsl = pl.nsl;
-    sp.ndd = pl.use_tc ? 8 : pl.Q / 64;
+    sp.ndd = pl.use_tc ? 4 : pl.Q / 64;
+    sp.ngh = pl.use_tc ? 8 : pl.P * pl.N / kStatePassElems;
     sp.x_bs = pl.x_bs; sp.dt_bs = pl.dt_bs; sp.bc_bs = pl.bc_bs;
     char *w = (char *)ws;
     sp.status = (unsigned int *)(w + lo.status);
-    sp.cs = (float *)(w + lo.cs);
-    sp.dtT = (float *)(w + lo.dtT);
     sp.Hst = (float *)(w + lo.Hst);
-    sp.Hbf = (__nv_bfloat16 *)(w + lo.Hbf);
     sp.hcarry = (float *)(w + lo.hcarry);
     sp.Gst = (float *)(w + lo.Gst);
-    sp.Gbf = (__nv_bfloat16 *)(w + lo.Gbf);
     sp.gcarry = (float *)(w + lo.gcarry);
-    sp.ghdot = (float *)(w + lo.ghdot);
-    sp.ddt_dir = (float *)(w + lo.ddt_dir);
-    sp.rho = (float *)(w + lo.rho);
-    sp.rho2 = nullptr;   // set by the backward driver on the tensor-core path
-    sp.psi = (float *)(w + lo.psi);
-    sp.psi2 = (float *)(w + lo.psi2);
-    sp.pB = (float *)(w + lo.pB);
-    sp.pC = (float *)(w + lo.pC);
     sp.dAp = (float *)(w + lo.dAp);
     sp.dDp = (float *)(w + lo.dDp);
+    select_copy(lo, ws, 0, sp);
 }
 
 static void set_segment(const Plan &pl, int k, SegParams &sp) {
@@ -330,32 +288,6 @@ static void set_segment(const Plan &pl, int k, SegParams &sp) {
     const int len = (pl.L - sp.t0 < pl.seg) ? pl.L - sp.t0 : pl.seg;
     sp.nc = len / pl.Q;
     sp.c0 = sp.t0 / pl.Q;
-    // Head ranges per group for the scan kernels (at least two heads per CTA so the shared score tile
-    // is reused).  Their outputs are per head, so this choice cannot change any result bit.
-    sp.nsplit_scan = best_head_split(sp.nc, pl.G, pl.B, pl.hpg, pl.hpg >= 2 ? pl.hpg / 2 : 1);
-}
-
-// Points the kernels at the first or the second copy of the scratch regions that exist twice.
-static void select_copy(const Layout &lo, void *ws, bool second, bool bwd, SegParams &sp) {
-    char *w = (char *)ws;
-    sp.cs = (float *)(w + (second ? lo.cs_b : lo.cs));
-    sp.dtT = (float *)(w + (second ? lo.dtT_b : lo.dtT));
-    sp.Hbf = (__nv_bfloat16 *)(w + (second ? lo.Hbf_b : lo.Hbf));
-    if (bwd) {
-        sp.Gbf = (__nv_bfloat16 *)(w + (second ? lo.Gbf_b : lo.Gbf));
-        sp.rho2 = (float *)(w + (second ? lo.rho2_b : lo.rho2));
-        sp.ghdot = (float *)(w + (second ? lo.ghdot_b : lo.ghdot));
-        sp.ddt_dir = (float *)(w + (second ? lo.ddt_dir_b : lo.ddt_dir));
-        sp.rho = (float *)(w + (second ? lo.rho_b : lo.rho));
-        sp.psi = (float *)(w + (second ? lo.psi_b : lo.psi));
-        sp.psi2 = (float *)(w + (second ? lo.psi2_b : lo.psi2));
-        sp.pB = (float *)(w + (second ? lo.pB_b : lo.pB));
-        sp.pC = (float *)(w + (second ? lo.pC_b : lo.pC));
-        if (sp.rhob) {   // the fused dB/dC kernel is in use
-            sp.rhob = (float *)(w + (second ? lo.rhob_b : lo.rhob));
-            sp.psib = (float *)(w + (second ? lo.psib_b : lo.psib));
-        }
-    }
 }
 
 static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt, const float *A,
@@ -393,7 +325,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         SideStreams *side = side_streams();
         if (!side) { g_last_cuda = (int)cudaGetLastError(); return SSD_ECUDA; }
         TcMaps maps_b;
-        select_copy(lo, ws, true, false, sp);
+        select_copy(lo, ws, 1, sp);
         if (!tc_make_maps(sp, maps_b)) return SSD_ECUDA;
         cudaStream_t chain = side->s[0];
         SSD_TRY(cudaEventRecord(side->start, st));
@@ -401,16 +333,15 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         for (int k = 0; k < pl.nseg; ++k) {
             const int par = k & 1;
             set_segment(pl, k, sp);
-            select_copy(lo, ws, par != 0, false, sp);
+            select_copy(lo, ws, par, sp);
             const TcMaps &mk = par ? maps_b : maps;
             if (k >= 2) SSD_TRY(cudaStreamWaitEvent(chain, side->big_done[par], 0));   // y of segment k-2 has read this copy
             {
                 cudaStream_t st = chain;
-                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_tc(sp, mk, STATE_MODE_FWD, st));
                 const float *init = (k == 0) ? h0 : sp.hcarry;
                 float *bnd = boundary ? boundary + (size_t)k * pl.H * PN : nullptr;
-                SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN,
-                                              (k == pl.nseg - 1) ? h_final : nullptr, true, st));
+                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, mk, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN,
+                                                              (k == pl.nseg - 1) ? h_final : nullptr, st));
                 SSD_TRY(cudaEventRecord(side->chain_done[par], st));
             }
             SSD_TRY(cudaStreamWaitEvent(st, side->chain_done[par], 0));
@@ -421,18 +352,17 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     }
     for (int k = 0; k < pl.nseg; ++k) {
         set_segment(pl, k, sp);
-        if (pl.use_tc) {   // the tensor-core chunk-state kernel computes the chunk cumsum itself
-            SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_tc(sp, maps, STATE_MODE_FWD, st));
-        } else {
-            SSD_LAUNCH(KIND_CUMSUM, launch_chunk_cumsum(sp, st));
-            SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_simt(sp, pl.dtype, STATE_MODE_FWD, st));
-        }
         const float *init = (k == 0) ? h0 : sp.hcarry;
-        float *bnd = boundary ? boundary + (size_t)k * pl.H * PN : nullptr;
-        SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN,
-                                      (k == pl.nseg - 1) ? h_final : nullptr, pl.use_tc, st));
-        if (pl.use_tc) SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, maps, SC_FWD, st));
-        else SSD_LAUNCH(KIND_SCAN_FWD, launch_masked_product_simt(sp, pl.dtype, MP_FWD, st));
+        float *bnd = boundary ? boundary + (size_t)k * pl.H * PN : nullptr, *fin = (k == pl.nseg - 1) ? h_final : nullptr;
+        if (pl.use_tc) {
+            SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, maps, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN, fin, st));
+            SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, maps, SC_FWD, st));
+            continue;
+        }
+        SSD_LAUNCH(KIND_CUMSUM, launch_chunk_cumsum(sp, st));
+        SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_simt(sp, pl.dtype, STATE_MODE_FWD, st));
+        SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN, fin, st));
+        SSD_LAUNCH(KIND_SCAN_FWD, launch_masked_product_simt(sp, pl.dtype, MP_FWD, st));
     }
     return SSD_OK;
 }
@@ -562,18 +492,11 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
     sp.x = x; sp.dt = dt; sp.A = A; sp.Bm = Bm; sp.Cm = Cm; sp.D = D; sp.dy = dy;
     sp.dx = dx; sp.ddt = ddt; sp.dB = dB; sp.dC = dC;
     sp.dx_skip = (shape->flags & SSD_FLAG_SKIP_GRAD) ? 1.f : 0.f;
-    if (pl.use_tc) sp.rho2 = (float *)((char *)ws + lo.rho2);
     SSD_TRY(cudaMemsetAsync(sp.status, 0, 256, st));
     TcMaps maps;
     if (pl.use_tc && !tc_make_maps(sp, maps)) return SSD_ECUDA;
     const long long PN = (long long)pl.P * pl.N;
-    const bool fused_bc = pl.use_tc && !(shape->flags & SSD_FLAG_SPLIT_BC);
-    if (fused_bc) {
-        sp.nsl = pl.nslf;
-        sp.bc_fused = 1;
-        sp.rhob = (float *)((char *)ws + lo.rhob);
-        sp.psib = (float *)((char *)ws + lo.psib);
-    }
+    const bool split_bc = (shape->flags & SSD_FLAG_SPLIT_BC) != 0;
     SideStreams *side = nullptr;
     if (pl.use_tc && !(shape->flags & SSD_FLAG_SERIAL) && !g_prof_on) {
         side = side_streams();
@@ -592,7 +515,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         const bool twin = pl.nseg >= kMinSegmentsForTwins;    // else one copy: chain(k) then also waits for tail(k+1)
         TcMaps maps_b;
         if (twin) {
-            select_copy(lo, ws, true, true, sp);
+            select_copy(lo, ws, 1, sp);
             if (!tc_make_maps(sp, maps_b)) return SSD_ECUDA;
         }
         cudaStream_t grads = side->s[0], recomp = side->s[4], tails = side->s[2];
@@ -603,16 +526,15 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         for (int k = pl.nseg - 1; k >= 0; --k) {
             par = twin ? ((pl.nseg - 1 - k) & 1) : 0;
             set_segment(pl, k, sp);
-            select_copy(lo, ws, par != 0, true, sp);
+            select_copy(lo, ws, par, sp);
             const TcMaps &mk = par ? maps_b : maps;
             // ---- chain(k), first half: Recompute_Forward.  Its copy was last read by big(k+2) and tail(k+2) (of k+1
             // when there is one copy only); the fp32 chunk sums belong to this stream alone.
             if (k + (twin ? 2 : 1) <= pl.nseg - 1) SSD_TRY(cudaStreamWaitEvent(recomp, side->tail_done[par], 0));
             {
                 cudaStream_t st = recomp;
-                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_tc(sp, mk, STATE_MODE_FWD, st));
-                SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, boundary + (size_t)k * pl.H * PN, (long long)pl.nseg * pl.H * PN,
-                                              nullptr, 0, nullptr, true, st));
+                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, mk, boundary + (size_t)k * pl.H * PN, (long long)pl.nseg * pl.H * PN,
+                                                              nullptr, 0, nullptr, st));
                 SSD_TRY(cudaEventRecord(side->rec_done[par], st));
             }
             // ---- chain(k), second half: the state gradients, which alone wait for segment k+1 (stream order: the
@@ -620,10 +542,9 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
             SSD_TRY(cudaStreamWaitEvent(grads, side->rec_done[par], 0));
             {
                 cudaStream_t st = grads;
-                SSD_LAUNCH(KIND_DSTATE, launch_chunk_state_tc(sp, mk, STATE_MODE_DSTATE, st));
                 const float *ginit = (k == pl.nseg - 1) ? dh_final : sp.gcarry;
                 float *gleft = (k == 0 && dh0) ? dh0 : sp.gcarry;
-                SSD_LAUNCH(KIND_STATE_PASS_BWD, launch_state_pass_bwd(sp, ginit, gleft, true, st));
+                SSD_LAUNCH(KIND_DSTATE, launch_chain_bwd(sp, mk, ginit, gleft, st));
                 SSD_TRY(cudaEventRecord(side->chain_done[par], st));
             }
             // ---- big(k); what it leaves for tail(k) (direct ddt, rho, psi, partial dB/dC slices) alternates too, and
@@ -634,11 +555,11 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
             SSD_TRY(cudaStreamWaitEvent(bcs, side->chain_done[par], 0));
             {
                 cudaStream_t st = bcs;
-                if (fused_bc) {
-                    SSD_LAUNCH(KIND_BWD_DBDC, launch_grad_bc_fused(sp, mk, st));
+                if (!split_bc) {
+                    SSD_LAUNCH(KIND_BWD_DBDC, launch_grad_bc(sp, mk, BC_DC | BC_DB, st));
                 } else {
-                    SSD_LAUNCH(KIND_BWD_DC, launch_grad_bc_tc(sp, mk, GB_DC, st));
-                    SSD_LAUNCH(KIND_BWD_DB, launch_grad_bc_tc(sp, mk, GB_DB, st));
+                    SSD_LAUNCH(KIND_BWD_DC, launch_grad_bc(sp, mk, BC_DC, st));
+                    SSD_LAUNCH(KIND_BWD_DB, launch_grad_bc(sp, mk, BC_DB, st));
                 }
                 SSD_TRY(cudaEventRecord(side->join[par], st));
             }
@@ -658,29 +579,27 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
     } else {
         for (int k = pl.nseg - 1; k >= 0; --k) {
             set_segment(pl, k, sp);
-            // Recompute_Forward: chunk-entry states of segment k from the stored boundary state
-            if (pl.use_tc) {   // the tensor-core chunk-state kernel computes the chunk cumsum itself
-                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_tc(sp, maps, STATE_MODE_FWD, st));
+            // Recompute_Forward: chunk-entry states of segment k from the stored boundary state; then backward through the
+            // segment: dh enters from the right, leaves to the left
+            const float *hin = boundary + (size_t)k * pl.H * PN, *ginit = (k == pl.nseg - 1) ? dh_final : sp.gcarry;
+            float *gleft = (k == 0 && dh0) ? dh0 : sp.gcarry;
+            if (pl.use_tc) {
+                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, maps, hin, (long long)pl.nseg * pl.H * PN, nullptr, 0, nullptr, st));
+                SSD_LAUNCH(KIND_DSTATE, launch_chain_bwd(sp, maps, ginit, gleft, st));
+                SSD_LAUNCH(KIND_BWD_DX, launch_scan_tc(sp, maps, SC_DX, st));
+                if (!split_bc) {
+                    SSD_LAUNCH(KIND_BWD_DBDC, launch_grad_bc(sp, maps, BC_DC | BC_DB, st));
+                } else {
+                    SSD_LAUNCH(KIND_BWD_DC, launch_grad_bc(sp, maps, BC_DC, st));
+                    SSD_LAUNCH(KIND_BWD_DB, launch_grad_bc(sp, maps, BC_DB, st));
+                }
             } else {
                 SSD_LAUNCH(KIND_CUMSUM, launch_chunk_cumsum(sp, st));
                 SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_simt(sp, pl.dtype, STATE_MODE_FWD, st));
-            }
-            SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, boundary + (size_t)k * pl.H * PN, (long long)pl.nseg * pl.H * PN,
-                                          nullptr, 0, nullptr, pl.use_tc, st));
-            // Backward through the segment; dh enters from the right, leaves to the left
-            if (pl.use_tc) SSD_LAUNCH(KIND_DSTATE, launch_chunk_state_tc(sp, maps, STATE_MODE_DSTATE, st));
-            else SSD_LAUNCH(KIND_DSTATE, launch_chunk_state_simt(sp, pl.dtype, STATE_MODE_DSTATE, st));
-            const float *ginit = (k == pl.nseg - 1) ? dh_final : sp.gcarry;
-            float *gleft = (k == 0 && dh0) ? dh0 : sp.gcarry;
-            SSD_LAUNCH(KIND_STATE_PASS_BWD, launch_state_pass_bwd(sp, ginit, gleft, pl.use_tc, st));
-            if (pl.use_tc) SSD_LAUNCH(KIND_BWD_DX, launch_scan_tc(sp, maps, SC_DX, st));
-            else SSD_LAUNCH(KIND_BWD_DX, launch_masked_product_simt(sp, pl.dtype, MP_BWD_DX, st));
-            if (fused_bc) {
-                SSD_LAUNCH(KIND_BWD_DBDC, launch_grad_bc_fused(sp, maps, st));
-            } else if (pl.use_tc) {
-                SSD_LAUNCH(KIND_BWD_DC, launch_grad_bc_tc(sp, maps, GB_DC, st));
-                SSD_LAUNCH(KIND_BWD_DB, launch_grad_bc_tc(sp, maps, GB_DB, st));
-            } else {
+                SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, hin, (long long)pl.nseg * pl.H * PN, nullptr, 0, nullptr, st));
+                SSD_LAUNCH(KIND_DSTATE, launch_chunk_state_simt(sp, pl.dtype, STATE_MODE_DSTATE, st));
+                SSD_LAUNCH(KIND_STATE_PASS_BWD, launch_state_pass_bwd(sp, ginit, gleft, st));
+                SSD_LAUNCH(KIND_BWD_DX, launch_masked_product_simt(sp, pl.dtype, MP_BWD_DX, st));
                 SSD_LAUNCH(KIND_BWD_DC, launch_masked_product_simt(sp, pl.dtype, MP_DC, st));
                 SSD_LAUNCH(KIND_BWD_DB, launch_masked_product_simt(sp, pl.dtype, MP_DB, st));
             }

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
+
 #include "ssd.h"
 
 namespace ssd {
@@ -32,7 +34,41 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
 }
+// Lets kernel K use `bytes` of dynamic shared memory; the attribute is set once per device.
+template <auto K> inline cudaError_t allow_smem(int bytes) {
+    static std::atomic<uint64_t> done{0};
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const uint64_t bit = 1ull << (dev & 63);
+    if (dev < 64 && (done.load(std::memory_order_relaxed) & bit)) return cudaSuccess;
+    e = cudaFuncSetAttribute(K, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    if (e == cudaSuccess) done.fetch_or(bit, std::memory_order_relaxed);
+    return e;
+}
 #endif
+
+constexpr int kNumSMs = 148;
+constexpr int kStatePassElems = 512;   // state elements per CTA of the CUDA-core state passes
+constexpr int kTcBlock = 128;     // steps per block of the tensor-core path, whatever (larger) chunk the caller names
+
+// Per (head, block of 128 steps) record of the tensor-core path, made once per segment by the forward chain and copied to
+// shared memory in one piece by every kernel that masks a tile (cs: inclusive cumsum of dt*A in the block, log2 units;
+// sub-tile: 32 steps).  Offsets in floats; the parts a kernel needs are adjacent.
+enum {
+    REC_CFX = 0,        // [128] e^{cs_t - cs[first of t's sub-tile]}
+    REC_BLK = 128,      // [4][4] e^{cs[32 i] - cs[32 j + 31]}, j < i
+    REC_DECAY = 144,    // e^{cs_last}
+    REC_CS = 160,       // [128] cs
+    REC_DT = 288,       // [128] dt
+    REC_CF = 416,       // [128] dt_s e^{cs[last of s's sub-tile] - cs_s}
+    REC_OC = 544,       // [128] e^{cs_t}
+    REC_OB = 672,       // [128] dt_s e^{cs_last - cs_s}
+    REC_FLOATS = 800
+};
+// Up to this many log2 units of decay inside a sub-tile, e^{cs_t - cs_s} on its diagonal is taken as a product of a row and a
+// column factor (one of them > 1, far from overflow) like everywhere else; beyond, element by element.
+constexpr float kMildDecay = 40.f;
 
 struct SegParams {
     int B, L, H, P, N, G, Q;
@@ -43,9 +79,8 @@ struct SegParams {
     int ncs;       // chunk capacity of the workspace (chunks of a full segment)
     int nct;       // chunks in the whole sequence (L / Q)
     int nsl;       // head slices per group in the dB/dC partial buffers
-    int bc_fused;  // 1: the fused dB/dC kernel wrote them: two slots per slice (see ssd_tc_bcf.cu), second parts of rho/psi
-    int ndd;          // partial sums of dD per (head, chunk) that the kernels of this path write (<= 16)
-    int nsplit_scan;  // head ranges per group in the tensor-core scan kernels (no effect on results)
+    int ndd;       // partial sums of dD per (head, chunk) that the kernels of this path write (<= 4)
+    int ngh;       // partial sums of <G,H> per (head, chunk) (<= 16)
     float dx_skip;    // 1 when dx also takes dy (a skip connection around the layer), else 0
     int64_t x_bs, dt_bs, bc_bs;  // batch strides, elements
 
@@ -57,25 +92,26 @@ struct SegParams {
 
     // workspace regions (all fp32 unless noted)
     unsigned int *status;  // [0] = error flag of bounded waits
-    float *cs;             // [B,H,ncs,Q]   inclusive cumsum of dt*A inside each chunk
-    float *dtT;            // [B,H,ncs,Q]   dt transposed to head-major
-    float *Hst;            // [B,ncs+1,H,P,N] slot c = state entering chunk c; slot nc = leaving the segment
-    float *Gst;            // [B,ncs+1,H,P,N] slot c+1 = dLoss/d(state leaving chunk c)
-    __nv_bfloat16 *Hbf;    // [B,ncs+1,H,P,N] bf16 copy of Hst (tensor-core path)
-    __nv_bfloat16 *Gbf;    // [B,ncs+1,H,P,N] bf16 copy of Gst (tensor-core path)
+    float *rec;            // tensor-core path: [B,H,ncs,REC_FLOATS]
+    float *cs;             // CUDA-core path: [B,H,ncs,Q] inclusive cumsum of dt*A inside each chunk
+    float *dtT;            // dt head-major, vector of (b, h, c) at dt_stride floats: [B,H,ncs,Q], or inside the records
+    int dt_stride;
+    float *Hst;            // CUDA-core path: [B,ncs+1,H,P,N] slot c = state entering chunk c; slot nc = leaving the segment
+    float *Gst;            // CUDA-core path: [B,ncs+1,H,P,N] slot c+1 = dLoss/d(state leaving chunk c)
+    __nv_bfloat16 *Hbf;    // tensor-core path: [B,ncs,H,N,P] (transposed) state entering block c
+    __nv_bfloat16 *Gbf;    // tensor-core path: [B,ncs,H,N,P] dLoss/d(state leaving block c)
     float *hcarry;         // [B,H,P,N]     state handed from segment to segment (forward)
     float *gcarry;         // [B,H,P,N]     state gradient handed right-to-left (backward)
     float *ghdot;          // [B,H,ncs,16]  partial sums of exp(cs_last) <Gout_c, H_in,c>
     float *ddt_dir;        // [B,H,ncs,Q]   direct part of ddt
     float *rho;            // [B,H,ncs,Q]   C_t . dC_t of this head (CUDA-core path: all of it; tensor-core
                            //               path: its intra-chunk part)
-    float *rhob, *psib;    // [B,H,ncs,Q]   fused dB/dC kernel: second parts of rho / psi (else NULL)
-    float *rho2;           // [B,H,ncs,Q]   tensor-core path: C_t . (inter-chunk part of this head's dC_t); else NULL
+    float *rho2, *rho2b;   // [B,H,ncs,Q]   tensor-core path: the two halves of C_t . (inter-chunk part of this head's dC_t); else NULL
     float *psi;            // [B,H,ncs,Q]   B_t . (intra-chunk part of this head's dB_t)
     float *psi2;           // [B,H,ncs,Q]   B_t . (inter-chunk part of this head's dB_t)
     float *pB, *pC;        // [B,seg,G,nsl,N] per-head-slice partial dB / dC
     float *dAp;            // [B,H,nct]     per-chunk partial of dA
-    float *dDp;            // [B,H,nct,16]  partials of dD, the first ndd of each group of 16 in use
+    float *dDp;            // [B,H,nct,4]   partials of dD, the first ndd of each group in use
 };
 
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
@@ -87,10 +123,8 @@ cudaError_t launch_chunk_state_simt(const SegParams &p, int dtype, int mode, cud
 // init: state entering the segment (NULL = zeros), batch stride init_bs elements;
 // boundary_out (nullable): where to store that state, batch stride bnd_bs; final_out nullable.
 cudaError_t launch_state_pass_fwd(const SegParams &p, const float *init, long long init_bs,
-                                  float *boundary_out, long long bnd_bs, float *final_out,
-                                  bool want_bf16, cudaStream_t st);
-cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, float *left_out,
-                                  bool want_bf16, cudaStream_t st);
+                                  float *boundary_out, long long bnd_bs, float *final_out, cudaStream_t st);
+cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, float *left_out, cudaStream_t st);
 cudaError_t launch_masked_product_simt(const SegParams &p, int dtype, int mode, cudaStream_t st);
 cudaError_t launch_bwd_finish(const SegParams &p, cudaStream_t st);
 cudaError_t launch_reduce_dbdc(const SegParams &p, int dtype, cudaStream_t st);
@@ -121,23 +155,27 @@ cudaError_t launch_decode_step(int dtype, int N, const void *x, const float *dt,
                                const void *Cm, const float *D, float *h, void *y, int B, int H, int P, int G,
                                long long x_bs, long long dt_bs, long long bc_bs, cudaStream_t st);
 
-// ssd_tc.cu : tensor-core (tcgen05 / TMEM / TMA) kernels, bf16 I/O
+// ssd_tc.cu : tensor maps of the tensor-core (tcgen05 / TMEM / TMA) kernels, bf16 I/O
 struct TcMaps {
-    CUtensorMap x, dy, Bm, Cm;  // [B][L][H*64] / [B][L][G*128], box 64 x 128 rows
-    CUtensorMap y, dx;          // outputs, same geometry as x; box 64 columns x 32 rows (TMA stores)
-    CUtensorMap Hbf, Gbf;       // bf16 chunk states as [rows][128], box 64 x 64 rows
+    CUtensorMap x, dy, Bm, Cm;  // [B][L][H*64] / [B][L][G*N], box 64 x 128 rows
+    CUtensorMap y, dx;          // outputs, same geometry as x
+    CUtensorMap H, G;           // bf16 states as [rows][64], box 64 x N rows
+    CUtensorMap Hst, Gst;       // the same for the stores of the chain kernels: box 32 x 32 rows, 64-byte swizzle
 };
-bool tc_supported(int dtype, int flags, int P, int N, int Q, int hpg);
+bool tc_supported(int dtype, int flags, int P, int N, int Q);
 bool tc_make_maps(const SegParams &p, TcMaps &m);
-cudaError_t launch_chunk_state_tc(const SegParams &p, const TcMaps &m, int mode, cudaStream_t st);
-// ssd_tc_scan.cu : y (SC_FWD) or dx, ddt_direct, dD partials (SC_DX)
+// ssd_tc_chain.cu : block sums and the recurrence over the blocks.  init: state (gradient) entering the segment (NULL = zeros),
+// batch stride init_bs; boundary_out (nullable): where to store that state, batch stride bnd_bs; final_out nullable.
+enum { CHAIN_FWD = 0, CHAIN_BWD = 1 };
+cudaError_t launch_chain_fwd(const SegParams &p, const TcMaps &m, const float *init, long long init_bs, float *boundary_out, long long bnd_bs,
+                             float *final_out, cudaStream_t st);
+cudaError_t launch_chain_bwd(const SegParams &p, const TcMaps &m, const float *init, float *left_out, cudaStream_t st);
+// ssd_tc_scan.cu : y (SC_FWD) or dx, ddt_direct, dD partials, psi2 (SC_DX)
 cudaError_t launch_scan_tc(const SegParams &p, const TcMaps &m, int mode, cudaStream_t st);
 enum { SC_FWD = 0, SC_DX = 1 };
-// ssd_tc_bc.cu : per-slice partial dC, rho (GB_DC) or partial dB, psi, psi2 (GB_DB)
-cudaError_t launch_grad_bc_tc(const SegParams &p, const TcMaps &m, int mode, cudaStream_t st);
-enum { GB_DC = 0, GB_DB = 1 };
-// ssd_tc_bcf.cu : dB and dC from one masked tile (partial slices, rho, psi and their second parts)
-cudaError_t launch_grad_bc_fused(const SegParams &p, const TcMaps &m, cudaStream_t st);
+// ssd_tc_bcf.cu : partial slices of dC and rho (BC_DC), of dB and psi (BC_DB), or both from one masked tile
+cudaError_t launch_grad_bc(const SegParams &p, const TcMaps &m, int what, cudaStream_t st);
+enum { BC_DC = 1, BC_DB = 2 };
 
 enum { STATE_MODE_FWD = 0, STATE_MODE_DSTATE = 1 };
 // kernel kinds, for the launch counter and the optional per-kind timing

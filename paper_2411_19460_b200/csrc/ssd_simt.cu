@@ -14,6 +14,7 @@
 // under the large kernels was hidden already.
 #define SP_THREADS 128
 #define SP_ELEMS (SP_THREADS * 4)
+static_assert(SP_ELEMS == ssd::kStatePassElems, "one partial of <G,H> per CTA of the backward pass");
 #ifndef SP_BWD_CTAS
 #define SP_BWD_CTAS 10
 #define SP_BWD_PF 4
@@ -168,7 +169,7 @@ cudaError_t launch_chunk_state_simt(const SegParams &p, int dtype, int mode, cud
 // segment-exit state to the next segment through hcarry.
 __global__ void __launch_bounds__(SP_THREADS, SP_FWD_CTAS)
 k_state_pass_fwd(SegParams p, const float *init, long long init_bs, float *boundary_out,
-                 long long bnd_bs, float *final_out, int want_bf16) {
+                 long long bnd_bs, float *final_out) {
     pdl_launch_dependents();
     pdl_wait();
     const int h = blockIdx.y, b = blockIdx.z;
@@ -180,19 +181,7 @@ k_state_pass_fwd(SegParams p, const float *init, long long init_bs, float *bound
     if (boundary_out)
         *reinterpret_cast<float4 *>(boundary_out + (size_t)b * bnd_bs + (size_t)h * PN + e) = carry;
     const float *csl = p.cs + vec_off(p, b, h, 0) + (p.Q - 1);
-    // tensor-core path: every later reader takes the bf16 copy, so the fp32 chunk-entry states are
-    // not written back (the fp32 carry still goes from segment to segment)
-    auto put = [&](size_t so, const float4 &v) {
-        if (!want_bf16) *reinterpret_cast<float4 *>(p.Hst + so) = v;
-        if (want_bf16) {
-            __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
-            __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
-            uint2 pk;
-            pk.x = *reinterpret_cast<unsigned int *>(&lo);
-            pk.y = *reinterpret_cast<unsigned int *>(&hi);
-            *reinterpret_cast<uint2 *>(p.Hbf + so) = pk;
-        }
-    };
+    auto put = [&](size_t so, const float4 &v) { *reinterpret_cast<float4 *>(p.Hst + so) = v; };
     put(slot_off(p, b, 0, h) + e, carry);
     // The chunk sums and decays do not depend on the carry: fetch eight chunks ahead of the serial
     // recurrence, so that a segment costs a few memory latencies instead of one per chunk.
@@ -222,10 +211,9 @@ k_state_pass_fwd(SegParams p, const float *init, long long init_bs, float *bound
 }
 
 cudaError_t launch_state_pass_fwd(const SegParams &p, const float *init, long long init_bs,
-                                  float *boundary_out, long long bnd_bs, float *final_out,
-                                  bool want_bf16, cudaStream_t st) {
+                                  float *boundary_out, long long bnd_bs, float *final_out, cudaStream_t st) {
     dim3 grid(p.P * p.N / SP_ELEMS, p.H, p.B);
-    return launch_pdl(k_state_pass_fwd, grid, dim3(SP_THREADS), 0, st, p, init, init_bs, boundary_out, bnd_bs, final_out, want_bf16 ? 1 : 0);
+    return launch_pdl(k_state_pass_fwd, grid, dim3(SP_THREADS), 0, st, p, init, init_bs, boundary_out, bnd_bs, final_out);
 }
 
 // ------------------------------------------------------------------ backward state passing
@@ -234,7 +222,7 @@ cudaError_t launch_state_pass_fwd(const SegParams &p, const float *init, long lo
 // the partial sums of exp(cs_last,c) <Gout_c, H_in,c> (one per CTA, summed later in a fixed order):
 // the part of da_t that couples the gradient from the right with the state from the left.
 __global__ void __launch_bounds__(SP_THREADS, SP_BWD_CTAS)
-k_state_pass_bwd(SegParams p, const float *init, float *left_out, int want_bf16) {
+k_state_pass_bwd(SegParams p, const float *init, float *left_out) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ float red[SP_BWD_PF][SP_THREADS / 32];
@@ -246,17 +234,7 @@ k_state_pass_bwd(SegParams p, const float *init, float *left_out, int want_bf16)
     float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);
     if (init) carry = *reinterpret_cast<const float4 *>(init + bh);
     const float *csl = p.cs + vec_off(p, b, h, 0) + (p.Q - 1);
-    auto put = [&](size_t so, const float4 &v) {
-        if (!want_bf16) *reinterpret_cast<float4 *>(p.Gst + so) = v;
-        if (want_bf16) {
-            __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y);
-            __nv_bfloat162 hi = __floats2bfloat162_rn(v.z, v.w);
-            uint2 pk;
-            pk.x = *reinterpret_cast<unsigned int *>(&lo);
-            pk.y = *reinterpret_cast<unsigned int *>(&hi);
-            *reinterpret_cast<uint2 *>(p.Gbf + so) = pk;
-        }
-    };
+    auto put = [&](size_t so, const float4 &v) { *reinterpret_cast<float4 *>(p.Gst + so) = v; };
     put(slot_off(p, b, p.nc, h) + e, carry);
     // Eight chunks at a time: their E_c, entry states and decays are fetched ahead of the serial
     // recurrence; the eight <Gout, H_in> partials of a batch share one block-wide reduction step.
@@ -269,14 +247,7 @@ k_state_pass_bwd(SegParams p, const float *init, float *left_out, int want_bf16)
             if (c0 - k >= 0) {
                 const size_t so = slot_off(p, b, c0 - k, h) + e;
                 ev[k] = *reinterpret_cast<const float4 *>(p.Gst + so);
-                if (want_bf16) {   // entry state from its bf16 copy (the fp32 one was not kept)
-                    const uint2 pk = *reinterpret_cast<const uint2 *>(p.Hbf + so);
-                    const float2 lo = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&pk.x));
-                    const float2 hi = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&pk.y));
-                    hv[k] = make_float4(lo.x, lo.y, hi.x, hi.y);
-                } else {
-                    hv[k] = *reinterpret_cast<const float4 *>(p.Hst + so);
-                }
+                hv[k] = *reinterpret_cast<const float4 *>(p.Hst + so);
                 dec[k] = csl[(size_t)(c0 - k) * p.Q];
             }
 #pragma unroll
@@ -309,10 +280,9 @@ k_state_pass_bwd(SegParams p, const float *init, float *left_out, int want_bf16)
     *reinterpret_cast<float4 *>(left_out + bh) = carry;
 }
 
-cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, float *left_out,
-                                  bool want_bf16, cudaStream_t st) {
+cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, float *left_out, cudaStream_t st) {
     dim3 grid(p.P * p.N / SP_ELEMS, p.H, p.B);
-    return launch_pdl(k_state_pass_bwd, grid, dim3(SP_THREADS), 0, st, p, init, left_out, want_bf16 ? 1 : 0);
+    return launch_pdl(k_state_pass_bwd, grid, dim3(SP_THREADS), 0, st, p, init, left_out);
 }
 
 // ------------------------------------------------------------------ masked products y, dx, dB, dC (FFMA)
@@ -540,7 +510,7 @@ __global__ void __launch_bounds__(256) k_masked_product_simt(SegParams p) {
             float s = 0.f;
 #pragma unroll
             for (int w = 0; w < 8; ++w) s += Mk[w];
-            p.dDp[((((size_t)b * p.H + h) * p.nct + p.c0 + c) << 4) + rt] = s;
+            p.dDp[((((size_t)b * p.H + h) * p.nct + p.c0 + c) << 2) + rt] = s;
         }
     } else {
         // per-head partial dC / dB rows: [B, seg, G, nsl, N]
@@ -626,19 +596,16 @@ __global__ void __launch_bounds__(HB * 32) k_bwd_finish(SegParams p) {
     const int c = blockIdx.x, h = blockIdx.y * HB + warp, b = blockIdx.z;
     const int Q = p.Q, per = Q >> 5;
     const size_t vo = vec_off(p, b, h, c) + (size_t)lane * per;
-    const int ngh = p.P * p.N / SP_ELEMS;       // partial sums per (head, chunk): one per CTA of the backward state pass
     float gh = 0.f;
-    for (int i = 0; i < ngh; ++i) gh += p.ghdot[((((size_t)b * p.H + h) * p.ncs + c) << 4) + i];
+    for (int i = 0; i < p.ngh; ++i) gh += p.ghdot[((((size_t)b * p.H + h) * p.ncs + c) << 4) + i];
     float dtv[8], dd[8], sfx[8], pfx[8];
     float run = 0.f;
 #pragma unroll
     for (int j = 7; j >= 0; --j)
         if (j < per) {
-            dtv[j] = p.dtT[vo + j];
+            dtv[j] = p.dtT[(((size_t)b * p.H + h) * p.ncs + c) * p.dt_stride + lane * per + j];
             dd[j] = p.ddt_dir[vo + j];
-            const float rh = p.rhob ? p.rho[vo + j] + p.rhob[vo + j] : p.rho[vo + j];
-            const float ps = p.psib ? p.psi[vo + j] + p.psib[vo + j] : p.psi[vo + j];
-            run += (rh - ps) + (p.rho2 ? p.rho2[vo + j] : 0.f);
+            run += (p.rho[vo + j] - p.psi[vo + j]) + (p.rho2 ? p.rho2[vo + j] + p.rho2b[vo + j] : 0.f);
             sfx[j] = run;
         }
     float incl = run;
@@ -698,7 +665,7 @@ cudaError_t launch_bwd_finish(const SegParams &p, cudaStream_t st) {
 
 // ------------------------------------------------------------------ dB / dC: sum the head slices of a group
 // Four consecutive n per thread (16-byte loads of the fp32 partial slices, one 8- or 16-byte store): the kernel only
-// moves bytes.  The order of the additions per element is fixed: slices in order, a slice's first slot before its second.
+// moves bytes.  The order of the additions per element is fixed: slices in order.
 __device__ __forceinline__ void add4(float4 &a, const float4 &b) {
     a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
 }
@@ -729,23 +696,10 @@ __global__ void __launch_bounds__(256) k_reduce_dbdc(SegParams p) {
     const size_t segcap = (size_t)p.ncs * p.Q;
     float4 sB = make_float4(0.f, 0.f, 0.f, 0.f), sC = sB;
     auto ld = [](const float *q) { return *reinterpret_cast<const float4 *>(q); };
-    if (p.bc_fused) {
-        // two slots per slice; the second exists only for dC rows of the upper half of a chunk and dB rows
-        // of the lower half (the rows that two tiles of the causal triangle contribute to)
-        const bool upper = ((tl % (size_t)p.Q) >= (size_t)(p.Q / 2));
-        const size_t src2 = ((((size_t)b * segcap + tl) * p.G + g) * (2 * p.nsl)) * p.N + n;
-        for (int s = 0; s < p.nsl; ++s) {
-            add4(sB, ld(p.pB + src2 + (size_t)(2 * s) * p.N));
-            if (!upper) add4(sB, ld(p.pB + src2 + (size_t)(2 * s + 1) * p.N));
-            add4(sC, ld(p.pC + src2 + (size_t)(2 * s) * p.N));
-            if (upper) add4(sC, ld(p.pC + src2 + (size_t)(2 * s + 1) * p.N));
-        }
-    } else {
-        const size_t src = ((((size_t)b * segcap + tl) * p.G + g) * p.nsl) * p.N + n;
-        for (int s = 0; s < p.nsl; ++s) {
-            add4(sB, ld(p.pB + src + (size_t)s * p.N));
-            add4(sC, ld(p.pC + src + (size_t)s * p.N));
-        }
+    const size_t src = ((((size_t)b * segcap + tl) * p.G + g) * p.nsl) * p.N + n;
+    for (int s = 0; s < p.nsl; ++s) {
+        add4(sB, ld(p.pB + src + (size_t)s * p.N));
+        add4(sC, ld(p.pC + src + (size_t)s * p.N));
     }
     const size_t dst = (size_t)b * p.bc_bs + ((size_t)p.t0 + tl) * p.G * p.N + (size_t)g * p.N + n;
     st4((T *)p.dB + dst, sB);
@@ -771,7 +725,7 @@ __global__ void __launch_bounds__(32) k_final_dAdD(SegParams p, float *dA, float
         const size_t base = ((size_t)b * p.H + h) * p.nct;
         for (int c = lane; c < p.nct; c += 32) {
             sA += (double)p.dAp[base + c];
-            for (int r = 0; r < nrt; ++r) sD += (double)p.dDp[((base + c) << 4) + r];
+            for (int r = 0; r < nrt; ++r) sD += (double)p.dDp[((base + c) << 2) + r];
         }
     }
 #pragma unroll

@@ -33,16 +33,19 @@ __device__ __forceinline__ void mbar_arrive_expect_tx(uint64_t *bar, uint32_t by
 __device__ __forceinline__ void mbar_arrive(uint64_t *bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// Returns whether the phase is complete; the hardware suspends the warp until it is or the time hint is over, so that a
+// waiting warp takes no issue slots.
+constexpr uint32_t kSuspendNs = 1000000;
 __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     uint32_t ok;
     asm volatile(
         "{\n"
         ".reg .pred p;\n"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
         "selp.u32 %0, 1, 0, p;\n"
         "}\n"
         : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity)
+        : "r"(smem_u32(bar)), "r"(parity), "r"(kSuspendNs)
         : "memory");
     return ok != 0;
 }
@@ -58,16 +61,11 @@ constexpr long long kWaitAbortedClk = 4000000ll;     // about 2 ms once aborted
 __device__ __forceinline__ bool mbar_wait_limited(uint64_t *bar, uint32_t parity, volatile uint32_t *abort_flag,
                                                   unsigned int *status, long long limit_clk) {
     if (mbar_try_wait(bar, parity)) return true;
-    // Not complete yet: poll with a short sleep in between, so that the waiting warps of a CTA do not
-    // flood the shared-memory pipe (every poll is a shared-memory access) that the MMAs read from.
     const long long start = clock64();
     const long long limit = (*abort_flag) ? kWaitAbortedClk : limit_clk;
-    uint32_t it = 0;
-    while (true) {
-        __nanosleep(20);
+    do {
         if (mbar_try_wait(bar, parity)) return true;
-        if ((++it & 255u) == 0 && clock64() - start > limit) break;
-    }
+    } while (clock64() - start <= limit);
     *abort_flag = 1u;
     atomicExch(status, 1u);
     return false;
@@ -75,6 +73,15 @@ __device__ __forceinline__ bool mbar_wait_limited(uint64_t *bar, uint32_t parity
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volatile uint32_t *abort_flag,
                                           unsigned int *status) {
     return mbar_wait_limited(bar, parity, abort_flag, status, kWaitLimitClk);
+}
+
+// True in one lane of a converged warp.  The single-thread roles branch on this and not on a lane number: the compiler then
+// knows that one thread is left and keeps descriptors in uniform registers (an MMA with N = 64 issues every 49-64 cycles
+// instead of every 82).
+__device__ __forceinline__ bool elect_one() {
+    uint32_t pred;
+    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(pred));
+    return pred != 0;
 }
 
 // ---------------------------------------------------------------- fences
@@ -124,6 +131,8 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, const void *s
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // all earlier stores of this thread have finished READING their shared-memory source
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
+// all but the latest store group have
+__device__ __forceinline__ void tma_store_wait_read_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 // all earlier stores of this thread are complete
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
@@ -230,6 +239,17 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *v) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// 32 lanes x 16 consecutive 32-bit columns, registers -> TMEM; complete (for this thread) after tmem_st_wait().
+__device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t *r) {
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%0], "
+        "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};" ::"r"(taddr),
+        "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]), "r"(r[9]), "r"(r[10]),
+        "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])
+        : "memory");
+}
+__device__ __forceinline__ void tmem_st_wait() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
 // ---------------------------------------------------------------- UMMA descriptors
 // Shared-memory matrix descriptor, 128-byte swizzle.  Operand tiles are stored as rows of 128 bytes
 // (64 bf16), 8 rows per 1024-byte swizzle atom, exactly what a SWIZZLE_128B TMA box of 64 elements
@@ -306,6 +326,18 @@ __device__ __forceinline__ void umma_bf16_fixed(uint32_t d_tmem, uint64_t adesc,
             "}\n" ::"r"(d_tmem),
             "l"(adesc), "l"(bdesc), "r"(idesc)
             : "memory");
+}
+// The same with the A operand in tensor memory: lane = row, two bf16 per 32-bit column, 16 elements of K = 8 columns.
+template <bool ACCUMULATE>
+__device__ __forceinline__ void umma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, uint64_t bdesc, uint32_t idesc) {
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "setp.ne.b32 p, %4, 0;\n"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n"
+        "}\n" ::"r"(d_tmem),
+        "r"(a_tmem), "l"(bdesc), "r"(idesc), "n"(ACCUMULATE ? 1 : 0)
+        : "memory");
 }
 __device__ __forceinline__ uint64_t umma_desc_words(uint32_t lo, uint32_t hi) {
     return ((uint64_t)hi << 32) | (uint64_t)lo;

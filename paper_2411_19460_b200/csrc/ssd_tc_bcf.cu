@@ -1,25 +1,22 @@
-// Tensor-core kernel for dB and dC together (bf16 I/O, P = 64, N = 128, Q = 256).  Both are products of
+// Tensor-core kernel for dB and dC (bf16 I/O, P = 64, N = 64 or 128), over blocks of T = 128 steps.  Both are products of
 // the same masked, per-head score tile
 //     W_h[t,s] = (dy_t . x_s) e^{cs_t-cs_s} dt_s   (s <= t),
-//   dC_t = sum_h [ sum_s W_h[t,s] B_s + e^{cs_t} dy_t^T H_in ]               (W as the K-major A operand)
-//   dB_s = sum_h [ sum_t W_h[t,s] C_t + dt_s e^{cs_last-cs_s} x_s^T Gout ]   (W as the MN-major A operand)
-// so a CTA masks one 128 x 128 tile of W per head and feeds it to both products.  Per head it also forms
-// the scalars of the decay gradient, rho_t = sum_s W[t,s] (C_t.B_s) and psi_s = sum_t W[t,s] (C_t.B_s):
-// row and column sums of one fp32 matrix.  (Eq. 1 of the paper regrouped by chunks; cs = inclusive cumsum
-// of dt*A inside the chunk.)
+//   dC_t = sum_h [ sum_s W_h[t,s] B_s + e^{cs_t} dy_t^T H_in ]
+//   dB_s = sum_h [ sum_t W_h[t,s] C_t + dt_s e^{cs_last-cs_s} x_s^T Gout ]
+// and both are linear in it, so a CTA, which owns (block, group, a range of the group's heads), masks the tile once per
+// head, adds it to a head sum kept in fp32 registers, and after the last head rounds the sum once and multiplies it by B
+// and by C.  Per head it also forms the scalars of the decay gradient, rho_t = sum_s W[t,s] (C_t.B_s) and
+// psi_s = sum_t W[t,s] (C_t.B_s): row and column sums of one fp32 matrix.  (Eq. 1 of the paper regrouped by blocks; cs =
+// inclusive cumsum of dt*A inside the block.)
 //
-// One CTA owns (chunk, tile, group, a range of the group's heads); the three causal tiles of a 256-step
-// chunk are (t-block, s-block) = (1,0) full, (0,0) and (1,1) diagonal.  TMEM holds CB = C B^T of the tile
-// (128 columns), the score buffer (128), and the two accumulators (128 each), which stay there across all
-// heads of the CTA and leave once, as fp32 partial slices that a later kernel adds in a fixed order.
-// Shared memory holds the C rows of the t-block and the B rows of the s-block for the whole CTA (operands
-// of CB, and the MN-major B operands of the two products), and per head the dy / x rows (double buffered),
-// one buffer for the scaled rows of an inter-chunk term, and the two bf16 chunk states (double buffered: the
-// second copies live where the head sum of W goes at the very end, which is free until then, so a state's
-// load has a whole head of time to land).
-// The inter-chunk terms are spread over the tiles: (0,0) adds dC's for t-block 0, (1,0) dB's for s-block 0,
-// (1,1) dC's for t-block 1 and then dB's for s-block 1.
-//   warp 0 producer (TMA) | warp 1 MMA issuer | warps 2..17 mask warps | warp 18 per-head vectors
+// Of the 16 32 x 32 sub-tiles of the tile ten are not above the diagonal: ten mask warps own one each for the whole CTA,
+// with its part of C B^T and of the head sum in registers (32 + 32), so that a head costs a warp one tensor-memory load
+// and its arithmetic.  A warp can only read the 32 tensor-memory lanes of its own quarter, so sub-tile (q, r) belongs to
+// warp 4 r + q, r <= q, and the six warps in between have the other roles:
+//   warp 4 producer (TMA) | warp 8 MMA issuer | warp 12 rho / psi out | warps 9, 13, 14 row scaling
+// Tensor memory: two score buffers and the two accumulators, 128 columns each.  The rows of a head are scaled in place for
+// the inter-block terms once its scores have been multiplied, and both terms go straight into the accumulators.
+// Bound by the instruction issue of the scheduler that holds the four sub-tiles of row quarter 3.
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
 
@@ -29,21 +26,19 @@ using namespace sm100;
 
 namespace {
 
-constexpr int GF_THREADS = 608;
-constexpr uint32_t GF_OFF_CT = 0;          // 32 KB  C rows of the t-block  [n-half][128 rows][128 B]
-constexpr uint32_t GF_OFF_BT = 32768;      // 32 KB  B rows of the s-block
-constexpr uint32_t GF_OFF_R = 65536;       // 2 x (dy rows of the t-block 16 KB | x rows of the s-block 16 KB)
-constexpr uint32_t GF_OFF_W = 131072;      // 32 KB  head sum of the masked tiles [s-half][128 t rows][128 B]; until then: states of odd heads
-constexpr uint32_t GF_OFF_SC = 163840;     // 16 KB  scaled rows of an inter-chunk term
-constexpr uint32_t GF_OFF_ST = 180224;     // 2 x 16 KB  bf16 chunk states (entering: H, gradient leaving: G) of even heads
-constexpr uint32_t GF_OFF_VEC = 212992;    // per-head vectors, double buffered
-constexpr uint32_t GF_VEC_FLOATS = 256 * 3 + 64;
-constexpr uint32_t GF_OFF_PART = GF_OFF_VEC + 2 * GF_VEC_FLOATS * 4;   // [head parity][rho: 4 slices x 128 rows | psi: 4 quarters x 128 cols]
-constexpr uint32_t GF_SMEM = GF_OFF_PART + 2 * 1024 * 4 + 1024;
+constexpr int GF_T = 128;
+constexpr int GF_THREADS = 512;
+constexpr int GF_VECS = 3;                        // record buffers; the part used, from the decays to the row scales
+constexpr int GF_REC0 = REC_BLK, GF_VEC_FLOATS = REC_FLOATS - REC_BLK;
 
-constexpr uint32_t TF_CB = 0, TF_S = 128, TF_ACCC = 256, TF_ACCB = 384;
+// Ring of four 32 KB slots: the block's C rows, its B rows (N/64 x 16 KB each), then one head per slot (dy rows 16 KB | x rows
+// 16 KB), then C and B again for the last products | 2 x (H^T | G^T, N x 128 B), at the end the head sum
+constexpr uint32_t GF_OFF_ST = 4 * 32768;
+__host__ __device__ constexpr uint32_t gf_off_vec(int ns) { return GF_OFF_ST + 2 * 2 * (uint32_t)ns * 128; }
+__host__ __device__ constexpr uint32_t gf_off_part(int ns) { return gf_off_vec(ns) + GF_VECS * GF_VEC_FLOATS * 4; }
+__host__ __device__ constexpr uint32_t gf_smem(int ns) { return gf_off_part(ns) + 2 * 1024 * 4 + 1024; }
 
-constexpr float kLog2eF = 1.4426950408889634f;
+constexpr uint32_t TF_ACCC = 256, TF_ACCB = 384;
 
 __device__ __forceinline__ float ex2g(float x) {
     float y;
@@ -60,54 +55,54 @@ __device__ __forceinline__ float2 unpack2g(uint32_t w) {
 
 }  // namespace
 
+// WHAT: BC_DC | BC_DB, or one of them (the cross-check with two launches)
+template <int NS, int WHAT>
 __global__ void __launch_bounds__(GF_THREADS, 1)
-k_grad_bc_fused(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDy,
-                const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmC,
-                const __grid_constant__ CUtensorMap tmH, const __grid_constant__ CUtensorMap tmG) {
+k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDy,
+          const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmH,
+          const __grid_constant__ CUtensorMap tmG) {
+    constexpr bool doC = (WHAT & BC_DC) != 0, doB = (WHAT & BC_DB) != 0;
+    constexpr uint32_t OFF_ST = GF_OFF_ST, ST = NS * 128;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t bar_ld, bar_cb, rfull[2], rempty[2], sfull, sempty, wfull, scfull, scempty, hfull[2], hempty[2],
-        gfull[2], gempty[2], stdone, accfull, vfull[2], vempty[2], pfull[2], pempty[2];
+    __shared__ uint64_t rfull[4], rempty[4], stfull[2], stempty[2], sfull[2], sempty[2], scfull[2], stdone, wfull, accfull, vfull[GF_VECS],
+        vempty[GF_VECS], pfull[2], pempty[2];
     __shared__ uint32_t tmem_base, abort_flag;
 
-    // 1-D grid: all full tiles first (they have the most mask work), then the two diagonal kinds
     const int nc = p.nc, nsl = p.nsl, ny = nsl * p.G;
-    const int third = (int)(gridDim.x / 3), jid = (int)blockIdx.x % third;
-    const int kind = (int)blockIdx.x / third;           // 0: tile (1,0)  1: tile (0,0)  2: tile (1,1)
-    const int tb = (kind == 1) ? 0 : 1, sb = (kind == 2) ? 1 : 0;
-    const bool diag = (tb == sb);
-    const bool doC = (kind != 0);                       // adds dC's inter-chunk term of its t-block
-    const bool doB = (kind != 1);                       // adds dB's inter-chunk term of its s-block
-    const int c = jid % nc, yid = (jid / nc) % ny, b = jid / (nc * ny);
+    const int c = (int)blockIdx.x % nc, yid = ((int)blockIdx.x / nc) % ny, b = (int)blockIdx.x / (nc * ny);
     const int g = yid / nsl, sl = yid % nsl;
     const int hps = (p.hpg + nsl - 1) / nsl;
     const int h_begin = g * p.hpg + sl * hps;
-    const int h_end = min(g * p.hpg + p.hpg, h_begin + hps);
-    const int nheads = max(h_end - h_begin, 0);
+    const int nheads = min(p.hpg - sl * hps, hps);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tok0 = p.t0 + c * 256;
+    const int q = warp & 3, sr = warp >> 2;         // tensor-memory quarter; column sub-tile
+    const uint32_t tlane = (uint32_t)(q * 32) << 16;
+    const int tok0 = p.t0 + c * GF_T;
+    unsigned char *vecs = smem + gf_off_vec(NS);
+    auto record = [&](int vb) { return reinterpret_cast<const float *>(vecs) + vb * GF_VEC_FLOATS - GF_REC0; };
+    float *parts = reinterpret_cast<float *>(smem + gf_off_part(NS));      // [head parity][rho: 4 sub-tiles x 128 | psi: 4 quarters x 128]
 
     if (tid == 0) {
-        mbar_init(&bar_ld, 1);
-        mbar_init(&bar_cb, 1);
-        for (int i = 0; i < 2; ++i) {
+        for (int i = 0; i < 4; ++i) {
             mbar_init(&rfull[i], 1);
-            mbar_init(&rempty[i], 1 + 16);    // the head's MMAs (one commit) + the mask warps that scaled its rows
-            mbar_init(&vfull[i], 1);
-            mbar_init(&vempty[i], 16);
-            mbar_init(&pfull[i], 16);         // the mask warps' partial sums of rho / psi of a head
-            mbar_init(&pempty[i], 1);
-            mbar_init(&hfull[i], 1);
-            mbar_init(&hempty[i], 1);
-            mbar_init(&gfull[i], 1);
-            mbar_init(&gempty[i], 1);
+            mbar_init(&rempty[i], 1);
         }
-        mbar_init(&sfull, 1);
-        mbar_init(&sempty, 16);
-        mbar_init(&wfull, 16);
-        mbar_init(&scfull, 16);
-        mbar_init(&scempty, 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&stfull[i], 1);
+            mbar_init(&stempty[i], 1);
+            mbar_init(&sfull[i], 1);
+            mbar_init(&sempty[i], 10);
+            mbar_init(&scfull[i], 3);
+            mbar_init(&pfull[i], 10);
+            mbar_init(&pempty[i], 1);
+        }
+        for (int i = 0; i < GF_VECS; ++i) {
+            mbar_init(&vfull[i], 1);
+            mbar_init(&vempty[i], 10 + 3);
+        }
         mbar_init(&stdone, 1);
+        mbar_init(&wfull, 10);
         mbar_init(&accfull, 1);
         abort_flag = 0;
         fence_barrier_init();
@@ -121,421 +116,312 @@ k_grad_bc_fused(SegParams p, const __grid_constant__ CUtensorMap tmX, const __gr
     const uint32_t tm = tmem_base;
     volatile uint32_t *abortp = &abort_flag;
 
-    if (warp == 0) {
+    if (warp == 4) {
         // ------------------------------------------------------------ producer
-        if (lane == 0 && nheads > 0) {
-            mbar_arrive_expect_tx(&bar_ld, 65536u);
-            for (int nh = 0; nh < 2; ++nh) {
-                tma_load_3d(smem + GF_OFF_CT + nh * 16384, &tmC, &bar_ld, g * 128 + nh * 64, tok0 + tb * 128, b);
-                tma_load_3d(smem + GF_OFF_BT + nh * 16384, &tmB, &bar_ld, g * 128 + nh * 64, tok0 + sb * 128, b);
-            }
-            const int rowH = (b * (p.ncs + 1) + c) * p.H, rowG = (b * (p.ncs + 1) + c + 1) * p.H;
-            for (int hi = 0; hi < nheads; ++hi) {
-                const int h = h_begin + hi, rbuf = hi & 1;
-                if (hi >= 2) mbar_wait(&rempty[rbuf], ((hi >> 1) - 1) & 1, abortp, p.status);
-                mbar_arrive_expect_tx(&rfull[rbuf], 32768);
-                tma_load_3d(smem + GF_OFF_R + rbuf * 32768, &tmDy, &rfull[rbuf], h * 64, tok0 + tb * 128, b);
-                tma_load_3d(smem + GF_OFF_R + rbuf * 32768 + 16384, &tmX, &rfull[rbuf], h * 64, tok0 + sb * 128, b);
-                unsigned char *stb = smem + (rbuf ? GF_OFF_W : GF_OFF_ST);   // states of odd heads: the spare buffer
-                if (doC) {
-                    if (hi >= 2) mbar_wait(&hempty[rbuf], ((hi >> 1) - 1) & 1, abortp, p.status);
-                    mbar_arrive_expect_tx(&hfull[rbuf], 16384);
-                    tma_load_3d(stb, &tmH, &hfull[rbuf], 0, (rowH + h) * 64, 0);
-                    tma_load_3d(stb + 8192, &tmH, &hfull[rbuf], 64, (rowH + h) * 64, 0);
+        if (elect_one()) {
+            // entry e of the ring: 0 C, 1 B, 2 + h head h, 2 + nheads C, 3 + nheads B
+            auto load_entry = [&](int e) {
+                const int slot = e & 3, hi = e - 2;
+                unsigned char *rb = smem + slot * 32768;
+                if (e >= 4) mbar_wait(&rempty[slot], ((e >> 2) - 1) & 1, abortp, p.status);
+                if (hi >= 0 && hi < nheads) {
+                    mbar_arrive_expect_tx(&rfull[slot], 32768);
+                    tma_load_3d(rb, &tmDy, &rfull[slot], (h_begin + hi) * 64, tok0, b);
+                    tma_load_3d(rb + 16384, &tmX, &rfull[slot], (h_begin + hi) * 64, tok0, b);
+                } else {
+                    mbar_arrive_expect_tx(&rfull[slot], NS * 256);
+                    if (e == 0 || hi == nheads) {
+#pragma unroll
+                        for (int nh = 0; nh < NS / 64; ++nh) tma_load_3d(rb + nh * 16384, &tmC, &rfull[slot], g * NS + nh * 64, tok0, b);
+                    } else {
+#pragma unroll
+                        for (int nh = 0; nh < NS / 64; ++nh) tma_load_3d(rb + nh * 16384, &tmB, &rfull[slot], g * NS + nh * 64, tok0, b);
+                    }
                 }
-                if (doB) {
-                    if (hi >= 2) mbar_wait(&gempty[rbuf], ((hi >> 1) - 1) & 1, abortp, p.status);
-                    mbar_arrive_expect_tx(&gfull[rbuf], 16384);
-                    tma_load_3d(stb + 16384, &tmG, &gfull[rbuf], 0, (rowG + h) * 64, 0);
-                    tma_load_3d(stb + 16384 + 8192, &tmG, &gfull[rbuf], 64, (rowG + h) * 64, 0);
-                }
+            };
+            const int strow = (b * p.ncs + c) * p.H;
+            load_entry(0);
+            load_entry(1);
+            load_entry(2);
+            for (int hi = 0; hi < nheads; ++hi) {      // rows run one head ahead of the states, which have two buffers
+                const int bf = hi & 1;
+                unsigned char *sb = smem + OFF_ST + bf * 2 * ST;
+                const int vb = hi % GF_VECS;
+                if (hi >= GF_VECS) mbar_wait(&vempty[vb], (hi / GF_VECS - 1) & 1, abortp, p.status);
+                mbar_arrive_expect_tx(&vfull[vb], GF_VEC_FLOATS * 4);
+                bulk_load(vecs + vb * GF_VEC_FLOATS * 4, p.rec + (((size_t)b * p.H + h_begin + hi) * p.ncs + c) * REC_FLOATS + GF_REC0, GF_VEC_FLOATS * 4,
+                          &vfull[vb]);
+                if (hi >= 2) mbar_wait(&stempty[bf], ((hi >> 1) - 1) & 1, abortp, p.status);
+                mbar_arrive_expect_tx(&stfull[bf], (doC ? ST : 0) + (doB ? ST : 0));
+                if (doC) tma_load_3d(sb, &tmH, &stfull[bf], 0, (strow + h_begin + hi) * NS, 0);
+                if (doB) tma_load_3d(sb + ST, &tmG, &stfull[bf], 0, (strow + h_begin + hi) * NS, 0);
+                load_entry(3 + hi);
             }
+            load_entry(3 + nheads);
         }
-    } else if (warp == 1) {
+    } else if (warp == 8) {
         // ------------------------------------------------------------ MMA issuer
-        if (lane == 0 && nheads > 0) {
-            const uint32_t idKK = umma_idesc_bf16(128, 128, false, false);   // CB and the scores: both operands K-major
-            const uint32_t idKM = umma_idesc_bf16(128, 128, false, true);    // W (K-major) x B rows (MN-major); scaled rows x state
-            const uint32_t idMM = umma_idesc_bf16(128, 128, true, true);     // W^T (MN-major) x C rows (MN-major)
-            // descriptors as (low word, high word): every offset below is a compile-time constant in 16-byte units
-            const uint64_t dCk = umma_desc_sw128(smem_u32(smem + GF_OFF_CT), 16, 1024), dBk = umma_desc_sw128(smem_u32(smem + GF_OFF_BT), 16, 1024);
-            const uint64_t dCm = umma_desc_sw128(smem_u32(smem + GF_OFF_CT), 16384, 1024), dBm = umma_desc_sw128(smem_u32(smem + GF_OFF_BT), 16384, 1024);
-            const uint64_t dRk = umma_desc_sw128(smem_u32(smem + GF_OFF_R), 16, 1024);
-            const uint64_t dWk = umma_desc_sw128(smem_u32(smem + GF_OFF_W), 16, 1024), dWm = umma_desc_sw128(smem_u32(smem + GF_OFF_W), 16384, 1024);
-            const uint64_t dSk = umma_desc_sw128(smem_u32(smem + GF_OFF_SC), 16, 1024);
-            const uint64_t dSt = umma_desc_sw128(smem_u32(smem + GF_OFF_ST), 8192, 1024);
-            const uint64_t dSt1 = umma_desc_sw128(smem_u32(smem + GF_OFF_W), 8192, 1024);    // states of odd heads
-            const uint32_t loCk = (uint32_t)dCk, hiK = (uint32_t)(dCk >> 32), loBk = (uint32_t)dBk;
-            const uint32_t loCm = (uint32_t)dCm, hiM = (uint32_t)(dCm >> 32), loBm = (uint32_t)dBm;
-            const uint32_t loRk = (uint32_t)dRk, loWk = (uint32_t)dWk, loWm = (uint32_t)dWm, loSk = (uint32_t)dSk;
-            const uint32_t loSt0 = (uint32_t)dSt, loSt1 = (uint32_t)dSt1, hiSt = (uint32_t)(dSt >> 32);
-
-            // CB tile, once
-            mbar_wait(&bar_ld, 0, abortp, p.status);
+        if (elect_one()) {
+            const uint32_t idS = umma_idesc_bf16(128, 128, false, false);      // C B^T and the scores: both operands K-major
+            const uint32_t idI = umma_idesc_bf16(128, NS, false, false);       // scaled rows x state (rows n of the transposed state)
+            const uint32_t idC = umma_idesc_bf16(128, NS, false, true), idB = umma_idesc_bf16(128, NS, true, true);
+            const uint32_t s0 = smem_u32(smem);
+            // descriptors as (low word, high word); every offset below is a constant in 16-byte units
+            const uint64_t dCk = umma_desc_sw128(s0, 16, 1024), dCm = umma_desc_sw128(s0, 16384, 1024);
+            const uint32_t loC = (uint32_t)dCk, hiK = (uint32_t)(dCk >> 32), loCm = (uint32_t)dCm, hiM = (uint32_t)(dCm >> 32);
+            const uint32_t loB = loC + 2048, loSt = loC + OFF_ST / 16, loWk = loSt, loWm = loCm + OFF_ST / 16;
+            mbar_wait(&rfull[0], 0, abortp, p.status);
+            mbar_wait(&rfull[1], 0, abortp, p.status);
             tc_fence_after_sync();
 #pragma unroll
-            for (int kk = 0; kk < 8; ++kk) {
-                const uint32_t o = (kk >> 2) * 1024 + (kk & 3) * 2;
-                if (kk == 0) umma_bf16_fixed<false>(tm + TF_CB, umma_desc_words(loCk + o, hiK), umma_desc_words(loBk + o, hiK), idKK);
-                else umma_bf16_fixed<true>(tm + TF_CB, umma_desc_words(loCk + o, hiK), umma_desc_words(loBk + o, hiK), idKK);
+            for (int k = 0; k < NS / 16; ++k) {        // C B^T of the tile, in score buffer 0
+                const uint32_t o = (k >> 2) * 1024 + (k & 3) * 2;
+                if (k == 0) umma_bf16_fixed<false>(tm, umma_desc_words(loC + o, hiK), umma_desc_words(loB + o, hiK), idS);
+                else umma_bf16_fixed<true>(tm, umma_desc_words(loC + o, hiK), umma_desc_words(loB + o, hiK), idS);
             }
-            umma_commit(&bar_cb);
-
-            // scores of head hi: dy rows (t-block) x x rows (s-block)^T, K = P
-            auto issue_scores = [&](int hi) {
-                const int rbuf = hi & 1;
-                mbar_wait(&rfull[rbuf], (hi >> 1) & 1, abortp, p.status);
+            umma_commit(&sfull[0]);
+            umma_commit(&rempty[0]);
+            umma_commit(&rempty[1]);
+            auto scores = [&](int hi) {                // use hi + 1 of the score buffers
+                const int u = hi + 1, bf = u & 1, e = hi + 2, slot = e & 3;
+                mbar_wait(&rfull[slot], (e >> 2) & 1, abortp, p.status);
+                if (u >= 2) mbar_wait(&sempty[bf], ((u >> 1) - 1) & 1, abortp, p.status);
                 tc_fence_after_sync();
-                const uint32_t lo_a = loRk + rbuf * 2048, lo_b = lo_a + 1024;
-                umma_bf16_fixed<false>(tm + TF_S, umma_desc_words(lo_a, hiK), umma_desc_words(lo_b, hiK), idKK);
+                const uint32_t a = loC + slot * 2048, x = a + 1024, d = tm + bf * 128;
+                umma_bf16_fixed<false>(d, umma_desc_words(a, hiK), umma_desc_words(x, hiK), idS);
 #pragma unroll
-                for (int k = 1; k < 4; ++k)
-                    umma_bf16_fixed<true>(tm + TF_S, umma_desc_words(lo_a + k * 2, hiK), umma_desc_words(lo_b + k * 2, hiK), idKK);
-                umma_commit(&sfull);
+                for (int k = 1; k < 4; ++k) umma_bf16_fixed<true>(d, umma_desc_words(a + k * 2, hiK), umma_desc_words(x + k * 2, hiK), idS);
+                umma_commit(&sfull[bf]);
             };
-
-            issue_scores(0);
-            uint32_t scuse = 0;   // uses of the scaled-rows buffer so far
+            scores(0);
             for (int hi = 0; hi < nheads; ++hi) {
-                // inter-chunk terms: scaled rows (K = p) times a chunk state.  A tile's first one is published by the
-                // mask warps before they mask the head, so it is issued first: the scaled-rows buffer is free again
-                // by the time tile (1,1) wants it for its second one.
-                const uint32_t loSt = (hi & 1) ? loSt1 : loSt0;
-                auto inter_dC = [&]() {   // dC += (e^{cs_t} dy_t) H_in
-                    mbar_wait(&hfull[hi & 1], (hi >> 1) & 1, abortp, p.status);
-                    mbar_wait(&scfull, scuse & 1, abortp, p.status);
-                    ++scuse;
-                    tc_fence_after_sync();
+                const int bf = hi & 1;
+                if (hi + 1 < nheads) scores(hi + 1);
+                mbar_wait(&stfull[bf], (hi >> 1) & 1, abortp, p.status);
+                mbar_wait(&scfull[bf], (hi >> 1) & 1, abortp, p.status);
+                tc_fence_after_sync();
+                const int slot = (hi + 2) & 3;
+                const uint32_t a = loC + slot * 2048, st = loSt + bf * (2 * ST / 16);
+                auto inter = [&](uint32_t acc, uint32_t rows, uint32_t state) {
+                    if (hi == 0) umma_bf16_fixed<false>(acc, umma_desc_words(rows, hiK), umma_desc_words(state, hiK), idI);
+                    else umma_bf16_fixed<true>(acc, umma_desc_words(rows, hiK), umma_desc_words(state, hiK), idI);
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint64_t ad = umma_desc_words(loSk + k * 2, hiK), bd = umma_desc_words(loSt + k * 128, hiSt);
-                        if (k == 0 && hi == 0) umma_bf16_fixed<false>(tm + TF_ACCC, ad, bd, idKM);
-                        else umma_bf16_fixed<true>(tm + TF_ACCC, ad, bd, idKM);
-                    }
-                    umma_commit(&scempty);
-                    umma_commit(&hempty[hi & 1]);
+                    for (int k = 1; k < 4; ++k) umma_bf16_fixed<true>(acc, umma_desc_words(rows + k * 2, hiK), umma_desc_words(state + k * 2, hiK), idI);
                 };
-                auto inter_dB = [&](bool first_into_acc) {   // dB += (dt_s e^{cs_last-cs_s} x_s) Gout
-                    mbar_wait(&gfull[hi & 1], (hi >> 1) & 1, abortp, p.status);
-                    mbar_wait(&scfull, scuse & 1, abortp, p.status);
-                    ++scuse;
-                    tc_fence_after_sync();
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const uint64_t ad = umma_desc_words(loSk + k * 2, hiK), bd = umma_desc_words(loSt + 1024 + k * 128, hiSt);
-                        if (k == 0 && first_into_acc) umma_bf16_fixed<false>(tm + TF_ACCB, ad, bd, idKM);
-                        else umma_bf16_fixed<true>(tm + TF_ACCB, ad, bd, idKM);
-                    }
-                    umma_commit(&scempty);
-                    umma_commit(&gempty[hi & 1]);
-                };
-                if (doC) inter_dC();
-                else inter_dB(hi == 0);
-                // next head's scores as soon as the mask warps are done with this head's (they read them last)
-                if (hi + 1 < nheads) {
-                    mbar_wait(&sempty, hi & 1, abortp, p.status);
-                    tc_fence_after_sync();
-                    issue_scores(hi + 1);
-                }
-                if (doC && doB) inter_dB(hi == 0);
-                umma_commit(&rempty[hi & 1]);
+                if (doC) inter(tm + TF_ACCC, a, st);
+                if (doB) inter(tm + TF_ACCB, a + 1024, st + ST / 16);
+                umma_commit(&rempty[slot]);
+                umma_commit(&stempty[bf]);
             }
-            umma_commit(&stdone);     // every product that read a chunk state is done: the spare buffer may take the head sum
-            // the head sum of the masked tiles (made in fp32 by the mask warps, rounded once): both products
+            umma_commit(&stdone);     // nothing reads the states any more: the head sum may take their place
+            const int ec = 2 + nheads, eb = 3 + nheads;
+            const uint32_t loCe = loCm + (ec & 3) * 2048, loBe = loCm + (eb & 3) * 2048;
+            mbar_wait(&rfull[ec & 3], (ec >> 2) & 1, abortp, p.status);
+            mbar_wait(&rfull[eb & 3], (eb >> 2) & 1, abortp, p.status);
             mbar_wait(&wfull, 0, abortp, p.status);
             tc_fence_after_sync();
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {   // dC += Wsum B : K = s
-                const uint64_t ad = umma_desc_words(loWk + (k >> 2) * 1024 + (k & 3) * 2, hiK);
-                const uint64_t bd = umma_desc_words(loBm + k * 128, hiM);
-                if (k == 0 && !doC) umma_bf16_fixed<false>(tm + TF_ACCC, ad, bd, idKM);
-                else umma_bf16_fixed<true>(tm + TF_ACCC, ad, bd, idKM);
-            }
+            for (int k = 0; k < 8; ++k)       // dC += Wsum B, K = s
+                if (doC)
+                    umma_bf16_fixed<true>(tm + TF_ACCC, umma_desc_words(loWk + (k >> 2) * 1024 + (k & 3) * 2, hiK), umma_desc_words(loBe + k * 128, hiM), idC);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {   // dB += Wsum^T C : K = t
-                const uint64_t ad = umma_desc_words(loWm + k * 128, hiM);
-                const uint64_t bd = umma_desc_words(loCm + k * 128, hiM);
-                if (k == 0 && !doB) umma_bf16_fixed<false>(tm + TF_ACCB, ad, bd, idMM);
-                else umma_bf16_fixed<true>(tm + TF_ACCB, ad, bd, idMM);
-            }
+            for (int k = 0; k < 8; ++k)       // dB += Wsum^T C, K = t
+                if (doB)
+                    umma_bf16_fixed<true>(tm + TF_ACCB, umma_desc_words(loWm + k * 128, hiM), umma_desc_words(loCe + k * 128, hiM), idB);
             umma_commit(&accfull);
         }
-    } else if (warp == 18) {
-        // ------------------------------------------------------------ vector warp
-        // Per head: the 256 cumulative sums (log2 units) and step sizes of the chunk, the column factor
-        // e^{cs[s|31] - cs[s]} dt_s of the mask factorisation and the 8 x 8 table of sub-tile-to-sub-tile
-        // decays, written to a double-buffered area one head ahead of the mask warps.
-        if (nheads > 0) {
-            float *vec = reinterpret_cast<float *>(smem + GF_OFF_VEC);
-            // rho / psi of a finished head: the mask warps' partial sums added in a fixed order.  Rows of t-block 1
-            // (columns of s-block 0) are covered by two tiles: the second part goes to rhob (psib), and the tile
-            // that has no partner writes a zero there.
-            auto finish_head = [&](int hj) {
-                const int par = hj & 1;
-                const float *pr = reinterpret_cast<const float *>(smem + GF_OFF_PART) + par * 1024;
-                mbar_wait(&pfull[par], (hj >> 1) & 1, abortp, p.status);
-                const size_t vb = (((size_t)b * p.H + h_begin + hj) * p.ncs + c) << 8;
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int i = k * 32 + lane;
-                    const float er = ((pr[i] + pr[128 + i]) + pr[256 + i]) + pr[384 + i];
-                    const float ep = ((pr[512 + i] + pr[640 + i]) + pr[768 + i]) + pr[896 + i];
-                    const size_t ro = vb + tb * 128 + i, so = vb + sb * 128 + i;
-                    if (kind == 2) p.rhob[ro] = er;
-                    else p.rho[ro] = er;
-                    if (kind == 1) p.rhob[ro] = 0.f;
-                    if (kind == 0) p.psib[so] = ep;
-                    else p.psi[so] = ep;
-                    if (kind == 2) p.psib[so] = 0.f;
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&pempty[par]);
-            };
-            for (int hi = 0; hi < nheads; ++hi) {
-                const int buf = hi & 1, h = h_begin + hi;
-                const size_t vo = ((((size_t)b * p.H + h) * p.ncs + c) << 8) + lane * 8;
-                const float4 c0 = __ldg(reinterpret_cast<const float4 *>(p.cs + vo));
-                const float4 c1 = __ldg(reinterpret_cast<const float4 *>(p.cs + vo + 4));
-                const float4 d0 = __ldg(reinterpret_cast<const float4 *>(p.dtT + vo));
-                const float4 d1 = __ldg(reinterpret_cast<const float4 *>(p.dtT + vo + 4));
-                if (hi >= 2) mbar_wait(&vempty[buf], ((hi >> 1) - 1) & 1, abortp, p.status);
-                float *cs2 = vec + buf * GF_VEC_FLOATS, *cf = cs2 + 256, *dtv = cs2 + 512, *blk = cs2 + 768;
-                const float cv[8] = {c0.x * kLog2eF, c0.y * kLog2eF, c0.z * kLog2eF, c0.w * kLog2eF,
-                                     c1.x * kLog2eF, c1.y * kLog2eF, c1.z * kLog2eF, c1.w * kLog2eF};
-                const float dv[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
-                *reinterpret_cast<float4 *>(cs2 + lane * 8) = make_float4(cv[0], cv[1], cv[2], cv[3]);
-                *reinterpret_cast<float4 *>(cs2 + lane * 8 + 4) = make_float4(cv[4], cv[5], cv[6], cv[7]);
-                *reinterpret_cast<float4 *>(dtv + lane * 8) = d0;
-                *reinterpret_cast<float4 *>(dtv + lane * 8 + 4) = d1;
-                __syncwarp();
-                const float ref = cs2[(lane * 8) | 31];
-                float o[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) o[k] = ex2g(ref - cv[k]) * dv[k];
-                *reinterpret_cast<float4 *>(cf + lane * 8) = make_float4(o[0], o[1], o[2], o[3]);
-                *reinterpret_cast<float4 *>(cf + lane * 8 + 4) = make_float4(o[4], o[5], o[6], o[7]);
-#pragma unroll
-                for (int w = 0; w < 2; ++w) {
-                    const int idx = lane + 32 * w, i = idx >> 3, j = idx & 7;   // blk[i][j] = e^{cs[32 i] - cs[32 j + 31]}, j < i
-                    blk[idx] = (j < i) ? ex2g(cs2[32 * i] - cs2[32 * j + 31]) : 0.f;
-                }
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&vfull[buf]);
-                if (hi >= 1) finish_head(hi - 1);
-            }
-            finish_head(nheads - 1);
-        }
-    } else if (nheads > 0) {
-        // ------------------------------------------------------------ mask warps
-        // Four warps per TMEM lane quarter: warp (q, quar) owns rows 32 q .. 32 q + 31 of the t-block and the
-        // 16-column slice `quar` of both 64-column halves of the tile.
-        const int q = warp & 3;
-        const int quar = (warp - 2) >> 2;
-        const int rl = q * 32 + lane;              // row inside the 128-row block (t for W and dC, s for dB)
-        const int r = tb * 128 + rl;               // t inside the chunk
-        const int rs = sb * 128 + rl;              // s inside the chunk, for the rows this thread scales for dB
-        const int isub = r >> 5;
-        const uint32_t tlane = (uint32_t)(q * 32) << 16;
-        float *vec = reinterpret_cast<float *>(smem + GF_OFF_VEC);
-        uint32_t scuse = 0;
-        float wsum[32];                             // this thread's row of sum_h W_h: columns w * 16 + j of its two slices
-#pragma unroll
-        for (int k = 0; k < 32; ++k) wsum[k] = 0.f;
-
+    } else if (warp == 12) {
+        // ------------------------------------------------------------ rho / psi of a finished head: the mask warps' partial sums
+        // added in a fixed order
+        const size_t vo0 = (((size_t)b * p.H + h_begin) * p.ncs + c) * GF_T, vstep = (size_t)p.ncs * GF_T;
         for (int hi = 0; hi < nheads; ++hi) {
-            float *cs2 = vec + (hi & 1) * GF_VEC_FLOATS, *cf = cs2 + 256, *dtv = cs2 + 512, *blk = cs2 + 768;
-            mbar_wait(&vfull[hi & 1], (hi >> 1) & 1, abortp, p.status);
-            const float csr = cs2[r];
-            const float rowf = ex2g(csr - cs2[r & ~31]);                 // e^{cs_t - cs[first row of t's sub-tile]}
-            const float offsC = ex2g(csr);                                // dC's inter-chunk row scale
-            const float offsB = dtv[rs] * ex2g(cs2[255] - cs2[rs]);       // dB's inter-chunk row scale
-            if (hi == 0) {
-                mbar_wait(&bar_cb, 0, abortp, p.status);
-                tc_fence_after_sync();
+            const float *pr = parts + (hi & 1) * 1024;
+            mbar_wait(&pfull[hi & 1], (hi >> 1) & 1, abortp, p.status);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = k * 32 + lane;
+                float er = pr[i], ep = pr[512 + k * 128 + i];
+#pragma unroll
+                for (int m = 1; m <= k; ++m) er += pr[m * 128 + i];
+#pragma unroll
+                for (int m = k + 1; m < 4; ++m) ep += pr[512 + m * 128 + i];
+                if (doC) p.rho[vo0 + hi * vstep + i] = er;
+                if (doB) p.psi[vo0 + hi * vstep + i] = ep;
             }
-
-            // ---- inter-chunk terms: the head's rows scaled per row, as one more K = P operand (dy rows of the
-            // t-block by e^{cs_t} for dC, x rows of the s-block by dt_s e^{cs_last-cs_s} for dB).  A tile's first one
-            // is published before the masking below, so that its MMAs run while W is being made.
-            auto scale_rows = [&](int which) {
-                const unsigned char *rrow = smem + GF_OFF_R + (hi & 1) * 32768 + which * 16384 + rl * 128;
-                unsigned char *srow = smem + GF_OFF_SC + rl * 128;
-                const float sc = which == 0 ? offsC : offsB;
-                uint4 o[2];
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&pempty[hi & 1]);
+        }
+    } else if (sr > q) {
+        // ------------------------------------------------------------ row scaling (warps 9, 13, 14): dy rows by e^{cs_t}, x rows
+        // by dt_s e^{cs_last-cs_s}, in place, once the head's scores have been multiplied
+        const int th = (warp == 9 ? 0 : warp == 13 ? 1 : 2) * 32 + lane;
+        constexpr int I0 = doC ? 0 : 1024, I1 = doB ? 2048 : 1024;
+        for (int hi = 0; hi < nheads; ++hi) {
+            const int vb = hi % GF_VECS, u = hi + 1, e = hi + 2;
+            const float *sc = record(vb) + REC_OC;          // row scales of dy, then of x
+            mbar_wait(&vfull[vb], (hi / GF_VECS) & 1, abortp, p.status);
+            mbar_wait(&rfull[e & 3], (e >> 2) & 1, abortp, p.status);
+            mbar_wait(&sfull[u & 1], (u >> 1) & 1, abortp, p.status);
+            uint4 *rows = reinterpret_cast<uint4 *>(smem + (e & 3) * 32768);
+            // eight 16-byte pieces in flight per thread: this role is three warps' worth of latency
+            for (int i = I0 + th; i < I1; i += 8 * 96) {
+                uint4 v[8];
+                float f[8];
 #pragma unroll
-                for (int k = 0; k < 2; ++k) {
-                    const uint4 qv = *reinterpret_cast<const uint4 *>(rrow + (((quar * 2 + k) ^ (rl & 7)) << 4));
-                    const uint32_t *qw = reinterpret_cast<const uint32_t *>(&qv);
-                    uint32_t *ow = reinterpret_cast<uint32_t *>(&o[k]);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 f = unpack2g(qw[e]);
-                        ow[e] = pack2g(f.x * sc, f.y * sc);
-                    }
+                for (int k = 0; k < 8; ++k) {
+                    const int j = min(i + k * 96, 2047);
+                    v[k] = rows[j];
+                    f[k] = sc[j >> 3];
                 }
-                if (scuse >= 1) mbar_wait(&scempty, (scuse - 1) & 1, abortp, p.status);
-                ++scuse;
 #pragma unroll
-                for (int k = 0; k < 2; ++k)
-                    *reinterpret_cast<uint4 *>(srow + (((quar * 2 + k) ^ (rl & 7)) << 4)) = o[k];
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&scfull);
-            };
-            mbar_wait(&rfull[hi & 1], (hi >> 1) & 1, abortp, p.status);
-            scale_rows(doC ? 0 : 1);
-
-            // ---- W = score o mask (fp32) for this thread's two 16-column slices, one after the other: added to
-            // the head sum; Z = W o CB gives the row sum (rho) and, through a transposing butterfly over the
-            // warp's 32 rows, the column sums (psi).  The score buffer is released after the second slice.
-            float2 dacc = make_float2(0.f, 0.f);
-            float csum = 0.f;                                // lanes 0..15: column j of slice 0, lanes 16..31: of slice 1
-            mbar_wait(&sfull, hi & 1, abortp, p.status);
-            tc_fence_after_sync();
+                for (int k = 0; k < 8; ++k) {
+                    uint32_t *w = reinterpret_cast<uint32_t *>(&v[k]);
 #pragma unroll
-            for (int w = 0; w < 2; ++w) {
-                const int cb = sb * 128 + w * 64 + quar * 16;   // first column of the slice (s in chunk)
-                const int jsub = cb >> 5;
-                if (diag && (jsub > isub)) continue;            // above the diagonal: W = 0 (uniform over the warp)
-                float vv[16], cbv[16];
-                tmem_ld16_nowait(tm + tlane + TF_S + w * 64 + quar * 16, vv);
-                tmem_ld16_nowait(tm + tlane + TF_CB + w * 64 + quar * 16, cbv);
-                tmem_ld_wait16(vv);
-                if (jsub != isub) {
-                    const float s1 = rowf * blk[isub * 8 + jsub];
-                    const float2 s1v = make_float2(s1, s1);
-#pragma unroll
-                    for (int k = 0; k < 16; k += 4) {
-                        const float4 cv = *reinterpret_cast<const float4 *>(cf + cb + k);
-                        const float2 w0 = __fmul2_rn(make_float2(vv[k], vv[k + 1]), __fmul2_rn(make_float2(cv.x, cv.y), s1v));
-                        const float2 w1 = __fmul2_rn(make_float2(vv[k + 2], vv[k + 3]), __fmul2_rn(make_float2(cv.z, cv.w), s1v));
-                        vv[k] = w0.x; vv[k + 1] = w0.y; vv[k + 2] = w1.x; vv[k + 3] = w1.y;
+                    for (int m = 0; m < 4; ++m) {
+                        const float2 t = __fmul2_rn(unpack2g(w[m]), make_float2(f[k], f[k]));
+                        w[m] = pack2g(t.x, t.y);
                     }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 16; k += 4) {
-                        const float4 cc = *reinterpret_cast<const float4 *>(cs2 + cb + k);
-                        const float4 d4 = *reinterpret_cast<const float4 *>(dtv + cb + k);
-                        const float ccv[4] = {cc.x, cc.y, cc.z, cc.w};
-                        const float dv[4] = {d4.x, d4.y, d4.z, d4.w};
-#pragma unroll
-                        for (int e = 0; e < 4; ++e) {
-                            const bool on = (cb + k + e) <= r;
-                            const float ex = ex2g(csr - ccv[e]) * dv[e];
-                            vv[k + e] = on ? vv[k + e] * ex : 0.f;
-                        }
-                    }
+                    if (i + k * 96 < I1) rows[i + k * 96] = v[k];
                 }
-                tmem_ld_wait16(cbv);
-#pragma unroll
-                for (int k = 0; k < 16; k += 2) {
-                    const float2 wv = make_float2(vv[k], vv[k + 1]);
-                    const float2 a = __fadd2_rn(make_float2(wsum[w * 16 + k], wsum[w * 16 + k + 1]), wv);
-                    wsum[w * 16 + k] = a.x;
-                    wsum[w * 16 + k + 1] = a.y;
-                    const float2 zz = __fmul2_rn(wv, make_float2(cbv[k], cbv[k + 1]));
-                    vv[k] = zz.x;
-                    vv[k + 1] = zz.y;
-                    dacc = __fadd2_rn(dacc, zz);
-                }
-                // column sums of Z over the warp's rows: 16 values -> lane l ends with column l & 15
-#pragma unroll
-                for (int o = 8, cnt = 16; o >= 1; o >>= 1, cnt >>= 1) {
-                    const bool up = (lane & o) != 0;
-#pragma unroll
-                    for (int i = 0; i < cnt / 2; ++i) {
-                        const float send = up ? vv[i] : vv[i + cnt / 2];
-                        const float keep = up ? vv[i + cnt / 2] : vv[i];
-                        vv[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-                    }
-                }
-                const float tot = vv[0] + __shfl_xor_sync(0xffffffffu, vv[0], 16);
-                if ((lane >> 4) == w) csum = tot;
             }
-            tc_fence_before_sync();
+            fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
-                mbar_arrive(&sempty);
-                mbar_arrive(&vempty[hi & 1]);
+                mbar_arrive(&scfull[hi & 1]);
+                mbar_arrive(&vempty[vb]);
             }
-            if (doC && doB) scale_rows(1);     // tile (1,1): its second inter-chunk term
+        }
+    } else {
+        // ------------------------------------------------------------ mask warps: rows t = 32 q + lane, columns 32 sr ..
+        const int rl = q * 32 + lane;
+        const uint32_t tS = tm + tlane + sr * 32;
+        float cb[32], wsum[32];
+        mbar_wait(&sfull[0], 0, abortp, p.status);
+        __syncwarp();
+        tc_fence_after_sync();
+        tmem_ld32(tS, cb);
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sempty[0]);
+#pragma unroll
+        for (int k = 0; k < 32; ++k) wsum[k] = 0.f;
+        for (int hi = 0; hi < nheads; ++hi) {
+            const int vb = hi % GF_VECS, u = hi + 1;
+            const float *rec = record(vb), *cs2 = rec + REC_CS;
+            mbar_wait(&vfull[vb], (hi / GF_VECS) & 1, abortp, p.status);
+            const float csr = cs2[rl], cs_lo = cs2[q * 32], cs_hi = cs2[q * 32 + 31];
+            mbar_wait(&sfull[u & 1], (u >> 1) & 1, abortp, p.status);
             __syncwarp();
-            if (lane == 0) mbar_arrive(&rempty[hi & 1]);     // this warp has read the head's rows
-
-            // ---- rho_t / psi_s: every warp leaves its partial sums (over its 16-column slice / its 32 rows) in
-            // shared memory; the vector warp adds them in a fixed order and writes them out, so no mask warp waits
-            // for another one here
-            {
-                const int par = hi & 1;
-                float *pr = reinterpret_cast<float *>(smem + GF_OFF_PART) + par * 1024;
-                if (hi >= 2) mbar_wait(&pempty[par], ((hi >> 1) - 1) & 1, abortp, p.status);
-                pr[quar * 128 + rl] = dacc.x + dacc.y;
-                const int lc = (lane >> 4) * 64 + quar * 16 + (lane & 15);     // column of the tile this lane holds
-                pr[512 + q * 128 + lc] = csum;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(&pfull[par]);
+            tc_fence_after_sync();
+            float v[32];
+            tmem_ld32(tS + (u & 1) * 128, v);
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sempty[u & 1]);
+            if (sr != q || cs_lo - cs_hi <= kMildDecay) {
+                const float f = sr != q ? ex2g(csr - cs_lo) * rec[REC_BLK + q * 4 + sr] : ex2g(csr - cs_hi);
+                const float2 f2 = make_float2(f, f);
+#pragma unroll
+                for (int k = 0; k < 32; k += 4) {
+                    const float4 cv = *reinterpret_cast<const float4 *>(rec + REC_CF + sr * 32 + k);
+                    const float2 w0 = __fmul2_rn(make_float2(v[k], v[k + 1]), __fmul2_rn(make_float2(cv.x, cv.y), f2));
+                    const float2 w1 = __fmul2_rn(make_float2(v[k + 2], v[k + 3]), __fmul2_rn(make_float2(cv.z, cv.w), f2));
+                    v[k] = w0.x; v[k + 1] = w0.y; v[k + 2] = w1.x; v[k + 3] = w1.y;
+                }
+            } else {                         // a stiff head's diagonal
+#pragma unroll
+                for (int k = 0; k < 32; ++k) v[k] *= ex2g(fminf(csr - cs2[sr * 32 + k], 0.f)) * rec[REC_DT + sr * 32 + k];
+            }
+            if (sr == q) {
+#pragma unroll
+                for (int k = 1; k < 32; ++k) v[k] = k <= lane ? v[k] : 0.f;
+            }
+            float2 racc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int k = 0; k < 32; k += 2) {
+                const float2 wv = make_float2(v[k], v[k + 1]);
+                const float2 a = __fadd2_rn(make_float2(wsum[k], wsum[k + 1]), wv);
+                wsum[k] = a.x;
+                wsum[k + 1] = a.y;
+                const float2 z = __fmul2_rn(wv, make_float2(cb[k], cb[k + 1]));
+                v[k] = z.x;
+                v[k + 1] = z.y;
+                racc = __fadd2_rn(racc, z);
+            }
+            // column sums over the warp's rows: transposing butterfly, lane l ends with column l
+#pragma unroll
+            for (int o = 16; o >= 1; o >>= 1) {
+                const bool up = (lane & o) != 0;
+#pragma unroll
+                for (int i = 0; i < o; ++i) {
+                    const float send = up ? v[i] : v[i + o], keep = up ? v[i + o] : v[i];
+                    v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                }
+            }
+            float *pr = parts + (hi & 1) * 1024;
+            if (hi >= 2) mbar_wait(&pempty[hi & 1], ((hi >> 1) - 1) & 1, abortp, p.status);
+            pr[sr * 128 + rl] = racc.x + racc.y;
+            pr[512 + q * 128 + sr * 32 + lane] = v[0];
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&vempty[vb]);
+                mbar_arrive(&pfull[hi & 1]);
             }
         }
-
-        // ---- the head sum of W, rounded once to bf16: [s-half w][row][128 B], this thread's 16 columns of a
-        // half = chunks quar * 2, quar * 2 + 1.  The buffer held chunk states until the last head's products ended.
+        // the head sum, rounded once to bf16: [s-half][128 rows t][128 B], zeros above the diagonal
         mbar_wait(&stdone, 0, abortp, p.status);
+        auto put = [&](int j, bool zero) {
+            unsigned char *row = smem + OFF_ST + (j >> 1) * 16384 + rl * 128;
 #pragma unroll
-        for (int w = 0; w < 2; ++w) {
-            unsigned char *mrow = smem + GF_OFF_W + w * 16384 + rl * 128;
-#pragma unroll
-            for (int ch = 0; ch < 2; ++ch) {
-                const float *a = wsum + w * 16 + ch * 8;
-                *reinterpret_cast<uint4 *>(mrow + (((quar * 2 + ch) ^ (rl & 7)) << 4)) =
-                    make_uint4(pack2g(a[0], a[1]), pack2g(a[2], a[3]), pack2g(a[4], a[5]), pack2g(a[6], a[7]));
+            for (int ch = 0; ch < 4; ++ch) {
+                const float *a = wsum + ch * 8;
+                const uint4 w = zero ? make_uint4(0u, 0u, 0u, 0u)
+                                     : make_uint4(pack2g(a[0], a[1]), pack2g(a[2], a[3]), pack2g(a[4], a[5]), pack2g(a[6], a[7]));
+                *reinterpret_cast<uint4 *>(row + ((((j & 1) * 4 + ch) ^ (rl & 7)) << 4)) = w;
             }
-        }
+        };
+        put(sr, false);
+        for (int j = q + 1 + sr; j < 4; j += q + 1) put(j, true);     // the quarter's zero sub-tiles, shared out
         fence_proxy_async_smem();
         __syncwarp();
         if (lane == 0) mbar_arrive(&wfull);
+    }
+    __syncwarp();
 
-        // ---- the CTA's partial slices of the group sums: [B, seg, G, 2 nsl, N] fp32.  Every row of an accumulator is
-        // 512 contiguous bytes of its slice.  Row-per-thread global stores would touch 32 different lines per
-        // instruction, so the two accumulators are staged in shared memory (every operand buffer is dead once the last
-        // products are done), rows padded to 528 bytes (conflict-free row-per-thread writes), and each row leaves as
-        // one bulk copy.
-        mbar_wait(&accfull, 0, abortp, p.status);
-        tc_fence_after_sync();
-        {
-            float *stgC = reinterpret_cast<float *>(smem), *stgB = reinterpret_cast<float *>(smem + 128 * 528);
-            float a[32];
-            tmem_ld32(tm + tlane + TF_ACCC + quar * 32, a);
+    // The CTA's partial slices of the group sums, [B, seg, G, nsl, N] fp32.  A row of an accumulator is N * 4 contiguous bytes
+    // of its slice: staged in shared memory (every operand buffer is dead once the last products are done), rows padded by 16
+    // bytes (conflict-free row-per-thread writes), and each row leaves as one bulk copy.
+    mbar_wait(&accfull, 0, abortp, p.status);
+    __syncwarp();
+    tc_fence_after_sync();
+    constexpr int PITCH = NS + 4;
+    float *stgC = reinterpret_cast<float *>(smem), *stgB = stgC + 128 * PITCH;
+    if (sr * 32 < NS) {
+        float a[32];
+        if (doC) {
+            tmem_ld32(tm + tlane + TF_ACCC + sr * 32, a);
 #pragma unroll
             for (int k = 0; k < 32; k += 4)
-                *reinterpret_cast<float4 *>(stgC + rl * 132 + quar * 32 + k) = make_float4(a[k], a[k + 1], a[k + 2], a[k + 3]);
-            tmem_ld32(tm + tlane + TF_ACCB + quar * 32, a);
+                *reinterpret_cast<float4 *>(stgC + (q * 32 + lane) * PITCH + sr * 32 + k) = make_float4(a[k], a[k + 1], a[k + 2], a[k + 3]);
+        }
+        if (doB) {
+            tmem_ld32(tm + tlane + TF_ACCB + sr * 32, a);
 #pragma unroll
             for (int k = 0; k < 32; k += 4)
-                *reinterpret_cast<float4 *>(stgB + rl * 132 + quar * 32 + k) = make_float4(a[k], a[k + 1], a[k + 2], a[k + 3]);
-            fence_proxy_async_smem();
-            asm volatile("bar.sync 1, 512;" ::: "memory");        // the sixteen mask warps
-            const int m = tid - 64;                               // 0..511 over the mask warps
-            if (m < 256) {
-                const size_t segcap = (size_t)p.ncs * 256;
-                const int nsl2 = 2 * nsl, row = m & 127;
-                if (m < 128) {
-                    // dC rows t: tiles (1,0) and (0,0) fill the even slot of their rows, (1,1) the odd slot of t-block 1
-                    const size_t tl = (size_t)c * 256 + tb * 128 + row;
-                    const int slot = sl * 2 + (kind == 2 ? 1 : 0);
-                    bulk_store(p.pC + ((((size_t)b * segcap + tl) * p.G + g) * nsl2 + slot) * 128, stgC + row * 132, 512);
-                } else {
-                    // dB rows s: tiles (0,0) and (1,1) fill the even slot of their rows, (1,0) the odd slot of s-block 0
-                    const size_t tl = (size_t)c * 256 + sb * 128 + row;
-                    const int slot = sl * 2 + (kind == 0 ? 1 : 0);
-                    bulk_store(p.pB + ((((size_t)b * segcap + tl) * p.G + g) * nsl2 + slot) * 128, stgB + row * 132, 512);
-                }
-                tma_store_commit();
-                tma_store_wait_all();
-            }
+                *reinterpret_cast<float4 *>(stgB + (q * 32 + lane) * PITCH + sr * 32 + k) = make_float4(a[k], a[k + 1], a[k + 2], a[k + 3]);
         }
     }
-
+    fence_proxy_async_smem();
     tc_fence_before_sync();
+    __syncthreads();
+    if (tid < 256 && (tid < 128 ? doC : doB)) {
+        const int row = tid & 127;
+        const size_t o = ((((size_t)b * p.ncs * GF_T + (size_t)c * GF_T + row) * p.G + g) * nsl + sl) * NS;
+        if (tid < 128) bulk_store(p.pC + o, stgC + row * PITCH, NS * 4);
+        else bulk_store(p.pB + o, stgB + row * PITCH, NS * 4);
+        tma_store_commit();
+        tma_store_wait_all();
+    }
     __syncthreads();
     if (warp == 0) {
         tc_fence_after_sync();
@@ -543,11 +429,18 @@ k_grad_bc_fused(SegParams p, const __grid_constant__ CUtensorMap tmX, const __gr
     }
 }
 
-cudaError_t launch_grad_bc_fused(const SegParams &p, const TcMaps &m, cudaStream_t st) {
-    dim3 grid(3 * p.nc * p.nsl * p.G * p.B);
-    cudaError_t e = cudaFuncSetAttribute(k_grad_bc_fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)GF_SMEM);
+template <int NS, int WHAT>
+static cudaError_t launch_bc(const SegParams &p, const TcMaps &m, cudaStream_t st) {
+    const cudaError_t e = allow_smem<k_grad_bc<NS, WHAT>>((int)gf_smem(NS));
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_grad_bc_fused, grid, dim3(GF_THREADS), (size_t)GF_SMEM, st, p, m.x, m.dy, m.Bm, m.Cm, m.Hbf, m.Gbf);
+    return launch_pdl(k_grad_bc<NS, WHAT>, dim3(p.nc * p.nsl * p.G * p.B), dim3(GF_THREADS), (size_t)gf_smem(NS), st, p, m.x, m.dy, m.Bm, m.Cm,
+                      m.H, m.G);
+}
+
+cudaError_t launch_grad_bc(const SegParams &p, const TcMaps &m, int what, cudaStream_t st) {
+    if (what == BC_DC) return p.N == 128 ? launch_bc<128, BC_DC>(p, m, st) : launch_bc<64, BC_DC>(p, m, st);
+    if (what == BC_DB) return p.N == 128 ? launch_bc<128, BC_DB>(p, m, st) : launch_bc<64, BC_DB>(p, m, st);
+    return p.N == 128 ? launch_bc<128, BC_DC | BC_DB>(p, m, st) : launch_bc<64, BC_DC | BC_DB>(p, m, st);
 }
 
 }  // namespace ssd

@@ -1,0 +1,390 @@
+// The state chain of a segment on the tensor cores (bf16 I/O, P = 64): chunk sums and the recurrence over the chunks
+// in one kernel.  Blocks of T = 128 steps; cs = inclusive cumsum of dt*A inside the block.
+//
+//   CHAIN_FWD: H_{c+1} = e^{cs_last} H_c + sum_s e^{cs_last-cs_s} dt_s x_s B_s^T     (also makes cs and dt head-major)
+//   CHAIN_BWD: G_{c-1} = e^{cs_last} G_c + sum_t e^{cs_t} dy_t C_t^T                 (G_c: gradient leaving block c)
+//              rho2_t  = e^{cs_t} dy_t . (H_in C_t),   <G,H> partials = e^{cs_last} <G_c, H_in,c>
+//
+// One CTA owns one (batch, head) and walks the segment's blocks.  A block's sum does not depend on the carried state, so
+// it is made by tcgen05 one block ahead; the carry (N x 64 fp32) never leaves the registers of the eight worker warps:
+// what is written per block is its bf16 copy, the operand of the large kernels, 16 KB, where separate kernels for the
+// sums and the recurrence moved 32 KB of fp32 sums out and in again on top.  States are kept transposed here, [N][64], so
+// that a thread's slice (one n, 32 p) is contiguous and leaves through a swizzled tile by one TMA store per warp.
+//   warp 0 producer (TMA) | warp 1 MMA issuer | warps 2, 3 records (CHAIN_FWD, alternate blocks) | warps 4..7 scale the rows |
+//   warps 8..15 carry
+// Bound by the chain's latency, about a step per 0.5 us per head, on as many SMs as there are heads; the large kernels of
+// the neighbouring segment run beside it.
+#include "ssd_internal.h"
+#include "ssd_sm100.cuh"
+
+namespace ssd {
+
+using namespace sm100;
+
+namespace {
+
+constexpr int CH_THREADS = 512;
+constexpr int CH_T = 128;
+constexpr int CH_STAGES = 3;
+constexpr int CH_VEC = 4;                 // CHAIN_FWD: vector buffers (weights of 128 rows + the block's decay)
+constexpr int CH_VEC_FLOATS = 132;
+constexpr float kLog2eC = 1.4426950408889634f;
+constexpr int CH_AHEAD = 4;               // L2 prefetch distance in blocks beyond the staged ones
+
+// stage: V (B or C rows) N/64 x 16 KB | X (x or dy rows) 16 KB | CHAIN_BWD: H_in^T, N rows of 128 B | weights 512 B, decay 16 B
+__host__ __device__ constexpr uint32_t ch_stage_bytes(int mode, int ns) { return (uint32_t)ns * 256 + 16384 + (mode ? (uint32_t)ns * 128 + 1024 : 0); }
+__host__ __device__ constexpr uint32_t ch_smem(int mode, int ns) {
+    return CH_STAGES * ch_stage_bytes(mode, ns) + (mode ? 1 : 2) * 8 * 2048 + (mode ? 0 : CH_VEC * CH_VEC_FLOATS * 4) + 1024;
+}
+
+__device__ __forceinline__ float ex2c(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ uint32_t pack2c(float a, float b) {
+    __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<uint32_t *>(&v);
+}
+__device__ __forceinline__ float2 unpack2c(uint32_t w) { return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w)); }
+
+}  // namespace
+
+template <int NS, int MODE>
+__global__ void __launch_bounds__(CH_THREADS, 1)
+k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, long long bnd_bs, float *carry_out, float *final_out,
+           const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmH,
+           const __grid_constant__ CUtensorMap tmOut) {
+    constexpr bool BWD = MODE == CHAIN_BWD;
+    constexpr uint32_t STAGE = ch_stage_bytes(MODE, NS), OFF_X = NS * 256, OFF_H = OFF_X + 16384, OFF_W = OFF_H + NS * 128;
+    constexpr uint32_t OFF_OUT = CH_STAGES * STAGE, OFF_VEC = OFF_OUT + (BWD ? 1 : 2) * 8 * 2048;
+    extern __shared__ unsigned char smem_raw[];
+    unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    __shared__ uint64_t full[CH_STAGES], scaled[CH_STAGES], empty[CH_STAGES], mdone[2], dempty[2], vfull[CH_VEC], vempty[CH_VEC];
+    __shared__ uint32_t tmem_base, abort_flag;
+
+    const int h = blockIdx.x, b = blockIdx.y, g = h / p.hpg, nc = p.nc;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    auto chunk_of = [&](int i) { return BWD ? nc - 1 - i : i; };
+    if (tid == 0) {
+        for (int i = 0; i < CH_STAGES; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&scaled[i], 4);
+            mbar_init(&empty[i], BWD ? 8 : 1);     // BWD: the carry warps read the stage last; FWD: the MMAs do
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(&mdone[i], 1);
+            mbar_init(&dempty[i], 8);
+        }
+        for (int i = 0; i < CH_VEC; ++i) {
+            mbar_init(&vfull[i], 1);
+            mbar_init(&vempty[i], 8);              // the carry warps, which read the decay last
+        }
+        abort_flag = 0;
+        fence_barrier_init();
+    }
+    constexpr uint32_t NCOL = BWD ? 256 : 128;     // block sum, double buffered; BWD: H_in C likewise
+    if (warp == 0) tmem_alloc(&tmem_base, NCOL);
+    tc_fence_before_sync();
+    __syncthreads();
+    tc_fence_after_sync();
+    pdl_launch_dependents();
+    pdl_wait();
+    const uint32_t tm = tmem_base;
+    volatile uint32_t *abortp = &abort_flag;
+
+    if (warp == 0) {
+        // ------------------------------------------------------------ producer
+        if (elect_one()) {
+            for (int i = 0; i < nc; ++i) {
+                const int st = i % CH_STAGES, c = chunk_of(i), tok = p.t0 + c * CH_T;
+                unsigned char *sb = smem + st * STAGE;
+                if (i >= CH_STAGES) mbar_wait(&empty[st], (i / CH_STAGES - 1) & 1, abortp, p.status);
+                mbar_arrive_expect_tx(&full[st], BWD ? STAGE - 1024 + 528 : STAGE);
+                tma_load_3d(sb + OFF_X, &tmX, &full[st], h * 64, tok, b);
+#pragma unroll
+                for (int nh = 0; nh < NS / 64; ++nh) tma_load_3d(sb + nh * 16384, &tmV, &full[st], g * NS + nh * 64, tok, b);
+                if (BWD) {
+                    const float *rec = p.rec + (((size_t)b * p.H + h) * p.ncs + c) * REC_FLOATS;
+                    tma_load_3d(sb + OFF_H, &tmH, &full[st], 0, ((b * p.ncs + c) * p.H + h) * NS, 0);
+                    bulk_load(sb + OFF_W, rec + REC_OC, 512, &full[st]);
+                    bulk_load(sb + OFF_W + 512, rec + REC_DECAY, 16, &full[st]);
+                }
+                if (i + CH_AHEAD < nc) tma_prefetch_3d(&tmX, h * 64, p.t0 + chunk_of(i + CH_AHEAD) * CH_T, b);
+            }
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------ MMA issuer
+        if (elect_one()) {
+            const uint32_t idD = umma_idesc_bf16(128, 64, true, true), idY = umma_idesc_bf16(128, 64, false, true);
+            for (int i = 0; i < nc; ++i) {
+                const int st = i % CH_STAGES, bf = i & 1;
+                const uint32_t sb = smem_u32(smem + st * STAGE);
+                // The sum as D[n][p]: V rows MN-major along n (for N = 64 the second 64 rows of the operand are whatever
+                // follows, the X tile; their lanes are not read), X rows MN-major along p
+                const uint64_t dV = umma_desc_sw128(sb, 16384, 1024), dX = umma_desc_sw128(sb + OFF_X, 16384, 1024);
+                const uint32_t loV = (uint32_t)dV, hiM = (uint32_t)(dV >> 32), loX = (uint32_t)dX, hiX = (uint32_t)(dX >> 32);
+                mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
+                mbar_wait(&scaled[st], (i / CH_STAGES) & 1, abortp, p.status);
+                if (i >= 2) mbar_wait(&dempty[bf], ((i >> 1) - 1) & 1, abortp, p.status);
+                tc_fence_after_sync();
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const uint64_t ad = umma_desc_words(loV + k * 128, hiM), bd = umma_desc_words(loX + k * 128, hiX);
+                    if (k == 0) umma_bf16_fixed<false>(tm + bf * 64, ad, bd, idD);
+                    else umma_bf16_fixed<true>(tm + bf * 64, ad, bd, idD);
+                }
+                if (BWD) {   // Y[t][p] = sum_n C[t][n] H_in[p][n]
+                    const uint64_t dC = umma_desc_sw128(sb, 16, 1024), dH = umma_desc_sw128(sb + OFF_H, 8192, 1024);
+                    const uint32_t loC = (uint32_t)dC, hiC = (uint32_t)(dC >> 32), loH = (uint32_t)dH, hiH = (uint32_t)(dH >> 32);
+#pragma unroll
+                    for (int k = 0; k < NS / 16; ++k) {
+                        const uint64_t ad = umma_desc_words(loC + (k >> 2) * 1024 + (k & 3) * 2, hiC), bd = umma_desc_words(loH + k * 128, hiH);
+                        if (k == 0) umma_bf16_fixed<false>(tm + 128 + bf * 64, ad, bd, idY);
+                        else umma_bf16_fixed<true>(tm + 128 + bf * 64, ad, bd, idY);
+                    }
+                }
+                if (!BWD) umma_commit(&empty[st]);
+                umma_commit(&mdone[bf]);
+            }
+        }
+    } else if (warp < 4) {
+        // ------------------------------------------------------------ records, a lane owns four consecutive steps
+        if (!BWD) {
+            const int first = warp - 2;
+            float *vec = reinterpret_cast<float *>(smem + OFF_VEC);
+            const float Ah = __ldg(p.A + h);
+            // fetched four of this warp's blocks ahead: the strided step sizes take longer to arrive than a block takes
+            auto fetch = [&](int i, float4 &v) {
+                const float *d = p.dt + (size_t)b * p.dt_bs + (size_t)(p.t0 + i * CH_T + lane * 4) * p.H + h;
+                v = make_float4(__ldg(d), __ldg(d + p.H), __ldg(d + 2 * (size_t)p.H), __ldg(d + 3 * (size_t)p.H));
+            };
+            float4 ring[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (first + 2 * k < nc) fetch(first + 2 * k, ring[k]);
+            for (int i0 = first; i0 < nc; i0 += 8)
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int i = i0 + 2 * k;
+                if (i >= nc) break;
+                const int vb = i % CH_VEC;
+                const float4 dt4 = ring[k];
+                if (i + 8 < nc) fetch(i + 8, ring[k]);
+                const float d[4] = {dt4.x, dt4.y, dt4.z, dt4.w};
+                float cs[4], run = 0.f;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    run += d[m] * Ah;
+                    cs[m] = run;
+                }
+                float incl = run;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const float t = __shfl_up_sync(0xffffffffu, incl, off);
+                    if (lane >= off) incl += t;
+                }
+                float excl = __shfl_up_sync(0xffffffffu, incl, 1);
+                if (lane == 0) excl = 0.f;
+#pragma unroll
+                for (int m = 0; m < 4; ++m) cs[m] += excl;
+                const float decay = expf(__shfl_sync(0xffffffffu, cs[3], 31));
+#pragma unroll
+                for (int m = 0; m < 4; ++m) cs[m] *= kLog2eC;
+                const float last = __shfl_sync(0xffffffffu, cs[3], 31);
+                float w[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) w[m] = ex2c(fminf(last - cs[m], 0.f)) * d[m];
+                if (i >= CH_VEC) mbar_wait(&vempty[vb], (i / CH_VEC - 1) & 1, abortp, p.status);
+                float *v = vec + vb * CH_VEC_FLOATS;
+                *reinterpret_cast<float4 *>(v + lane * 4) = make_float4(w[0], w[1], w[2], w[3]);
+                if (lane == 0) v[128] = decay;
+                __syncwarp();
+                if (lane == 0) mbar_arrive(&vfull[vb]);
+                const float lo = __shfl_sync(0xffffffffu, cs[3], lane | 7), hi = __shfl_sync(0xffffffffu, cs[0], lane & ~7);
+                const float bi = __shfl_sync(0xffffffffu, cs[0], ((lane >> 2) & 3) * 8), bj = __shfl_sync(0xffffffffu, cs[3], (lane & 3) * 8 + 7);
+                float *rec = p.rec + (((size_t)b * p.H + h) * p.ncs + i) * REC_FLOATS;
+                auto put = [&](int part, float x, float y, float z, float u) {
+                    *reinterpret_cast<float4 *>(rec + part + lane * 4) = make_float4(x, y, z, u);
+                };
+                put(REC_CFX, ex2c(cs[0] - hi), ex2c(cs[1] - hi), ex2c(cs[2] - hi), ex2c(cs[3] - hi));
+                if (lane < 16) rec[REC_BLK + lane] = (lane & 3) < (lane >> 2) ? ex2c(bi - bj) : 0.f;
+                else if (lane < 20) rec[REC_DECAY + lane - 16] = decay;
+                put(REC_CS, cs[0], cs[1], cs[2], cs[3]);
+                put(REC_DT, d[0], d[1], d[2], d[3]);
+                put(REC_CF, ex2c(lo - cs[0]) * d[0], ex2c(lo - cs[1]) * d[1], ex2c(lo - cs[2]) * d[2], ex2c(lo - cs[3]) * d[3]);
+                put(REC_OC, ex2c(cs[0]), ex2c(cs[1]), ex2c(cs[2]), ex2c(cs[3]));
+                put(REC_OB, w[0], w[1], w[2], w[3]);
+            }
+        }
+    } else if (warp < 8) {
+        // ------------------------------------------------------------ the blocks' rows times their weights, in place (a weight is
+        // uniform along a row, so the swizzle does not matter)
+        const int th = tid - 128;
+        for (int i = 0; i < nc; ++i) {
+            const int st = i % CH_STAGES;
+            unsigned char *sb = smem + st * STAGE;
+            const float *w = BWD ? reinterpret_cast<const float *>(sb + OFF_W) : reinterpret_cast<const float *>(smem + OFF_VEC) + (i % CH_VEC) * CH_VEC_FLOATS;
+            mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
+            if (!BWD) mbar_wait(&vfull[i % CH_VEC], (i / CH_VEC) & 1, abortp, p.status);
+            uint4 *x4 = reinterpret_cast<uint4 *>(sb + OFF_X) + th;
+            uint4 v[8];
+            float f[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                v[k] = x4[k * 128];
+                f[k] = w[(th >> 3) + 16 * k];
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                uint32_t *e = reinterpret_cast<uint32_t *>(&v[k]);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float2 t = __fmul2_rn(unpack2c(e[m]), make_float2(f[k], f[k]));
+                    e[m] = pack2c(t.x, t.y);
+                }
+                x4[k * 128] = v[k];
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&scaled[st]);
+        }
+    } else {
+        // ------------------------------------------------------------ carry: warp (q, half) holds state rows
+        // n = 32 q + lane, columns p = 32 half ..; as rows of time, t = 32 q + lane
+        const int q = warp & 3, half = (warp - 8) >> 2;
+        const bool act = q * 32 < NS;
+        const uint32_t tl = tm + ((uint32_t)(q * 32) << 16) + half * 32;
+        const float *vec = reinterpret_cast<const float *>(smem + OFF_VEC);
+        unsigned char *stg = smem + OFF_OUT + (warp - 8) * 2048;      // [CHAIN_FWD: 2 buffers][32 rows][64 B], 64-byte swizzle
+        const size_t so = (size_t)h * 64 * NS + (size_t)(half * 32) * NS + q * 32 + lane;
+        float carry[32];
+#pragma unroll
+        for (int j = 0; j < 32; ++j) carry[j] = init && act ? init[(size_t)b * init_bs + so + (size_t)j * NS] : 0.f;
+        if (bnd_out && act) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) bnd_out[(size_t)b * bnd_bs + so + (size_t)j * NS] = carry[j];
+        }
+
+        for (int i = 0; i < nc; ++i) {
+            const int st = i % CH_STAGES, bf = i & 1, c = chunk_of(i);
+            // the carried state in bf16: H entering block c, or the gradient leaving it
+            if (act) {
+                unsigned char *tile = stg + (BWD ? 0 : bf * 16384), *row = tile + lane * 64;
+                if (lane == 0) {
+                    if (BWD) tma_store_wait_read();
+                    else tma_store_wait_read_but_one();
+                }
+                __syncwarp();
+#pragma unroll
+                for (int ch = 0; ch < 4; ++ch) {
+                    const float *a = carry + ch * 8;
+                    *reinterpret_cast<uint4 *>(row + ((ch ^ ((lane >> 1) & 3)) << 4)) =
+                        make_uint4(pack2c(a[0], a[1]), pack2c(a[2], a[3]), pack2c(a[4], a[5]), pack2c(a[6], a[7]));
+                }
+                fence_proxy_async_smem();
+                __syncwarp();
+                if (lane == 0) {
+                    tma_store_3d(&tmOut, tile, half * 32, ((b * p.ncs + c) * p.H + h) * NS + q * 32, 0);
+                    tma_store_commit();
+                }
+            }
+            // where this block's decay (and H_in) come from
+            if (BWD) mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
+            else mbar_wait(&vfull[i % CH_VEC], (i / CH_VEC) & 1, abortp, p.status);
+            const float decay = BWD ? *reinterpret_cast<const float *>(smem + st * STAGE + OFF_W + 512) : vec[(i % CH_VEC) * CH_VEC_FLOATS + 128];
+            float dot = 0.f;
+            if (BWD && act) {       // <G, H_in> over this thread's slice
+                const unsigned char *hr = smem + st * STAGE + OFF_H + (q * 32 + lane) * 128;
+#pragma unroll
+                for (int ch = 0; ch < 4; ++ch) {
+                    const uint4 hv = *reinterpret_cast<const uint4 *>(hr + (((half * 4 + ch) ^ (lane & 7)) << 4));
+                    const uint32_t *e = reinterpret_cast<const uint32_t *>(&hv);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        const float2 f = unpack2c(e[m]);
+                        dot = fmaf(carry[ch * 8 + 2 * m], f.x, dot);
+                        dot = fmaf(carry[ch * 8 + 2 * m + 1], f.y, dot);
+                    }
+                }
+            }
+            mbar_wait(&mdone[bf], (i >> 1) & 1, abortp, p.status);
+            __syncwarp();
+            tc_fence_after_sync();
+            float d[32];
+            if (act) {
+                tmem_ld32(tl + bf * 64, d);
+#pragma unroll
+                for (int j = 0; j < 32; ++j) carry[j] = fmaf(decay, carry[j], d[j]);
+            }
+            if (BWD) {
+                tmem_ld32(tl + 128 + bf * 64, d);
+                const unsigned char *dr = smem + st * STAGE + OFF_X + (q * 32 + lane) * 128;
+                float r2 = 0.f;
+#pragma unroll
+                for (int ch = 0; ch < 4; ++ch) {
+                    const uint4 dv = *reinterpret_cast<const uint4 *>(dr + (((half * 4 + ch) ^ (lane & 7)) << 4));
+                    const uint32_t *e = reinterpret_cast<const uint32_t *>(&dv);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) {
+                        const float2 f = unpack2c(e[m]);
+                        r2 = fmaf(f.x, d[ch * 8 + 2 * m], r2);
+                        r2 = fmaf(f.y, d[ch * 8 + 2 * m + 1], r2);
+                    }
+                }
+                const size_t vo = ((size_t)b * p.H + h) * p.ncs + c;
+                (half ? p.rho2b : p.rho2)[vo * CH_T + q * 32 + lane] = r2;
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+                if (lane == 0) p.ghdot[vo * 16 + (warp - 8)] = decay * dot;
+            }
+            tc_fence_before_sync();
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&dempty[bf]);
+                if (BWD) mbar_arrive(&empty[st]);
+                else mbar_arrive(&vempty[i % CH_VEC]);
+            }
+        }
+        if (act) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) carry_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];
+            if (final_out) {
+#pragma unroll
+                for (int j = 0; j < 32; ++j) final_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];
+            }
+            if (lane == 0) tma_store_wait_all();
+        }
+    }
+    tc_fence_before_sync();
+    __syncthreads();
+    if (warp == 0) {
+        tc_fence_after_sync();
+        tmem_dealloc(tm, NCOL);
+    }
+}
+
+template <int NS, int MODE>
+static cudaError_t launch_chain(const SegParams &p, const TcMaps &m, const float *init, long long init_bs, float *bnd_out, long long bnd_bs,
+                                float *carry_out, float *final_out, cudaStream_t st) {
+    constexpr uint32_t smem = ch_smem(MODE, NS);
+    const cudaError_t e = allow_smem<k_chain_tc<NS, MODE>>((int)smem);
+    if (e != cudaSuccess) return e;
+    const bool bwd = MODE == CHAIN_BWD;
+    return launch_pdl(k_chain_tc<NS, MODE>, dim3(p.H, p.B), dim3(CH_THREADS), (size_t)smem, st, p, init, init_bs, bnd_out, bnd_bs, carry_out,
+                      final_out, bwd ? m.dy : m.x, bwd ? m.Cm : m.Bm, m.H, bwd ? m.Gst : m.Hst);
+}
+
+cudaError_t launch_chain_fwd(const SegParams &p, const TcMaps &m, const float *init, long long init_bs, float *boundary_out, long long bnd_bs,
+                             float *final_out, cudaStream_t st) {
+    return p.N == 128 ? launch_chain<128, CHAIN_FWD>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st)
+                      : launch_chain<64, CHAIN_FWD>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st);
+}
+cudaError_t launch_chain_bwd(const SegParams &p, const TcMaps &m, const float *init, float *left_out, cudaStream_t st) {
+    const long long bs = (long long)p.H * 64 * p.N;
+    return p.N == 128 ? launch_chain<128, CHAIN_BWD>(p, m, init, bs, nullptr, 0, left_out, nullptr, st)
+                      : launch_chain<64, CHAIN_BWD>(p, m, init, bs, nullptr, 0, left_out, nullptr, st);
+}
+
+}  // namespace ssd
