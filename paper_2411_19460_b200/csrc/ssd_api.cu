@@ -47,7 +47,7 @@ static void prof_end(ProfEvent *ev, cudaStream_t st) {
 // Scratch regions of one call.  What the kernels of neighbouring segments touch at the same time exists twice on the
 // tensor-core path (copy k & 1 belongs to segment k).
 struct Layout {
-    size_t status, Hst, hcarry, Gst, gcarry, dAp, dDp;
+    size_t status, Hst, hcarry, Gst, gcarry, cbt, dAp, dDp;
     size_t rec[2], cs[2], dtT[2], Hbf[2];
     size_t Gbf[2], ghdot[2], ddt_dir[2], rho[2], rho2[2], rho2b[2], psi[2], psi2[2], pB[2], pC[2];
     size_t total;
@@ -117,9 +117,10 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
         ((size_t)pl.x_bs * pl.esz) % 16 || ((size_t)pl.bc_bs * pl.esz) % 16)
         return SSD_EALIGN;
     pl.serial = (s->flags & SSD_FLAG_SERIAL) != 0;
-    // Partial slices of the dB/dC head sums.  CUDA-core kernels: one head per slice.  Tensor-core kernel: one slice per CTA
-    // head range.
-    pl.nsl = pl.use_tc ? bc_head_split(pl.G, pl.hpg) : pl.hpg;
+    // Partial slices of the dB/dC head sums: one per CTA head range; on the CUDA-core path ranges of four heads (two where there
+    // are few), each with a slot per 64-step tile and one for the inter-chunk term.
+    const int per_range = pl.hpg >= 16 ? 4 : 2;
+    pl.nsl = pl.use_tc ? bc_head_split(pl.G, pl.hpg) : (pl.hpg + per_range - 1) / per_range * (pl.Q / 64 + 1);
     return SSD_OK;
 }
 
@@ -149,6 +150,7 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
         take2(lo.cs, vec, false);
         take2(lo.dtT, vec, false);
         lo.Hst = take(st);
+        lo.cbt = take((size_t)pl.B * pl.ncs * pl.G * pl.Q * pl.Q * sizeof(float));
     }
     if (bwd) {
         lo.gcarry = take(BH * PN * sizeof(float));
@@ -157,12 +159,11 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
         take2(lo.ghdot, BH * pl.ncs * 16 * sizeof(float), twin);
         const bool vtwin = twins && pl.use_tc;
         take2(lo.ddt_dir, vec, vtwin);
-        take2(lo.rho, vec, vtwin);
-        if (pl.use_tc) {
-            take2(lo.rho2, vec, vtwin);
-            take2(lo.rho2b, vec, vtwin);
-        }
-        take2(lo.psi, vec, vtwin);
+        const size_t vec_tiles = pl.use_tc ? vec : vec * (pl.Q / 64);
+        take2(lo.rho, vec_tiles, vtwin);
+        take2(lo.rho2, vec, vtwin);
+        if (pl.use_tc) take2(lo.rho2b, vec, vtwin);
+        take2(lo.psi, vec_tiles, vtwin);
         take2(lo.psi2, vec, vtwin);
         const size_t part = (size_t)pl.B * pl.seg * pl.G * pl.nsl * pl.N * sizeof(float);
         take2(lo.pB, part, twin);
@@ -275,6 +276,8 @@ static void fill_params(const Plan &pl, const Layout &lo, void *ws, SegParams &s
     char *w = (char *)ws;
     sp.status = (unsigned int *)(w + lo.status);
     sp.Hst = (float *)(w + lo.Hst);
+    sp.cbt = (float *)(w + lo.cbt);
+    sp.tiles = pl.use_tc ? 0 : pl.Q / 64;
     sp.hcarry = (float *)(w + lo.hcarry);
     sp.Gst = (float *)(w + lo.Gst);
     sp.gcarry = (float *)(w + lo.gcarry);
@@ -359,10 +362,9 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
             SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, maps, SC_FWD, st));
             continue;
         }
-        SSD_LAUNCH(KIND_CUMSUM, launch_chunk_cumsum(sp, st));
-        SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_simt(sp, pl.dtype, STATE_MODE_FWD, st));
+        SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, pl.dtype, SIMT_SUMS, st));
         SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN, fin, st));
-        SSD_LAUNCH(KIND_SCAN_FWD, launch_masked_product_simt(sp, pl.dtype, MP_FWD, st));
+        SSD_LAUNCH(KIND_SCAN_FWD, launch_simt(sp, pl.dtype, SIMT_Y, st));
     }
     return SSD_OK;
 }
@@ -570,8 +572,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
             SSD_TRY(cudaStreamWaitEvent(tails, side->join[par], 0));
             {
                 cudaStream_t st = tails;
-                SSD_LAUNCH(KIND_BWD_FINISH, launch_bwd_finish(sp, st));
-                SSD_LAUNCH(KIND_REDUCE_DBDC, launch_reduce_dbdc(sp, pl.dtype, st));
+                SSD_LAUNCH(KIND_BWD_FINISH, launch_bwd_tail(sp, pl.dtype, st));
                 SSD_TRY(cudaEventRecord(side->tail_done[par], st));
             }
         }
@@ -594,17 +595,13 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
                     SSD_LAUNCH(KIND_BWD_DB, launch_grad_bc(sp, maps, BC_DB, st));
                 }
             } else {
-                SSD_LAUNCH(KIND_CUMSUM, launch_chunk_cumsum(sp, st));
-                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chunk_state_simt(sp, pl.dtype, STATE_MODE_FWD, st));
+                SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, pl.dtype, SIMT_SUMS, st));
                 SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, hin, (long long)pl.nseg * pl.H * PN, nullptr, 0, nullptr, st));
-                SSD_LAUNCH(KIND_DSTATE, launch_chunk_state_simt(sp, pl.dtype, STATE_MODE_DSTATE, st));
+                SSD_LAUNCH(KIND_DSTATE, launch_simt(sp, pl.dtype, SIMT_DSTATE, st));
                 SSD_LAUNCH(KIND_STATE_PASS_BWD, launch_state_pass_bwd(sp, ginit, gleft, st));
-                SSD_LAUNCH(KIND_BWD_DX, launch_masked_product_simt(sp, pl.dtype, MP_BWD_DX, st));
-                SSD_LAUNCH(KIND_BWD_DC, launch_masked_product_simt(sp, pl.dtype, MP_DC, st));
-                SSD_LAUNCH(KIND_BWD_DB, launch_masked_product_simt(sp, pl.dtype, MP_DB, st));
+                SSD_LAUNCH(KIND_BWD_DX, launch_simt(sp, pl.dtype, SIMT_BWD, st));
             }
-            SSD_LAUNCH(KIND_BWD_FINISH, launch_bwd_finish(sp, st));
-            SSD_LAUNCH(KIND_REDUCE_DBDC, launch_reduce_dbdc(sp, pl.dtype, st));
+            SSD_LAUNCH(KIND_BWD_FINISH, launch_bwd_tail(sp, pl.dtype, st));
         }
     }
     SSD_LAUNCH(KIND_FINAL, launch_final_dAdD(sp, dA, dD, (shape->flags & SSD_FLAG_ACCUM_PARAM_GRADS) != 0, st));

@@ -81,6 +81,7 @@ struct SegParams {
     int nsl;       // head slices per group in the dB/dC partial buffers
     int ndd;       // partial sums of dD per (head, chunk) that the kernels of this path write (<= 4)
     int ngh;       // partial sums of <G,H> per (head, chunk) (<= 16)
+    int tiles;     // CUDA-core path: 64-step tiles per chunk (rho, psi and the slices come per tile); tensor-core path: 0
     float dx_skip;    // 1 when dx also takes dy (a skip connection around the layer), else 0
     int64_t x_bs, dt_bs, bc_bs;  // batch strides, elements
 
@@ -104,10 +105,10 @@ struct SegParams {
     float *gcarry;         // [B,H,P,N]     state gradient handed right-to-left (backward)
     float *ghdot;          // [B,H,ncs,16]  partial sums of exp(cs_last) <Gout_c, H_in,c>
     float *ddt_dir;        // [B,H,ncs,Q]   direct part of ddt
-    float *rho;            // [B,H,ncs,Q]   C_t . dC_t of this head (CUDA-core path: all of it; tensor-core
-                           //               path: its intra-chunk part)
-    float *rho2, *rho2b;   // [B,H,ncs,Q]   tensor-core path: the two halves of C_t . (inter-chunk part of this head's dC_t); else NULL
-    float *psi;            // [B,H,ncs,Q]   B_t . (intra-chunk part of this head's dB_t)
+    float *cbt;            // CUDA-core path: [B,ncs,G,Q,Q] C B^T, causal 64 x 64 tiles
+    float *rho;            // [B,H,ncs,Q]   C_t . (intra-chunk part of this head's dC_t); CUDA-core path: [B,H,ncs,tiles,Q] by column tile
+    float *rho2, *rho2b;   // [B,H,ncs,Q]   C_t . (inter-chunk part of this head's dC_t); tensor-core path: in two halves
+    float *psi;            // [B,H,ncs,Q]   B_t . (intra-chunk part of this head's dB_t); CUDA-core path: [B,H,ncs,tiles,Q] by row tile
     float *psi2;           // [B,H,ncs,Q]   B_t . (inter-chunk part of this head's dB_t)
     float *pB, *pC;        // [B,seg,G,nsl,N] per-head-slice partial dB / dC
     float *dAp;            // [B,H,nct]     per-chunk partial of dA
@@ -118,16 +119,14 @@ static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; 
 
 // ---- kernel launchers (each returns the cudaError_t of its launch) ----
 // ssd_simt.cu : CUDA-core kernels, any I/O dtype
-cudaError_t launch_chunk_cumsum(const SegParams &p, cudaStream_t st);
-cudaError_t launch_chunk_state_simt(const SegParams &p, int dtype, int mode, cudaStream_t st);
+enum { SIMT_SUMS = 0, SIMT_DSTATE, SIMT_Y, SIMT_BWD };   // chunk sums, cumsum and C B^T | state-gradient sums | y | dx, dB, dC slices
+cudaError_t launch_simt(const SegParams &p, int dtype, int what, cudaStream_t st);
 // init: state entering the segment (NULL = zeros), batch stride init_bs elements;
 // boundary_out (nullable): where to store that state, batch stride bnd_bs; final_out nullable.
 cudaError_t launch_state_pass_fwd(const SegParams &p, const float *init, long long init_bs,
                                   float *boundary_out, long long bnd_bs, float *final_out, cudaStream_t st);
 cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, float *left_out, cudaStream_t st);
-cudaError_t launch_masked_product_simt(const SegParams &p, int dtype, int mode, cudaStream_t st);
-cudaError_t launch_bwd_finish(const SegParams &p, cudaStream_t st);
-cudaError_t launch_reduce_dbdc(const SegParams &p, int dtype, cudaStream_t st);
+cudaError_t launch_bwd_tail(const SegParams &p, int dtype, cudaStream_t st);
 cudaError_t launch_final_dAdD(const SegParams &p, float *dA, float *dD, bool accumulate, cudaStream_t st);
 // ssd_glue.cu : layer-axis glue of a layer stack
 cudaError_t launch_glue(int dtype, bool transpose, const void *a, const void *b, const float *W, void *out,
@@ -184,6 +183,5 @@ enum {
     KIND_STATE_PASS_BWD, KIND_BWD_DX, KIND_BWD_DC, KIND_BWD_DB, KIND_BWD_FINISH, KIND_REDUCE_DBDC,
     KIND_FINAL, KIND_GLUE, KIND_DECODE, KIND_BWD_DBDC, KIND_CONV, KIND_NORM, KIND_COUNT
 };
-enum { MP_FWD = 0, MP_BWD_DX = 1, MP_DC = 2, MP_DB = 3 };
 
 }  // namespace ssd

@@ -1,7 +1,6 @@
-// CUDA-core kernels of libssd: the bandwidth-bound steps (chunk cumsum, inter-chunk state
-// passing, segment-boundary store/reload, the backward's scans and reductions) for every dtype,
-// and FFMA versions of the contractions, which serve the fp32 mode (1e-4 parity rules out
-// reduced-precision tensor-core inputs) and cross-check the tensor-core kernels.
+// CUDA-core kernels of libssd: the backward's finishing scans and reductions for every path, and inter-chunk state passing
+// and FFMA versions of the contractions, which serve the fp32 mode (1e-4 parity rules out reduced-precision tensor-core
+// inputs) and chunks of 64, and cross-check the tensor-core kernels.
 //
 // Notation per (batch b, head h), chunk of Q steps: a_t = dt_t*A_h, cs_t = inclusive cumsum of a
 // inside the chunk, H_in = state entering the chunk, Gout = dLoss/d(state leaving the chunk).
@@ -35,131 +34,23 @@ template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16 *p,
     *p = __float2bfloat16_rn(v);
 }
 
+__device__ __forceinline__ void add4(float4 &a, const float4 &b) {
+    a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
+}
+__device__ __forceinline__ void st4(float *p, const float4 &v) { *reinterpret_cast<float4 *>(p) = v; }
+__device__ __forceinline__ void st4(__nv_bfloat16 *p, const float4 &v) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+    uint2 pk;
+    pk.x = *reinterpret_cast<const unsigned int *>(&lo);
+    pk.y = *reinterpret_cast<const unsigned int *>(&hi);
+    *reinterpret_cast<uint2 *>(p) = pk;
+}
+
 __device__ __forceinline__ size_t slot_off(const SegParams &p, int b, int slot, int h) {
     return (((size_t)b * (p.ncs + 1) + slot) * p.H + h) * (size_t)(p.P * p.N);
 }
 __device__ __forceinline__ size_t vec_off(const SegParams &p, int b, int h, int c) {
     return (((size_t)b * p.H + h) * p.ncs + c) * (size_t)p.Q;
-}
-
-// ------------------------------------------------------------------ chunk cumsum
-// One CTA per (chunk, block of 8 heads, batch), one warp per head.  The dt[b, t, h0..h0+7] pieces
-// (32 contiguous bytes per step) are staged through shared memory; a lane owns Q/32 consecutive
-// steps (serial prefix), lane totals are combined with a warp-shuffle scan.
-__global__ void __launch_bounds__(256) k_chunk_cumsum(SegParams p) {
-    __shared__ float tile[256][9];
-    const int c = blockIdx.x, h0 = blockIdx.y * 8, b = blockIdx.z;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int Q = p.Q, per = Q >> 5;
-    const size_t tok0 = (size_t)p.t0 + (size_t)c * Q;
-    const int nh = min(8, p.H - h0);
-    for (int idx = tid; idx < Q * 8; idx += 256) {
-        const int t = idx >> 3, hh = idx & 7;
-        if (hh < nh) tile[t][hh] = __ldg(p.dt + (size_t)b * p.dt_bs + (tok0 + t) * p.H + h0 + hh);
-    }
-    __syncthreads();
-    const int hh = warp;
-    if (hh >= nh) return;
-    const float Ah = __ldg(p.A + h0 + hh);
-    float a[8], d[8];
-    float run = 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        if (j < per) {
-            d[j] = tile[lane * per + j][hh];
-            run += d[j] * Ah;
-            a[j] = run;
-        }
-    float incl = run;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float v = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += v;
-    }
-    float excl = __shfl_up_sync(0xffffffffu, incl, 1);
-    if (lane == 0) excl = 0.f;
-    const size_t o = vec_off(p, b, h0 + hh, c) + (size_t)lane * per;
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        if (j < per) {
-            p.cs[o + j] = a[j] + excl;
-            p.dtT[o + j] = d[j];
-        }
-}
-
-cudaError_t launch_chunk_cumsum(const SegParams &p, cudaStream_t st) {
-    k_chunk_cumsum<<<dim3(p.nc, (p.H + 7) / 8, p.B), 256, 0, st>>>(p);
-    return cudaGetLastError();
-}
-
-// ------------------------------------------------------------------ chunk sums / state-gradient sums (FFMA)
-// mode FWD   : S_c[p,n] = sum_s exp(cs_last - cs_s) dt_s x_s[p] B_s[n]     -> Hst slot c+1
-// mode DSTATE: E_c[p,n] = sum_t exp(cs_t) dy_t[p] C_t[n]                   -> Gst slot c
-template <typename T, int NS>
-__global__ void __launch_bounds__(256) k_chunk_state_simt(SegParams p, int mode) {
-    __shared__ float xs[32][64];
-    __shared__ float bs[32][NS];
-    __shared__ float wsm[256];
-    const int c = blockIdx.x, h = blockIdx.y, b = blockIdx.z, g = h / p.hpg;
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    const int Q = p.Q;
-    const T *rowsrc = (const T *)(mode == STATE_MODE_FWD ? p.x : p.dy);
-    const T *colsrc = (const T *)(mode == STATE_MODE_FWD ? p.Bm : p.Cm);
-    const size_t tok0 = (size_t)p.t0 + (size_t)c * Q;
-    const float *csb = p.cs + vec_off(p, b, h, c);
-    const float *dtb = p.dtT + vec_off(p, b, h, c);
-    const float cl = csb[Q - 1];
-    for (int t = tid; t < Q; t += 256)
-        wsm[t] = (mode == STATE_MODE_FWD) ? expf(fminf(cl - csb[t], 0.f)) * dtb[t] : expf(csb[t]);
-    __syncthreads();
-    constexpr int NJ = NS / 16;
-    float acc[4][NJ];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) acc[i][j] = 0.f;
-    const size_t HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
-    for (int s0 = 0; s0 < Q; s0 += 32) {
-        for (int idx = tid; idx < 32 * 64; idx += 256) {
-            const int r = idx >> 6, pp = idx & 63;
-            xs[r][pp] = ldf(rowsrc + (size_t)b * p.x_bs + (tok0 + s0 + r) * HP + (size_t)h * 64 + pp) * wsm[s0 + r];
-        }
-        for (int idx = tid; idx < 32 * NS; idx += 256) {
-            const int r = idx / NS, nn = idx % NS;
-            bs[r][nn] = ldf(colsrc + (size_t)b * p.bc_bs + (tok0 + s0 + r) * GN + (size_t)g * NS + nn);
-        }
-        __syncthreads();
-#pragma unroll 4
-        for (int kk = 0; kk < 32; ++kk) {
-            float xv[4], bv[NJ];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) xv[i] = xs[kk][ty * 4 + i];
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) bv[j] = bs[kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < NJ; ++j) acc[i][j] = fmaf(xv[i], bv[j], acc[i][j]);
-        }
-        __syncthreads();
-    }
-    float *out = (mode == STATE_MODE_FWD) ? p.Hst + slot_off(p, b, c + 1, h) : p.Gst + slot_off(p, b, c, h);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) out[(size_t)(ty * 4 + i) * NS + tx + 16 * j] = acc[i][j];
-}
-
-cudaError_t launch_chunk_state_simt(const SegParams &p, int dtype, int mode, cudaStream_t st) {
-    dim3 grid(p.nc, p.H, p.B);
-    if (dtype == SSD_DTYPE_F32) {
-        if (p.N == 64) k_chunk_state_simt<float, 64><<<grid, 256, 0, st>>>(p, mode);
-        else k_chunk_state_simt<float, 128><<<grid, 256, 0, st>>>(p, mode);
-    } else {
-        if (p.N == 64) k_chunk_state_simt<__nv_bfloat16, 64><<<grid, 256, 0, st>>>(p, mode);
-        else k_chunk_state_simt<__nv_bfloat16, 128><<<grid, 256, 0, st>>>(p, mode);
-    }
-    return cudaGetLastError();
 }
 
 // ------------------------------------------------------------------ forward state passing, boundary store / reload
@@ -285,293 +176,514 @@ cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, float *
     return launch_pdl(k_state_pass_bwd, grid, dim3(SP_THREADS), 0, st, p, init, left_out);
 }
 
-// ------------------------------------------------------------------ masked products y, dx, dB, dC (FFMA)
-// One generic "score -> decay mask -> times values (+ inter-chunk term)" kernel, 64x64 tiles:
-//   score[r,c] = <Rv_r, Cv_c>            (length KD)
-//   acc[r,:]  += mask(r,c) * score[r,c] * V_c      (width WD)
-//   acc[r,j]  += offscale_r * <Rv_r, S_j>          S = chunk state, viewed [WD, KD]
-// MP_FWD    rows t: Rv=C, Cv=B, V=x , mask=[s<=t] e^{cs_t-cs_s} dt_s, S=H_in[p][n], off e^{cs_t}
-//           y_t = acc + D x_t
-// MP_BWD_DX rows s: Rv=B, Cv=C, V=dy, mask=[t>=s] e^{cs_t-cs_s},     S=Gout[p][n], off e^{cs_last-cs_s}
-//           dx_s = D dy_s + dt_s acc ; ddt_direct_s = <x_s, acc> ; dD partial = sum dy x
-// MP_DC     rows t: Rv=dy, Cv=x, V=B, mask as MP_FWD,               S=H_in^T[n][p], off e^{cs_t}
-//           per-head dC_t = acc ; rho_t = <C_t, acc>   (= dy_t . (y_t - D x_t))
-// MP_DB     rows s: Rv=x, Cv=dy, V=C, mask=[t>=s] e^{cs_t-cs_s} dt_s, S=Gout^T[n][p], off dt_s e^{cs_last-cs_s}
-//           per-head dB_s = acc ; psi_s = <B_s, intra-chunk part>, psi2_s = <B_s, inter-chunk part>
-//           (psi + psi2 = dt_s ddt_direct_s, but psi is built from the same masked products as rho,
-//           so rho - psi cancels cleanly in the suffix sums of da)
+// ------------------------------------------------------------------ FFMA contractions
+// One shape for all of them: a 64 x 64 output tile per CTA of 256 threads, 4 x 4 outputs per thread, operands staged 64 steps
+// of the contraction at a time as [k][64] (rows padded to 68 floats), so that a step of k costs a thread two 16-byte
+// shared-memory reads for 16 multiply-adds (packed two to an instruction).  The next stage's global loads are in flight while
+// a stage is multiplied.  Bound by the FFMA rate and the shared-memory reads beside it.
+//
+// What does not depend on the head is not done per head: C B^T is made once per group (k_simt_sums writes it, 64 x 64 causal
+// tiles), and dB / dC come from a head sum of the masked tiles, one product per CTA instead of two per head.
+constexpr int ST_LD = 68;
+struct SimtTiles {
+    float a[64][ST_LD], b[64][ST_LD];
+};
+
+template <typename T> __device__ __forceinline__ float4 ld4f(const T *p);
+template <> __device__ __forceinline__ float4 ld4f<float>(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
+template <> __device__ __forceinline__ float4 ld4f<__nv_bfloat16>(const __nv_bfloat16 *p) {
+    const uint2 v = __ldg(reinterpret_cast<const uint2 *>(p));
+    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.x));
+    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.y));
+    return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// A 64 x 64 tile of a row-major matrix on its way to shared memory: four float4 per thread.
+//   direct:     row = tid / 16 + 16 k, columns (tid % 16) * 4 ..            -> s[row][col]      (rows run along k)
+//   transposed: row = (tid % 8) + 8 * (tid / 32) , columns ((tid / 8) % 4) * 4 + 16 k -> s[col][row]   (columns run along k)
+template <typename T> __device__ __forceinline__ void tile_load(float4 (&r)[4], const T *src, size_t stride, bool transposed) {
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!transposed) r[k] = ld4f(src + (size_t)((tid >> 4) + 16 * k) * stride + (tid & 15) * 4);
+        else r[k] = ld4f(src + (size_t)((tid & 7) + 8 * (tid >> 5)) * stride + ((tid >> 3) & 3) * 4 + 16 * k);
+    }
+}
+// The same from scratch that an earlier kernel of the call wrote: coherent loads.
+__device__ __forceinline__ void tile_load_ws(float4 (&r)[4], const float *src, size_t stride, bool transposed) {
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float *q = !transposed ? src + (size_t)((tid >> 4) + 16 * k) * stride + (tid & 15) * 4
+                                     : src + (size_t)((tid & 7) + 8 * (tid >> 5)) * stride + ((tid >> 3) & 3) * 4 + 16 * k;
+        r[k] = *reinterpret_cast<const float4 *>(q);
+    }
+}
+__device__ __forceinline__ void tile_store(float (*s)[ST_LD], const float4 (&r)[4], bool transposed) {
+    const int tid = threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        if (!transposed) {
+            *reinterpret_cast<float4 *>(&s[(tid >> 4) + 16 * k][(tid & 15) * 4]) = r[k];
+        } else {
+            const int row = (tid & 7) + 8 * (tid >> 5), c = ((tid >> 3) & 3) * 4 + 16 * k;
+            s[c][row] = r[k].x; s[c + 1][row] = r[k].y; s[c + 2][row] = r[k].z; s[c + 3][row] = r[k].w;
+        }
+    }
+}
+// acc[i][j] += sum_k a[k][4 ty + i] b[k][4 tx + j]
+__device__ __forceinline__ void tile_mma(float2 (&acc)[4][2], const float (*a)[ST_LD], const float (*b)[ST_LD]) {
+    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
+#pragma unroll 8
+    for (int k = 0; k < 64; ++k) {
+        const float4 av = *reinterpret_cast<const float4 *>(&a[k][ty * 4]), bv = *reinterpret_cast<const float4 *>(&b[k][tx * 4]);
+        const float am[4] = {av.x, av.y, av.z, av.w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 a2 = make_float2(am[i], am[i]);
+            acc[i][0] = __ffma2_rn(a2, make_float2(bv.x, bv.y), acc[i][0]);
+            acc[i][1] = __ffma2_rn(a2, make_float2(bv.z, bv.w), acc[i][1]);
+        }
+    }
+}
+__device__ __forceinline__ void zero_acc(float2 (&acc)[4][2]) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+}
+// sum over the 16 lanes of a half warp that share ty
+__device__ __forceinline__ float sum_tx(float v) {
+#pragma unroll
+    for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
+    return v;
+}
+// causal tile pair number -> (row tile, column tile), column <= row
+__device__ __forceinline__ void pair_of(int idx, int &rt, int &ct) {
+    rt = 0;
+    while (idx > rt) idx -= ++rt;
+    ct = idx;
+}
+// C B^T of (b, chunk, group): [Q][Q] row-major in t
+__device__ __forceinline__ float *cb_of(const SegParams &p, int b, int c, int g) {
+    return p.cbt + (((size_t)b * p.ncs + c) * p.G + g) * (size_t)(p.Q * p.Q);
+}
+
+// mode FWD   : S_c[p,n] = sum_s exp(cs_last - cs_s) dt_s x_s[p] B_s[n]     -> Hst slot c+1   (and cs, dtT, C B^T)
+// mode DSTATE: E_c[p,n] = sum_t exp(cs_t) dy_t[p] C_t[n]                   -> Gst slot c
 template <typename T, int NS, int MODE>
-__global__ void __launch_bounds__(256) k_masked_product_simt(SegParams p) {
-    constexpr int KD = (MODE < 2) ? NS : 64;
-    constexpr int WD = (MODE < 2) ? 64 : NS;
-    constexpr int NJ = WD / 16;
-    constexpr int KP = KD + 1;
-    constexpr bool LOWER = (MODE == MP_FWD || MODE == MP_DC);
-    extern __shared__ float sm[];
-    float *Rv = sm;
-    float *Cv = Rv + 64 * KP;
-    float *V = Cv + 64 * KP;
-    float *Mk = V + 64 * WD;
-    float *css = Mk + 64 * 65;
-    float *dts = css + 256;
-
-    const int Q = p.Q, nrt = Q >> 6;
-    const int c = blockIdx.x / nrt, rt = blockIdx.x % nrt;
-    const int h = blockIdx.y, b = blockIdx.z, g = h / p.hpg;
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15;
-    const size_t tok0 = (size_t)p.t0 + (size_t)c * Q;
+__global__ void __launch_bounds__(256) k_simt_sums(SegParams p) {
+    pdl_launch_dependents();
+    pdl_wait();
+    __shared__ SimtTiles sm;
+    __shared__ float wsm[256], tot[8];
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, nh = NS / 64;
     const size_t HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
-    const T *xlike_base_x = (const T *)p.x + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
-    const T *xlike_base_dy = (const T *)p.dy + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
-    const T *bc_base_B = (const T *)p.Bm + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS;
-    const T *bc_base_C = (const T *)p.Cm + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS;
+    int id = blockIdx.x;
+    const int nsum = p.nc * nh * p.H * p.B;
+    float2 acc[4][2];
+    float4 ra[4], rb[4];
+    zero_acc(acc);
+    if (MODE == STATE_MODE_FWD && id >= nsum) {      // a causal tile of C B^T
+        id -= nsum;
+        const int npair = nrt * (nrt + 1) / 2;
+        int rt, ct;
+        pair_of(id % npair, rt, ct);
+        id /= npair;
+        const int g = id % p.G, c = (id / p.G) % p.nc, b = id / (p.G * p.nc);
+        const size_t o = (size_t)b * p.bc_bs + ((size_t)p.t0 + (size_t)c * Q) * GN + (size_t)g * NS;
+        const T *C = (const T *)p.Cm + o + (size_t)rt * 64 * GN, *Bp = (const T *)p.Bm + o + (size_t)ct * 64 * GN;
+        for (int k0 = 0; k0 < NS; k0 += 64) {
+            tile_load(ra, C + k0, GN, true);
+            tile_load(rb, Bp + k0, GN, true);
+            if (k0) __syncthreads();
+            tile_store(sm.a, ra, true);
+            tile_store(sm.b, rb, true);
+            __syncthreads();
+            tile_mma(acc, sm.a, sm.b);
+        }
+        float *out = cb_of(p, b, c, g) + (size_t)(rt * 64 + ty * 4) * Q + ct * 64 + tx * 4;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4 *>(out + (size_t)i * Q) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+        return;
+    }
+    const int n0 = (id % nh) * 64;
+    id /= nh;
+    const int h = id % p.H, c = (id / p.H) % p.nc, b = id / (p.H * p.nc), g = h / p.hpg;
+    const size_t tok0 = (size_t)p.t0 + (size_t)c * Q;
+    const T *rows = (const T *)(MODE == STATE_MODE_FWD ? p.x : p.dy) + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
+    const T *cols = (const T *)(MODE == STATE_MODE_FWD ? p.Bm : p.Cm) + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS + n0;
+    tile_load(ra, rows, HP, false);
+    tile_load(rb, cols, GN, false);
+    if (MODE == STATE_MODE_FWD) {
+        // the chunk cumsum: a thread per step, shuffle scans of 32 and the warps' totals
+        const int lane = tid & 31, warp = tid >> 5;
+        float d = 0.f, v = 0.f;
+        if (tid < Q) {
+            d = __ldg(p.dt + (size_t)b * p.dt_bs + (tok0 + tid) * p.H + h);
+            v = d * __ldg(p.A + h);
+        }
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float t = __shfl_up_sync(0xffffffffu, v, off);
+            if (lane >= off) v += t;
+        }
+        if (lane == 31) tot[warp] = v;
+        __syncthreads();
+        float before = 0.f, last = 0.f;
+        for (int w = 0; w < Q / 32; ++w) {
+            if (w < warp) before += tot[w];
+            last += tot[w];
+        }
+        v += before;
+        if (tid < Q) {
+            wsm[tid] = expf(fminf(last - v, 0.f)) * d;
+            if (n0 == 0) {
+                p.cs[vec_off(p, b, h, c) + tid] = v;
+                p.dtT[vec_off(p, b, h, c) + tid] = d;
+            }
+        }
+    } else if (tid < Q) {
+        wsm[tid] = expf(p.cs[vec_off(p, b, h, c) + tid]);
+    }
+    __syncthreads();
+    for (int s0 = 0; s0 < Q; s0 += 64) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float w = wsm[s0 + ty + 16 * k];
+            ra[k].x *= w; ra[k].y *= w; ra[k].z *= w; ra[k].w *= w;
+        }
+        tile_store(sm.a, ra, false);
+        tile_store(sm.b, rb, false);
+        __syncthreads();
+        if (s0 + 64 < Q) {
+            tile_load(ra, rows + (size_t)(s0 + 64) * HP, HP, false);
+            tile_load(rb, cols + (size_t)(s0 + 64) * GN, GN, false);
+        }
+        tile_mma(acc, sm.a, sm.b);
+        __syncthreads();
+    }
+    float *out = (MODE == STATE_MODE_FWD ? p.Hst + slot_off(p, b, c + 1, h) : p.Gst + slot_off(p, b, c, h)) + (size_t)(ty * 4) * NS + n0 + tx * 4;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        *reinterpret_cast<float4 *>(out + (size_t)i * NS) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+}
 
-    const T *rsrc, *csrc, *vsrc;
-    size_t rstride, vstride;  // rsrc/csrc share a stride
-    if (MODE == MP_FWD) { rsrc = bc_base_C; csrc = bc_base_B; vsrc = xlike_base_x; rstride = GN; vstride = HP; }
-    else if (MODE == MP_BWD_DX) { rsrc = bc_base_B; csrc = bc_base_C; vsrc = xlike_base_dy; rstride = GN; vstride = HP; }
-    else if (MODE == MP_DC) { rsrc = xlike_base_dy; csrc = xlike_base_x; vsrc = bc_base_B; rstride = HP; vstride = GN; }
-    else { rsrc = xlike_base_x; csrc = xlike_base_dy; vsrc = bc_base_C; rstride = HP; vstride = GN; }
-
+// One 64-row tile of y (DX = false) or of dx (DX = true) of one head:
+//   y_t  = sum_{s<=t} CB[t,s] e^{cs_t-cs_s} dt_s x_s + e^{cs_t} C_t H_in + D x_t
+//   u_s  = sum_{t>=s} CB[t,s] e^{cs_t-cs_s} dy_t     + e^{cs_last-cs_s} B_s Gout ;  dx_s = D dy_s + dt_s u_s ,
+//   ddt_direct_s = x_s . u_s , psi2_s = dt_s e^{cs_last-cs_s} x_s . (Gout B_s) , dD partial = sum dy.x
+template <typename T, int NS, bool DX>
+__device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm, float *css, float *dts, float *red, int c, int rt, int h, int b) {
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, g = h / p.hpg, r0 = rt * 64;
+    const size_t tok0 = (size_t)p.t0 + (size_t)c * Q, HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
+    const size_t xo = (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
+    const T *vals = (const T *)(DX ? p.dy : p.x) + xo;
+    const T *rowv = (const T *)(DX ? p.Bm : p.Cm) + (size_t)b * p.bc_bs + (tok0 + r0) * GN + (size_t)g * NS;
+    const float *St = DX ? p.Gst + slot_off(p, b, c + 1, h) : p.Hst + slot_off(p, b, c, h), *CB = cb_of(p, b, c, g);
+    float4 ra[4], rb[4];
+    float2 acc[4][2];
+    zero_acc(acc);
+    tile_load(ra, rowv, GN, true);
+    tile_load_ws(rb, St, NS, true);
     for (int t = tid; t < Q; t += 256) {
         css[t] = p.cs[vec_off(p, b, h, c) + t];
         dts[t] = p.dtT[vec_off(p, b, h, c) + t];
     }
-    const int r0 = rt * 64;
-    for (int idx = tid; idx < 64 * KD; idx += 256) {
-        const int r = idx / KD, k = idx % KD;
-        Rv[r * KP + k] = ldf(rsrc + (size_t)(r0 + r) * rstride + k);
-    }
-    float acc[4][NJ];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < NJ; ++j) acc[i][j] = 0.f;
-    __syncthreads();
-
-    const float cs_last = css[Q - 1];
-    const int ct_begin = LOWER ? 0 : rt, ct_end = LOWER ? rt : nrt - 1;
-    for (int ct = ct_begin; ct <= ct_end; ++ct) {
-        const int c0 = ct * 64;
-        for (int idx = tid; idx < 64 * KD; idx += 256) {
-            const int r = idx / KD, k = idx % KD;
-            Cv[r * KP + k] = ldf(csrc + (size_t)(c0 + r) * rstride + k);
-        }
-        for (int idx = tid; idx < 64 * WD; idx += 256) {
-            const int r = idx / WD, j = idx % WD;
-            V[r * WD + j] = ldf(vsrc + (size_t)(c0 + r) * vstride + j);
-        }
+    auto load_vals = [&](int ct) {      // CB tile and value rows of column tile ct
+        // DX = false: rows t = r0 .., columns s = 64 ct .. ; DX = true: the tile's rows are the CB matrix's columns
+        if (!DX) tile_load_ws(ra, CB + (size_t)r0 * Q + ct * 64, Q, true);
+        else tile_load_ws(ra, CB + (size_t)ct * 64 * Q + r0, Q, false);
+        tile_load(rb, vals + (size_t)ct * 64 * HP, HP, false);
+    };
+    const int ct0 = DX ? rt : 0, ct1 = DX ? nrt : rt + 1;
+    for (int k0 = 0; k0 < NS; k0 += 64) {
+        tile_store(sm.a, ra, true);
+        tile_store(sm.b, rb, true);
         __syncthreads();
-        float s[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-#pragma unroll 4
-        for (int k = 0; k < KD; ++k) {
-            float rv[4], cv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) rv[i] = Rv[(ty * 4 + i) * KP + k];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cv[j] = Cv[(tx + 16 * j) * KP + k];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) s[i][j] = fmaf(rv[i], cv[j], s[i][j]);
+        if (k0 + 64 < NS) {
+            tile_load(ra, rowv + k0 + 64, GN, true);
+            tile_load_ws(rb, St + k0 + 64, NS, true);
+        } else {
+            load_vals(ct0);
         }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int r = r0 + ty * 4 + i, cc = c0 + tx + 16 * j;
-                float m;
-                if (LOWER) m = (cc <= r) ? expf(fminf(css[r] - css[cc], 0.f)) * dts[cc] : 0.f;
-                else if (MODE == MP_BWD_DX) m = (cc >= r) ? expf(fminf(css[cc] - css[r], 0.f)) : 0.f;
-                else m = (cc >= r) ? expf(fminf(css[cc] - css[r], 0.f)) * dts[r] : 0.f;
-                Mk[(ty * 4 + i) * 65 + tx + 16 * j] = s[i][j] * m;
-            }
-        __syncthreads();
-#pragma unroll 4
-        for (int k = 0; k < 64; ++k) {
-            float mv[4], vv[NJ];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) mv[i] = Mk[(ty * 4 + i) * 65 + k];
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) vv[j] = V[k * WD + tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < NJ; ++j) acc[i][j] = fmaf(mv[i], vv[j], acc[i][j]);
-        }
+        tile_mma(acc, sm.a, sm.b);
         __syncthreads();
     }
-
-    // dB rows: psi_intra_s = <B_s, intra-chunk part of dB_s>, taken before the inter-chunk term is added
-    float dot_intra[4] = {0.f, 0.f, 0.f, 0.f};
-    if (MODE == MP_DB) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-#pragma unroll
-            for (int j = 0; j < NJ; ++j)
-                dot_intra[i] = fmaf(ldf(bc_base_B + (size_t)(r0 + ty * 4 + i) * GN + tx + 16 * j), acc[i][j], dot_intra[i]);
-#pragma unroll
-            for (int off = 8; off > 0; off >>= 1) dot_intra[i] += __shfl_xor_sync(0xffffffffu, dot_intra[i], off);
-        }
-    }
-
-    // inter-chunk term
-    const float *St = (MODE == MP_FWD || MODE == MP_DC) ? p.Hst + slot_off(p, b, c, h)
-                                                        : p.Gst + slot_off(p, b, c + 1, h);
-    float offs[4];
+    // the inter-chunk term is complete: scale its rows
+    const float cl = css[Q - 1];
+    float dd2[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int r = r0 + ty * 4 + i;
-        if (MODE == MP_FWD || MODE == MP_DC) offs[i] = expf(css[r]);
-        else if (MODE == MP_BWD_DX) offs[i] = expf(fminf(cs_last - css[r], 0.f));
-        else offs[i] = dts[r] * expf(fminf(cs_last - css[r], 0.f));
+        const float o = DX ? expf(fminf(cl - css[r], 0.f)) : expf(css[r]);
+        acc[i][0].x *= o; acc[i][0].y *= o; acc[i][1].x *= o; acc[i][1].y *= o;
+        if (DX) {
+            const float4 xv = ld4f((const T *)p.x + xo + (size_t)r * HP + tx * 4);
+            dd2[i] = xv.x * acc[i][0].x + xv.y * acc[i][0].y + xv.z * acc[i][1].x + xv.w * acc[i][1].y;
+        }
     }
+    for (int ct = ct0; ct < ct1; ++ct) {
+        // masked tile: a[k = column of the mask][row]
 #pragma unroll
-    for (int q = 0; q < WD / 64; ++q) {
-        if (MODE < 2) {
-            for (int idx = tid; idx < 64 * KD; idx += 256) {
-                const int jl = idx / KD, k = idx % KD;
-                Cv[jl * KP + k] = St[(size_t)(64 * q + jl) * NS + k];
-            }
-        } else {
-            for (int idx = tid; idx < 64 * 64; idx += 256) {
-                const int pp = idx >> 6, jl = idx & 63;
-                Cv[jl * KP + pp] = St[(size_t)pp * NS + 64 * q + jl];
+        for (int k = 0; k < 4; ++k) {
+            float *e = reinterpret_cast<float *>(&ra[k]);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                // as tile_load laid them out: not DX (transposed) row t, column s; DX (direct) row t, column s
+                const int t = DX ? ct * 64 + ty + 16 * k : r0 + (tid & 7) + 8 * (tid >> 5);
+                const int s = DX ? r0 + tx * 4 + i : ct * 64 + ((tid >> 3) & 3) * 4 + 16 * k + i;
+                e[i] = s <= t ? e[i] * expf(fminf(css[t] - css[s], 0.f)) * (DX ? 1.f : dts[s]) : 0.f;
             }
         }
+        tile_store(sm.a, ra, !DX);
+        tile_store(sm.b, rb, false);
         __syncthreads();
-        float s[4][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) s[i][j] = 0.f;
-#pragma unroll 4
-        for (int k = 0; k < KD; ++k) {
-            float rv[4], cv[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) rv[i] = Rv[(ty * 4 + i) * KP + k];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cv[j] = Cv[(tx + 16 * j) * KP + k];
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) s[i][j] = fmaf(rv[i], cv[j], s[i][j]);
-        }
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][4 * q + j] = fmaf(offs[i], s[i][j], acc[i][4 * q + j]);
+        if (ct + 1 < ct1) load_vals(ct + 1);
+        tile_mma(acc, sm.a, sm.b);
         __syncthreads();
     }
-
-    // epilogues
-    if (MODE == MP_FWD) {
-        const float Dh = __ldg(p.D + h);
-        T *yb = (T *)p.y + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
+    const float Dh = __ldg(p.D + h) + (DX ? p.dx_skip : 0.f);      // dx: D dy, plus dy itself under a skip connection
+    float dsum = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int r = r0 + ty * 4 + i, pp = tx + 16 * j;
-                const float xv = ldf(xlike_base_x + (size_t)r * HP + pp);
-                stf(yb + (size_t)r * HP + pp, fmaf(Dh, xv, acc[i][j]));
+    for (int i = 0; i < 4; ++i) {
+        const int r = r0 + ty * 4 + i;
+        const size_t o = xo + (size_t)r * HP + tx * 4;
+        const float4 v = ld4f((const T *)(DX ? p.dy : p.x) + o);
+        const float s = DX ? dts[r] : 1.f;
+        st4((T *)(DX ? p.dx : p.y) + o, make_float4(fmaf(Dh, v.x, s * acc[i][0].x), fmaf(Dh, v.y, s * acc[i][0].y), fmaf(Dh, v.z, s * acc[i][1].x),
+                                                    fmaf(Dh, v.w, s * acc[i][1].y)));
+        if (DX) {
+            const float4 xv = ld4f((const T *)p.x + o);
+            const float dd = sum_tx(xv.x * acc[i][0].x + xv.y * acc[i][0].y + xv.z * acc[i][1].x + xv.w * acc[i][1].y);
+            const float d2 = sum_tx(dd2[i]);
+            dsum += v.x * xv.x + v.y * xv.y + v.z * xv.z + v.w * xv.w;
+            if (tx == 0) {
+                p.ddt_dir[vec_off(p, b, h, c) + r] = dd;
+                p.psi2[vec_off(p, b, h, c) + r] = dts[r] * d2;
             }
-    } else if (MODE == MP_BWD_DX) {
-        const float Dh = __ldg(p.D + h) + p.dx_skip;      // D dy, plus dy itself under a skip connection
-        T *dxb = (T *)p.dx + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
-        float dsum = 0.f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = r0 + ty * 4 + i;
-            float dd = 0.f;
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int pp = tx + 16 * j;
-                const float xv = ldf(xlike_base_x + (size_t)r * HP + pp);
-                const float dyv = ldf(xlike_base_dy + (size_t)r * HP + pp);
-                stf(dxb + (size_t)r * HP + pp, fmaf(Dh, dyv, dts[r] * acc[i][j]));
-                dd = fmaf(xv, acc[i][j], dd);
-                dsum = fmaf(dyv, xv, dsum);
-            }
-#pragma unroll
-            for (int off = 8; off > 0; off >>= 1) dd += __shfl_xor_sync(0xffffffffu, dd, off);
-            if (tx == 0) p.ddt_dir[vec_off(p, b, h, c) + r] = dd;
         }
-        // deterministic block sum of dy*x
+    }
+    if (DX) {       // deterministic block sum of dy*x
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, off);
-        if ((tid & 31) == 0) Mk[tid >> 5] = dsum;
+        if ((tid & 31) == 0) red[tid >> 5] = dsum;
         __syncthreads();
         if (tid == 0) {
             float s = 0.f;
 #pragma unroll
-            for (int w = 0; w < 8; ++w) s += Mk[w];
+            for (int w = 0; w < 8; ++w) s += red[w];
             p.dDp[((((size_t)b * p.H + h) * p.nct + p.c0 + c) << 2) + rt] = s;
         }
-    } else {
-        // per-head partial dC / dB rows: [B, seg, G, nsl, N]
-        // (acc here already holds intra-chunk + inter-chunk parts; dot_intra was taken before)
-        float *pb = (MODE == MP_DC) ? p.pC : p.pB;
-        const int sl = (h % p.hpg) / (p.hpg / p.nsl);
-        const size_t segcap = (size_t)p.ncs * Q;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = r0 + ty * 4 + i;
-            const size_t tl = (size_t)c * Q + r;
-            float *row = pb + ((((size_t)b * segcap + tl) * p.G + g) * p.nsl + sl) * NS;
-            float dot = 0.f;
-#pragma unroll
-            for (int j = 0; j < NJ; ++j) {
-                const int nn = tx + 16 * j;
-                row[nn] = acc[i][j];
-                dot = fmaf(ldf((MODE == MP_DC ? bc_base_C : bc_base_B) + (size_t)r * GN + nn), acc[i][j], dot);
-            }
-#pragma unroll
-            for (int off = 8; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-            if (tx == 0) {
-                if (MODE == MP_DC) {
-                    p.rho[vec_off(p, b, h, c) + r] = dot;
-                } else {
-                    p.psi[vec_off(p, b, h, c) + r] = dot_intra[i];
-                    p.psi2[vec_off(p, b, h, c) + r] = dot - dot_intra[i];
-                }
-            }
-        }
     }
-}
-
-template <typename T, int NS, int MODE>
-static cudaError_t launch_mp(const SegParams &p, cudaStream_t st) {
-    constexpr int KD = (MODE < 2) ? NS : 64;
-    constexpr int WD = (MODE < 2) ? 64 : NS;
-    const size_t smem = sizeof(float) * (2 * 64 * (KD + 1) + 64 * WD + 64 * 65 + 512);
-    cudaError_t e = cudaFuncSetAttribute(k_masked_product_simt<T, NS, MODE>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid(p.nc * (p.Q / 64), p.H, p.B);
-    k_masked_product_simt<T, NS, MODE><<<grid, 256, smem, st>>>(p);
-    return cudaGetLastError();
 }
 
 template <typename T, int NS>
-static cudaError_t launch_mp_mode(const SegParams &p, int mode, cudaStream_t st) {
-    switch (mode) {
-        case MP_FWD: return launch_mp<T, NS, MP_FWD>(p, st);
-        case MP_BWD_DX: return launch_mp<T, NS, MP_BWD_DX>(p, st);
-        case MP_DC: return launch_mp<T, NS, MP_DC>(p, st);
-        default: return launch_mp<T, NS, MP_DB>(p, st);
-    }
+__global__ void __launch_bounds__(256) k_simt_y(SegParams p) {
+    pdl_launch_dependents();
+    pdl_wait();
+    __shared__ SimtTiles sm;
+    __shared__ float css[256], dts[256];
+    const int nrt = p.Q >> 6;
+    simt_row_tile<T, NS, false>(p, sm, css, dts, nullptr, blockIdx.x / nrt, blockIdx.x % nrt, blockIdx.y, blockIdx.z);
 }
 
-cudaError_t launch_masked_product_simt(const SegParams &p, int dtype, int mode, cudaStream_t st) {
-    if (dtype == SSD_DTYPE_F32)
-        return p.N == 64 ? launch_mp_mode<float, 64>(p, mode, st) : launch_mp_mode<float, 128>(p, mode, st);
-    return p.N == 64 ? launch_mp_mode<__nv_bfloat16, 64>(p, mode, st)
-                     : launch_mp_mode<__nv_bfloat16, 128>(p, mode, st);
+// The large kernel of the backward: tiles of dx, and the partial slices of dB and dC.  Per (chunk, head range):
+//   causal tile pair (tt, ts): W_h = (dy_tt x_ts^T) o mask per head, rho / psi partial sums of W_h o CB, head sum of W_h; then
+//                  slices dC[tt] = Wsum B_ts and dB[ts] = Wsum^T C_tt
+//   inter dC, tile tt : sum_h e^{cs_t} dy_t H_in (and rho2 per head);  inter dB, tile ts : sum_h dt_s e^{cs_last-cs_s} x_s Gout
+// A slice has Q/64 + 1 slots per head range: dC by ts (dB by tt), the last one the inter-chunk term.
+template <typename T, int NS>
+__global__ void __launch_bounds__(256) k_simt_bwd(SegParams p, int n_dx) {
+    pdl_launch_dependents();
+    pdl_wait();
+    __shared__ SimtTiles sm;
+    __shared__ float css[256], dts[256], red[8][64];
+    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, npair = nrt * (nrt + 1) / 2;
+    int id = blockIdx.x;
+    if (id >= (int)gridDim.x - n_dx) {
+        id -= (int)gridDim.x - n_dx;
+        const int rt = id % nrt, h = (id / nrt) % p.H, c = (id / (nrt * p.H)) % p.nc, b = id / (nrt * p.H * p.nc);
+        simt_row_tile<T, NS, true>(p, sm, css, dts, red[0], c, rt, h, b);
+        return;
+    }
+    const int per = npair + 2 * nrt, role = id % per;
+    id /= per;
+    const int rng = p.nsl / (nrt + 1);                         // head ranges per group
+    const int sl = id % rng, g = (id / rng) % p.G, c = (id / (rng * p.G)) % p.nc, b = id / (rng * p.G * p.nc);
+    const int hps = (p.hpg + rng - 1) / rng, h0 = g * p.hpg + sl * hps, h1 = min(h0 + hps, (g + 1) * p.hpg);
+    const size_t tok0 = (size_t)p.t0 + (size_t)c * Q, HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
+    const T *xb = (const T *)p.x + (size_t)b * p.x_bs + tok0 * HP, *dyb = (const T *)p.dy + (size_t)b * p.x_bs + tok0 * HP;
+    const T *Bb = (const T *)p.Bm + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS, *Cb = (const T *)p.Cm + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS;
+    auto load_vec = [&](int h) {
+        for (int t = tid; t < Q; t += 256) {
+            css[t] = p.cs[vec_off(p, b, h, c) + t];
+            dts[t] = p.dtT[vec_off(p, b, h, c) + t];
+        }
+    };
+    auto write_slice = [&](float *part, const float2 (&acc)[4][2], int row0, int slot, int n0) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const size_t tl = (size_t)b * p.ncs * Q + (size_t)c * Q + row0 + ty * 4 + i;
+            *reinterpret_cast<float4 *>(part + ((tl * p.G + g) * p.nsl + sl * (nrt + 1) + slot) * NS + n0 + tx * 4) =
+                make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+        }
+    };
+    float4 ra[4], rb[4];
+    float2 acc[4][2];
+    if (role < npair) {
+        int tt, ts;
+        pair_of(role, tt, ts);
+        const float *CB = cb_of(p, b, c, g) + (size_t)(tt * 64 + ty * 4) * Q + ts * 64 + tx * 4;
+        float4 cb[4];
+        float ws[4][4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            cb[i] = *reinterpret_cast<const float4 *>(CB + (size_t)i * Q);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) ws[i][j] = 0.f;
+        }
+        tile_load(ra, dyb + (size_t)tt * 64 * HP + (size_t)h0 * 64, HP, true);
+        tile_load(rb, xb + (size_t)ts * 64 * HP + (size_t)h0 * 64, HP, true);
+        for (int h = h0; h < h1; ++h) {
+            load_vec(h);
+            tile_store(sm.a, ra, true);
+            tile_store(sm.b, rb, true);
+            __syncthreads();
+            if (h + 1 < h1) {
+                tile_load(ra, dyb + (size_t)tt * 64 * HP + (size_t)(h + 1) * 64, HP, true);
+                tile_load(rb, xb + (size_t)ts * 64 * HP + (size_t)(h + 1) * 64, HP, true);
+            }
+            zero_acc(acc);
+            tile_mma(acc, sm.a, sm.b);
+            float col[4] = {0.f, 0.f, 0.f, 0.f};
+            const size_t vo = (vec_off(p, b, h, c) * nrt);      // rho, psi: [B,H,ncs,Q/64 tiles,Q]
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int t = tt * 64 + ty * 4 + i;
+                const float s4[4] = {acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y}, c4[4] = {cb[i].x, cb[i].y, cb[i].z, cb[i].w};
+                float row = 0.f;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int s = ts * 64 + tx * 4 + j;
+                    const float w = s <= t ? s4[j] * expf(fminf(css[t] - css[s], 0.f)) * dts[s] : 0.f;
+                    ws[i][j] += w;
+                    row = fmaf(w, c4[j], row);
+                    col[j] = fmaf(w, c4[j], col[j]);
+                }
+                row = sum_tx(row);
+                if (tx == 0) p.rho[vo + (size_t)ts * Q + t] = row;
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                col[j] += __shfl_xor_sync(0xffffffffu, col[j], 16);
+                if ((tid & 16) == 0) red[tid >> 5][tx * 4 + j] = col[j];
+            }
+            __syncthreads();
+            if (tid < 64) {
+                float s = 0.f;
+#pragma unroll
+                for (int w = 0; w < 8; ++w) s += red[w][tid];
+                p.psi[vo + (size_t)tt * Q + ts * 64 + tid] = s;
+            }
+            // red, css and dts are rewritten only after the next head's first barrier or by the threads that read them here
+            __syncthreads();
+        }
+        // dC[tt] = Wsum B_ts: a[k = s][t]
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            *reinterpret_cast<float4 *>(&sm.a[tx * 4 + j][ty * 4]) = make_float4(ws[0][j], ws[1][j], ws[2][j], ws[3][j]);
+        for (int n0 = 0; n0 < NS; n0 += 64) {
+            tile_load(rb, Bb + (size_t)ts * 64 * GN + n0, GN, false);
+            tile_store(sm.b, rb, false);
+            __syncthreads();
+            zero_acc(acc);
+            tile_mma(acc, sm.a, sm.b);
+            write_slice(p.pC, acc, tt * 64, ts, n0);
+            __syncthreads();
+        }
+        // dB[ts] = Wsum^T C_tt: a[k = t][s]
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4 *>(&sm.a[ty * 4 + i][tx * 4]) = make_float4(ws[i][0], ws[i][1], ws[i][2], ws[i][3]);
+        for (int n0 = 0; n0 < NS; n0 += 64) {
+            tile_load(rb, Cb + (size_t)tt * 64 * GN + n0, GN, false);
+            tile_store(sm.b, rb, false);
+            __syncthreads();
+            zero_acc(acc);
+            tile_mma(acc, sm.a, sm.b);
+            write_slice(p.pB, acc, ts * 64, tt, n0);
+            __syncthreads();
+        }
+        return;
+    }
+    // inter-chunk terms of one row tile: the head's rows scaled per row, times the chunk state (rows p)
+    const bool isC = role - npair < nrt;
+    const int rt = (role - npair) % nrt;
+    float2 tot[NS / 64][4][2];
+#pragma unroll
+    for (int m = 0; m < NS / 64; ++m) zero_acc(tot[m]);
+    for (int h = h0; h < h1; ++h) {
+        const float *St = isC ? p.Hst + slot_off(p, b, c, h) : p.Gst + slot_off(p, b, c + 1, h);
+        load_vec(h);
+        tile_load(ra, (isC ? dyb : xb) + (size_t)rt * 64 * HP + (size_t)h * 64, HP, true);
+        tile_load_ws(rb, St, NS, false);
+        tile_store(sm.a, ra, true);
+        float rho2[4] = {0.f, 0.f, 0.f, 0.f}, sc[4];
+#pragma unroll
+        for (int m = 0; m < NS / 64; ++m) {
+            tile_store(sm.b, rb, false);
+            __syncthreads();
+            if (m == 0) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = rt * 64 + ty * 4 + i;
+                    sc[i] = isC ? expf(css[r]) : dts[r] * expf(fminf(css[Q - 1] - css[r], 0.f));
+                }
+            }
+            if (m + 1 < NS / 64) tile_load_ws(rb, St + 64 * (m + 1), NS, false);
+            zero_acc(acc);
+            tile_mma(acc, sm.a, sm.b);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 s2 = make_float2(sc[i], sc[i]);
+                const float2 a0 = __fmul2_rn(acc[i][0], s2), a1 = __fmul2_rn(acc[i][1], s2);
+                tot[m][i][0] = __fadd2_rn(tot[m][i][0], a0);
+                tot[m][i][1] = __fadd2_rn(tot[m][i][1], a1);
+                if (isC) {
+                    const float4 cv = ld4f(Cb + (size_t)(rt * 64 + ty * 4 + i) * GN + m * 64 + tx * 4);
+                    rho2[i] += cv.x * a0.x + cv.y * a0.y + cv.z * a1.x + cv.w * a1.y;
+                }
+            }
+            __syncthreads();
+        }
+        if (isC) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float v = sum_tx(rho2[i]);
+                if (tx == 0) p.rho2[vec_off(p, b, h, c) + rt * 64 + ty * 4 + i] = v;
+            }
+        }
+    }
+#pragma unroll
+    for (int m = 0; m < NS / 64; ++m) write_slice(isC ? p.pC : p.pB, tot[m], rt * 64, nrt, m * 64);
+}
+
+template <typename T, int NS>
+static cudaError_t simt_launch(const SegParams &p, int what, cudaStream_t st) {
+    const int nrt = p.Q / 64, npair = nrt * (nrt + 1) / 2, nsum = p.nc * (NS / 64) * p.H * p.B;
+    switch (what) {
+        case SIMT_SUMS: return launch_pdl(k_simt_sums<T, NS, STATE_MODE_FWD>, dim3(nsum + p.nc * npair * p.G * p.B), dim3(256), 0, st, p);
+        case SIMT_DSTATE: return launch_pdl(k_simt_sums<T, NS, STATE_MODE_DSTATE>, dim3(nsum), dim3(256), 0, st, p);
+        case SIMT_Y: return launch_pdl(k_simt_y<T, NS>, dim3(p.nc * nrt, p.H, p.B), dim3(256), 0, st, p);
+        default: {
+            const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 1)) * p.G * p.B;
+            return launch_pdl(k_simt_bwd<T, NS>, dim3(n_bc + n_dx), dim3(256), 0, st, p, n_dx);
+        }
+    }
+}
+cudaError_t launch_simt(const SegParams &p, int dtype, int what, cudaStream_t st) {
+    if (dtype == SSD_DTYPE_F32) return p.N == 64 ? simt_launch<float, 64>(p, what, st) : simt_launch<float, 128>(p, what, st);
+    return p.N == 64 ? simt_launch<__nv_bfloat16, 64>(p, what, st) : simt_launch<__nv_bfloat16, 128>(p, what, st);
 }
 
 // ------------------------------------------------------------------ da, ddt, dA partial
@@ -582,109 +694,97 @@ cudaError_t launch_masked_product_simt(const SegParams &p, int dtype, int mode, 
 // + sum_{t'>=t} rho_inter_t'                outputs at/after t reading the chunk-entry state (rho2)
 // + sum_{s<t}   psi2_s                      inputs before t feeding the chunk-exit gradient
 // + exp(cs_last) <Gout, H_in>
-// (the CUDA-core kernels store rho = rho_intra + rho_inter as one vector and no rho2).  Suffix/prefix scans: serial inside a lane,
+// Suffix/prefix scans: serial inside a lane,
 // warp shuffles across lanes.  Then ddt = ddt_direct + A da, dA partial = sum_t dt_t da_t.
-// One CTA per (chunk, HB consecutive heads), one warp per head.  ddt is [B, L, H]: a head's values of consecutive
-// steps lie H floats apart, so the HB heads' results go through a shared-memory tile and leave as rows of HB
-// consecutive floats (whole 32-byte sectors for HB = 8) instead of one 4-byte store per sector.
-template <int HB>
-__global__ void __launch_bounds__(HB * 32) k_bwd_finish(SegParams p) {
-    pdl_launch_dependents();
-    pdl_wait();
-    __shared__ float tile[HB > 1 ? 256 * (HB + 1) : 1];
+// One CTA per (chunk, eight consecutive heads), one warp per head.  ddt is [B, L, H]: a head's values of consecutive
+// steps lie H floats apart, so the eight heads' results go through a shared-memory tile and leave as rows of eight
+// consecutive floats (whole 32-byte sectors) instead of one 4-byte store per sector.
+constexpr int FIN_HB = 8;
+__device__ __forceinline__ void bwd_finish(const SegParams &p, int id) {
+    __shared__ float tile[256 * (FIN_HB + 1)];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int c = blockIdx.x, h = blockIdx.y * HB + warp, b = blockIdx.z;
+    const int nhb = (p.H + FIN_HB - 1) / FIN_HB;
+    const int c = id % p.nc, hb = (id / p.nc) % nhb, b = id / (p.nc * nhb), h = hb * FIN_HB + warp, nh = min(FIN_HB, p.H - hb * FIN_HB);
     const int Q = p.Q, per = Q >> 5;
-    const size_t vo = vec_off(p, b, h, c) + (size_t)lane * per;
-    float gh = 0.f;
-    for (int i = 0; i < p.ngh; ++i) gh += p.ghdot[((((size_t)b * p.H + h) * p.ncs + c) << 4) + i];
-    float dtv[8], dd[8], sfx[8], pfx[8];
-    float run = 0.f;
+    if (warp < nh) {
+        const size_t hc = ((size_t)b * p.H + h) * p.ncs + c, vo = hc * Q + (size_t)lane * per;
+        float gh = 0.f;
+        for (int i = 0; i < p.ngh; ++i) gh += p.ghdot[(hc << 4) + i];
+        float dtv[8], dd[8], sfx[8], pfx[8];
+        float run = 0.f;
 #pragma unroll
-    for (int j = 7; j >= 0; --j)
-        if (j < per) {
-            dtv[j] = p.dtT[(((size_t)b * p.H + h) * p.ncs + c) * p.dt_stride + lane * per + j];
-            dd[j] = p.ddt_dir[vo + j];
-            run += (p.rho[vo + j] - p.psi[vo + j]) + (p.rho2 ? p.rho2[vo + j] + p.rho2b[vo + j] : 0.f);
-            sfx[j] = run;
+        for (int j = 7; j >= 0; --j)
+            if (j < per) {
+                dtv[j] = p.dtT[hc * p.dt_stride + lane * per + j];
+                dd[j] = p.ddt_dir[vo + j];
+                float r1, p1;
+                if (p.tiles) {      // CUDA-core path: partial sums per 64 x 64 tile of the masked products
+                    const size_t to = hc * p.tiles * Q + lane * per + j;
+                    const int t0 = (lane * per + j) >> 6;
+                    r1 = p.rho[to];
+                    for (int t = 1; t <= t0; ++t) r1 += p.rho[to + (size_t)t * Q];
+                    p1 = p.psi[to + (size_t)t0 * Q];
+                    for (int t = t0 + 1; t < p.tiles; ++t) p1 += p.psi[to + (size_t)t * Q];
+                } else {
+                    r1 = p.rho[vo + j];
+                    p1 = p.psi[vo + j];
+                }
+                run += (r1 - p1) + (p.rho2b ? p.rho2[vo + j] + p.rho2b[vo + j] : p.rho2[vo + j]);
+                sfx[j] = run;
+            }
+        float incl = run;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float t = __shfl_down_sync(0xffffffffu, incl, off);
+            if (lane + off < 32) incl += t;
         }
-    float incl = run;
+        float excl = __shfl_down_sync(0xffffffffu, incl, 1);
+        if (lane == 31) excl = 0.f;
+        // exclusive prefix of psi2
+        float prun = 0.f;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float t = __shfl_down_sync(0xffffffffu, incl, off);
-        if (lane + off < 32) incl += t;
+        for (int j = 0; j < 8; ++j)
+            if (j < per) {
+                pfx[j] = prun;
+                prun += p.psi2[vo + j];
+            }
+        float pincl = prun;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float t = __shfl_up_sync(0xffffffffu, pincl, off);
+            if (lane >= off) pincl += t;
+        }
+        float pexcl = __shfl_up_sync(0xffffffffu, pincl, 1);
+        if (lane == 0) pexcl = 0.f;
+        const float Ah = __ldg(p.A + h);
+        float sA = 0.f;
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+            if (j < per) {
+                const float da = ((sfx[j] + excl) + (pfx[j] + pexcl)) + gh;
+                tile[(lane * per + j) * (FIN_HB + 1) + warp] = fmaf(Ah, da, dd[j]);
+                sA = fmaf(dtv[j], da, sA);
+            }
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) sA += __shfl_xor_sync(0xffffffffu, sA, off);
+        if (lane == 0) p.dAp[((size_t)b * p.H + h) * p.nct + p.c0 + c] = sA;
     }
-    float excl = __shfl_down_sync(0xffffffffu, incl, 1);
-    if (lane == 31) excl = 0.f;
-    // exclusive prefix of psi2
-    float prun = 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        if (j < per) {
-            pfx[j] = prun;
-            prun += p.psi2[vo + j];
-        }
-    float pincl = prun;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float t = __shfl_up_sync(0xffffffffu, pincl, off);
-        if (lane >= off) pincl += t;
+    __syncthreads();
+    float *out = p.ddt + (size_t)b * p.dt_bs + ((size_t)p.t0 + (size_t)c * Q) * p.H + (size_t)hb * FIN_HB;
+    for (int i = threadIdx.x; i < Q * FIN_HB; i += 256) {
+        const int t = i / FIN_HB, hh = i % FIN_HB;
+        if (hh < nh) out[(size_t)t * p.H + hh] = tile[t * (FIN_HB + 1) + hh];
     }
-    float pexcl = __shfl_up_sync(0xffffffffu, pincl, 1);
-    if (lane == 0) pexcl = 0.f;
-    const float Ah = __ldg(p.A + h);
-    const size_t tok0 = (size_t)p.t0 + (size_t)c * Q + (size_t)lane * per;
-    float sA = 0.f;
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-        if (j < per) {
-            const float da = ((sfx[j] + excl) + (pfx[j] + pexcl)) + gh;
-            const float v = fmaf(Ah, da, dd[j]);
-            if (HB > 1) tile[(lane * per + j) * (HB + 1) + warp] = v;
-            else p.ddt[(size_t)b * p.dt_bs + (tok0 + j) * p.H + h] = v;
-            sA = fmaf(dtv[j], da, sA);
-        }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) sA += __shfl_xor_sync(0xffffffffu, sA, off);
-    if (lane == 0) p.dAp[((size_t)b * p.H + h) * p.nct + p.c0 + c] = sA;
-    if (HB > 1) {
-        __syncthreads();
-        float *out = p.ddt + (size_t)b * p.dt_bs + ((size_t)p.t0 + (size_t)c * Q) * p.H + (size_t)blockIdx.y * HB;
-        for (int i = threadIdx.x; i < Q * HB; i += HB * 32) {
-            const int t = i / HB, hh = i % HB;
-            out[(size_t)t * p.H + hh] = tile[t * (HB + 1) + hh];
-        }
-    }
-}
-
-cudaError_t launch_bwd_finish(const SegParams &p, cudaStream_t st) {
-    if (p.H % 8 == 0) return launch_pdl(k_bwd_finish<8>, dim3(p.nc, p.H / 8, p.B), dim3(256), 0, st, p);
-    if (p.H % 4 == 0) return launch_pdl(k_bwd_finish<4>, dim3(p.nc, p.H / 4, p.B), dim3(128), 0, st, p);
-    return launch_pdl(k_bwd_finish<1>, dim3(p.nc, p.H, p.B), dim3(32), 0, st, p);
 }
 
 // ------------------------------------------------------------------ dB / dC: sum the head slices of a group
 // Four consecutive n per thread (16-byte loads of the fp32 partial slices, one 8- or 16-byte store): the kernel only
 // moves bytes.  The order of the additions per element is fixed: slices in order.
-__device__ __forceinline__ void add4(float4 &a, const float4 &b) {
-    a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
-}
-__device__ __forceinline__ void st4(float *p, const float4 &v) { *reinterpret_cast<float4 *>(p) = v; }
-__device__ __forceinline__ void st4(__nv_bfloat16 *p, const float4 &v) {
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
-    uint2 pk;
-    pk.x = *reinterpret_cast<const unsigned int *>(&lo);
-    pk.y = *reinterpret_cast<const unsigned int *>(&hi);
-    *reinterpret_cast<uint2 *>(p) = pk;
-}
-
 template <typename T>
-__global__ void __launch_bounds__(256) k_reduce_dbdc(SegParams p) {
-    pdl_launch_dependents();
-    pdl_wait();
+__device__ __forceinline__ void reduce_dbdc(const SegParams &p, int id) {
     const int N4 = p.N >> 2;
     const size_t total = (size_t)p.B * p.nc * p.Q * p.G * N4;
-    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+    const size_t i = (size_t)id * 256 + threadIdx.x;
     if (i >= total) return;
     const int n = (int)(i % N4) * 4;
     size_t r = i / N4;
@@ -697,35 +797,60 @@ __global__ void __launch_bounds__(256) k_reduce_dbdc(SegParams p) {
     float4 sB = make_float4(0.f, 0.f, 0.f, 0.f), sC = sB;
     auto ld = [](const float *q) { return *reinterpret_cast<const float4 *>(q); };
     const size_t src = ((((size_t)b * segcap + tl) * p.G + g) * p.nsl) * p.N + n;
-    for (int s = 0; s < p.nsl; ++s) {
-        add4(sB, ld(p.pB + src + (size_t)s * p.N));
-        add4(sC, ld(p.pC + src + (size_t)s * p.N));
+    if (p.tiles) {
+        // CUDA-core path: per head range one slot per 64-step tile and one for the inter-chunk term; a row of tile rt has dC
+        // slots 0 .. rt and dB slots rt .. tiles - 1
+        const int rt = (int)(tl % (size_t)p.Q) >> 6;
+        for (int s0 = 0; s0 < p.nsl; s0 += p.tiles + 1)
+            for (int t = 0; t <= p.tiles; ++t) {
+                if (t >= rt) add4(sB, ld(p.pB + src + (size_t)(s0 + t) * p.N));
+                if (t <= rt || t == p.tiles) add4(sC, ld(p.pC + src + (size_t)(s0 + t) * p.N));
+            }
+    } else {
+        for (int s = 0; s < p.nsl; ++s) {
+            add4(sB, ld(p.pB + src + (size_t)s * p.N));
+            add4(sC, ld(p.pC + src + (size_t)s * p.N));
+        }
     }
     const size_t dst = (size_t)b * p.bc_bs + ((size_t)p.t0 + tl) * p.G * p.N + (size_t)g * p.N + n;
     st4((T *)p.dB + dst, sB);
     st4((T *)p.dC + dst, sC);
 }
 
-cudaError_t launch_reduce_dbdc(const SegParams &p, int dtype, cudaStream_t st) {
+// Both in one launch: the two short finishing steps of a segment.
+template <typename T>
+__global__ void __launch_bounds__(256) k_bwd_tail(SegParams p, int nfin) {
+    pdl_launch_dependents();
+    pdl_wait();
+    if ((int)blockIdx.x < nfin) bwd_finish(p, blockIdx.x);
+    else reduce_dbdc<T>(p, blockIdx.x - nfin);
+}
+
+cudaError_t launch_bwd_tail(const SegParams &p, int dtype, cudaStream_t st) {
+    const int nfin = p.nc * ((p.H + FIN_HB - 1) / FIN_HB) * p.B;
     const size_t total = (size_t)p.B * p.nc * p.Q * p.G * (p.N / 4);
-    const unsigned blocks = (unsigned)((total + 255) / 256);
-    if (dtype == SSD_DTYPE_F32) return launch_pdl(k_reduce_dbdc<float>, dim3(blocks), dim3(256), 0, st, p);
-    return launch_pdl(k_reduce_dbdc<__nv_bfloat16>, dim3(blocks), dim3(256), 0, st, p);
+    const dim3 grid((unsigned)(nfin + (total + 255) / 256));
+    if (dtype == SSD_DTYPE_F32) return launch_pdl(k_bwd_tail<float>, grid, dim3(256), 0, st, p, nfin);
+    return launch_pdl(k_bwd_tail<__nv_bfloat16>, grid, dim3(256), 0, st, p, nfin);
 }
 
 // ------------------------------------------------------------------ dA, dD over (batch, chunks)
-// One warp per head; lanes stride over the per-chunk partials in fp64, then a fixed shuffle tree.
-__global__ void __launch_bounds__(32) k_final_dAdD(SegParams p, float *dA, float *dD, int accumulate) {
+// One CTA per head; threads stride over the per-chunk partials in fp64, then a fixed tree.
+__global__ void __launch_bounds__(256) k_final_dAdD(SegParams p, float *dA, float *dD, int accumulate) {
     pdl_launch_dependents();
     pdl_wait();
-    const int h = blockIdx.x, lane = threadIdx.x;
-    const int nrt = p.ndd;
+    __shared__ double red[2][8];
+    const int h = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     double sA = 0.0, sD = 0.0;
     for (int b = 0; b < p.B; ++b) {
         const size_t base = ((size_t)b * p.H + h) * p.nct;
-        for (int c = lane; c < p.nct; c += 32) {
+        for (int c = threadIdx.x; c < p.nct; c += 256) {
             sA += (double)p.dAp[base + c];
-            for (int r = 0; r < nrt; ++r) sD += (double)p.dDp[((base + c) << 2) + r];
+            const float4 d4 = *reinterpret_cast<const float4 *>(p.dDp + ((base + c) << 2));
+            const float d[4] = {d4.x, d4.y, d4.z, d4.w};
+#pragma unroll
+            for (int r = 0; r < 4; ++r)
+                if (r < p.ndd) sD += (double)d[r];
         }
     }
 #pragma unroll
@@ -734,13 +859,24 @@ __global__ void __launch_bounds__(32) k_final_dAdD(SegParams p, float *dA, float
         sD += __shfl_xor_sync(0xffffffffu, sD, off);
     }
     if (lane == 0) {
-        dA[h] = accumulate ? dA[h] + (float)sA : (float)sA;
-        dD[h] = accumulate ? dD[h] + (float)sD : (float)sD;
+        red[0][warp] = sA;
+        red[1][warp] = sD;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        double a = 0.0, d = 0.0;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            a += red[0][w];
+            d += red[1][w];
+        }
+        dA[h] = accumulate ? dA[h] + (float)a : (float)a;
+        dD[h] = accumulate ? dD[h] + (float)d : (float)d;
     }
 }
 
 cudaError_t launch_final_dAdD(const SegParams &p, float *dA, float *dD, bool accumulate, cudaStream_t st) {
-    return launch_pdl(k_final_dAdD, dim3(p.H), dim3(32), 0, st, p, dA, dD, accumulate ? 1 : 0);
+    return launch_pdl(k_final_dAdD, dim3(p.H), dim3(256), 0, st, p, dA, dD, accumulate ? 1 : 0);
 }
 
 }  // namespace ssd
