@@ -8,8 +8,8 @@
 // Bandwidth-shaped kernels over 512 adjacent channels per CTA, a thread owning 4 of them with a sliding window in
 // registers; rows reach shared memory by bulk async copies, one per token row (the channels of a row are contiguous:
 // up to 1 KB), so that many kilobytes per SM are in flight without holding registers, and results go straight to
-// global memory (8 or 16 bytes per thread, coalesced over the channels).  Forward: one 32-token tile per CTA, staged
-// whole (plus the three-token halo).  Backward: a range of tokens per CTA streamed through a ring of 8-token stages.
+// global memory (8 or 16 bytes per thread, coalesced over the channels).  A CTA walks a range of tokens, streamed through a ring
+// of 8-token stages.
 // Weight and bias gradients: one partial per backward CTA, then a fixed-order sum (no atomics).
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
@@ -22,27 +22,10 @@ namespace {
 
 constexpr int CV_THREADS = 128;   // x 4 channels = 512 channels per CTA
 constexpr int CV_CH = 4;          // channels per thread: one 8-byte bf16 vector (16 bytes in fp32)
-constexpr int CV_TILE_F = 32;     // tokens per CTA, forward
 
-// 1 / (1 + e^-x) from one ex2.approx and one rcp.approx (relative error of the order of 1e-7; the kernels are bound
-// by instruction issue, not by memory, and an IEEE division alone would cost as much as the rest of an element)
-__device__ __forceinline__ float sigmoid_fast(float x) {
-    float e, r;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(x * -1.4426950408889634f));
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.f + e));
-    return r;
-}
-
-template <typename T> __device__ __forceinline__ void ld4(const T *p, float *f);
-template <> __device__ __forceinline__ void ld4<float>(const float *p, float *f) {
+__device__ __forceinline__ void ld4(const float *p, float *f) {
     const float4 a = *reinterpret_cast<const float4 *>(p);
     f[0] = a.x; f[1] = a.y; f[2] = a.z; f[3] = a.w;
-}
-template <> __device__ __forceinline__ void ld4<__nv_bfloat16>(const __nv_bfloat16 *p, float *f) {
-    const uint2 v = *reinterpret_cast<const uint2 *>(p);
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.x));
-    const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.y));
-    f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y;
 }
 template <typename T> __device__ __forceinline__ void st4(T *p, const float *f);
 template <> __device__ __forceinline__ void st4<float>(float *p, const float *f) {
@@ -56,7 +39,7 @@ template <> __device__ __forceinline__ void st4<__nv_bfloat16>(__nv_bfloat16 *p,
     *reinterpret_cast<uint2 *>(p) = v;
 }
 
-// The same four channels as two pairs, for the packed two-lane fp32 instructions of the backward kernel.
+// Four channels as two pairs, for the packed two-lane fp32 instructions.
 template <typename T> __device__ __forceinline__ void ld2x2(const T *p, float2 &a, float2 &b);
 template <> __device__ __forceinline__ void ld2x2<float>(const float *p, float2 &a, float2 &b) {
     const float4 v = *reinterpret_cast<const float4 *>(p);
@@ -68,6 +51,8 @@ template <> __device__ __forceinline__ void ld2x2<__nv_bfloat16>(const __nv_bflo
     a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.x));
     b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.y));
 }
+// 1 / (1 + e^-x) from one ex2.approx and one rcp.approx each (relative error of the order of 1e-7; an IEEE division alone would
+// cost as much as the rest of an element)
 __device__ __forceinline__ float2 sigmoid_fast2(float2 x) {
     const float2 t = __fmul2_rn(x, make_float2(-1.4426950408889634f, -1.4426950408889634f));
     float2 e, r;
@@ -79,89 +64,117 @@ __device__ __forceinline__ float2 sigmoid_fast2(float2 x) {
     return r;
 }
 
-// Stage rows [t_first, t_last) of a [L, C] tensor (channels cbase .. cbase + nch) into shared memory, row r of the
-// stage = token t_first + r, 512 channels of room per row.  Tokens in front of the segment come from the carried
-// state (3 rows) or are zero-filled; called by one thread, completion on `bar`.
-template <typename T>
-__device__ __forceinline__ void stage_rows(T *stage, const T *src, const T *state, long long t_first, long long t_last, int C,
-                                           int cbase, int nch, uint64_t *bar) {
-    const uint32_t row_bytes = (uint32_t)nch * sizeof(T);
-    uint32_t total = 0;
-    for (long long t = t_first; t < t_last; ++t)
-        if (t >= 0 || state) total += row_bytes;
-    if (total) mbar_arrive_expect_tx(bar, total);
-    else mbar_arrive(bar);
-    for (long long t = t_first; t < t_last; ++t) {
-        T *dst = stage + (size_t)(t - t_first) * 512;
-        if (t >= 0) bulk_load(dst, src + (size_t)t * C + cbase, row_bytes, bar);
-        else if (state) bulk_load(dst, state + (size_t)(3 + t) * C + cbase, row_bytes, bar);
-    }
-}
+constexpr int CV_STG_TOK = 8;                  // tokens per stage of a ring
+constexpr int CV_RING_THREADS = CV_THREADS + 32;   // four compute warps and the producer warp
 
+// Forward over a range of consecutive tokens: the rows of u stream through a ring of 8-token stages filled by a producer warp
+// with one bulk copy per row, and a thread keeps the last three inputs of its four channels in registers, so nothing is read
+// twice inside a range.  Bound by memory; the arithmetic runs on channel pairs in packed instructions (one 32-token tile per
+// CTA, staged whole and worked through element by element, left 1.6 waves of CTAs and took 24.5 us for 4096 x 5376 bf16).
+constexpr int CV_FWD_STAGES = 4;
 template <typename T>
-__global__ void __launch_bounds__(CV_THREADS) k_conv_fwd(const T *u, long long u_bs, const float *w, const float *bias,
-                                                         const T *state_in, T *out, T *state_out, int L, int C) {
+__global__ void __launch_bounds__(CV_RING_THREADS) k_conv_fwd(const T *u, long long u_bs, const float *w, const float *bias,
+                                                              const T *state_in, T *out, T *state_out, int L, int C, int RL) {
     extern __shared__ __align__(128) unsigned char cv_smem[];
-    __shared__ uint64_t bar;
+    __shared__ uint64_t full[CV_FWD_STAGES], empty[CV_FWD_STAGES];
     __shared__ uint32_t abort_flag;
     __shared__ unsigned int status_dummy;
-    T *su = reinterpret_cast<T *>(cv_smem);                       // [CV_TILE_F + 3][512]
+    T *ring = reinterpret_cast<T *>(cv_smem);                     // [stage][CV_STG_TOK][512]
     pdl_launch_dependents();
     pdl_wait();       // the previous kernel of the stream (a neighbouring segment's) has finished
     const int cbase = blockIdx.x * 512, nch = min(512, C - cbase);
-    const int c0 = cbase + threadIdx.x * CV_CH;
     const int b = blockIdx.z;
-    const long long t_begin = (long long)blockIdx.y * CV_TILE_F, t_end = min(t_begin + (long long)CV_TILE_F, (long long)L);
+    const int r_begin = blockIdx.y * RL, ntok = min(RL, L - r_begin), nst = (ntok + CV_STG_TOK - 1) / CV_STG_TOK;
     const T *ub = u + (size_t)b * u_bs;
     const T *sb = state_in ? state_in + (size_t)b * 3 * C : nullptr;
-    T *ob = out + (size_t)b * u_bs;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     if (threadIdx.x == 0) {
-        mbar_init(&bar, 1);
+        for (int i = 0; i < CV_FWD_STAGES; ++i) {
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], CV_THREADS / 32);
+        }
         abort_flag = 0;
         status_dummy = 0;
         fence_barrier_init();
     }
-    // rows in front of the segment without a carried state: zeros (plain stores, before the barrier below)
-    if (!sb && t_begin < 3)
-        for (int i = threadIdx.x; i < (int)(3 - t_begin) * 512; i += CV_THREADS) su[i] = (T)0.f;
     __syncthreads();
-    if (threadIdx.x == 0) stage_rows(su, ub, sb, t_begin - 3, t_end, C, cbase, nch, &bar);
-    const bool active = c0 < C;
-    float wk[CV_CH][4], bs[CV_CH];
+    if (warp == CV_THREADS / 32) {
+        if (elect_one()) {
+            const uint32_t row_bytes = (uint32_t)nch * sizeof(T);
+            for (int i = 0; i < nst; ++i) {
+                const int slot = i % CV_FWD_STAGES, n = min(CV_STG_TOK, ntok - i * CV_STG_TOK);
+                if (i >= CV_FWD_STAGES) mbar_wait(&empty[slot], (i / CV_FWD_STAGES - 1) & 1, &abort_flag, &status_dummy);
+                mbar_arrive_expect_tx(&full[slot], (uint32_t)n * row_bytes);
+                const T *src = ub + (size_t)(r_begin + i * CV_STG_TOK) * C + cbase;
+                T *dst = ring + (size_t)slot * (CV_STG_TOK * 512);
+                for (int j = 0; j < n; ++j) bulk_load(dst + (size_t)j * 512, src + (size_t)j * C, row_bytes, &full[slot]);
+            }
+        }
+        return;
+    }
+    const int c0 = cbase + threadIdx.x * CV_CH;
+    const bool active = c0 < C;      // inactive threads (past the last channel) still take part in the hand-overs
+    float2 wk[2][4], bs[2], x0[2], x1[2], x2[2], x3[2];
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        wk[i][0] = wk[i][1] = wk[i][2] = wk[i][3] = bs[i] = make_float2(0.f, 0.f);
+        x0[i] = x1[i] = x2[i] = x3[i] = make_float2(0.f, 0.f);
+    }
     if (active) {
 #pragma unroll
-        for (int i = 0; i < CV_CH; ++i) {
-            const float4 wv = *reinterpret_cast<const float4 *>(w + (size_t)(c0 + i) * 4);
-            wk[i][0] = wv.x; wk[i][1] = wv.y; wk[i][2] = wv.z; wk[i][3] = wv.w;
-            bs[i] = bias[c0 + i];
+        for (int i = 0; i < 2; ++i) {
+            const float4 wa = *reinterpret_cast<const float4 *>(w + (size_t)(c0 + 2 * i) * 4);
+            const float4 wb = *reinterpret_cast<const float4 *>(w + (size_t)(c0 + 2 * i + 1) * 4);
+            wk[i][0] = make_float2(wa.x, wb.x); wk[i][1] = make_float2(wa.y, wb.y);
+            wk[i][2] = make_float2(wa.z, wb.z); wk[i][3] = make_float2(wa.w, wb.w);
+            bs[i] = make_float2(bias[c0 + 2 * i], bias[c0 + 2 * i + 1]);
         }
+        // the three inputs in front: of the sequence, else the carried state, else zeros
+        auto before = [&](int t, float2 (&v)[2]) {
+            if (t >= 0) ld2x2(ub + (size_t)t * C + c0, v[0], v[1]);
+            else if (sb) ld2x2(sb + (size_t)(3 + t) * C + c0, v[0], v[1]);
+        };
+        before(r_begin - 3, x0);
+        before(r_begin - 2, x1);
+        before(r_begin - 1, x2);
     }
-    mbar_wait(&bar, 0, &abort_flag, &status_dummy);
-    if (!active) return;
-    const T *sp = su + threadIdx.x * CV_CH;
-    float x0[CV_CH], x1[CV_CH], x2[CV_CH], x3[CV_CH];   // u[t-3], u[t-2], u[t-1], u[t]
-    ld4(sp, x0);
-    ld4(sp + 512, x1);
-    ld4(sp + 1024, x2);
-    const int nt = (int)(t_end - t_begin);
-#pragma unroll 4
-    for (int j = 0; j < nt; ++j) {
-        ld4(sp + (size_t)(j + 3) * 512, x3);
-        float o[CV_CH];
+    T *op = out + (size_t)b * u_bs + (size_t)r_begin * C + c0;
+    auto token = [&](const T *sp) {
+        ld2x2(sp, x3[0], x3[1]);
+        float2 o[2];
 #pragma unroll
-        for (int i = 0; i < CV_CH; ++i) {
-            const float pre = fmaf(wk[i][3], x3[i], fmaf(wk[i][2], x2[i], fmaf(wk[i][1], x1[i], fmaf(wk[i][0], x0[i], bs[i]))));
-            o[i] = pre * sigmoid_fast(pre);
+        for (int i = 0; i < 2; ++i) {
+            const float2 pre = __ffma2_rn(wk[i][3], x3[i], __ffma2_rn(wk[i][2], x2[i], __ffma2_rn(wk[i][1], x1[i], __ffma2_rn(wk[i][0], x0[i], bs[i]))));
+            o[i] = __fmul2_rn(pre, sigmoid_fast2(pre));
             x0[i] = x1[i]; x1[i] = x2[i]; x2[i] = x3[i];
         }
-        st4(ob + (size_t)(t_begin + j) * C + c0, o);
+        const float f[4] = {o[0].x, o[0].y, o[1].x, o[1].y};
+        st4(op, f);
+        op += C;
+    };
+    for (int i = 0; i < nst; ++i) {
+        const int slot = i % CV_FWD_STAGES, n = min(CV_STG_TOK, ntok - i * CV_STG_TOK);
+        mbar_wait(&full[slot], (i / CV_FWD_STAGES) & 1, &abort_flag, &status_dummy);
+        if (active) {
+            const T *sp = ring + (size_t)slot * (CV_STG_TOK * 512) + threadIdx.x * CV_CH;
+            if (n == CV_STG_TOK) {
+#pragma unroll
+                for (int j = 0; j < CV_STG_TOK; ++j) token(sp + j * 512);
+            } else {
+                for (int j = 0; j < n; ++j) token(sp + j * 512);
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&empty[slot]);      // this warp has read the stage
     }
     // the last three inputs of the segment are the state of the next one
-    if (state_out && t_end == L) {
-        T *so = state_out + (size_t)b * 3 * C;
-        st4(so + c0, x0);
-        st4(so + (size_t)C + c0, x1);
-        st4(so + (size_t)2 * C + c0, x2);
+    if (active && state_out && r_begin + ntok == L) {
+        T *so = state_out + (size_t)b * 3 * C + c0;
+        const float f0[4] = {x0[0].x, x0[0].y, x0[1].x, x0[1].y}, f1[4] = {x1[0].x, x1[0].y, x1[1].x, x1[1].y},
+                    f2[4] = {x2[0].x, x2[0].y, x2[1].x, x2[1].y};
+        st4(so, f0);
+        st4(so + (size_t)C, f1);
+        st4(so + (size_t)2 * C, f2);
     }
 }
 
@@ -172,12 +185,10 @@ __global__ void __launch_bounds__(CV_THREADS) k_conv_fwd(const T *u, long long u
 // as `dtail`).  The rows of u and dout stream through a ring of 8-token stages filled by a producer warp with one
 // bulk copy per row, so the loads of later stages are in flight while a stage is being consumed.
 // dw, dbias: one partial per range, the range's own tokens.
-constexpr int CV_STG_TOK = 8;
 constexpr int CV_STAGES = 3;
-constexpr int CV_BWD_THREADS = CV_THREADS + 32;   // four compute warps and the producer warp
 
 template <typename T>
-__global__ void __launch_bounds__(CV_BWD_THREADS, 4)
+__global__ void __launch_bounds__(CV_RING_THREADS, 4)
 k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const T *state_in, const T *dout,
            const float *dtail, T *du, float *dstate, float *part, int L, int C, int RL) {
     extern __shared__ __align__(128) unsigned char cv_smem[];
@@ -207,7 +218,7 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
     __syncthreads();
     if (warp == CV_THREADS / 32) {
         // ---- producer
-        if (lane == 0) {
+        if (elect_one()) {
             const uint32_t row_bytes = (uint32_t)nch * sizeof(T);
             for (int i = 0; i < nst; ++i) {
                 const int slot = i % CV_STAGES;
@@ -264,7 +275,10 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
     }
     // dpre of token s from its input x3 (the window x0..x2 holds the three before it) and g = dout[s]; own tokens
     // also feed the weight and bias gradients.  Then the windows move on and du[s - 3] is complete.
-    auto token = [&](long long s, const float2 *g, bool own, bool formed) {
+    // `inner`: a token in a whole stage that is not the range's first; the du it completes lies in the range and meets neither
+    // the segment's head nor the gradient from its right, so that nothing is asked per token.
+    T *dup = dub + ((size_t)r_begin - 3) * C + c0;       // du of three tokens back
+    auto token = [&](long long s, const float2 *g, bool own, bool formed, bool inner) {
         float2 dp[NP];
 #pragma unroll
         for (int i = 0; i < NP; ++i) {
@@ -286,7 +300,7 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
             }
             d0[i] = d1[i]; d1[i] = d2[i]; d2[i] = d3[i]; d3[i] = dp[i];
         }
-        if (head_range && s == 2) {
+        if (!inner && head_range && s == 2) {
             // What the first three dpre rows of the segment (now d1, d2, d3) send to the three tokens in front of it:
             // token -3 feeds pre[0] through w[0]; token -2: pre[0] w[1], pre[1] w[0]; token -1: pre[0] w[2], pre[1] w[1],
             // pre[2] w[0].
@@ -312,7 +326,7 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
             st4(ds + (size_t)2 * C, e);
         }
         const long long t = s - 3;
-        if (t >= r_begin) {
+        if (inner || t >= r_begin) {
             float o[CV_CH];
 #pragma unroll
             for (int i = 0; i < NP; ++i) {
@@ -320,14 +334,15 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
                 o[2 * i] = v.x;
                 o[2 * i + 1] = v.y;
             }
-            if (dtail && t >= (long long)L - 3) {
+            if (!inner && dtail && t >= (long long)L - 3) {
                 float e[CV_CH];
                 ld4(dtail + ((size_t)b * 3 + (size_t)(t - ((long long)L - 3))) * C + c0, e);
 #pragma unroll
                 for (int i = 0; i < CV_CH; ++i) o[i] += e[i];
             }
-            st4(dub + (size_t)t * C + c0, o);
+            st4(dup, o);
         }
+        dup += C;
     };
     for (int i = 0; i < nst; ++i) {
         const int slot = i % CV_STAGES;
@@ -336,12 +351,22 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
             const T *spu = ring + (size_t)slot * (2 * CV_STG_TOK * 512) + threadIdx.x * CV_CH, *spg = spu + CV_STG_TOK * 512;
             const long long t0 = r_begin + (long long)i * CV_STG_TOK;
             const int n = (int)min((long long)CV_STG_TOK, r_end - t0);
-#pragma unroll 4
-            for (int j = 0; j < n; ++j) {
-                float2 g[NP];
-                ld2x2(spu + (size_t)j * 512, x3[0], x3[1]);
-                ld2x2(spg + (size_t)j * 512, g[0], g[1]);
-                token(t0 + j, g, true, true);
+            if (i > 0 && n == CV_STG_TOK) {
+#pragma unroll
+                for (int j = 0; j < CV_STG_TOK; ++j) {
+                    float2 g[NP];
+                    ld2x2(spu + (size_t)j * 512, x3[0], x3[1]);
+                    ld2x2(spg + (size_t)j * 512, g[0], g[1]);
+                    token(t0 + j, g, true, true, true);
+                }
+            } else {
+#pragma unroll 1
+                for (int j = 0; j < n; ++j) {
+                    float2 g[NP];
+                    ld2x2(spu + (size_t)j * 512, x3[0], x3[1]);
+                    ld2x2(spg + (size_t)j * 512, g[0], g[1]);
+                    token(t0 + j, g, true, true, false);
+                }
             }
         }
         __syncwarp();
@@ -357,7 +382,7 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
             ld2x2(ub + (size_t)s * C + c0, x3[0], x3[1]);
             ld2x2(gb + (size_t)s * C + c0, g[0], g[1]);
         }
-        token(s, g, false, formed);
+        token(s, g, false, formed, false);
     }
     // partial weight / bias gradients of this range: part[b][range][5][C]
     {
@@ -407,35 +432,34 @@ __global__ void __launch_bounds__(256) k_conv_reduce(const float *part, float *d
     }
 }
 
+// Tokens per CTA: about `per_sm` CTAs per SM over the whole launch, whole stages, at least `least`.
+static int conv_range_len(int B, int L, int C, int per_sm, int least) {
+    const int nblk = (C + 511) / 512;
+    int want = (per_sm * kNumSMs) / (nblk * B);
+    if (want < 1) want = 1;
+    const int rl = ((L + want - 1) / want + CV_STG_TOK - 1) / CV_STG_TOK * CV_STG_TOK;
+    return rl < least ? least : rl;
+}
+
 template <typename T>
 cudaError_t conv_fwd_t(const T *u, long long u_bs, const float *w, const float *bias, const T *state_in, T *out, T *state_out,
                        int B, int L, int C, cudaStream_t st) {
-    const int smem = (CV_TILE_F + 3) * 512 * (int)sizeof(T);
-    cudaError_t e = cudaFuncSetAttribute(k_conv_fwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const int smem = CV_FWD_STAGES * CV_STG_TOK * 512 * (int)sizeof(T);
+    const cudaError_t e = allow_smem<k_conv_fwd<T>>(smem);
     if (e != cudaSuccess) return e;
-    dim3 grid((C + 511) / 512, (L + CV_TILE_F - 1) / CV_TILE_F, B);
-    return launch_pdl(k_conv_fwd<T>, grid, dim3(CV_THREADS), (size_t)smem, st, u, u_bs, w, bias, state_in, out, state_out, L, C);
-}
-
-// Tokens per CTA of the backward: about four CTAs per SM over the whole launch, whole stages, and never
-// more ranges than conv_tiles() promises scratch for.
-static int conv_range_len(int B, int L, int C) {
-    const int nblk = (C + 511) / 512;
-    int want = (4 * 148) / (nblk * B);
-    if (want < 1) want = 1;
-    int rl = ((L + want - 1) / want + CV_STG_TOK - 1) / CV_STG_TOK * CV_STG_TOK;
-    if (rl < 32) rl = 32;
-    return rl;
+    const int RL = conv_range_len(B, L, C, sizeof(T) == 2 ? 6 : 3, 16);
+    dim3 grid((C + 511) / 512, (L + RL - 1) / RL, B);
+    return launch_pdl(k_conv_fwd<T>, grid, dim3(CV_RING_THREADS), (size_t)smem, st, u, u_bs, w, bias, state_in, out, state_out, L, C, RL);
 }
 
 template <typename T>
 cudaError_t conv_bwd_t(const T *u, long long u_bs, const float *w, const float *bias, const T *state_in, const T *dout,
                        const float *dtail, T *du, float *dstate, float *part, int B, int L, int C, int RL, cudaStream_t st) {
     const int smem = CV_STAGES * 2 * CV_STG_TOK * 512 * (int)sizeof(T);
-    cudaError_t e = cudaFuncSetAttribute(k_conv_bwd<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    const cudaError_t e = allow_smem<k_conv_bwd<T>>(smem);
     if (e != cudaSuccess) return e;
     dim3 grid((C + 511) / 512, (L + RL - 1) / RL, B);
-    return launch_pdl(k_conv_bwd<T>, grid, dim3(CV_BWD_THREADS), (size_t)smem, st, u, u_bs, w, bias, state_in, dout, dtail, du, dstate,
+    return launch_pdl(k_conv_bwd<T>, grid, dim3(CV_RING_THREADS), (size_t)smem, st, u, u_bs, w, bias, state_in, dout, dtail, du, dstate,
                       part, L, C, RL);
 }
 
@@ -455,7 +479,7 @@ cudaError_t launch_conv_fwd(int dtype, const void *u, long long u_bs, const floa
 cudaError_t launch_conv_bwd(int dtype, const void *u, long long u_bs, const float *w, const float *bias,
                             const void *state_in, const void *dout, const float *dtail, void *du, float *dstate,
                             float *dw, float *dbias, int accumulate, float *part, int B, int L, int C, cudaStream_t st) {
-    const int RL = conv_range_len(B, L, C);
+    const int RL = conv_range_len(B, L, C, 4, 32);      // never more ranges than conv_tiles() promises scratch for
     cudaError_t e;
     if (dtype == SSD_DTYPE_F32)
         e = conv_bwd_t<float>((const float *)u, u_bs, w, bias, (const float *)state_in, (const float *)dout, dtail, (float *)du,

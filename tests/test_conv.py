@@ -127,3 +127,28 @@ def test_conv_rejects_bad_arguments():
     with pytest.raises(libssd.SSDError):
         libssd.ssd_conv_fwd(torch.zeros(1, 8, 12, device="cuda"), torch.zeros(12, 4, device="cuda"),
                             torch.zeros(12, device="cuda"))       # C % 8
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("L", [3, 8, 17, 40, 203, 3001])
+def test_conv_token_ranges_and_stages(L, dtype):
+    """Ranges that end inside a stage, one range and many, a channel block that is mostly empty; carried state and gradient."""
+    from paper_2411_19460_b200 import libssd
+    from tests.parity_util import TOL, relerr
+
+    C = 520
+    td = torch.float32 if dtype == "fp32" else torch.bfloat16
+    gen = torch.Generator().manual_seed(L)
+    u, g = (torch.randn(1, L, C, generator=gen).to(td).cuda() for _ in range(2))
+    st = torch.randn(1, 3, C, generator=gen).to(td).cuda()
+    dtail = torch.randn(1, 3, C, generator=gen).cuda()
+    w, bias = (torch.randn(C, 4, generator=gen) * 0.5).cuda(), (torch.randn(C, generator=gen) * 0.1).cuda()
+    f64 = lambda t: t.detach().double().cpu().numpy()
+    out_ref, _, _ = orc.conv_fwd(f64(u), f64(w), f64(bias), f64(st))
+    refs = orc.conv_bwd(f64(u), f64(w), f64(bias), f64(st), f64(g), f64(dtail))
+    out, so = libssd.ssd_conv_fwd(u, w, bias, st)
+    got = libssd.ssd_conv_bwd(u, w, bias, st, g, dtail)
+    assert torch.equal(so, u[:, -3:]) and relerr(out, out_ref) <= TOL[dtype]
+    for a, r in zip(got, refs):
+        assert relerr(a, r) <= TOL[dtype]

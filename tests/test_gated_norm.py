@@ -81,3 +81,23 @@ def test_gated_norm_rejects_bad_arguments():
         libssd.ssd_gated_norm_fwd(y, y, gamma, group=10)              # D % group
     with pytest.raises(libssd.SSDError):
         libssd.ssd_gated_norm_fwd(y, y, gamma, group=6)               # group % 4
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("rows,D,group", [(1, 5120, 5120), (5, 1536, 512), (1205, 2048, 2048), (2500, 64, 64), (37, 24, 12), (9, 8192, 8192)])
+def test_gated_norm_row_splits_and_rings(rows, D, group, dtype):
+    """One row, few rows per CTA, an uneven last CTA, more rows than the ring holds, rows that no ring takes."""
+    from paper_2411_19460_b200 import libssd
+    from tests.parity_util import TOL, relerr
+
+    td = torch.float32 if dtype == "fp32" else torch.bfloat16
+    gen = torch.Generator().manual_seed(rows)
+    y, z, g = (torch.randn(rows, D, generator=gen).to(td).cuda() for _ in range(3))
+    gamma = (1.0 + 0.1 * torch.randn(D, generator=gen)).cuda()
+    f64 = lambda t: t.detach().double().cpu().numpy()
+    out_ref, _, _ = orc.gated_norm_fwd(f64(y), f64(z), f64(gamma), group)
+    refs = orc.gated_norm_bwd(f64(y), f64(z), f64(gamma), f64(g), group)
+    assert relerr(libssd.ssd_gated_norm_fwd(y, z, gamma, group=group), out_ref) <= TOL[dtype]
+    for a, r in zip(libssd.ssd_gated_norm_bwd(y, z, gamma, g, group=group), refs):
+        assert relerr(a, r) <= TOL[dtype]
