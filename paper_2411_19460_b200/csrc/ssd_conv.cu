@@ -400,12 +400,13 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
     }
 }
 
-// dw[c][k], dbias[c] from the tile partials, in fp64 and in a fixed order: a CTA owns 32 adjacent channels of one of the
-// five rows (four taps, bias); its eight warps take the tiles round-robin (coalesced 128-byte reads, several in flight),
-// then the eight partial sums are added in warp order.
-__global__ void __launch_bounds__(256) k_conv_reduce(const float *part, float *dw, float *dbias, int C, int ntiles, int B,
-                                                     int accumulate) {
-    __shared__ double red[8][32];
+// dw[c][k], dbias[c] from the partials of the ranges, in fp64 and in a fixed order: a CTA owns 32 adjacent channels of one of the
+// five rows (four taps, bias); its sixteen warps take the ranges round-robin (coalesced 128-byte reads, four in flight), then
+// the sixteen sums are added in warp order.
+constexpr int CV_RED_WARPS = 16;
+__global__ void __launch_bounds__(CV_RED_WARPS * 32) k_conv_reduce(const float *part, float *dw, float *dbias, int C, int total,
+                                                                   int accumulate) {
+    __shared__ double red[CV_RED_WARPS][32];
     pdl_launch_dependents();
     pdl_wait();
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -413,16 +414,20 @@ __global__ void __launch_bounds__(256) k_conv_reduce(const float *part, float *d
     const int k = blockIdx.x / nblk, c = (blockIdx.x % nblk) * 32 + lane;
     double s = 0.0;
     if (c < C) {
-        const long long total = (long long)B * ntiles;
-#pragma unroll 4
-        for (long long t = wp; t < total; t += 8) s += (double)part[((size_t)t * 5 + k) * C + c];
+        for (int t0 = wp; t0 < total; t0 += 4 * CV_RED_WARPS) {
+            float v[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) v[m] = t0 + m * CV_RED_WARPS < total ? part[((size_t)(t0 + m * CV_RED_WARPS) * 5 + k) * C + c] : 0.f;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) s += (double)v[m];
+        }
     }
     red[wp][lane] = s;
     __syncthreads();
     if (wp == 0 && c < C) {
         double tot = 0.0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) tot += red[i][lane];
+        for (int i = 0; i < CV_RED_WARPS; ++i) tot += red[i][lane];
         if (k < 4) {
             float *d = dw + (size_t)c * 4 + k;
             *d = accumulate ? *d + (float)tot : (float)tot;
@@ -488,8 +493,8 @@ cudaError_t launch_conv_bwd(int dtype, const void *u, long long u_bs, const floa
         e = conv_bwd_t<__nv_bfloat16>((const __nv_bfloat16 *)u, u_bs, w, bias, (const __nv_bfloat16 *)state_in,
                                       (const __nv_bfloat16 *)dout, dtail, (__nv_bfloat16 *)du, dstate, part, B, L, C, RL, st);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_conv_reduce, dim3(5 * ((C + 31) / 32)), dim3(256), (size_t)0, st, (const float *)part, dw, dbias, C,
-                      (L + RL - 1) / RL, B, accumulate);
+    return launch_pdl(k_conv_reduce, dim3(5 * ((C + 31) / 32)), dim3(CV_RED_WARPS * 32), (size_t)0, st, (const float *)part, dw, dbias, C,
+                      (L + RL - 1) / RL * B, accumulate);
 }
 
 }  // namespace ssd

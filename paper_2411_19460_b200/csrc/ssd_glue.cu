@@ -5,8 +5,6 @@
 // Bandwidth-shaped kernels; bf16 or fp32 I/O.  fp32: CUDA cores, fp32 arithmetic.  bf16: the 64 x 64 product runs on
 // the tensor cores through warp-level mma (W rounded to bf16 once per CTA, fp32 accumulation): at 4096 multiply-adds
 // per 128-byte row the CUDA-core version was five times over its memory time.
-#include <mma.h>
-
 #include "ssd_internal.h"
 
 namespace ssd {
@@ -87,95 +85,101 @@ __global__ void __launch_bounds__(128) k_glue(const T *a, const T *b, const floa
     }
 }
 
-// The same product for bf16 rows on the tensor cores.  A warp owns 16 consecutive rows (one contiguous 2 KB block of
-// the row-major [rows][64] tensor): it fetches them with 16-byte loads that cover whole 512-byte spans per instruction,
-// forms Z = a (+ b) in bf16 and parks it in a padded shared-memory tile, multiplies it by the bf16 copy of W with
-// 4 x 4 warp-level mma steps (fp32 accumulation), and sends the 16 result rows out the same way, through a padded
-// fp32 staging tile.  Row strides of 72 elements keep the fragment accesses off one bank.
-constexpr int GL_LD = 72;
-template <bool TRANSPOSE>
+// The same product for bf16 rows on the tensor cores (warp-level mma, fp32 accumulation).  A warp owns 16 consecutive rows at a
+// time, one contiguous 2 KB block of the row-major [rows][64] tensor, and everything stays in registers: the order of the
+// contraction index is free, so a lane's A fragments are the 16-byte pieces it loads (four lanes cover 64 contiguous bytes of a
+// row), and so is the order of the output columns, so what a lane stores is two 16-byte pieces per row.  W, rounded to bf16, is
+// laid out for both orders once per CTA.  The next tile's rows are requested before the current ones are multiplied.
+//   step s of the contraction, lane group j = lane % 4: columns 32 (s / 2) + 8 j + 4 (s % 2) + {0, 1 | 2, 3}
+//   output tile t, column c:                            column  32 (t / 4) + 8 (c / 2) + 2 (t % 4) + c % 2
+// Bound by memory; with both sides going through shared-memory tiles the kernel took 37 us for 4096 x 80 rows (126 MB).
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ uint32_t pack_bf16(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t *>(&v);
+}
+template <bool TRANSPOSE, bool ADD>
 __global__ void __launch_bounds__(128) k_glue_bf16_mma(const __nv_bfloat16 *a, const __nv_bfloat16 *b, const float *W,
                                                        __nv_bfloat16 *out, long long rows_per_batch, long long bstride, int B) {
-    using namespace nvcuda;
-    __shared__ __align__(32) __nv_bfloat16 Wb[64 * GL_LD];
-    __shared__ __align__(32) __nv_bfloat16 zs[4][16 * GL_LD];
-    __shared__ __align__(32) float stage[4][16 * GL_LD];
-    for (int idx = threadIdx.x; idx < 4096; idx += 128) Wb[(idx >> 6) * GL_LD + (idx & 63)] = __float2bfloat16_rn(W[idx]);
-    __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long ntiles = rows_per_batch * B / 16;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, j = lane & 3, r = lane >> 2;
+    // B operand: element (k, n) = M[n][k], M = W or W^T; this lane holds n-column r of every tile, k pairs of group j
+    uint32_t wf[8][4][2];
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+        const int n = 32 * (t >> 2) + 8 * (r >> 1) + 2 * (t & 3) + (r & 1);
+#pragma unroll
+        for (int s = 0; s < 4; ++s)
+#pragma unroll
+            for (int i = 0; i < 2; ++i) {
+                const int k = 32 * (s >> 1) + 8 * j + 4 * (s & 1) + 2 * i;
+                const float w0 = TRANSPOSE ? W[k * 64 + n] : W[n * 64 + k], w1 = TRANSPOSE ? W[(k + 1) * 64 + n] : W[n * 64 + k + 1];
+                wf[t][s][i] = pack_bf16(w0, w1);
+            }
+    }
+    const long long ntiles = rows_per_batch * B / 16, step = (long long)gridDim.x * 4;
     auto tile_offset = [&](long long t) {
-        const long long row0 = t * 16, bb = row0 / rows_per_batch, rr = row0 % rows_per_batch;
-        return (size_t)bb * bstride + (size_t)rr * 64;
+        const long long row0 = t * 16, bb = row0 / rows_per_batch, rr = row0 - bb * rows_per_batch;
+        return (size_t)bb * bstride + (size_t)rr * 64 + (size_t)r * 64 + j * 8;
     };
-    // 16-byte chunk c of a tile's block (128 of them): row c / 8, columns (c % 8) * 8 ..; the next tile's rows are
-    // requested as soon as the current ones have been parked in shared memory
-    uint4 va[4], vb[4];
+    uint4 va[2][2], vb[2][2];      // [row r, r + 8][columns 0.. / 32..]
     auto fetch = [&](size_t off) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) va[q] = __ldg(reinterpret_cast<const uint4 *>(a + off) + q * 32 + lane);
-        if (b) {
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-            for (int q = 0; q < 4; ++q) vb[q] = __ldg(reinterpret_cast<const uint4 *>(b + off) + q * 32 + lane);
-        }
-    };
-    const long long t_first = (long long)blockIdx.x * 4 + warp, t_step = (long long)gridDim.x * 4;
-    if (t_first < ntiles) fetch(tile_offset(t_first));
-    for (long long t = t_first; t < ntiles; t += t_step) {
-        const size_t off = tile_offset(t);
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint4 z = va[q];
-            if (b) {
-                __nv_bfloat162 *zp = reinterpret_cast<__nv_bfloat162 *>(&z);
-                const __nv_bfloat162 *bp = reinterpret_cast<const __nv_bfloat162 *>(&vb[q]);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) zp[i] = __hadd2(zp[i], bp[i]);
+            for (int i = 0; i < 2; ++i) {
+                va[h][i] = __ldg(reinterpret_cast<const uint4 *>(a + off + h * 8 * 64 + i * 32));
+                if (ADD) vb[h][i] = __ldg(reinterpret_cast<const uint4 *>(b + off + h * 8 * 64 + i * 32));
             }
-            const int c = q * 32 + lane;
-            *reinterpret_cast<uint4 *>(&zs[warp][(c >> 3) * GL_LD + (c & 7) * 8]) = z;
-        }
-        if (t + t_step < ntiles) fetch(tile_offset(t + t_step));
-        __syncwarp();
-        wmma::fragment<wmma::matrix_a, 16, 16, 16, __nv_bfloat16, wmma::row_major> za[4];
+    };
+    long long t = (long long)blockIdx.x * 4 + warp;
+    if (t >= ntiles) return;
+    size_t off = tile_offset(t);
+    fetch(off);
+    while (true) {
+        uint32_t z[2][2][4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) wmma::load_matrix_sync(za[k], zs[warp] + k * 16, GL_LD);
-        // out[row, i] = sum_j M[i][j] z[j]: the B operand is element (k = j, n = i) = M[i][j].  M = W: W[n][k], i.e. W
-        // read column-major; M = W^T: W[k][n], row-major.
+        for (int h = 0; h < 2; ++h)
 #pragma unroll
-        for (int n = 0; n < 4; ++n) {
-            wmma::fragment<wmma::accumulator, 16, 16, 16, float> acc;
-            wmma::fill_fragment(acc, 0.f);
+            for (int i = 0; i < 2; ++i) {
+                const uint32_t x[4] = {va[h][i].x, va[h][i].y, va[h][i].z, va[h][i].w}, y[4] = {vb[h][i].x, vb[h][i].y, vb[h][i].z, vb[h][i].w};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                if (TRANSPOSE) {
-                    wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, wmma::row_major> mb;
-                    wmma::load_matrix_sync(mb, Wb + (k * 16) * GL_LD + n * 16, GL_LD);
-                    wmma::mma_sync(acc, za[k], mb, acc);
-                } else {
-                    wmma::fragment<wmma::matrix_b, 16, 16, 16, __nv_bfloat16, wmma::col_major> mb;
-                    wmma::load_matrix_sync(mb, Wb + (n * 16) * GL_LD + k * 16, GL_LD);
-                    wmma::mma_sync(acc, za[k], mb, acc);
+                for (int e = 0; e < 4; ++e) {
+                    z[h][i][e] = x[e];
+                    if (ADD) {
+                        const __nv_bfloat162 s = __hadd2(*reinterpret_cast<const __nv_bfloat162 *>(&x[e]), *reinterpret_cast<const __nv_bfloat162 *>(&y[e]));
+                        z[h][i][e] = *reinterpret_cast<const uint32_t *>(&s);
+                    }
                 }
             }
-            wmma::store_matrix_sync(stage[warp] + n * 16, acc, GL_LD, wmma::mem_row_major);
+        const size_t cur = off;
+        t += step;
+        const bool more = t < ntiles;
+        if (more) {
+            off = tile_offset(t);
+            fetch(off);
         }
-        __syncwarp();
+        float acc[8][4];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            const int c = q * 32 + lane;
-            const float *src = stage[warp] + (c >> 3) * GL_LD + (c & 7) * 8;
-            const float4 v0 = *reinterpret_cast<const float4 *>(src), v1 = *reinterpret_cast<const float4 *>(src + 4);
-            __nv_bfloat162 p0 = __floats2bfloat162_rn(v0.x, v0.y), p1 = __floats2bfloat162_rn(v0.z, v0.w);
-            __nv_bfloat162 p2 = __floats2bfloat162_rn(v1.x, v1.y), p3 = __floats2bfloat162_rn(v1.z, v1.w);
-            uint4 pk;
-            pk.x = *reinterpret_cast<unsigned int *>(&p0);
-            pk.y = *reinterpret_cast<unsigned int *>(&p1);
-            pk.z = *reinterpret_cast<unsigned int *>(&p2);
-            pk.w = *reinterpret_cast<unsigned int *>(&p3);
-            *(reinterpret_cast<uint4 *>(out + off) + c) = pk;
+        for (int n = 0; n < 8; ++n) {
+            acc[n][0] = acc[n][1] = acc[n][2] = acc[n][3] = 0.f;
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                const uint32_t af[4] = {z[0][s >> 1][2 * (s & 1)], z[1][s >> 1][2 * (s & 1)], z[0][s >> 1][2 * (s & 1) + 1], z[1][s >> 1][2 * (s & 1) + 1]};
+                mma_bf16(acc[n], af, wf[n][s][0], wf[n][s][1]);
+            }
         }
-        __syncwarp();      // both tiles are reused by the warp's next 16 rows
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                *reinterpret_cast<uint4 *>(out + cur + h * 8 * 64 + i * 32) =
+                    make_uint4(pack_bf16(acc[4 * i][2 * h], acc[4 * i][2 * h + 1]), pack_bf16(acc[4 * i + 1][2 * h], acc[4 * i + 1][2 * h + 1]),
+                               pack_bf16(acc[4 * i + 2][2 * h], acc[4 * i + 2][2 * h + 1]), pack_bf16(acc[4 * i + 3][2 * h], acc[4 * i + 3][2 * h + 1]));
+        if (!more) break;
     }
 }
 
@@ -215,9 +219,12 @@ cudaError_t launch_glue(int dtype, bool transpose, const void *a, const void *b,
         else k_glue<float, false><<<blocks, 128, 0, st>>>((const float *)a, (const float *)b, W, (float *)out, rows_per_batch, bstride, B);
     } else if (rows_per_batch % 16 == 0) {
         const long long tiles = total / 16;
-        const unsigned mblocks = (unsigned)((tiles + 3) / 4 < 148 * 6 ? (tiles + 3) / 4 : 148 * 6);   // six 37 KB CTAs fit an SM: one wave
-        if (transpose) k_glue_bf16_mma<true><<<mblocks, 128, 0, st>>>((const __nv_bfloat16 *)a, (const __nv_bfloat16 *)b, W, (__nv_bfloat16 *)out, rows_per_batch, bstride, B);
-        else k_glue_bf16_mma<false><<<mblocks, 128, 0, st>>>((const __nv_bfloat16 *)a, (const __nv_bfloat16 *)b, W, (__nv_bfloat16 *)out, rows_per_batch, bstride, B);
+        const unsigned most = 148 * 3;      // three CTAs of 160-register threads fit an SM: one wave
+        const unsigned mblocks = (unsigned)((tiles + 3) / 4 < most ? (tiles + 3) / 4 : most);
+        const __nv_bfloat16 *pa = (const __nv_bfloat16 *)a, *pb = (const __nv_bfloat16 *)b;
+        __nv_bfloat16 *po = (__nv_bfloat16 *)out;
+        if (transpose) k_glue_bf16_mma<true, false><<<mblocks, 128, 0, st>>>(pa, pb, W, po, rows_per_batch, bstride, B);
+        else k_glue_bf16_mma<false, true><<<mblocks, 128, 0, st>>>(pa, pb, W, po, rows_per_batch, bstride, B);
     } else {
         if (transpose) k_glue<__nv_bfloat16, true><<<blocks, 128, 0, st>>>((const __nv_bfloat16 *)a, (const __nv_bfloat16 *)b, W, (__nv_bfloat16 *)out, rows_per_batch, bstride, B);
         else k_glue<__nv_bfloat16, false><<<blocks, 128, 0, st>>>((const __nv_bfloat16 *)a, (const __nv_bfloat16 *)b, W, (__nv_bfloat16 *)out, rows_per_batch, bstride, B);

@@ -255,8 +255,10 @@ k_gated_norm_staged(const T *y, const T *z, const float *gamma, float eps, const
         abort_flag = 0;
         status_dummy = 0;
         fence_barrier_init();
+        pdl_wait();
         for (int j = 0; j < stages && j < nrows; ++j) issue(j, j);
     }
+    pdl_wait();
     float2 gm[NV][2], dg[NV][2];
 #pragma unroll
     for (int k = 0; k < NV; ++k) {
@@ -348,6 +350,7 @@ k_gated_norm_staged(const T *y, const T *z, const float *gamma, float eps, const
             }
         }
     }
+    pdl_launch_dependents();     // not earlier: the next launch fills the GPU in one wave and wants it free
     if (BWD) {
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
@@ -378,23 +381,30 @@ template <typename T> StagedPlan staged_plan(long long rows, int D, int group, i
     return {stages, (int)rpc};
 }
 
-// dgamma from the tile partials, in fp64 and in a fixed order: a CTA owns 32 adjacent channels; its eight warps take the
-// tiles round-robin (coalesced reads, several in flight), then the eight partial sums are added in warp order.
-__global__ void __launch_bounds__(256) k_gated_norm_reduce(const float *part, float *dgamma, int D, int ntiles, int accumulate) {
-    __shared__ double red[8][32];
+// dgamma from the partial sums, in fp64 and in a fixed order: a CTA owns 32 adjacent channels; its 32 warps take the partials
+// round-robin, eight loads in flight each, then the 32 sums are added in warp order.  A few microseconds of latency behind
+// every backward call: with eight warps and four loads in flight it took 10 us for 293 partials.
+__global__ void __launch_bounds__(1024) k_gated_norm_reduce(const float *part, float *dgamma, int D, int ntiles, int accumulate) {
+    __shared__ double red[32][32];
+    pdl_wait();
     const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
     const int c = blockIdx.x * 32 + lane;
     double s = 0.0;
     if (c < D) {
-#pragma unroll 4
-        for (int t = wp; t < ntiles; t += 8) s += (double)part[(size_t)t * D + c];
+        for (int t0 = wp; t0 < ntiles; t0 += 8 * 32) {
+            float v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[k] = t0 + 32 * k < ntiles ? part[(size_t)(t0 + 32 * k) * D + c] : 0.f;
+#pragma unroll
+            for (int k = 0; k < 8; ++k) s += (double)v[k];
+        }
     }
     red[wp][lane] = s;
     __syncthreads();
     if (wp == 0 && c < D) {
         double tot = 0.0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) tot += red[i][lane];
+        for (int i = 0; i < 32; ++i) tot += red[i][lane];
         dgamma[c] = accumulate ? dgamma[c] + (float)tot : (float)tot;
     }
 }
@@ -409,9 +419,8 @@ static cudaError_t launch_staged(const StagedPlan &pl, const T *y, const T *z, c
     const size_t ring = (size_t)pl.stages * (BWD ? 3 : 2) * group * sizeof(T);
     const cudaError_t e = allow_smem<k_gated_norm_staged<T, NV, BWD>>(220 * 1024);
     if (e != cudaSuccess) return e;
-    k_gated_norm_staged<T, NV, BWD><<<dim3((unsigned)((rows + pl.rpc - 1) / pl.rpc), D / group), GN_THREADS, ring, st>>>(
-        y, z, gamma, eps, dout, o1, o2, part, rows, D, group, pl.rpc, pl.stages);
-    return cudaGetLastError();
+    return launch_pdl(k_gated_norm_staged<T, NV, BWD>, dim3((unsigned)((rows + pl.rpc - 1) / pl.rpc), D / group), dim3(GN_THREADS), ring, st, y, z,
+                      gamma, eps, dout, o1, o2, part, rows, D, group, pl.rpc, pl.stages);
 }
 // 4-channel vectors per thread, rounded up to an instantiated count
 #define GN_BY_NEED(CALL)           \
@@ -477,8 +486,7 @@ cudaError_t launch_gated_norm_bwd(int dtype, const void *y, const void *z, const
         e = norm_bwd_t<__nv_bfloat16>((const __nv_bfloat16 *)y, (const __nv_bfloat16 *)z, gamma, eps, (const __nv_bfloat16 *)dout,
                                       (__nv_bfloat16 *)dy, (__nv_bfloat16 *)dz, part, rows, D, group, parts, st);
     if (e != cudaSuccess) return e;
-    k_gated_norm_reduce<<<(D + 31) / 32, 256, 0, st>>>(part, dgamma, D, parts, accumulate);
-    return cudaGetLastError();
+    return launch_pdl(k_gated_norm_reduce, dim3((D + 31) / 32), dim3(1024), 0, st, (const float *)part, dgamma, D, parts, accumulate);
 }
 
 }  // namespace ssd
