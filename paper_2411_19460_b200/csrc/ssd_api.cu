@@ -49,7 +49,7 @@ static void prof_end(ProfEvent *ev, cudaStream_t st) {
 struct Layout {
     size_t status, Hst, hcarry, Gst, gcarry, cbt, dAp, dDp;
     size_t rec[2], cs[2], dtT[2], Hbf[2];
-    size_t Gbf[2], ghdot[2], ddt_dir[2], rho[2], rho2[2], rho2b[2], psi[2], psi2[2], pB[2], pC[2];
+    size_t Gbf[2], ghdot[2], ddt_dir[2], rho[2], rho2[2], psi[2], psi2[2], pB[2], pC[2];
     size_t total;
 };
 
@@ -162,7 +162,6 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
         const size_t vec_tiles = pl.use_tc ? vec : vec * (pl.Q / 64);
         take2(lo.rho, vec_tiles, vtwin);
         take2(lo.rho2, vec, vtwin);
-        if (pl.use_tc) take2(lo.rho2b, vec, vtwin);
         take2(lo.psi, vec_tiles, vtwin);
         take2(lo.psi2, vec, vtwin);
         const size_t part = (size_t)pl.B * pl.seg * pl.G * pl.nsl * pl.N * sizeof(float);
@@ -259,7 +258,6 @@ static void select_copy(const Layout &lo, void *ws, int k, SegParams &sp) {
     sp.ddt_dir = f(lo.ddt_dir);
     sp.rho = f(lo.rho);
     sp.rho2 = f(lo.rho2);
-    sp.rho2b = f(lo.rho2b);
     sp.psi = f(lo.psi);
     sp.psi2 = f(lo.psi2);
     sp.pB = f(lo.pB);

@@ -62,9 +62,9 @@ enum {
     REC_CS = 160,       // [128] cs
     REC_DT = 288,       // [128] dt
     REC_CF = 416,       // [128] dt_s e^{cs[last of s's sub-tile] - cs_s}
-    REC_OC = 544,       // [128] e^{cs_t}
-    REC_OB = 672,       // [128] dt_s e^{cs_last - cs_s}
-    REC_FLOATS = 800
+    REC_OC = 544,       // [128] e^{cs_t}, as a RowScale
+    REC_OB = 800,       // [128] dt_s e^{cs_last - cs_s}, as a RowScale
+    REC_FLOATS = 1056
 };
 // Up to this many log2 units of decay inside a sub-tile, e^{cs_t - cs_s} on its diagonal is taken as a product of a row and a
 // column factor (one of them > 1, far from overflow) like everywhere else; beyond, element by element.
@@ -107,7 +107,7 @@ struct SegParams {
     float *ddt_dir;        // [B,H,ncs,Q]   direct part of ddt
     float *cbt;            // CUDA-core path: [B,ncs,G,Q,Q] C B^T, causal 64 x 64 tiles
     float *rho;            // [B,H,ncs,Q]   C_t . (intra-chunk part of this head's dC_t); CUDA-core path: [B,H,ncs,tiles,Q] by column tile
-    float *rho2, *rho2b;   // [B,H,ncs,Q]   C_t . (inter-chunk part of this head's dC_t); tensor-core path: in two halves
+    float *rho2;           // [B,H,ncs,Q]   C_t . (inter-chunk part of this head's dC_t)
     float *psi;            // [B,H,ncs,Q]   B_t . (intra-chunk part of this head's dB_t); CUDA-core path: [B,H,ncs,tiles,Q] by row tile
     float *psi2;           // [B,H,ncs,Q]   B_t . (inter-chunk part of this head's dB_t)
     float *pB, *pC;        // [B,seg,G,nsl,N] per-head-slice partial dB / dC

@@ -729,7 +729,7 @@ __device__ __forceinline__ void bwd_finish(const SegParams &p, int id) {
                     r1 = p.rho[vo + j];
                     p1 = p.psi[vo + j];
                 }
-                run += (r1 - p1) + (p.rho2b ? p.rho2[vo + j] + p.rho2b[vo + j] : p.rho2[vo + j]);
+                run += (r1 - p1) + p.rho2[vo + j];
                 sfx[j] = run;
             }
         float incl = run;

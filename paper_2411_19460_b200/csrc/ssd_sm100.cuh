@@ -50,6 +50,21 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t parity) {
     return ok != 0;
 }
 
+// The same without any suspension.
+__device__ __forceinline__ bool mbar_test(uint64_t *bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n"
+        ".reg .pred p;\n"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n"
+        "}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+
 // Every wait in these kernels is bounded.  `abort_flag` is a CTA-shared word: once any wait has
 // given up, later waits only poll briefly (so copies still in flight get a last chance to land)
 // and the kernel runs to its normal end, frees its TMEM and returns; `status` is the global word
@@ -60,7 +75,7 @@ constexpr long long kWaitAbortedClk = 4000000ll;     // about 2 ms once aborted
 // The wait with an explicit limit (clock cycles) for a wait that has not yet been given up on.
 __device__ __forceinline__ bool mbar_wait_limited(uint64_t *bar, uint32_t parity, volatile uint32_t *abort_flag,
                                                   unsigned int *status, long long limit_clk) {
-    if (mbar_try_wait(bar, parity)) return true;
+    if (mbar_test(bar, parity)) return true;
     const long long start = clock64();
     const long long limit = (*abort_flag) ? kWaitAbortedClk : limit_clk;
     do {
@@ -131,8 +146,6 @@ __device__ __forceinline__ void tma_store_3d(const CUtensorMap *m, const void *s
 __device__ __forceinline__ void tma_store_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 // all earlier stores of this thread have finished READING their shared-memory source
 __device__ __forceinline__ void tma_store_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
-// all but the latest store group have
-__device__ __forceinline__ void tma_store_wait_read_but_one() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 // all earlier stores of this thread are complete
 __device__ __forceinline__ void tma_store_wait_all() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 
@@ -347,6 +360,27 @@ __device__ __forceinline__ uint64_t umma_desc_words(uint32_t lo, uint32_t hi) {
 __device__ __forceinline__ void umma_commit(uint64_t *bar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                  : "memory");
+}
+
+// A factor that rows of bf16 are multiplied by, as two bf16 (each twice, for packed arithmetic): s = hi + lo up to 2^-17 s.
+// x s is then a packed multiply and a packed multiply-add whose one rounding is the result's, two instructions for two elements
+// instead of four through fp32, to the same accuracy.
+struct RowScale { uint32_t hi, lo; };
+__device__ __forceinline__ RowScale row_scale(float s) {
+    const __nv_bfloat16 h = __float2bfloat16_rn(s), l = __float2bfloat16_rn(s - __bfloat162float(h));
+    const __nv_bfloat162 h2 = __halves2bfloat162(h, h), l2 = __halves2bfloat162(l, l);
+    return {*reinterpret_cast<const uint32_t *>(&h2), *reinterpret_cast<const uint32_t *>(&l2)};
+}
+__device__ __forceinline__ uint32_t scale2(uint32_t x, const RowScale &s) {
+    const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162 *>(&x);
+    const __nv_bfloat162 r = __hfma2(v, *reinterpret_cast<const __nv_bfloat162 *>(&s.hi), __hmul2(v, *reinterpret_cast<const __nv_bfloat162 *>(&s.lo)));
+    return *reinterpret_cast<const uint32_t *>(&r);
+}
+__device__ __forceinline__ void scale8(uint4 &v, const RowScale &s) {
+    v.x = scale2(v.x, s);
+    v.y = scale2(v.y, s);
+    v.z = scale2(v.z, s);
+    v.w = scale2(v.w, s);
 }
 
 // Byte offset of the 16-byte chunk (row r, logical chunk j of 8) inside a 128B-swizzled tile whose

@@ -49,9 +49,6 @@ __device__ __forceinline__ uint32_t pack2g(float a, float b) {
     __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
     return *reinterpret_cast<uint32_t *>(&v);
 }
-__device__ __forceinline__ float2 unpack2g(uint32_t w) {
-    return __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&w));
-}
 
 }  // namespace
 
@@ -258,7 +255,7 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
         constexpr int I0 = doC ? 0 : 1024, I1 = doB ? 2048 : 1024;
         for (int hi = 0; hi < nheads; ++hi) {
             const int vb = hi % GF_VECS, u = hi + 1, e = hi + 2;
-            const float *sc = record(vb) + REC_OC;          // row scales of dy, then of x
+            const RowScale *sc = reinterpret_cast<const RowScale *>(record(vb) + REC_OC);      // of dy, then of x
             mbar_wait(&vfull[vb], (hi / GF_VECS) & 1, abortp, p.status);
             mbar_wait(&rfull[e & 3], (e >> 2) & 1, abortp, p.status);
             mbar_wait(&sfull[u & 1], (u >> 1) & 1, abortp, p.status);
@@ -266,7 +263,7 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
             // eight 16-byte pieces in flight per thread: this role is three warps' worth of latency
             for (int i = I0 + th; i < I1; i += 8 * 96) {
                 uint4 v[8];
-                float f[8];
+                RowScale f[8];
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const int j = min(i + k * 96, 2047);
@@ -275,12 +272,7 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
                 }
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
-                    uint32_t *w = reinterpret_cast<uint32_t *>(&v[k]);
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        const float2 t = __fmul2_rn(unpack2g(w[m]), make_float2(f[k], f[k]));
-                        w[m] = pack2g(t.x, t.y);
-                    }
+                    scale8(v[k], f[k]);
                     if (i + k * 96 < I1) rows[i + k * 96] = v[k];
                 }
             }

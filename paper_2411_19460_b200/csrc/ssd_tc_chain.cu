@@ -10,8 +10,8 @@
 // what is written per block is its bf16 copy, the operand of the large kernels, 16 KB, where separate kernels for the
 // sums and the recurrence moved 32 KB of fp32 sums out and in again on top.  States are kept transposed here, [N][64], so
 // that a thread's slice (one n, 32 p) is contiguous and leaves through a swizzled tile by one TMA store per warp.
-//   warp 0 producer (TMA) | warp 1 MMA issuer | warps 2, 3 records (CHAIN_FWD, alternate blocks) | warps 4..7 scale the rows |
-//   warps 8..15 carry
+//   warp 0 producer (TMA) | warp 1 MMA issuer | warps 2, 3 records (CHAIN_FWD, alternate blocks) | warps 4..11 scale the rows |
+//   warps 12..19 carry | warps 20..23 rho2 (CHAIN_BWD)
 // Bound by the chain's latency, about a step per 0.5 us per head, on as many SMs as there are heads; the large kernels of
 // the neighbouring segment run beside it.
 #include "ssd_internal.h"
@@ -23,18 +23,18 @@ using namespace sm100;
 
 namespace {
 
-constexpr int CH_THREADS = 512;
+__host__ __device__ constexpr int ch_threads(int mode) { return mode ? 768 : 640; }
 constexpr int CH_T = 128;
-constexpr int CH_STAGES = 3;
+__host__ __device__ constexpr int ch_stages(int mode) { return mode ? 3 : 4; }
 constexpr int CH_VEC = 4;                 // CHAIN_FWD: vector buffers (weights of 128 rows + the block's decay)
-constexpr int CH_VEC_FLOATS = 132;
+constexpr int CH_VEC_FLOATS = 260;
 constexpr float kLog2eC = 1.4426950408889634f;
 constexpr int CH_AHEAD = 4;               // L2 prefetch distance in blocks beyond the staged ones
 
-// stage: V (B or C rows) N/64 x 16 KB | X (x or dy rows) 16 KB | CHAIN_BWD: H_in^T, N rows of 128 B | weights 512 B, decay 16 B
-__host__ __device__ constexpr uint32_t ch_stage_bytes(int mode, int ns) { return (uint32_t)ns * 256 + 16384 + (mode ? (uint32_t)ns * 128 + 1024 : 0); }
+// stage: V (B or C rows) N/64 x 16 KB | X (x or dy rows) 16 KB | CHAIN_BWD: H_in^T, N rows of 128 B | row scales 1 KB, decay 16 B
+__host__ __device__ constexpr uint32_t ch_stage_bytes(int mode, int ns) { return (uint32_t)ns * 256 + 16384 + (mode ? (uint32_t)ns * 128 + 2048 : 0); }
 __host__ __device__ constexpr uint32_t ch_smem(int mode, int ns) {
-    return CH_STAGES * ch_stage_bytes(mode, ns) + (mode ? 1 : 2) * 8 * 2048 + (mode ? 0 : CH_VEC * CH_VEC_FLOATS * 4) + 1024;
+    return ch_stages(mode) * ch_stage_bytes(mode, ns) + 8 * 2048 + (mode ? 0 : CH_VEC * CH_VEC_FLOATS * 4) + 1024;
 }
 
 __device__ __forceinline__ float ex2c(float x) {
@@ -51,13 +51,14 @@ __device__ __forceinline__ float2 unpack2c(uint32_t w) { return __bfloat1622floa
 }  // namespace
 
 template <int NS, int MODE>
-__global__ void __launch_bounds__(CH_THREADS, 1)
+__global__ void __launch_bounds__(ch_threads(MODE), 1)
 k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, long long bnd_bs, float *carry_out, float *final_out,
            const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmH,
            const __grid_constant__ CUtensorMap tmOut) {
     constexpr bool BWD = MODE == CHAIN_BWD;
+    constexpr int CH_STAGES = ch_stages(MODE);
     constexpr uint32_t STAGE = ch_stage_bytes(MODE, NS), OFF_X = NS * 256, OFF_H = OFF_X + 16384, OFF_W = OFF_H + NS * 128;
-    constexpr uint32_t OFF_OUT = CH_STAGES * STAGE, OFF_VEC = OFF_OUT + (BWD ? 1 : 2) * 8 * 2048;
+    constexpr uint32_t OFF_OUT = CH_STAGES * STAGE, OFF_VEC = OFF_OUT + 8 * 2048;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     __shared__ uint64_t full[CH_STAGES], scaled[CH_STAGES], empty[CH_STAGES], mdone[2], dempty[2], vfull[CH_VEC], vempty[CH_VEC];
@@ -69,12 +70,12 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     if (tid == 0) {
         for (int i = 0; i < CH_STAGES; ++i) {
             mbar_init(&full[i], 1);
-            mbar_init(&scaled[i], 4);
-            mbar_init(&empty[i], BWD ? 8 : 1);     // BWD: the carry warps read the stage last; FWD: the MMAs do
+            mbar_init(&scaled[i], 8);
+            mbar_init(&empty[i], BWD ? 8 + 4 : 1); // BWD: the carry and rho2 warps read the stage last; FWD: the MMAs do
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&mdone[i], 1);
-            mbar_init(&dempty[i], 8);
+            mbar_init(&dempty[i], BWD ? 8 + 4 : 8);
         }
         for (int i = 0; i < CH_VEC; ++i) {
             mbar_init(&vfull[i], 1);
@@ -100,15 +101,15 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 const int st = i % CH_STAGES, c = chunk_of(i), tok = p.t0 + c * CH_T;
                 unsigned char *sb = smem + st * STAGE;
                 if (i >= CH_STAGES) mbar_wait(&empty[st], (i / CH_STAGES - 1) & 1, abortp, p.status);
-                mbar_arrive_expect_tx(&full[st], BWD ? STAGE - 1024 + 528 : STAGE);
+                mbar_arrive_expect_tx(&full[st], BWD ? STAGE - 1024 + 16 : STAGE);
                 tma_load_3d(sb + OFF_X, &tmX, &full[st], h * 64, tok, b);
 #pragma unroll
                 for (int nh = 0; nh < NS / 64; ++nh) tma_load_3d(sb + nh * 16384, &tmV, &full[st], g * NS + nh * 64, tok, b);
                 if (BWD) {
                     const float *rec = p.rec + (((size_t)b * p.H + h) * p.ncs + c) * REC_FLOATS;
                     tma_load_3d(sb + OFF_H, &tmH, &full[st], 0, ((b * p.ncs + c) * p.H + h) * NS, 0);
-                    bulk_load(sb + OFF_W, rec + REC_OC, 512, &full[st]);
-                    bulk_load(sb + OFF_W + 512, rec + REC_DECAY, 16, &full[st]);
+                    bulk_load(sb + OFF_W, rec + REC_OC, 1024, &full[st]);
+                    bulk_load(sb + OFF_W + 1024, rec + REC_DECAY, 16, &full[st]);
                 }
                 if (i + CH_AHEAD < nc) tma_prefetch_3d(&tmX, h * 64, p.t0 + chunk_of(i + CH_AHEAD) * CH_T, b);
             }
@@ -197,8 +198,16 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 for (int m = 0; m < 4; ++m) w[m] = ex2c(fminf(last - cs[m], 0.f)) * d[m];
                 if (i >= CH_VEC) mbar_wait(&vempty[vb], (i / CH_VEC - 1) & 1, abortp, p.status);
                 float *v = vec + vb * CH_VEC_FLOATS;
-                *reinterpret_cast<float4 *>(v + lane * 4) = make_float4(w[0], w[1], w[2], w[3]);
-                if (lane == 0) v[128] = decay;
+                RowScale ob[4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) ob[m] = row_scale(w[m]);
+                auto put_scales = [&](float *dst, const RowScale (&sc)[4]) {
+                    uint4 *d4 = reinterpret_cast<uint4 *>(dst) + lane * 2;
+                    d4[0] = make_uint4(sc[0].hi, sc[0].lo, sc[1].hi, sc[1].lo);
+                    d4[1] = make_uint4(sc[2].hi, sc[2].lo, sc[3].hi, sc[3].lo);
+                };
+                put_scales(v, ob);
+                if (lane == 0) v[256] = decay;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&vfull[vb]);
                 const float lo = __shfl_sync(0xffffffffu, cs[3], lane | 7), hi = __shfl_sync(0xffffffffu, cs[0], lane & ~7);
@@ -213,50 +222,77 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 put(REC_CS, cs[0], cs[1], cs[2], cs[3]);
                 put(REC_DT, d[0], d[1], d[2], d[3]);
                 put(REC_CF, ex2c(lo - cs[0]) * d[0], ex2c(lo - cs[1]) * d[1], ex2c(lo - cs[2]) * d[2], ex2c(lo - cs[3]) * d[3]);
-                put(REC_OC, ex2c(cs[0]), ex2c(cs[1]), ex2c(cs[2]), ex2c(cs[3]));
-                put(REC_OB, w[0], w[1], w[2], w[3]);
+                const RowScale oc[4] = {row_scale(ex2c(cs[0])), row_scale(ex2c(cs[1])), row_scale(ex2c(cs[2])), row_scale(ex2c(cs[3]))};
+                put_scales(rec + REC_OC, oc);
+                put_scales(rec + REC_OB, ob);
             }
         }
-    } else if (warp < 8) {
+    } else if (warp < 12) {
         // ------------------------------------------------------------ the blocks' rows times their weights, in place (a weight is
         // uniform along a row, so the swizzle does not matter)
         const int th = tid - 128;
         for (int i = 0; i < nc; ++i) {
             const int st = i % CH_STAGES;
             unsigned char *sb = smem + st * STAGE;
-            const float *w = BWD ? reinterpret_cast<const float *>(sb + OFF_W) : reinterpret_cast<const float *>(smem + OFF_VEC) + (i % CH_VEC) * CH_VEC_FLOATS;
+            const RowScale *w = reinterpret_cast<const RowScale *>(BWD ? sb + OFF_W : smem + OFF_VEC + (i % CH_VEC) * CH_VEC_FLOATS * 4);
             mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
             if (!BWD) mbar_wait(&vfull[i % CH_VEC], (i / CH_VEC) & 1, abortp, p.status);
             uint4 *x4 = reinterpret_cast<uint4 *>(sb + OFF_X) + th;
-            uint4 v[8];
-            float f[8];
+            uint4 v[4];
+            RowScale f[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                v[k] = x4[k * 128];
-                f[k] = w[(th >> 3) + 16 * k];
+            for (int k = 0; k < 4; ++k) {
+                v[k] = x4[k * 256];
+                f[k] = w[(th >> 3) + 32 * k];
             }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                uint32_t *e = reinterpret_cast<uint32_t *>(&v[k]);
-#pragma unroll
-                for (int m = 0; m < 4; ++m) {
-                    const float2 t = __fmul2_rn(unpack2c(e[m]), make_float2(f[k], f[k]));
-                    e[m] = pack2c(t.x, t.y);
-                }
-                x4[k * 128] = v[k];
+            for (int k = 0; k < 4; ++k) {
+                scale8(v[k], f[k]);
+                x4[k * 256] = v[k];
             }
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&scaled[st]);
         }
+    } else if (BWD && warp >= 20) {
+        // ------------------------------------------------------------ rho2: row dot of the scaled dy row and H_in C, t = 32 q + lane
+        const int q = warp & 3, r = q * 32 + lane;
+        for (int i = 0; i < nc; ++i) {
+            const int st = i % CH_STAGES, bf = i & 1, c = chunk_of(i);
+            const unsigned char *dr = smem + st * STAGE + OFF_X + r * 128;
+            mbar_wait(&mdone[bf], (i >> 1) & 1, abortp, p.status);
+            __syncwarp();
+            tc_fence_after_sync();
+            float2 acc = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                float d[32];
+                tmem_ld32(tm + ((uint32_t)(q * 32) << 16) + 128 + bf * 64 + hf * 32, d);
+#pragma unroll
+                for (int ch = 0; ch < 4; ++ch) {
+                    const uint4 dv = *reinterpret_cast<const uint4 *>(dr + (((hf * 4 + ch) ^ (r & 7)) << 4));
+                    const uint32_t *e = reinterpret_cast<const uint32_t *>(&dv);
+#pragma unroll
+                    for (int m = 0; m < 4; ++m) acc = __ffma2_rn(unpack2c(e[m]), make_float2(d[ch * 8 + 2 * m], d[ch * 8 + 2 * m + 1]), acc);
+                }
+            }
+            tc_fence_before_sync();
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                mbar_arrive(&dempty[bf]);
+                mbar_arrive(&empty[st]);
+            }
+            p.rho2[(((size_t)b * p.H + h) * p.ncs + c) * CH_T + r] = acc.x + acc.y;
+        }
     } else {
         // ------------------------------------------------------------ carry: warp (q, half) holds state rows
         // n = 32 q + lane, columns p = 32 half ..; as rows of time, t = 32 q + lane
-        const int q = warp & 3, half = (warp - 8) >> 2;
+        const int q = warp & 3, half = (warp - 12) >> 2;
         const bool act = q * 32 < NS;
         const uint32_t tl = tm + ((uint32_t)(q * 32) << 16) + half * 32;
         const float *vec = reinterpret_cast<const float *>(smem + OFF_VEC);
-        unsigned char *stg = smem + OFF_OUT + (warp - 8) * 2048;      // [CHAIN_FWD: 2 buffers][32 rows][64 B], 64-byte swizzle
+        unsigned char *stg = smem + OFF_OUT + (warp - 12) * 2048, *row = stg + lane * 64;      // [32 rows][64 B], 64-byte swizzle
         const size_t so = (size_t)h * 64 * NS + (size_t)(half * 32) * NS + q * 32 + lane;
         float carry[32];
 #pragma unroll
@@ -265,16 +301,11 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
 #pragma unroll
             for (int j = 0; j < 32; ++j) bnd_out[(size_t)b * bnd_bs + so + (size_t)j * NS] = carry[j];
         }
-
         for (int i = 0; i < nc; ++i) {
             const int st = i % CH_STAGES, bf = i & 1, c = chunk_of(i);
-            // the carried state in bf16: H entering block c, or the gradient leaving it
+            // the carried state in bf16 (H entering block c, or the gradient leaving it) on its way out while the block's sum is made
             if (act) {
-                unsigned char *tile = stg + (BWD ? 0 : bf * 16384), *row = tile + lane * 64;
-                if (lane == 0) {
-                    if (BWD) tma_store_wait_read();
-                    else tma_store_wait_read_but_one();
-                }
+                if (lane == 0) tma_store_wait_read();
                 __syncwarp();
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
@@ -285,15 +316,12 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 fence_proxy_async_smem();
                 __syncwarp();
                 if (lane == 0) {
-                    tma_store_3d(&tmOut, tile, half * 32, ((b * p.ncs + c) * p.H + h) * NS + q * 32, 0);
+                    tma_store_3d(&tmOut, stg, half * 32, ((b * p.ncs + c) * p.H + h) * NS + q * 32, 0);
                     tma_store_commit();
                 }
             }
-            // where this block's decay (and H_in) come from
-            if (BWD) mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
-            else mbar_wait(&vfull[i % CH_VEC], (i / CH_VEC) & 1, abortp, p.status);
-            const float decay = BWD ? *reinterpret_cast<const float *>(smem + st * STAGE + OFF_W + 512) : vec[(i % CH_VEC) * CH_VEC_FLOATS + 128];
-            float dot = 0.f;
+            if (BWD) mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);      // H_in and the decay have landed
+            float2 dot = make_float2(0.f, 0.f);
             if (BWD && act) {       // <G, H_in> over this thread's slice
                 const unsigned char *hr = smem + st * STAGE + OFF_H + (q * 32 + lane) * 128;
 #pragma unroll
@@ -301,42 +329,24 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                     const uint4 hv = *reinterpret_cast<const uint4 *>(hr + (((half * 4 + ch) ^ (lane & 7)) << 4));
                     const uint32_t *e = reinterpret_cast<const uint32_t *>(&hv);
 #pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        const float2 f = unpack2c(e[m]);
-                        dot = fmaf(carry[ch * 8 + 2 * m], f.x, dot);
-                        dot = fmaf(carry[ch * 8 + 2 * m + 1], f.y, dot);
-                    }
+                    for (int m = 0; m < 4; ++m) dot = __ffma2_rn(make_float2(carry[ch * 8 + 2 * m], carry[ch * 8 + 2 * m + 1]), unpack2c(e[m]), dot);
                 }
             }
             mbar_wait(&mdone[bf], (i >> 1) & 1, abortp, p.status);
             __syncwarp();
             tc_fence_after_sync();
-            float d[32];
+            // (CHAIN_FWD: the scaling warps waited for the decay's buffer before the products could start)
+            const float decay = BWD ? *reinterpret_cast<const float *>(smem + st * STAGE + OFF_W + 1024) : vec[(i % CH_VEC) * CH_VEC_FLOATS + 256];
             if (act) {
+                float d[32];
                 tmem_ld32(tl + bf * 64, d);
+                const float2 dec2 = make_float2(decay, decay);
 #pragma unroll
-                for (int j = 0; j < 32; ++j) carry[j] = fmaf(decay, carry[j], d[j]);
-            }
-            if (BWD) {
-                tmem_ld32(tl + 128 + bf * 64, d);
-                const unsigned char *dr = smem + st * STAGE + OFF_X + (q * 32 + lane) * 128;
-                float r2 = 0.f;
-#pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {
-                    const uint4 dv = *reinterpret_cast<const uint4 *>(dr + (((half * 4 + ch) ^ (lane & 7)) << 4));
-                    const uint32_t *e = reinterpret_cast<const uint32_t *>(&dv);
-#pragma unroll
-                    for (int m = 0; m < 4; ++m) {
-                        const float2 f = unpack2c(e[m]);
-                        r2 = fmaf(f.x, d[ch * 8 + 2 * m], r2);
-                        r2 = fmaf(f.y, d[ch * 8 + 2 * m + 1], r2);
-                    }
+                for (int j = 0; j < 32; j += 2) {
+                    const float2 v = __ffma2_rn(dec2, make_float2(carry[j], carry[j + 1]), make_float2(d[j], d[j + 1]));
+                    carry[j] = v.x;
+                    carry[j + 1] = v.y;
                 }
-                const size_t vo = ((size_t)b * p.H + h) * p.ncs + c;
-                (half ? p.rho2b : p.rho2)[vo * CH_T + q * 32 + lane] = r2;
-#pragma unroll
-                for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-                if (lane == 0) p.ghdot[vo * 16 + (warp - 8)] = decay * dot;
             }
             tc_fence_before_sync();
             fence_proxy_async_smem();
@@ -345,6 +355,12 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 mbar_arrive(&dempty[bf]);
                 if (BWD) mbar_arrive(&empty[st]);
                 else mbar_arrive(&vempty[i % CH_VEC]);
+            }
+            if (BWD) {
+                float dt = dot.x + dot.y;
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) dt += __shfl_xor_sync(0xffffffffu, dt, off);
+                if (lane == 0) p.ghdot[((((size_t)b * p.H + h) * p.ncs + c) << 4) + (warp - 12)] = decay * dt;
             }
         }
         if (act) {
@@ -372,7 +388,7 @@ static cudaError_t launch_chain(const SegParams &p, const TcMaps &m, const float
     const cudaError_t e = allow_smem<k_chain_tc<NS, MODE>>((int)smem);
     if (e != cudaSuccess) return e;
     const bool bwd = MODE == CHAIN_BWD;
-    return launch_pdl(k_chain_tc<NS, MODE>, dim3(p.H, p.B), dim3(CH_THREADS), (size_t)smem, st, p, init, init_bs, bnd_out, bnd_bs, carry_out,
+    return launch_pdl(k_chain_tc<NS, MODE>, dim3(p.H, p.B), dim3(ch_threads(MODE)), (size_t)smem, st, p, init, init_bs, bnd_out, bnd_bs, carry_out,
                       final_out, bwd ? m.dy : m.x, bwd ? m.Cm : m.Bm, m.H, bwd ? m.Gst : m.Hst);
 }
 
