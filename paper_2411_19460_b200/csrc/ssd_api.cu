@@ -44,18 +44,19 @@ static void prof_end(ProfEvent *ev, cudaStream_t st) {
     if (ev) cudaEventRecord(ev->b, st);
 }
 
-// Scratch regions of one call.  What the kernels of neighbouring segments touch at the same time exists twice on the
-// tensor-core path (copy k & 1 belongs to segment k).
+// Scratch regions of one call.  What the kernels of neighbouring segments touch at the same time exists more than once on the
+// tensor-core path: the records and states that the forward chain leaves three times, so that it runs two segments ahead (the
+// backward's critical path is then the gradient chain alone; with two copies it waited for the large kernels two segments
+// back: 24 heads, 2048-token segments, 52 us a segment instead of 36), the rest twice.
 struct Layout {
-    size_t status, Hst, hcarry, Gst, gcarry, cbt, dAp, dDp;
-    size_t rec[2], cs[2], dtT[2], Hbf[2];
+    size_t status, Hst, hcarry, Gst, gcarry, cbt, dAp, dDp, cs, dtT;
+    size_t rec[3], Hbf[3];
     size_t Gbf[2], ghdot[2], ddt_dir[2], rho[2], rho2[2], psi[2], psi2[2], pB[2], pC[2];
     size_t total;
 };
 
-// Second copies of the per-segment scratch (and with them the state chain running one segment ahead) pay only when
-// there are segments enough to pipeline; with two or three long segments they would cost a third more scratch for
-// a per cent or two.
+// All the copies of the per-segment scratch (and with them the forward's state chain running ahead of y) pay only when there are
+// segments enough to pipeline; two or three long segments get a second copy of the forward chain's output and one of the rest.
 static const int kMinSegmentsForTwins = 4;
 
 struct Plan {
@@ -124,7 +125,9 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
     return SSD_OK;
 }
 
-// `twins`: whether the second copies may exist at all (not for callers that keep every kernel in order on one
+static int chain_copies(int nseg) { return nseg >= kMinSegmentsForTwins ? 3 : nseg > 1 ? 2 : 1; }
+
+// `twins`: whether the second and third copies may exist at all (not for callers that keep every kernel in order on one
 // stream: SSD_FLAG_SERIAL and the built-in scratch of ssd_fwd_static_ws).
 static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
     const size_t PN = (size_t)pl.P * pl.N, BH = (size_t)pl.B * pl.H;
@@ -138,17 +141,20 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
         r[0] = take(bytes);
         r[1] = two ? take(bytes) : r[0];
     };
+    auto take3 = [&](size_t (&r)[3], size_t bytes, int copies) {
+        for (int i = 0; i < 3; ++i) r[i] = i < copies ? take(bytes) : r[i - copies];
+    };
     memset(&lo, 0, sizeof(lo));
     lo.status = take(256);
     lo.hcarry = take(BH * PN * sizeof(float));
-    // the vectors and records (a fraction of the states) exist twice for any number of segments, so that the scratch is a function of
-    // the segment length that only rises
+    // the vectors and records (a fraction of the states) exist as often for any number of segments, so that the scratch is a
+    // function of the segment length that only rises
     if (pl.use_tc) {
-        take2(lo.rec, BH * pl.ncs * REC_FLOATS * sizeof(float), twins);
-        take2(lo.Hbf, stb, twin);
+        take3(lo.rec, BH * pl.ncs * REC_FLOATS * sizeof(float), twins ? 3 : 1);
+        take3(lo.Hbf, stb, twins ? chain_copies(pl.nseg) : 1);
     } else {
-        take2(lo.cs, vec, false);
-        take2(lo.dtT, vec, false);
+        lo.cs = take(vec);
+        lo.dtT = take(vec);
         lo.Hst = take(st);
         lo.cbt = take((size_t)pl.B * pl.ncs * pl.G * pl.Q * pl.Q * sizeof(float));
     }
@@ -196,13 +202,13 @@ static int check_device() {
 // state-gradient part of the chain, s[1] / s[3] the dB/dC kernel of even / odd segments beside dx on the caller's
 // stream, s[2] a segment's two finishing kernels.  Created on first use, never
 // destroyed (they hold no device memory); the caller's stream stays the only one the caller has to order
-// against.  Events indexed [2] alternate with the segment, like the second copies of the scratch regions.
+// against.  Events indexed [2] and [3] go round with the segment, like the copies of the scratch regions.
 struct SideStreams {
     int dev = -1;
     cudaStream_t s[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // gradient chain | dB/dC, even | tails | dB/dC, odd | recompute
     cudaEvent_t start = nullptr;
-    cudaEvent_t chain_done[2] = {nullptr, nullptr}, big_done[2] = {nullptr, nullptr}, tail_done[2] = {nullptr, nullptr};
-    cudaEvent_t rec_done[2] = {nullptr, nullptr}, join[2] = {nullptr, nullptr}, dx_done[2] = {nullptr, nullptr};
+    cudaEvent_t chain_done[2] = {nullptr, nullptr}, big_done[3] = {nullptr, nullptr, nullptr}, tail_done[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t rec_done[3] = {nullptr, nullptr, nullptr}, join[2] = {nullptr, nullptr}, dx_done[2] = {nullptr, nullptr};
 };
 static SideStreams *side_streams() {
     static thread_local std::vector<SideStreams> all;
@@ -214,8 +220,8 @@ static SideStreams *side_streams() {
     a.dev = dev;
     for (int i = 0; i < 5; ++i)
         if (cudaStreamCreateWithFlags(&a.s[i], cudaStreamNonBlocking) != cudaSuccess) return nullptr;
-    cudaEvent_t *evs[] = {&a.start, &a.chain_done[0], &a.chain_done[1], &a.big_done[0], &a.big_done[1], &a.tail_done[0],
-                          &a.tail_done[1], &a.rec_done[0], &a.rec_done[1], &a.join[0], &a.join[1], &a.dx_done[0], &a.dx_done[1]};
+    cudaEvent_t *evs[] = {&a.start, &a.chain_done[0], &a.chain_done[1], &a.big_done[0], &a.big_done[1], &a.big_done[2], &a.tail_done[0],
+                          &a.tail_done[1], &a.tail_done[2], &a.rec_done[0], &a.rec_done[1], &a.rec_done[2], &a.join[0], &a.join[1], &a.dx_done[0], &a.dx_done[1]};
     for (cudaEvent_t *ev : evs)
         if (cudaEventCreateWithFlags(ev, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     all.push_back(a);
@@ -244,15 +250,16 @@ static SideStreams *side_streams() {
         }                                               \
     } while (0)
 
-// Points the kernels at copy 0 or 1 of the scratch regions that may exist twice.
-static void select_copy(const Layout &lo, void *ws, int k, SegParams &sp) {
+// Points the kernels at copy kc of the regions that the forward chain writes and copy k of the others.
+static void select_copy(const Layout &lo, void *ws, int kc, int k, SegParams &sp) {
     char *w = (char *)ws;
-    auto f = [&](const size_t (&r)[2]) { return r[k] ? (float *)(w + r[k]) : nullptr; };
-    sp.rec = f(lo.rec);
-    sp.cs = f(lo.cs);
-    sp.dtT = sp.rec ? sp.rec + REC_DT : f(lo.dtT);
+    auto at = [&](size_t r) { return r ? (float *)(w + r) : nullptr; };
+    auto f = [&](const size_t (&r)[2]) { return at(r[k]); };
+    sp.rec = at(lo.rec[kc]);
+    sp.cs = at(lo.cs);
+    sp.dtT = sp.rec ? sp.rec + REC_DT : at(lo.dtT);
     sp.dt_stride = sp.rec ? (int)REC_FLOATS : sp.Q;
-    sp.Hbf = (__nv_bfloat16 *)f(lo.Hbf);
+    sp.Hbf = (__nv_bfloat16 *)at(lo.Hbf[kc]);
     sp.Gbf = (__nv_bfloat16 *)f(lo.Gbf);
     sp.ghdot = f(lo.ghdot);
     sp.ddt_dir = f(lo.ddt_dir);
@@ -269,6 +276,7 @@ static void fill_params(const Plan &pl, const Layout &lo, void *ws, SegParams &s
     sp.B = pl.B; sp.L = pl.L; sp.H = pl.H; sp.P = pl.P; sp.N = pl.N; sp.G = pl.G; sp.Q = pl.Q;
     sp.hpg = pl.hpg; sp.ncs = pl.ncs; sp.nct = pl.nct; sp.nsl = pl.nsl;
     sp.ndd = pl.use_tc ? 4 : pl.Q / 64;
+    sp.scan_ctas = kNumSMs;
     sp.ngh = pl.use_tc ? 8 : pl.P * pl.N / kStatePassElems;
     sp.x_bs = pl.x_bs; sp.dt_bs = pl.dt_bs; sp.bc_bs = pl.bc_bs;
     char *w = (char *)ws;
@@ -281,7 +289,7 @@ static void fill_params(const Plan &pl, const Layout &lo, void *ws, SegParams &s
     sp.gcarry = (float *)(w + lo.gcarry);
     sp.dAp = (float *)(w + lo.dAp);
     sp.dDp = (float *)(w + lo.dDp);
-    select_copy(lo, ws, 0, sp);
+    select_copy(lo, ws, 0, 0, sp);
 }
 
 static void set_segment(const Plan &pl, int k, SegParams &sp) {
@@ -289,6 +297,26 @@ static void set_segment(const Plan &pl, int k, SegParams &sp) {
     const int len = (pl.L - sp.t0 < pl.seg) ? pl.L - sp.t0 : pl.seg;
     sp.nc = len / pl.Q;
     sp.c0 = sp.t0 / pl.Q;
+}
+
+// CTAs of the y / dx kernel (its results do not depend on them).  It takes the whole GPU unless the segments are pipelined and
+// small: then the kernels that run beside it (chain kernels, one CTA per head; dB/dC) get SMs of their own, because a chain
+// that waits for the large kernel to finish makes the segments serial (24 heads, 2048-token segments: a chain kernel takes 15
+// us on 24 SMs, y 8 us on all of them).  Not where less than a quarter of the GPU would be left for it.
+static int scan_ctas(const SegParams &sp, bool pipelined, bool bwd) {
+    if (!pipelined) return kNumSMs;
+    const int beside = sp.B * sp.H * (bwd ? 2 : 1) + (bwd ? sp.nc * sp.nsl * sp.G * sp.B : 0);
+    return kNumSMs - beside >= kNumSMs / 4 ? kNumSMs - beside : kNumSMs;
+}
+
+// The tensor maps of copies 0 .. n-1 of the forward chain's output, each with the gradients' copy of the same parity.
+static bool state_maps(const Layout &lo, void *ws, const SegParams &sp0, TcMaps *m, int n) {
+    SegParams sp = sp0;
+    for (int i = 0; i < n; ++i) {
+        select_copy(lo, ws, i, i & 1, sp);
+        if (!tc_state_maps(sp, m[i])) return false;
+    }
+    return true;
 }
 
 static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt, const float *A,
@@ -321,33 +349,32 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     if (pl.use_tc && pl.nseg >= kMinSegmentsForTwins && may_use_helper_stream && !pl.serial && !g_prof_on) {
         // Algorithm 1 with the state chain one segment ahead: chunk states and state pass of segment k run on a
         // helper stream while the caller's stream still computes y of segment k-1, whose last, partly idle wave
-        // they fill.  What both touch (cumulative sums, dt per chunk, bf16 chunk states) exists twice and
-        // alternates; the fp32 chunk sums and the carried state belong to the chain alone.
+        // they fill.  What both touch (records, bf16 states) exists three times and goes round; the carried state belongs
+        // to the chain alone.
         SideStreams *side = side_streams();
         if (!side) { g_last_cuda = (int)cudaGetLastError(); return SSD_ECUDA; }
-        TcMaps maps_b;
-        select_copy(lo, ws, 1, sp);
-        if (!tc_make_maps(sp, maps_b)) return SSD_ECUDA;
+        TcMaps mk[3] = {maps, maps, maps};
+        if (!state_maps(lo, ws, sp, mk, 3)) return SSD_ECUDA;
         cudaStream_t chain = side->s[0];
         SSD_TRY(cudaEventRecord(side->start, st));
         SSD_TRY(cudaStreamWaitEvent(chain, side->start, 0));
         for (int k = 0; k < pl.nseg; ++k) {
-            const int par = k & 1;
+            const int par = k & 1, cp = k % 3;
             set_segment(pl, k, sp);
-            select_copy(lo, ws, par, sp);
-            const TcMaps &mk = par ? maps_b : maps;
-            if (k >= 2) SSD_TRY(cudaStreamWaitEvent(chain, side->big_done[par], 0));   // y of segment k-2 has read this copy
+            select_copy(lo, ws, cp, par, sp);
+            if (k >= 3) SSD_TRY(cudaStreamWaitEvent(chain, side->big_done[cp], 0));   // y of segment k-3 has read this copy
             {
                 cudaStream_t st = chain;
                 const float *init = (k == 0) ? h0 : sp.hcarry;
                 float *bnd = boundary ? boundary + (size_t)k * pl.H * PN : nullptr;
-                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, mk, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN,
+                SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, mk[cp], init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN,
                                                               (k == pl.nseg - 1) ? h_final : nullptr, st));
                 SSD_TRY(cudaEventRecord(side->chain_done[par], st));
             }
             SSD_TRY(cudaStreamWaitEvent(st, side->chain_done[par], 0));
-            SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, mk, SC_FWD, st));
-            if (k + 2 < pl.nseg) SSD_TRY(cudaEventRecord(side->big_done[par], st));
+            sp.scan_ctas = scan_ctas(sp, true, false);
+            SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, mk[cp], SC_FWD, st));
+            if (k + 3 < pl.nseg) SSD_TRY(cudaEventRecord(side->big_done[cp], st));
         }
         return SSD_OK;
     }
@@ -510,36 +537,35 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         //   tail(k) : the two short finishing kernels.
         // chain(k-1) runs on its own stream while big(k) is busy and fills the SMs that big(k)'s last, partly
         // idle wave leaves free; tail(k) runs under big(k-1)'s predecessors likewise.  What chain(k-1) writes and
-        // big(k) / tail(k) read exists twice and alternates with the segment (cumulative sums, dt per chunk, both
-        // bf16 state copies, rho2, <G,H>); the fp32 chunk sums and the carried gradient belong to the chain alone.
-        const bool twin = pl.nseg >= kMinSegmentsForTwins;    // else one copy: chain(k) then also waits for tail(k+1)
-        TcMaps maps_b;
-        if (twin) {
-            select_copy(lo, ws, 1, sp);
-            if (!tc_make_maps(sp, maps_b)) return SSD_ECUDA;
-        }
+        // big(k) / tail(k) read exists more than once and goes round with the segments; the carried gradient belongs to the
+        // chain alone.
+        const bool twin = pl.nseg >= kMinSegmentsForTwins;    // else one copy of what the gradient chain writes
+        const int ncp = chain_copies(pl.nseg), npar = twin ? 2 : 1;
+        TcMaps cmaps[3] = {maps, maps, maps};
+        if (!state_maps(lo, ws, sp, cmaps, ncp)) return SSD_ECUDA;
         cudaStream_t grads = side->s[0], recomp = side->s[4], tails = side->s[2];
         SSD_TRY(cudaEventRecord(side->start, st));
         SSD_TRY(cudaStreamWaitEvent(recomp, side->start, 0));
         SSD_TRY(cudaStreamWaitEvent(grads, side->start, 0));
-        int par = 0;
         for (int k = pl.nseg - 1; k >= 0; --k) {
-            par = twin ? ((pl.nseg - 1 - k) & 1) : 0;
+            const int i = pl.nseg - 1 - k, par = i % npar, cp = i % ncp;
             set_segment(pl, k, sp);
-            select_copy(lo, ws, par, sp);
-            const TcMaps &mk = par ? maps_b : maps;
-            // ---- chain(k), first half: Recompute_Forward.  Its copy was last read by big(k+2) and tail(k+2) (of k+1
-            // when there is one copy only); the fp32 chunk sums belong to this stream alone.
-            if (k + (twin ? 2 : 1) <= pl.nseg - 1) SSD_TRY(cudaStreamWaitEvent(recomp, side->tail_done[par], 0));
+            select_copy(lo, ws, cp, par, sp);
+            TcMaps mk = cmaps[cp];
+            if (par != (cp & 1)) { mk.G = cmaps[par].G; mk.Gst = cmaps[par].Gst; }
+            // ---- chain(k), first half: Recompute_Forward.  Its copy was last read by big(k + ncp) and tail(k + ncp).
+            if (i >= ncp) SSD_TRY(cudaStreamWaitEvent(recomp, side->tail_done[(i - ncp) % 3], 0));
             {
                 cudaStream_t st = recomp;
                 SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, mk, boundary + (size_t)k * pl.H * PN, (long long)pl.nseg * pl.H * PN,
                                                               nullptr, 0, nullptr, st));
-                SSD_TRY(cudaEventRecord(side->rec_done[par], st));
+                SSD_TRY(cudaEventRecord(side->rec_done[cp], st));
             }
             // ---- chain(k), second half: the state gradients, which alone wait for segment k+1 (stream order: the
             // gradient handed left, and the fp32 contributions that belong to this stream alone)
-            SSD_TRY(cudaStreamWaitEvent(grads, side->rec_done[par], 0));
+            // What it writes was last read by big and tail of the segment npar before.
+            SSD_TRY(cudaStreamWaitEvent(grads, side->rec_done[cp], 0));
+            if (i >= npar) SSD_TRY(cudaStreamWaitEvent(grads, side->tail_done[(i - npar) % 3], 0));
             {
                 cudaStream_t st = grads;
                 const float *ginit = (k == pl.nseg - 1) ? dh_final : sp.gcarry;
@@ -548,7 +574,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
                 SSD_TRY(cudaEventRecord(side->chain_done[par], st));
             }
             // ---- big(k); what it leaves for tail(k) (direct ddt, rho, psi, partial dB/dC slices) alternates too, and
-            // chain(k) has already waited for tail(k+2), the last reader of this copy.  The dB/dC kernels of
+            // chain(k) has already waited for the last reader of this copy.  The dB/dC kernels of
             // neighbouring segments are on different streams: with short segments one alone does not fill the GPU.
             cudaStream_t bcs = side->s[par ? 3 : 1];
             SSD_TRY(cudaStreamWaitEvent(st, side->chain_done[par], 0));
@@ -563,6 +589,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
                 }
                 SSD_TRY(cudaEventRecord(side->join[par], st));
             }
+            sp.scan_ctas = scan_ctas(sp, twin, true);
             SSD_LAUNCH(KIND_BWD_DX, launch_scan_tc(sp, mk, SC_DX, st));
             SSD_TRY(cudaEventRecord(side->dx_done[par], st));
             // ---- tail(k), after both
@@ -571,10 +598,10 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
             {
                 cudaStream_t st = tails;
                 SSD_LAUNCH(KIND_BWD_FINISH, launch_bwd_tail(sp, pl.dtype, st));
-                SSD_TRY(cudaEventRecord(side->tail_done[par], st));
+                SSD_TRY(cudaEventRecord(side->tail_done[i % 3], st));
             }
         }
-        SSD_TRY(cudaStreamWaitEvent(st, side->tail_done[par], 0));   // the finishing stream is in order: this covers every segment
+        SSD_TRY(cudaStreamWaitEvent(st, side->tail_done[(pl.nseg - 1) % 3], 0));   // the finishing stream is in order: this covers every segment
     } else {
         for (int k = pl.nseg - 1; k >= 0; --k) {
             set_segment(pl, k, sp);

@@ -80,6 +80,7 @@ struct SegParams {
     int nct;       // chunks in the whole sequence (L / Q)
     int nsl;       // head slices per group in the dB/dC partial buffers
     int ndd;       // partial sums of dD per (head, chunk) that the kernels of this path write (<= 4)
+    int scan_ctas; // CTAs of the y / dx kernel, at most (no effect on results)
     int ngh;       // partial sums of <G,H> per (head, chunk) (<= 16)
     int tiles;     // CUDA-core path: 64-step tiles per chunk (rho, psi and the slices come per tile); tensor-core path: 0
     float dx_skip;    // 1 when dx also takes dy (a skip connection around the layer), else 0
@@ -163,6 +164,7 @@ struct TcMaps {
 };
 bool tc_supported(int dtype, int flags, int P, int N, int Q);
 bool tc_make_maps(const SegParams &p, TcMaps &m);
+bool tc_state_maps(const SegParams &p, TcMaps &m);
 // ssd_tc_chain.cu : block sums and the recurrence over the blocks.  init: state (gradient) entering the segment (NULL = zeros),
 // batch stride init_bs; boundary_out (nullable): where to store that state, batch stride bnd_bs; final_out nullable.
 enum { CHAIN_FWD = 0, CHAIN_BWD = 1 };

@@ -59,7 +59,12 @@ bool tc_make_maps(const SegParams &p, TcMaps &m) {
     if (p.dx) ok = ok && make_map3(&m.dx, p.dx, HP, p.L, p.B, HP, p.x_bs, 128);
     if (p.Bm) ok = ok && make_map3(&m.Bm, p.Bm, GN, p.L, p.B, GN, p.bc_bs, 128);
     if (p.Cm) ok = ok && make_map3(&m.Cm, p.Cm, GN, p.L, p.B, GN, p.bc_bs, 128);
-    // bf16 states viewed as [B*ncs*H*N rows][64]
+    return ok && tc_state_maps(p, m);
+}
+
+// The maps of the bf16 states alone, viewed as [B*ncs*H*N rows][64].
+bool tc_state_maps(const SegParams &p, TcMaps &m) {
+    bool ok = true;
     const uint64_t srows = (uint64_t)p.B * p.ncs * p.H * p.N;
     if (p.Hbf) {
         ok = ok && make_map3(&m.H, p.Hbf, 64, srows, 1, 64, srows * 64, p.N);

@@ -89,22 +89,35 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    pdl_launch_dependents();
-    pdl_wait();
+    // What the kernel before this one in the stream may still write, or still read where this one writes, is waited for in the
+    // roles that touch it; x, dt, B, C and dy are older than that kernel, so the first blocks are loaded and scaled under its end.
     const uint32_t tm = tmem_base;
     volatile uint32_t *abortp = &abort_flag;
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (elect_one()) {
-            for (int i = 0; i < nc; ++i) {
-                const int st = i % CH_STAGES, c = chunk_of(i), tok = p.t0 + c * CH_T;
+            auto load_inputs = [&](int i) {
+                const int st = i % CH_STAGES, tok = p.t0 + chunk_of(i) * CH_T;
                 unsigned char *sb = smem + st * STAGE;
-                if (i >= CH_STAGES) mbar_wait(&empty[st], (i / CH_STAGES - 1) & 1, abortp, p.status);
                 mbar_arrive_expect_tx(&full[st], BWD ? STAGE - 1024 + 16 : STAGE);
                 tma_load_3d(sb + OFF_X, &tmX, &full[st], h * 64, tok, b);
 #pragma unroll
                 for (int nh = 0; nh < NS / 64; ++nh) tma_load_3d(sb + nh * 16384, &tmV, &full[st], g * NS + nh * 64, tok, b);
+            };
+            const int ahead = nc < CH_STAGES ? nc : CH_STAGES;
+            for (int i = 0; i < ahead; ++i) load_inputs(i);
+            if (BWD) pdl_wait();                   // the records and states of the forward chain
+            for (int i = 0; i < nc; ++i) {
+                const int st = i % CH_STAGES, c = chunk_of(i);
+                unsigned char *sb = smem + st * STAGE;
+                if (i >= CH_STAGES) {
+                    mbar_wait(&empty[st], (i / CH_STAGES - 1) & 1, abortp, p.status);
+                    load_inputs(i);
+                }
+                // the next launch's first loads and products take about as long as the blocks that are left here; much earlier,
+                // and its CTAs would hold SMs idle
+                if (i + CH_STAGES + 1 == nc) pdl_launch_dependents();
                 if (BWD) {
                     const float *rec = p.rec + (((size_t)b * p.H + h) * p.ncs + c) * REC_FLOATS;
                     tma_load_3d(sb + OFF_H, &tmH, &full[st], 0, ((b * p.ncs + c) * p.H + h) * NS, 0);
@@ -113,6 +126,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 }
                 if (i + CH_AHEAD < nc) tma_prefetch_3d(&tmX, h * 64, p.t0 + chunk_of(i + CH_AHEAD) * CH_T, b);
             }
+            if (nc <= CH_STAGES) pdl_launch_dependents();
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
@@ -210,6 +224,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 if (lane == 0) v[256] = decay;
                 __syncwarp();
                 if (lane == 0) mbar_arrive(&vfull[vb]);
+                if (i == first) pdl_wait();        // the earlier kernels have read what this copy of the records held
                 const float lo = __shfl_sync(0xffffffffu, cs[3], lane | 7), hi = __shfl_sync(0xffffffffu, cs[0], lane & ~7);
                 const float bi = __shfl_sync(0xffffffffu, cs[0], ((lane >> 2) & 3) * 8), bj = __shfl_sync(0xffffffffu, cs[3], (lane & 3) * 8 + 7);
                 float *rec = p.rec + (((size_t)b * p.H + h) * p.ncs + i) * REC_FLOATS;
@@ -257,6 +272,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     } else if (BWD && warp >= 20) {
         // ------------------------------------------------------------ rho2: row dot of the scaled dy row and H_in C, t = 32 q + lane
         const int q = warp & 3, r = q * 32 + lane;
+        pdl_wait();
         for (int i = 0; i < nc; ++i) {
             const int st = i % CH_STAGES, bf = i & 1, c = chunk_of(i);
             const unsigned char *dr = smem + st * STAGE + OFF_X + r * 128;
@@ -295,6 +311,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
         unsigned char *stg = smem + OFF_OUT + (warp - 12) * 2048, *row = stg + lane * 64;      // [32 rows][64 B], 64-byte swizzle
         const size_t so = (size_t)h * 64 * NS + (size_t)(half * 32) * NS + q * 32 + lane;
         float carry[32];
+        pdl_wait();                                // the carry that the previous segment's launch left; the earlier states have been read
 #pragma unroll
         for (int j = 0; j < 32; ++j) carry[j] = init && act ? init[(size_t)b * init_bs + so + (size_t)j * NS] : 0.f;
         if (bnd_out && act) {

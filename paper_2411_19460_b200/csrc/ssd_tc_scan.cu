@@ -13,7 +13,7 @@
 // tensor memory twice: scores (fp32, 128 columns, made once per block and group), two masked tiles (bf16, 64 columns
 // each, the A operand straight from tensor memory: no shared-memory ring, no proxy fence) and two pairs of accumulators.
 //
-// Work is the flat list of (batch, block, head); each of up to 148 CTAs takes an equal, contiguous part of it, so that the
+// Work is the flat list of (batch, block, head); each CTA (one per SM, fewer where other kernels run beside it) takes an equal, contiguous part of it, so that the
 // scores are made again only where a part crosses into the next block or group and every SM ends at the same time.  The
 // heads are per-output, so the cut points change no bit.  Roles, meeting only through mbarriers:
 //   warp 0 producer: ring of stages, one per head (value rows, chunk state, record of the mask's factors; SC_DX: x rows in
@@ -458,7 +458,7 @@ static cudaError_t launch_scan(const SegParams &p, const TcMaps &m, cudaStream_t
     cudaError_t e = allow_smem<k_scan_tc<NS, MODE>>((int)smem);
     if (e != cudaSuccess) return e;
     const long long units = (long long)p.B * p.nc * p.H;
-    const dim3 grid((unsigned)(units < kNumSMs ? units : kNumSMs));
+    const dim3 grid((unsigned)(units < p.scan_ctas ? units : p.scan_ctas));
     if (MODE == SC_FWD) return launch_pdl(k_scan_tc<NS, MODE>, grid, dim3(SC_THREADS), (size_t)smem, st, p, m.Cm, m.Bm, m.x, m.H, m.y, m.x);
     return launch_pdl(k_scan_tc<NS, MODE>, grid, dim3(SC_THREADS), (size_t)smem, st, p, m.Bm, m.Cm, m.dy, m.G, m.dx, m.x);
 }
