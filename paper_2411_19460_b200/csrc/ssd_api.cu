@@ -66,24 +66,26 @@ struct Plan {
     size_t esz;
 };
 
-// Head ranges per group for the dB/dC kernel, whose CTAs are (block, head range), for a reference launch of 32 blocks: the
-// launch's share of the GPU (a part of a wave still takes the time of its slowest CTA; beyond one wave the kernels of
-// neighbouring segments fill each other's gaps) times the time of a CTA, eight head-times of set-up and output plus its
-// heads.  A function of H and G only, so the summation order of dB/dC does not depend on the segment length.
-static int bc_head_split(int groups, int hpg) {
+// Head ranges per group for the dB/dC kernel, whose CTAs are (block, head range).  The launches of two neighbouring segments run
+// at the same time, beside the other kernels, so what counts is the time on the SMs, (CTAs) x (eight head-times of set-up and
+// output plus the heads of the range), once three launches of 32 blocks (or the whole sequence, if it is shorter) make a wave
+// (measured against one launch and two: 80 heads, 4096-token segments, 7.03 -> 6.80 -> 6.72 ms a step); below that the time
+// of one CTA.  A function of the sequence alone, so the summation order of dB/dC does not depend on the
+// segment length.
+static const int kBcBlocks = 96;
+static int bc_head_split(int blocks, int groups, int hpg) {
     int best = 1;
     double best_t = -1;
     const int max_split = hpg >= 4 ? hpg / 4 : 1;
     for (int ns = 1; ns <= max_split; ++ns) {
         const int hps = (hpg + ns - 1) / ns;
         if ((hpg + hps - 1) / hps != ns) continue;      // would leave an empty range
-        const double waves = 32.0 * groups * ns / kNumSMs;
+        const double waves = (double)(blocks < kBcBlocks ? blocks : kBcBlocks) * groups * ns / kNumSMs;
         const double t = (waves > 1 ? waves : 1) * (8 + hps);
         if (best_t < 0 || t < best_t) { best_t = t; best = ns; }
     }
     return best;
 }
-
 static int make_plan(const ssd_shape_t *s, Plan &pl) {
     if (!s) return SSD_EINVAL;
     if (s->B <= 0 || s->L <= 0 || s->H <= 0 || s->P <= 0 || s->N <= 0 || s->G <= 0 || s->chunk <= 0 ||
@@ -121,7 +123,7 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
     // Partial slices of the dB/dC head sums: one per CTA head range; on the CUDA-core path ranges of four heads (two where there
     // are few), each with a slot per 64-step tile and one for the inter-chunk term.
     const int per_range = pl.hpg >= 16 ? 4 : 2;
-    pl.nsl = pl.use_tc ? bc_head_split(pl.G, pl.hpg) : (pl.hpg + per_range - 1) / per_range * (pl.Q / 64 + 1);
+    pl.nsl = pl.use_tc ? bc_head_split(pl.B * pl.nct, pl.G, pl.hpg) : (pl.hpg + per_range - 1) / per_range * (pl.Q / 64 + 1);
     return SSD_OK;
 }
 
