@@ -4,6 +4,7 @@
 // for one SSD layer.  Checkpoint memory is set by the segment length: the scratch holds the chunk
 // states of ONE segment, the boundary buffer one state per segment.
 #include <atomic>
+#include <cmath>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -70,8 +71,7 @@ struct Plan {
 // at the same time, beside the other kernels, so what counts is the time on the SMs, (CTAs) x (eight head-times of set-up and
 // output plus the heads of the range), once three launches of 32 blocks (or the whole sequence, if it is shorter) make a wave
 // (measured against one launch and two: 80 heads, 4096-token segments, 7.03 -> 6.80 -> 6.72 ms a step); below that the time
-// of one CTA.  A function of the sequence alone, so the summation order of dB/dC does not depend on the
-// segment length.
+// of one CTA.  A function of the sequence alone, so the summation order of dB/dC does not depend on the segment length.
 static const int kBcBlocks = 96;
 static int bc_head_split(int blocks, int groups, int hpg) {
     int best = 1;
@@ -81,11 +81,13 @@ static int bc_head_split(int blocks, int groups, int hpg) {
         const int hps = (hpg + ns - 1) / ns;
         if ((hpg + hps - 1) / hps != ns) continue;      // would leave an empty range
         const double waves = (double)(blocks < kBcBlocks ? blocks : kBcBlocks) * groups * ns / kNumSMs;
-        const double t = (waves > 1 ? waves : 1) * (8 + hps);
+        // a short sequence is one launch or two, whose last wave takes as long as a full one
+        const double t = (blocks < kBcBlocks ? ceil(waves) : waves > 1 ? waves : 1) * (8 + hps);
         if (best_t < 0 || t < best_t) { best_t = t; best = ns; }
     }
     return best;
 }
+
 static int make_plan(const ssd_shape_t *s, Plan &pl) {
     if (!s) return SSD_EINVAL;
     if (s->B <= 0 || s->L <= 0 || s->H <= 0 || s->P <= 0 || s->N <= 0 || s->G <= 0 || s->chunk <= 0 ||
