@@ -56,8 +56,8 @@ struct Layout {
     size_t total;
 };
 
-// All the copies of the per-segment scratch (and with them the forward's state chain running ahead of y) pay only when there are
-// segments enough to pipeline; two or three long segments get a second copy of the forward chain's output and one of the rest.
+// All the copies of the per-segment scratch pay only when there are segments enough to pipeline; two or three long segments get
+// a second copy of the forward chain's output and one of the rest.
 static const int kMinSegmentsForTwins = 4;
 
 struct Plan {
@@ -353,20 +353,21 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     if (pl.use_tc && pl.nseg >= kMinSegmentsForTwins && may_use_helper_stream && !pl.serial && !g_prof_on) {
         // Algorithm 1 with the state chain one segment ahead: chunk states and state pass of segment k run on a
         // helper stream while the caller's stream still computes y of segment k-1, whose last, partly idle wave
-        // they fill.  What both touch (records, bf16 states) exists three times and goes round; the carried state belongs
+        // they fill.  What both touch (records, bf16 states) exists two or three times and goes round; the carried state belongs
         // to the chain alone.
         SideStreams *side = side_streams();
         if (!side) { g_last_cuda = (int)cudaGetLastError(); return SSD_ECUDA; }
+        const int ncp = chain_copies(pl.nseg);
         TcMaps mk[3] = {maps, maps, maps};
-        if (!state_maps(lo, ws, sp, mk, 3)) return SSD_ECUDA;
+        if (!state_maps(lo, ws, sp, mk, ncp)) return SSD_ECUDA;
         cudaStream_t chain = side->s[0];
         SSD_TRY(cudaEventRecord(side->start, st));
         SSD_TRY(cudaStreamWaitEvent(chain, side->start, 0));
         for (int k = 0; k < pl.nseg; ++k) {
-            const int par = k & 1, cp = k % 3;
+            const int par = k & 1, cp = k % ncp;
             set_segment(pl, k, sp);
             select_copy(lo, ws, cp, par, sp);
-            if (k >= 3) SSD_TRY(cudaStreamWaitEvent(chain, side->big_done[cp], 0));   // y of segment k-3 has read this copy
+            if (k >= ncp) SSD_TRY(cudaStreamWaitEvent(chain, side->big_done[cp], 0));   // y of segment k - ncp has read this copy
             {
                 cudaStream_t st = chain;
                 const float *init = (k == 0) ? h0 : sp.hcarry;
@@ -376,9 +377,9 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
                 SSD_TRY(cudaEventRecord(side->chain_done[par], st));
             }
             SSD_TRY(cudaStreamWaitEvent(st, side->chain_done[par], 0));
-            sp.scan_ctas = scan_ctas(sp, true, false);
+            sp.scan_ctas = scan_ctas(sp, k + 1 < pl.nseg, false);
             SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, mk[cp], SC_FWD, st));
-            if (k + 3 < pl.nseg) SSD_TRY(cudaEventRecord(side->big_done[cp], st));
+            if (k + ncp < pl.nseg) SSD_TRY(cudaEventRecord(side->big_done[cp], st));
         }
         return SSD_OK;
     }

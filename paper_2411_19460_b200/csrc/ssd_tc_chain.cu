@@ -293,7 +293,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 }
             }
             tc_fence_before_sync();
-            fence_proxy_async_smem();
+            fence_proxy_async_smem();      // the row has been read before a TMA load may overwrite it
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&dempty[bf]);
@@ -366,7 +366,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 }
             }
             tc_fence_before_sync();
-            fence_proxy_async_smem();
+            if (BWD) fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&dempty[bf]);
