@@ -50,8 +50,8 @@ static void prof_end(ProfEvent *ev, cudaStream_t st) {
 // backward's critical path is then the gradient chain alone; with two copies it waited for the large kernels two segments
 // back: 24 heads, 2048-token segments, 52 us a segment instead of 36), the rest twice.
 struct Layout {
-    size_t status, Hst, hcarry, Gst, gcarry, cbt, dAp, dDp, cs, dtT;
-    size_t rec[3], Hbf[3];
+    size_t status, hcarry, Gst, gcarry, dAp, dDp;
+    size_t rec[3], Hbf[3], cs[2], dtT[2], Hst[2], cbt[2];
     size_t Gbf[2], ghdot[2], ddt_dir[2], rho[2], rho2[2], psi[2], psi2[2], pB[2], pC[2];
     size_t total;
 };
@@ -157,10 +157,13 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
         take3(lo.rec, BH * pl.ncs * REC_FLOATS * sizeof(float), twins ? 3 : 1);
         take3(lo.Hbf, stb, twins ? chain_copies(pl.nseg) : 1);
     } else {
-        lo.cs = take(vec);
-        lo.dtT = take(vec);
-        lo.Hst = take(st);
-        lo.cbt = take((size_t)pl.B * pl.ncs * pl.G * pl.Q * pl.Q * sizeof(float));
+        // two copies where a launch works on two neighbouring segments: y beside the next segment's sums, and in the backward,
+        // where only the step sizes meet, the finishing steps beside them
+        const bool two = twins && pl.nseg > 1;
+        take2(lo.cs, vec, two && !bwd);
+        take2(lo.dtT, vec, two);
+        take2(lo.Hst, st, two && !bwd);
+        take2(lo.cbt, (size_t)pl.B * pl.ncs * pl.G * pl.Q * pl.Q * sizeof(float), two && !bwd);
     }
     if (bwd) {
         lo.gcarry = take(BH * PN * sizeof(float));
@@ -260,10 +263,12 @@ static void select_copy(const Layout &lo, void *ws, int kc, int k, SegParams &sp
     auto at = [&](size_t r) { return r ? (float *)(w + r) : nullptr; };
     auto f = [&](const size_t (&r)[2]) { return at(r[k]); };
     sp.rec = at(lo.rec[kc]);
-    sp.cs = at(lo.cs);
-    sp.dtT = sp.rec ? sp.rec + REC_DT : at(lo.dtT);
+    sp.cs = f(lo.cs);
+    sp.dtT = sp.rec ? sp.rec + REC_DT : f(lo.dtT);
     sp.dt_stride = sp.rec ? (int)REC_FLOATS : sp.Q;
     sp.Hbf = (__nv_bfloat16 *)at(lo.Hbf[kc]);
+    sp.Hst = f(lo.Hst);
+    sp.cbt = f(lo.cbt);
     sp.Gbf = (__nv_bfloat16 *)f(lo.Gbf);
     sp.ghdot = f(lo.ghdot);
     sp.ddt_dir = f(lo.ddt_dir);
@@ -285,8 +290,6 @@ static void fill_params(const Plan &pl, const Layout &lo, void *ws, SegParams &s
     sp.x_bs = pl.x_bs; sp.dt_bs = pl.dt_bs; sp.bc_bs = pl.bc_bs;
     char *w = (char *)ws;
     sp.status = (unsigned int *)(w + lo.status);
-    sp.Hst = (float *)(w + lo.Hst);
-    sp.cbt = (float *)(w + lo.cbt);
     sp.tiles = pl.use_tc ? 0 : pl.Q / 64;
     sp.hcarry = (float *)(w + lo.hcarry);
     sp.Gst = (float *)(w + lo.Gst);
@@ -383,6 +386,8 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         }
         return SSD_OK;
     }
+    const bool beside = may_use_helper_stream && !pl.serial;      // CUDA cores: the next segment's sums in the launch of y
+    SegParams next;
     for (int k = 0; k < pl.nseg; ++k) {
         set_segment(pl, k, sp);
         const float *init = (k == 0) ? h0 : sp.hcarry;
@@ -392,9 +397,16 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
             SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, maps, SC_FWD, st));
             continue;
         }
-        SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, pl.dtype, SIMT_SUMS, st));
+        select_copy(lo, ws, 0, k & 1, sp);
+        if (k == 0 || !beside) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, pl.dtype, SIMT_SUMS, st));
         SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN, fin, st));
-        SSD_LAUNCH(KIND_SCAN_FWD, launch_simt(sp, pl.dtype, SIMT_Y, st));
+        const bool ahead = beside && k + 1 < pl.nseg;
+        if (ahead) {
+            next = sp;
+            set_segment(pl, k + 1, next);
+            select_copy(lo, ws, 0, (k + 1) & 1, next);
+        }
+        SSD_LAUNCH(KIND_SCAN_FWD, launch_simt(sp, ahead ? &next : nullptr, pl.dtype, SIMT_Y, st));
     }
     return SSD_OK;
 }
@@ -625,11 +637,17 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
                     SSD_LAUNCH(KIND_BWD_DB, launch_grad_bc(sp, maps, BC_DB, st));
                 }
             } else {
-                SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, pl.dtype, SIMT_SUMS, st));
-                SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, hin, (long long)pl.nseg * pl.H * PN, nullptr, 0, nullptr, st));
-                SSD_LAUNCH(KIND_DSTATE, launch_simt(sp, pl.dtype, SIMT_DSTATE, st));
-                SSD_LAUNCH(KIND_STATE_PASS_BWD, launch_state_pass_bwd(sp, ginit, gleft, st));
-                SSD_LAUNCH(KIND_BWD_DX, launch_simt(sp, pl.dtype, SIMT_BWD, st));
+                select_copy(lo, ws, 0, k & 1, sp);
+                if (k == pl.nseg - 1 || pl.serial) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, pl.dtype, SIMT_SUMS_GRAD, st));
+                SSD_LAUNCH(KIND_STATE_PASS_BWD, launch_state_pass_bwd(sp, hin, (long long)pl.nseg * pl.H * PN, ginit, gleft, st));
+                SSD_LAUNCH(KIND_BWD_DX, launch_simt(sp, nullptr, pl.dtype, SIMT_BWD, st));
+                if (k > 0 && !pl.serial) {
+                    SegParams next = sp;
+                    set_segment(pl, k - 1, next);
+                    select_copy(lo, ws, 0, (k - 1) & 1, next);
+                    SSD_LAUNCH(KIND_BWD_FINISH, launch_simt(sp, &next, pl.dtype, SIMT_TAIL, st));
+                    continue;
+                }
             }
             SSD_LAUNCH(KIND_BWD_FINISH, launch_bwd_tail(sp, pl.dtype, st));
         }

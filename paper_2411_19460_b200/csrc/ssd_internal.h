@@ -120,13 +120,16 @@ static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; 
 
 // ---- kernel launchers (each returns the cudaError_t of its launch) ----
 // ssd_simt.cu : CUDA-core kernels, any I/O dtype
-enum { SIMT_SUMS = 0, SIMT_DSTATE, SIMT_Y, SIMT_BWD };   // chunk sums, cumsum and C B^T | state-gradient sums | y | dx, dB, dC slices
-cudaError_t launch_simt(const SegParams &p, int dtype, int what, cudaStream_t st);
+// SIMT_SUMS: chunk sums, cumsum and C B^T | SIMT_SUMS_GRAD: also the state-gradient sums | SIMT_Y: y, and the sums of segment
+// `next` if given | SIMT_BWD: dx, slices of dB and dC | SIMT_TAIL: finishing steps and the sums (with gradients) of segment `next`
+enum { SIMT_SUMS = 0, SIMT_SUMS_GRAD, SIMT_Y, SIMT_BWD, SIMT_TAIL };
+cudaError_t launch_simt(const SegParams &p, const SegParams *next, int dtype, int what, cudaStream_t st);
 // init: state entering the segment (NULL = zeros), batch stride init_bs elements;
 // boundary_out (nullable): where to store that state, batch stride bnd_bs; final_out nullable.
 cudaError_t launch_state_pass_fwd(const SegParams &p, const float *init, long long init_bs,
                                   float *boundary_out, long long bnd_bs, float *final_out, cudaStream_t st);
-cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, float *left_out, cudaStream_t st);
+// the backward's: entry states from init, then the gradients from ginit (NULL = zeros), handed left to gleft
+cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, long long init_bs, const float *ginit, float *gleft, cudaStream_t st);
 cudaError_t launch_bwd_tail(const SegParams &p, int dtype, cudaStream_t st);
 cudaError_t launch_final_dAdD(const SegParams &p, float *dA, float *dD, bool accumulate, cudaStream_t st);
 // ssd_glue.cu : layer-axis glue of a layer stack
@@ -178,7 +181,6 @@ enum { SC_FWD = 0, SC_DX = 1 };
 cudaError_t launch_grad_bc(const SegParams &p, const TcMaps &m, int what, cudaStream_t st);
 enum { BC_DC = 1, BC_DB = 2 };
 
-enum { STATE_MODE_FWD = 0, STATE_MODE_DSTATE = 1 };
 // kernel kinds, for the launch counter and the optional per-kind timing
 enum {
     KIND_CUMSUM = 0, KIND_CHUNK_STATE, KIND_STATE_PASS_FWD, KIND_SCAN_FWD, KIND_DSTATE,

@@ -7,19 +7,12 @@
 // All of it is Eq. 1 of the paper regrouped by chunks; the segment hand-off is Algorithms 1 and 2.
 #include "ssd_internal.h"
 
-// State-pass CTAs: 128 threads at 48 registers (6 K registers, almost no shared memory), small enough to fit on an SM
-// beside a CTA of the large tensor-core kernels, which leave about 6.5 K registers free.  The backward pass gained 4 %
-// from the smaller CTAs by itself; the step time did not change measurably, so whatever of these passes can hide
-// under the large kernels was hidden already.
+// State-pass CTAs: 128 threads, at most 48 registers, so that a segment's CTAs are resident at once; chunks fetched ahead.
 #define SP_THREADS 128
 #define SP_ELEMS (SP_THREADS * 4)
+#define SP_CTAS 10
+#define SP_PF 4
 static_assert(SP_ELEMS == ssd::kStatePassElems, "one partial of <G,H> per CTA of the backward pass");
-#ifndef SP_BWD_CTAS
-#define SP_BWD_CTAS 10
-#define SP_BWD_PF 4
-#define SP_FWD_CTAS 10
-#define SP_FWD_PF 4
-#endif
 namespace ssd {
 
 // ------------------------------------------------------------------ small helpers
@@ -53,88 +46,70 @@ __device__ __forceinline__ size_t vec_off(const SegParams &p, int b, int h, int 
     return (((size_t)b * p.H + h) * p.ncs + c) * (size_t)p.Q;
 }
 
-// ------------------------------------------------------------------ forward state passing, boundary store / reload
-// H_{c+1} = exp(cs_last,c) H_c + S_c, strictly sequential in c for every (b,h,p,n) element, so the
-// bits do not depend on how the sequence is cut into segments.  Each thread owns one float4.
-// Also stores the segment-entry state into `boundary` (the sequence-axis checkpoint) and hands the
-// segment-exit state to the next segment through hcarry.
-__global__ void __launch_bounds__(SP_THREADS, SP_FWD_CTAS)
-k_state_pass_fwd(SegParams p, const float *init, long long init_bs, float *boundary_out,
-                 long long bnd_bs, float *final_out) {
+// ------------------------------------------------------------------ state passing, boundary store / reload
+// Forward: H_{c+1} = exp(cs_last,c) H_c + S_c, strictly sequential in c for every (b,h,p,n) element, so the bits do not depend
+// on how the sequence is cut into segments.  Each thread owns one float4.  In the forward call (BWD = false) it also stores the
+// segment-entry state into `boundary` (the sequence-axis checkpoint) and hands the segment-exit state on through hcarry.
+//
+// Backward call (BWD = true): the entry states first, as above, then by the same threads (an element's pass back needs
+// no other element's states: one launch instead of two) Gslot[nc] = gradient arriving from the right (or dh_final) and,
+// going left, Gslot[c] = exp(cs_last,c) Gslot[c+1] + E_c.  Gslot[c+1] is Gout of chunk c.  Also emits, per chunk, the partial
+// sums of exp(cs_last,c) <Gout_c, H_in,c> (one per CTA, summed later in a fixed order): the part of da_t that couples the
+// gradient from the right with the state from the left.
+//
+// Bound by the latency of its loads: the sums and decays do not depend on the carry, so four chunks are fetched ahead of the
+// serial recurrence.
+template <bool BWD>
+__global__ void __launch_bounds__(SP_THREADS, SP_CTAS)
+k_state_pass(SegParams p, const float *init, long long init_bs, float *boundary_out, long long bnd_bs, float *final_out, const float *ginit,
+             float *gleft) {
     pdl_launch_dependents();
     pdl_wait();
-    const int h = blockIdx.y, b = blockIdx.z;
-    const int PN = p.P * p.N;
-    const int e = blockIdx.x * SP_ELEMS + threadIdx.x * 4;
-    const size_t bh = ((size_t)b * p.H + h) * PN + e;
-    float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (init) carry = *reinterpret_cast<const float4 *>(init + (size_t)b * init_bs + (size_t)h * PN + e);
-    if (boundary_out)
-        *reinterpret_cast<float4 *>(boundary_out + (size_t)b * bnd_bs + (size_t)h * PN + e) = carry;
-    const float *csl = p.cs + vec_off(p, b, h, 0) + (p.Q - 1);
-    auto put = [&](size_t so, const float4 &v) { *reinterpret_cast<float4 *>(p.Hst + so) = v; };
-    put(slot_off(p, b, 0, h) + e, carry);
-    // The chunk sums and decays do not depend on the carry: fetch eight chunks ahead of the serial
-    // recurrence, so that a segment costs a few memory latencies instead of one per chunk.
-    constexpr int PF = SP_FWD_PF;
-    for (int c0 = 1; c0 <= p.nc; c0 += PF) {
-        float4 sv[PF];
-        float dec[PF];
-#pragma unroll
-        for (int k = 0; k < PF; ++k)
-            if (c0 + k <= p.nc) {
-                sv[k] = *reinterpret_cast<const float4 *>(p.Hst + slot_off(p, b, c0 + k, h) + e);
-                dec[k] = csl[(size_t)(c0 + k - 1) * p.Q];
-            }
-#pragma unroll
-        for (int k = 0; k < PF; ++k)
-            if (c0 + k <= p.nc) {
-                const float decay = expf(dec[k]);
-                carry.x = fmaf(decay, carry.x, sv[k].x);
-                carry.y = fmaf(decay, carry.y, sv[k].y);
-                carry.z = fmaf(decay, carry.z, sv[k].z);
-                carry.w = fmaf(decay, carry.w, sv[k].w);
-                put(slot_off(p, b, c0 + k, h) + e, carry);
-            }
-    }
-    *reinterpret_cast<float4 *>(p.hcarry + bh) = carry;
-    if (final_out) *reinterpret_cast<float4 *>(final_out + bh) = carry;
-}
-
-cudaError_t launch_state_pass_fwd(const SegParams &p, const float *init, long long init_bs,
-                                  float *boundary_out, long long bnd_bs, float *final_out, cudaStream_t st) {
-    dim3 grid(p.P * p.N / SP_ELEMS, p.H, p.B);
-    return launch_pdl(k_state_pass_fwd, grid, dim3(SP_THREADS), 0, st, p, init, init_bs, boundary_out, bnd_bs, final_out);
-}
-
-// ------------------------------------------------------------------ backward state passing
-// Gslot[nc] = gradient arriving from the segment on the right (or dh_final); going left,
-// Gslot[c] = exp(cs_last,c) Gslot[c+1] + E_c.  Gslot[c+1] is Gout of chunk c.  Also emits, per chunk,
-// the partial sums of exp(cs_last,c) <Gout_c, H_in,c> (one per CTA, summed later in a fixed order):
-// the part of da_t that couples the gradient from the right with the state from the left.
-__global__ void __launch_bounds__(SP_THREADS, SP_BWD_CTAS)
-k_state_pass_bwd(SegParams p, const float *init, float *left_out) {
-    pdl_launch_dependents();
-    pdl_wait();
-    __shared__ float red[SP_BWD_PF][SP_THREADS / 32];
+    __shared__ float red[SP_PF][SP_THREADS / 32];
     const int h = blockIdx.y, b = blockIdx.z;
     const int PN = p.P * p.N;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int e = blockIdx.x * SP_ELEMS + tid * 4;
     const size_t bh = ((size_t)b * p.H + h) * PN + e;
     float4 carry = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (init) carry = *reinterpret_cast<const float4 *>(init + bh);
+    if (init) carry = *reinterpret_cast<const float4 *>(init + (size_t)b * init_bs + (size_t)h * PN + e);
+    if (!BWD && boundary_out)
+        *reinterpret_cast<float4 *>(boundary_out + (size_t)b * bnd_bs + (size_t)h * PN + e) = carry;
     const float *csl = p.cs + vec_off(p, b, h, 0) + (p.Q - 1);
-    auto put = [&](size_t so, const float4 &v) { *reinterpret_cast<float4 *>(p.Gst + so) = v; };
-    put(slot_off(p, b, p.nc, h) + e, carry);
-    // Eight chunks at a time: their E_c, entry states and decays are fetched ahead of the serial
-    // recurrence; the eight <Gout, H_in> partials of a batch share one block-wide reduction step.
-    constexpr int PF = SP_BWD_PF;
-    for (int c0 = p.nc - 1; c0 >= 0; c0 -= PF) {
-        float4 ev[PF], hv[PF];
-        float dec[PF];
+    *reinterpret_cast<float4 *>(p.Hst + slot_off(p, b, 0, h) + e) = carry;
+    for (int c0 = 1; c0 <= p.nc; c0 += SP_PF) {
+        float4 sv[SP_PF];
+        float dec[SP_PF];
 #pragma unroll
-        for (int k = 0; k < PF; ++k)
+        for (int k = 0; k < SP_PF; ++k)
+            if (c0 + k <= p.nc) {
+                sv[k] = *reinterpret_cast<const float4 *>(p.Hst + slot_off(p, b, c0 + k, h) + e);
+                dec[k] = csl[(size_t)(c0 + k - 1) * p.Q];
+            }
+#pragma unroll
+        for (int k = 0; k < SP_PF; ++k)
+            if (c0 + k <= p.nc) {
+                const float decay = expf(dec[k]);
+                carry.x = fmaf(decay, carry.x, sv[k].x);
+                carry.y = fmaf(decay, carry.y, sv[k].y);
+                carry.z = fmaf(decay, carry.z, sv[k].z);
+                carry.w = fmaf(decay, carry.w, sv[k].w);
+                *reinterpret_cast<float4 *>(p.Hst + slot_off(p, b, c0 + k, h) + e) = carry;
+            }
+    }
+    if (!BWD) {
+        *reinterpret_cast<float4 *>(p.hcarry + bh) = carry;
+        if (final_out) *reinterpret_cast<float4 *>(final_out + bh) = carry;
+        return;
+    }
+    carry = ginit ? *reinterpret_cast<const float4 *>(ginit + bh) : make_float4(0.f, 0.f, 0.f, 0.f);
+    *reinterpret_cast<float4 *>(p.Gst + slot_off(p, b, p.nc, h) + e) = carry;
+    // the <Gout, H_in> partials of a batch share one block-wide reduction step
+    for (int c0 = p.nc - 1; c0 >= 0; c0 -= SP_PF) {
+        float4 ev[SP_PF], hv[SP_PF];
+        float dec[SP_PF];
+#pragma unroll
+        for (int k = 0; k < SP_PF; ++k)
             if (c0 - k >= 0) {
                 const size_t so = slot_off(p, b, c0 - k, h) + e;
                 ev[k] = *reinterpret_cast<const float4 *>(p.Gst + so);
@@ -142,7 +117,7 @@ k_state_pass_bwd(SegParams p, const float *init, float *left_out) {
                 dec[k] = csl[(size_t)(c0 - k) * p.Q];
             }
 #pragma unroll
-        for (int k = 0; k < PF; ++k)
+        for (int k = 0; k < SP_PF; ++k)
             if (c0 - k >= 0) {
                 // carry is Gout of chunk c = c0 - k here; hv[k] is the state entering chunk c
                 const float decay = expf(dec[k]);
@@ -157,10 +132,10 @@ k_state_pass_bwd(SegParams p, const float *init, float *left_out) {
                 carry.y = fmaf(decay, carry.y, ev[k].y);
                 carry.z = fmaf(decay, carry.z, ev[k].z);
                 carry.w = fmaf(decay, carry.w, ev[k].w);
-                put(slot_off(p, b, c0 - k, h) + e, carry);
+                *reinterpret_cast<float4 *>(p.Gst + slot_off(p, b, c0 - k, h) + e) = carry;
             }
         __syncthreads();
-        if (tid < PF && c0 - tid >= 0) {
+        if (tid < SP_PF && c0 - tid >= 0) {
             float s = 0.f;
 #pragma unroll
             for (int w = 0; w < SP_THREADS / 32; ++w) s += red[tid][w];
@@ -168,12 +143,17 @@ k_state_pass_bwd(SegParams p, const float *init, float *left_out) {
         }
         __syncthreads();
     }
-    *reinterpret_cast<float4 *>(left_out + bh) = carry;
+    *reinterpret_cast<float4 *>(gleft + bh) = carry;
 }
 
-cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, float *left_out, cudaStream_t st) {
+cudaError_t launch_state_pass_fwd(const SegParams &p, const float *init, long long init_bs,
+                                  float *boundary_out, long long bnd_bs, float *final_out, cudaStream_t st) {
     dim3 grid(p.P * p.N / SP_ELEMS, p.H, p.B);
-    return launch_pdl(k_state_pass_bwd, grid, dim3(SP_THREADS), 0, st, p, init, left_out);
+    return launch_pdl(k_state_pass<false>, grid, dim3(SP_THREADS), 0, st, p, init, init_bs, boundary_out, bnd_bs, final_out, nullptr, nullptr);
+}
+cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, long long init_bs, const float *ginit, float *gleft, cudaStream_t st) {
+    dim3 grid(p.P * p.N / SP_ELEMS, p.H, p.B);
+    return launch_pdl(k_state_pass<true>, grid, dim3(SP_THREADS), 0, st, p, init, init_bs, nullptr, 0, nullptr, ginit, gleft);
 }
 
 // ------------------------------------------------------------------ FFMA contractions
@@ -267,23 +247,25 @@ __device__ __forceinline__ float *cb_of(const SegParams &p, int b, int c, int g)
     return p.cbt + (((size_t)b * p.ncs + c) * p.G + g) * (size_t)(p.Q * p.Q);
 }
 
-// mode FWD   : S_c[p,n] = sum_s exp(cs_last - cs_s) dt_s x_s[p] B_s[n]     -> Hst slot c+1   (and cs, dtT, C B^T)
-// mode DSTATE: E_c[p,n] = sum_t exp(cs_t) dy_t[p] C_t[n]                   -> Gst slot c
-template <typename T, int NS, int MODE>
-__global__ void __launch_bounds__(256) k_simt_sums(SegParams p) {
-    pdl_launch_dependents();
-    pdl_wait();
-    __shared__ SimtTiles sm;
-    __shared__ float wsm[256], tot[8];
+// What a segment's chunks need before the states can be passed on, by block number:
+//   S_c[p,n] = sum_s exp(cs_last - cs_s) dt_s x_s[p] B_s[n]     -> Hst slot c+1   (and cs, dtT)
+//   with grads: E_c[p,n] = sum_t exp(cs_t) dy_t[p] C_t[n]       -> Gst slot c      (its CTAs make the cumsum again)
+//   the causal tiles of C B^T
+template <typename T, int NS> __host__ __device__ __forceinline__ int simt_n_sums(const SegParams &p, bool grads) {
+    const int nrt = p.Q >> 6;
+    return p.nc * p.B * ((NS / 64) * p.H * (grads ? 2 : 1) + p.G * (nrt * (nrt + 1) / 2));
+}
+template <typename T, int NS> __device__ __forceinline__ void simt_sums(const SegParams &p, SimtTiles &sm, float *wsm, float *tot, int id, bool grads) {
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, nh = NS / 64;
     const size_t HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
-    int id = blockIdx.x;
     const int nsum = p.nc * nh * p.H * p.B;
     float2 acc[4][2];
     float4 ra[4], rb[4];
     zero_acc(acc);
-    if (MODE == STATE_MODE_FWD && id >= nsum) {      // a causal tile of C B^T
-        id -= nsum;
+    const bool dst = grads && id >= nsum && id < 2 * nsum;
+    if (dst) id -= nsum;
+    else if (id >= nsum) {      // a causal tile of C B^T
+        id -= grads ? 2 * nsum : nsum;
         const int npair = nrt * (nrt + 1) / 2;
         int rt, ct;
         pair_of(id % npair, rt, ct);
@@ -310,40 +292,36 @@ __global__ void __launch_bounds__(256) k_simt_sums(SegParams p) {
     id /= nh;
     const int h = id % p.H, c = (id / p.H) % p.nc, b = id / (p.H * p.nc), g = h / p.hpg;
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q;
-    const T *rows = (const T *)(MODE == STATE_MODE_FWD ? p.x : p.dy) + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
-    const T *cols = (const T *)(MODE == STATE_MODE_FWD ? p.Bm : p.Cm) + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS + n0;
+    const T *rows = (const T *)(dst ? p.dy : p.x) + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
+    const T *cols = (const T *)(dst ? p.Cm : p.Bm) + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS + n0;
     tile_load(ra, rows, HP, false);
     tile_load(rb, cols, GN, false);
-    if (MODE == STATE_MODE_FWD) {
-        // the chunk cumsum: a thread per step, shuffle scans of 32 and the warps' totals
-        const int lane = tid & 31, warp = tid >> 5;
-        float d = 0.f, v = 0.f;
-        if (tid < Q) {
-            d = __ldg(p.dt + (size_t)b * p.dt_bs + (tok0 + tid) * p.H + h);
-            v = d * __ldg(p.A + h);
-        }
+    // the chunk cumsum: a thread per step, shuffle scans of 32 and the warps' totals
+    const int lane = tid & 31, warp = tid >> 5;
+    float d = 0.f, v = 0.f;
+    if (tid < Q) {
+        d = __ldg(p.dt + (size_t)b * p.dt_bs + (tok0 + tid) * p.H + h);
+        v = d * __ldg(p.A + h);
+    }
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-            const float t = __shfl_up_sync(0xffffffffu, v, off);
-            if (lane >= off) v += t;
+    for (int off = 1; off < 32; off <<= 1) {
+        const float t = __shfl_up_sync(0xffffffffu, v, off);
+        if (lane >= off) v += t;
+    }
+    if (lane == 31) tot[warp] = v;
+    __syncthreads();
+    float before = 0.f, last = 0.f;
+    for (int w = 0; w < Q / 32; ++w) {
+        if (w < warp) before += tot[w];
+        last += tot[w];
+    }
+    v += before;
+    if (tid < Q) {
+        wsm[tid] = dst ? expf(v) : expf(fminf(last - v, 0.f)) * d;
+        if (n0 == 0 && !dst) {
+            p.cs[vec_off(p, b, h, c) + tid] = v;
+            p.dtT[vec_off(p, b, h, c) + tid] = d;
         }
-        if (lane == 31) tot[warp] = v;
-        __syncthreads();
-        float before = 0.f, last = 0.f;
-        for (int w = 0; w < Q / 32; ++w) {
-            if (w < warp) before += tot[w];
-            last += tot[w];
-        }
-        v += before;
-        if (tid < Q) {
-            wsm[tid] = expf(fminf(last - v, 0.f)) * d;
-            if (n0 == 0) {
-                p.cs[vec_off(p, b, h, c) + tid] = v;
-                p.dtT[vec_off(p, b, h, c) + tid] = d;
-            }
-        }
-    } else if (tid < Q) {
-        wsm[tid] = expf(p.cs[vec_off(p, b, h, c) + tid]);
     }
     __syncthreads();
     for (int s0 = 0; s0 < Q; s0 += 64) {
@@ -362,10 +340,18 @@ __global__ void __launch_bounds__(256) k_simt_sums(SegParams p) {
         tile_mma(acc, sm.a, sm.b);
         __syncthreads();
     }
-    float *out = (MODE == STATE_MODE_FWD ? p.Hst + slot_off(p, b, c + 1, h) : p.Gst + slot_off(p, b, c, h)) + (size_t)(ty * 4) * NS + n0 + tx * 4;
+    float *out = (dst ? p.Gst + slot_off(p, b, c, h) : p.Hst + slot_off(p, b, c + 1, h)) + (size_t)(ty * 4) * NS + n0 + tx * 4;
 #pragma unroll
     for (int i = 0; i < 4; ++i)
         *reinterpret_cast<float4 *>(out + (size_t)i * NS) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+}
+
+template <typename T, int NS> __global__ void __launch_bounds__(256) k_simt_sums(SegParams p, bool grads) {
+    pdl_launch_dependents();
+    pdl_wait();
+    __shared__ SimtTiles sm;
+    __shared__ float wsm[256], tot[8];
+    simt_sums<T, NS>(p, sm, wsm, tot, blockIdx.x, grads);
 }
 
 // One 64-row tile of y (DX = false) or of dx (DX = true) of one head:
@@ -477,14 +463,22 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
     }
 }
 
+// y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
+// wait for nothing of this one, and a launch of a few microseconds is saved per segment.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256) k_simt_y(SegParams p) {
+__global__ void __launch_bounds__(256) k_simt_y(SegParams p, SegParams nx, int n_next) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
     __shared__ float css[256], dts[256];
-    const int nrt = p.Q >> 6;
-    simt_row_tile<T, NS, false>(p, sm, css, dts, nullptr, blockIdx.x / nrt, blockIdx.x % nrt, blockIdx.y, blockIdx.z);
+    const int nrt = p.Q >> 6, ny = (int)gridDim.x - n_next;
+    int id = blockIdx.x;
+    if (id >= ny) {
+        simt_sums<T, NS>(nx, sm, css, dts, id - ny, false);
+        return;
+    }
+    const int rt = id % nrt, c = (id / nrt) % p.nc, h = (id / (nrt * p.nc)) % p.H, b = id / (nrt * p.nc * p.H);
+    simt_row_tile<T, NS, false>(p, sm, css, dts, nullptr, c, rt, h, b);
 }
 
 // The large kernel of the backward: tiles of dx, and the partial slices of dB and dC.  Per (chunk, head range):
@@ -668,24 +662,6 @@ __global__ void __launch_bounds__(256) k_simt_bwd(SegParams p, int n_dx) {
     for (int m = 0; m < NS / 64; ++m) write_slice(isC ? p.pC : p.pB, tot[m], rt * 64, nrt, m * 64);
 }
 
-template <typename T, int NS>
-static cudaError_t simt_launch(const SegParams &p, int what, cudaStream_t st) {
-    const int nrt = p.Q / 64, npair = nrt * (nrt + 1) / 2, nsum = p.nc * (NS / 64) * p.H * p.B;
-    switch (what) {
-        case SIMT_SUMS: return launch_pdl(k_simt_sums<T, NS, STATE_MODE_FWD>, dim3(nsum + p.nc * npair * p.G * p.B), dim3(256), 0, st, p);
-        case SIMT_DSTATE: return launch_pdl(k_simt_sums<T, NS, STATE_MODE_DSTATE>, dim3(nsum), dim3(256), 0, st, p);
-        case SIMT_Y: return launch_pdl(k_simt_y<T, NS>, dim3(p.nc * nrt, p.H, p.B), dim3(256), 0, st, p);
-        default: {
-            const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 1)) * p.G * p.B;
-            return launch_pdl(k_simt_bwd<T, NS>, dim3(n_bc + n_dx), dim3(256), 0, st, p, n_dx);
-        }
-    }
-}
-cudaError_t launch_simt(const SegParams &p, int dtype, int what, cudaStream_t st) {
-    if (dtype == SSD_DTYPE_F32) return p.N == 64 ? simt_launch<float, 64>(p, what, st) : simt_launch<float, 128>(p, what, st);
-    return p.N == 64 ? simt_launch<__nv_bfloat16, 64>(p, what, st) : simt_launch<__nv_bfloat16, 128>(p, what, st);
-}
-
 // ------------------------------------------------------------------ da, ddt, dA partial
 // One warp per (b, h, chunk).  With g_t = dLoss/dh_t and h_{t-1} split into their intra-chunk and
 // inter-chunk parts, da_t = exp(a_t) <g_t, h_{t-1}> is the sum of four terms, none of which
@@ -700,8 +676,8 @@ cudaError_t launch_simt(const SegParams &p, int dtype, int what, cudaStream_t st
 // steps lie H floats apart, so the eight heads' results go through a shared-memory tile and leave as rows of eight
 // consecutive floats (whole 32-byte sectors) instead of one 4-byte store per sector.
 constexpr int FIN_HB = 8;
-__device__ __forceinline__ void bwd_finish(const SegParams &p, int id) {
-    __shared__ float tile[256 * (FIN_HB + 1)];
+constexpr int FIN_TILE = 256 * (FIN_HB + 1);
+__device__ __forceinline__ void bwd_finish(const SegParams &p, float *tile, int id) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nhb = (p.H + FIN_HB - 1) / FIN_HB;
     const int c = id % p.nc, hb = (id / p.nc) % nhb, b = id / (p.nc * nhb), h = hb * FIN_HB + warp, nh = min(FIN_HB, p.H - hb * FIN_HB);
@@ -822,16 +798,60 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_bwd_tail(SegParams p, int nfin) {
     pdl_launch_dependents();
     pdl_wait();
-    if ((int)blockIdx.x < nfin) bwd_finish(p, blockIdx.x);
+    __shared__ float tile[FIN_TILE];
+    if ((int)blockIdx.x < nfin) bwd_finish(p, tile, blockIdx.x);
     else reduce_dbdc<T>(p, blockIdx.x - nfin);
 }
+// CUDA-core path: the same with the sums of the next segment (to the left) in front, which share no scratch with it but the step
+// sizes, of which there are two copies.
+template <typename T, int NS>
+__global__ void __launch_bounds__(256) k_simt_tail(SegParams p, SegParams nx, int n_next, int nfin) {
+    pdl_launch_dependents();
+    pdl_wait();
+    __shared__ SimtTiles sm;
+    __shared__ float wsm[256], tot[8];
+    static_assert(sizeof(SimtTiles) >= FIN_TILE * sizeof(float), "the finishing step's tile");
+    const int id = (int)blockIdx.x - n_next;
+    if (id < 0) simt_sums<T, NS>(nx, sm, wsm, tot, blockIdx.x, true);
+    else if (id < nfin) bwd_finish(p, &sm.a[0][0], id);
+    else reduce_dbdc<T>(p, id - nfin);
+}
 
+static int tail_finish_ctas(const SegParams &p) { return p.nc * ((p.H + FIN_HB - 1) / FIN_HB) * p.B; }
+static int tail_reduce_ctas(const SegParams &p) { return (int)(((size_t)p.B * p.nc * p.Q * p.G * (p.N / 4) + 255) / 256); }
 cudaError_t launch_bwd_tail(const SegParams &p, int dtype, cudaStream_t st) {
-    const int nfin = p.nc * ((p.H + FIN_HB - 1) / FIN_HB) * p.B;
-    const size_t total = (size_t)p.B * p.nc * p.Q * p.G * (p.N / 4);
-    const dim3 grid((unsigned)(nfin + (total + 255) / 256));
+    const int nfin = tail_finish_ctas(p);
+    const dim3 grid(nfin + tail_reduce_ctas(p));
     if (dtype == SSD_DTYPE_F32) return launch_pdl(k_bwd_tail<float>, grid, dim3(256), 0, st, p, nfin);
     return launch_pdl(k_bwd_tail<__nv_bfloat16>, grid, dim3(256), 0, st, p, nfin);
+}
+
+template <typename T, int NS>
+static cudaError_t simt_launch(const SegParams &p, const SegParams *next, int what, cudaStream_t st) {
+    const int nrt = p.Q / 64, npair = nrt * (nrt + 1) / 2;
+    switch (what) {
+        case SIMT_SUMS:
+        case SIMT_SUMS_GRAD: {
+            const bool grads = what == SIMT_SUMS_GRAD;
+            return launch_pdl(k_simt_sums<T, NS>, dim3(simt_n_sums<T, NS>(p, grads)), dim3(256), 0, st, p, grads);
+        }
+        case SIMT_Y: {
+            const int n_next = next ? simt_n_sums<T, NS>(*next, false) : 0;
+            return launch_pdl(k_simt_y<T, NS>, dim3(p.nc * nrt * p.H * p.B + n_next), dim3(256), 0, st, p, next ? *next : p, n_next);
+        }
+        case SIMT_TAIL: {
+            const int nfin = tail_finish_ctas(p), n_next = simt_n_sums<T, NS>(*next, true);
+            return launch_pdl(k_simt_tail<T, NS>, dim3(n_next + nfin + tail_reduce_ctas(p)), dim3(256), 0, st, p, *next, n_next, nfin);
+        }
+        default: {
+            const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 1)) * p.G * p.B;
+            return launch_pdl(k_simt_bwd<T, NS>, dim3(n_bc + n_dx), dim3(256), 0, st, p, n_dx);
+        }
+    }
+}
+cudaError_t launch_simt(const SegParams &p, const SegParams *next, int dtype, int what, cudaStream_t st) {
+    if (dtype == SSD_DTYPE_F32) return p.N == 64 ? simt_launch<float, 64>(p, next, what, st) : simt_launch<float, 128>(p, next, what, st);
+    return p.N == 64 ? simt_launch<__nv_bfloat16, 64>(p, next, what, st) : simt_launch<__nv_bfloat16, 128>(p, next, what, st);
 }
 
 // ------------------------------------------------------------------ dA, dD over (batch, chunks)
