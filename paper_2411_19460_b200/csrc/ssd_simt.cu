@@ -346,7 +346,7 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
         *reinterpret_cast<float4 *>(out + (size_t)i * NS) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
 }
 
-template <typename T, int NS> __global__ void __launch_bounds__(256) k_simt_sums(SegParams p, bool grads) {
+template <typename T, int NS> __global__ void __launch_bounds__(256, 3) k_simt_sums(SegParams p, bool grads) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
@@ -466,7 +466,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
 // y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
 // wait for nothing of this one, and a launch of a few microseconds is saved per segment.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256) k_simt_y(SegParams p, SegParams nx, int n_next) {
+__global__ void __launch_bounds__(256, 3) k_simt_y(SegParams p, SegParams nx, int n_next) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
@@ -487,7 +487,7 @@ __global__ void __launch_bounds__(256) k_simt_y(SegParams p, SegParams nx, int n
 //   inter dC, tile tt : sum_h e^{cs_t} dy_t H_in (and rho2 per head);  inter dB, tile ts : sum_h dt_s e^{cs_last-cs_s} x_s Gout
 // A slice has Q/64 + 1 slots per head range: dC by ts (dB by tt), the last one the inter-chunk term.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256) k_simt_bwd(SegParams p, int n_dx) {
+__global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
@@ -805,7 +805,7 @@ __global__ void __launch_bounds__(256) k_bwd_tail(SegParams p, int nfin) {
 // CUDA-core path: the same with the sums of the next segment (to the left) in front, which share no scratch with it but the step
 // sizes, of which there are two copies.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256) k_simt_tail(SegParams p, SegParams nx, int n_next, int nfin) {
+__global__ void __launch_bounds__(256, 3) k_simt_tail(SegParams p, SegParams nx, int n_next, int nfin) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
