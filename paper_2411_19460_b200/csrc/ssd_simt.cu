@@ -359,7 +359,7 @@ template <typename T, int NS> __global__ void __launch_bounds__(256, 3) k_simt_s
 //   u_s  = sum_{t>=s} CB[t,s] e^{cs_t-cs_s} dy_t     + e^{cs_last-cs_s} B_s Gout ;  dx_s = D dy_s + dt_s u_s ,
 //   ddt_direct_s = x_s . u_s , psi2_s = dt_s e^{cs_last-cs_s} x_s . (Gout B_s) , dD partial = sum dy.x
 template <typename T, int NS, bool DX>
-__device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm, float *css, float *dts, float *red, int c, int rt, int h, int b) {
+__device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm, float *css, float *dts, float *fac, float *red, int c, int rt, int h, int b) {
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, g = h / p.hpg, r0 = rt * 64;
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q, HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
     const size_t xo = (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
@@ -395,6 +395,16 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
         tile_mma(acc, sm.a, sm.b);
         __syncthreads();
     }
+    // Off the diagonal tile the mask factors at the tile's edge m (its first row; dx: last), where both factors are <= 1:
+    // e^{cs_t-cs_s} = e^{cs_t-cs_m} e^{cs_m-cs_s}.  An exponential per step instead of one per element.
+    const int m = DX ? r0 + 63 : r0;
+    if (nrt > 1) {
+        for (int t = tid; t < Q; t += 256) {
+            const float d = css[t] - css[m];
+            fac[t] = expf(fminf(t >= m ? d : -d, 0.f)) * (DX || t >= m ? 1.f : dts[t]);
+        }
+        __syncthreads();
+    }
     // the inter-chunk term is complete: scale its rows
     const float cl = css[Q - 1];
     float dd2[4];
@@ -410,6 +420,14 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
     }
     for (int ct = ct0; ct < ct1; ++ct) {
         // masked tile: a[k = column of the mask][row]
+        if (ct != rt) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const float one = fac[DX ? ct * 64 + ty + 16 * k : r0 + (tid & 7) + 8 * (tid >> 5)];
+                const float4 four = *reinterpret_cast<const float4 *>(fac + (DX ? r0 + tx * 4 : ct * 64 + ((tid >> 3) & 3) * 4 + 16 * k));
+                ra[k].x *= one * four.x; ra[k].y *= one * four.y; ra[k].z *= one * four.z; ra[k].w *= one * four.w;
+            }
+        } else
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             float *e = reinterpret_cast<float *>(&ra[k]);
@@ -464,13 +482,14 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
 }
 
 // y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
-// wait for nothing of this one, and a launch of a few microseconds is saved per segment.
+// wait for nothing of this one, and a launch of a few microseconds is saved per segment.  N = 64 is left at two CTAs per SM: three
+// would spill, and its layers are small.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256, 3) k_simt_y(SegParams p, SegParams nx, int n_next) {
+__global__ void __launch_bounds__(256, NS == 64 ? 2 : 3) k_simt_y(SegParams p, SegParams nx, int n_next) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
-    __shared__ float css[256], dts[256];
+    __shared__ __align__(16) float css[256], dts[256], fac[256];
     const int nrt = p.Q >> 6, ny = (int)gridDim.x - n_next;
     int id = blockIdx.x;
     if (id >= ny) {
@@ -478,7 +497,7 @@ __global__ void __launch_bounds__(256, 3) k_simt_y(SegParams p, SegParams nx, in
         return;
     }
     const int rt = id % nrt, c = (id / nrt) % p.nc, h = (id / (nrt * p.nc)) % p.H, b = id / (nrt * p.nc * p.H);
-    simt_row_tile<T, NS, false>(p, sm, css, dts, nullptr, c, rt, h, b);
+    simt_row_tile<T, NS, false>(p, sm, css, dts, fac, nullptr, c, rt, h, b);
 }
 
 // The large kernel of the backward: tiles of dx, and the partial slices of dB and dC.  Per (chunk, head range):
@@ -491,13 +510,13 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
-    __shared__ float css[256], dts[256], red[8][64];
+    __shared__ __align__(16) float css[256], dts[256], fac[256], red[8][64];
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, npair = nrt * (nrt + 1) / 2;
     int id = blockIdx.x;
     if (id >= (int)gridDim.x - n_dx) {
         id -= (int)gridDim.x - n_dx;
         const int rt = id % nrt, h = (id / nrt) % p.H, c = (id / (nrt * p.H)) % p.nc, b = id / (nrt * p.H * p.nc);
-        simt_row_tile<T, NS, true>(p, sm, css, dts, red[0], c, rt, h, b);
+        simt_row_tile<T, NS, true>(p, sm, css, dts, fac, red[0], c, rt, h, b);
         return;
     }
     const int per = npair + 2 * nrt, role = id % per;
@@ -540,6 +559,11 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
         tile_load(rb, xb + (size_t)ts * 64 * HP + (size_t)h0 * 64, HP, true);
         for (int h = h0; h < h1; ++h) {
             load_vec(h);
+            if (tt != ts && tid < 128) {      // the mask's factors at the row tile's first step, as for y
+                const float *cs = p.cs + vec_off(p, b, h, c), ref = cs[tt * 64];
+                const int t = (tid < 64 ? tt : ts - 1) * 64 + tid;
+                fac[tid] = tid < 64 ? expf(fminf(cs[t] - ref, 0.f)) : expf(fminf(ref - cs[t], 0.f)) * p.dtT[vec_off(p, b, h, c) + t];
+            }
             tile_store(sm.a, ra, true);
             tile_store(sm.b, rb, true);
             __syncthreads();
@@ -555,11 +579,21 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
             for (int i = 0; i < 4; ++i) {
                 const int t = tt * 64 + ty * 4 + i;
                 const float s4[4] = {acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y}, c4[4] = {cb[i].x, cb[i].y, cb[i].z, cb[i].w};
-                float row = 0.f;
+                float row = 0.f, e4[4];
+                if (tt != ts) {
+                    const float one = fac[ty * 4 + i];
+                    const float4 four = *reinterpret_cast<const float4 *>(fac + 64 + tx * 4);
+                    e4[0] = one * four.x; e4[1] = one * four.y; e4[2] = one * four.z; e4[3] = one * four.w;
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const int s = ts * 64 + tx * 4 + j;
+                        e4[j] = s <= t ? expf(fminf(css[t] - css[s], 0.f)) * dts[s] : 0.f;
+                    }
+                }
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const int s = ts * 64 + tx * 4 + j;
-                    const float w = s <= t ? s4[j] * expf(fminf(css[t] - css[s], 0.f)) * dts[s] : 0.f;
+                    const float w = s4[j] * e4[j];
                     ws[i][j] += w;
                     row = fmaf(w, c4[j], row);
                     col[j] = fmaf(w, c4[j], col[j]);
@@ -579,7 +613,7 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
                 for (int w = 0; w < 8; ++w) s += red[w][tid];
                 p.psi[vo + (size_t)tt * Q + ts * 64 + tid] = s;
             }
-            // red, css and dts are rewritten only after the next head's first barrier or by the threads that read them here
+            // red, css, dts and fac are rewritten only after the next head's first barrier or by the threads that read them here
             __syncthreads();
         }
         // dC[tt] = Wsum B_ts: a[k = s][t]
