@@ -93,20 +93,18 @@ def load_peaks():
 
 
 # ----------------------------------------------------------------------------- DRAM traffic from ncu
-# dram__bytes_read.sum + dram__bytes_write.sum per launch, from the `ncu --set full` capture summarised in
-# profiles/ncu_full_all_kernels_cfg2_geometry.txt, taken at workload 2's launch geometry (one launch = 4096 tokens x
+# dram__bytes_read.sum + dram__bytes_write.sum per launch, from the `ncu` capture summarised in
+# profiles/ncu_all_kernels_cfg2_geometry.txt, taken at workload 2's launch geometry (one launch = 4096 tokens x
 # 80 heads).  A figure is used only while the kernel's source file still has the hash it had when the counters were
 # taken; for the other workloads it is scaled by tokens x heads per launch (the traffic of these kernels grows in
 # proportion).
 NCU_TRAFFIC = {
     # kernel kind: (bytes per launch, source file, sha256 of that file at capture time)
-    "bwd_dBdC": (139.4e6, "ssd_tc_bcf.cu", "dea27dee76a18e163bad504ab1ea872d692421f290753dcb7e87928a10f9f10c"),
-    "bwd_dx": (165.8e6, "ssd_tc_scan.cu", "8456e62e2f5db54b7c0b95e493eead1031cbb85dbd1e34e93385165c68151b98"),
-    "chunk_scan_fwd": (89.2e6, "ssd_tc_scan.cu", "8456e62e2f5db54b7c0b95e493eead1031cbb85dbd1e34e93385165c68151b98"),
-    "chunk_state": (47.8e6, "ssd_tc.cu", "443a66c3f770fd0077e43b67055287dd8166d54e8c90b99a3bedc785227b7f08"),
-    "dstate_contrib": (70.9e6, "ssd_tc.cu", "443a66c3f770fd0077e43b67055287dd8166d54e8c90b99a3bedc785227b7f08"),
-    "state_pass_fwd": (45.4e6, "ssd_simt.cu", "701070c9421ce252f39d2b71218181c3ccaac7433187a73effa60c6cfa5de8f7"),
-    "state_pass_bwd": (68.4e6, "ssd_simt.cu", "701070c9421ce252f39d2b71218181c3ccaac7433187a73effa60c6cfa5de8f7"),
+    "bwd_dBdC": (183.7e6, "ssd_tc_bcf.cu", "05d951ddd3b1d12573fabf8612c4c4413df5aa4bd8d077bd87952e6c3c7d9632"),
+    "bwd_dx": (154.7e6, "ssd_tc_scan.cu", "b52bb89997529d34f8ca36599dac8f3931ba7b25be489e6b47094179374f7444"),
+    "chunk_scan_fwd": (99.8e6, "ssd_tc_scan.cu", "b52bb89997529d34f8ca36599dac8f3931ba7b25be489e6b47094179374f7444"),
+    "chunk_state": (56.1e6, "ssd_tc_chain.cu", "0c1b41e1c993482dd72040140c19ac5e5dfb7ef4dc590f254d2ee51a6951ab89"),
+    "dstate_contrib": (102.4e6, "ssd_tc_chain.cu", "0c1b41e1c993482dd72040140c19ac5e5dfb7ef4dc590f254d2ee51a6951ab89"),
 }
 NCU_UNITS = 4096 * 80
 

@@ -16,7 +16,8 @@
 //   warp 4 producer (TMA) | warp 8 MMA issuer | warp 12 rho / psi out | warps 9, 13, 14 row scaling
 // Tensor memory: two score buffers and the two accumulators, 128 columns each.  The rows of a head are scaled in place for
 // the inter-block terms once its scores have been multiplied, and both terms go straight into the accumulators.
-// Bound by the instruction issue of the scheduler that holds the four sub-tiles of row quarter 3.
+// Bound by the instruction issue of the scheduler that holds the four sub-tiles of row quarter 3.  4096 steps of 80 heads: 78 us
+// on 64 SMs (48 % of their issue slots), 94 us on 144 before, with 256-step chunks as three tiles.
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
 

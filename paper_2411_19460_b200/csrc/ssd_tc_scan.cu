@@ -13,9 +13,10 @@
 // tensor memory twice: scores (fp32, 128 columns, made once per block and group), two masked tiles (bf16, 64 columns
 // each, the A operand straight from tensor memory: no shared-memory ring, no proxy fence) and two pairs of accumulators.
 //
-// Work is the flat list of (batch, block, head); each CTA (one per SM, fewer where other kernels run beside it) takes an equal, contiguous part of it, so that the
-// scores are made again only where a part crosses into the next block or group and every SM ends at the same time.  The
-// heads are per-output, so the cut points change no bit.  Roles, meeting only through mbarriers:
+// Work is the flat list of (batch, block, head); each CTA (one per SM, fewer where other kernels run beside it) takes an
+// equal, contiguous part of it, so that the scores are made again only where a part crosses into the next block or group and
+// every SM ends at the same time.  The heads are per-output, so the cut points change no bit.  Roles, meeting only through
+// mbarriers:
 //   warp 0 producer: ring of stages, one per head (value rows, chunk state, record of the mask's factors; SC_DX: x rows in
 //          a ring of their own); the columns operand of the scores takes a stage of the ring too
 //   warps 1, 2 MMA issuers, of alternate heads (one thread needs longer per head than the products take): acc2 = Rows State,
@@ -28,6 +29,9 @@
 // column of the column sub-tile), three factors that are each <= 1 because cs is non-increasing.  On the diagonal the same
 // product without the middle factor has one factor > 1; it is used where the decay inside the sub-tile is mild, and only stiff
 // heads are exponentiated element by element.
+//
+// Bound by the instruction issue of the mask warps (45 % of the slots of a busy SM, tensor pipe 16 %, DRAM 38 %).  4096 steps of
+// 80 heads, alone on the GPU: y 46 -> 32 us, dx 57 -> 44 us against one CTA per (256-step chunk, row half, head range).
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
 
