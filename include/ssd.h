@@ -103,9 +103,9 @@ typedef struct ssd_shape {
 
 /* Bytes of scratch `ws` that `op` needs for this shape (0 on an invalid shape).  Grows with
  * seg/chunk (the per-segment chunk states: the "grid cell" term of Eq. 4), not with L, apart from
- * 8 bytes per (batch, head, chunk) of dA/dD partial sums in the backward.  With four segments or more
- * the tensor-core path keeps second copies of what neighbouring segments' kernels touch at the same
- * time, unless shape->flags has SSD_FLAG_SERIAL: size the buffer with the flags the call will use.
+ * 20 bytes per (batch, head, chunk) of dA/dD partial sums in the backward.  With two segments or more
+ * there are second and third copies of what neighbouring segments' kernels touch at the same time,
+ * unless shape->flags has SSD_FLAG_SERIAL: size the buffer with the flags the call will use.
  * Whether the tensor-core path is taken depends on the CUDA driver being present (it resolves the
  * tensor-map encoder at run time), so the answer is the one for the machine the query runs on. */
 size_t ssd_workspace_bytes(const ssd_shape_t *shape, int op);
