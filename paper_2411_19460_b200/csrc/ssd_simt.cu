@@ -255,7 +255,7 @@ template <typename T, int NS> __host__ __device__ __forceinline__ int simt_n_sum
     const int nrt = p.Q >> 6;
     return p.nc * p.B * ((NS / 64) * p.H * (grads ? 2 : 1) + p.G * (nrt * (nrt + 1) / 2));
 }
-template <typename T, int NS> __device__ __forceinline__ void simt_sums(const SegParams &p, SimtTiles &sm, float *wsm, float *tot, int id, bool grads) {
+template <typename T, int NS> __device__ __forceinline__ void simt_sums(const SegParams &p, SimtTiles &sm, float *wsm, int id, bool grads) {
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, nh = NS / 64;
     const size_t HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
     const int nsum = p.nc * nh * p.H * p.B;
@@ -296,32 +296,40 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
     const T *cols = (const T *)(dst ? p.Cm : p.Bm) + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS + n0;
     tile_load(ra, rows, HP, false);
     tile_load(rb, cols, GN, false);
-    // the chunk cumsum: a thread per step, shuffle scans of 32 and the warps' totals
-    const int lane = tid & 31, warp = tid >> 5;
-    float d = 0.f, v = 0.f;
-    if (tid < Q) {
-        d = __ldg(p.dt + (size_t)b * p.dt_bs + (tok0 + tid) * p.H + h);
-        v = d * __ldg(p.A + h);
-    }
+    // the chunk cumsum by one warp: a lane sums its Q/32 consecutive steps in order, then a shuffle scan over the lanes
+    if (tid < 32) {
+        const int per = Q >> 5;
+        const float Ah = __ldg(p.A + h);
+        float d[8], v[8], run = 0.f;
 #pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const float t = __shfl_up_sync(0xffffffffu, v, off);
-        if (lane >= off) v += t;
-    }
-    if (lane == 31) tot[warp] = v;
-    __syncthreads();
-    float before = 0.f, last = 0.f;
-    for (int w = 0; w < Q / 32; ++w) {
-        if (w < warp) before += tot[w];
-        last += tot[w];
-    }
-    v += before;
-    if (tid < Q) {
-        wsm[tid] = dst ? expf(v) : expf(fminf(last - v, 0.f)) * d;
-        if (n0 == 0 && !dst) {
-            p.cs[vec_off(p, b, h, c) + tid] = v;
-            p.dtT[vec_off(p, b, h, c) + tid] = d;
+        for (int k = 0; k < 8; ++k)
+            if (k < per) d[k] = __ldg(p.dt + (size_t)b * p.dt_bs + (tok0 + tid * per + k) * p.H + h);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (k < per) {
+                run += d[k] * Ah;
+                v[k] = run;
+            }
+        float incl = run;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const float t = __shfl_up_sync(0xffffffffu, incl, off);
+            if (tid >= off) incl += t;
         }
+        float excl = __shfl_up_sync(0xffffffffu, incl, 1);
+        if (tid == 0) excl = 0.f;
+        const float last = __shfl_sync(0xffffffffu, run + excl, 31);
+#pragma unroll
+        for (int k = 0; k < 8; ++k)
+            if (k < per) {
+                const int t = tid * per + k;
+                const float cs = v[k] + excl;
+                wsm[t] = dst ? expf(cs) : expf(fminf(last - cs, 0.f)) * d[k];
+                if (n0 == 0 && !dst) {
+                    p.cs[vec_off(p, b, h, c) + t] = cs;
+                    p.dtT[vec_off(p, b, h, c) + t] = d[k];
+                }
+            }
     }
     __syncthreads();
     for (int s0 = 0; s0 < Q; s0 += 64) {
@@ -350,8 +358,8 @@ template <typename T, int NS> __global__ void __launch_bounds__(256, 3) k_simt_s
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
-    __shared__ float wsm[256], tot[8];
-    simt_sums<T, NS>(p, sm, wsm, tot, blockIdx.x, grads);
+    __shared__ float wsm[256];
+    simt_sums<T, NS>(p, sm, wsm, blockIdx.x, grads);
 }
 
 // One 64-row tile of y (DX = false) or of dx (DX = true) of one head:
@@ -493,7 +501,7 @@ __global__ void __launch_bounds__(256, NS == 64 ? 2 : 3) k_simt_y(SegParams p, S
     const int nrt = p.Q >> 6, ny = (int)gridDim.x - n_next;
     int id = blockIdx.x;
     if (id >= ny) {
-        simt_sums<T, NS>(nx, sm, css, dts, id - ny, false);
+        simt_sums<T, NS>(nx, sm, css, id - ny, false);
         return;
     }
     const int rt = id % nrt, c = (id / nrt) % p.nc, h = (id / (nrt * p.nc)) % p.H, b = id / (nrt * p.nc * p.H);
@@ -595,8 +603,11 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
                 for (int j = 0; j < 4; ++j) {
                     const float w = s4[j] * e4[j];
                     ws[i][j] += w;
-                    row = fmaf(w, c4[j], row);
-                    col[j] = fmaf(w, c4[j], col[j]);
+                    // s = t adds the same to rho_t and psi_t, of which only sums of differences are used: left out of both, or with
+                    // strong decays, where it is the largest term, its rounding would be most of the error of dA
+                    const float wc = i == j && tx == ty && tt == ts ? 0.f : w;
+                    row = fmaf(wc, c4[j], row);
+                    col[j] = fmaf(wc, c4[j], col[j]);
                 }
                 row = sum_tx(row);
                 if (tx == 0) p.rho[vo + (size_t)ts * Q + t] = row;
@@ -843,10 +854,10 @@ __global__ void __launch_bounds__(256, 3) k_simt_tail(SegParams p, SegParams nx,
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
-    __shared__ float wsm[256], tot[8];
+    __shared__ float wsm[256];
     static_assert(sizeof(SimtTiles) >= FIN_TILE * sizeof(float), "the finishing step's tile");
     const int id = (int)blockIdx.x - n_next;
-    if (id < 0) simt_sums<T, NS>(nx, sm, wsm, tot, blockIdx.x, true);
+    if (id < 0) simt_sums<T, NS>(nx, sm, wsm, blockIdx.x, true);
     else if (id < nfin) bwd_finish(p, &sm.a[0][0], id);
     else reduce_dbdc<T>(p, id - nfin);
 }
