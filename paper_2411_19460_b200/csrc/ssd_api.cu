@@ -286,6 +286,7 @@ static void fill_params(const Plan &pl, const Layout &lo, void *ws, SegParams &s
     sp.hpg = pl.hpg; sp.ncs = pl.ncs; sp.nct = pl.nct; sp.nsl = pl.nsl;
     sp.ndd = pl.use_tc ? 4 : pl.Q / 64;
     sp.scan_ctas = kNumSMs;
+    sp.chain_heads = 1;
     sp.ngh = pl.use_tc ? 8 : pl.P * pl.N / kStatePassElems;
     sp.x_bs = pl.x_bs; sp.dt_bs = pl.dt_bs; sp.bc_bs = pl.bc_bs;
     char *w = (char *)ws;
@@ -306,13 +307,20 @@ static void set_segment(const Plan &pl, int k, SegParams &sp) {
     sp.c0 = sp.t0 / pl.Q;
 }
 
+// Heads per CTA of the forward chain.  Two where a CTA per head would not fit one wave, and where the segments are pipelined
+// and there are heads enough: then the SM time counts, not the latency of a segment.
+static int chain_heads(const Plan &pl, bool pipelined) {
+    const int ctas = pl.B * pl.H;
+    return pl.hpg % 2 == 0 && (ctas > kNumSMs || (pipelined && ctas > kNumSMs / 2)) ? 2 : 1;
+}
+
 // CTAs of the y / dx kernel (its results do not depend on them).  It takes the whole GPU unless the segments are pipelined and
 // small: then the kernels that run beside it (chain kernels, one CTA per head; dB/dC) get SMs of their own, because a chain
 // that waits for the large kernel to finish makes the segments serial (24 heads, 2048-token segments: a chain kernel takes 15
 // us on 24 SMs, y 8 us on all of them).  Not where less than a quarter of the GPU would be left for it.
 static int scan_ctas(const SegParams &sp, bool pipelined, bool bwd) {
     if (!pipelined) return kNumSMs;
-    const int beside = sp.B * sp.H * (bwd ? 2 : 1) + (bwd ? sp.nc * sp.nsl * sp.G * sp.B : 0);
+    const int beside = sp.B * sp.H / sp.chain_heads + (bwd ? sp.B * sp.H : 0) + (bwd ? sp.nc * sp.nsl * sp.G * sp.B : 0);
     return kNumSMs - beside >= kNumSMs / 4 ? kNumSMs - beside : kNumSMs;
 }
 
@@ -364,6 +372,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         TcMaps mk[3] = {maps, maps, maps};
         if (!state_maps(lo, ws, sp, mk, ncp)) return SSD_ECUDA;
         cudaStream_t chain = side->s[0];
+        sp.chain_heads = chain_heads(pl, true);
         SSD_TRY(cudaEventRecord(side->start, st));
         SSD_TRY(cudaStreamWaitEvent(chain, side->start, 0));
         for (int k = 0; k < pl.nseg; ++k) {
@@ -386,6 +395,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         }
         return SSD_OK;
     }
+    sp.chain_heads = chain_heads(pl, false);
     const bool beside = may_use_helper_stream && !pl.serial;      // CUDA cores: the next segment's sums in the launch of y
     SegParams next;
     for (int k = 0; k < pl.nseg; ++k) {
@@ -558,6 +568,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         // chain alone.
         const bool twin = pl.nseg >= kMinSegmentsForTwins;    // else one copy of what the gradient chain writes
         const int ncp = chain_copies(pl.nseg), npar = twin ? 2 : 1;
+        sp.chain_heads = chain_heads(pl, pl.nseg > 1);
         TcMaps cmaps[3] = {maps, maps, maps};
         if (!state_maps(lo, ws, sp, cmaps, ncp)) return SSD_ECUDA;
         cudaStream_t grads = side->s[0], recomp = side->s[4], tails = side->s[2];
@@ -620,6 +631,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         }
         SSD_TRY(cudaStreamWaitEvent(st, side->tail_done[(pl.nseg - 1) % 3], 0));   // the finishing stream is in order: this covers every segment
     } else {
+        sp.chain_heads = chain_heads(pl, false);
         for (int k = pl.nseg - 1; k >= 0; --k) {
             set_segment(pl, k, sp);
             // Recompute_Forward: chunk-entry states of segment k from the stored boundary state; then backward through the

@@ -81,6 +81,7 @@ struct SegParams {
     int nsl;       // head slices per group in the dB/dC partial buffers
     int ndd;       // partial sums of dD per (head, chunk) that the kernels of this path write (<= 4)
     int scan_ctas; // CTAs of the y / dx kernel, at most (no effect on results)
+    int chain_heads; // heads per CTA of the forward chain, 1 or 2 (no effect on results)
     int ngh;       // partial sums of <G,H> per (head, chunk) (<= 16)
     int tiles;     // CUDA-core path: 64-step tiles per chunk (rho, psi and the slices come per tile); tensor-core path: 0
     float dx_skip;    // 1 when dx also takes dy (a skip connection around the layer), else 0

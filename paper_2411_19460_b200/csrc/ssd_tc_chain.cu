@@ -5,7 +5,7 @@
 //   CHAIN_BWD: G_{c-1} = e^{cs_last} G_c + sum_t e^{cs_t} dy_t C_t^T                 (G_c: gradient leaving block c)
 //              rho2_t  = e^{cs_t} dy_t . (H_in C_t),   <G,H> partials = e^{cs_last} <G_c, H_in,c>
 //
-// One CTA owns one (batch, head) and walks the segment's blocks.  A block's sum does not depend on the carried state, so
+// One CTA owns one (batch, head), or in the forward two heads of a group, and walks the segment's blocks.  A block's sum does not depend on the carried state, so
 // it is made by tcgen05 one block ahead; the carry (N x 64 fp32) never leaves the registers of the eight worker warps:
 // what is written per block is its bf16 copy, the operand of the large kernels, 16 KB, where separate kernels for the
 // sums and the recurrence moved 32 KB of fp32 sums out and in again on top.  States are kept transposed here, [N][64], so
@@ -25,19 +25,30 @@ using namespace sm100;
 
 namespace {
 
-__host__ __device__ constexpr int ch_threads(int mode) { return mode ? 768 : 640; }
+// heads per CTA: one, or in the forward two of the same group, which then share the block's B rows and a product of N = 128
+__host__ __device__ constexpr int ch_rec_warps(int heads) { return heads == 2 ? 4 : 2; }
+__host__ __device__ constexpr int ch_threads(int mode, int heads) { return 32 * (2 + ch_rec_warps(heads) + 8 + 8 * heads + (mode ? 4 : 0)); }
 constexpr int CH_T = 128;
-__host__ __device__ constexpr int ch_stages(int mode) { return mode ? 3 : 4; }
-constexpr int CH_VEC = 4;                 // CHAIN_FWD: vector buffers (weights of 128 rows + the block's decay)
-constexpr int CH_VEC_FLOATS = 260;
+__host__ __device__ constexpr int ch_stages(int mode, int heads) { return mode || heads == 2 ? 3 : 4; }
+// CHAIN_FWD: vector buffers per head (weights of 128 rows + the block's decay); for two heads the weights' bf16 pairs are packed
+__host__ __device__ constexpr int ch_vec(int heads) { return heads == 2 ? 2 : 4; }
+__host__ __device__ constexpr int ch_vec_floats(int heads) { return heads == 2 ? 132 : 260; }
 constexpr float kLog2eC = 1.4426950408889634f;
 constexpr int CH_AHEAD = 4;               // L2 prefetch distance in blocks beyond the staged ones
 
-// stage: V (B or C rows) N/64 x 16 KB | X (x or dy rows) 16 KB | CHAIN_BWD: H_in^T, N rows of 128 B | row scales 1 KB, decay 16 B
-__host__ __device__ constexpr uint32_t ch_stage_bytes(int mode, int ns) { return (uint32_t)ns * 256 + 16384 + (mode ? (uint32_t)ns * 128 + 2048 : 0); }
-__host__ __device__ constexpr uint32_t ch_smem(int mode, int ns) {
-    return ch_stages(mode) * ch_stage_bytes(mode, ns) + 8 * 2048 + (mode ? 0 : CH_VEC * CH_VEC_FLOATS * 4) + 1024;
+// stage: V (B or C rows) N/64 x 16 KB | X (x or dy rows) 16 KB per head | CHAIN_BWD: H_in^T, N rows of 128 B | row scales 1 KB, decay 16 B
+__host__ __device__ constexpr uint32_t ch_stage_bytes(int mode, int ns, int heads) {
+    return (uint32_t)ns * 256 + (uint32_t)heads * 16384 + (mode ? (uint32_t)ns * 128 + 2048 : 0);
 }
+__host__ __device__ constexpr uint32_t ch_off_vec(int mode, int ns, int heads) {
+    return ch_stages(mode, heads) * ch_stage_bytes(mode, ns, heads) + heads * 8 * 2048;
+}
+__host__ __device__ constexpr uint32_t ch_off_bar(int mode, int ns, int heads) {
+    return ch_off_vec(mode, ns, heads) + (mode ? 0 : heads * ch_vec(heads) * ch_vec_floats(heads) * 4);
+}
+// for the alignment of the stages: two heads leave no room for all of 1 KB, but no static shared memory is in front of them
+__host__ __device__ constexpr uint32_t ch_slack(int heads) { return heads == 2 ? 512 : 1024; }
+__host__ __device__ constexpr uint32_t ch_smem(int mode, int ns, int heads) { return ch_off_bar(mode, ns, heads) + 256 + ch_slack(heads); }
 
 __device__ __forceinline__ float ex2c(float x) {
     float y;
@@ -52,21 +63,29 @@ __device__ __forceinline__ float2 unpack2c(uint32_t w) { return __bfloat1622floa
 
 }  // namespace
 
-template <int NS, int MODE>
-__global__ void __launch_bounds__(ch_threads(MODE), 1)
+template <int NS, int MODE, int HEADS>
+__global__ void __launch_bounds__(ch_threads(MODE, HEADS), 1)
 k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, long long bnd_bs, float *carry_out, float *final_out,
            const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmH,
            const __grid_constant__ CUtensorMap tmOut) {
     constexpr bool BWD = MODE == CHAIN_BWD;
-    constexpr int CH_STAGES = ch_stages(MODE);
-    constexpr uint32_t STAGE = ch_stage_bytes(MODE, NS), OFF_X = NS * 256, OFF_H = OFF_X + 16384, OFF_W = OFF_H + NS * 128;
-    constexpr uint32_t OFF_OUT = CH_STAGES * STAGE, OFF_VEC = OFF_OUT + 8 * 2048;
-    extern __shared__ unsigned char smem_raw[];
+    static_assert(!BWD || HEADS == 1, "the backward has a head per CTA");
+    constexpr int CH_STAGES = ch_stages(MODE, HEADS), CH_VEC = ch_vec(HEADS), VEC_FLOATS = ch_vec_floats(HEADS), DECAY_AT = VEC_FLOATS - 4;
+    constexpr int SCALE0 = 2 + ch_rec_warps(HEADS), CARRY0 = SCALE0 + 8, RHO0 = CARRY0 + 8 * HEADS;      // first warps of the roles
+    constexpr uint32_t STAGE = ch_stage_bytes(MODE, NS, HEADS), OFF_X = NS * 256, OFF_H = OFF_X + HEADS * 16384, OFF_W = OFF_H + NS * 128;
+    constexpr uint32_t OFF_OUT = CH_STAGES * STAGE, OFF_VEC = ch_off_vec(MODE, NS, HEADS), OFF_BAR = ch_off_bar(MODE, NS, HEADS);
+    extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t full[CH_STAGES], scaled[CH_STAGES], empty[CH_STAGES], mdone[2], dempty[2], vfull[CH_VEC], vempty[CH_VEC];
-    __shared__ uint32_t tmem_base, abort_flag;
+    if ((uint32_t)(smem - smem_raw) > ch_slack(HEADS)) {        // the same for every CTA; not reached
+        if (threadIdx.x == 0) *p.status = 1u;
+        return;
+    }
+    uint64_t *const full = reinterpret_cast<uint64_t *>(smem + OFF_BAR), *const scaled = full + CH_STAGES, *const empty = scaled + CH_STAGES;
+    uint64_t *const mdone = empty + CH_STAGES, *const dempty = mdone + 2, *const vfull = dempty + 2, *const vempty = vfull + HEADS * CH_VEC;
+    uint32_t *const words = reinterpret_cast<uint32_t *>(vempty + HEADS * CH_VEC);
+    static_assert((3 * CH_STAGES + 4 + 2 * HEADS * CH_VEC) * 8 + 8 <= 256, "barriers");
 
-    const int h = blockIdx.x, b = blockIdx.y, g = h / p.hpg, nc = p.nc;
+    const int h0 = blockIdx.x * HEADS, b = blockIdx.y, g = h0 / p.hpg, nc = p.nc;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     auto chunk_of = [&](int i) { return BWD ? nc - 1 - i : i; };
     if (tid == 0) {
@@ -77,24 +96,24 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&mdone[i], 1);
-            mbar_init(&dempty[i], BWD ? 8 + 4 : 8);
+            mbar_init(&dempty[i], BWD ? 8 + 4 : 8 * HEADS);
         }
-        for (int i = 0; i < CH_VEC; ++i) {
+        for (int i = 0; i < HEADS * CH_VEC; ++i) {
             mbar_init(&vfull[i], 1);
             mbar_init(&vempty[i], 8);              // the carry warps, which read the decay last
         }
-        abort_flag = 0;
+        words[1] = 0;
         fence_barrier_init();
     }
-    constexpr uint32_t NCOL = BWD ? 256 : 128;     // block sum, double buffered; BWD: H_in C likewise
-    if (warp == 0) tmem_alloc(&tmem_base, NCOL);
+    constexpr uint32_t NCOL = BWD ? 256 : 128 * HEADS;     // block sum, double buffered; BWD: H_in C likewise
+    if (warp == 0) tmem_alloc(&words[0], NCOL);
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
     // What the kernel before this one in the stream may still write, or still read where this one writes, is waited for in the
     // roles that touch it; x, dt, B, C and dy are older than that kernel, so the first blocks are loaded and scaled under its end.
-    const uint32_t tm = tmem_base;
-    volatile uint32_t *abortp = &abort_flag;
+    const uint32_t tm = words[0];
+    volatile uint32_t *abortp = &words[1];
 
     if (warp == 0) {
         // ------------------------------------------------------------ producer
@@ -103,7 +122,8 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 const int st = i % CH_STAGES, tok = p.t0 + chunk_of(i) * CH_T;
                 unsigned char *sb = smem + st * STAGE;
                 mbar_arrive_expect_tx(&full[st], BWD ? STAGE - 1024 + 16 : STAGE);
-                tma_load_3d(sb + OFF_X, &tmX, &full[st], h * 64, tok, b);
+#pragma unroll
+                for (int k = 0; k < HEADS; ++k) tma_load_3d(sb + OFF_X + k * 16384, &tmX, &full[st], (h0 + k) * 64, tok, b);
 #pragma unroll
                 for (int nh = 0; nh < NS / 64; ++nh) tma_load_3d(sb + nh * 16384, &tmV, &full[st], g * NS + nh * 64, tok, b);
             };
@@ -121,19 +141,21 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 // and its CTAs would hold SMs idle
                 if (i + CH_STAGES + 1 == nc) pdl_launch_dependents();
                 if (BWD) {
-                    const float *rec = p.rec + (((size_t)b * p.H + h) * p.ncs + c) * REC_FLOATS;
-                    tma_load_3d(sb + OFF_H, &tmH, &full[st], 0, ((b * p.ncs + c) * p.H + h) * NS, 0);
+                    const float *rec = p.rec + (((size_t)b * p.H + h0) * p.ncs + c) * REC_FLOATS;
+                    tma_load_3d(sb + OFF_H, &tmH, &full[st], 0, ((b * p.ncs + c) * p.H + h0) * NS, 0);
                     bulk_load(sb + OFF_W, rec + REC_OC, 1024, &full[st]);
                     bulk_load(sb + OFF_W + 1024, rec + REC_DECAY, 16, &full[st]);
                 }
-                if (i + CH_AHEAD < nc) tma_prefetch_3d(&tmX, h * 64, p.t0 + chunk_of(i + CH_AHEAD) * CH_T, b);
+                if (i + CH_AHEAD < nc)
+#pragma unroll
+                    for (int k = 0; k < HEADS; ++k) tma_prefetch_3d(&tmX, (h0 + k) * 64, p.t0 + chunk_of(i + CH_AHEAD) * CH_T, b);
             }
             if (nc <= CH_STAGES) pdl_launch_dependents();
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer
         if (elect_one()) {
-            const uint32_t idD = umma_idesc_bf16(128, 64, true, true), idY = umma_idesc_bf16(128, 64, false, true);
+            const uint32_t idD = umma_idesc_bf16(128, 64 * HEADS, true, true), idY = umma_idesc_bf16(128, 64, false, true);
             for (int i = 0; i < nc; ++i) {
                 const int st = i % CH_STAGES, bf = i & 1;
                 const uint32_t sb = smem_u32(smem + st * STAGE);
@@ -148,8 +170,8 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
 #pragma unroll
                 for (int k = 0; k < 8; ++k) {
                     const uint64_t ad = umma_desc_words(loV + k * 128, hiM), bd = umma_desc_words(loX + k * 128, hiX);
-                    if (k == 0) umma_bf16_fixed<false>(tm + bf * 64, ad, bd, idD);
-                    else umma_bf16_fixed<true>(tm + bf * 64, ad, bd, idD);
+                    if (k == 0) umma_bf16_fixed<false>(tm + bf * 64 * HEADS, ad, bd, idD);
+                    else umma_bf16_fixed<true>(tm + bf * 64 * HEADS, ad, bd, idD);
                 }
                 if (BWD) {   // Y[t][p] = sum_n C[t][n] H_in[p][n]
                     const uint64_t dC = umma_desc_sw128(sb, 16, 1024), dH = umma_desc_sw128(sb + OFF_H, 8192, 1024);
@@ -165,11 +187,11 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 umma_commit(&mdone[bf]);
             }
         }
-    } else if (warp < 4) {
+    } else if (warp < SCALE0) {
         // ------------------------------------------------------------ records, a lane owns four consecutive steps
         if (!BWD) {
-            const int first = warp - 2;
-            float *vec = reinterpret_cast<float *>(smem + OFF_VEC);
+            const int first = (warp - 2) & 1, hl = (warp - 2) >> 1, h = h0 + hl;
+            float *vec = reinterpret_cast<float *>(smem + OFF_VEC) + hl * CH_VEC * VEC_FLOATS;
             const float Ah = __ldg(p.A + h);
             // fetched four of this warp's blocks ahead: the strided step sizes take longer to arrive than a block takes
             auto fetch = [&](int i, float4 &v) {
@@ -185,7 +207,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
             for (int k = 0; k < 4; ++k) {
                 const int i = i0 + 2 * k;
                 if (i >= nc) break;
-                const int vb = i % CH_VEC;
+                const int vb = i % CH_VEC, vbar = hl * CH_VEC + vb;
                 const float4 dt4 = ring[k];
                 if (i + 8 < nc) fetch(i + 8, ring[k]);
                 const float d[4] = {dt4.x, dt4.y, dt4.z, dt4.w};
@@ -212,8 +234,8 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 float w[4];
 #pragma unroll
                 for (int m = 0; m < 4; ++m) w[m] = ex2c(fminf(last - cs[m], 0.f)) * d[m];
-                if (i >= CH_VEC) mbar_wait(&vempty[vb], (i / CH_VEC - 1) & 1, abortp, p.status);
-                float *v = vec + vb * CH_VEC_FLOATS;
+                if (i >= CH_VEC) mbar_wait(&vempty[vbar], (i / CH_VEC - 1) & 1, abortp, p.status);
+                float *v = vec + vb * VEC_FLOATS;
                 RowScale ob[4];
 #pragma unroll
                 for (int m = 0; m < 4; ++m) ob[m] = row_scale(w[m]);
@@ -222,10 +244,14 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                     d4[0] = make_uint4(sc[0].hi, sc[0].lo, sc[1].hi, sc[1].lo);
                     d4[1] = make_uint4(sc[2].hi, sc[2].lo, sc[3].hi, sc[3].lo);
                 };
-                put_scales(v, ob);
-                if (lane == 0) v[256] = decay;
+                if (HEADS == 2)
+                    *reinterpret_cast<uint4 *>(v + lane * 4) = make_uint4(__byte_perm(ob[0].hi, ob[0].lo, 0x5410), __byte_perm(ob[1].hi, ob[1].lo, 0x5410),
+                                                                          __byte_perm(ob[2].hi, ob[2].lo, 0x5410), __byte_perm(ob[3].hi, ob[3].lo, 0x5410));
+                else
+                    put_scales(v, ob);
+                if (lane == 0) v[DECAY_AT] = decay;
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&vfull[vb]);
+                if (lane == 0) mbar_arrive(&vfull[vbar]);
                 if (i == first) pdl_wait();        // the earlier kernels have read what this copy of the records held
                 const float lo = __shfl_sync(0xffffffffu, cs[3], lane | 7), hi = __shfl_sync(0xffffffffu, cs[0], lane & ~7);
                 const float bi = __shfl_sync(0xffffffffu, cs[0], ((lane >> 2) & 3) * 8), bj = __shfl_sync(0xffffffffu, cs[3], (lane & 3) * 8 + 7);
@@ -244,34 +270,43 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 put_scales(rec + REC_OB, ob);
             }
         }
-    } else if (warp < 12) {
+    } else if (warp < CARRY0) {
         // ------------------------------------------------------------ the blocks' rows times their weights, in place (a weight is
         // uniform along a row, so the swizzle does not matter)
-        const int th = tid - 128;
+        const int th = tid - SCALE0 * 32;
         for (int i = 0; i < nc; ++i) {
             const int st = i % CH_STAGES;
             unsigned char *sb = smem + st * STAGE;
-            const RowScale *w = reinterpret_cast<const RowScale *>(BWD ? sb + OFF_W : smem + OFF_VEC + (i % CH_VEC) * CH_VEC_FLOATS * 4);
             mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
-            if (!BWD) mbar_wait(&vfull[i % CH_VEC], (i / CH_VEC) & 1, abortp, p.status);
-            uint4 *x4 = reinterpret_cast<uint4 *>(sb + OFF_X) + th;
-            uint4 v[4];
-            RowScale f[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                v[k] = x4[k * 256];
-                f[k] = w[(th >> 3) + 32 * k];
-            }
+            for (int hl = 0; hl < HEADS; ++hl) {
+                const unsigned char *w = BWD ? sb + OFF_W : smem + OFF_VEC + (hl * CH_VEC + i % CH_VEC) * VEC_FLOATS * 4;
+                if (!BWD) mbar_wait(&vfull[hl * CH_VEC + i % CH_VEC], (i / CH_VEC) & 1, abortp, p.status);
+                uint4 *x4 = reinterpret_cast<uint4 *>(sb + OFF_X + hl * 16384) + th;
+                uint4 v[4];
+                RowScale f[4];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                scale8(v[k], f[k]);
-                x4[k * 256] = v[k];
+                for (int k = 0; k < 4; ++k) {
+                    v[k] = x4[k * 256];
+                    const int r = (th >> 3) + 32 * k;
+                    if (HEADS == 2) {
+                        const uint32_t pk = reinterpret_cast<const uint32_t *>(w)[r];
+                        f[k] = {__byte_perm(pk, 0, 0x1010), __byte_perm(pk, 0, 0x3232)};
+                    } else {
+                        f[k] = reinterpret_cast<const RowScale *>(w)[r];
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    scale8(v[k], f[k]);
+                    x4[k * 256] = v[k];
+                }
             }
             fence_proxy_async_smem();
             __syncwarp();
             if (lane == 0) mbar_arrive(&scaled[st]);
         }
-    } else if (BWD && warp >= 20) {
+    } else if (BWD && warp >= RHO0) {
         // ------------------------------------------------------------ rho2: row dot of the scaled dy row and H_in C, t = 32 q + lane
         const int q = warp & 3, r = q * 32 + lane;
         pdl_wait();
@@ -301,16 +336,17 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 mbar_arrive(&dempty[bf]);
                 mbar_arrive(&empty[st]);
             }
-            p.rho2[(((size_t)b * p.H + h) * p.ncs + c) * CH_T + r] = acc.x + acc.y;
+            p.rho2[(((size_t)b * p.H + h0) * p.ncs + c) * CH_T + r] = acc.x + acc.y;
         }
     } else {
         // ------------------------------------------------------------ carry: warp (q, half) holds state rows
         // n = 32 q + lane, columns p = 32 half ..; as rows of time, t = 32 q + lane
-        const int q = warp & 3, half = (warp - 12) >> 2;
+        const int w = (warp - CARRY0) & 7, hl = (warp - CARRY0) >> 3, h = h0 + hl;
+        const int q = warp & 3, half = w >> 2;
         const bool act = q * 32 < NS;
-        const uint32_t tl = tm + ((uint32_t)(q * 32) << 16) + half * 32;
-        const float *vec = reinterpret_cast<const float *>(smem + OFF_VEC);
-        unsigned char *stg = smem + OFF_OUT + (warp - 12) * 2048, *row = stg + lane * 64;      // [32 rows][64 B], 64-byte swizzle
+        const uint32_t tl = tm + ((uint32_t)(q * 32) << 16) + hl * 64 + half * 32;
+        const float *vec = reinterpret_cast<const float *>(smem + OFF_VEC) + hl * CH_VEC * VEC_FLOATS;
+        unsigned char *stg = smem + OFF_OUT + (warp - CARRY0) * 2048, *row = stg + lane * 64;      // [32 rows][64 B], 64-byte swizzle
         const size_t so = (size_t)h * 64 * NS + (size_t)(half * 32) * NS + q * 32 + lane;
         float carry[32];
         pdl_wait();                                // the carry that the previous segment's launch left; the earlier states have been read
@@ -355,16 +391,21 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
             __syncwarp();
             tc_fence_after_sync();
             // (CHAIN_FWD: the scaling warps waited for the decay's buffer before the products could start)
-            const float decay = BWD ? *reinterpret_cast<const float *>(smem + st * STAGE + OFF_W + 1024) : vec[(i % CH_VEC) * CH_VEC_FLOATS + 256];
+            const float decay = BWD ? *reinterpret_cast<const float *>(smem + st * STAGE + OFF_W + 1024) : vec[(i % CH_VEC) * VEC_FLOATS + DECAY_AT];
             if (act) {
-                float d[32];
-                tmem_ld32(tl + bf * 64, d);
                 const float2 dec2 = make_float2(decay, decay);
+                constexpr int PART = 32 / HEADS;          // two heads: 64 registers a thread
 #pragma unroll
-                for (int j = 0; j < 32; j += 2) {
-                    const float2 v = __ffma2_rn(dec2, make_float2(carry[j], carry[j + 1]), make_float2(d[j], d[j + 1]));
-                    carry[j] = v.x;
-                    carry[j + 1] = v.y;
+                for (int c0 = 0; c0 < 32; c0 += PART) {
+                    float d[PART];
+                    if constexpr (HEADS == 2) tmem_ld16(tl + bf * 64 * HEADS + c0, d);
+                    else tmem_ld32(tl + bf * 64, d);
+#pragma unroll
+                    for (int j = 0; j < PART; j += 2) {
+                        const float2 v = __ffma2_rn(dec2, make_float2(carry[c0 + j], carry[c0 + j + 1]), make_float2(d[j], d[j + 1]));
+                        carry[c0 + j] = v.x;
+                        carry[c0 + j + 1] = v.y;
+                    }
                 }
             }
             tc_fence_before_sync();
@@ -373,13 +414,13 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
             if (lane == 0) {
                 mbar_arrive(&dempty[bf]);
                 if (BWD) mbar_arrive(&empty[st]);
-                else mbar_arrive(&vempty[i % CH_VEC]);
+                else mbar_arrive(&vempty[hl * CH_VEC + i % CH_VEC]);
             }
             if (BWD) {
                 float dt = dot.x + dot.y;
 #pragma unroll
                 for (int off = 16; off > 0; off >>= 1) dt += __shfl_xor_sync(0xffffffffu, dt, off);
-                if (lane == 0) p.ghdot[((((size_t)b * p.H + h) * p.ncs + c) << 4) + (warp - 12)] = decay * dt;
+                if (lane == 0) p.ghdot[((((size_t)b * p.H + h) * p.ncs + c) << 4) + w] = decay * dt;
             }
         }
         if (act) {
@@ -400,26 +441,30 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     }
 }
 
-template <int NS, int MODE>
+template <int NS, int MODE, int HEADS>
 static cudaError_t launch_chain(const SegParams &p, const TcMaps &m, const float *init, long long init_bs, float *bnd_out, long long bnd_bs,
                                 float *carry_out, float *final_out, cudaStream_t st) {
-    constexpr uint32_t smem = ch_smem(MODE, NS);
-    const cudaError_t e = allow_smem<k_chain_tc<NS, MODE>>((int)smem);
+    constexpr uint32_t smem = ch_smem(MODE, NS, HEADS);
+    static_assert(smem <= 232448, "shared memory of a CTA");
+    const cudaError_t e = allow_smem<k_chain_tc<NS, MODE, HEADS>>((int)smem);
     if (e != cudaSuccess) return e;
     const bool bwd = MODE == CHAIN_BWD;
-    return launch_pdl(k_chain_tc<NS, MODE>, dim3(p.H, p.B), dim3(ch_threads(MODE)), (size_t)smem, st, p, init, init_bs, bnd_out, bnd_bs, carry_out,
-                      final_out, bwd ? m.dy : m.x, bwd ? m.Cm : m.Bm, m.H, bwd ? m.Gst : m.Hst);
+    return launch_pdl(k_chain_tc<NS, MODE, HEADS>, dim3(p.H / HEADS, p.B), dim3(ch_threads(MODE, HEADS)), (size_t)smem, st, p, init, init_bs, bnd_out,
+                      bnd_bs, carry_out, final_out, bwd ? m.dy : m.x, bwd ? m.Cm : m.Bm, m.H, bwd ? m.Gst : m.Hst);
 }
 
 cudaError_t launch_chain_fwd(const SegParams &p, const TcMaps &m, const float *init, long long init_bs, float *boundary_out, long long bnd_bs,
                              float *final_out, cudaStream_t st) {
-    return p.N == 128 ? launch_chain<128, CHAIN_FWD>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st)
-                      : launch_chain<64, CHAIN_FWD>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st);
+    if (p.chain_heads == 2)
+        return p.N == 128 ? launch_chain<128, CHAIN_FWD, 2>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st)
+                          : launch_chain<64, CHAIN_FWD, 2>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st);
+    return p.N == 128 ? launch_chain<128, CHAIN_FWD, 1>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st)
+                      : launch_chain<64, CHAIN_FWD, 1>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st);
 }
 cudaError_t launch_chain_bwd(const SegParams &p, const TcMaps &m, const float *init, float *left_out, cudaStream_t st) {
     const long long bs = (long long)p.H * 64 * p.N;
-    return p.N == 128 ? launch_chain<128, CHAIN_BWD>(p, m, init, bs, nullptr, 0, left_out, nullptr, st)
-                      : launch_chain<64, CHAIN_BWD>(p, m, init, bs, nullptr, 0, left_out, nullptr, st);
+    return p.N == 128 ? launch_chain<128, CHAIN_BWD, 1>(p, m, init, bs, nullptr, 0, left_out, nullptr, st)
+                      : launch_chain<64, CHAIN_BWD, 1>(p, m, init, bs, nullptr, 0, left_out, nullptr, st);
 }
 
 }  // namespace ssd
