@@ -31,6 +31,8 @@ __host__ __device__ constexpr int ch_threads(int mode, int heads) { return 32 * 
 constexpr int CH_T = 128;
 __host__ __device__ constexpr int ch_stages(int mode, int heads) { return mode || heads == 2 ? 3 : 4; }
 // CHAIN_FWD: vector buffers per head (weights of 128 rows + the block's decay); for two heads the weights' bf16 pairs are packed
+// (a buffer belongs to one record warp: a warp that took buffers in turn with others could wait for a phase two ahead of the
+// barrier's and pass at once, so their number is a multiple of the head's record warps)
 __host__ __device__ constexpr int ch_vec(int heads) { return heads == 2 ? 2 : 4; }
 __host__ __device__ constexpr int ch_vec_floats(int heads) { return heads == 2 ? 132 : 260; }
 constexpr float kLog2eC = 1.4426950408889634f;
@@ -71,6 +73,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     constexpr bool BWD = MODE == CHAIN_BWD;
     static_assert(!BWD || HEADS == 1, "the backward has a head per CTA");
     constexpr int CH_STAGES = ch_stages(MODE, HEADS), CH_VEC = ch_vec(HEADS), VEC_FLOATS = ch_vec_floats(HEADS), DECAY_AT = VEC_FLOATS - 4;
+    static_assert(CH_VEC % (ch_rec_warps(HEADS) / HEADS) == 0, "a vector buffer belongs to one record warp");
     constexpr int SCALE0 = 2 + ch_rec_warps(HEADS), CARRY0 = SCALE0 + 8, RHO0 = CARRY0 + 8 * HEADS;      // first warps of the roles
     constexpr uint32_t STAGE = ch_stage_bytes(MODE, NS, HEADS), OFF_X = NS * 256, OFF_H = OFF_X + HEADS * 16384, OFF_W = OFF_H + NS * 128;
     constexpr uint32_t OFF_OUT = CH_STAGES * STAGE, OFF_VEC = ch_off_vec(MODE, NS, HEADS), OFF_BAR = ch_off_bar(MODE, NS, HEADS);
