@@ -100,11 +100,11 @@ def load_peaks():
 # proportion).
 NCU_TRAFFIC = {
     # kernel kind: (bytes per launch, source file, sha256 of that file at capture time)
-    "bwd_dBdC": (183.7e6, "ssd_tc_bcf.cu", "05d951ddd3b1d12573fabf8612c4c4413df5aa4bd8d077bd87952e6c3c7d9632"),
-    "bwd_dx": (154.7e6, "ssd_tc_scan.cu", "b52bb89997529d34f8ca36599dac8f3931ba7b25be489e6b47094179374f7444"),
-    "chunk_scan_fwd": (99.8e6, "ssd_tc_scan.cu", "b52bb89997529d34f8ca36599dac8f3931ba7b25be489e6b47094179374f7444"),
-    "chunk_state": (56.1e6, "ssd_tc_chain.cu", "0c1b41e1c993482dd72040140c19ac5e5dfb7ef4dc590f254d2ee51a6951ab89"),
-    "dstate_contrib": (102.4e6, "ssd_tc_chain.cu", "0c1b41e1c993482dd72040140c19ac5e5dfb7ef4dc590f254d2ee51a6951ab89"),
+    "bwd_dBdC": (183.6e6, "ssd_tc_bcf.cu", "05d951ddd3b1d12573fabf8612c4c4413df5aa4bd8d077bd87952e6c3c7d9632"),
+    "bwd_dx": (154.3e6, "ssd_tc_scan.cu", "b52bb89997529d34f8ca36599dac8f3931ba7b25be489e6b47094179374f7444"),
+    "chunk_scan_fwd": (100.0e6, "ssd_tc_scan.cu", "b52bb89997529d34f8ca36599dac8f3931ba7b25be489e6b47094179374f7444"),
+    "chunk_state": (55.6e6, "ssd_tc_chain.cu", "84487affb68f5deb7d2f1f3e89a247edcde310d52bb50a7538f9baa8c094eb9d"),
+    "dstate_contrib": (102.4e6, "ssd_tc_chain.cu", "84487affb68f5deb7d2f1f3e89a247edcde310d52bb50a7538f9baa8c094eb9d"),
 }
 NCU_UNITS = 4096 * 80
 
