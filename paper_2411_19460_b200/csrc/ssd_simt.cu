@@ -180,13 +180,17 @@ template <> __device__ __forceinline__ float4 ld4f<__nv_bfloat16>(const __nv_bfl
 
 // A 64 x 64 tile of a row-major matrix on its way to shared memory: four float4 per thread.
 //   direct:     row = tid / 16 + 16 k, columns (tid % 16) * 4 ..            -> s[row][col]      (rows run along k)
-//   transposed: row = (tid % 8) + 8 * (tid / 32) , columns ((tid / 8) % 4) * 4 + 16 k -> s[col][row]   (columns run along k)
+//   transposed: row = tr_row(), columns tr_col(k) ..                        -> s[col][row]      (columns run along k)
+// (a warp of the transposed store holds 16 rows of two column groups, 4 x 68 floats = 16 banks apart: no conflicts; eight rows of
+// four groups conflicted two ways)
+__device__ __forceinline__ int tr_row() { return (threadIdx.x & 15) + 16 * ((threadIdx.x >> 5) & 3); }
+__device__ __forceinline__ int tr_col(int k) { return ((threadIdx.x >> 4) & 1) * 4 + (threadIdx.x >> 7) * 8 + 16 * k; }
 template <typename T> __device__ __forceinline__ void tile_load(float4 (&r)[4], const T *src, size_t stride, bool transposed) {
     const int tid = threadIdx.x;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         if (!transposed) r[k] = ld4f(src + (size_t)((tid >> 4) + 16 * k) * stride + (tid & 15) * 4);
-        else r[k] = ld4f(src + (size_t)((tid & 7) + 8 * (tid >> 5)) * stride + ((tid >> 3) & 3) * 4 + 16 * k);
+        else r[k] = ld4f(src + (size_t)tr_row() * stride + tr_col(k));
     }
 }
 // The same from scratch that an earlier kernel of the call wrote: coherent loads.
@@ -195,7 +199,7 @@ __device__ __forceinline__ void tile_load_ws(float4 (&r)[4], const float *src, s
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const float *q = !transposed ? src + (size_t)((tid >> 4) + 16 * k) * stride + (tid & 15) * 4
-                                     : src + (size_t)((tid & 7) + 8 * (tid >> 5)) * stride + ((tid >> 3) & 3) * 4 + 16 * k;
+                                     : src + (size_t)tr_row() * stride + tr_col(k);
         r[k] = *reinterpret_cast<const float4 *>(q);
     }
 }
@@ -206,7 +210,7 @@ __device__ __forceinline__ void tile_store(float (*s)[ST_LD], const float4 (&r)[
         if (!transposed) {
             *reinterpret_cast<float4 *>(&s[(tid >> 4) + 16 * k][(tid & 15) * 4]) = r[k];
         } else {
-            const int row = (tid & 7) + 8 * (tid >> 5), c = ((tid >> 3) & 3) * 4 + 16 * k;
+            const int row = tr_row(), c = tr_col(k);
             s[c][row] = r[k].x; s[c + 1][row] = r[k].y; s[c + 2][row] = r[k].z; s[c + 3][row] = r[k].w;
         }
     }
@@ -431,8 +435,8 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
         if (ct != rt) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float one = fac[DX ? ct * 64 + ty + 16 * k : r0 + (tid & 7) + 8 * (tid >> 5)];
-                const float4 four = *reinterpret_cast<const float4 *>(fac + (DX ? r0 + tx * 4 : ct * 64 + ((tid >> 3) & 3) * 4 + 16 * k));
+                const float one = fac[DX ? ct * 64 + ty + 16 * k : r0 + tr_row()];
+                const float4 four = *reinterpret_cast<const float4 *>(fac + (DX ? r0 + tx * 4 : ct * 64 + tr_col(k)));
                 ra[k].x *= one * four.x; ra[k].y *= one * four.y; ra[k].z *= one * four.z; ra[k].w *= one * four.w;
             }
         } else
@@ -442,8 +446,8 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 // as tile_load laid them out: not DX (transposed) row t, column s; DX (direct) row t, column s
-                const int t = DX ? ct * 64 + ty + 16 * k : r0 + (tid & 7) + 8 * (tid >> 5);
-                const int s = DX ? r0 + tx * 4 + i : ct * 64 + ((tid >> 3) & 3) * 4 + 16 * k + i;
+                const int t = DX ? ct * 64 + ty + 16 * k : r0 + tr_row();
+                const int s = DX ? r0 + tx * 4 + i : ct * 64 + tr_col(k) + i;
                 e[i] = s <= t ? e[i] * expf(fminf(css[t] - css[s], 0.f)) * (DX ? 1.f : dts[s]) : 0.f;
             }
         }
