@@ -164,6 +164,7 @@ __global__ void __launch_bounds__(CV_RING_THREADS) k_conv_fwd(const T *u, long l
                 for (int j = 0; j < n; ++j) token(sp + j * 512);
             }
         }
+        fence_proxy_async_smem();                      // its reads are over before a bulk copy may overwrite the stage
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[slot]);      // this warp has read the stage
     }
@@ -369,6 +370,7 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
                 }
             }
         }
+        fence_proxy_async_smem();                      // its reads are over before a bulk copy may overwrite the stage
         __syncwarp();
         if (lane == 0) mbar_arrive(&empty[slot]);      // this warp has read the stage
     }

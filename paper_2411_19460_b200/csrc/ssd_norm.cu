@@ -309,6 +309,7 @@ k_gated_norm_staged(const T *y, const T *z, const float *gamma, float eps, const
             if (BWD) sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
         }
         if (lane == 0) red[j & 1][warp] = sum;
+        fence_proxy_async_smem();                         // this thread's reads are over before a bulk copy may overwrite the stage
         __syncthreads();                                  // the sums are there, and every thread has read the stage
         if (threadIdx.x == 0 && j + stages < nrows) issue(j + stages, st);
         if (++st == stages) { st = 0; par ^= 1u; }

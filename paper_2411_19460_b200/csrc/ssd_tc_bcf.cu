@@ -355,6 +355,7 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
             if (hi >= 2) mbar_wait(&pempty[hi & 1], ((hi >> 1) - 1) & 1, abortp, p.status);
             pr[sr * 128 + rl] = racc.x + racc.y;
             pr[512 + q * 128 + sr * 32 + lane] = v[0];
+            fence_proxy_async_smem();      // the record has been read before a bulk copy may overwrite it
             __syncwarp();
             if (lane == 0) {
                 mbar_arrive(&vempty[vb]);
