@@ -106,6 +106,9 @@ typedef struct ssd_shape {
  * 20 bytes per (batch, head, chunk) of dA/dD partial sums in the backward.  With two segments or more
  * there are second and third copies of what neighbouring segments' kernels touch at the same time,
  * unless shape->flags has SSD_FLAG_SERIAL: size the buffer with the flags the call will use.
+ * The tensor-core path takes bf16 calls with N = 128, chunk = 256 and an even H/G; its states, masked tiles and
+ * decayed rows are bf16 between the kernels (fp32 outputs within 2e-3).  All other calls, and those with
+ * SSD_FLAG_FORCE_SIMT, keep them in fp32.
  * Whether the tensor-core path is taken depends on the CUDA driver being present (it resolves the
  * tensor-map encoder at run time), so the answer is the one for the machine the query runs on. */
 size_t ssd_workspace_bytes(const ssd_shape_t *shape, int op);

@@ -103,7 +103,7 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
     if (seg % s->chunk) return SSD_EINVAL;
     if (s->x_bstride < 0 || s->dt_bstride < 0 || s->bc_bstride < 0) return SSD_EINVAL;
     pl.B = s->B; pl.L = s->L; pl.H = s->H; pl.P = s->P; pl.N = s->N; pl.G = s->G;
-    pl.use_tc = tc_supported(s->dtype, s->flags, s->P, s->N, s->chunk);
+    pl.use_tc = tc_supported(s->dtype, s->flags, s->P, s->N, s->chunk, s->H / s->G);
     pl.Q = pl.use_tc ? kTcBlock : s->chunk;
     pl.seg = seg;
     pl.nseg = (s->L + seg - 1) / seg;

@@ -50,7 +50,8 @@ template <auto K> inline cudaError_t allow_smem(int bytes) {
 
 constexpr int kNumSMs = 148;
 constexpr int kStatePassElems = 512;   // state elements per CTA of the CUDA-core state passes
-constexpr int kTcBlock = 128;     // steps per block of the tensor-core path, whatever (larger) chunk the caller names
+constexpr int kTcBlock = 128;     // steps per block of the tensor-core path, half the caller's chunk
+constexpr int kTcState = 128;     // its state size N
 
 // Per (head, block of 128 steps) record of the tensor-core path, made once per segment by the forward chain and copied to
 // shared memory in one piece by every kernel that masks a tile (cs: inclusive cumsum of dt*A in the block, log2 units;
@@ -166,7 +167,7 @@ struct TcMaps {
     CUtensorMap H, G;           // bf16 states as [rows][64], box 64 x N rows
     CUtensorMap Hst, Gst;       // the same for the stores of the chain kernels: box 32 x 32 rows, 64-byte swizzle
 };
-bool tc_supported(int dtype, int flags, int P, int N, int Q);
+bool tc_supported(int dtype, int flags, int P, int N, int chunk, int heads_per_group);
 bool tc_make_maps(const SegParams &p, TcMaps &m);
 bool tc_state_maps(const SegParams &p, TcMaps &m);
 // ssd_tc_chain.cu : block sums and the recurrence over the blocks.  init: state (gradient) entering the segment (NULL = zeros),

@@ -42,10 +42,14 @@ static bool make_map3(CUtensorMap *m, const void *ptr, uint64_t dim0, uint64_t d
                CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The kernels work on blocks of 128 steps, so a chunk of 64 (whose segments may be an odd number of them) is not theirs.
-bool tc_supported(int dtype, int flags, int P, int N, int Q) {
-    return dtype == SSD_DTYPE_BF16 && !(flags & SSD_FLAG_FORCE_SIMT) && P == 64 && (N == 64 || N == 128) && Q % kTcBlock == 0 &&
-           encode_fn() != nullptr;
+// The tensor-core kernels round decayed rows, masked tiles and states to bf16, so that a call's fp32 outputs (states, ddt, dA)
+// are within 2e-3 of the exact ones; the CUDA-core kernels keep all of it in fp32 (1e-6).  Which bf16 calls take which is
+// therefore part of what a caller gets: N = 64, chunks below 256 and odd numbers of heads per group have fp32 intermediates.
+// On the tensor cores, which could run them, 2 x 8192 steps of 32 heads with N = 64 took 378 us instead of 2250, and h_final was
+// off by 1.7e-3 instead of 8e-7, ddt by 2.1e-3 instead of 3e-7 (4096 of these steps).
+bool tc_supported(int dtype, int flags, int P, int N, int chunk, int heads_per_group) {
+    return dtype == SSD_DTYPE_BF16 && !(flags & SSD_FLAG_FORCE_SIMT) && P == 64 && N == kTcState && chunk == 2 * kTcBlock &&
+           heads_per_group % 2 == 0 && encode_fn() != nullptr;
 }
 
 // Builds the tensor maps of one API call.  x/dy/Bm/Cm may be null when the call does not use them.

@@ -1,4 +1,4 @@
-// Tensor-core kernel for dB and dC (bf16 I/O, P = 64, N = 64 or 128), over blocks of T = 128 steps.  Both are products of
+// Tensor-core kernel for dB and dC (bf16 I/O, P = 64, N = 128), over blocks of T = 128 steps.  Both are products of
 // the same masked, per-head score tile
 //     W_h[t,s] = (dy_t . x_s) e^{cs_t-cs_s} dt_s   (s <= t),
 //   dC_t = sum_h [ sum_s W_h[t,s] B_s + e^{cs_t} dy_t^T H_in ]
@@ -27,7 +27,7 @@ using namespace sm100;
 
 namespace {
 
-constexpr int GF_T = 128;
+constexpr int GF_T = kTcBlock, NS = kTcState;
 constexpr int GF_THREADS = 512;
 constexpr int GF_VECS = 3;                        // record buffers; the part used, from the decays to the row scales
 constexpr int GF_REC0 = REC_BLK, GF_VEC_FLOATS = REC_FLOATS - REC_BLK;
@@ -35,9 +35,9 @@ constexpr int GF_REC0 = REC_BLK, GF_VEC_FLOATS = REC_FLOATS - REC_BLK;
 // Ring of four 32 KB slots: the block's C rows, its B rows (N/64 x 16 KB each), then one head per slot (dy rows 16 KB | x rows
 // 16 KB), then C and B again for the last products | 2 x (H^T | G^T, N x 128 B), at the end the head sum
 constexpr uint32_t GF_OFF_ST = 4 * 32768;
-__host__ __device__ constexpr uint32_t gf_off_vec(int ns) { return GF_OFF_ST + 2 * 2 * (uint32_t)ns * 128; }
-__host__ __device__ constexpr uint32_t gf_off_part(int ns) { return gf_off_vec(ns) + GF_VECS * GF_VEC_FLOATS * 4; }
-__host__ __device__ constexpr uint32_t gf_smem(int ns) { return gf_off_part(ns) + 2 * 1024 * 4 + 1024; }
+constexpr uint32_t GF_OFF_VEC = GF_OFF_ST + 2 * 2 * (uint32_t)NS * 128;
+constexpr uint32_t GF_OFF_PART = GF_OFF_VEC + GF_VECS * GF_VEC_FLOATS * 4;
+constexpr uint32_t GF_SMEM = GF_OFF_PART + 2 * 1024 * 4 + 1024;
 
 constexpr uint32_t TF_ACCC = 256, TF_ACCB = 384;
 
@@ -54,7 +54,7 @@ __device__ __forceinline__ uint32_t pack2g(float a, float b) {
 }  // namespace
 
 // WHAT: BC_DC | BC_DB, or one of them (the cross-check with two launches)
-template <int NS, int WHAT>
+template <int WHAT>
 __global__ void __launch_bounds__(GF_THREADS, 1)
 k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmDy,
           const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmC, const __grid_constant__ CUtensorMap tmH,
@@ -77,9 +77,9 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
     const int q = warp & 3, sr = warp >> 2;         // tensor-memory quarter; column sub-tile
     const uint32_t tlane = (uint32_t)(q * 32) << 16;
     const int tok0 = p.t0 + c * GF_T;
-    unsigned char *vecs = smem + gf_off_vec(NS);
+    unsigned char *vecs = smem + GF_OFF_VEC;
     auto record = [&](int vb) { return reinterpret_cast<const float *>(vecs) + vb * GF_VEC_FLOATS - GF_REC0; };
-    float *parts = reinterpret_cast<float *>(smem + gf_off_part(NS));      // [head parity][rho: 4 sub-tiles x 128 | psi: 4 quarters x 128]
+    float *parts = reinterpret_cast<float *>(smem + GF_OFF_PART);      // [head parity][rho: 4 sub-tiles x 128 | psi: 4 quarters x 128]
 
     if (tid == 0) {
         for (int i = 0; i < 4; ++i) {
@@ -390,7 +390,7 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
     tc_fence_after_sync();
     constexpr int PITCH = NS + 4;
     float *stgC = reinterpret_cast<float *>(smem), *stgB = stgC + 128 * PITCH;
-    if (sr * 32 < NS) {
+    {
         float a[32];
         if (doC) {
             tmem_ld32(tm + tlane + TF_ACCC + sr * 32, a);
@@ -423,18 +423,18 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
     }
 }
 
-template <int NS, int WHAT>
+template <int WHAT>
 static cudaError_t launch_bc(const SegParams &p, const TcMaps &m, cudaStream_t st) {
-    const cudaError_t e = allow_smem<k_grad_bc<NS, WHAT>>((int)gf_smem(NS));
+    const cudaError_t e = allow_smem<k_grad_bc<WHAT>>((int)GF_SMEM);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_grad_bc<NS, WHAT>, dim3(p.nc * p.nsl * p.G * p.B), dim3(GF_THREADS), (size_t)gf_smem(NS), st, p, m.x, m.dy, m.Bm, m.Cm,
+    return launch_pdl(k_grad_bc<WHAT>, dim3(p.nc * p.nsl * p.G * p.B), dim3(GF_THREADS), (size_t)GF_SMEM, st, p, m.x, m.dy, m.Bm, m.Cm,
                       m.H, m.G);
 }
 
 cudaError_t launch_grad_bc(const SegParams &p, const TcMaps &m, int what, cudaStream_t st) {
-    if (what == BC_DC) return p.N == 128 ? launch_bc<128, BC_DC>(p, m, st) : launch_bc<64, BC_DC>(p, m, st);
-    if (what == BC_DB) return p.N == 128 ? launch_bc<128, BC_DB>(p, m, st) : launch_bc<64, BC_DB>(p, m, st);
-    return p.N == 128 ? launch_bc<128, BC_DC | BC_DB>(p, m, st) : launch_bc<64, BC_DC | BC_DB>(p, m, st);
+    if (what == BC_DC) return launch_bc<BC_DC>(p, m, st);
+    if (what == BC_DB) return launch_bc<BC_DB>(p, m, st);
+    return launch_bc<BC_DC | BC_DB>(p, m, st);
 }
 
 }  // namespace ssd

@@ -28,7 +28,7 @@ namespace {
 // heads per CTA: one, or in the forward two of the same group, which then share the block's B rows and a product of N = 128
 __host__ __device__ constexpr int ch_rec_warps(int heads) { return heads == 2 ? 4 : 2; }
 __host__ __device__ constexpr int ch_threads(int mode, int heads) { return 32 * (2 + ch_rec_warps(heads) + 8 + 8 * heads + (mode ? 4 : 0)); }
-constexpr int CH_T = 128;
+constexpr int CH_T = kTcBlock, NS = kTcState;
 __host__ __device__ constexpr int ch_stages(int mode, int heads) { return mode || heads == 2 ? 3 : 4; }
 // CHAIN_FWD: vector buffers per head (weights of 128 rows + the block's decay); for two heads the weights' bf16 pairs are packed
 // (a buffer belongs to one record warp: a warp that took buffers in turn with others could wait for a phase two ahead of the
@@ -39,18 +39,18 @@ constexpr float kLog2eC = 1.4426950408889634f;
 constexpr int CH_AHEAD = 4;               // L2 prefetch distance in blocks beyond the staged ones
 
 // stage: V (B or C rows) N/64 x 16 KB | X (x or dy rows) 16 KB per head | CHAIN_BWD: H_in^T, N rows of 128 B | row scales 1 KB, decay 16 B
-__host__ __device__ constexpr uint32_t ch_stage_bytes(int mode, int ns, int heads) {
-    return (uint32_t)ns * 256 + (uint32_t)heads * 16384 + (mode ? (uint32_t)ns * 128 + 2048 : 0);
+__host__ __device__ constexpr uint32_t ch_stage_bytes(int mode, int heads) {
+    return (uint32_t)NS * 256 + (uint32_t)heads * 16384 + (mode ? (uint32_t)NS * 128 + 2048 : 0);
 }
-__host__ __device__ constexpr uint32_t ch_off_vec(int mode, int ns, int heads) {
-    return ch_stages(mode, heads) * ch_stage_bytes(mode, ns, heads) + heads * 8 * 2048;
+__host__ __device__ constexpr uint32_t ch_off_vec(int mode, int heads) {
+    return ch_stages(mode, heads) * ch_stage_bytes(mode, heads) + heads * 8 * 2048;
 }
-__host__ __device__ constexpr uint32_t ch_off_bar(int mode, int ns, int heads) {
-    return ch_off_vec(mode, ns, heads) + (mode ? 0 : heads * ch_vec(heads) * ch_vec_floats(heads) * 4);
+__host__ __device__ constexpr uint32_t ch_off_bar(int mode, int heads) {
+    return ch_off_vec(mode, heads) + (mode ? 0 : heads * ch_vec(heads) * ch_vec_floats(heads) * 4);
 }
 // for the alignment of the stages: two heads leave no room for all of 1 KB, but no static shared memory is in front of them
 __host__ __device__ constexpr uint32_t ch_slack(int heads) { return heads == 2 ? 512 : 1024; }
-__host__ __device__ constexpr uint32_t ch_smem(int mode, int ns, int heads) { return ch_off_bar(mode, ns, heads) + 256 + ch_slack(heads); }
+__host__ __device__ constexpr uint32_t ch_smem(int mode, int heads) { return ch_off_bar(mode, heads) + 256 + ch_slack(heads); }
 
 __device__ __forceinline__ float ex2c(float x) {
     float y;
@@ -65,7 +65,7 @@ __device__ __forceinline__ float2 unpack2c(uint32_t w) { return __bfloat1622floa
 
 }  // namespace
 
-template <int NS, int MODE, int HEADS>
+template <int MODE, int HEADS>
 __global__ void __launch_bounds__(ch_threads(MODE, HEADS), 1)
 k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, long long bnd_bs, float *carry_out, float *final_out,
            const __grid_constant__ CUtensorMap tmX, const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmH,
@@ -75,8 +75,8 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     constexpr int CH_STAGES = ch_stages(MODE, HEADS), CH_VEC = ch_vec(HEADS), VEC_FLOATS = ch_vec_floats(HEADS), DECAY_AT = VEC_FLOATS - 4;
     static_assert(CH_VEC % (ch_rec_warps(HEADS) / HEADS) == 0, "a vector buffer belongs to one record warp");
     constexpr int SCALE0 = 2 + ch_rec_warps(HEADS), CARRY0 = SCALE0 + 8, RHO0 = CARRY0 + 8 * HEADS;      // first warps of the roles
-    constexpr uint32_t STAGE = ch_stage_bytes(MODE, NS, HEADS), OFF_X = NS * 256, OFF_H = OFF_X + HEADS * 16384, OFF_W = OFF_H + NS * 128;
-    constexpr uint32_t OFF_OUT = CH_STAGES * STAGE, OFF_VEC = ch_off_vec(MODE, NS, HEADS), OFF_BAR = ch_off_bar(MODE, NS, HEADS);
+    constexpr uint32_t STAGE = ch_stage_bytes(MODE, HEADS), OFF_X = NS * 256, OFF_H = OFF_X + HEADS * 16384, OFF_W = OFF_H + NS * 128;
+    constexpr uint32_t OFF_OUT = CH_STAGES * STAGE, OFF_VEC = ch_off_vec(MODE, HEADS), OFF_BAR = ch_off_bar(MODE, HEADS);
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     if ((uint32_t)(smem - smem_raw) > ch_slack(HEADS)) {        // the same for every CTA; not reached
@@ -162,8 +162,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
             for (int i = 0; i < nc; ++i) {
                 const int st = i % CH_STAGES, bf = i & 1;
                 const uint32_t sb = smem_u32(smem + st * STAGE);
-                // The sum as D[n][p]: V rows MN-major along n (for N = 64 the second 64 rows of the operand are whatever
-                // follows, the X tile; their lanes are not read), X rows MN-major along p
+                // The sum as D[n][p]: V rows MN-major along n, X rows MN-major along p
                 const uint64_t dV = umma_desc_sw128(sb, 16384, 1024), dX = umma_desc_sw128(sb + OFF_X, 16384, 1024);
                 const uint32_t loV = (uint32_t)dV, hiM = (uint32_t)(dV >> 32), loX = (uint32_t)dX, hiX = (uint32_t)(dX >> 32);
                 mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
@@ -346,7 +345,6 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
         // n = 32 q + lane, columns p = 32 half ..; as rows of time, t = 32 q + lane
         const int w = (warp - CARRY0) & 7, hl = (warp - CARRY0) >> 3, h = h0 + hl;
         const int q = warp & 3, half = w >> 2;
-        const bool act = q * 32 < NS;
         const uint32_t tl = tm + ((uint32_t)(q * 32) << 16) + hl * 64 + half * 32;
         const float *vec = reinterpret_cast<const float *>(smem + OFF_VEC) + hl * CH_VEC * VEC_FLOATS;
         unsigned char *stg = smem + OFF_OUT + (warp - CARRY0) * 2048, *row = stg + lane * 64;      // [32 rows][64 B], 64-byte swizzle
@@ -354,33 +352,31 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
         float carry[32];
         pdl_wait();                                // the carry that the previous segment's launch left; the earlier states have been read
 #pragma unroll
-        for (int j = 0; j < 32; ++j) carry[j] = init && act ? init[(size_t)b * init_bs + so + (size_t)j * NS] : 0.f;
-        if (bnd_out && act) {
+        for (int j = 0; j < 32; ++j) carry[j] = init ? init[(size_t)b * init_bs + so + (size_t)j * NS] : 0.f;
+        if (bnd_out) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) bnd_out[(size_t)b * bnd_bs + so + (size_t)j * NS] = carry[j];
         }
         for (int i = 0; i < nc; ++i) {
             const int st = i % CH_STAGES, bf = i & 1, c = chunk_of(i);
             // the carried state in bf16 (H entering block c, or the gradient leaving it) on its way out while the block's sum is made
-            if (act) {
-                if (lane == 0) tma_store_wait_read();
-                __syncwarp();
+            if (lane == 0) tma_store_wait_read();
+            __syncwarp();
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {
-                    const float *a = carry + ch * 8;
-                    *reinterpret_cast<uint4 *>(row + ((ch ^ ((lane >> 1) & 3)) << 4)) =
-                        make_uint4(pack2c(a[0], a[1]), pack2c(a[2], a[3]), pack2c(a[4], a[5]), pack2c(a[6], a[7]));
-                }
-                fence_proxy_async_smem();
-                __syncwarp();
-                if (lane == 0) {
-                    tma_store_3d(&tmOut, stg, half * 32, ((b * p.ncs + c) * p.H + h) * NS + q * 32, 0);
-                    tma_store_commit();
-                }
+            for (int ch = 0; ch < 4; ++ch) {
+                const float *a = carry + ch * 8;
+                *reinterpret_cast<uint4 *>(row + ((ch ^ ((lane >> 1) & 3)) << 4)) =
+                    make_uint4(pack2c(a[0], a[1]), pack2c(a[2], a[3]), pack2c(a[4], a[5]), pack2c(a[6], a[7]));
+            }
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) {
+                tma_store_3d(&tmOut, stg, half * 32, ((b * p.ncs + c) * p.H + h) * NS + q * 32, 0);
+                tma_store_commit();
             }
             if (BWD) mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);      // H_in and the decay have landed
             float2 dot = make_float2(0.f, 0.f);
-            if (BWD && act) {       // <G, H_in> over this thread's slice
+            if (BWD) {              // <G, H_in> over this thread's slice
                 const unsigned char *hr = smem + st * STAGE + OFF_H + (q * 32 + lane) * 128;
 #pragma unroll
                 for (int ch = 0; ch < 4; ++ch) {
@@ -395,20 +391,18 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
             tc_fence_after_sync();
             // (CHAIN_FWD: the scaling warps waited for the decay's buffer before the products could start)
             const float decay = BWD ? *reinterpret_cast<const float *>(smem + st * STAGE + OFF_W + 1024) : vec[(i % CH_VEC) * VEC_FLOATS + DECAY_AT];
-            if (act) {
-                const float2 dec2 = make_float2(decay, decay);
-                constexpr int PART = 32 / HEADS;          // two heads: 64 registers a thread
+            const float2 dec2 = make_float2(decay, decay);
+            constexpr int PART = 32 / HEADS;          // two heads: 64 registers a thread
 #pragma unroll
-                for (int c0 = 0; c0 < 32; c0 += PART) {
-                    float d[PART];
-                    if constexpr (HEADS == 2) tmem_ld16(tl + bf * 64 * HEADS + c0, d);
-                    else tmem_ld32(tl + bf * 64, d);
+            for (int c0 = 0; c0 < 32; c0 += PART) {
+                float d[PART];
+                if constexpr (HEADS == 2) tmem_ld16(tl + bf * 64 * HEADS + c0, d);
+                else tmem_ld32(tl + bf * 64, d);
 #pragma unroll
-                    for (int j = 0; j < PART; j += 2) {
-                        const float2 v = __ffma2_rn(dec2, make_float2(carry[c0 + j], carry[c0 + j + 1]), make_float2(d[j], d[j + 1]));
-                        carry[c0 + j] = v.x;
-                        carry[c0 + j + 1] = v.y;
-                    }
+                for (int j = 0; j < PART; j += 2) {
+                    const float2 v = __ffma2_rn(dec2, make_float2(carry[c0 + j], carry[c0 + j + 1]), make_float2(d[j], d[j + 1]));
+                    carry[c0 + j] = v.x;
+                    carry[c0 + j + 1] = v.y;
                 }
             }
             tc_fence_before_sync();
@@ -426,15 +420,13 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 if (lane == 0) p.ghdot[((((size_t)b * p.H + h) * p.ncs + c) << 4) + w] = decay * dt;
             }
         }
-        if (act) {
 #pragma unroll
-            for (int j = 0; j < 32; ++j) carry_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];
-            if (final_out) {
+        for (int j = 0; j < 32; ++j) carry_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];
+        if (final_out) {
 #pragma unroll
-                for (int j = 0; j < 32; ++j) final_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];
-            }
-            if (lane == 0) tma_store_wait_all();
+            for (int j = 0; j < 32; ++j) final_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];
         }
+        if (lane == 0) tma_store_wait_all();
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -444,30 +436,25 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     }
 }
 
-template <int NS, int MODE, int HEADS>
+template <int MODE, int HEADS>
 static cudaError_t launch_chain(const SegParams &p, const TcMaps &m, const float *init, long long init_bs, float *bnd_out, long long bnd_bs,
                                 float *carry_out, float *final_out, cudaStream_t st) {
-    constexpr uint32_t smem = ch_smem(MODE, NS, HEADS);
+    constexpr uint32_t smem = ch_smem(MODE, HEADS);
     static_assert(smem <= 232448, "shared memory of a CTA");
-    const cudaError_t e = allow_smem<k_chain_tc<NS, MODE, HEADS>>((int)smem);
+    const cudaError_t e = allow_smem<k_chain_tc<MODE, HEADS>>((int)smem);
     if (e != cudaSuccess) return e;
     const bool bwd = MODE == CHAIN_BWD;
-    return launch_pdl(k_chain_tc<NS, MODE, HEADS>, dim3(p.H / HEADS, p.B), dim3(ch_threads(MODE, HEADS)), (size_t)smem, st, p, init, init_bs, bnd_out,
+    return launch_pdl(k_chain_tc<MODE, HEADS>, dim3(p.H / HEADS, p.B), dim3(ch_threads(MODE, HEADS)), (size_t)smem, st, p, init, init_bs, bnd_out,
                       bnd_bs, carry_out, final_out, bwd ? m.dy : m.x, bwd ? m.Cm : m.Bm, m.H, bwd ? m.Gst : m.Hst);
 }
 
 cudaError_t launch_chain_fwd(const SegParams &p, const TcMaps &m, const float *init, long long init_bs, float *boundary_out, long long bnd_bs,
                              float *final_out, cudaStream_t st) {
-    if (p.chain_heads == 2)
-        return p.N == 128 ? launch_chain<128, CHAIN_FWD, 2>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st)
-                          : launch_chain<64, CHAIN_FWD, 2>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st);
-    return p.N == 128 ? launch_chain<128, CHAIN_FWD, 1>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st)
-                      : launch_chain<64, CHAIN_FWD, 1>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st);
+    if (p.chain_heads == 2) return launch_chain<CHAIN_FWD, 2>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st);
+    return launch_chain<CHAIN_FWD, 1>(p, m, init, init_bs, boundary_out, bnd_bs, p.hcarry, final_out, st);
 }
 cudaError_t launch_chain_bwd(const SegParams &p, const TcMaps &m, const float *init, float *left_out, cudaStream_t st) {
-    const long long bs = (long long)p.H * 64 * p.N;
-    return p.N == 128 ? launch_chain<128, CHAIN_BWD, 1>(p, m, init, bs, nullptr, 0, left_out, nullptr, st)
-                      : launch_chain<64, CHAIN_BWD, 1>(p, m, init, bs, nullptr, 0, left_out, nullptr, st);
+    return launch_chain<CHAIN_BWD, 1>(p, m, init, (long long)p.H * 64 * NS, nullptr, 0, left_out, nullptr, st);
 }
 
 }  // namespace ssd

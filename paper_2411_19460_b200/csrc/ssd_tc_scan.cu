@@ -1,5 +1,5 @@
 // Tensor-core kernel for the two masked products whose score matrix is shared by the heads of a group (bf16 I/O, P = 64,
-// N = 64 or 128), over blocks of T = 128 steps:
+// N = 128), over blocks of T = 128 steps:
 //
 //   SC_FWD: y_t  = sum_{s<=t} (C_t.B_s) e^{cs_t-cs_s} dt_s x_s + e^{cs_t} C_t H_in + D x_t
 //   SC_DX : u_s  = sum_{t>=s} (B_s.C_t) e^{cs_t-cs_s} dy_t      + e^{cs_last-cs_s} B_s Gout
@@ -41,7 +41,7 @@ using namespace sm100;
 
 namespace {
 
-constexpr int SC_T = 128;
+constexpr int SC_T = kTcBlock, NS = kTcState;
 constexpr int SC_THREADS = 28 * 32;
 // part of the record a stage holds: y from the decays to the column factors, dx from the dx column factors to the step sizes
 __host__ __device__ constexpr int sc_rec_first(int mode) { return mode == SC_DX ? (int)REC_CFX : (int)REC_BLK; }
@@ -50,11 +50,11 @@ static_assert(SC_REC_BYTES == (REC_CF - REC_CFX) * 4 && SC_REC_BYTES <= 2048, "b
 
 // rows operand N/64 x 16 KB | stages: value rows 16 KB, state N rows of 128 B (the columns operand fits one), record 2 KB |
 // SC_DX: ring of x rows, 16 KB each, which only the epilogue reads
-__host__ __device__ constexpr uint32_t sc_stage_bytes(int ns) { return 16384 + (uint32_t)ns * 128 + 2048; }
+constexpr uint32_t SC_STAGE = 16384 + (uint32_t)NS * 128 + 2048;
 __host__ __device__ constexpr int sc_stages(int mode) { return mode == SC_DX ? 4 : 5; }
 constexpr int SC_XR = 3;
-__host__ __device__ constexpr uint32_t sc_smem(int mode, int ns) {
-    return (uint32_t)ns * 256 + sc_stages(mode) * sc_stage_bytes(ns) + (mode == SC_DX ? SC_XR * 16384 : 0) + 1024;
+__host__ __device__ constexpr uint32_t sc_smem(int mode) {
+    return (uint32_t)NS * 256 + sc_stages(mode) * SC_STAGE + (mode == SC_DX ? SC_XR * 16384 : 0) + 1024;
 }
 
 constexpr float kLog2e = 1.4426950408889634f;
@@ -80,14 +80,14 @@ __device__ __forceinline__ void unpack8(const uint4 &q, float *f) {
 
 }  // namespace
 
-template <int NS, int MODE>
+template <int MODE>
 __global__ void __launch_bounds__(SC_THREADS, 1)
 k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_constant__ CUtensorMap tmCol,
           const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmSt, const __grid_constant__ CUtensorMap tmOut,
           const __grid_constant__ CUtensorMap tmXr) {
     constexpr bool FWD = MODE == SC_FWD;
     constexpr int NST = sc_stages(MODE);
-    constexpr uint32_t STAGE = sc_stage_bytes(NS), OFF_ST = 16384, OFF_REC = OFF_ST + NS * 128;
+    constexpr uint32_t STAGE = SC_STAGE, OFF_ST = 16384, OFF_REC = OFF_ST + NS * 128;
     constexpr uint32_t OFF_RING = NS * 256, OFF_XR = OFF_RING + NST * STAGE;
     constexpr int REC0 = sc_rec_first(MODE);
     // Of a mask group's eight warps (quarter q, column parity) the one whose two sub-tiles are zero idles
@@ -456,20 +456,19 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
     }
 }
 
-template <int NS, int MODE>
+template <int MODE>
 static cudaError_t launch_scan(const SegParams &p, const TcMaps &m, cudaStream_t st) {
-    constexpr uint32_t smem = sc_smem(MODE, NS);
-    cudaError_t e = allow_smem<k_scan_tc<NS, MODE>>((int)smem);
+    constexpr uint32_t smem = sc_smem(MODE);
+    cudaError_t e = allow_smem<k_scan_tc<MODE>>((int)smem);
     if (e != cudaSuccess) return e;
     const long long units = (long long)p.B * p.nc * p.H;
     const dim3 grid((unsigned)(units < p.scan_ctas ? units : p.scan_ctas));
-    if (MODE == SC_FWD) return launch_pdl(k_scan_tc<NS, MODE>, grid, dim3(SC_THREADS), (size_t)smem, st, p, m.Cm, m.Bm, m.x, m.H, m.y, m.x);
-    return launch_pdl(k_scan_tc<NS, MODE>, grid, dim3(SC_THREADS), (size_t)smem, st, p, m.Bm, m.Cm, m.dy, m.G, m.dx, m.x);
+    if (MODE == SC_FWD) return launch_pdl(k_scan_tc<MODE>, grid, dim3(SC_THREADS), (size_t)smem, st, p, m.Cm, m.Bm, m.x, m.H, m.y, m.x);
+    return launch_pdl(k_scan_tc<MODE>, grid, dim3(SC_THREADS), (size_t)smem, st, p, m.Bm, m.Cm, m.dy, m.G, m.dx, m.x);
 }
 
 cudaError_t launch_scan_tc(const SegParams &p, const TcMaps &m, int mode, cudaStream_t st) {
-    if (mode == SC_FWD) return p.N == 128 ? launch_scan<128, SC_FWD>(p, m, st) : launch_scan<64, SC_FWD>(p, m, st);
-    return p.N == 128 ? launch_scan<128, SC_DX>(p, m, st) : launch_scan<64, SC_DX>(p, m, st);
+    return mode == SC_FWD ? launch_scan<SC_FWD>(p, m, st) : launch_scan<SC_DX>(p, m, st);
 }
 
 }  // namespace ssd

@@ -1,7 +1,8 @@
-"""The edges of what a launch covers, against the fp64 oracle: blocks of 128 steps on the tensor-core path (one block, odd
-numbers of blocks and heads, N = 64 and 128, five and more segments so that every scratch copy is used twice, stiff and mild
-decays, head ranges of dB/dC, one and two heads per CTA of the forward chain), and CUDA-core launches that carry the sums of the neighbouring segment (one segment, two, a short
-last one, one 64-step tile per chunk and four).  In order on one stream the same bits come out."""
+"""The edges of what a launch covers, against the fp64 oracle: blocks of 128 steps on the tensor-core path (chunks of 256, N = 128,
+an even number of heads per group: one chunk, two heads, five and more segments so that every scratch copy is used twice, a
+short last segment, stiff and mild decays, head ranges of dB/dC, one and two heads per CTA of the forward chain), and CUDA-core
+launches that carry the sums of the neighbouring segment (one segment, two, a short last one, one 64-step tile per chunk and
+four, both state sizes, odd numbers of heads, both dtypes).  In order on one stream the same bits come out."""
 import pytest
 import torch
 
@@ -21,7 +22,13 @@ STIFF = dict(a_max=64.0, dt_lo=1e-4, dt_hi=1.0)
     ("bf16", 1792, 6, 2, 128, 256, 256, STIFF),
     ("bf16", 768, 9, 1, 64, 128, 128, dict(B=2)),
     ("bf16", 1024, 20, 1, 128, 256, 512, {}),
-    ("bf16", 1152, 76, 2, 128, 128, 256, {}),          # two heads per CTA of the forward chain
+    ("bf16", 256, 2, 1, 128, 256, 256, {}),
+    ("bf16", 1792, 12, 2, 128, 256, 256, STIFF),
+    ("bf16", 2304, 6, 3, 128, 256, 512, dict(B=2)),
+    ("bf16", 1280, 76, 2, 128, 256, 256, {}),          # two heads per CTA of the forward chain
+    ("bf16", 1280, 76, 1, 128, 256, 256, STIFF),
+    ("bf16", 768, 76, 1, 128, 256, 768, dict(B=2)),
+    ("bf16", 1152, 76, 2, 128, 128, 256, {}),
     ("bf16", 640, 76, 1, 64, 128, 128, STIFF),
     ("bf16", 384, 76, 1, 128, 128, 384, dict(B=2)),
     ("fp32", 64, 1, 1, 64, 64, 64, {}),
