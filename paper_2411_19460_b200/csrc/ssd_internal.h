@@ -107,7 +107,7 @@ struct SegParams {
     float *hcarry;         // [B,H,P,N]     state handed from segment to segment (forward)
     float *gcarry;         // [B,H,P,N]     state gradient handed right-to-left (backward)
     float *ghdot;          // [B,H,ncs,16]  partial sums of exp(cs_last) <Gout_c, H_in,c>
-    float *ddt_dir;        // [B,H,ncs,Q]   direct part of ddt
+    float *ddt_dir;        // [B,H,ncs,Q]   direct part of ddt (tensor-core path: read where dt is next to zero, see bwd_finish)
     float *cbt;            // CUDA-core path: [B,ncs,G,Q,Q] C B^T, causal 64 x 64 tiles
     float *rho;            // [B,H,ncs,Q]   C_t . (intra-chunk part of this head's dC_t); CUDA-core path: [B,H,ncs,tiles,Q] by column tile
     float *rho2;           // [B,H,ncs,Q]   C_t . (inter-chunk part of this head's dC_t)

@@ -371,6 +371,8 @@ __device__ __forceinline__ RowScale row_scale(float s) {
     const __nv_bfloat162 h2 = __halves2bfloat162(h, h), l2 = __halves2bfloat162(l, l);
     return {*reinterpret_cast<const uint32_t *>(&h2), *reinterpret_cast<const uint32_t *>(&l2)};
 }
+// the factor itself, to 2^-17
+__device__ __forceinline__ float row_scale_value(const RowScale &s) { return __uint_as_float(s.hi << 16) + __uint_as_float(s.lo << 16); }
 __device__ __forceinline__ uint32_t scale2(uint32_t x, const RowScale &s) {
     const __nv_bfloat162 v = *reinterpret_cast<const __nv_bfloat162 *>(&x);
     const __nv_bfloat162 r = __hfma2(v, *reinterpret_cast<const __nv_bfloat162 *>(&s.hi), __hmul2(v, *reinterpret_cast<const __nv_bfloat162 *>(&s.lo)));

@@ -5,6 +5,10 @@
 //   CHAIN_BWD: G_{c-1} = e^{cs_last} G_c + sum_t e^{cs_t} dy_t C_t^T                 (G_c: gradient leaving block c)
 //              rho2_t  = e^{cs_t} dy_t . (H_in C_t),   <G,H> partials = e^{cs_last} <G_c, H_in,c>
 //
+// rho2 goes into ddt and dA by suffix sums, so its dy rows are the ones before scaling and rounding: a product of their own ahead
+// of the block's sum, and the scaling warps wait until the rows have been read.  With the scaled rows ddt was 4 to 10 % further
+// from the exact one than with blocks of 256 steps; the order costs the backward 2 us of 51.6 (4096 steps of 80 heads).
+//
 // One CTA owns one (batch, head), or in the forward two heads of a group, and walks the segment's blocks.  A block's sum does not depend on the carried state, so
 // it is made by tcgen05 one block ahead; the carry (N x 64 fp32) never leaves the registers of the eight worker warps:
 // what is written per block is its bf16 copy, the operand of the large kernels, 16 KB, where separate kernels for the
@@ -86,6 +90,8 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     uint64_t *const full = reinterpret_cast<uint64_t *>(smem + OFF_BAR), *const scaled = full + CH_STAGES, *const empty = scaled + CH_STAGES;
     uint64_t *const mdone = empty + CH_STAGES, *const dempty = mdone + 2, *const vfull = dempty + 2, *const vempty = vfull + HEADS * CH_VEC;
     uint32_t *const words = reinterpret_cast<uint32_t *>(vempty + HEADS * CH_VEC);
+    // CHAIN_BWD has no vector buffers; in their barriers' place: H_in C made, read; the stage's rows read for rho2
+    uint64_t *const ydone = vfull, *const yempty = vfull + 2, *const rowread = vempty;
     static_assert((3 * CH_STAGES + 4 + 2 * HEADS * CH_VEC) * 8 + 8 <= 256, "barriers");
 
     const int h0 = blockIdx.x * HEADS, b = blockIdx.y, g = h0 / p.hpg, nc = p.nc;
@@ -95,15 +101,15 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
         for (int i = 0; i < CH_STAGES; ++i) {
             mbar_init(&full[i], 1);
             mbar_init(&scaled[i], 8);
-            mbar_init(&empty[i], BWD ? 8 + 4 : 1); // BWD: the carry and rho2 warps read the stage last; FWD: the MMAs do
+            mbar_init(&empty[i], BWD ? 8 : 1);     // BWD: the carry warps read the stage last; FWD: the MMAs do
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(&mdone[i], 1);
-            mbar_init(&dempty[i], BWD ? 8 + 4 : 8 * HEADS);
+            mbar_init(&dempty[i], 8 * HEADS);
         }
         for (int i = 0; i < HEADS * CH_VEC; ++i) {
-            mbar_init(&vfull[i], 1);
-            mbar_init(&vempty[i], 8);              // the carry warps, which read the decay last
+            mbar_init(&vfull[i], BWD && i >= 2 ? 4 : 1);
+            mbar_init(&vempty[i], BWD ? 4 : 8);    // the carry warps, which read the decay last
         }
         words[1] = 0;
         fence_barrier_init();
@@ -166,6 +172,19 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 const uint64_t dV = umma_desc_sw128(sb, 16384, 1024), dX = umma_desc_sw128(sb + OFF_X, 16384, 1024);
                 const uint32_t loV = (uint32_t)dV, hiM = (uint32_t)(dV >> 32), loX = (uint32_t)dX, hiX = (uint32_t)(dX >> 32);
                 mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
+                if (BWD) {   // Y[t][p] = sum_n C[t][n] H_in[p][n], for rho2
+                    const uint64_t dC = umma_desc_sw128(sb, 16, 1024), dH = umma_desc_sw128(sb + OFF_H, 8192, 1024);
+                    const uint32_t loC = (uint32_t)dC, hiC = (uint32_t)(dC >> 32), loH = (uint32_t)dH, hiH = (uint32_t)(dH >> 32);
+                    if (i >= 2) mbar_wait(&yempty[bf], ((i >> 1) - 1) & 1, abortp, p.status);
+                    tc_fence_after_sync();
+#pragma unroll
+                    for (int k = 0; k < NS / 16; ++k) {
+                        const uint64_t ad = umma_desc_words(loC + (k >> 2) * 1024 + (k & 3) * 2, hiC), bd = umma_desc_words(loH + k * 128, hiH);
+                        if (k == 0) umma_bf16_fixed<false>(tm + 128 + bf * 64, ad, bd, idY);
+                        else umma_bf16_fixed<true>(tm + 128 + bf * 64, ad, bd, idY);
+                    }
+                    umma_commit(&ydone[bf]);
+                }
                 mbar_wait(&scaled[st], (i / CH_STAGES) & 1, abortp, p.status);
                 if (i >= 2) mbar_wait(&dempty[bf], ((i >> 1) - 1) & 1, abortp, p.status);
                 tc_fence_after_sync();
@@ -174,16 +193,6 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                     const uint64_t ad = umma_desc_words(loV + k * 128, hiM), bd = umma_desc_words(loX + k * 128, hiX);
                     if (k == 0) umma_bf16_fixed<false>(tm + bf * 64 * HEADS, ad, bd, idD);
                     else umma_bf16_fixed<true>(tm + bf * 64 * HEADS, ad, bd, idD);
-                }
-                if (BWD) {   // Y[t][p] = sum_n C[t][n] H_in[p][n]
-                    const uint64_t dC = umma_desc_sw128(sb, 16, 1024), dH = umma_desc_sw128(sb + OFF_H, 8192, 1024);
-                    const uint32_t loC = (uint32_t)dC, hiC = (uint32_t)(dC >> 32), loH = (uint32_t)dH, hiH = (uint32_t)(dH >> 32);
-#pragma unroll
-                    for (int k = 0; k < NS / 16; ++k) {
-                        const uint64_t ad = umma_desc_words(loC + (k >> 2) * 1024 + (k & 3) * 2, hiC), bd = umma_desc_words(loH + k * 128, hiH);
-                        if (k == 0) umma_bf16_fixed<false>(tm + 128 + bf * 64, ad, bd, idY);
-                        else umma_bf16_fixed<true>(tm + 128 + bf * 64, ad, bd, idY);
-                    }
                 }
                 if (!BWD) umma_commit(&empty[st]);
                 umma_commit(&mdone[bf]);
@@ -298,6 +307,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                         f[k] = reinterpret_cast<const RowScale *>(w)[r];
                     }
                 }
+                if (BWD) mbar_wait(&rowread[st], (i / CH_STAGES) & 1, abortp, p.status);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
                     scale8(v[k], f[k]);
@@ -309,36 +319,41 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
             if (lane == 0) mbar_arrive(&scaled[st]);
         }
     } else if (BWD && warp >= RHO0) {
-        // ------------------------------------------------------------ rho2: row dot of the scaled dy row and H_in C, t = 32 q + lane
+        // ------------------------------------------------------------ rho2: row dot of the dy row and H_in C, t = 32 q + lane.
+        // The row is read before it is scaled and rounded, its factor multiplies the sum; the product needs no scaled rows and
+        // is made ahead of the block's sum.
         const int q = warp & 3, r = q * 32 + lane;
         pdl_wait();
         for (int i = 0; i < nc; ++i) {
             const int st = i % CH_STAGES, bf = i & 1, c = chunk_of(i);
-            const unsigned char *dr = smem + st * STAGE + OFF_X + r * 128;
-            mbar_wait(&mdone[bf], (i >> 1) & 1, abortp, p.status);
+            const unsigned char *sb = smem + st * STAGE, *dr = sb + OFF_X + r * 128;
+            mbar_wait(&full[st], (i / CH_STAGES) & 1, abortp, p.status);
+            uint4 dv[8];
+#pragma unroll
+            for (int ch = 0; ch < 8; ++ch) dv[ch] = *reinterpret_cast<const uint4 *>(dr + ((ch ^ (r & 7)) << 4));
+            const RowScale f = reinterpret_cast<const RowScale *>(sb + OFF_W)[r];
+            fence_proxy_async_smem();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&rowread[st]);
+            mbar_wait(&ydone[bf], (i >> 1) & 1, abortp, p.status);
             __syncwarp();
             tc_fence_after_sync();
             float2 acc = make_float2(0.f, 0.f);
 #pragma unroll
-            for (int hf = 0; hf < 2; ++hf) {
-                float d[32];
-                tmem_ld32(tm + ((uint32_t)(q * 32) << 16) + 128 + bf * 64 + hf * 32, d);
+            for (int part = 0; part < 4; ++part) {
+                float d[16];
+                tmem_ld16(tm + ((uint32_t)(q * 32) << 16) + 128 + bf * 64 + part * 16, d);
 #pragma unroll
-                for (int ch = 0; ch < 4; ++ch) {
-                    const uint4 dv = *reinterpret_cast<const uint4 *>(dr + (((hf * 4 + ch) ^ (r & 7)) << 4));
-                    const uint32_t *e = reinterpret_cast<const uint32_t *>(&dv);
+                for (int ch = 0; ch < 2; ++ch) {
+                    const uint32_t *e = reinterpret_cast<const uint32_t *>(&dv[part * 2 + ch]);
 #pragma unroll
                     for (int m = 0; m < 4; ++m) acc = __ffma2_rn(unpack2c(e[m]), make_float2(d[ch * 8 + 2 * m], d[ch * 8 + 2 * m + 1]), acc);
                 }
             }
             tc_fence_before_sync();
-            fence_proxy_async_smem();      // the row has been read before a TMA load may overwrite it
             __syncwarp();
-            if (lane == 0) {
-                mbar_arrive(&dempty[bf]);
-                mbar_arrive(&empty[st]);
-            }
-            p.rho2[(((size_t)b * p.H + h0) * p.ncs + c) * CH_T + r] = acc.x + acc.y;
+            if (lane == 0) mbar_arrive(&yempty[bf]);
+            p.rho2[(((size_t)b * p.H + h0) * p.ncs + c) * CH_T + r] = row_scale_value(f) * (acc.x + acc.y);
         }
     } else {
         // ------------------------------------------------------------ carry: warp (q, half) holds state rows

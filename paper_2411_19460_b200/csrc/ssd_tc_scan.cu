@@ -5,6 +5,7 @@
 //   SC_DX : u_s  = sum_{t>=s} (B_s.C_t) e^{cs_t-cs_s} dy_t      + e^{cs_last-cs_s} B_s Gout
 //                   dx_s = D dy_s + dt_s u_s ;  ddt_direct_s = x_s . u_s ;  dD partial = sum dy.x ;
 //                   psi2_s = dt_s e^{cs_last-cs_s} x_s . (Gout B_s)   (inter-block part of B_s . dB_s)
+//                   (ddt_direct carries the masked tile's rounding; the finishing step has a better one unless dt_s is zero)
 //
 // (Eq. 1 of the paper regrouped by blocks; cs = inclusive cumsum of dt*A inside the block.)
 //
