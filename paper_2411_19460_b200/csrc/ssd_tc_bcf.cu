@@ -4,7 +4,7 @@
 //   dC_t = sum_h [ sum_s W_h[t,s] B_s + e^{cs_t} dy_t^T H_in ]
 //   dB_s = sum_h [ sum_t W_h[t,s] C_t + dt_s e^{cs_last-cs_s} x_s^T Gout ]
 // and both are linear in it, so a CTA, which owns (block, group, a range of the group's heads), masks the tile once per
-// head, adds it to a head sum kept in fp32 registers, and after the last head rounds the sum once and multiplies it by B
+// head, adds it to a head sum kept in fp32 registers, and after the last head multiplies the sum, as two bf16 parts, by B
 // and by C.  Per head it also forms the scalars of the decay gradient, rho_t = sum_s W[t,s] (C_t.B_s) and
 // psi_s = sum_t W[t,s] (C_t.B_s): row and column sums of one fp32 matrix.  (Eq. 1 of the paper regrouped by blocks; cs =
 // inclusive cumsum of dt*A inside the block.)
@@ -16,7 +16,9 @@
 //   warp 4 producer (TMA) | warp 8 MMA issuer | warp 12 rho / psi out | warps 9, 13, 14 row scaling
 // Tensor memory: two score buffers and the two accumulators, 128 columns each.  The rows of a head are scaled in place for
 // the inter-block terms once its scores have been multiplied, and both terms go straight into the accumulators.
-// Bound by the instruction issue of the scheduler that holds the four sub-tiles of row quarter 3.  4096 steps of 80 heads: 78 us
+// The head sum's second part takes dB from 2.42e-3 to 1.81e-3 of the exact one and dC from 2.64e-3 to 2.36e-3 (bf16 outputs: 1.66e-3;
+// 256-step blocks with one part: 2.39e-3, 2.62e-3) for 1.2 us of 76 (4096 steps of 80 heads, 96 CTAs).
+// Bound by the instruction issue of the scheduler that holds the four sub-tiles of row quarter 3.  4096 steps of 80 heads: 77 us
 // on 64 SMs (48 % of their issue slots), 94 us on 144 before, with 256-step chunks as three tiles.
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
@@ -33,11 +35,14 @@ constexpr int GF_VECS = 3;                        // record buffers; the part us
 constexpr int GF_REC0 = REC_BLK, GF_VEC_FLOATS = REC_FLOATS - REC_BLK;
 
 // Ring of four 32 KB slots: the block's C rows, its B rows (N/64 x 16 KB each), then one head per slot (dy rows 16 KB | x rows
-// 16 KB), then C and B again for the last products | 2 x (H^T | G^T, N x 128 B), at the end the head sum
+// 16 KB), then C and B again for the last products | 2 x (H^T | G^T, N x 128 B), at the end the two parts of the head sum
 constexpr uint32_t GF_OFF_ST = 4 * 32768;
 constexpr uint32_t GF_OFF_VEC = GF_OFF_ST + 2 * 2 * (uint32_t)NS * 128;
 constexpr uint32_t GF_OFF_PART = GF_OFF_VEC + GF_VECS * GF_VEC_FLOATS * 4;
 constexpr uint32_t GF_SMEM = GF_OFF_PART + 2 * 1024 * 4 + 1024;
+
+constexpr uint32_t GF_WPART = 128 * 256;          // a part of the head sum
+static_assert(2 * GF_WPART <= GF_OFF_VEC - GF_OFF_ST, "the head sum in the states' place");
 
 constexpr uint32_t TF_ACCC = 256, TF_ACCB = 384;
 
@@ -219,13 +224,18 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
             mbar_wait(&wfull, 0, abortp, p.status);
             tc_fence_after_sync();
 #pragma unroll
-            for (int k = 0; k < 8; ++k)       // dC += Wsum B, K = s
-                if (doC)
-                    umma_bf16_fixed<true>(tm + TF_ACCC, umma_desc_words(loWk + (k >> 2) * 1024 + (k & 3) * 2, hiK), umma_desc_words(loBe + k * 128, hiM), idC);
+            for (int part = 0; part < 2; ++part) {
+                const uint32_t o = part * (GF_WPART / 16);
 #pragma unroll
-            for (int k = 0; k < 8; ++k)       // dB += Wsum^T C, K = t
-                if (doB)
-                    umma_bf16_fixed<true>(tm + TF_ACCB, umma_desc_words(loWm + k * 128, hiM), umma_desc_words(loCe + k * 128, hiM), idB);
+                for (int k = 0; k < 8; ++k)       // dC += Wsum B, K = s
+                    if (doC)
+                        umma_bf16_fixed<true>(tm + TF_ACCC, umma_desc_words(loWk + o + (k >> 2) * 1024 + (k & 3) * 2, hiK),
+                                              umma_desc_words(loBe + k * 128, hiM), idC);
+#pragma unroll
+                for (int k = 0; k < 8; ++k)       // dB += Wsum^T C, K = t
+                    if (doB)
+                        umma_bf16_fixed<true>(tm + TF_ACCB, umma_desc_words(loWm + o + k * 128, hiM), umma_desc_words(loCe + k * 128, hiM), idB);
+            }
             umma_commit(&accfull);
         }
     } else if (warp == 12) {
@@ -362,16 +372,24 @@ k_grad_bc(SegParams p, const __grid_constant__ CUtensorMap tmX, const __grid_con
                 mbar_arrive(&pfull[hi & 1]);
             }
         }
-        // the head sum, rounded once to bf16: [s-half][128 rows t][128 B], zeros above the diagonal
+        // the head sum in two bf16 parts, what the first one's rounding leaves in the second: [part][s-half][128 rows t][128 B],
+        // zeros above the diagonal
         mbar_wait(&stdone, 0, abortp, p.status);
         auto put = [&](int j, bool zero) {
             unsigned char *row = smem + OFF_ST + (j >> 1) * 16384 + rl * 128;
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {
-                const float *a = wsum + ch * 8;
-                const uint4 w = zero ? make_uint4(0u, 0u, 0u, 0u)
-                                     : make_uint4(pack2g(a[0], a[1]), pack2g(a[2], a[3]), pack2g(a[4], a[5]), pack2g(a[6], a[7]));
-                *reinterpret_cast<uint4 *>(row + ((((j & 1) * 4 + ch) ^ (rl & 7)) << 4)) = w;
+                uint32_t w[2][4];
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float a = wsum[ch * 8 + 2 * m], b = wsum[ch * 8 + 2 * m + 1];
+                    w[0][m] = zero ? 0u : pack2g(a, b);
+                    w[1][m] = zero ? 0u : pack2g(a - __uint_as_float(w[0][m] << 16), b - __uint_as_float(w[0][m] & 0xffff0000u));
+                }
+                const uint32_t o = (((j & 1) * 4 + ch) ^ (rl & 7)) << 4;
+#pragma unroll
+                for (int part = 0; part < 2; ++part)
+                    *reinterpret_cast<uint4 *>(row + part * GF_WPART + o) = make_uint4(w[part][0], w[part][1], w[part][2], w[part][3]);
             }
         };
         put(sr, false);

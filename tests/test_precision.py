@@ -33,9 +33,10 @@ def test_fp32_outputs_of_shapes_with_fp32_intermediates(L, H, N, G, chunk, seg):
     assert max(errs.values()) <= pu.TOL["fp32"], errs
 
 
-def rounded_algebra_ddt(i, T=128):
-    """ddt with the roundings that the tensor-core path cannot do without, in fp64 otherwise: bf16 states (where they meet dy, x and
-    the other state) and bf16 decayed rows in the state sums.  Everything between two steps of one block is exact.  B = G = 1."""
+def rounded_algebra(i, T=128):
+    """ddt, dB and dC with the roundings that the tensor-core path cannot do without, in fp64 otherwise: bf16 states (where they meet
+    dy, x and the other state), bf16 decayed rows where they meet a state or make a state sum, bf16 dB and dC.  Everything between
+    two steps of one block is exact.  B = G = 1."""
     def bf(v):
         return v.float().bfloat16().double()
 
@@ -50,12 +51,13 @@ def rounded_algebra_ddt(i, T=128):
         states.append(h)
         w = torch.exp(cs[:, c, -1:] - cs[:, c]) * dt[:, s]
         h = torch.exp(cs[:, c, -1])[:, None, None] * h + torch.einsum("hsp,sn->hpn", bf(x[:, s] * w[..., None]), Bm[s])
-    ddt, g = torch.empty_like(dt), i["dh_final"][0]
+    ddt, dB, dC, g = torch.empty_like(dt), torch.empty_like(Bm), torch.empty_like(Cm), i["dh_final"][0]
     causal = torch.tril(torch.ones(T, T, dtype=torch.bool, device=x.device))
     for c in reversed(range(L // T)):
         s, k = slice(c * T, (c + 1) * T), cs[:, c]
         mask = torch.exp((k[:, :, None] - k[:, None, :]).masked_fill(~causal, -1e9))
-        z = torch.einsum("htp,hsp->hts", dy[:, s], x[:, s]) * mask * (Cm[s] @ Bm[s].T)
+        wd = torch.einsum("htp,hsp->hts", dy[:, s], x[:, s]) * mask
+        z = wd * (Cm[s] @ Bm[s].T)
         rho2 = torch.einsum("htp,hpn,tn->ht", dy[:, s] * torch.exp(k)[..., None], bf(states[c]), Cm[s])
         inter = torch.exp(k[:, -1:] - k) * torch.einsum("hsp,hpn,sn->hs", x[:, s], bf(g), Bm[s])
         gh = torch.exp(k[:, -1]) * (g * bf(states[c])).sum((1, 2))
@@ -63,24 +65,29 @@ def rounded_algebra_ddt(i, T=128):
         psi2 = dt[:, s] * inter
         da = right.flip(-1).cumsum(-1).flip(-1) + psi2.cumsum(-1) - psi2 + gh[:, None]
         ddt[:, s] = z.sum(1) + inter + A[:, None] * da
-        g = torch.exp(k[:, -1])[:, None, None] * g + torch.einsum("htp,tn->hpn", bf(dy[:, s] * torch.exp(k)[..., None]), Cm[s])
-    return ddt.T[None]
+        dyd, xd = bf(dy[:, s] * torch.exp(k)[..., None]), bf(x[:, s] * (torch.exp(k[:, -1:] - k) * dt[:, s])[..., None])
+        wsum = (wd * dt[:, None, s]).sum(0)
+        dC[s] = wsum @ Bm[s] + torch.einsum("htp,hpn->tn", dyd, bf(states[c]))
+        dB[s] = wsum.T @ Cm[s] + torch.einsum("hsp,hpn->sn", xd, bf(g))
+        g = torch.exp(k[:, -1])[:, None, None] * g + torch.einsum("htp,tn->hpn", dyd, Cm[s])
+    return dict(ddt=ddt.T[None], dB=bf(dB)[None, :, None], dC=bf(dC)[None, :, None])
 
 
 @pytest.mark.parametrize("extra", [{}, dict(a_max=64.0, dt_lo=1e-4, dt_hi=1.0)], ids=["mild", "stiff"])
-def test_ddt_of_the_tensor_core_path_has_only_the_states_roundings(extra):
-    """Masked tiles and decayed rows rounded to bf16 stay out of ddt: head by head, its error is that of the algebra above
-    (a rounding differs from the kernels' where an fp32 sum falls on the other side: 10 % for that and for fp32 itself)."""
+def test_gradients_of_the_tensor_core_path_have_only_the_states_roundings(extra):
+    """Masked tiles rounded to bf16 stay out of ddt, dB and dC: their errors, of ddt head by head, are those of the algebra above (a
+    rounding differs from the kernels' where an fp32 sum falls on the other side: 10 % for that and for fp32 itself)."""
     cfg = config(2048, 16, 128, 1, 256, 512, **extra)
-    worst = []
+    errs = {k: [0.0, 0.0] for k in ("ddt", "dB", "dC")}
     for seed in (1, 2):
         inp = make_inputs(cfg, "cuda", seed=seed)
-        ref = torch.from_numpy(pu.run_oracle(to_f64_numpy(inp), cfg.seg)["ddt"]).cuda()
-        got = pu.run_gpu(cfg, inp)["ddt"].double()
-        err = [((v - ref).norm(dim=1) / ref.norm(dim=1)).pow(2).mean().sqrt().item() for v in (got, rounded_algebra_ddt(inp))]
-        worst.append(err)
-    gpu, algebra = (sum(e[j] ** 2 for e in worst) ** 0.5 for j in (0, 1))
-    assert gpu <= 1.1 * algebra, worst
+        ref, got, algebra = pu.run_oracle(to_f64_numpy(inp), cfg.seg), pu.run_gpu(cfg, inp), rounded_algebra(inp)
+        for k, e in errs.items():
+            r = torch.from_numpy(ref[k]).cuda()
+            for j, v in enumerate((got[k].double(), algebra[k])):
+                e[j] += ((v - r).norm(dim=1) / r.norm(dim=1)).pow(2).mean().item()
+    assert all(gpu <= 1.1 ** 2 * alg for gpu, alg in errs.values()), errs
+    print(errs)
 
 
 @pytest.mark.parametrize("flags", [0, libssd.SSD_FLAG_FORCE_SIMT])
