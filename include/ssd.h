@@ -139,9 +139,12 @@ int ssd_fwd(const ssd_shape_t *shape, const void *x, const float *dt, const floa
  *
  * Same arguments and results as ssd_fwd (bit-identical outputs), minus ws / ws_bytes.
  *  - Every kernel runs in order on `stream`, so the scratch is laid out as for SSD_FLAG_SERIAL (no
- *    second copies).  Returns SSD_ETOOLARGE, with nothing enqueued, when that layout --
- *    ssd_workspace_bytes(shape with SSD_FLAG_SERIAL set, SSD_OP_FWD) -- exceeds SSD_STATIC_WS_BYTES:
- *    shrink `seg` (scratch grows with seg/chunk, not with L) or use ssd_fwd with your own buffer.
+ *    second copies).  Returns SSD_ETOOLARGE, with nothing enqueued, when that layout exceeds
+ *    SSD_STATIC_WS_BYTES: shrink `seg` (scratch grows with seg/chunk, not with L) or use ssd_fwd with your
+ *    own buffer.  Tensor-core path: ssd_workspace_bytes(shape with SSD_FLAG_SERIAL set, SSD_OP_FWD) bytes.
+ *    CUDA-core path: 256 + 8 B H seg + 4 B H P N (seg/chunk + 2) bytes, each part rounded up to 256; that is
+ *    ssd_workspace_bytes without the products C B^T (4 B G chunk seg bytes), which the kernels make again
+ *    where they do not fit.
  *  - The first call on each device looks up the device address of the built-in array (with that
  *    device current).  Make that first call outside any CUDA stream capture.
  *  - All calls on one device share the one array, and it keeps whatever the previous call left

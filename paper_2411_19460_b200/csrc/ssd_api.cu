@@ -63,6 +63,7 @@ static const int kMinSegmentsForTwins = 4;
 struct Plan {
     int B, L, H, P, N, G, Q, seg, nseg, ncs, nct, hpg, nsl, dtype;   // Q: steps per chunk (CUDA cores) or block (tensor cores)
     bool use_tc, serial;
+    bool keep_cb;          // CUDA cores: the scratch holds C B^T (always, except in the built-in one)
     int64_t x_bs, dt_bs, bc_bs;
     size_t esz;
 };
@@ -122,6 +123,7 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
         ((size_t)pl.x_bs * pl.esz) % 16 || ((size_t)pl.bc_bs * pl.esz) % 16)
         return SSD_EALIGN;
     pl.serial = (s->flags & SSD_FLAG_SERIAL) != 0;
+    pl.keep_cb = true;
     // Partial slices of the dB/dC head sums: one per CTA head range; on the CUDA-core path ranges of four heads (two where there
     // are few), each with a slot per 64-step tile and one for the inter-chunk term.
     const int per_range = pl.hpg >= 16 ? 4 : 2;
@@ -163,7 +165,7 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
         take2(lo.cs, vec, two && !bwd);
         take2(lo.dtT, vec, two);
         take2(lo.Hst, st, two && !bwd);
-        take2(lo.cbt, (size_t)pl.B * pl.ncs * pl.G * pl.Q * pl.Q * sizeof(float), two && !bwd);
+        if (pl.keep_cb) take2(lo.cbt, (size_t)pl.B * pl.ncs * pl.G * pl.Q * pl.Q * sizeof(float), two && !bwd);
     }
     if (bwd) {
         lo.gcarry = take(BH * PN * sizeof(float));
@@ -184,6 +186,15 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
         lo.dDp = take(BH * pl.nct * 4 * sizeof(float));
     }
     lo.total = o;
+}
+
+// Layout of the built-in scratch: in order on one stream, so no second copies, and C B^T only if there is room for it.  What fits
+// is then what fitted when every tile of y made its own part of C B^T: 8 bytes a step and head, and the states.
+static void make_static_layout(Plan &pl, Layout &lo) {
+    make_layout(pl, SSD_OP_FWD, lo, false);
+    if (lo.total <= (size_t)SSD_STATIC_WS_BYTES || pl.use_tc) return;
+    pl.keep_cb = false;
+    make_layout(pl, SSD_OP_FWD, lo, false);
 }
 
 static bool misaligned(const void *p) { return ((uintptr_t)p & 15u) != 0; }
@@ -339,7 +350,7 @@ static bool state_maps(const Layout &lo, void *ws, const SegParams &sp0, TcMaps 
 static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt, const float *A,
                         const void *Bm, const void *Cm, const float *D, const float *h0, void *y,
                         float *h_final, float *boundary, bool need_boundary, void *ws,
-                        size_t ws_bytes, void *stream, bool may_use_helper_stream = true) {
+                        size_t ws_bytes, void *stream, bool built_in_ws = false) {
     Plan pl;
     int rc = make_plan(shape, pl);
     if (rc) return rc;
@@ -350,7 +361,9 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         (boundary && misaligned(boundary)))
         return SSD_EALIGN;
     Layout lo;
-    make_layout(pl, need_boundary ? SSD_OP_FWD_SEG : SSD_OP_FWD, lo, may_use_helper_stream && !pl.serial);
+    const bool beside = !built_in_ws && !pl.serial;       // work of neighbouring segments side by side
+    if (built_in_ws) make_static_layout(pl, lo);
+    else make_layout(pl, need_boundary ? SSD_OP_FWD_SEG : SSD_OP_FWD, lo, beside);
     if (((uintptr_t)ws & 255u) || ws_bytes < lo.total) return SSD_EWORKSPACE;
     rc = check_device();
     if (rc) return rc;
@@ -363,7 +376,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     TcMaps maps;
     if (pl.use_tc && !tc_make_maps(sp, maps)) return SSD_ECUDA;
     const long long PN = (long long)pl.P * pl.N;
-    if (pl.use_tc && pl.nseg >= kMinSegmentsForTwins && may_use_helper_stream && !pl.serial && !g_prof_on) {
+    if (pl.use_tc && pl.nseg >= kMinSegmentsForTwins && beside && !g_prof_on) {
         // Algorithm 1 with the state chain one segment ahead: chunk states and state pass of segment k run on a
         // helper stream while the caller's stream still computes y of segment k-1, whose last, partly idle wave
         // they fill.  What both touch (records, bf16 states) exists two or three times and goes round; the carried state belongs
@@ -398,7 +411,6 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         return SSD_OK;
     }
     sp.chain_heads = chain_heads(pl, false);
-    const bool beside = may_use_helper_stream && !pl.serial;      // CUDA cores: the next segment's sums in the launch of y
     SegParams next;
     for (int k = 0; k < pl.nseg; ++k) {
         set_segment(pl, k, sp);
@@ -412,7 +424,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         select_copy(lo, ws, 0, k & 1, sp);
         if (k == 0 || !beside) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, pl.dtype, SIMT_SUMS, st));
         SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN, fin, st));
-        const bool ahead = beside && k + 1 < pl.nseg;
+        const bool ahead = beside && k + 1 < pl.nseg;      // the next segment's sums in the launch of y
         if (ahead) {
             next = sp;
             set_segment(pl, k + 1, next);
@@ -501,7 +513,7 @@ int ssd_fwd_static_ws(const ssd_shape_t *shape, const void *x, const float *dt, 
     int rc = make_plan(shape, pl);
     if (rc) return rc;
     Layout lo;
-    make_layout(pl, SSD_OP_FWD, lo, false);      // in order on one stream: no second copies
+    make_static_layout(pl, lo);
     if (lo.total > (size_t)SSD_STATIC_WS_BYTES) return SSD_ETOOLARGE;
     if (!x || !dt || !A || !Bm || !Cm || !D || !y) return SSD_EINVAL;
     rc = check_device();
@@ -512,7 +524,7 @@ int ssd_fwd_static_ws(const ssd_shape_t *shape, const void *x, const float *dt, 
     // forward_impl zeroes the status word on the stream and writes every other scratch region
     // before reading it, so stale contents of the shared array cannot leak into the outputs.
     return forward_impl(shape, x, dt, A, Bm, Cm, D, h0, y, h_final, nullptr, false, ws,
-                        (size_t)SSD_STATIC_WS_BYTES, stream, false);
+                        (size_t)SSD_STATIC_WS_BYTES, stream, true);
 }
 
 int ssd_fwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, const float *A,

@@ -108,7 +108,7 @@ struct SegParams {
     float *gcarry;         // [B,H,P,N]     state gradient handed right-to-left (backward)
     float *ghdot;          // [B,H,ncs,16]  partial sums of exp(cs_last) <Gout_c, H_in,c>
     float *ddt_dir;        // [B,H,ncs,Q]   direct part of ddt (tensor-core path: read where dt is next to zero, see bwd_finish)
-    float *cbt;            // CUDA-core path: [B,ncs,G,Q,Q] C B^T, causal 64 x 64 tiles
+    float *cbt;            // CUDA-core path: [B,ncs,G,Q,Q] C B^T, causal 64 x 64 tiles (null: made again where used, y in order only)
     float *rho;            // [B,H,ncs,Q]   C_t . (intra-chunk part of this head's dC_t); CUDA-core path: [B,H,ncs,tiles,Q] by column tile
     float *rho2;           // [B,H,ncs,Q]   C_t . (inter-chunk part of this head's dC_t)
     float *psi;            // [B,H,ncs,Q]   B_t . (intra-chunk part of this head's dB_t); CUDA-core path: [B,H,ncs,tiles,Q] by row tile

@@ -254,10 +254,10 @@ __device__ __forceinline__ float *cb_of(const SegParams &p, int b, int c, int g)
 // What a segment's chunks need before the states can be passed on, by block number:
 //   S_c[p,n] = sum_s exp(cs_last - cs_s) dt_s x_s[p] B_s[n]     -> Hst slot c+1   (and cs, dtT)
 //   with grads: E_c[p,n] = sum_t exp(cs_t) dy_t[p] C_t[n]       -> Gst slot c      (its CTAs make the cumsum again)
-//   the causal tiles of C B^T
+//   the causal tiles of C B^T, where the scratch has room for them
 template <typename T, int NS> __host__ __device__ __forceinline__ int simt_n_sums(const SegParams &p, bool grads) {
     const int nrt = p.Q >> 6;
-    return p.nc * p.B * ((NS / 64) * p.H * (grads ? 2 : 1) + p.G * (nrt * (nrt + 1) / 2));
+    return p.nc * p.B * ((NS / 64) * p.H * (grads ? 2 : 1) + (p.cbt ? p.G * (nrt * (nrt + 1) / 2) : 0));
 }
 template <typename T, int NS> __device__ __forceinline__ void simt_sums(const SegParams &p, SimtTiles &sm, float *wsm, int id, bool grads) {
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, nh = NS / 64;
@@ -370,14 +370,16 @@ template <typename T, int NS> __global__ void __launch_bounds__(256, 3) k_simt_s
 //   y_t  = sum_{s<=t} CB[t,s] e^{cs_t-cs_s} dt_s x_s + e^{cs_t} C_t H_in + D x_t
 //   u_s  = sum_{t>=s} CB[t,s] e^{cs_t-cs_s} dy_t     + e^{cs_last-cs_s} B_s Gout ;  dx_s = D dy_s + dt_s u_s ,
 //   ddt_direct_s = x_s . u_s , psi2_s = dt_s e^{cs_last-cs_s} x_s . (Gout B_s) , dD partial = sum dy.x
-template <typename T, int NS, bool DX>
+// CB false (y only): the tiles of C B^T are not in the scratch and are made here, per head, with the same operations in the same
+// order, so with the same bits.
+template <typename T, int NS, bool DX, bool CB>
 __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm, float *css, float *dts, float *fac, float *red, int c, int rt, int h, int b) {
     const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, g = h / p.hpg, r0 = rt * 64;
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q, HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
     const size_t xo = (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
     const T *vals = (const T *)(DX ? p.dy : p.x) + xo;
     const T *rowv = (const T *)(DX ? p.Bm : p.Cm) + (size_t)b * p.bc_bs + (tok0 + r0) * GN + (size_t)g * NS;
-    const float *St = DX ? p.Gst + slot_off(p, b, c + 1, h) : p.Hst + slot_off(p, b, c, h), *CB = cb_of(p, b, c, g);
+    const float *St = DX ? p.Gst + slot_off(p, b, c + 1, h) : p.Hst + slot_off(p, b, c, h), *cbt = cb_of(p, b, c, g);
     float4 ra[4], rb[4];
     float2 acc[4][2];
     zero_acc(acc);
@@ -389,8 +391,8 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
     }
     auto load_vals = [&](int ct) {      // CB tile and value rows of column tile ct
         // DX = false: rows t = r0 .., columns s = 64 ct .. ; DX = true: the tile's rows are the CB matrix's columns
-        if (!DX) tile_load_ws(ra, CB + (size_t)r0 * Q + ct * 64, Q, true);
-        else tile_load_ws(ra, CB + (size_t)ct * 64 * Q + r0, Q, false);
+        if (!DX && CB) tile_load_ws(ra, cbt + (size_t)r0 * Q + ct * 64, Q, true);
+        else if (DX) tile_load_ws(ra, cbt + (size_t)ct * 64 * Q + r0, Q, false);
         tile_load(rb, vals + (size_t)ct * 64 * HP, HP, false);
     };
     const int ct0 = DX ? rt : 0, ct1 = DX ? nrt : rt + 1;
@@ -401,7 +403,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
         if (k0 + 64 < NS) {
             tile_load(ra, rowv + k0 + 64, GN, true);
             tile_load_ws(rb, St + k0 + 64, NS, true);
-        } else {
+        } else if (CB) {
             load_vals(ct0);
         }
         tile_mma(acc, sm.a, sm.b);
@@ -432,7 +434,33 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
     }
     for (int ct = ct0; ct < ct1; ++ct) {
         // masked tile: a[k = column of the mask][row]
-        if (ct != rt) {
+        if constexpr (!CB) {
+            const T *colv = (const T *)p.Bm + (size_t)b * p.bc_bs + (tok0 + ct * 64) * GN + (size_t)g * NS;
+            float2 cb[4][2];
+            zero_acc(cb);
+            for (int k0 = 0; k0 < NS; k0 += 64) {
+                tile_load(ra, rowv + k0, GN, true);
+                tile_load(rb, colv + k0, GN, true);
+                tile_store(sm.a, ra, true);
+                tile_store(sm.b, rb, true);
+                __syncthreads();
+                tile_mma(cb, sm.a, sm.b);
+                __syncthreads();
+            }
+            load_vals(ct);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int s = ct * 64 + tx * 4 + j;
+                float e[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int t = r0 + ty * 4 + i;
+                    const float v = j < 2 ? (j ? cb[i][0].y : cb[i][0].x) : (j == 3 ? cb[i][1].y : cb[i][1].x);
+                    e[i] = ct != rt ? v * (fac[t] * fac[s]) : s <= t ? v * expf(fminf(css[t] - css[s], 0.f)) * dts[s] : 0.f;
+                }
+                *reinterpret_cast<float4 *>(&sm.a[tx * 4 + j][ty * 4]) = make_float4(e[0], e[1], e[2], e[3]);
+            }
+        } else if (ct != rt) {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const float one = fac[DX ? ct * 64 + ty + 16 * k : r0 + tr_row()];
@@ -451,10 +479,10 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
                 e[i] = s <= t ? e[i] * expf(fminf(css[t] - css[s], 0.f)) * (DX ? 1.f : dts[s]) : 0.f;
             }
         }
-        tile_store(sm.a, ra, !DX);
+        if (CB) tile_store(sm.a, ra, !DX);
         tile_store(sm.b, rb, false);
         __syncthreads();
-        if (ct + 1 < ct1) load_vals(ct + 1);
+        if (CB && ct + 1 < ct1) load_vals(ct + 1);
         tile_mma(acc, sm.a, sm.b);
         __syncthreads();
     }
@@ -496,8 +524,8 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
 // y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
 // wait for nothing of this one, and a launch of a few microseconds is saved per segment.  N = 64 is left at two CTAs per SM: three
 // would spill, and its layers are small.
-template <typename T, int NS>
-__global__ void __launch_bounds__(256, NS == 64 ? 2 : 3) k_simt_y(SegParams p, SegParams nx, int n_next) {
+template <typename T, int NS, bool CB>
+__global__ void __launch_bounds__(256, NS == 64 || !CB ? 2 : 3) k_simt_y(SegParams p, SegParams nx, int n_next) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
@@ -509,7 +537,7 @@ __global__ void __launch_bounds__(256, NS == 64 ? 2 : 3) k_simt_y(SegParams p, S
         return;
     }
     const int rt = id % nrt, c = (id / nrt) % p.nc, h = (id / (nrt * p.nc)) % p.H, b = id / (nrt * p.nc * p.H);
-    simt_row_tile<T, NS, false>(p, sm, css, dts, fac, nullptr, c, rt, h, b);
+    simt_row_tile<T, NS, false, CB>(p, sm, css, dts, fac, nullptr, c, rt, h, b);
 }
 
 // The large kernel of the backward: tiles of dx, and the partial slices of dB and dC.  Per (chunk, head range):
@@ -528,7 +556,7 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
     if (id >= (int)gridDim.x - n_dx) {
         id -= (int)gridDim.x - n_dx;
         const int rt = id % nrt, h = (id / nrt) % p.H, c = (id / (nrt * p.H)) % p.nc, b = id / (nrt * p.H * p.nc);
-        simt_row_tile<T, NS, true>(p, sm, css, dts, fac, red[0], c, rt, h, b);
+        simt_row_tile<T, NS, true, true>(p, sm, css, dts, fac, red[0], c, rt, h, b);
         return;
     }
     const int per = npair + 2 * nrt, role = id % per;
@@ -893,7 +921,9 @@ static cudaError_t simt_launch(const SegParams &p, const SegParams *next, int wh
         }
         case SIMT_Y: {
             const int n_next = next ? simt_n_sums<T, NS>(*next, false) : 0;
-            return launch_pdl(k_simt_y<T, NS>, dim3(p.nc * nrt * p.H * p.B + n_next), dim3(256), 0, st, p, next ? *next : p, n_next);
+            const dim3 grid(p.nc * nrt * p.H * p.B + n_next);
+            if (!p.cbt) return launch_pdl(k_simt_y<T, NS, false>, grid, dim3(256), 0, st, p, p, 0);      // never with `next`
+            return launch_pdl(k_simt_y<T, NS, true>, grid, dim3(256), 0, st, p, next ? *next : p, n_next);
         }
         case SIMT_TAIL: {
             const int nfin = tail_finish_ctas(p), n_next = simt_n_sums<T, NS>(*next, true);

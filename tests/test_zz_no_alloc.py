@@ -6,6 +6,7 @@ with different inputs, and compares each result with the ordinary ssd_fwd on the
 second call finds the first call's leftovers in the shared array and must not be affected by them.
 It passes both alone in a fresh process and after the rest of the suite."""
 import ctypes
+import itertools
 
 import pytest
 import torch
@@ -59,3 +60,47 @@ def test_static_scratch_is_sized_without_the_second_copies():
     serial = libssd.workspace_bytes(mk(libssd.SSD_FLAG_SERIAL), libssd.SSD_OP_FWD)
     default = libssd.workspace_bytes(mk(0), libssd.SSD_OP_FWD)
     assert 0 < serial <= default
+
+
+def test_static_scratch_takes_every_cuda_core_shape_whose_states_fit():
+    """What the built-in scratch has to hold is the states of a segment and two vectors; the products C B^T, which ssd_fwd keeps in
+    its own scratch, must not decide what fits (the size is asked before the pointers, so null ones say which it was)."""
+    ssd_build.build()
+    L = libssd.lib()
+    up = lambda v: (v + 255) // 256 * 256
+    seen = {True: 0, False: 0}
+    for dtype, H, G, N, chunk, ncs, B in itertools.product((libssd.SSD_DTYPE_F32, libssd.SSD_DTYPE_BF16), (4, 8, 24, 32), (1, 4, 8),
+                                                           (64, 128), (64, 128, 256), (1, 2, 3, 4, 8, 16, 32), (1, 2)):
+        if H % G:
+            continue
+        flags = libssd.SSD_FLAG_FORCE_SIMT if dtype == libssd.SSD_DTYPE_BF16 else 0
+        seg = chunk * ncs
+        shape = libssd.SSDShape(B, 4 * seg, H, 64, N, G, chunk, seg, dtype, flags, 0, 0, 0)
+        state = B * H * 64 * N * 4
+        need = 256 + 2 * up(B * H * seg * 4) + up(state * (ncs + 1)) + up(state)
+        fits = need <= libssd.SSD_STATIC_WS_BYTES
+        rc = L.ssd_fwd_static_ws(ctypes.byref(shape), None, None, None, None, None, None, None, None, None, None)
+        assert rc == (libssd.SSD_EINVAL if fits else libssd.SSD_ETOOLARGE), (dtype, H, G, N, chunk, ncs, B, need)
+        seen[fits] += 1
+    assert min(seen.values()) > 100
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,L,H,G,N,chunk,seg", [
+    ("fp32", 2304, 32, 8, 64, 256, 1024),
+    ("fp32", 2048, 24, 8, 128, 256, 1024),
+    ("fp32", 512, 16, 16, 64, 256, 512),
+    ("fp32", 4096, 8, 8, 128, 128, 2048),
+    ("bf16", 2048, 32, 16, 64, 256, 1024),
+])
+def test_static_scratch_without_room_for_the_products_gives_the_same_bits(dtype, L, H, G, N, chunk, seg):
+    cfg = CONFIGS[0].scaled(name="static", dtype=dtype, B=1, L=L, H=H, P=64, N=N, G=G, chunk=chunk, seg=seg, h0_std=0.1)
+    inp = make_inputs(cfg, "cuda")
+    args = (inp["x"], inp["dt"], inp["A"], inp["Bm"], inp["Cm"], inp["D"], inp["h0"])
+    shape = libssd.make_shape(inp["x"], inp["Bm"], chunk, seg, flags=libssd.SSD_FLAG_SERIAL)
+    assert libssd.workspace_bytes(shape, libssd.SSD_OP_FWD) > libssd.SSD_STATIC_WS_BYTES
+    y_ref, h_ref = libssd.ssd_fwd(*args, chunk=chunk, seg=seg)
+    y, hf = torch.full_like(inp["x"], float("nan")), torch.full_like(h_ref, float("nan"))
+    libssd.ssd_fwd_static_ws(*args, chunk=chunk, seg=seg, y=y, h_final=hf)
+    torch.cuda.synchronize()
+    assert torch.equal(y, y_ref) and torch.equal(hf, h_ref)
