@@ -104,8 +104,11 @@ typedef struct ssd_shape {
 /* Bytes of scratch `ws` that `op` needs for this shape (0 on an invalid shape).  Grows with
  * seg/chunk (the per-segment chunk states: the "grid cell" term of Eq. 4), not with L, apart from
  * 20 bytes per (batch, head, chunk) of dA/dD partial sums in the backward.  With two segments or more
- * there are second and third copies of what neighbouring segments' kernels touch at the same time,
- * unless shape->flags has SSD_FLAG_SERIAL: size the buffer with the flags the call will use.
+ * there are second and third copies of what neighbouring segments' kernels touch at the same time (tensor-core
+ * path: 3 times the forward's and 2.5 times the backward's scratch; CUDA-core path: up to 64 MiB more in
+ * the forward), unless shape->flags has SSD_FLAG_SERIAL: size the buffer with the flags the call will use.
+ * The CUDA-core path also keeps the products C B^T of a segment, 4 B G chunk seg bytes (not in ssd_fwd_static_ws
+ * where they do not fit).
  * The tensor-core path takes bf16 calls with N = 128, chunk = 256 and an even H/G; its states, masked tiles and
  * decayed rows are bf16 between the kernels (fp32 outputs within 2e-3).  All other calls, and those with
  * SSD_FLAG_FORCE_SIMT, keep them in fp32.

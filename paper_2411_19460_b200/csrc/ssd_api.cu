@@ -89,6 +89,19 @@ static int bc_head_split(int blocks, int groups, int hpg) {
     return best;
 }
 
+// The same for the CUDA-core kernel, whose ranges have Q/64 + 3 slots each: ranges of four heads, of two where there are few, so
+// that a short sequence has CTAs enough (8 heads, 256-step chunks, backward: 2048 steps 265 us, with half the ranges 320; 4096
+// steps 353 and 341).  Long ones (64 chunks and more, counted per group) have them anyway, and the slots cost time and memory:
+// there no more of them than two per head, what a slice for each head would take (2 x 8192 steps of 8 heads 999 -> 918 us, 8192 of
+// 80 heads in 8 groups 3976 -> 3373 us and 985 -> 381 MB of scratch).
+static int simt_head_ranges(const Plan &pl) {
+    const int per_range = pl.hpg >= 16 ? 4 : 2, slots = pl.Q / 64 + 3;
+    int n = (pl.hpg + per_range - 1) / per_range;
+    if (pl.B * pl.nct * pl.G >= 64 && n * slots > 2 * pl.hpg) n = 2 * pl.hpg >= slots ? 2 * pl.hpg / slots : 1;
+    const int hps = (pl.hpg + n - 1) / n;
+    return (pl.hpg + hps - 1) / hps;                    // no empty range
+}
+
 static int make_plan(const ssd_shape_t *s, Plan &pl) {
     if (!s) return SSD_EINVAL;
     if (s->B <= 0 || s->L <= 0 || s->H <= 0 || s->P <= 0 || s->N <= 0 || s->G <= 0 || s->chunk <= 0 ||
@@ -124,11 +137,17 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
         return SSD_EALIGN;
     pl.serial = (s->flags & SSD_FLAG_SERIAL) != 0;
     pl.keep_cb = true;
-    // Partial slices of the dB/dC head sums: one per CTA head range; on the CUDA-core path ranges of four heads (two where there
-    // are few), each with a slot per 64-step tile and one for the inter-chunk term.
-    const int per_range = pl.hpg >= 16 ? 4 : 2;
-    pl.nsl = pl.use_tc ? bc_head_split(pl.B * pl.nct, pl.G, pl.hpg) : (pl.hpg + per_range - 1) / per_range * (pl.Q / 64 + 1);
+    // Partial slices of the dB/dC head sums: one per CTA head range
+    pl.nsl = pl.use_tc ? bc_head_split(pl.B * pl.nct, pl.G, pl.hpg) : simt_head_ranges(pl) * (pl.Q / 64 + 3);
     return SSD_OK;
+}
+
+// CUDA cores: whether the sums of a segment ride in a launch of its neighbour.  In the forward that takes second copies of states
+// and C B^T, up to 64 MiB of them: 17 MiB are worth 7 % (24 heads, 2048-step segments, 868 -> 803 us), 20 MiB 10 % (80 heads,
+// 1024 steps, 1544 -> 1391), 38 MiB 6 %, 74 MiB 2 % (80 heads, 4096 steps, 1351 -> 1326).
+static bool simt_overlap(const Plan &pl, bool bwd) {
+    const size_t copy = ((size_t)pl.B * pl.H * (pl.ncs + 1) * pl.P * pl.N + (size_t)pl.B * pl.ncs * pl.G * pl.Q * pl.Q) * sizeof(float);
+    return pl.nseg > 1 && (bwd || copy <= (size_t)64 << 20);
 }
 
 static int chain_copies(int nseg) { return nseg >= kMinSegmentsForTwins ? 3 : nseg > 1 ? 2 : 1; }
@@ -161,7 +180,7 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
     } else {
         // two copies where a launch works on two neighbouring segments: y beside the next segment's sums, and in the backward,
         // where only the step sizes meet, the finishing steps beside them
-        const bool two = twins && pl.nseg > 1;
+        const bool two = twins && simt_overlap(pl, bwd);
         take2(lo.cs, vec, two && !bwd);
         take2(lo.dtT, vec, two);
         take2(lo.Hst, st, two && !bwd);
@@ -180,8 +199,8 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
         take2(lo.psi, vec_tiles, vtwin);
         take2(lo.psi2, vec, vtwin);
         const size_t part = (size_t)pl.B * pl.seg * pl.G * pl.nsl * pl.N * sizeof(float);
-        take2(lo.pB, part, twin);
         take2(lo.pC, part, twin);
+        if (pl.use_tc) take2(lo.pB, part, twin);
         lo.dAp = take(BH * pl.nct * sizeof(float));
         lo.dDp = take(BH * pl.nct * 4 * sizeof(float));
     }
@@ -411,6 +430,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         return SSD_OK;
     }
     sp.chain_heads = chain_heads(pl, false);
+    const bool overlap = beside && simt_overlap(pl, false);
     SegParams next;
     for (int k = 0; k < pl.nseg; ++k) {
         set_segment(pl, k, sp);
@@ -422,9 +442,9 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
             continue;
         }
         select_copy(lo, ws, 0, k & 1, sp);
-        if (k == 0 || !beside) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, pl.dtype, SIMT_SUMS, st));
+        if (k == 0 || !overlap) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, pl.dtype, SIMT_SUMS, st));
         SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN, fin, st));
-        const bool ahead = beside && k + 1 < pl.nseg;      // the next segment's sums in the launch of y
+        const bool ahead = overlap && k + 1 < pl.nseg;      // the next segment's sums in the launch of y
         if (ahead) {
             next = sp;
             set_segment(pl, k + 1, next);

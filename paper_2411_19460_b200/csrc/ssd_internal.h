@@ -79,7 +79,7 @@ struct SegParams {
     int c0;        // global index of the segment's first chunk
     int ncs;       // chunk capacity of the workspace (chunks of a full segment)
     int nct;       // chunks in the whole sequence (L / Q)
-    int nsl;       // head slices per group in the dB/dC partial buffers
+    int nsl;       // slices per group in the dB/dC partial buffers: head ranges, or slots of all ranges (CUDA-core path)
     int ndd;       // partial sums of dD per (head, chunk) that the kernels of this path write (<= 4)
     int scan_ctas; // CTAs of the y / dx kernel, at most (no effect on results)
     int chain_heads; // heads per CTA of the forward chain, 1 or 2 (no effect on results)
@@ -113,7 +113,7 @@ struct SegParams {
     float *rho2;           // [B,H,ncs,Q]   C_t . (inter-chunk part of this head's dC_t)
     float *psi;            // [B,H,ncs,Q]   B_t . (intra-chunk part of this head's dB_t); CUDA-core path: [B,H,ncs,tiles,Q] by row tile
     float *psi2;           // [B,H,ncs,Q]   B_t . (inter-chunk part of this head's dB_t)
-    float *pB, *pC;        // [B,seg,G,nsl,N] per-head-slice partial dB / dC
+    float *pB, *pC;        // [B,seg,G,nsl,N] partial dB / dC; CUDA-core path: one buffer, pC, for both
     float *dAp;            // [B,H,nct]     per-chunk partial of dA
     float *dDp;            // [B,H,nct,4]   partials of dD, the first ndd of each group in use
 };

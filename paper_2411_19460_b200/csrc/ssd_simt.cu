@@ -544,7 +544,8 @@ __global__ void __launch_bounds__(256, NS == 64 || !CB ? 2 : 3) k_simt_y(SegPara
 //   causal tile pair (tt, ts): W_h = (dy_tt x_ts^T) o mask per head, rho / psi partial sums of W_h o CB, head sum of W_h; then
 //                  slices dC[tt] = Wsum B_ts and dB[ts] = Wsum^T C_tt
 //   inter dC, tile tt : sum_h e^{cs_t} dy_t H_in (and rho2 per head);  inter dB, tile ts : sum_h dt_s e^{cs_last-cs_s} x_s Gout
-// A slice has Q/64 + 1 slots per head range: dC by ts (dB by tt), the last one the inter-chunk term.
+// A row of tile r has dC slots for ts <= r and dB slots for tt >= r, so the two share Q/64 + 3 slots per head range: dC by ts, dB by
+// tt + 1, then the inter-chunk terms of both.
 template <typename T, int NS>
 __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
     pdl_launch_dependents();
@@ -561,7 +562,7 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
     }
     const int per = npair + 2 * nrt, role = id % per;
     id /= per;
-    const int rng = p.nsl / (nrt + 1);                         // head ranges per group
+    const int rng = p.nsl / (nrt + 3);                         // head ranges per group
     const int sl = id % rng, g = (id / rng) % p.G, c = (id / (rng * p.G)) % p.nc, b = id / (rng * p.G * p.nc);
     const int hps = (p.hpg + rng - 1) / rng, h0 = g * p.hpg + sl * hps, h1 = min(h0 + hps, (g + 1) * p.hpg);
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q, HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
@@ -573,11 +574,11 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
             dts[t] = p.dtT[vec_off(p, b, h, c) + t];
         }
     };
-    auto write_slice = [&](float *part, const float2 (&acc)[4][2], int row0, int slot, int n0) {
+    auto write_slice = [&](const float2 (&acc)[4][2], int row0, int slot, int n0) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const size_t tl = (size_t)b * p.ncs * Q + (size_t)c * Q + row0 + ty * 4 + i;
-            *reinterpret_cast<float4 *>(part + ((tl * p.G + g) * p.nsl + sl * (nrt + 1) + slot) * NS + n0 + tx * 4) =
+            *reinterpret_cast<float4 *>(p.pC + ((tl * p.G + g) * p.nsl + sl * (nrt + 3) + slot) * NS + n0 + tx * 4) =
                 make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
         }
     };
@@ -669,7 +670,7 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
             __syncthreads();
             zero_acc(acc);
             tile_mma(acc, sm.a, sm.b);
-            write_slice(p.pC, acc, tt * 64, ts, n0);
+            write_slice(acc, tt * 64, ts, n0);
             __syncthreads();
         }
         // dB[ts] = Wsum^T C_tt: a[k = t][s]
@@ -682,7 +683,7 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
             __syncthreads();
             zero_acc(acc);
             tile_mma(acc, sm.a, sm.b);
-            write_slice(p.pB, acc, ts * 64, tt, n0);
+            write_slice(acc, ts * 64, tt + 1, n0);
             __syncthreads();
         }
         return;
@@ -736,7 +737,7 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
         }
     }
 #pragma unroll
-    for (int m = 0; m < NS / 64; ++m) write_slice(isC ? p.pC : p.pB, tot[m], rt * 64, nrt, m * 64);
+    for (int m = 0; m < NS / 64; ++m) write_slice(tot[m], rt * 64, isC ? nrt + 1 : nrt + 2, m * 64);
 }
 
 // ------------------------------------------------------------------ da, ddt, dA partial
@@ -857,14 +858,13 @@ __device__ __forceinline__ void reduce_dbdc(const SegParams &p, int id) {
     auto ld = [](const float *q) { return *reinterpret_cast<const float4 *>(q); };
     const size_t src = ((((size_t)b * segcap + tl) * p.G + g) * p.nsl) * p.N + n;
     if (!TC) {
-        // CUDA-core path: per head range one slot per 64-step tile and one for the inter-chunk term; a row of tile rt has dC
-        // slots 0 .. rt and dB slots rt .. tiles - 1
+        // CUDA-core path: per head range, of a row of tile rt, dC slots 0 .. rt, dB slots rt + 1 .. tiles, then the inter-chunk terms
         const int rt = (int)(tl % (size_t)p.Q) >> 6;
-        for (int s0 = 0; s0 < p.nsl; s0 += p.tiles + 1)
-            for (int t = 0; t <= p.tiles; ++t) {
-                if (t >= rt) add4(sB, ld(p.pB + src + (size_t)(s0 + t) * p.N));
-                if (t <= rt || t == p.tiles) add4(sC, ld(p.pC + src + (size_t)(s0 + t) * p.N));
-            }
+        for (int s0 = 0; s0 < p.nsl; s0 += p.tiles + 3) {
+            for (int t = 0; t <= p.tiles; ++t) add4(t <= rt ? sC : sB, ld(p.pC + src + (size_t)(s0 + t) * p.N));
+            add4(sC, ld(p.pC + src + (size_t)(s0 + p.tiles + 1) * p.N));
+            add4(sB, ld(p.pC + src + (size_t)(s0 + p.tiles + 2) * p.N));
+        }
     } else {
         for (int s = 0; s < p.nsl; ++s) {
             add4(sB, ld(p.pB + src + (size_t)s * p.N));
@@ -930,7 +930,7 @@ static cudaError_t simt_launch(const SegParams &p, const SegParams *next, int wh
             return launch_pdl(k_simt_tail<T, NS>, dim3(n_next + nfin + tail_reduce_ctas(p)), dim3(256), 0, st, p, *next, n_next, nfin);
         }
         default: {
-            const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 1)) * p.G * p.B;
+            const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 3)) * p.G * p.B;
             return launch_pdl(k_simt_bwd<T, NS>, dim3(n_bc + n_dx), dim3(256), 0, st, p, n_dx);
         }
     }

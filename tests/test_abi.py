@@ -50,6 +50,23 @@ def test_workspace_scales_with_segment_not_length(L):
     assert libssd.boundary_bytes(shape(seg=0)) == 4 * 64 * 128 * 4
 
 
+@pytest.mark.parametrize("kw", [
+    dict(L=8192, H=80, G=8, seg=4096), dict(L=8192, H=80, G=1, seg=4096), dict(L=8192, H=8, seg=2048, B=2), dict(L=16384, H=32, G=4, seg=8192),
+    dict(L=8192, H=32, N=64, chunk=128, seg=4096),
+])
+def test_cuda_core_scratch_is_no_larger_than_a_slice_per_head(L, kw):
+    """The backward's partial dB and dC take what one slice per head would, beside two sets of states, the products C B^T and a few
+    vectors; running neighbouring segments side by side costs the forward 64 MiB at most."""
+    s = shape(**dict(kw, dtype=libssd.SSD_DTYPE_F32))
+    vec = 4 * s.B * s.seg * s.H
+    state = 4 * s.B * s.H * 64 * s.N
+    bound = 2 * state * (s.seg // s.chunk + 3) + 2 * vec * s.N + 4 * s.B * s.seg * s.G * s.chunk + 24 * vec
+    assert libssd.workspace_bytes(s, libssd.SSD_OP_BWD_SEG) <= bound
+    serial = shape(**dict(kw, dtype=libssd.SSD_DTYPE_F32, flags=libssd.SSD_FLAG_SERIAL))
+    for op in (libssd.SSD_OP_FWD, libssd.SSD_OP_FWD_SEG):
+        assert libssd.workspace_bytes(s, op) <= libssd.workspace_bytes(serial, op) + (64 << 20) + 2 * vec
+
+
 @pytest.mark.parametrize("kw,code", [
     (dict(H=3, G=2), libssd.SSD_EINVAL),
     (dict(L=1000), libssd.SSD_EINVAL),

@@ -36,6 +36,9 @@ STIFF = dict(a_max=64.0, dt_lo=1e-4, dt_hi=1.0)
     ("fp32", 1280, 5, 1, 128, 256, 512, STIFF),
     ("fp32", 512, 2, 2, 128, 128, 256, dict(B=2)),
     ("bf16", 192, 3, 1, 128, 64, 64, {}),
+    ("fp32", 4096, 16, 4, 64, 256, 1024, {}),          # long sequences: fewer head ranges of dB/dC
+    ("fp32", 8192, 5, 1, 64, 128, 2048, STIFF),
+    ("fp32", 8320, 32, 1, 128, 64, 4160, {}),          # segments too large to run side by side in the forward
 ])
 def test_launch_edges(dtype, L, H, G, N, chunk, seg, extra):
     cfg = CONFIGS[0].scaled(**dict(dict(name="edge", dtype=dtype, B=1, L=L, H=H, P=64, N=N, G=G, chunk=chunk, seg=seg, h0_std=0.1,
