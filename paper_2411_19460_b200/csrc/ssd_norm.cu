@@ -323,8 +323,9 @@ k_gated_norm_staged(const T *y, const T *z, const float *gamma, float eps, const
         const float n = rsqrtf(sum.x * rgroup + eps);
         const float2 n2 = make_float2(n, n);
         const size_t base = base0 + (size_t)j * D;
-        // xh = v n ;  dvh = dout gamma ;  c = mean(dvh xh) ;  dv = n (dvh - xh c)
-        const float c = n * n * n * sum.y * rgroup;
+        // xh = v n ;  dvh = dout gamma ;  c = mean(dvh xh) ;  dv = n (dvh - xh c).  No power of n by itself: it leaves the range of
+        // fp32 where v, its square and the gradient do not.
+        const float c = n * sum.y * rgroup;
         const float2 c2 = make_float2(-c, -c), one2 = make_float2(1.f, 1.f);
 #pragma unroll
         for (int k = 0; k < NV; ++k) {
@@ -338,8 +339,9 @@ k_gated_norm_staged(const T *y, const T *z, const float *gamma, float eps, const
                     } else {
                         const float2 yy = ry[k].pair(e), g = rg[k].pair(e), qq = q[k][e], s = sgm[k][e];
                         const float2 v = __fmul2_rn(yy, qq);
-                        dg[k][e] = __ffma2_rn(g, __fmul2_rn(v, n2), dg[k][e]);
-                        const float2 dv = __ffma2_rn(__fmul2_rn(g, gm[k][e]), n2, __fmul2_rn(v, c2));
+                        const float2 xh = __fmul2_rn(v, n2);
+                        dg[k][e] = __ffma2_rn(g, xh, dg[k][e]);
+                        const float2 dv = __fmul2_rn(n2, __ffma2_rn(xh, c2, __fmul2_rn(g, gm[k][e])));
                         o1[e] = __fmul2_rn(dv, qq);                                       // y silu(z): d / dy
                         // silu'(z) = s (1 + z (1 - s)) = s + q (1 - s)
                         const float2 ds = __ffma2_rn(qq, __ffma2_rn(s, make_float2(-1.f, -1.f), one2), s);

@@ -101,3 +101,25 @@ def test_gated_norm_row_splits_and_rings(rows, D, group, dtype):
     assert relerr(libssd.ssd_gated_norm_fwd(y, z, gamma, group=group), out_ref) <= TOL[dtype]
     for a, r in zip(libssd.ssd_gated_norm_bwd(y, z, gamma, g, group=group), refs):
         assert relerr(a, r) <= TOL[dtype]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("scale,eps", [(1e15, 1e-5), (1e-15, 0.0)])
+@pytest.mark.parametrize("D,group", [(1024, 1024), (8192, 8192)])
+def test_gated_norm_of_rows_far_from_one(D, group, scale, eps, dtype):
+    """A normalisation does not depend on its input's scale: whatever fp32 holds the squares of has the same accuracy."""
+    from paper_2411_19460_b200 import libssd
+    from tests.parity_util import TOL, relerr
+
+    td = torch.float32 if dtype == "fp32" else torch.bfloat16
+    gen = torch.Generator().manual_seed(3)
+    y, z, g = (torch.randn(12, D, generator=gen).to(td).cuda() for _ in range(3))
+    y = y * scale
+    gamma = (1.0 + 0.1 * torch.randn(D, generator=gen)).cuda()
+    f64 = lambda t: t.detach().double().cpu().numpy()
+    out_ref, _, _ = orc.gated_norm_fwd(f64(y), f64(z), f64(gamma), group, eps=eps)
+    refs = orc.gated_norm_bwd(f64(y), f64(z), f64(gamma), f64(g), group, eps=eps)
+    assert relerr(libssd.ssd_gated_norm_fwd(y, z, gamma, group=group, eps=eps), out_ref) <= TOL[dtype]
+    for a, r in zip(libssd.ssd_gated_norm_bwd(y, z, gamma, g, group=group, eps=eps), refs):
+        assert relerr(a, r) <= TOL[dtype]
