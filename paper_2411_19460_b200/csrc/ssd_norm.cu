@@ -11,18 +11,18 @@ namespace ssd {
 
 using namespace sm100;
 
-// Partial sums of dgamma that a backward call may leave: one per CTA, at most two CTAs per SM in the staged kernel (of at least
-// four rows each) and one per 16 rows in the other.
+// Partial sums of dgamma that a backward call may leave: one per 16 rows, and one more for each CTA of the staged kernel (at most
+// two per SM, of at least four rows each), whose rows may end in the middle of sixteen.
 long long gated_norm_tiles(long long rows) {
-    const long long a = (rows + 3) / 4 < 2 * kNumSMs ? (rows + 3) / 4 : 2 * kNumSMs, b = (rows + 15) / 16;
-    return a > b ? a : b;
+    const long long a = (rows + 3) / 4 < 2 * kNumSMs ? (rows + 3) / 4 : 2 * kNumSMs;
+    return a + (rows + 15) / 16;
 }
 
 namespace {
 
 constexpr int GN_THREADS = 256;
 constexpr int GN_MAXV = 8;        // four-channel vectors per thread, at most (the kernels are instantiated for 1, 2, 4, 5 and 8)
-constexpr int GN_ROWS = 16;       // rows per CTA
+constexpr int GN_ROWS = 16;       // rows of a partial sum of dgamma, at most; rows per CTA of the kernels without a ring
 constexpr int GN_MAX_STAGES = 8;  // rows in flight per CTA in the staged kernels, at most
 
 template <typename T> __device__ __forceinline__ void gld4(const T *p, float *f);
@@ -269,6 +269,16 @@ k_gated_norm_staged(const T *y, const T *z, const float *gamma, float eps, const
         gm[k][1] = make_float2(g4.z, g4.w);
         dg[k][0] = dg[k][1] = make_float2(0.f, 0.f);
     }
+    // Row j ends a partial sum of dgamma: fp32 over 16 rows at most, whatever a CTA's share of a long call, fp64 from there on
+    auto leave_sum = [&](int j) {
+        const size_t tile = (size_t)blockIdx.x * ((rpc + GN_ROWS - 1) / GN_ROWS) + j / GN_ROWS;
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+            const int i = threadIdx.x + k * GN_THREADS;
+            if (i < nv) st_pairs(part + tile * D + (size_t)gi * group + (size_t)i * 4, dg[k][0], dg[k][1]);
+            dg[k][0] = dg[k][1] = make_float2(0.f, 0.f);
+        }
+    };
     __syncthreads();
     const float rgroup = 1.f / (float)group;
     int st = 0;
@@ -352,20 +362,15 @@ k_gated_norm_staged(const T *y, const T *z, const float *gamma, float eps, const
                 if (BWD) st_pairs(dz + base + (size_t)i * 4, o2[0], o2[1]);
             }
         }
+        if (BWD && (j + 1) % GN_ROWS == 0 && j + 1 < nrows) leave_sum(j);
     }
     pdl_launch_dependents();     // not earlier: the next launch fills the GPU in one wave and wants it free
-    if (BWD) {
-#pragma unroll
-        for (int k = 0; k < NV; ++k) {
-            const int i = threadIdx.x + k * GN_THREADS;
-            if (i < nv) st_pairs(part + (size_t)blockIdx.x * D + (size_t)gi * group + (size_t)i * 4, dg[k][0], dg[k][1]);
-        }
-    }
+    if (BWD) leave_sum(nrows - 1);
 }
 
 // Ring of a staged launch: as many rows as fit 110 KB (two CTAs per SM, bf16) or else 220 KB; 0: not even two rows fit.
 struct StagedPlan { int stages, rpc; };
-template <typename T> StagedPlan staged_plan(long long rows, int D, int group, int tensors, bool partials) {
+template <typename T> StagedPlan staged_plan(long long rows, int D, int group, int tensors) {
     const int need = (group / 4 + GN_THREADS - 1) / GN_THREADS, stage = tensors * group * (int)sizeof(T);
     if (need > 5 || (group * sizeof(T)) % 16) return {0, 0};
     int stages = 110 * 1024 / stage, per_sm = sizeof(T) == 2 ? 2 : 1;
@@ -375,12 +380,10 @@ template <typename T> StagedPlan staged_plan(long long rows, int D, int group, i
     }
     if (stages < 2) return {0, 0};
     if (stages > GN_MAX_STAGES) stages = GN_MAX_STAGES;
-    // rows per CTA: one even wave over the GPU, at least four (the ring has to fill); with partial sums, no more CTAs than
-    // the scratch holds
+    // rows per CTA: one even wave over the GPU, at least four (the ring has to fill)
     const long long ctas = (long long)kNumSMs * per_sm / (D / group) > 0 ? (long long)kNumSMs * per_sm / (D / group) : 1;
     long long rpc = (rows + ctas - 1) / ctas;
     if (rpc < 4) rpc = 4;
-    if (partials && (rows + rpc - 1) / rpc > gated_norm_tiles(rows)) rpc = (rows + gated_norm_tiles(rows) - 1) / gated_norm_tiles(rows);
     return {stages, (int)rpc};
 }
 
@@ -437,7 +440,7 @@ template <typename T>
 static cudaError_t norm_fwd_t(const T *y, const T *z, const float *gamma, float eps, T *out, long long rows, int D, int group,
                               cudaStream_t st) {
     const int need = (group / 4 + GN_THREADS - 1) / GN_THREADS;
-    const StagedPlan pl = staged_plan<T>(rows, D, group, 2, false);
+    const StagedPlan pl = staged_plan<T>(rows, D, group, 2);
     if (pl.stages) {
 #define GN_CASE(NV) return launch_staged<T, NV, false>(pl, y, z, gamma, eps, (const T *)nullptr, out, (T *)nullptr, (float *)nullptr, rows, D, group, st)
         GN_BY_NEED(GN_CASE);
@@ -454,9 +457,10 @@ template <typename T>
 static cudaError_t norm_bwd_t(const T *y, const T *z, const float *gamma, float eps, const T *dout, T *dy, T *dz, float *part,
                               long long rows, int D, int group, int &parts, cudaStream_t st) {
     const int need = (group / 4 + GN_THREADS - 1) / GN_THREADS;
-    const StagedPlan pl = staged_plan<T>(rows, D, group, 3, true);
+    const StagedPlan pl = staged_plan<T>(rows, D, group, 3);
     if (pl.stages) {
-        parts = (int)((rows + pl.rpc - 1) / pl.rpc);
+        const long long full = (rows - 1) / pl.rpc, last = rows - full * pl.rpc;      // CTAs before the last one, its rows
+        parts = (int)(full * ((pl.rpc + GN_ROWS - 1) / GN_ROWS) + (last + GN_ROWS - 1) / GN_ROWS);
 #define GN_CASE(NV) return launch_staged<T, NV, true>(pl, y, z, gamma, eps, dout, dy, dz, part, rows, D, group, st)
         GN_BY_NEED(GN_CASE);
 #undef GN_CASE

@@ -123,3 +123,19 @@ def test_gated_norm_of_rows_far_from_one(D, group, scale, eps, dtype):
     assert relerr(libssd.ssd_gated_norm_fwd(y, z, gamma, group=group, eps=eps), out_ref) <= TOL[dtype]
     for a, r in zip(libssd.ssd_gated_norm_bwd(y, z, gamma, g, group=group, eps=eps), refs):
         assert relerr(a, r) <= TOL[dtype]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("rows,D,group", [(65536, 256, 256), (8192, 1024, 128), (4099, 2048, 2048)])
+def test_gated_norm_dgamma_of_long_calls_is_summed_in_short_pieces(rows, D, group):
+    """However many rows a CTA takes, fp32 sums of dgamma end after 16 of them.  Relative error of 16 terms of either sign in order:
+    sqrt(16 / 2) 2^-25; of a term itself (reciprocal root, sigmoid, products): about 2^-23.  One sum over 222 rows: 3e-7."""
+    from paper_2411_19460_b200 import libssd
+
+    gen = torch.Generator(device="cuda").manual_seed(rows)
+    y, z, g = (torch.randn(rows, D, generator=gen, device="cuda") for _ in range(3))
+    gamma = 1.0 + 0.1 * torch.randn(D, generator=gen, device="cuda")
+    v = (y.double() * z.double() * torch.sigmoid(z.double())).view(rows, -1, group)
+    ref = ((v * torch.rsqrt((v * v).mean(-1, keepdim=True) + 1e-5)).view(rows, D) * g.double()).sum(0)
+    _, _, dg = libssd.ssd_gated_norm_bwd(y, z, gamma, g, group=group)
+    assert ((dg.double() - ref).norm() / ref.norm()).item() <= 2e-7
