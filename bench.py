@@ -54,7 +54,6 @@ def kind_model(cfg):
     st = 4.0 * HPN / Q                       # one fp32 chunk state per Q tokens
     return {
         # kind: (bound, flops/token, bytes/token)
-        "chunk_cumsum": ("hbm", 0.0, 12.0 * H),
         "chunk_state": ("tensor", 2.0 * HPN, e * (H * P + G * N) + st),
         "state_pass_fwd": ("hbm", 0.0, 2.0 * st),
         "chunk_scan_fwd": ("tensor", 2.0 * HPN + 2 * k * Q * (G * N + H * P), e * (2 * H * P + 2 * G * N) + st),
@@ -65,8 +64,7 @@ def kind_model(cfg):
         "bwd_dB": ("tensor", 2.0 * HPN + 2 * k * Q * (G * N), e * (2 * H * P + 2 * G * N) + st),
         # dB and dC from one masked tile: scores once, the two products of the head-summed tile, two state terms
         "bwd_dBdC": ("tensor", 4.0 * HPN + 2 * k * Q * (H * P + 2 * G * N), e * (2 * H * P + 2 * G * N) + 2 * st),
-        "bwd_finish": ("hbm", 0.0, 16.0 * H),
-        "reduce_dBdC": ("hbm", 0.0, 2.0 * e * G * N),
+        "bwd_finish": ("hbm", 0.0, 16.0 * H + 2.0 * e * G * N),      # with the sums of dB and dC
         "final_dAdD": ("hbm", 0.0, 0.0),
     }
 

@@ -25,8 +25,8 @@ static std::vector<ProfEvent> g_prof_pool;
 static size_t g_prof_used = 0;
 
 static const char *const kKindNames[KIND_COUNT] = {
-    "chunk_cumsum", "chunk_state", "state_pass_fwd", "chunk_scan_fwd", "dstate_contrib",
-    "state_pass_bwd", "bwd_dx", "bwd_dC", "bwd_dB", "bwd_finish", "reduce_dBdC", "final_dAdD", "glue", "decode_step", "bwd_dBdC", "conv1d", "gated_norm"};
+    "chunk_state", "state_pass_fwd", "chunk_scan_fwd", "dstate_contrib",
+    "state_pass_bwd", "bwd_dx", "bwd_dC", "bwd_dB", "bwd_finish", "final_dAdD", "glue", "decode_step", "bwd_dBdC", "conv1d", "gated_norm"};
 
 static ProfEvent *prof_begin(int kind, cudaStream_t st) {
     if (!g_prof_on) return nullptr;
@@ -171,7 +171,7 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
     };
     memset(&lo, 0, sizeof(lo));
     lo.status = take(256);
-    lo.hcarry = take(BH * PN * sizeof(float));
+    if (!bwd) lo.hcarry = take(BH * PN * sizeof(float));      // the backward starts every segment from `boundary`
     // the vectors and records (a fraction of the states) exist as often for any number of segments, so that the scratch is a
     // function of the segment length that only rises
     if (pl.use_tc) {
@@ -237,7 +237,7 @@ static int check_device() {
 // Helper streams per (host thread, device) with the events that fork them off the caller's stream and join them
 // back: s[4] recomputes a segment's chunk states (in the forward: the whole state chain is on s[0]), s[0] runs the
 // state-gradient part of the chain, s[1] / s[3] the dB/dC kernel of even / odd segments beside dx on the caller's
-// stream, s[2] a segment's two finishing kernels.  Created on first use, never
+// stream, s[2] a segment's finishing kernel.  Created on first use, never
 // destroyed (they hold no device memory); the caller's stream stays the only one the caller has to order
 // against.  Events indexed [2] and [3] go round with the segment, like the copies of the scratch regions.
 struct SideStreams {
@@ -322,7 +322,7 @@ static void fill_params(const Plan &pl, const Layout &lo, void *ws, SegParams &s
     char *w = (char *)ws;
     sp.status = (unsigned int *)(w + lo.status);
     sp.tiles = pl.use_tc ? 0 : pl.Q / 64;
-    sp.hcarry = (float *)(w + lo.hcarry);
+    sp.hcarry = lo.hcarry ? (float *)(w + lo.hcarry) : nullptr;
     sp.Gst = (float *)(w + lo.Gst);
     sp.gcarry = (float *)(w + lo.gcarry);
     sp.dAp = (float *)(w + lo.dAp);
@@ -396,10 +396,9 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     if (pl.use_tc && !tc_make_maps(sp, maps)) return SSD_ECUDA;
     const long long PN = (long long)pl.P * pl.N;
     if (pl.use_tc && pl.nseg >= kMinSegmentsForTwins && beside && !g_prof_on) {
-        // Algorithm 1 with the state chain one segment ahead: chunk states and state pass of segment k run on a
-        // helper stream while the caller's stream still computes y of segment k-1, whose last, partly idle wave
-        // they fill.  What both touch (records, bf16 states) exists two or three times and goes round; the carried state belongs
-        // to the chain alone.
+        // Algorithm 1 with the state chain ahead: it runs on a helper stream, up to as many segments ahead of y on the caller's
+        // stream as there are copies of what both touch (records, bf16 states), and fills what y leaves idle.  The carried state
+        // belongs to the chain alone.
         SideStreams *side = side_streams();
         if (!side) { g_last_cuda = (int)cudaGetLastError(); return SSD_ECUDA; }
         const int ncp = chain_copies(pl.nseg);
@@ -595,7 +594,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         //   chain(k): Recompute_Forward (chunk states, forward state pass), the state-gradient contributions and
         //             the backward state pass -- all it takes from segment k+1 is the state gradient handed left;
         //   big(k)  : dx on the caller's stream beside dB/dC on a second one -- they read what chain(k) left;
-        //   tail(k) : the two short finishing kernels.
+        //   tail(k) : the finishing kernel.
         // chain(k-1) runs on its own stream while big(k) is busy and fills the SMs that big(k)'s last, partly
         // idle wave leaves free; tail(k) runs under big(k-1)'s predecessors likewise.  What chain(k-1) writes and
         // big(k) / tail(k) read exists more than once and goes round with the segments; the carried gradient belongs to the
@@ -624,7 +623,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
                 SSD_TRY(cudaEventRecord(side->rec_done[cp], st));
             }
             // ---- chain(k), second half: the state gradients, which alone wait for segment k+1 (stream order: the
-            // gradient handed left, and the fp32 contributions that belong to this stream alone)
+            // gradient handed left)
             // What it writes was last read by big and tail of the segment npar before.
             SSD_TRY(cudaStreamWaitEvent(grads, side->rec_done[cp], 0));
             if (i >= npar) SSD_TRY(cudaStreamWaitEvent(grads, side->tail_done[(i - npar) % 3], 0));

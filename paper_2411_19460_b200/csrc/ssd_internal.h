@@ -104,7 +104,7 @@ struct SegParams {
     float *Gst;            // CUDA-core path: [B,ncs+1,H,P,N] slot c+1 = dLoss/d(state leaving chunk c)
     __nv_bfloat16 *Hbf;    // tensor-core path: [B,ncs,H,N,P] (transposed) state entering block c
     __nv_bfloat16 *Gbf;    // tensor-core path: [B,ncs,H,N,P] dLoss/d(state leaving block c)
-    float *hcarry;         // [B,H,P,N]     state handed from segment to segment (forward)
+    float *hcarry;         // [B,H,P,N]     state handed from segment to segment (forward; null in the backward, which does not)
     float *gcarry;         // [B,H,P,N]     state gradient handed right-to-left (backward)
     float *ghdot;          // [B,H,ncs,16]  partial sums of exp(cs_last) <Gout_c, H_in,c>
     float *ddt_dir;        // [B,H,ncs,Q]   direct part of ddt (tensor-core path: read where dt is next to zero, see bwd_finish)
@@ -185,9 +185,8 @@ enum { BC_DC = 1, BC_DB = 2 };
 
 // kernel kinds, for the launch counter and the optional per-kind timing
 enum {
-    KIND_CUMSUM = 0, KIND_CHUNK_STATE, KIND_STATE_PASS_FWD, KIND_SCAN_FWD, KIND_DSTATE,
-    KIND_STATE_PASS_BWD, KIND_BWD_DX, KIND_BWD_DC, KIND_BWD_DB, KIND_BWD_FINISH, KIND_REDUCE_DBDC,
-    KIND_FINAL, KIND_GLUE, KIND_DECODE, KIND_BWD_DBDC, KIND_CONV, KIND_NORM, KIND_COUNT
+    KIND_CHUNK_STATE = 0, KIND_STATE_PASS_FWD, KIND_SCAN_FWD, KIND_DSTATE, KIND_STATE_PASS_BWD, KIND_BWD_DX, KIND_BWD_DC, KIND_BWD_DB,
+    KIND_BWD_FINISH, KIND_FINAL, KIND_GLUE, KIND_DECODE, KIND_BWD_DBDC, KIND_CONV, KIND_NORM, KIND_COUNT
 };
 
 }  // namespace ssd

@@ -16,17 +16,6 @@ static_assert(SP_ELEMS == ssd::kStatePassElems, "one partial of <G,H> per CTA of
 namespace ssd {
 
 // ------------------------------------------------------------------ small helpers
-template <typename T> __device__ __forceinline__ float ldf(const T *p);
-template <> __device__ __forceinline__ float ldf<float>(const float *p) { return __ldg(p); }
-template <> __device__ __forceinline__ float ldf<__nv_bfloat16>(const __nv_bfloat16 *p) {
-    return __bfloat162float(*p);
-}
-template <typename T> __device__ __forceinline__ void stf(T *p, float v);
-template <> __device__ __forceinline__ void stf<float>(float *p, float v) { *p = v; }
-template <> __device__ __forceinline__ void stf<__nv_bfloat16>(__nv_bfloat16 *p, float v) {
-    *p = __float2bfloat16_rn(v);
-}
-
 __device__ __forceinline__ void add4(float4 &a, const float4 &b) {
     a.x += b.x; a.y += b.y; a.z += b.z; a.w += b.w;
 }

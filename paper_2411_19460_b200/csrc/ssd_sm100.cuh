@@ -13,12 +13,6 @@ __device__ __forceinline__ uint32_t smem_u32(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
 
-__device__ __forceinline__ unsigned long long globaltimer_ns() {
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-
 // ---------------------------------------------------------------- mbarrier
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(count) : "memory");
@@ -111,15 +105,6 @@ __device__ __forceinline__ void tc_fence_after_sync() {
 }
 
 // ---------------------------------------------------------------- TMA (tiled loads, no multicast)
-__device__ __forceinline__ void tma_prefetch_desc(const CUtensorMap *m) {
-    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(m)) : "memory");
-}
-__device__ __forceinline__ void tma_load_2d(void *dst, const CUtensorMap *m, uint64_t *bar, int x, int y) {
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
-        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(bar)), "r"(x), "r"(y)
-        : "memory");
-}
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *m, uint64_t *bar, int x, int y,
                                             int z) {
     asm volatile(
@@ -195,31 +180,9 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float *v) {
     for (int i = 0; i < 32; ++i) v[i] = __uint_as_float(r[i]);
 }
 
-// The same load without the wait: issue several, then tmem_ld_wait32() on each array before use.
-__device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, float *v) {
-    uint32_t *r = reinterpret_cast<uint32_t *>(v);
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
-          "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),
-          "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr)
-        : "memory");
-}
-// Waits for every outstanding TMEM load of this thread.  The 32 values are passed through the
-// statement as read-write operands so that the compiler cannot move a use of them above the wait;
-// call it once per array filled by tmem_ld32_nowait.
-__device__ __forceinline__ void tmem_ld_wait32(float *v) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+f"(v[0]), "+f"(v[1]), "+f"(v[2]), "+f"(v[3]), "+f"(v[4]), "+f"(v[5]), "+f"(v[6]), "+f"(v[7]), "+f"(v[8]), "+f"(v[9]), "+f"(v[10]), "+f"(v[11]), "+f"(v[12]), "+f"(v[13]), "+f"(v[14]), "+f"(v[15]), "+f"(v[16]), "+f"(v[17]), "+f"(v[18]), "+f"(v[19]), "+f"(v[20]), "+f"(v[21]), "+f"(v[22]), "+f"(v[23]), "+f"(v[24]), "+f"(v[25]), "+f"(v[26]), "+f"(v[27]), "+f"(v[28]), "+f"(v[29]), "+f"(v[30]), "+f"(v[31])
-                 :
-                 : "memory");
-}
-
-// 16-column variants of the non-waiting load and of the dependency-carrying wait.
+// 16 consecutive columns without the wait: issue several, then tmem_ld_wait16() on each array before use.  It waits for every
+// outstanding tensor-memory load of the thread; the values pass through it as read-write operands, so that the compiler cannot
+// move a use of them above it.
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float *v) {
     uint32_t *r = reinterpret_cast<uint32_t *>(v);
     asm volatile(
@@ -283,12 +246,6 @@ __device__ __forceinline__ uint64_t umma_desc_sw128(uint32_t saddr, uint32_t lbo
     return d;
 }
 
-// The same descriptor for a start address `bytes` further on (a multiple of 16; the address field is the
-// low 14 bits in units of 16 bytes and shared memory is smaller than 256 KB, so a plain add cannot carry out).
-__device__ __forceinline__ uint64_t umma_desc_advance(uint64_t desc, uint32_t bytes) {
-    return desc + (uint64_t)(bytes >> 4);
-}
-
 // Instruction descriptor for kind::f16 with bf16 A/B and fp32 accumulation.
 __device__ __forceinline__ uint32_t umma_idesc_bf16(uint32_t M, uint32_t N, bool a_mn_major, bool b_mn_major) {
     uint32_t d = 0;
@@ -302,23 +259,10 @@ __device__ __forceinline__ uint32_t umma_idesc_bf16(uint32_t M, uint32_t N, bool
     return d;
 }
 
-// D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread.
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
-                                          uint32_t accumulate) {
-    asm volatile(
-        "{\n"
-        ".reg .pred p;\n"
-        "setp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n"
-        "}\n" ::"r"(d_tmem),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
-// The same with the accumulate flag fixed at compile time, and a descriptor rebuilt from its two words.
-// The thread that issues the MMAs executes roughly one dependent instruction every five cycles, so the
-// per-MMA bookkeeping decides whether the tensor pipe stays fed: issue loops are fully unrolled and
-// advance only the low descriptor word (the 14-bit address field, in 16-byte units, never carries out).
+// D[tmem] (+)= A[smem] * B[smem]; issued by ONE thread.  The accumulate flag is fixed at compile time and a descriptor is rebuilt
+// from its two words: the thread that issues the MMAs executes roughly one dependent instruction every five cycles, so the
+// per-MMA bookkeeping decides whether the tensor pipe stays fed; issue loops are fully unrolled and advance only the low
+// descriptor word (the 14-bit address field, in 16-byte units, never carries out).
 template <bool ACCUMULATE>
 __device__ __forceinline__ void umma_bf16_fixed(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc) {
     if (ACCUMULATE)
@@ -383,12 +327,6 @@ __device__ __forceinline__ void scale8(uint4 &v, const RowScale &s) {
     v.y = scale2(v.y, s);
     v.z = scale2(v.z, s);
     v.w = scale2(v.w, s);
-}
-
-// Byte offset of the 16-byte chunk (row r, logical chunk j of 8) inside a 128B-swizzled tile whose
-// base is 1024-byte aligned and whose rows are 128 bytes.
-__device__ __forceinline__ uint32_t sw128_off(uint32_t r, uint32_t j) {
-    return r * 128u + ((j ^ (r & 7u)) << 4);
 }
 
 }  // namespace sm100

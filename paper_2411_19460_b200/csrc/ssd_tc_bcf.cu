@@ -17,7 +17,7 @@
 // Tensor memory: two score buffers and the two accumulators, 128 columns each.  The rows of a head are scaled in place for
 // the inter-block terms once its scores have been multiplied, and both terms go straight into the accumulators.
 // The head sum's second part takes dB from 2.42e-3 to 1.81e-3 of the exact one and dC from 2.64e-3 to 2.36e-3 (bf16 outputs: 1.66e-3;
-// 256-step blocks with one part: 2.39e-3, 2.62e-3) for 1.2 us of 76 (4096 steps of 80 heads, 96 CTAs).
+// 256-step blocks with one part: 2.39e-3, 2.62e-3) for 1.2 us of 76 (4096 steps of 80 heads, 64 CTAs).
 // Bound by the instruction issue of the scheduler that holds the four sub-tiles of row quarter 3.  4096 steps of 80 heads: 77 us
 // on 64 SMs (48 % of their issue slots), 94 us on 144 before, with 256-step chunks as three tiles.
 #include "ssd_internal.h"

@@ -435,8 +435,10 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 if (lane == 0) p.ghdot[((((size_t)b * p.H + h) * p.ncs + c) << 4) + w] = decay * dt;
             }
         }
+        if (carry_out) {
 #pragma unroll
-        for (int j = 0; j < 32; ++j) carry_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];
+            for (int j = 0; j < 32; ++j) carry_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];
+        }
         if (final_out) {
 #pragma unroll
             for (int j = 0; j < 32; ++j) final_out[(size_t)b * p.H * 64 * NS + so + (size_t)j * NS] = carry[j];

@@ -58,8 +58,6 @@ __host__ __device__ constexpr uint32_t sc_smem(int mode) {
     return (uint32_t)NS * 256 + sc_stages(mode) * SC_STAGE + (mode == SC_DX ? SC_XR * 16384 : 0) + 1024;
 }
 
-constexpr float kLog2e = 1.4426950408889634f;
-
 __device__ __forceinline__ float ex2f(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
