@@ -70,9 +70,13 @@ struct Plan {
 
 // Head ranges per group for the dB/dC kernel, whose CTAs are (block, head range).  The launches of two neighbouring segments run
 // at the same time, beside the other kernels, so what counts is the time on the SMs, (CTAs) x (eight head-times of set-up and
-// output plus the heads of the range), once three launches of 32 blocks (or the whole sequence, if it is shorter) make a wave
-// (measured against one launch and two: 80 heads, 4096-token segments, 7.03 -> 6.80 -> 6.72 ms a step); below that the time
-// of one CTA.  A function of the sequence alone, so the summation order of dB/dC does not depend on the segment length.
+// output plus the heads of the range), once three launches of 32 blocks (or the whole sequence, if it is shorter) make a wave;
+// below that the time of one CTA.  A function of the sequence alone, so that the summation order of dB/dC does not depend on the
+// segment length, and therefore the best for one segment length, 4096.  The backward of 32768 steps, us, with a wave out of one
+// launch of 32 blocks, of two, three and six:
+//   80 heads, seg 1024: 1580 1735 2052 3008   2048: 1317 1249 1330 1762   4096: 1182 1192 1107 1227   8192: 1244 1186 1146 1097
+//   24 heads             853  988  986 1289          759  658  658  809          685  588  595  566          650  639  640  580
+// (8 groups of 10 heads: the same within 2 %.)
 static const int kBcBlocks = 96;
 static int bc_head_split(int blocks, int groups, int hpg) {
     int best = 1;
@@ -340,7 +344,8 @@ static void set_segment(const Plan &pl, int k, SegParams &sp) {
 // Heads per CTA of the forward chain.  Two where a CTA per head would not fit one wave, and in a pipelined backward with heads
 // enough: the other kernels of a segment take longer than the chain there, so that its SM time counts and not its latency
 // (4096 steps of 80 heads: 60 us on 40 SMs against 38 on 80; in the forward, where only y is beside it, 63 us a segment
-// against 57).
+// against 57).  Backward of 65536 steps, us, one head and two per CTA: 64 heads, seg 4096 1820 and 1877, seg 8192 1720 and 1844;
+// 80 heads the same within 1 %, in 8 groups 2659 and 2604; 96 heads 2650 and 2594.  2 x 64 heads: 1 to 3 % for one.
 static int chain_heads(const Plan &pl, bool pipelined_bwd) {
     const int ctas = pl.B * pl.H;
     return pl.hpg % 2 == 0 && (ctas > kNumSMs || (pipelined_bwd && ctas > kNumSMs / 2)) ? 2 : 1;

@@ -511,10 +511,12 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm,
 }
 
 // y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
-// wait for nothing of this one, and a launch of a few microseconds is saved per segment.  N = 64 is left at two CTAs per SM: three
-// would spill, and its layers are small.
+// wait for nothing of this one, and a launch of a few microseconds is saved per segment.  Two CTAs per SM: held to the 80
+// registers of three, N = 128 spills (36 bytes stored, 120 loaded) and the forward takes 276 us instead of 233 (8192 steps of 4
+// heads, chunks of 128; 24 heads 396 and 383, chunks of 256 445 and 434), while N = 64 gains 5 % with chunks of 64 and loses 2 %
+// with longer ones.
 template <typename T, int NS, bool CB>
-__global__ void __launch_bounds__(256, NS == 64 || !CB ? 2 : 3) k_simt_y(SegParams p, SegParams nx, int n_next) {
+__global__ void __launch_bounds__(256, 2) k_simt_y(SegParams p, SegParams nx, int n_next) {
     pdl_launch_dependents();
     pdl_wait();
     __shared__ SimtTiles sm;
