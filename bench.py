@@ -92,17 +92,17 @@ def load_peaks():
 
 # ----------------------------------------------------------------------------- DRAM traffic from ncu
 # dram__bytes_read.sum + dram__bytes_write.sum per launch, from the `ncu` capture summarised in
-# profiles/ncu_all_kernels_cfg2_geometry.txt, taken at workload 2's launch geometry (one launch = 4096 tokens x
+# profiles/ncu_all_kernels.txt, taken at workload 2's launch geometry (one launch = 4096 tokens x
 # 80 heads).  A figure is used only while the kernel's source file still has the hash it had when the counters were
 # taken; for the other workloads it is scaled by tokens x heads per launch (the traffic of these kernels grows in
 # proportion).
 NCU_TRAFFIC = {
     # kernel kind: (bytes per launch, source file, sha256 of that file at capture time)
-    "bwd_dBdC": (183.6e6, "ssd_tc_bcf.cu", "05d951ddd3b1d12573fabf8612c4c4413df5aa4bd8d077bd87952e6c3c7d9632"),
-    "bwd_dx": (154.3e6, "ssd_tc_scan.cu", "b52bb89997529d34f8ca36599dac8f3931ba7b25be489e6b47094179374f7444"),
-    "chunk_scan_fwd": (100.0e6, "ssd_tc_scan.cu", "b52bb89997529d34f8ca36599dac8f3931ba7b25be489e6b47094179374f7444"),
-    "chunk_state": (55.6e6, "ssd_tc_chain.cu", "84487affb68f5deb7d2f1f3e89a247edcde310d52bb50a7538f9baa8c094eb9d"),
-    "dstate_contrib": (102.4e6, "ssd_tc_chain.cu", "84487affb68f5deb7d2f1f3e89a247edcde310d52bb50a7538f9baa8c094eb9d"),
+    "bwd_dBdC": (186.8e6, "ssd_tc_bcf.cu", "51f5a8d666b2691a66187e335a7bd4f840d22bd964f40c53ccda40da5802fac5"),
+    "bwd_dx": (157.5e6, "ssd_tc_scan.cu", "aa370c278cf8083eb45a0489ffc389bb5cd7df5b08f34d5c823e9a23a0ac9efa"),
+    "chunk_scan_fwd": (103.1e6, "ssd_tc_scan.cu", "aa370c278cf8083eb45a0489ffc389bb5cd7df5b08f34d5c823e9a23a0ac9efa"),
+    "chunk_state": (57.8e6, "ssd_tc_chain.cu", "0711662a0facb55ee7ac2037a72f4bb29c4870c36a21f70c318b14fffd514b65"),
+    "dstate_contrib": (106.7e6, "ssd_tc_chain.cu", "0711662a0facb55ee7ac2037a72f4bb29c4870c36a21f70c318b14fffd514b65"),
 }
 NCU_UNITS = 4096 * 80
 

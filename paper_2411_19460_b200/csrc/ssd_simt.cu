@@ -149,7 +149,7 @@ cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, long lo
 // One shape for all of them: a 64 x 64 output tile per CTA of 256 threads, 4 x 4 outputs per thread, operands staged 64 steps
 // of the contraction at a time as [k][64] (rows padded to 68 floats), so that a step of k costs a thread two 16-byte
 // shared-memory reads for 16 multiply-adds (packed two to an instruction).  The next stage's global loads are in flight while
-// a stage is multiplied.  Bound by the FFMA rate and the shared-memory reads beside it.
+// a stage is multiplied.  Bound by the shared-memory reads (65 % of the pipe's wavefronts in the large kernel, the FMA pipe at 44 %).
 //
 // What does not depend on the head is not done per head: C B^T is made once per group (k_simt_sums writes it, 64 x 64 causal
 // tiles), and dB / dC come from a head sum of the masked tiles, one product per CTA instead of two per head.

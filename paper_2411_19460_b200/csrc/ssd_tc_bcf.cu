@@ -18,8 +18,9 @@
 // the inter-block terms once its scores have been multiplied, and both terms go straight into the accumulators.
 // The head sum's second part takes dB from 2.42e-3 to 1.81e-3 of the exact one and dC from 2.64e-3 to 2.36e-3 (bf16 outputs: 1.66e-3;
 // 256-step blocks with one part: 2.39e-3, 2.62e-3) for 1.2 us of 76 (4096 steps of 80 heads, 64 CTAs).
-// Bound by the instruction issue of the scheduler that holds the four sub-tiles of row quarter 3.  4096 steps of 80 heads: 77 us
-// on 64 SMs (48 % of their issue slots), 94 us on 144 before, with 256-step chunks as three tiles.
+// Of what it uses, shared memory (61 % of the wavefronts of a busy SM) and the scheduler that holds the four sub-tiles of row
+// quarter 3 (56 % of its issue slots, 48 % on average) are nearest a limit; 16 warps leave the rest as latency.  4096 steps of 80
+// heads: 77 us on 64 SMs, 94 us on 144 before, with 256-step chunks as three tiles.
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
 

@@ -9,14 +9,14 @@
 // of the block's sum, and the scaling warps wait until the rows have been read.  With the scaled rows ddt was 4 to 10 % further
 // from the exact one than with blocks of 256 steps; the order costs the backward 2 us of 51.6 (4096 steps of 80 heads).
 //
-// One CTA owns one (batch, head), or in the forward two heads of a group, and walks the segment's blocks.  A block's sum does not depend on the carried state, so
-// it is made by tcgen05 one block ahead; the carry (N x 64 fp32) never leaves the registers of the eight worker warps:
+// One CTA owns one (batch, head), or in the forward two heads of a group, and walks the segment's blocks.  A block's sum does not
+// depend on the carried state, so it is made by tcgen05 one block ahead; the carry (N x 64 fp32) never leaves the registers of the eight worker warps:
 // what is written per block is its bf16 copy, the operand of the large kernels, 16 KB, where separate kernels for the
 // sums and the recurrence moved 32 KB of fp32 sums out and in again on top.  States are kept transposed here, [N][64], so
 // that a thread's slice (one n, 32 p) is contiguous and leaves through a swizzled tile by one TMA store per warp.
 //   warp 0 producer (TMA) | warp 1 MMA issuer | warps 2, 3 records (CHAIN_FWD, alternate blocks) | warps 4..11 scale the rows |
 //   warps 12..19 carry | warps 20..23 rho2 (CHAIN_BWD)
-// Bound by the chain's latency on as many SMs as there are heads: a step takes 0.85 us (backward 1.2), most of it the carry warps'
+// Bound by the chain's latency on as many SMs as there are heads: a step takes 0.8 us (backward 1.4), most of it the carry warps'
 // pack, proxy fence and store.  Storing the state with ordinary 32-byte stores instead (32 lines per warp instruction) made 24
 // heads 9 % slower, sixteen carry warps of half the width 2 %.  4096 steps of 80 heads: 38 and 54 us, where chunk sums,
 // state-gradient sums and the two passes took 28 + 12 and 37 + 24 us of the whole GPU and the large kernels now run beside it.

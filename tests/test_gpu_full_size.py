@@ -53,7 +53,7 @@ def test_config2_full_size_sampled_heads():
 def test_config2_launch_geometry_all_outputs_on_a_prefix():
     """Config 2's per-launch geometry (80 heads in one group, 4096-token segments, default path) on its first
     16384 tokens: EVERY output against the oracle, dB and dC included -- the sums over 80 heads that the fused
-    kernel forms in three head ranges and rounds once."""
+    kernel forms in head ranges."""
     cfg = CONFIGS[2].scaled(L=16384)
     errs = pu.full_parity(cfg)
     print(errs)
