@@ -852,9 +852,18 @@ __device__ __forceinline__ void reduce_dbdc(const SegParams &p, int id) {
         // CUDA-core path: per head range, of a row of tile rt, dC slots 0 .. rt, dB slots rt + 1 .. tiles, then the inter-chunk terms
         const int rt = (int)(tl % (size_t)p.Q) >> 6;
         for (int s0 = 0; s0 < p.nsl; s0 += p.tiles + 3) {
-            for (int t = 0; t <= p.tiles; ++t) add4(t <= rt ? sC : sB, ld(p.pC + src + (size_t)(s0 + t) * p.N));
-            add4(sC, ld(p.pC + src + (size_t)(s0 + p.tiles + 1) * p.N));
-            add4(sB, ld(p.pC + src + (size_t)(s0 + p.tiles + 2) * p.N));
+            float4 v[5];                                // all of a range's loads in flight
+#pragma unroll
+            for (int t = 0; t < 5; ++t)
+                if (t <= p.tiles) v[t] = ld(p.pC + src + (size_t)(s0 + t) * p.N);
+            const float4 interC = ld(p.pC + src + (size_t)(s0 + p.tiles + 1) * p.N), interB = ld(p.pC + src + (size_t)(s0 + p.tiles + 2) * p.N);
+#pragma unroll
+            for (int t = 0; t < 5; ++t) {
+                if (t <= rt) add4(sC, v[t]);
+                else if (t <= p.tiles) add4(sB, v[t]);
+            }
+            add4(sC, interC);
+            add4(sB, interB);
         }
     } else {
         for (int s = 0; s < p.nsl; ++s) {
