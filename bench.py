@@ -369,7 +369,7 @@ def measure_layer(args, rep, dev, cfg, full=True):
         step_roof = dict(flops_per_token=fl, bytes_per_token=by, roofline_ms=t_roof * 1e3,
                          frac=t_roof * 1e3 / ms_per_step, peaks="bf16 tensor (burst) and HBM copy, " + peaks["source"])
     else:
-        # fp32 mode runs on the CUDA cores (TF32 cannot hold 1e-4): its flop roof is the plain FFMA rate, measured here
+        # fp32 operands go to the tensor cores as three bf16 parts (TF32 cannot hold 1e-4); the roof stays the plain FFMA rate, measured here
         ffma = measure_ffma_tflops(dev)
         t_roof = max(fl * tokens / (ffma * 1e12), by * tokens / (peaks["hbm_gbs"] * 1e9))
         step_roof = dict(flops_per_token=fl, bytes_per_token=by, roofline_ms=t_roof * 1e3,
@@ -471,7 +471,7 @@ def measure_layer(args, rep, dev, cfg, full=True):
     avg_s = dom_ms * 1e-3 / max(dom_n, 1)
     peak_kind = "HBM copy"
     if bound == "tensor" and cfg.dtype != "bf16":
-        # the fp32 mode runs these contractions on the CUDA cores: plain-ALU bound, against the measured FFMA rate
+        # fp32 contractions (three bf16 parts per operand on the tensor cores) against the measured FFMA rate
         bound = "alu"
         achieved = fl_tok * tok_per_launch / avg_s / 1e12
         peak = measure_ffma_tflops(dev)
@@ -957,7 +957,7 @@ def main():
     ap.add_argument("--config", type=int, default=None, help="index into the five workloads (default: the largest "
                     "single-layer one, 4, with workloads 2 and 0 reported beside it)")
     ap.add_argument("--seg", type=int, default=0, help="override the segment length")
-    ap.add_argument("--simt", action="store_true", help="force the CUDA-core kernels")
+    ap.add_argument("--simt", action="store_true", help="force the split-path kernels")
     ap.add_argument("--layer-interval", type=int, default=1, help="config 3: keep the input of every l-th layer")
     ap.add_argument("--stack-len", type=int, default=0, help="config 3: sequence length (default 131072 at layer interval 1, else the configuration's own)")
     ap.add_argument("--stream-len", type=int, default=0, help="forward-only streaming over this many tokens "

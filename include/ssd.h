@@ -53,7 +53,7 @@ enum { SSD_DTYPE_F32 = 0, SSD_DTYPE_BF16 = 1 };
 
 /* shape.flags */
 enum {
-    SSD_FLAG_FORCE_SIMT = 1,       /* bf16 I/O: use the CUDA-core kernels instead of the tensor-core ones */
+    SSD_FLAG_FORCE_SIMT = 1,       /* bf16 I/O: use the kernels that keep their intermediates in fp32 */
     SSD_FLAG_ACCUM_PARAM_GRADS = 2,/* ssd_bwd_segmented: dA and dD are added to, not overwritten (a driver that
                                       back-propagates one grid cell at a time sums them over the cells) */
     SSD_FLAG_SKIP_GRAD = 16,       /* ssd_bwd_segmented: dx += dy, the gradient that a skip connection around the layer
@@ -105,9 +105,9 @@ typedef struct ssd_shape {
  * seg/chunk (the per-segment chunk states: the "grid cell" term of Eq. 4), not with L, apart from
  * 20 bytes per (batch, head, chunk) of dA/dD partial sums in the backward.  With two segments or more
  * there are second and third copies of what neighbouring segments' kernels touch at the same time (tensor-core
- * path: 3 times the forward's and 2.5 times the backward's scratch; CUDA-core path: up to 64 MiB more in
+ * path: 3 times the forward's and 2.5 times the backward's scratch; split path: up to 64 MiB more in
  * the forward), unless shape->flags has SSD_FLAG_SERIAL: size the buffer with the flags the call will use.
- * The CUDA-core path also keeps the products C B^T of a segment, 4 B G chunk seg bytes (not in ssd_fwd_static_ws
+ * The split path also keeps the products C B^T of a segment, 4 B G chunk seg bytes (not in ssd_fwd_static_ws
  * where they do not fit).
  * The tensor-core path takes bf16 calls with N = 128, chunk = 256 and an even H/G; its states, masked tiles and
  * decayed rows are bf16 between the kernels (fp32 outputs within 2e-3).  All other calls, and those with
@@ -145,7 +145,7 @@ int ssd_fwd(const ssd_shape_t *shape, const void *x, const float *dt, const floa
  *    second copies).  Returns SSD_ETOOLARGE, with nothing enqueued, when that layout exceeds
  *    SSD_STATIC_WS_BYTES: shrink `seg` (scratch grows with seg/chunk, not with L) or use ssd_fwd with your
  *    own buffer.  Tensor-core path: ssd_workspace_bytes(shape with SSD_FLAG_SERIAL set, SSD_OP_FWD) bytes.
- *    CUDA-core path: 256 + 8 B H seg + 4 B H P N (seg/chunk + 2) bytes, each part rounded up to 256; that is
+ *    split path: 256 + 8 B H seg + 4 B H P N (seg/chunk + 2) bytes, each part rounded up to 256; that is
  *    ssd_workspace_bytes without the products C B^T (4 B G chunk seg bytes), which the kernels make again
  *    where they do not fit.
  *  - The first call on each device looks up the device address of the built-in array (with that

@@ -61,9 +61,9 @@ struct Layout {
 static const int kMinSegmentsForTwins = 4;
 
 struct Plan {
-    int B, L, H, P, N, G, Q, seg, nseg, ncs, nct, hpg, nsl, dtype;   // Q: steps per chunk (CUDA cores) or block (tensor cores)
+    int B, L, H, P, N, G, Q, seg, nseg, ncs, nct, hpg, nsl, dtype;   // Q: steps per chunk (split path) or block (tensor cores)
     bool use_tc, serial;
-    bool keep_cb;          // CUDA cores: the scratch holds C B^T (always, except in the built-in one)
+    bool keep_cb;          // split path: the scratch holds C B^T (always, except in the built-in one)
     int64_t x_bs, dt_bs, bc_bs;
     size_t esz;
 };
@@ -93,7 +93,7 @@ static int bc_head_split(int blocks, int groups, int hpg) {
     return best;
 }
 
-// The same for the CUDA-core kernel, whose ranges have Q/64 + 3 slots each: ranges of four heads, of two where there are few, so
+// The same for the kernel of the split path, whose ranges have Q/64 + 3 slots each: ranges of four heads, of two where there are few, so
 // that a short sequence has CTAs enough (8 heads, 256-step chunks, backward: 2048 steps 265 us, with half the ranges 320; 4096
 // steps 353 and 341).  Long ones (64 chunks and more, counted per group) have them anyway, and the slots cost time and memory:
 // there no more of them than two per head, what a slice for each head would take (2 x 8192 steps of 8 heads 999 -> 918 us, 8192 of
@@ -146,7 +146,7 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
     return SSD_OK;
 }
 
-// CUDA cores: whether the sums of a segment ride in a launch of its neighbour.  In the forward that takes second copies of states
+// split path: whether the sums of a segment ride in a launch of its neighbour.  In the forward that takes second copies of states
 // and C B^T, up to 64 MiB of them: 17 MiB are worth 7 % (24 heads, 2048-step segments, 868 -> 803 us), 20 MiB 10 % (80 heads,
 // 1024 steps, 1544 -> 1391), 38 MiB 6 %, 74 MiB 2 % (80 heads, 4096 steps, 1351 -> 1326).
 static bool simt_overlap(const Plan &pl, bool bwd) {

@@ -49,7 +49,7 @@ template <auto K> inline cudaError_t allow_smem(int bytes) {
 #endif
 
 constexpr int kNumSMs = 148;
-constexpr int kStatePassElems = 512;   // state elements per CTA of the CUDA-core state passes
+constexpr int kStatePassElems = 512;   // state elements per CTA of the state passes
 constexpr int kTcBlock = 128;     // steps per block of the tensor-core path, half the caller's chunk
 constexpr int kTcState = 128;     // its state size N
 
@@ -79,12 +79,12 @@ struct SegParams {
     int c0;        // global index of the segment's first chunk
     int ncs;       // chunk capacity of the workspace (chunks of a full segment)
     int nct;       // chunks in the whole sequence (L / Q)
-    int nsl;       // slices per group in the dB/dC partial buffers: head ranges, or slots of all ranges (CUDA-core path)
+    int nsl;       // slices per group in the dB/dC partial buffers: head ranges, or slots of all ranges (split path)
     int ndd;       // partial sums of dD per (head, chunk) that the kernels of this path write (<= 4)
     int scan_ctas; // CTAs of the y / dx kernel, at most (no effect on results)
     int chain_heads; // heads per CTA of the forward chain, 1 or 2 (no effect on results)
     int ngh;       // partial sums of <G,H> per (head, chunk) (<= 16)
-    int tiles;     // CUDA-core path: 64-step tiles per chunk (rho, psi and the slices come per tile); tensor-core path: 0
+    int tiles;     // split path: 64-step tiles per chunk (rho, psi and the slices come per tile); tensor-core path: 0
     float dx_skip;    // 1 when dx also takes dy (a skip connection around the layer), else 0
     int64_t x_bs, dt_bs, bc_bs;  // batch strides, elements
 
@@ -97,23 +97,23 @@ struct SegParams {
     // workspace regions (all fp32 unless noted)
     unsigned int *status;  // [0] = error flag of bounded waits
     float *rec;            // tensor-core path: [B,H,ncs,REC_FLOATS]
-    float *cs;             // CUDA-core path: [B,H,ncs,Q] inclusive cumsum of dt*A inside each chunk
+    float *cs;             // split path: [B,H,ncs,Q] inclusive cumsum of dt*A inside each chunk
     float *dtT;            // dt head-major, vector of (b, h, c) at dt_stride floats: [B,H,ncs,Q], or inside the records
     int dt_stride;
-    float *Hst;            // CUDA-core path: [B,ncs+1,H,P,N] slot c = state entering chunk c; slot nc = leaving the segment
-    float *Gst;            // CUDA-core path: [B,ncs+1,H,P,N] slot c+1 = dLoss/d(state leaving chunk c)
+    float *Hst;            // split path: [B,ncs+1,H,P,N] slot c = state entering chunk c; slot nc = leaving the segment
+    float *Gst;            // split path: [B,ncs+1,H,P,N] slot c+1 = dLoss/d(state leaving chunk c)
     __nv_bfloat16 *Hbf;    // tensor-core path: [B,ncs,H,N,P] (transposed) state entering block c
     __nv_bfloat16 *Gbf;    // tensor-core path: [B,ncs,H,N,P] dLoss/d(state leaving block c)
     float *hcarry;         // [B,H,P,N]     state handed from segment to segment (forward; null in the backward, which does not)
     float *gcarry;         // [B,H,P,N]     state gradient handed right-to-left (backward)
     float *ghdot;          // [B,H,ncs,16]  partial sums of exp(cs_last) <Gout_c, H_in,c>
     float *ddt_dir;        // [B,H,ncs,Q]   direct part of ddt (tensor-core path: read where dt is next to zero, see bwd_finish)
-    float *cbt;            // CUDA-core path: [B,ncs,G,Q,Q] C B^T, causal 64 x 64 tiles (null: made again where used, y in order only)
-    float *rho;            // [B,H,ncs,Q]   C_t . (intra-chunk part of this head's dC_t); CUDA-core path: [B,H,ncs,tiles,Q] by column tile
+    float *cbt;            // split path: [B,ncs,G,Q,Q] C B^T, causal 64 x 64 tiles (null: made again where used, y in order only)
+    float *rho;            // [B,H,ncs,Q]   C_t . (intra-chunk part of this head's dC_t); split path: [B,H,ncs,tiles,Q] by column tile
     float *rho2;           // [B,H,ncs,Q]   C_t . (inter-chunk part of this head's dC_t)
-    float *psi;            // [B,H,ncs,Q]   B_t . (intra-chunk part of this head's dB_t); CUDA-core path: [B,H,ncs,tiles,Q] by row tile
+    float *psi;            // [B,H,ncs,Q]   B_t . (intra-chunk part of this head's dB_t); split path: [B,H,ncs,tiles,Q] by row tile
     float *psi2;           // [B,H,ncs,Q]   B_t . (inter-chunk part of this head's dB_t)
-    float *pB, *pC;        // [B,seg,G,nsl,N] partial dB / dC; CUDA-core path: one buffer, pC, for both
+    float *pB, *pC;        // [B,seg,G,nsl,N] partial dB / dC; split path: one buffer, pC, for both
     float *dAp;            // [B,H,nct]     per-chunk partial of dA
     float *dDp;            // [B,H,nct,4]   partials of dD, the first ndd of each group in use
 };
@@ -121,7 +121,7 @@ struct SegParams {
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
 // ---- kernel launchers (each returns the cudaError_t of its launch) ----
-// ssd_simt.cu : CUDA-core kernels, any I/O dtype
+// ssd_simt.cu : kernels of the split path (fp32 operands as bf16 parts), any I/O dtype
 // SIMT_SUMS: chunk sums, cumsum and C B^T | SIMT_SUMS_GRAD: also the state-gradient sums | SIMT_Y: y, and the sums of segment
 // `next` if given | SIMT_BWD: dx, slices of dB and dC | SIMT_TAIL: finishing steps and the sums (with gradients) of segment `next`
 enum { SIMT_SUMS = 0, SIMT_SUMS_GRAD, SIMT_Y, SIMT_BWD, SIMT_TAIL };

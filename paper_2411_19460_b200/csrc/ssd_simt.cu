@@ -1,11 +1,13 @@
-// CUDA-core kernels of libssd: the backward's finishing scans and reductions for every path, and inter-chunk state passing
-// and FFMA versions of the contractions, which serve the fp32 mode (1e-4 parity rules out reduced-precision tensor-core
-// inputs) and chunks of 64, and cross-check the tensor-core kernels.
+// The split path: the kernels of fp32 calls (1e-4 parity rules out operands rounded to 16 bits or TF32), of bf16 calls whose
+// intermediates stay in fp32, and a cross-check of the tensor-core kernels.  fp32 operands go to the tensor cores as three bf16
+// parts (ssd_split.cuh).  Also here: inter-chunk state passing of that path, and the backward's finishing scans and reductions of
+// every path.
 //
 // Notation per (batch b, head h), chunk of Q steps: a_t = dt_t*A_h, cs_t = inclusive cumsum of a
 // inside the chunk, H_in = state entering the chunk, Gout = dLoss/d(state leaving the chunk).
 // All of it is Eq. 1 of the paper regrouped by chunks; the segment hand-off is Algorithms 1 and 2.
 #include "ssd_internal.h"
+#include "ssd_split.cuh"
 
 // State-pass CTAs: 128 threads, at most 48 registers, so that a segment's CTAs are resident at once; chunks fetched ahead.
 #define SP_THREADS 128
@@ -14,6 +16,10 @@
 #define SP_PF 4
 static_assert(SP_ELEMS == ssd::kStatePassElems, "one partial of <G,H> per CTA of the backward pass");
 namespace ssd {
+
+// the finishing step: heads per CTA, its shared-memory tile
+constexpr int FIN_HB = 8;
+constexpr int FIN_TILE = 256 * (FIN_HB + 1);
 
 // ------------------------------------------------------------------ small helpers
 __device__ __forceinline__ void add4(float4 &a, const float4 &b) {
@@ -145,18 +151,25 @@ cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, long lo
     return launch_pdl(k_state_pass<true>, grid, dim3(SP_THREADS), 0, st, p, init, init_bs, nullptr, 0, nullptr, ginit, gleft);
 }
 
-// ------------------------------------------------------------------ FFMA contractions
-// One shape for all of them: a 64 x 64 output tile per CTA of 256 threads, 4 x 4 outputs per thread, operands staged 64 steps
-// of the contraction at a time as [k][64] (rows padded to 68 floats), so that a step of k costs a thread two 16-byte
-// shared-memory reads for 16 multiply-adds (packed two to an instruction).  The next stage's global loads are in flight while
-// a stage is multiplied.  Bound by the shared-memory reads (65 % of the pipe's wavefronts in the large kernel, the FMA pipe at 44 %).
+// ------------------------------------------------------------------ contractions
+// One shape for all of them: a 64 x 64 output tile per CTA of eight warps, 64 steps of the contraction at a time, on the tensor
+// cores with fp32 operands as three bf16 parts (ssd_split.cuh): three products where the other operand is bf16 as it stands, six
+// where both are fp32, one where neither is.  Operands are staged as rows, split on the way; the next stage's global loads are in
+// flight while a stage is multiplied.  With FFMA on the CUDA cores (4 x 4 outputs per thread, bound by the shared-memory reads) the
+// large kernel took 309 us (2 x 2048 steps of 32 heads, N = 64, chunk 128, bf16) and 215 us (2 x 1024 of 24, N = 128, fp32), now 139 and
+// 143.  Bound by latency at 16 warps per SM (issue 45, 38 %, tensor pipe 25, 45 %, shared memory 45, 49 %); held to the 80 registers of
+// three CTAs per SM it spills and takes the same time.
 //
 // What does not depend on the head is not done per head: C B^T is made once per group (k_simt_sums writes it, 64 x 64 causal
 // tiles), and dB / dC come from a head sum of the masked tiles, one product per CTA instead of two per head.
-constexpr int ST_LD = 68;
-struct SimtTiles {
-    float a[64][ST_LD], b[64][ST_LD];
+template <typename T> struct SimtSmem {
+    static constexpr int PT = SplitParts<T>::n;      // parts of a value of the caller's tensors
+    SplitTile t[3 + PT];
+    float css[256], dts[256], fac[256], red[6][64];
 };
+constexpr int ST_LD = 72;                            // floats per row of an output tile staged in t[0], t[1]
+static_assert(64 * ST_LD * sizeof(float) <= 2 * sizeof(SplitTile), "an fp32 output tile in the place of two parts");
+static_assert(FIN_TILE * sizeof(float) <= 2 * sizeof(SplitTile), "the finishing step's tile");
 
 template <typename T> __device__ __forceinline__ float4 ld4f(const T *p);
 template <> __device__ __forceinline__ float4 ld4f<float>(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
@@ -166,68 +179,21 @@ template <> __device__ __forceinline__ float4 ld4f<__nv_bfloat16>(const __nv_bfl
     const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&v.y));
     return make_float4(a.x, a.y, b.x, b.y);
 }
-
-// A 64 x 64 tile of a row-major matrix on its way to shared memory: four float4 per thread.
-//   direct:     row = tid / 16 + 16 k, columns (tid % 16) * 4 ..            -> s[row][col]      (rows run along k)
-//   transposed: row = tr_row(), columns tr_col(k) ..                        -> s[col][row]      (columns run along k)
-// (a warp of the transposed store holds 16 rows of two column groups, 4 x 68 floats = 16 banks apart: no conflicts; eight rows of
-// four groups conflicted two ways)
-__device__ __forceinline__ int tr_row() { return (threadIdx.x & 15) + 16 * ((threadIdx.x >> 5) & 3); }
-__device__ __forceinline__ int tr_col(int k) { return ((threadIdx.x >> 4) & 1) * 4 + (threadIdx.x >> 7) * 8 + 16 * k; }
-template <typename T> __device__ __forceinline__ void tile_load(float4 (&r)[4], const T *src, size_t stride, bool transposed) {
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (!transposed) r[k] = ld4f(src + (size_t)((tid >> 4) + 16 * k) * stride + (tid & 15) * 4);
-        else r[k] = ld4f(src + (size_t)tr_row() * stride + tr_col(k));
-    }
+__device__ __forceinline__ float2 ld2f(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
+__device__ __forceinline__ float2 ld2f(const __nv_bfloat16 *p) {
+    const uint32_t v = __ldg(reinterpret_cast<const uint32_t *>(p));
+    return make_float2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
-// The same from scratch that an earlier kernel of the call wrote: coherent loads.
-__device__ __forceinline__ void tile_load_ws(float4 (&r)[4], const float *src, size_t stride, bool transposed) {
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const float *q = !transposed ? src + (size_t)((tid >> 4) + 16 * k) * stride + (tid & 15) * 4
-                                     : src + (size_t)tr_row() * stride + tr_col(k);
-        r[k] = *reinterpret_cast<const float4 *>(q);
-    }
-}
-__device__ __forceinline__ void tile_store(float (*s)[ST_LD], const float4 (&r)[4], bool transposed) {
-    const int tid = threadIdx.x;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        if (!transposed) {
-            *reinterpret_cast<float4 *>(&s[(tid >> 4) + 16 * k][(tid & 15) * 4]) = r[k];
-        } else {
-            const int row = tr_row(), c = tr_col(k);
-            s[c][row] = r[k].x; s[c + 1][row] = r[k].y; s[c + 2][row] = r[k].z; s[c + 3][row] = r[k].w;
-        }
-    }
-}
-// acc[i][j] += sum_k a[k][4 ty + i] b[k][4 tx + j]
-__device__ __forceinline__ void tile_mma(float2 (&acc)[4][2], const float (*a)[ST_LD], const float (*b)[ST_LD]) {
-    const int ty = threadIdx.x >> 4, tx = threadIdx.x & 15;
-#pragma unroll 8
-    for (int k = 0; k < 64; ++k) {
-        const float4 av = *reinterpret_cast<const float4 *>(&a[k][ty * 4]), bv = *reinterpret_cast<const float4 *>(&b[k][tx * 4]);
-        const float am[4] = {av.x, av.y, av.z, av.w};
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float2 a2 = make_float2(am[i], am[i]);
-            acc[i][0] = __ffma2_rn(a2, make_float2(bv.x, bv.y), acc[i][0]);
-            acc[i][1] = __ffma2_rn(a2, make_float2(bv.z, bv.w), acc[i][1]);
-        }
-    }
-}
-__device__ __forceinline__ void zero_acc(float2 (&acc)[4][2]) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
-}
-// sum over the 16 lanes of a half warp that share ty
+// sum over the 16 lanes of a half warp
 __device__ __forceinline__ float sum_tx(float v) {
 #pragma unroll
     for (int off = 8; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
     return v;
+}
+// sum over the four lanes that share an accumulator row
+__device__ __forceinline__ float sum_quad(float v) {
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    return v + __shfl_xor_sync(0xffffffffu, v, 2);
 }
 // causal tile pair number -> (row tile, column tile), column <= row
 __device__ __forceinline__ void pair_of(int idx, int &rt, int &ct) {
@@ -239,6 +205,25 @@ __device__ __forceinline__ void pair_of(int idx, int &rt, int &ct) {
 __device__ __forceinline__ float *cb_of(const SegParams &p, int b, int c, int g) {
     return p.cbt + (((size_t)b * p.ncs + c) * p.G + g) * (size_t)(p.Q * p.Q);
 }
+// an output tile in accumulator layout to rows of `stride` floats: four lanes fill a 32-byte sector
+template <bool SPLIT = true> __device__ __forceinline__ void store_acc(const Acc &acc, float *out, size_t stride) {
+#pragma unroll
+    for (int half = 0; half < 2; ++half)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            *reinterpret_cast<float2 *>(out + (size_t)acc_row(half) * stride + acc_col(j)) = acc.get<SPLIT>(j, half);
+}
+// two neighbouring elements of an accumulator-layout tile as three parts
+__device__ __forceinline__ void put_acc(SplitTile *s, int half, int j, float a, float b) {
+    uint32_t w[3];
+    split2(a, b, w);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) *reinterpret_cast<uint32_t *>(&s[q].v[acc_row(half)][acc_col(j)]) = w[q];
+}
+
+// Up to this decay (natural units) inside a 64-step tile the mask on its diagonal is a product of two factors, beyond it an
+// exponential per element.  Factors of arguments up to 8 are rounded like cumulative sums of that size.
+constexpr float kMildTile = 8.f;
 
 // What a segment's chunks need before the states can be passed on, by block number:
 //   S_c[p,n] = sum_s exp(cs_last - cs_s) dt_s x_s[p] B_s[n]     -> Hst slot c+1   (and cs, dtT)
@@ -248,13 +233,15 @@ template <typename T, int NS> __host__ __device__ __forceinline__ int simt_n_sum
     const int nrt = p.Q >> 6;
     return p.nc * p.B * ((NS / 64) * p.H * (grads ? 2 : 1) + (p.cbt ? p.G * (nrt * (nrt + 1) / 2) : 0));
 }
-template <typename T, int NS> __device__ __forceinline__ void simt_sums(const SegParams &p, SimtTiles &sm, float *wsm, int id, bool grads) {
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, nh = NS / 64;
+template <typename T, int NS> __device__ __forceinline__ void simt_sums(const SegParams &p, SimtSmem<T> &sm, int id, bool grads) {
+    constexpr int PT = SimtSmem<T>::PT;
+    const int tid = threadIdx.x, Q = p.Q, nrt = Q >> 6, nh = NS / 64;
     const size_t HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
     const int nsum = p.nc * nh * p.H * p.B;
-    float2 acc[4][2];
-    float4 ra[4], rb[4];
-    zero_acc(acc);
+    float *wsm = sm.css;
+    Acc acc;
+    TileRegs<T> ra, rb;
+    acc.zero();
     const bool dst = grads && id >= nsum && id < 2 * nsum;
     if (dst) id -= nsum;
     else if (id >= nsum) {      // a causal tile of C B^T
@@ -267,18 +254,15 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
         const size_t o = (size_t)b * p.bc_bs + ((size_t)p.t0 + (size_t)c * Q) * GN + (size_t)g * NS;
         const T *C = (const T *)p.Cm + o + (size_t)rt * 64 * GN, *Bp = (const T *)p.Bm + o + (size_t)ct * 64 * GN;
         for (int k0 = 0; k0 < NS; k0 += 64) {
-            tile_load(ra, C + k0, GN, true);
-            tile_load(rb, Bp + k0, GN, true);
+            tile_load(ra, C + k0, GN);
+            tile_load(rb, Bp + k0, GN);
             if (k0) __syncthreads();
-            tile_store(sm.a, ra, true);
-            tile_store(sm.b, rb, true);
+            tile_store(sm.t, ra);
+            tile_store(sm.t + PT, rb);
             __syncthreads();
-            tile_mma(acc, sm.a, sm.b);
+            tile_mma<PT, PT, false, false>(acc, sm.t, sm.t + PT);
         }
-        float *out = cb_of(p, b, c, g) + (size_t)(rt * 64 + ty * 4) * Q + ct * 64 + tx * 4;
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-            *reinterpret_cast<float4 *>(out + (size_t)i * Q) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+        store_acc<(PT > 1)>(acc, cb_of(p, b, c, g) + (size_t)rt * 64 * Q + ct * 64, Q);
         return;
     }
     const int n0 = (id % nh) * 64;
@@ -287,8 +271,8 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q;
     const T *rows = (const T *)(dst ? p.dy : p.x) + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
     const T *cols = (const T *)(dst ? p.Cm : p.Bm) + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS + n0;
-    tile_load(ra, rows, HP, false);
-    tile_load(rb, cols, GN, false);
+    tile_load(ra, rows, HP);
+    tile_load(rb, cols, GN);
     // the chunk cumsum by one warp: a lane sums its Q/32 consecutive steps in order, then a shuffle scan over the lanes
     if (tid < 32) {
         const int per = Q >> 5;
@@ -327,32 +311,31 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
     __syncthreads();
     for (int s0 = 0; s0 < Q; s0 += 64) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            const float w = wsm[s0 + ty + 16 * k];
-            ra[k].x *= w; ra[k].y *= w; ra[k].z *= w; ra[k].w *= w;
+        for (int k = 0; k < TileRegs<T>::N; ++k) {
+            const float w = wsm[s0 + ra.row(k)];
+            float f[TileRegs<T>::COLS];
+            ra.get(k, f);
+#pragma unroll
+            for (int i = 0; i < TileRegs<T>::COLS; ++i) f[i] *= w;
+            put_split(sm.t, ra.row(k), ra.col(), f);
         }
-        tile_store(sm.a, ra, false);
-        tile_store(sm.b, rb, false);
+        tile_store(sm.t + 3, rb);
         __syncthreads();
         if (s0 + 64 < Q) {
-            tile_load(ra, rows + (size_t)(s0 + 64) * HP, HP, false);
-            tile_load(rb, cols + (size_t)(s0 + 64) * GN, GN, false);
+            tile_load(ra, rows + (size_t)(s0 + 64) * HP, HP);
+            tile_load(rb, cols + (size_t)(s0 + 64) * GN, GN);
         }
-        tile_mma(acc, sm.a, sm.b);
+        tile_mma<3, PT, true, true>(acc, sm.t, sm.t + 3);
         __syncthreads();
     }
-    float *out = (dst ? p.Gst + slot_off(p, b, c, h) : p.Hst + slot_off(p, b, c + 1, h)) + (size_t)(ty * 4) * NS + n0 + tx * 4;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-        *reinterpret_cast<float4 *>(out + (size_t)i * NS) = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+    store_acc(acc, (dst ? p.Gst + slot_off(p, b, c, h) : p.Hst + slot_off(p, b, c + 1, h)) + n0, NS);
 }
 
-template <typename T, int NS> __global__ void __launch_bounds__(256, 3) k_simt_sums(SegParams p, bool grads) {
+template <typename T, int NS> __global__ void __launch_bounds__(256, 2) k_simt_sums(SegParams p, bool grads) {
+    extern __shared__ __align__(16) unsigned char smem[];
     pdl_launch_dependents();
     pdl_wait();
-    __shared__ SimtTiles sm;
-    __shared__ float wsm[256];
-    simt_sums<T, NS>(p, sm, wsm, blockIdx.x, grads);
+    simt_sums<T, NS>(p, *reinterpret_cast<SimtSmem<T> *>(smem), blockIdx.x, grads);
 }
 
 // One 64-row tile of y (DX = false) or of dx (DX = true) of one head:
@@ -362,173 +345,192 @@ template <typename T, int NS> __global__ void __launch_bounds__(256, 3) k_simt_s
 // CB false (y only): the tiles of C B^T are not in the scratch and are made here, per head, with the same operations in the same
 // order, so with the same bits.
 template <typename T, int NS, bool DX, bool CB>
-__device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtTiles &sm, float *css, float *dts, float *fac, float *red, int c, int rt, int h, int b) {
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, g = h / p.hpg, r0 = rt * 64;
+__device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &sm, int c, int rt, int h, int b) {
+    constexpr int PT = SimtSmem<T>::PT;
+    float *css = sm.css, *dts = sm.dts, *fac = sm.fac, *facd = sm.red[5];
+    const int tid = threadIdx.x, Q = p.Q, nrt = Q >> 6, g = h / p.hpg, r0 = rt * 64;
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q, HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
     const size_t xo = (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
     const T *vals = (const T *)(DX ? p.dy : p.x) + xo;
     const T *rowv = (const T *)(DX ? p.Bm : p.Cm) + (size_t)b * p.bc_bs + (tok0 + r0) * GN + (size_t)g * NS;
     const float *St = DX ? p.Gst + slot_off(p, b, c + 1, h) : p.Hst + slot_off(p, b, c, h), *cbt = cb_of(p, b, c, g);
-    float4 ra[4], rb[4];
-    float2 acc[4][2];
-    zero_acc(acc);
-    tile_load(ra, rowv, GN, true);
-    tile_load_ws(rb, St, NS, true);
+    TileRegs<T> rv;
+    TileRegs<float> rf;
+    Acc acc;
+    acc.zero();
+    tile_load(rv, rowv, GN);
+    tile_load<true>(rf, St, NS);
     for (int t = tid; t < Q; t += 256) {
         css[t] = p.cs[vec_off(p, b, h, c) + t];
         dts[t] = p.dtT[vec_off(p, b, h, c) + t];
     }
-    auto load_vals = [&](int ct) {      // CB tile and value rows of column tile ct
-        // DX = false: rows t = r0 .., columns s = 64 ct .. ; DX = true: the tile's rows are the CB matrix's columns
-        if (!DX && CB) tile_load_ws(ra, cbt + (size_t)r0 * Q + ct * 64, Q, true);
-        else if (DX) tile_load_ws(ra, cbt + (size_t)ct * 64 * Q + r0, Q, false);
-        tile_load(rb, vals + (size_t)ct * 64 * HP, HP, false);
+    // CB tile and value rows of column tile ct: rows t, columns s of the CB matrix; for dx its columns are the output's rows
+    auto load_vals = [&](int ct) {
+        if (CB) tile_load<true>(rf, DX ? cbt + (size_t)ct * 64 * Q + r0 : cbt + (size_t)r0 * Q + ct * 64, Q);
+        tile_load(rv, vals + (size_t)ct * 64 * HP, HP);
     };
     const int ct0 = DX ? rt : 0, ct1 = DX ? nrt : rt + 1;
     for (int k0 = 0; k0 < NS; k0 += 64) {
-        tile_store(sm.a, ra, true);
-        tile_store(sm.b, rb, true);
+        tile_store(sm.t, rv);
+        tile_store(sm.t + PT, rf);
         __syncthreads();
         if (k0 + 64 < NS) {
-            tile_load(ra, rowv + k0 + 64, GN, true);
-            tile_load_ws(rb, St + k0 + 64, NS, true);
+            tile_load(rv, rowv + k0 + 64, GN);
+            tile_load<true>(rf, St + k0 + 64, NS);
         } else if (CB) {
             load_vals(ct0);
         }
-        tile_mma(acc, sm.a, sm.b);
+        tile_mma<PT, 3, false, false>(acc, sm.t, sm.t + PT);
         __syncthreads();
     }
     // Off the diagonal tile the mask factors at the tile's edge m (its first row; dx: last), where both factors are <= 1:
     // e^{cs_t-cs_s} = e^{cs_t-cs_m} e^{cs_m-cs_s}.  An exponential per step instead of one per element.
+    // On it one of the two is >= 1, and their product no worse than the difference of the cumulative sums where those are close:
+    // facd, for mild decays.
     const int m = DX ? r0 + 63 : r0;
-    if (nrt > 1) {
-        for (int t = tid; t < Q; t += 256) {
-            const float d = css[t] - css[m];
-            fac[t] = expf(fminf(t >= m ? d : -d, 0.f)) * (DX || t >= m ? 1.f : dts[t]);
-        }
-        __syncthreads();
+    const bool mild = css[r0] - css[r0 + 63] <= kMildTile;
+    for (int t = tid; t < Q; t += 256) {
+        const float d = css[t] - css[m];
+        fac[t] = expf(fminf(t >= m ? d : -d, 0.f)) * (DX || t >= m ? 1.f : dts[t]);
     }
+    if (tid < 64) facd[tid] = DX ? expf(css[r0 + tid] - css[m]) : expf(css[m] - css[r0 + tid]) * dts[r0 + tid];
+    __syncthreads();
     // the inter-chunk term is complete: scale its rows
     const float cl = css[Q - 1];
-    float dd2[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = r0 + ty * 4 + i;
+    for (int half = 0; half < 2; ++half) {
+        const int r = r0 + acc_row(half);
         const float o = DX ? expf(fminf(cl - css[r], 0.f)) : expf(css[r]);
-        acc[i][0].x *= o; acc[i][0].y *= o; acc[i][1].x *= o; acc[i][1].y *= o;
+        float dd2 = 0.f;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const float2 v = __fmul2_rn(make_float2(o, o), acc.get(j, half));
+            acc.set(j, half, v);
+            if (DX) {
+                const float2 xv = ld2f((const T *)p.x + xo + (size_t)r * HP + acc_col(j));
+                dd2 += xv.x * v.x + xv.y * v.y;
+            }
+        }
         if (DX) {
-            const float4 xv = ld4f((const T *)p.x + xo + (size_t)r * HP + tx * 4);
-            dd2[i] = xv.x * acc[i][0].x + xv.y * acc[i][0].y + xv.z * acc[i][1].x + xv.w * acc[i][1].y;
+            dd2 = sum_quad(dd2);
+            if ((tid & 3) == 0) sm.red[tid >> 7][acc_row(half)] = dd2;
         }
     }
     for (int ct = ct0; ct < ct1; ++ct) {
-        // masked tile: a[k = column of the mask][row]
         if constexpr (!CB) {
             const T *colv = (const T *)p.Bm + (size_t)b * p.bc_bs + (tok0 + ct * 64) * GN + (size_t)g * NS;
-            float2 cb[4][2];
-            zero_acc(cb);
+            Acc cb;
+            cb.zero();
             for (int k0 = 0; k0 < NS; k0 += 64) {
-                tile_load(ra, rowv + k0, GN, true);
-                tile_load(rb, colv + k0, GN, true);
-                tile_store(sm.a, ra, true);
-                tile_store(sm.b, rb, true);
+                TileRegs<T> rc;
+                tile_load(rv, rowv + k0, GN);
+                tile_load(rc, colv + k0, GN);
+                tile_store(sm.t, rv);
+                tile_store(sm.t + PT, rc);
                 __syncthreads();
-                tile_mma(cb, sm.a, sm.b);
+                tile_mma<PT, PT, false, false>(cb, sm.t, sm.t + PT);
                 __syncthreads();
             }
             load_vals(ct);
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int s = ct * 64 + tx * 4 + j;
-                float e[4];
+            for (int half = 0; half < 2; ++half)
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int t = r0 + ty * 4 + i;
-                    const float v = j < 2 ? (j ? cb[i][0].y : cb[i][0].x) : (j == 3 ? cb[i][1].y : cb[i][1].x);
-                    e[i] = ct != rt ? v * (fac[t] * fac[s]) : s <= t ? v * expf(fminf(css[t] - css[s], 0.f)) * dts[s] : 0.f;
+                for (int j = 0; j < 4; ++j) {
+                    const int t = r0 + acc_row(half), s = ct * 64 + acc_col(j);
+                    const float2 v2 = cb.template get<(PT > 1)>(j, half);
+                    float e[2] = {v2.x, v2.y};
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        if (ct != rt) e[i] *= fac[t] * fac[s + i];
+                        else if (mild) e[i] = s + i <= t ? e[i] * (fac[t] * facd[acc_col(j) + i]) : 0.f;
+                        else e[i] = s + i <= t ? e[i] * expf(fminf(css[t] - css[s + i], 0.f)) * dts[s + i] : 0.f;
+                    }
+                    put_acc(sm.t, half, j, e[0], e[1]);
                 }
-                *reinterpret_cast<float4 *>(&sm.a[tx * 4 + j][ty * 4]) = make_float4(e[0], e[1], e[2], e[3]);
-            }
-        } else if (ct != rt) {
+        } else {
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
-                const float one = fac[DX ? ct * 64 + ty + 16 * k : r0 + tr_row()];
-                const float4 four = *reinterpret_cast<const float4 *>(fac + (DX ? r0 + tx * 4 : ct * 64 + tr_col(k)));
-                ra[k].x *= one * four.x; ra[k].y *= one * four.y; ra[k].z *= one * four.z; ra[k].w *= one * four.w;
-            }
-        } else
+                // rows t, columns s
+                float e[4];
+                rf.get(k, e);
+                const int t = (DX ? ct * 64 : r0) + rf.row(k), s = (DX ? r0 : ct * 64) + rf.col();
+                if (ct != rt || mild) {
+                    const float one = DX && ct == rt ? facd[rf.row(k)] : fac[t];
+                    const float4 four = *reinterpret_cast<const float4 *>(!DX && ct == rt ? facd + rf.col() : fac + s);
+                    e[0] *= one * four.x; e[1] *= one * four.y; e[2] *= one * four.z; e[3] *= one * four.w;
+                    if (ct == rt) {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            float *e = reinterpret_cast<float *>(&ra[k]);
+                        for (int i = 0; i < 4; ++i) e[i] = s + i <= t ? e[i] : 0.f;
+                    }
+                } else {
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                // as tile_load laid them out: not DX (transposed) row t, column s; DX (direct) row t, column s
-                const int t = DX ? ct * 64 + ty + 16 * k : r0 + tr_row();
-                const int s = DX ? r0 + tx * 4 + i : ct * 64 + tr_col(k) + i;
-                e[i] = s <= t ? e[i] * expf(fminf(css[t] - css[s], 0.f)) * (DX ? 1.f : dts[s]) : 0.f;
+                    for (int i = 0; i < 4; ++i) e[i] = s + i <= t ? e[i] * expf(fminf(css[t] - css[s + i], 0.f)) * (DX ? 1.f : dts[s + i]) : 0.f;
+                }
+                put_split(sm.t, rf.row(k), rf.col(), e);
             }
         }
-        if (CB) tile_store(sm.a, ra, !DX);
-        tile_store(sm.b, rb, false);
+        tile_store(sm.t + 3, rv);
         __syncthreads();
         if (CB && ct + 1 < ct1) load_vals(ct + 1);
-        tile_mma(acc, sm.a, sm.b);
+        tile_mma<3, PT, DX, true>(acc, sm.t, sm.t + 3);
         __syncthreads();
     }
+    // through shared memory, so that the caller's rows are read and written in whole sectors
+    float *stg = reinterpret_cast<float *>(sm.t);
+    store_acc(acc, stg, ST_LD);
+    __syncthreads();
     const float Dh = __ldg(p.D + h) + (DX ? p.dx_skip : 0.f);      // dx: D dy, plus dy itself under a skip connection
-    float dsum = 0.f;
+    float dsum = 0.f, dprev = 0.f;
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int r = r0 + ty * 4 + i;
-        const size_t o = xo + (size_t)r * HP + tx * 4;
+    for (int k = 0; k < 4; ++k) {
+        const int rl = (tid >> 4) + 16 * k, r = r0 + rl, cl4 = (tid & 15) * 4;
+        const size_t o = xo + (size_t)r * HP + cl4;
+        const float4 a = *reinterpret_cast<const float4 *>(stg + rl * ST_LD + cl4);
         const float4 v = ld4f((const T *)(DX ? p.dy : p.x) + o);
         const float s = DX ? dts[r] : 1.f;
-        st4((T *)(DX ? p.dx : p.y) + o, make_float4(fmaf(Dh, v.x, s * acc[i][0].x), fmaf(Dh, v.y, s * acc[i][0].y), fmaf(Dh, v.z, s * acc[i][1].x),
-                                                    fmaf(Dh, v.w, s * acc[i][1].y)));
+        st4((T *)(DX ? p.dx : p.y) + o, make_float4(fmaf(Dh, v.x, s * a.x), fmaf(Dh, v.y, s * a.y), fmaf(Dh, v.z, s * a.z), fmaf(Dh, v.w, s * a.w)));
         if (DX) {
             const float4 xv = ld4f((const T *)p.x + o);
-            const float dd = sum_tx(xv.x * acc[i][0].x + xv.y * acc[i][0].y + xv.z * acc[i][1].x + xv.w * acc[i][1].y);
-            const float d2 = sum_tx(dd2[i]);
-            dsum += v.x * xv.x + v.y * xv.y + v.z * xv.z + v.w * xv.w;
-            if (tx == 0) {
+            const float dd = sum_tx(xv.x * a.x + xv.y * a.y + xv.z * a.z + xv.w * a.w);
+            const float dk = (v.x * xv.x + v.y * xv.y) + (v.z * xv.z + v.w * xv.w);
+            if (k & 1) dsum += dprev + dk;
+            else dprev = dk;
+            if ((tid & 15) == 0) {
                 p.ddt_dir[vec_off(p, b, h, c) + r] = dd;
-                p.psi2[vec_off(p, b, h, c) + r] = dts[r] * d2;
+                p.psi2[vec_off(p, b, h, c) + r] = dts[r] * (sm.red[0][rl] + sm.red[1][rl]);
             }
         }
     }
     if (DX) {       // deterministic block sum of dy*x
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, off);
-        if ((tid & 31) == 0) red[tid >> 5] = dsum;
+        if ((tid & 31) == 0) sm.red[2][tid >> 5] = dsum;
         __syncthreads();
         if (tid == 0) {
             float s = 0.f;
 #pragma unroll
-            for (int w = 0; w < 8; ++w) s += red[w];
+            for (int w = 0; w < 8; ++w) s += sm.red[2][w];
             p.dDp[((((size_t)b * p.H + h) * p.nct + p.c0 + c) << 2) + rt] = s;
         }
     }
 }
 
 // y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
-// wait for nothing of this one, and a launch of a few microseconds is saved per segment.  Two CTAs per SM: held to the 80
-// registers of three, N = 128 spills (36 bytes stored, 120 loaded) and the forward takes 276 us instead of 233 (8192 steps of 4
-// heads, chunks of 128; 24 heads 396 and 383, chunks of 256 445 and 434), while N = 64 gains 5 % with chunks of 64 and loses 2 %
-// with longer ones.
+// wait for nothing of this one, and a launch of a few microseconds is saved per segment.
 template <typename T, int NS, bool CB>
 __global__ void __launch_bounds__(256, 2) k_simt_y(SegParams p, SegParams nx, int n_next) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();
     pdl_wait();
-    __shared__ SimtTiles sm;
-    __shared__ __align__(16) float css[256], dts[256], fac[256];
     const int nrt = p.Q >> 6, ny = (int)gridDim.x - n_next;
     int id = blockIdx.x;
     if (id >= ny) {
-        simt_sums<T, NS>(nx, sm, css, id - ny, false);
+        simt_sums<T, NS>(nx, sm, id - ny, false);
         return;
     }
     const int rt = id % nrt, c = (id / nrt) % p.nc, h = (id / (nrt * p.nc)) % p.H, b = id / (nrt * p.nc * p.H);
-    simt_row_tile<T, NS, false, CB>(p, sm, css, dts, fac, nullptr, c, rt, h, b);
+    simt_row_tile<T, NS, false, CB>(p, sm, c, rt, h, b);
 }
 
 // The large kernel of the backward: tiles of dx, and the partial slices of dB and dC.  Per (chunk, head range):
@@ -539,16 +541,17 @@ __global__ void __launch_bounds__(256, 2) k_simt_y(SegParams p, SegParams nx, in
 // tt + 1, then the inter-chunk terms of both.
 template <typename T, int NS>
 __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
+    constexpr int PT = SimtSmem<T>::PT;
+    extern __shared__ __align__(16) unsigned char smem[];
+    SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();
     pdl_wait();
-    __shared__ SimtTiles sm;
-    __shared__ __align__(16) float css[256], dts[256], fac[256], red[8][64];
-    const int tid = threadIdx.x, ty = tid >> 4, tx = tid & 15, Q = p.Q, nrt = Q >> 6, npair = nrt * (nrt + 1) / 2;
+    const int tid = threadIdx.x, lane = tid & 31, Q = p.Q, nrt = Q >> 6, npair = nrt * (nrt + 1) / 2;
     int id = blockIdx.x;
     if (id >= (int)gridDim.x - n_dx) {
         id -= (int)gridDim.x - n_dx;
         const int rt = id % nrt, h = (id / nrt) % p.H, c = (id / (nrt * p.H)) % p.nc, b = id / (nrt * p.H * p.nc);
-        simt_row_tile<T, NS, true, true>(p, sm, css, dts, fac, red[0], c, rt, h, b);
+        simt_row_tile<T, NS, true, true>(p, sm, c, rt, h, b);
         return;
     }
     const int per = npair + 2 * nrt, role = id % per;
@@ -559,176 +562,197 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q, HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
     const T *xb = (const T *)p.x + (size_t)b * p.x_bs + tok0 * HP, *dyb = (const T *)p.dy + (size_t)b * p.x_bs + tok0 * HP;
     const T *Bb = (const T *)p.Bm + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS, *Cb = (const T *)p.Cm + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS;
-    auto load_vec = [&](int h) {
-        for (int t = tid; t < Q; t += 256) {
-            css[t] = p.cs[vec_off(p, b, h, c) + t];
-            dts[t] = p.dtT[vec_off(p, b, h, c) + t];
-        }
+    auto slice = [&](int row0, int slot, int n0) {
+        return p.pC + ((((size_t)b * p.ncs * Q + (size_t)c * Q + row0) * p.G + g) * p.nsl + sl * (nrt + 3) + slot) * NS + n0;
     };
-    auto write_slice = [&](const float2 (&acc)[4][2], int row0, int slot, int n0) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const size_t tl = (size_t)b * p.ncs * Q + (size_t)c * Q + row0 + ty * 4 + i;
-            *reinterpret_cast<float4 *>(p.pC + ((tl * p.G + g) * p.nsl + sl * (nrt + 3) + slot) * NS + n0 + tx * 4) =
-                make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
-        }
-    };
-    float4 ra[4], rb[4];
-    float2 acc[4][2];
+    const size_t slice_stride = (size_t)p.G * p.nsl * NS;
+    Acc acc;
     if (role < npair) {
         int tt, ts;
         pair_of(role, tt, ts);
-        const float *CB = cb_of(p, b, c, g) + (size_t)(tt * 64 + ty * 4) * Q + ts * 64 + tx * 4;
-        float4 cb[4];
-        float ws[4][4];
+        TileRegs<T> ra, rb;
+        float2 cb[2][4], ws[2][4];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            cb[i] = *reinterpret_cast<const float4 *>(CB + (size_t)i * Q);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) ws[i][j] = 0.f;
-        }
-        tile_load(ra, dyb + (size_t)tt * 64 * HP + (size_t)h0 * 64, HP, true);
-        tile_load(rb, xb + (size_t)ts * 64 * HP + (size_t)h0 * 64, HP, true);
-        for (int h = h0; h < h1; ++h) {
-            load_vec(h);
-            if (tt != ts && tid < 128) {      // the mask's factors at the row tile's first step, as for y
-                const float *cs = p.cs + vec_off(p, b, h, c), ref = cs[tt * 64];
-                const int t = (tid < 64 ? tt : ts - 1) * 64 + tid;
-                fac[tid] = tid < 64 ? expf(fminf(cs[t] - ref, 0.f)) : expf(fminf(ref - cs[t], 0.f)) * p.dtT[vec_off(p, b, h, c) + t];
-            }
-            tile_store(sm.a, ra, true);
-            tile_store(sm.b, rb, true);
-            __syncthreads();
-            if (h + 1 < h1) {
-                tile_load(ra, dyb + (size_t)tt * 64 * HP + (size_t)(h + 1) * 64, HP, true);
-                tile_load(rb, xb + (size_t)ts * 64 * HP + (size_t)(h + 1) * 64, HP, true);
-            }
-            zero_acc(acc);
-            tile_mma(acc, sm.a, sm.b);
-            float col[4] = {0.f, 0.f, 0.f, 0.f};
-            const size_t vo = (vec_off(p, b, h, c) * nrt);      // rho, psi: [B,H,ncs,Q/64 tiles,Q]
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const int t = tt * 64 + ty * 4 + i;
-                const float s4[4] = {acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y}, c4[4] = {cb[i].x, cb[i].y, cb[i].z, cb[i].w};
-                float row = 0.f, e4[4];
-                if (tt != ts) {
-                    const float one = fac[ty * 4 + i];
-                    const float4 four = *reinterpret_cast<const float4 *>(fac + 64 + tx * 4);
-                    e4[0] = one * four.x; e4[1] = one * four.y; e4[2] = one * four.z; e4[3] = one * four.w;
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const int s = ts * 64 + tx * 4 + j;
-                        e4[j] = s <= t ? expf(fminf(css[t] - css[s], 0.f)) * dts[s] : 0.f;
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const float w = s4[j] * e4[j];
-                    ws[i][j] += w;
-                    // s = t adds the same to rho_t and psi_t, of which only sums of differences are used: left out of both, or with
-                    // strong decays, where it is the largest term, its rounding would be most of the error of dA
-                    const float wc = i == j && tx == ty && tt == ts ? 0.f : w;
-                    row = fmaf(wc, c4[j], row);
-                    col[j] = fmaf(wc, c4[j], col[j]);
-                }
-                row = sum_tx(row);
-                if (tx == 0) p.rho[vo + (size_t)ts * Q + t] = row;
-            }
+        for (int half = 0; half < 2; ++half)
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                col[j] += __shfl_xor_sync(0xffffffffu, col[j], 16);
-                if ((tid & 16) == 0) red[tid >> 5][tx * 4 + j] = col[j];
+                cb[half][j] = *reinterpret_cast<const float2 *>(cb_of(p, b, c, g) + (size_t)(tt * 64 + acc_row(half)) * Q + ts * 64 + acc_col(j));
+                ws[half][j] = make_float2(0.f, 0.f);
+            }
+        // a head's vectors, a value each of 128 threads: the mask's factors at the row tile's first step, as for y, or, on the
+        // diagonal of a stiff head, cumulative sum and step size
+        float *rowv = sm.fac, *colv = sm.fac + 64;
+        const bool diag = tt == ts;
+        float va = 0.f, vb = 0.f, vref, vlast;
+        auto load_head = [&](int h) {
+            tile_load(ra, dyb + (size_t)tt * 64 * HP + (size_t)h * 64, HP);
+            tile_load(rb, xb + (size_t)ts * 64 * HP + (size_t)h * 64, HP);
+            const size_t vo = vec_off(p, b, h, c);
+            if (tid < 128) {
+                const size_t o = vo + (tid < 64 ? tt : ts) * 64 + (tid & 63);
+                va = p.cs[o];
+                vb = p.dtT[o];
+            }
+            vref = p.cs[vo + tt * 64];
+            vlast = p.cs[vo + tt * 64 + 63];
+        };
+        load_head(h0);
+        for (int h = h0; h < h1; ++h) {
+            tile_store(sm.t, ra);
+            tile_store(sm.t + PT, rb);
+            const bool factors = !diag || vref - vlast <= kMildTile;
+            if (tid < 128) {
+                const float d = tid < 64 ? va - vref : vref - va, e = expf(diag ? d : fminf(d, 0.f));
+                sm.fac[tid] = factors ? (tid < 64 ? e : e * vb) : (tid < 64 ? va : vb);
             }
             __syncthreads();
-            if (tid < 64) {
-                float s = 0.f;
+            if (h + 1 < h1) load_head(h + 1);
+            acc.zero();
+            tile_mma<PT, PT, false, false>(acc, sm.t, sm.t + PT);
+            float2 row[2], col[4];
 #pragma unroll
-                for (int w = 0; w < 8; ++w) s += red[w][tid];
-                p.psi[vo + (size_t)tt * Q + ts * 64 + tid] = s;
+            for (int j = 0; j < 4; ++j) col[j] = make_float2(0.f, 0.f);
+            row[0] = row[1] = col[0];
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+                const int t = acc_row(half);
+                const float one = rowv[t];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int s = acc_col(j);
+                    const float2 two = *reinterpret_cast<const float2 *>(colv + s);
+                    float2 e;
+                    if (factors) {
+                        e = __fmul2_rn(make_float2(one, one), two);
+                    } else {
+                        e.x = expf(fminf(one - rowv[s], 0.f)) * two.x;
+                        e.y = expf(fminf(one - rowv[s + 1], 0.f)) * two.y;
+                    }
+                    float2 w = __fmul2_rn(acc.get<(PT > 1)>(j, half), e);
+                    if (diag) {
+                        w.x = s <= t ? w.x : 0.f;
+                        w.y = s < t ? w.y : 0.f;
+                    }
+                    ws[half][j] = __fadd2_rn(ws[half][j], w);
+                    // s = t adds the same to rho_t and psi_t, of which only sums of differences are used: left out of both, or with
+                    // strong decays, where it is the largest term, its rounding would be most of the error of dA
+                    if (diag) {
+                        w.x = s == t ? 0.f : w.x;
+                        w.y = s + 1 == t ? 0.f : w.y;
+                    }
+                    row[half] = __ffma2_rn(w, cb[half][j], row[half]);
+                    col[j] = __ffma2_rn(w, cb[half][j], col[j]);
+                }
+                const float r = sum_quad(row[half].x + row[half].y);
+                if ((lane & 3) == 0) sm.red[tid >> 7][t] = r;
             }
-            // red, css, dts and fac are rewritten only after the next head's first barrier or by the threads that read them here
-            __syncthreads();
-        }
-        // dC[tt] = Wsum B_ts: a[k = s][t]
+            // column sums over the warp's rows: transposing butterfly, the eight lanes of a column pair end with a column each
+            const int gl = lane >> 2;
+            float cv[8] = {col[0].x, col[0].y, col[1].x, col[1].y, col[2].x, col[2].y, col[3].x, col[3].y};
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
-            *reinterpret_cast<float4 *>(&sm.a[tx * 4 + j][ty * 4]) = make_float4(ws[0][j], ws[1][j], ws[2][j], ws[3][j]);
-        for (int n0 = 0; n0 < NS; n0 += 64) {
-            tile_load(rb, Bb + (size_t)ts * 64 * GN + n0, GN, false);
-            tile_store(sm.b, rb, false);
-            __syncthreads();
-            zero_acc(acc);
-            tile_mma(acc, sm.a, sm.b);
-            write_slice(acc, tt * 64, ts, n0);
-            __syncthreads();
-        }
-        // dB[ts] = Wsum^T C_tt: a[k = t][s]
+            for (int o = 4; o >= 1; o >>= 1) {
+                const bool up = (gl & o) != 0;
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-            *reinterpret_cast<float4 *>(&sm.a[ty * 4 + i][tx * 4]) = make_float4(ws[i][0], ws[i][1], ws[i][2], ws[i][3]);
-        for (int n0 = 0; n0 < NS; n0 += 64) {
-            tile_load(rb, Cb + (size_t)tt * 64 * GN + n0, GN, false);
-            tile_store(sm.b, rb, false);
+                for (int i = 0; i < o; ++i) {
+                    const float send = up ? cv[i] : cv[i + o], keep = up ? cv[i + o] : cv[i];
+                    cv[i] = keep + __shfl_xor_sync(0xffffffffu, send, o * 4);
+                }
+            }
+            sm.red[2 + ((tid >> 5) & 3)][acc_col(gl >> 1) + (gl & 1)] = cv[0];
             __syncthreads();
-            zero_acc(acc);
-            tile_mma(acc, sm.a, sm.b);
-            write_slice(acc, ts * 64, tt + 1, n0);
+            const size_t vo = (vec_off(p, b, h, c) * nrt);      // rho, psi: [B,H,ncs,Q/64 tiles,Q]
+            if (tid < 64) p.rho[vo + (size_t)ts * Q + tt * 64 + tid] = sm.red[0][tid] + sm.red[1][tid];
+            else if (tid < 128) p.psi[vo + (size_t)tt * Q + ts * 64 + tid - 64] = (sm.red[2][tid - 64] + sm.red[3][tid - 64]) + (sm.red[4][tid - 64] + sm.red[5][tid - 64]);
+            // red and the tiles are rewritten only after the next head's first barrier or by threads that are past this one
+        }
+        // dC[tt] = Wsum B_ts and dB[ts] = Wsum^T C_tt
+#pragma unroll
+        for (int half = 0; half < 2; ++half)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) put_acc(sm.t, half, j, ws[half][j].x, ws[half][j].y);
+        tile_load(rb, Bb + (size_t)ts * 64 * GN, GN);
+#pragma unroll 1
+        for (int n0 = 0; n0 < 2 * NS; n0 += 64) {
+            const bool isB = n0 >= NS;
+            const int n = isB ? n0 - NS : n0;
+            tile_store(sm.t + 3, rb);
+            __syncthreads();
+            if (n0 + 64 < 2 * NS) tile_load(rb, n0 + 64 >= NS ? Cb + (size_t)tt * 64 * GN + n0 + 64 - NS : Bb + (size_t)ts * 64 * GN + n0 + 64, GN);
+            acc.zero();
+            if (isB) tile_mma<3, PT, true, true>(acc, sm.t, sm.t + 3);
+            else tile_mma<3, PT, false, true>(acc, sm.t, sm.t + 3);
+            store_acc(acc, isB ? slice(ts * 64, tt + 1, n) : slice(tt * 64, ts, n), slice_stride);
             __syncthreads();
         }
         return;
     }
-    // inter-chunk terms of one row tile: the head's rows scaled per row, times the chunk state (rows p)
+    // inter-chunk terms of one row tile: the head's rows times the chunk state (rows p), the products scaled per row
     const bool isC = role - npair < nrt;
     const int rt = (role - npair) % nrt;
-    float2 tot[NS / 64][4][2];
+    TileRegs<T> ra;
+    TileRegs<float> rf;
+    float2 tot[NS / 64][2][4];
 #pragma unroll
-    for (int m = 0; m < NS / 64; ++m) zero_acc(tot[m]);
+    for (int m = 0; m < NS / 64; ++m)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) tot[m][0][j] = tot[m][1][j] = make_float2(0.f, 0.f);
+    auto state = [&](int h) { return isC ? p.Hst + slot_off(p, b, c, h) : p.Gst + slot_off(p, b, c + 1, h); };
+    const T *rows = (isC ? dyb : xb) + (size_t)rt * 64 * HP;
+    tile_load(ra, rows + (size_t)h0 * 64, HP);
+    tile_load<true>(rf, state(h0), NS);
     for (int h = h0; h < h1; ++h) {
-        const float *St = isC ? p.Hst + slot_off(p, b, c, h) : p.Gst + slot_off(p, b, c + 1, h);
-        load_vec(h);
-        tile_load(ra, (isC ? dyb : xb) + (size_t)rt * 64 * HP + (size_t)h * 64, HP, true);
-        tile_load_ws(rb, St, NS, false);
-        tile_store(sm.a, ra, true);
-        float rho2[4] = {0.f, 0.f, 0.f, 0.f}, sc[4];
+        const size_t vo = vec_off(p, b, h, c);
+        const float cl = p.cs[vo + Q - 1];
+        float sc[2], rho2[2] = {0.f, 0.f};
+#pragma unroll
+        for (int half = 0; half < 2; ++half) {
+            const float v = p.cs[vo + rt * 64 + acc_row(half)];
+            sc[half] = isC ? expf(v) : p.dtT[vo + rt * 64 + acc_row(half)] * expf(fminf(cl - v, 0.f));
+        }
 #pragma unroll
         for (int m = 0; m < NS / 64; ++m) {
-            tile_store(sm.b, rb, false);
+            if (m == 0) tile_store(sm.t, ra);
+            tile_store(sm.t + PT, rf);
             __syncthreads();
-            if (m == 0) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = rt * 64 + ty * 4 + i;
-                    sc[i] = isC ? expf(css[r]) : dts[r] * expf(fminf(css[Q - 1] - css[r], 0.f));
-                }
+            if (m + 1 < NS / 64) {
+                tile_load<true>(rf, state(h) + 64 * (m + 1), NS);
+            } else if (h + 1 < h1) {
+                tile_load(ra, rows + (size_t)(h + 1) * 64, HP);
+                tile_load<true>(rf, state(h + 1), NS);
             }
-            if (m + 1 < NS / 64) tile_load_ws(rb, St + 64 * (m + 1), NS, false);
-            zero_acc(acc);
-            tile_mma(acc, sm.a, sm.b);
+            acc.zero();
+            tile_mma<PT, 3, false, true>(acc, sm.t, sm.t + PT);
 #pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 s2 = make_float2(sc[i], sc[i]);
-                const float2 a0 = __fmul2_rn(acc[i][0], s2), a1 = __fmul2_rn(acc[i][1], s2);
-                tot[m][i][0] = __fadd2_rn(tot[m][i][0], a0);
-                tot[m][i][1] = __fadd2_rn(tot[m][i][1], a1);
-                if (isC) {
-                    const float4 cv = ld4f(Cb + (size_t)(rt * 64 + ty * 4 + i) * GN + m * 64 + tx * 4);
-                    rho2[i] += cv.x * a0.x + cv.y * a0.y + cv.z * a1.x + cv.w * a1.y;
+            for (int half = 0; half < 2; ++half)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const float2 a = __fmul2_rn(make_float2(sc[half], sc[half]), acc.get(j, half));
+                    tot[m][half][j] = __fadd2_rn(tot[m][half][j], a);
+                    if (isC) {
+                        const float2 cv = ld2f(Cb + (size_t)(rt * 64 + acc_row(half)) * GN + m * 64 + acc_col(j));
+                        rho2[half] += cv.x * a.x + cv.y * a.y;
+                    }
+                }
+            if (isC && m + 1 == NS / 64) {
+#pragma unroll
+                for (int half = 0; half < 2; ++half) {
+                    const float v = sum_quad(rho2[half]);
+                    if ((lane & 3) == 0) sm.red[tid >> 7][acc_row(half)] = v;
                 }
             }
             __syncthreads();
         }
-        if (isC) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float v = sum_tx(rho2[i]);
-                if (tx == 0) p.rho2[vec_off(p, b, h, c) + rt * 64 + ty * 4 + i] = v;
-            }
-        }
+        if (isC && tid < 64) p.rho2[vo + rt * 64 + tid] = sm.red[0][tid] + sm.red[1][tid];
     }
 #pragma unroll
-    for (int m = 0; m < NS / 64; ++m) write_slice(tot[m], rt * 64, isC ? nrt + 1 : nrt + 2, m * 64);
+    for (int m = 0; m < NS / 64; ++m) {
+        float *out = slice(rt * 64, isC ? nrt + 1 : nrt + 2, m * 64);
+#pragma unroll
+        for (int half = 0; half < 2; ++half)
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+                *reinterpret_cast<float2 *>(out + (size_t)acc_row(half) * slice_stride + acc_col(j)) = tot[m][half][j];
+    }
 }
 
 // ------------------------------------------------------------------ da, ddt, dA partial
@@ -745,8 +769,6 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
 // One CTA per (chunk, eight consecutive heads), one warp per head.  ddt is [B, L, H]: a head's values of consecutive
 // steps lie H floats apart, so the eight heads' results go through a shared-memory tile and leave as rows of eight
 // consecutive floats (whole 32-byte sectors) instead of one 4-byte store per sector.
-constexpr int FIN_HB = 8;
-constexpr int FIN_TILE = 256 * (FIN_HB + 1);
 constexpr float kLeastStep = 1e-18f;      // far above the dt at which a product with it would lose bits
 template <bool TC> __device__ __forceinline__ void bwd_finish(const SegParams &p, float *tile, int id) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -849,7 +871,7 @@ __device__ __forceinline__ void reduce_dbdc(const SegParams &p, int id) {
     auto ld = [](const float *q) { return *reinterpret_cast<const float4 *>(q); };
     const size_t src = ((((size_t)b * segcap + tl) * p.G + g) * p.nsl) * p.N + n;
     if (!TC) {
-        // CUDA-core path: per head range, of a row of tile rt, dC slots 0 .. rt, dB slots rt + 1 .. tiles, then the inter-chunk terms
+        // split path: per head range, of a row of tile rt, dC slots 0 .. rt, dB slots rt + 1 .. tiles, then the inter-chunk terms
         const int rt = (int)(tl % (size_t)p.Q) >> 6;
         for (int s0 = 0; s0 < p.nsl; s0 += p.tiles + 3) {
             float4 v[5];                                // all of a range's loads in flight
@@ -885,18 +907,17 @@ __global__ void __launch_bounds__(256) k_bwd_tail(SegParams p, int nfin) {
     if ((int)blockIdx.x < nfin) bwd_finish<TC>(p, tile, blockIdx.x);
     else reduce_dbdc<T, TC>(p, blockIdx.x - nfin);
 }
-// CUDA-core path: the same with the sums of the next segment (to the left) in front, which share no scratch with it but the step
+// split path: the same with the sums of the next segment (to the left) in front, which share no scratch with it but the step
 // sizes, of which there are two copies.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256, 3) k_simt_tail(SegParams p, SegParams nx, int n_next, int nfin) {
+__global__ void __launch_bounds__(256, 2) k_simt_tail(SegParams p, SegParams nx, int n_next, int nfin) {
+    extern __shared__ __align__(16) unsigned char smem[];
+    SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();
     pdl_wait();
-    __shared__ SimtTiles sm;
-    __shared__ float wsm[256];
-    static_assert(sizeof(SimtTiles) >= FIN_TILE * sizeof(float), "the finishing step's tile");
     const int id = (int)blockIdx.x - n_next;
-    if (id < 0) simt_sums<T, NS>(nx, sm, wsm, blockIdx.x, true);
-    else if (id < nfin) bwd_finish<false>(p, &sm.a[0][0], id);
+    if (id < 0) simt_sums<T, NS>(nx, sm, blockIdx.x, true);
+    else if (id < nfin) bwd_finish<false>(p, reinterpret_cast<float *>(sm.t), id);
     else reduce_dbdc<T, false>(p, id - nfin);
 }
 
@@ -910,6 +931,11 @@ cudaError_t launch_bwd_tail(const SegParams &p, int dtype, cudaStream_t st) {
     return launch_pdl(k_bwd_tail<__nv_bfloat16, true>, grid, dim3(256), 0, st, p, nfin);
 }
 
+template <auto K, typename T, typename... Args> static cudaError_t simt_start(int ctas, cudaStream_t st, Args &&...args) {
+    const cudaError_t e = allow_smem<K>((int)sizeof(SimtSmem<T>));
+    if (e != cudaSuccess) return e;
+    return launch_pdl(K, dim3(ctas), dim3(256), sizeof(SimtSmem<T>), st, args...);
+}
 template <typename T, int NS>
 static cudaError_t simt_launch(const SegParams &p, const SegParams *next, int what, cudaStream_t st) {
     const int nrt = p.Q / 64, npair = nrt * (nrt + 1) / 2;
@@ -917,21 +943,20 @@ static cudaError_t simt_launch(const SegParams &p, const SegParams *next, int wh
         case SIMT_SUMS:
         case SIMT_SUMS_GRAD: {
             const bool grads = what == SIMT_SUMS_GRAD;
-            return launch_pdl(k_simt_sums<T, NS>, dim3(simt_n_sums<T, NS>(p, grads)), dim3(256), 0, st, p, grads);
+            return simt_start<k_simt_sums<T, NS>, T>(simt_n_sums<T, NS>(p, grads), st, p, grads);
         }
         case SIMT_Y: {
-            const int n_next = next ? simt_n_sums<T, NS>(*next, false) : 0;
-            const dim3 grid(p.nc * nrt * p.H * p.B + n_next);
-            if (!p.cbt) return launch_pdl(k_simt_y<T, NS, false>, grid, dim3(256), 0, st, p, p, 0);      // never with `next`
-            return launch_pdl(k_simt_y<T, NS, true>, grid, dim3(256), 0, st, p, next ? *next : p, n_next);
+            const int n_next = next ? simt_n_sums<T, NS>(*next, false) : 0, n = p.nc * nrt * p.H * p.B + n_next;
+            if (!p.cbt) return simt_start<k_simt_y<T, NS, false>, T>(n, st, p, p, 0);      // never with `next`
+            return simt_start<k_simt_y<T, NS, true>, T>(n, st, p, next ? *next : p, n_next);
         }
         case SIMT_TAIL: {
             const int nfin = tail_finish_ctas(p), n_next = simt_n_sums<T, NS>(*next, true);
-            return launch_pdl(k_simt_tail<T, NS>, dim3(n_next + nfin + tail_reduce_ctas(p)), dim3(256), 0, st, p, *next, n_next, nfin);
+            return simt_start<k_simt_tail<T, NS>, T>(n_next + nfin + tail_reduce_ctas(p), st, p, *next, n_next, nfin);
         }
         default: {
             const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 3)) * p.G * p.B;
-            return launch_pdl(k_simt_bwd<T, NS>, dim3(n_bc + n_dx), dim3(256), 0, st, p, n_dx);
+            return simt_start<k_simt_bwd<T, NS>, T>(n_bc + n_dx, st, p, n_dx);
         }
     }
 }
