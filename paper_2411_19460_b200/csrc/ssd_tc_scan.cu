@@ -18,12 +18,13 @@
 // equal, contiguous part of it, so that the scores are made again only where a part crosses into the next block or group and
 // every SM ends at the same time.  The heads are per-output, so the cut points change no bit.  Roles, meeting only through
 // mbarriers:
-//   warp 0 producer: ring of stages, one per head (value rows, chunk state, record of the mask's factors; SC_DX: x rows in
-//          a ring of their own); the columns operand of the scores takes a stage of the ring too
+//   warp 0 producer: a ring of value rows (and the record of the mask's factors) and one of states, a turn of each per head; the
+//          columns operand of the scores takes a turn too
+//   SC_DX: warp 7, without a sub-tile to mask, producer of the x rows, in a ring of their own
 //   warps 1, 2 MMA issuers, of alternate heads (one thread needs longer per head than the products take): acc2 = Rows State,
 //          acc1 = M V, one commit per head
 //   warp 3 output: one TMA store per head, then the stage is free
-//   warps 4..19 mask: two groups of seven take alternate heads and own one masked tile each
+//   warps 4..19 mask: two groups of seven (of eight, one has no sub-tile) take alternate heads and own one masked tile each
 //   warps 20..27 epilogue: two groups of four take alternate heads
 // The decay mask is factored per 32 x 32 sub-tile: strictly off-diagonal sub-tiles use
 //   e^{cs_t-cs_s} = e^{cs_t-cs_i0} * e^{cs_i0-cs_j1} * e^{cs_j1-cs_s}      (i0 = first row of the row sub-tile, j1 = last
@@ -31,10 +32,11 @@
 // product without the middle factor has one factor > 1; it is used where the decay inside the sub-tile is mild, and only stiff
 // heads are exponentiated element by element.
 //
-// Nothing is at a limit (y, dx: issue 45, 43 % of the slots and 47 % on the busiest scheduler, shared memory 39, 31 %, DRAM 39, 44 %,
-// tensor pipe 16, 12 %): a head's mask, products and output follow one another through barriers, and two heads in flight do not
-// cover it.  28 warps of 72 registers spill (76 bytes stored in y, 148 in dx).  4096 steps of
-// 80 heads, alone on the GPU: y 46 -> 32 us, dx 57 -> 44 us against one CTA per (256-step chunk, row half, head range).
+// Alone on the GPU y is bound by HBM (126 MB for 4096 steps of 80 heads in 20 us once its first tiles are there), dx by the latency of
+// a head's hand-overs (168 MB in 30 us; issue 43 % of the slots, shared memory 188 KB a head of 385 KB in that time).  28 warps of 72
+// registers spill (76 bytes stored in y, 152 in dx).  Beside the chain, dB/dC and the next segment, which hold the other SMs, what
+// counts is the time per head; split rings took the forward of 9472 x 3 steps of 64 heads from 279 to 273 us and 131072 steps of 80 heads,
+// forward and backward, from 6.15 to 6.05 ms.
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
 
@@ -51,14 +53,25 @@ __host__ __device__ constexpr int sc_rec_first(int mode) { return mode == SC_DX 
 constexpr uint32_t SC_REC_BYTES = (REC_OC - REC_BLK) * 4;
 static_assert(SC_REC_BYTES == (REC_CF - REC_CFX) * 4 && SC_REC_BYTES <= 2048, "both parts are of one size");
 
-// rows operand N/64 x 16 KB | stages: value rows 16 KB, state N rows of 128 B (the columns operand fits one), record 2 KB |
-// SC_DX: ring of x rows, 16 KB each, which only the epilogue reads
-constexpr uint32_t SC_STAGE = 16384 + (uint32_t)NS * 128 + 2048;
-__host__ __device__ constexpr int sc_stages(int mode) { return mode == SC_DX ? 4 : 5; }
+// rows operand N/64 x 16 KB | ring of value rows 16 KB (output when done) and record 2 KB | ring of states, N rows of 128 B |
+// SC_DX: ring of x rows, 16 KB each, which only the epilogue reads.  The columns operand of the scores takes a turn of the first
+// two rings, half in each.
+// A head's value rows are held from their load (3000 to 4500 cycles) until its output has been read, 9200 cycles (y), 10500 (dx); its
+// state only until its product with the rows, which waits for no mask.  In one ring of five (dx: four) stages of both, with the loads of x
+// in the same order, a head took 2350 (3000) cycles per SM, its slots' lifetime over their number.
+constexpr uint32_t SC_VAL = 16384 + 2048, SC_STB = (uint32_t)NS * 128;
+__host__ __device__ constexpr int sc_vals(int mode) { return mode == SC_DX ? 5 : 7; }
+__host__ __device__ constexpr int sc_states(int mode) { return mode == SC_DX ? 3 : 4; }
 constexpr int SC_XR = 3;
 __host__ __device__ constexpr uint32_t sc_smem(int mode) {
-    return (uint32_t)NS * 256 + sc_stages(mode) * SC_STAGE + (mode == SC_DX ? SC_XR * 16384 : 0) + 1024;
+    return (uint32_t)NS * 256 + sc_vals(mode) * SC_VAL + sc_states(mode) * SC_STB + (mode == SC_DX ? SC_XR * 16384 : 0) + 1024;
 }
+// a role's place in a ring: slot and completed passes over it
+template <int N> struct Turn {
+    int slot = 0;
+    uint32_t use = 0;
+    __device__ __forceinline__ void next() { if (++slot == N) { slot = 0; ++use; } }
+};
 
 __device__ __forceinline__ float ex2f(float x) {
     float y;
@@ -87,9 +100,9 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
           const __grid_constant__ CUtensorMap tmV, const __grid_constant__ CUtensorMap tmSt, const __grid_constant__ CUtensorMap tmOut,
           const __grid_constant__ CUtensorMap tmXr) {
     constexpr bool FWD = MODE == SC_FWD;
-    constexpr int NST = sc_stages(MODE);
-    constexpr uint32_t STAGE = SC_STAGE, OFF_ST = 16384, OFF_REC = OFF_ST + NS * 128;
-    constexpr uint32_t OFF_RING = NS * 256, OFF_XR = OFF_RING + NST * STAGE;
+    constexpr int NV = sc_vals(MODE), NST = sc_states(MODE);
+    // states first: tiles stay on 1 KB boundaries
+    constexpr uint32_t OFF_ST = NS * 256, OFF_VAL = OFF_ST + NST * SC_STB, OFF_XR = OFF_VAL + NV * 16384, OFF_REC = OFF_XR + (FWD ? 0 : SC_XR * 16384);
     constexpr int REC0 = sc_rec_first(MODE);
     // Of a mask group's eight warps (quarter q, column parity) the one whose two sub-tiles are zero idles
     constexpr int QALONE = FWD ? 0 : 3, SUBIDLE = FWD ? 1 : 0;
@@ -97,7 +110,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
     constexpr uint32_t TM_M = 128, TM_ACC = 256;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t full[NST], empty[NST], outfull[NST], xrfull[SC_XR], xrempty[SC_XR], sdone, sfree, rowsfree, mfull[2], accfull[2], accempty[2];
+    __shared__ uint64_t vfull[NV], vempty[NV], outfull[NV], stfull[NST], stempty[NST], xrfull[SC_XR], xrempty[SC_XR], sdone, sfree, rowsfree, mfull[2], accfull[2], accempty[2];
     __shared__ uint32_t tmem_base, abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -105,10 +118,14 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
     const int u_begin = (int)(units * blockIdx.x / gridDim.x), u_end = (int)(units * (blockIdx.x + 1) / gridDim.x);
 
     if (tid == 0) {
-        for (int i = 0; i < NST; ++i) {
-            mbar_init(&full[i], 1);
-            mbar_init(&empty[i], 1);
+        for (int i = 0; i < NV; ++i) {
+            mbar_init(&vfull[i], 1);
+            mbar_init(&vempty[i], 1);
             mbar_init(&outfull[i], 4);
+        }
+        for (int i = 0; i < NST; ++i) {
+            mbar_init(&stfull[i], 1);
+            mbar_init(&stempty[i], 1);
         }
         for (int i = 0; i < SC_XR; ++i) {
             mbar_init(&xrfull[i], 1);
@@ -150,36 +167,33 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (elect_one()) {
-            int slot = 0, nrun = 0;
-            uint32_t use = 0, hc = 0;        // completed passes over the ring, heads so far
-            auto next = [&]() { if (++slot == NST) { slot = 0; ++use; } };
+            Turn<NV> v;
+            Turn<NST> t;
+            int nrun = 0;
             for (int u = u_begin; u < u_end; ++nrun) {
                 const Run r = run_at(u);
                 const int tok = p.t0 + r.c * SC_T;
-                if (use) mbar_wait(&empty[slot], (use - 1) & 1, abortp, p.status);
+                if (t.use) mbar_wait(&stempty[t.slot], (t.use - 1) & 1, abortp, p.status);
+                if (v.use) mbar_wait(&vempty[v.slot], (v.use - 1) & 1, abortp, p.status);
                 if (nrun) mbar_wait(&rowsfree, (nrun - 1) & 1, abortp, p.status);
-                mbar_arrive_expect_tx(&full[slot], 2 * NS * 256);
-#pragma unroll
-                for (int nh = 0; nh < NS / 64; ++nh) {
-                    tma_load_3d(smem + nh * 16384, &tmRow, &full[slot], r.g * NS + nh * 64, tok, r.b);
-                    tma_load_3d(smem + OFF_RING + slot * STAGE + nh * 16384, &tmCol, &full[slot], r.g * NS + nh * 64, tok, r.b);
-                }
-                next();
+                mbar_arrive_expect_tx(&vfull[v.slot], NS * 256 + 16384);
+                mbar_arrive_expect_tx(&stfull[t.slot], 16384);
+                tma_load_3d(smem, &tmRow, &vfull[v.slot], r.g * NS, tok, r.b);
+                tma_load_3d(smem + 16384, &tmRow, &vfull[v.slot], r.g * NS + 64, tok, r.b);
+                tma_load_3d(smem + OFF_VAL + v.slot * 16384, &tmCol, &vfull[v.slot], r.g * NS, tok, r.b);
+                tma_load_3d(smem + OFF_ST + t.slot * SC_STB, &tmCol, &stfull[t.slot], r.g * NS + 64, tok, r.b);
+                v.next();
+                t.next();
                 const int strow = (r.b * p.ncs + r.c) * p.H;
-                for (int k = 0; k < r.n; ++k, ++hc, next()) {
+                for (int k = 0; k < r.n; ++k, v.next(), t.next()) {
                     const int h = r.h0 + k;
-                    unsigned char *sb = smem + OFF_RING + slot * STAGE;
-                    if (use) mbar_wait(&empty[slot], (use - 1) & 1, abortp, p.status);
-                    mbar_arrive_expect_tx(&full[slot], OFF_REC + SC_REC_BYTES);
-                    tma_load_3d(sb + OFF_ST, &tmSt, &full[slot], 0, (strow + h) * NS, 0);
-                    tma_load_3d(sb, &tmV, &full[slot], h * 64, tok, r.b);
-                    bulk_load(sb + OFF_REC, p.rec + (((size_t)r.b * p.H + h) * p.ncs + r.c) * REC_FLOATS + REC0, SC_REC_BYTES, &full[slot]);
-                    if (!FWD) {
-                        const uint32_t xs = hc % SC_XR, xuse = hc / SC_XR;
-                        if (xuse) mbar_wait(&xrempty[xs], (xuse - 1) & 1, abortp, p.status);
-                        mbar_arrive_expect_tx(&xrfull[xs], 16384);
-                        tma_load_3d(smem + OFF_XR + xs * 16384, &tmXr, &xrfull[xs], h * 64, tok, r.b);
-                    }
+                    if (t.use) mbar_wait(&stempty[t.slot], (t.use - 1) & 1, abortp, p.status);
+                    mbar_arrive_expect_tx(&stfull[t.slot], SC_STB);
+                    tma_load_3d(smem + OFF_ST + t.slot * SC_STB, &tmSt, &stfull[t.slot], 0, (strow + h) * NS, 0);
+                    if (v.use) mbar_wait(&vempty[v.slot], (v.use - 1) & 1, abortp, p.status);
+                    mbar_arrive_expect_tx(&vfull[v.slot], 16384 + SC_REC_BYTES);
+                    tma_load_3d(smem + OFF_VAL + v.slot * 16384, &tmV, &vfull[v.slot], h * 64, tok, r.b);
+                    bulk_load(smem + OFF_REC + v.slot * 2048, p.rec + (((size_t)r.b * p.H + h) * p.ncs + r.c) * REC_FLOATS + REC0, SC_REC_BYTES, &vfull[v.slot]);
                 }
                 u += r.n;
             }
@@ -191,40 +205,45 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
         if (elect_one()) {
             constexpr uint32_t KB = NS / 16;
             const uint32_t idS = umma_idesc_bf16(128, 128, false, false), id64 = umma_idesc_bf16(128, 64, false, true);
-            const uint64_t dR = umma_desc_sw128(smem_u32(smem), 16, 1024), dV0 = umma_desc_sw128(smem_u32(smem + OFF_RING), 8192, 1024);
+            const uint64_t dR = umma_desc_sw128(smem_u32(smem), 16, 1024), dV0 = umma_desc_sw128(smem_u32(smem + OFF_VAL), 8192, 1024);
             const uint32_t loR = (uint32_t)dR, hiR = (uint32_t)(dR >> 32), loV0 = (uint32_t)dV0, hiV = (uint32_t)(dV0 >> 32);
-            int slot = 0, nrun = 0;
-            uint32_t use = 0, hc = 0;
-            auto next = [&]() { if (++slot == NST) { slot = 0; ++use; } };
+            const uint32_t loC0 = loR + OFF_VAL / 16, loC1 = loR + OFF_ST / 16, loS0 = loV0 - OFF_VAL / 16 + OFF_ST / 16;
+            Turn<NV> v;
+            Turn<NST> t;
+            int nrun = 0;
+            uint32_t hc = 0;
             for (int u = u_begin; u < u_end; ++nrun) {
                 const Run r = run_at(u);
                 if (mine == 0) {
-                    mbar_wait(&full[slot], use & 1, abortp, p.status);
+                    mbar_wait(&vfull[v.slot], v.use & 1, abortp, p.status);
+                    mbar_wait(&stfull[t.slot], t.use & 1, abortp, p.status);
                     if (nrun) mbar_wait(&sfree, (nrun - 1) & 1, abortp, p.status);
                     tc_fence_after_sync();
-                    const uint32_t loC = (uint32_t)umma_desc_sw128(smem_u32(smem + OFF_RING) + slot * STAGE, 16, 1024);
+                    const uint32_t lo0 = loC0 + v.slot * 1024, lo1 = loC1 + t.slot * (SC_STB / 16);
 #pragma unroll
                     for (int k = 0; k < KB; ++k) {
-                        const uint32_t o = (k >> 2) * 1024 + (k & 3) * 2;
-                        if (k == 0) umma_bf16_fixed<false>(tm, umma_desc_words(loR + o, hiR), umma_desc_words(loC + o, hiR), idS);
-                        else umma_bf16_fixed<true>(tm, umma_desc_words(loR + o, hiR), umma_desc_words(loC + o, hiR), idS);
+                        const uint32_t o = (k >> 2) * 1024 + (k & 3) * 2, c = (k < 4 ? lo0 : lo1) + (k & 3) * 2;
+                        if (k == 0) umma_bf16_fixed<false>(tm, umma_desc_words(loR + o, hiR), umma_desc_words(c, hiR), idS);
+                        else umma_bf16_fixed<true>(tm, umma_desc_words(loR + o, hiR), umma_desc_words(c, hiR), idS);
                     }
                     umma_commit(&sdone);
-                    umma_commit(&empty[slot]);     // the scores are made: their columns operand is dead
+                    umma_commit(&vempty[v.slot]);     // the scores are made: their columns operand is dead
+                    umma_commit(&stempty[t.slot]);
                 } else {
-                    // The run's rows are in place once its scores are made.  (Not `full`: that slot is refilled as soon as the
+                    // The run's rows are in place once its scores are made.  (Not `vfull`: that slot is refilled as soon as the
                     // scores are made, possibly before this thread gets here.  The scores of the next run cannot be made before
                     // this thread has released the rows of this one.)
                     mbar_wait(&sdone, nrun & 1, abortp, p.status);
                 }
-                next();
-                for (int k = 0; k < r.n; ++k, ++hc, next()) {
+                v.next();
+                t.next();
+                for (int k = 0; k < r.n; ++k, ++hc, v.next(), t.next()) {
                     if ((hc & 1) != mine) continue;
                     const uint32_t bf = hc & 1, par = (hc >> 1) & 1;
                     const uint32_t acc1 = tm + TM_ACC + bf * 128, acc2 = acc1 + 64, mA = tm + TM_M + bf * 64;
-                    const uint32_t loV = loV0 + slot * (STAGE / 16), loS = loV + OFF_ST / 16;
+                    const uint32_t loV = loV0 + v.slot * 1024, loS = loS0 + t.slot * (SC_STB / 16);
                     if (hc >= 2) mbar_wait(&accempty[bf], par ^ 1u, abortp, p.status);
-                    mbar_wait(&full[slot], use & 1, abortp, p.status);
+                    mbar_wait(&stfull[t.slot], t.use & 1, abortp, p.status);
                     tc_fence_after_sync();
 #pragma unroll
                     for (int kk = 0; kk < KB; ++kk) {      // Rows (K = n) x state^T rows n (MN-major over p)
@@ -232,6 +251,8 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                         if (kk == 0) umma_bf16_fixed<false>(acc2, ad, bd, id64);
                         else umma_bf16_fixed<true>(acc2, ad, bd, id64);
                     }
+                    umma_commit(&stempty[t.slot]);
+                    mbar_wait(&vfull[v.slot], v.use & 1, abortp, p.status);
                     mbar_wait(&mfull[bf], par, abortp, p.status);
                     tc_fence_after_sync();
 #pragma unroll
@@ -249,22 +270,19 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
     } else if (warp == 3) {
         // ------------------------------------------------------------ output warp
         if (elect_one()) {
-            int slot = 0;
-            uint32_t outs[NST];      // completed outputs per slot (the columns operand's turn has none)
-#pragma unroll
-            for (int i = 0; i < NST; ++i) outs[i] = 0;
-            auto next = [&]() { if (++slot == NST) slot = 0; };
+            Turn<NV> v;
+            uint32_t outs = 0;       // parity of the completed outputs per slot (the columns operand's turn has none)
             for (int u = u_begin; u < u_end;) {
                 const Run r = run_at(u);
                 const int tok = p.t0 + r.c * SC_T;
-                next();
-                for (int k = 0; k < r.n; ++k, next()) {
-                    mbar_wait(&outfull[slot], outs[slot] & 1, abortp, p.status);
-                    ++outs[slot];
-                    tma_store_3d(&tmOut, smem + OFF_RING + slot * STAGE, (r.h0 + k) * 64, tok, r.b);
+                v.next();
+                for (int k = 0; k < r.n; ++k, v.next()) {
+                    mbar_wait(&outfull[v.slot], (outs >> v.slot) & 1, abortp, p.status);
+                    outs ^= 1u << v.slot;
+                    tma_store_3d(&tmOut, smem + OFF_VAL + v.slot * 16384, (r.h0 + k) * 64, tok, r.b);
                     tma_store_commit();
                     tma_store_wait_read();
-                    mbar_arrive(&empty[slot]);
+                    mbar_arrive(&vempty[v.slot]);
                 }
                 u += r.n;
             }
@@ -287,20 +305,20 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                     if (is_zero(j) && ((j & 1) == sub || q == QALONE)) tmem_st16(tM + j * 16, z);
                 tmem_st_wait();
             }
-            int slot = 0, nrun = 0;
-            uint32_t use = 0, hc = 0;
-            auto next = [&]() { if (++slot == NST) { slot = 0; ++use; } };
+            Turn<NV> vt;
+            int nrun = 0;
+            uint32_t hc = 0;
             for (int u = u_begin; u < u_end; ++nrun) {
                 const Run rn = run_at(u);
-                next();
+                vt.next();
                 mbar_wait(&sdone, nrun & 1, abortp, p.status);
                 tc_fence_after_sync();
-                for (int k = 0; k < rn.n; ++k, ++hc, next()) {
+                for (int k = 0; k < rn.n; ++k, ++hc, vt.next()) {
                     if ((int)(hc & 1) != gp) continue;
                     const uint32_t turn = hc >> 1;
-                    const float *rec = reinterpret_cast<const float *>(smem + OFF_RING + slot * STAGE + OFF_REC) - REC0;
+                    const float *rec = reinterpret_cast<const float *>(smem + OFF_REC + vt.slot * 2048) - REC0;
                     const float *cs2 = rec + REC_CS;
-                    mbar_wait(&full[slot], use & 1, abortp, p.status);
+                    mbar_wait(&vfull[vt.slot], vt.use & 1, abortp, p.status);
                     const float csr = cs2[r], cs_lo = cs2[q * 32], cs_hi = cs2[q * 32 + 31];
                     const float rowf = FWD ? ex2f(csr - cs_lo) : ex2f(cs_hi - csr);      // off the diagonal, <= 1
                     bool waited = turn == 0;
@@ -357,7 +375,21 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                 if (lane == 0) mbar_arrive(&sfree);
                 u += rn.n;
             }
+        } else if (!FWD && gp == 0 && elect_one()) {
+            // an idle warp: producer of the x rows, which may run ahead of the stages or behind them
+            uint32_t hc = 0;
+            for (int u = u_begin; u < u_end;) {
+                const Run rn = run_at(u);
+                for (int k = 0; k < rn.n; ++k, ++hc) {
+                    const uint32_t xs = hc % SC_XR, xuse = hc / SC_XR;
+                    if (xuse) mbar_wait(&xrempty[xs], (xuse - 1) & 1, abortp, p.status);
+                    mbar_arrive_expect_tx(&xrfull[xs], 16384);
+                    tma_load_3d(smem + OFF_XR + xs * 16384, &tmXr, &xrfull[xs], (rn.h0 + k) * 64, p.t0 + rn.c * SC_T, rn.b);
+                }
+                u += rn.n;
+            }
         }
+        __syncwarp();
     } else if (warp >= 20) {
         // ------------------------------------------------------------ epilogue warps
         // Group eg takes alternate heads, warp q of a group the rows 32 q .. of the block.  x (and dy) come from the tiles
@@ -365,23 +397,22 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
         const int q = warp & 3, eg = (warp - 20) >> 2;
         const int r = q * 32 + lane;
         const uint32_t tl = tm + ((uint32_t)(q * 32) << 16) + TM_ACC + eg * 128;
-        int slot = 0;
-        uint32_t use = 0, hc = 0;
-        auto next = [&]() { if (++slot == NST) { slot = 0; ++use; } };
+        Turn<NV> vt;
+        uint32_t hc = 0;
         for (int u = u_begin; u < u_end;) {
             const Run rn = run_at(u);
-            next();
-            for (int k = 0; k < rn.n; ++k, ++hc, next()) {
+            vt.next();
+            for (int k = 0; k < rn.n; ++k, ++hc, vt.next()) {
                 if ((int)(hc & 1) != eg) continue;
                 const int h = rn.h0 + k;
-                const float *rec = reinterpret_cast<const float *>(smem + OFF_RING + slot * STAGE + OFF_REC) - REC0;
-                mbar_wait(&full[slot], use & 1, abortp, p.status);
+                const float *rec = reinterpret_cast<const float *>(smem + OFF_REC + vt.slot * 2048) - REC0;
+                mbar_wait(&vfull[vt.slot], vt.use & 1, abortp, p.status);
                 const float csr = rec[REC_CS + r];
                 const float offs = FWD ? ex2f(csr) : ex2f(rec[REC_CS + 127] - csr);
                 const float dtr = rec[REC_DT + r];
                 const float Dh = __ldg(p.D + h);
                 const float Dx = Dh + (FWD ? 0.f : p.dx_skip);       // dx: D dy, plus dy itself under a skip connection
-                unsigned char *vrow = smem + OFF_RING + slot * STAGE + r * 128;       // x row (SC_FWD) / dy row (SC_DX), then output
+                unsigned char *vrow = smem + OFF_VAL + vt.slot * 16384 + r * 128;       // x row (SC_FWD) / dy row (SC_DX), then output
                 const uint32_t xs = hc % SC_XR;
                 const unsigned char *xrow = smem + OFF_XR + xs * 16384 + r * 128;      // SC_DX: x row
                 if (!FWD) mbar_wait(&xrfull[xs], (hc / SC_XR) & 1, abortp, p.status);
@@ -430,7 +461,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                 __syncwarp();
                 if (lane == 0) {
                     mbar_arrive(&accempty[eg]);
-                    mbar_arrive(&outfull[slot]);
+                    mbar_arrive(&outfull[vt.slot]);
                     if (!FWD) mbar_arrive(&xrempty[xs]);
                 }
                 if (!FWD) {
