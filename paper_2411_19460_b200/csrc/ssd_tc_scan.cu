@@ -110,7 +110,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
     constexpr uint32_t TM_M = 128, TM_ACC = 256;
     extern __shared__ unsigned char smem_raw[];
     unsigned char *smem = (unsigned char *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    __shared__ uint64_t vfull[NV], vempty[NV], outfull[NV], stfull[NST], stempty[NST], xrfull[SC_XR], xrempty[SC_XR], sdone, sfree, rowsfree, mfull[2], accfull[2], accempty[2];
+    __shared__ uint64_t full[NV + NST], empty[NV + NST], outfull[NV], xrfull[SC_XR], xrempty[SC_XR], sdone, sfree, rowsfree, mfull[2], accfull[2], accempty[2];
     __shared__ uint32_t tmem_base, abort_flag;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -118,15 +118,11 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
     const int u_begin = (int)(units * blockIdx.x / gridDim.x), u_end = (int)(units * (blockIdx.x + 1) / gridDim.x);
 
     if (tid == 0) {
-        for (int i = 0; i < NV; ++i) {
-            mbar_init(&vfull[i], 1);
-            mbar_init(&vempty[i], 1);
-            mbar_init(&outfull[i], 4);
+        for (int i = 0; i < NV + NST; ++i) {       // value rows, states
+            mbar_init(&full[i], 1);
+            mbar_init(&empty[i], 1);
         }
-        for (int i = 0; i < NST; ++i) {
-            mbar_init(&stfull[i], 1);
-            mbar_init(&stempty[i], 1);
-        }
+        for (int i = 0; i < NV; ++i) mbar_init(&outfull[i], 4);
         for (int i = 0; i < SC_XR; ++i) {
             mbar_init(&xrfull[i], 1);
             mbar_init(&xrempty[i], 4);
@@ -173,27 +169,27 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
             for (int u = u_begin; u < u_end; ++nrun) {
                 const Run r = run_at(u);
                 const int tok = p.t0 + r.c * SC_T;
-                if (t.use) mbar_wait(&stempty[t.slot], (t.use - 1) & 1, abortp, p.status);
-                if (v.use) mbar_wait(&vempty[v.slot], (v.use - 1) & 1, abortp, p.status);
+                if (t.use) mbar_wait(&empty[NV + t.slot], (t.use - 1) & 1, abortp, p.status);
+                if (v.use) mbar_wait(&empty[v.slot], (v.use - 1) & 1, abortp, p.status);
                 if (nrun) mbar_wait(&rowsfree, (nrun - 1) & 1, abortp, p.status);
-                mbar_arrive_expect_tx(&vfull[v.slot], NS * 256 + 16384);
-                mbar_arrive_expect_tx(&stfull[t.slot], 16384);
-                tma_load_3d(smem, &tmRow, &vfull[v.slot], r.g * NS, tok, r.b);
-                tma_load_3d(smem + 16384, &tmRow, &vfull[v.slot], r.g * NS + 64, tok, r.b);
-                tma_load_3d(smem + OFF_VAL + v.slot * 16384, &tmCol, &vfull[v.slot], r.g * NS, tok, r.b);
-                tma_load_3d(smem + OFF_ST + t.slot * SC_STB, &tmCol, &stfull[t.slot], r.g * NS + 64, tok, r.b);
+                mbar_arrive_expect_tx(&full[v.slot], NS * 256 + 16384);
+                mbar_arrive_expect_tx(&full[NV + t.slot], 16384);
+                tma_load_3d(smem, &tmRow, &full[v.slot], r.g * NS, tok, r.b);
+                tma_load_3d(smem + 16384, &tmRow, &full[v.slot], r.g * NS + 64, tok, r.b);
+                tma_load_3d(smem + OFF_VAL + v.slot * 16384, &tmCol, &full[v.slot], r.g * NS, tok, r.b);
+                tma_load_3d(smem + OFF_ST + t.slot * SC_STB, &tmCol, &full[NV + t.slot], r.g * NS + 64, tok, r.b);
                 v.next();
                 t.next();
                 const int strow = (r.b * p.ncs + r.c) * p.H;
                 for (int k = 0; k < r.n; ++k, v.next(), t.next()) {
                     const int h = r.h0 + k;
-                    if (t.use) mbar_wait(&stempty[t.slot], (t.use - 1) & 1, abortp, p.status);
-                    mbar_arrive_expect_tx(&stfull[t.slot], SC_STB);
-                    tma_load_3d(smem + OFF_ST + t.slot * SC_STB, &tmSt, &stfull[t.slot], 0, (strow + h) * NS, 0);
-                    if (v.use) mbar_wait(&vempty[v.slot], (v.use - 1) & 1, abortp, p.status);
-                    mbar_arrive_expect_tx(&vfull[v.slot], 16384 + SC_REC_BYTES);
-                    tma_load_3d(smem + OFF_VAL + v.slot * 16384, &tmV, &vfull[v.slot], h * 64, tok, r.b);
-                    bulk_load(smem + OFF_REC + v.slot * 2048, p.rec + (((size_t)r.b * p.H + h) * p.ncs + r.c) * REC_FLOATS + REC0, SC_REC_BYTES, &vfull[v.slot]);
+                    if (t.use) mbar_wait(&empty[NV + t.slot], (t.use - 1) & 1, abortp, p.status);
+                    mbar_arrive_expect_tx(&full[NV + t.slot], SC_STB);
+                    tma_load_3d(smem + OFF_ST + t.slot * SC_STB, &tmSt, &full[NV + t.slot], 0, (strow + h) * NS, 0);
+                    if (v.use) mbar_wait(&empty[v.slot], (v.use - 1) & 1, abortp, p.status);
+                    mbar_arrive_expect_tx(&full[v.slot], 16384 + SC_REC_BYTES);
+                    tma_load_3d(smem + OFF_VAL + v.slot * 16384, &tmV, &full[v.slot], h * 64, tok, r.b);
+                    bulk_load(smem + OFF_REC + v.slot * 2048, p.rec + (((size_t)r.b * p.H + h) * p.ncs + r.c) * REC_FLOATS + REC0, SC_REC_BYTES, &full[v.slot]);
                 }
                 u += r.n;
             }
@@ -215,8 +211,8 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
             for (int u = u_begin; u < u_end; ++nrun) {
                 const Run r = run_at(u);
                 if (mine == 0) {
-                    mbar_wait(&vfull[v.slot], v.use & 1, abortp, p.status);
-                    mbar_wait(&stfull[t.slot], t.use & 1, abortp, p.status);
+                    mbar_wait(&full[v.slot], v.use & 1, abortp, p.status);
+                    mbar_wait(&full[NV + t.slot], t.use & 1, abortp, p.status);
                     if (nrun) mbar_wait(&sfree, (nrun - 1) & 1, abortp, p.status);
                     tc_fence_after_sync();
                     const uint32_t lo0 = loC0 + v.slot * 1024, lo1 = loC1 + t.slot * (SC_STB / 16);
@@ -227,10 +223,10 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                         else umma_bf16_fixed<true>(tm, umma_desc_words(loR + o, hiR), umma_desc_words(c, hiR), idS);
                     }
                     umma_commit(&sdone);
-                    umma_commit(&vempty[v.slot]);     // the scores are made: their columns operand is dead
-                    umma_commit(&stempty[t.slot]);
+                    umma_commit(&empty[v.slot]);     // the scores are made: their columns operand is dead
+                    umma_commit(&empty[NV + t.slot]);
                 } else {
-                    // The run's rows are in place once its scores are made.  (Not `vfull`: that slot is refilled as soon as the
+                    // The run's rows are in place once its scores are made.  (Not `full`: that slot is refilled as soon as the
                     // scores are made, possibly before this thread gets here.  The scores of the next run cannot be made before
                     // this thread has released the rows of this one.)
                     mbar_wait(&sdone, nrun & 1, abortp, p.status);
@@ -243,7 +239,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                     const uint32_t acc1 = tm + TM_ACC + bf * 128, acc2 = acc1 + 64, mA = tm + TM_M + bf * 64;
                     const uint32_t loV = loV0 + v.slot * 1024, loS = loS0 + t.slot * (SC_STB / 16);
                     if (hc >= 2) mbar_wait(&accempty[bf], par ^ 1u, abortp, p.status);
-                    mbar_wait(&stfull[t.slot], t.use & 1, abortp, p.status);
+                    mbar_wait(&full[NV + t.slot], t.use & 1, abortp, p.status);
                     tc_fence_after_sync();
 #pragma unroll
                     for (int kk = 0; kk < KB; ++kk) {      // Rows (K = n) x state^T rows n (MN-major over p)
@@ -251,8 +247,8 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                         if (kk == 0) umma_bf16_fixed<false>(acc2, ad, bd, id64);
                         else umma_bf16_fixed<true>(acc2, ad, bd, id64);
                     }
-                    umma_commit(&stempty[t.slot]);
-                    mbar_wait(&vfull[v.slot], v.use & 1, abortp, p.status);
+                    umma_commit(&empty[NV + t.slot]);
+                    mbar_wait(&full[v.slot], v.use & 1, abortp, p.status);
                     mbar_wait(&mfull[bf], par, abortp, p.status);
                     tc_fence_after_sync();
 #pragma unroll
@@ -282,7 +278,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                     tma_store_3d(&tmOut, smem + OFF_VAL + v.slot * 16384, (r.h0 + k) * 64, tok, r.b);
                     tma_store_commit();
                     tma_store_wait_read();
-                    mbar_arrive(&vempty[v.slot]);
+                    mbar_arrive(&empty[v.slot]);
                 }
                 u += r.n;
             }
@@ -318,7 +314,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                     const uint32_t turn = hc >> 1;
                     const float *rec = reinterpret_cast<const float *>(smem + OFF_REC + vt.slot * 2048) - REC0;
                     const float *cs2 = rec + REC_CS;
-                    mbar_wait(&vfull[vt.slot], vt.use & 1, abortp, p.status);
+                    mbar_wait(&full[vt.slot], vt.use & 1, abortp, p.status);
                     const float csr = cs2[r], cs_lo = cs2[q * 32], cs_hi = cs2[q * 32 + 31];
                     const float rowf = FWD ? ex2f(csr - cs_lo) : ex2f(cs_hi - csr);      // off the diagonal, <= 1
                     bool waited = turn == 0;
@@ -375,18 +371,20 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                 if (lane == 0) mbar_arrive(&sfree);
                 u += rn.n;
             }
-        } else if (!FWD && gp == 0 && elect_one()) {
-            // an idle warp: producer of the x rows, which may run ahead of the stages or behind them
-            uint32_t hc = 0;
-            for (int u = u_begin; u < u_end;) {
-                const Run rn = run_at(u);
-                for (int k = 0; k < rn.n; ++k, ++hc) {
-                    const uint32_t xs = hc % SC_XR, xuse = hc / SC_XR;
-                    if (xuse) mbar_wait(&xrempty[xs], (xuse - 1) & 1, abortp, p.status);
-                    mbar_arrive_expect_tx(&xrfull[xs], 16384);
-                    tma_load_3d(smem + OFF_XR + xs * 16384, &tmXr, &xrfull[xs], (rn.h0 + k) * 64, p.t0 + rn.c * SC_T, rn.b);
+        } else if (!FWD && gp == 0) {
+            // an idle warp: producer of the x rows, which may run ahead of the value rows or behind them
+            if (elect_one()) {
+                uint32_t hc = 0;
+                for (int u = u_begin; u < u_end;) {
+                    const Run rn = run_at(u);
+                    for (int k = 0; k < rn.n; ++k, ++hc) {
+                        const uint32_t xs = hc % SC_XR, xuse = hc / SC_XR;
+                        if (xuse) mbar_wait(&xrempty[xs], (xuse - 1) & 1, abortp, p.status);
+                        mbar_arrive_expect_tx(&xrfull[xs], 16384);
+                        tma_load_3d(smem + OFF_XR + xs * 16384, &tmXr, &xrfull[xs], (rn.h0 + k) * 64, p.t0 + rn.c * SC_T, rn.b);
+                    }
+                    u += rn.n;
                 }
-                u += rn.n;
             }
         }
         __syncwarp();
@@ -406,7 +404,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                 if ((int)(hc & 1) != eg) continue;
                 const int h = rn.h0 + k;
                 const float *rec = reinterpret_cast<const float *>(smem + OFF_REC + vt.slot * 2048) - REC0;
-                mbar_wait(&vfull[vt.slot], vt.use & 1, abortp, p.status);
+                mbar_wait(&full[vt.slot], vt.use & 1, abortp, p.status);
                 const float csr = rec[REC_CS + r];
                 const float offs = FWD ? ex2f(csr) : ex2f(rec[REC_CS + 127] - csr);
                 const float dtr = rec[REC_DT + r];
