@@ -105,7 +105,8 @@ typedef struct ssd_shape {
  * seg/chunk (the per-segment chunk states: the "grid cell" term of Eq. 4), not with L, apart from
  * 20 bytes per (batch, head, chunk) of dA/dD partial sums in the backward.  With two segments or more
  * there are second and third copies of what neighbouring segments' kernels touch at the same time (tensor-core
- * path: 3 times the forward's and 2.5 times the backward's scratch; split path: up to 64 MiB more in
+ * path: 3 times the forward's and 2.5 times the backward's scratch, 3.5 times where a segment's bf16 states take
+ * 16 MiB or less; split path: up to 64 MiB more in
  * the forward), unless shape->flags has SSD_FLAG_SERIAL: size the buffer with the flags the call will use.
  * The split path also keeps the products C B^T of a segment, 4 B G chunk seg bytes (not in ssd_fwd_static_ws
  * where they do not fit).

@@ -46,13 +46,15 @@ static void prof_end(ProfEvent *ev, cudaStream_t st) {
 }
 
 // Scratch regions of one call.  What the kernels of neighbouring segments touch at the same time exists more than once on the
-// tensor-core path: the records and states that the forward chain leaves three times, so that it runs two segments ahead (the
-// backward's critical path is then the gradient chain alone; with two copies it waited for the large kernels two segments
-// back: 24 heads, 2048-token segments, 52 us a segment instead of 36), the rest twice.
+// tensor-core path: the records and states that the forward chain leaves three times, so that it runs two segments ahead (with
+// two copies it waited for the large kernels two segments back: 24 heads, 2048-token segments, 52 us a segment instead of 36),
+// the rest twice; where they are small, once more each (chain_copies).
+static const int kChainCopies = 4, kGradCopies = 3;      // at most
 struct Layout {
     size_t status, hcarry, Gst, gcarry, dAp, dDp;
-    size_t rec[3], Hbf[3], cs[2], dtT[2], Hst[2], cbt[2];
-    size_t Gbf[2], ghdot[2], ddt_dir[2], rho[2], rho2[2], psi[2], psi2[2], pB[2], pC[2];
+    size_t rec[kChainCopies], Hbf[kChainCopies], cs[2], dtT[2], Hst[2], cbt[2];
+    size_t Gbf[kGradCopies], ghdot[kGradCopies], ddt_dir[kGradCopies], rho[kGradCopies], rho2[kGradCopies], psi[kGradCopies], psi2[kGradCopies],
+        pB[kGradCopies], pC[kGradCopies];
     size_t total;
 };
 
@@ -154,7 +156,17 @@ static bool simt_overlap(const Plan &pl, bool bwd) {
     return pl.nseg > 1 && (bwd || copy <= (size_t)64 << 20);
 }
 
-static int chain_copies(int nseg) { return nseg >= kMinSegmentsForTwins ? 3 : nseg > 1 ? 2 : 1; }
+// Copies of what the forward chain leaves, and of what the gradient chain and the large kernels leave (tensor-core path).  A copy comes
+// back when its segment's tail is done: chain, dB/dC beside dx, tail and the hand-overs take 77 us of 24 heads and 2048 steps, so with
+// two copies a segment can start every 38 us, while the gradient chain alone takes 28; the recompute likewise with three.  Where
+// the copies are small that latency is the bound, and there is one more of each: backward of 8 segments of that size 352 -> 316 us,
+// 16 of 1024 steps 513 -> 437 us (64 heads: 915 -> 716, 80: 1055 -> 820); 64 heads, 8 of 2048 (16 MiB) 602 -> 527 us; with 80 heads and 4096 steps, where SM time is the bound, 8 segments take the same with and without.
+static const size_t kSmallStates = (size_t)16 << 20;
+static bool small_states(const Plan &pl) { return (size_t)pl.B * pl.H * pl.ncs * pl.P * pl.N * 2 <= kSmallStates; }
+static int chain_copies(const Plan &pl, bool bwd) {
+    return pl.nseg >= kMinSegmentsForTwins ? (bwd && small_states(pl) ? 4 : 3) : pl.nseg > 1 ? 2 : 1;
+}
+static int grad_copies(const Plan &pl) { return pl.nseg >= kMinSegmentsForTwins ? (small_states(pl) ? 3 : 2) : 1; }
 
 // `twins`: whether the second and third copies may exist at all (not for callers that keep every kernel in order on one
 // stream: SSD_FLAG_SERIAL and the built-in scratch of ssd_fwd_static_ws).
@@ -163,24 +175,24 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
     const size_t vec = BH * pl.ncs * pl.Q * sizeof(float);
     const size_t st = BH * (pl.ncs + 1) * PN * sizeof(float), stb = BH * pl.ncs * PN * 2;
     const bool bwd = (op == SSD_OP_BWD_SEG);
-    const bool twin = twins && pl.use_tc && pl.nseg >= kMinSegmentsForTwins;
+    const int ncp = twins ? chain_copies(pl, bwd) : 1, ngc = twins && pl.use_tc ? grad_copies(pl) : 1;
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes, 256); return r; };
     auto take2 = [&](size_t (&r)[2], size_t bytes, bool two) {
         r[0] = take(bytes);
         r[1] = two ? take(bytes) : r[0];
     };
-    auto take3 = [&](size_t (&r)[3], size_t bytes, int copies) {
-        for (int i = 0; i < 3; ++i) r[i] = i < copies ? take(bytes) : r[i - copies];
+    auto take_n = [&](auto &r, size_t bytes, int copies) {
+        for (int i = 0; i < (int)(sizeof(r) / sizeof(r[0])); ++i) r[i] = i < copies ? take(bytes) : r[i % copies];
     };
     memset(&lo, 0, sizeof(lo));
     lo.status = take(256);
+    const int vcopies = bwd && small_states(pl) ? 3 : 2;      // of the vectors; of the records one more
     if (!bwd) lo.hcarry = take(BH * PN * sizeof(float));      // the backward starts every segment from `boundary`
-    // the vectors and records (a fraction of the states) exist as often for any number of segments, so that the scratch is a
-    // function of the segment length that only rises
+    // the vectors and records (a fraction of the states) exist as often for any number of segments
     if (pl.use_tc) {
-        take3(lo.rec, BH * pl.ncs * REC_FLOATS * sizeof(float), twins ? 3 : 1);
-        take3(lo.Hbf, stb, twins ? chain_copies(pl.nseg) : 1);
+        take_n(lo.rec, BH * pl.ncs * REC_FLOATS * sizeof(float), twins ? vcopies + 1 : 1);
+        take_n(lo.Hbf, stb, ncp);
     } else {
         // two copies where a launch works on two neighbouring segments: y beside the next segment's sums, and in the backward,
         // where only the step sizes meet, the finishing steps beside them
@@ -192,19 +204,19 @@ static void make_layout(const Plan &pl, int op, Layout &lo, bool twins) {
     }
     if (bwd) {
         lo.gcarry = take(BH * PN * sizeof(float));
-        if (pl.use_tc) take2(lo.Gbf, stb, twin);
+        if (pl.use_tc) take_n(lo.Gbf, stb, ngc);
         else lo.Gst = take(st);
-        take2(lo.ghdot, BH * pl.ncs * 16 * sizeof(float), twin);
-        const bool vtwin = twins && pl.use_tc;
-        take2(lo.ddt_dir, vec, vtwin);
+        take_n(lo.ghdot, BH * pl.ncs * 16 * sizeof(float), ngc);
+        const int vn = twins && pl.use_tc ? vcopies : 1;
+        take_n(lo.ddt_dir, vec, vn);
         const size_t vec_tiles = pl.use_tc ? vec : vec * (pl.Q / 64);
-        take2(lo.rho, vec_tiles, vtwin);
-        take2(lo.rho2, vec, vtwin);
-        take2(lo.psi, vec_tiles, vtwin);
-        take2(lo.psi2, vec, vtwin);
+        take_n(lo.rho, vec_tiles, vn);
+        take_n(lo.rho2, vec, vn);
+        take_n(lo.psi, vec_tiles, vn);
+        take_n(lo.psi2, vec, vn);
         const size_t part = (size_t)pl.B * pl.seg * pl.G * pl.nsl * pl.N * sizeof(float);
-        take2(lo.pC, part, twin);
-        if (pl.use_tc) take2(lo.pB, part, twin);
+        take_n(lo.pC, part, ngc);
+        if (pl.use_tc) take_n(lo.pB, part, ngc);
         lo.dAp = take(BH * pl.nct * sizeof(float));
         lo.dDp = take(BH * pl.nct * 4 * sizeof(float));
     }
@@ -243,13 +255,13 @@ static int check_device() {
 // state-gradient part of the chain, s[1] / s[3] the dB/dC kernel of even / odd segments beside dx on the caller's
 // stream, s[2] a segment's finishing kernel.  Created on first use, never
 // destroyed (they hold no device memory); the caller's stream stays the only one the caller has to order
-// against.  Events indexed [2] and [3] go round with the segment, like the copies of the scratch regions.
+// against.  A wait refers to the last record before it, so an event that is waited for before it is recorded again serves every
+// segment; those that are waited for some segments later go round with the copies of the scratch regions.
 struct SideStreams {
     int dev = -1;
     cudaStream_t s[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};   // gradient chain | dB/dC, even | tails | dB/dC, odd | recompute
     cudaEvent_t start = nullptr;
-    cudaEvent_t chain_done[2] = {nullptr, nullptr}, big_done[3] = {nullptr, nullptr, nullptr}, tail_done[3] = {nullptr, nullptr, nullptr};
-    cudaEvent_t rec_done[3] = {nullptr, nullptr, nullptr}, join[2] = {nullptr, nullptr}, dx_done[2] = {nullptr, nullptr};
+    cudaEvent_t chain_done = nullptr, big_done[kChainCopies] = {}, tail_done[kChainCopies] = {}, rec_done = nullptr, join = nullptr, dx_done = nullptr;
 };
 static SideStreams *side_streams() {
     static thread_local std::vector<SideStreams> all;
@@ -261,8 +273,11 @@ static SideStreams *side_streams() {
     a.dev = dev;
     for (int i = 0; i < 5; ++i)
         if (cudaStreamCreateWithFlags(&a.s[i], cudaStreamNonBlocking) != cudaSuccess) return nullptr;
-    cudaEvent_t *evs[] = {&a.start, &a.chain_done[0], &a.chain_done[1], &a.big_done[0], &a.big_done[1], &a.big_done[2], &a.tail_done[0],
-                          &a.tail_done[1], &a.tail_done[2], &a.rec_done[0], &a.rec_done[1], &a.rec_done[2], &a.join[0], &a.join[1], &a.dx_done[0], &a.dx_done[1]};
+    std::vector<cudaEvent_t *> evs = {&a.start, &a.chain_done, &a.rec_done, &a.join, &a.dx_done};
+    for (int i = 0; i < kChainCopies; ++i) {
+        evs.push_back(&a.big_done[i]);
+        evs.push_back(&a.tail_done[i]);
+    }
     for (cudaEvent_t *ev : evs)
         if (cudaEventCreateWithFlags(ev, cudaEventDisableTiming) != cudaSuccess) return nullptr;
     all.push_back(a);
@@ -295,7 +310,7 @@ static SideStreams *side_streams() {
 static void select_copy(const Layout &lo, void *ws, int kc, int k, SegParams &sp) {
     char *w = (char *)ws;
     auto at = [&](size_t r) { return r ? (float *)(w + r) : nullptr; };
-    auto f = [&](const size_t (&r)[2]) { return at(r[k]); };
+    auto f = [&](const auto &r) { return at(r[k]); };
     sp.rec = at(lo.rec[kc]);
     sp.cs = f(lo.cs);
     sp.dtT = sp.rec ? sp.rec + REC_DT : f(lo.dtT);
@@ -361,12 +376,17 @@ static int scan_ctas(const SegParams &sp, bool pipelined, bool bwd) {
     return kNumSMs - beside >= kNumSMs / 4 ? kNumSMs - beside : kNumSMs;
 }
 
-// The tensor maps of copies 0 .. n-1 of the forward chain's output, each with the gradients' copy of the same parity.
-static bool state_maps(const Layout &lo, void *ws, const SegParams &sp0, TcMaps *m, int n) {
+// The tensor maps of copies 0 .. nh-1 of the forward chain's output and 0 .. ng-1 of the gradients.
+static bool state_maps(const Layout &lo, void *ws, const SegParams &sp0, TcMaps *mh, int nh, TcMaps *mg, int ng) {
     SegParams sp = sp0;
-    for (int i = 0; i < n; ++i) {
-        select_copy(lo, ws, i, i & 1, sp);
-        if (!tc_state_maps(sp, m[i])) return false;
+    for (int i = 0; i < nh || i < ng; ++i) {
+        select_copy(lo, ws, i < nh ? i : 0, i < ng ? i : 0, sp);
+        SegParams one = sp;
+        one.Gbf = nullptr;
+        if (i < nh && !tc_state_maps(one, mh[i])) return false;
+        one = sp;
+        one.Hbf = nullptr;
+        if (i < ng && !tc_state_maps(one, mg[i])) return false;
     }
     return true;
 }
@@ -406,17 +426,17 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         // belongs to the chain alone.
         SideStreams *side = side_streams();
         if (!side) { g_last_cuda = (int)cudaGetLastError(); return SSD_ECUDA; }
-        const int ncp = chain_copies(pl.nseg);
-        TcMaps mk[3] = {maps, maps, maps};
-        if (!state_maps(lo, ws, sp, mk, ncp)) return SSD_ECUDA;
+        const int ncp = chain_copies(pl, false);
+        TcMaps mk[kChainCopies] = {maps, maps, maps, maps};
+        if (!state_maps(lo, ws, sp, mk, ncp, nullptr, 0)) return SSD_ECUDA;
         cudaStream_t chain = side->s[0];
         sp.chain_heads = chain_heads(pl, false);
         SSD_TRY(cudaEventRecord(side->start, st));
         SSD_TRY(cudaStreamWaitEvent(chain, side->start, 0));
         for (int k = 0; k < pl.nseg; ++k) {
-            const int par = k & 1, cp = k % ncp;
+            const int cp = k % ncp;
             set_segment(pl, k, sp);
-            select_copy(lo, ws, cp, par, sp);
+            select_copy(lo, ws, cp, 0, sp);
             if (k >= ncp) SSD_TRY(cudaStreamWaitEvent(chain, side->big_done[cp], 0));   // y of segment k - ncp has read this copy
             {
                 cudaStream_t st = chain;
@@ -424,9 +444,9 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
                 float *bnd = boundary ? boundary + (size_t)k * pl.H * PN : nullptr;
                 SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, mk[cp], init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN,
                                                               (k == pl.nseg - 1) ? h_final : nullptr, st));
-                SSD_TRY(cudaEventRecord(side->chain_done[par], st));
+                SSD_TRY(cudaEventRecord(side->chain_done, st));
             }
-            SSD_TRY(cudaStreamWaitEvent(st, side->chain_done[par], 0));
+            SSD_TRY(cudaStreamWaitEvent(st, side->chain_done, 0));
             sp.scan_ctas = scan_ctas(sp, k + 1 < pl.nseg, false);
             SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, mk[cp], SC_FWD, st));
             if (k + ncp < pl.nseg) SSD_TRY(cudaEventRecord(side->big_done[cp], st));
@@ -605,10 +625,10 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         // big(k) / tail(k) read exists more than once and goes round with the segments; the carried gradient belongs to the
         // chain alone.
         const bool twin = pl.nseg >= kMinSegmentsForTwins;    // else one copy of what the gradient chain writes
-        const int ncp = chain_copies(pl.nseg), npar = twin ? 2 : 1;
+        const int ncp = chain_copies(pl, true), npar = grad_copies(pl);
         sp.chain_heads = chain_heads(pl, pl.nseg > 1);
-        TcMaps cmaps[3] = {maps, maps, maps};
-        if (!state_maps(lo, ws, sp, cmaps, ncp)) return SSD_ECUDA;
+        TcMaps cmaps[kChainCopies] = {maps, maps, maps, maps}, gmaps[kGradCopies];
+        if (!state_maps(lo, ws, sp, cmaps, ncp, gmaps, npar)) return SSD_ECUDA;
         cudaStream_t grads = side->s[0], recomp = side->s[4], tails = side->s[2];
         SSD_TRY(cudaEventRecord(side->start, st));
         SSD_TRY(cudaStreamWaitEvent(recomp, side->start, 0));
@@ -618,33 +638,34 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
             set_segment(pl, k, sp);
             select_copy(lo, ws, cp, par, sp);
             TcMaps mk = cmaps[cp];
-            if (par != (cp & 1)) { mk.G = cmaps[par].G; mk.Gst = cmaps[par].Gst; }
+            mk.G = gmaps[par].G;
+            mk.Gst = gmaps[par].Gst;
             // ---- chain(k), first half: Recompute_Forward.  Its copy was last read by big(k + ncp) and tail(k + ncp).
-            if (i >= ncp) SSD_TRY(cudaStreamWaitEvent(recomp, side->tail_done[(i - ncp) % 3], 0));
+            if (i >= ncp) SSD_TRY(cudaStreamWaitEvent(recomp, side->tail_done[(i - ncp) % kChainCopies], 0));
             {
                 cudaStream_t st = recomp;
                 SSD_LAUNCH(KIND_CHUNK_STATE, launch_chain_fwd(sp, mk, boundary + (size_t)k * pl.H * PN, (long long)pl.nseg * pl.H * PN,
                                                               nullptr, 0, nullptr, st));
-                SSD_TRY(cudaEventRecord(side->rec_done[cp], st));
+                SSD_TRY(cudaEventRecord(side->rec_done, st));
             }
             // ---- chain(k), second half: the state gradients, which alone wait for segment k+1 (stream order: the
             // gradient handed left)
             // What it writes was last read by big and tail of the segment npar before.
-            SSD_TRY(cudaStreamWaitEvent(grads, side->rec_done[cp], 0));
-            if (i >= npar) SSD_TRY(cudaStreamWaitEvent(grads, side->tail_done[(i - npar) % 3], 0));
+            SSD_TRY(cudaStreamWaitEvent(grads, side->rec_done, 0));
+            if (i >= npar) SSD_TRY(cudaStreamWaitEvent(grads, side->tail_done[(i - npar) % kChainCopies], 0));
             {
                 cudaStream_t st = grads;
                 const float *ginit = (k == pl.nseg - 1) ? dh_final : sp.gcarry;
                 float *gleft = (k == 0 && dh0) ? dh0 : sp.gcarry;
                 SSD_LAUNCH(KIND_DSTATE, launch_chain_bwd(sp, mk, ginit, gleft, st));
-                SSD_TRY(cudaEventRecord(side->chain_done[par], st));
+                SSD_TRY(cudaEventRecord(side->chain_done, st));
             }
             // ---- big(k); what it leaves for tail(k) (direct ddt, rho, psi, partial dB/dC slices) alternates too, and
             // chain(k) has already waited for the last reader of this copy.  The dB/dC kernels of
             // neighbouring segments are on different streams: with short segments one alone does not fill the GPU.
-            cudaStream_t bcs = side->s[par ? 3 : 1];
-            SSD_TRY(cudaStreamWaitEvent(st, side->chain_done[par], 0));
-            SSD_TRY(cudaStreamWaitEvent(bcs, side->chain_done[par], 0));
+            cudaStream_t bcs = side->s[i & 1 ? 3 : 1];
+            SSD_TRY(cudaStreamWaitEvent(st, side->chain_done, 0));
+            SSD_TRY(cudaStreamWaitEvent(bcs, side->chain_done, 0));
             {
                 cudaStream_t st = bcs;
                 if (!split_bc) {
@@ -653,21 +674,21 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
                     SSD_LAUNCH(KIND_BWD_DC, launch_grad_bc(sp, mk, BC_DC, st));
                     SSD_LAUNCH(KIND_BWD_DB, launch_grad_bc(sp, mk, BC_DB, st));
                 }
-                SSD_TRY(cudaEventRecord(side->join[par], st));
+                SSD_TRY(cudaEventRecord(side->join, st));
             }
             sp.scan_ctas = scan_ctas(sp, twin, true);
             SSD_LAUNCH(KIND_BWD_DX, launch_scan_tc(sp, mk, SC_DX, st));
-            SSD_TRY(cudaEventRecord(side->dx_done[par], st));
+            SSD_TRY(cudaEventRecord(side->dx_done, st));
             // ---- tail(k), after both
-            SSD_TRY(cudaStreamWaitEvent(tails, side->dx_done[par], 0));
-            SSD_TRY(cudaStreamWaitEvent(tails, side->join[par], 0));
+            SSD_TRY(cudaStreamWaitEvent(tails, side->dx_done, 0));
+            SSD_TRY(cudaStreamWaitEvent(tails, side->join, 0));
             {
                 cudaStream_t st = tails;
                 SSD_LAUNCH(KIND_BWD_FINISH, launch_bwd_tail(sp, pl.dtype, st));
-                SSD_TRY(cudaEventRecord(side->tail_done[i % 3], st));
+                SSD_TRY(cudaEventRecord(side->tail_done[i % kChainCopies], st));
             }
         }
-        SSD_TRY(cudaStreamWaitEvent(st, side->tail_done[(pl.nseg - 1) % 3], 0));   // the finishing stream is in order: this covers every segment
+        SSD_TRY(cudaStreamWaitEvent(st, side->tail_done[(pl.nseg - 1) % kChainCopies], 0));   // the finishing stream is in order: this covers every segment
     } else {
         sp.chain_heads = chain_heads(pl, false);
         for (int k = pl.nseg - 1; k >= 0; --k) {
