@@ -251,7 +251,7 @@ static int check_device() {
 }
 
 // Helper streams per (host thread, device) with the events that fork them off the caller's stream and join them
-// back: s[4] recomputes a segment's chunk states (in the forward: the whole state chain is on s[0]), s[0] runs the
+// back: s[4] recomputes a segment's chunk states (in the forward: the whole state chain is on s[0], y of odd segments on s[1]), s[0] runs the
 // state-gradient part of the chain, s[1] / s[3] the dB/dC kernel of even / odd segments beside dx on the caller's
 // stream, s[2] a segment's finishing kernel.  Created on first use, never
 // destroyed (they hold no device memory); the caller's stream stays the only one the caller has to order
@@ -446,11 +446,20 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
                                                               (k == pl.nseg - 1) ? h_final : nullptr, st));
                 SSD_TRY(cudaEventRecord(side->chain_done, st));
             }
-            SSD_TRY(cudaStreamWaitEvent(st, side->chain_done, 0));
+            // y of a segment waits for its chain alone: on two streams in turn its CTAs take the SMs of the one before as they come free,
+            // where in one stream the next launch began some 6 us after the end (80 heads, 4096 steps: a segment 54 -> 49 us; dx of
+            // neighbouring segments on two streams: no change there, 24 heads 2 % slower)
+            cudaStream_t ys = k & 1 ? side->s[1] : st;
+            SSD_TRY(cudaStreamWaitEvent(ys, side->chain_done, 0));
             sp.scan_ctas = scan_ctas(sp, k + 1 < pl.nseg, false);
-            SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, mk[cp], SC_FWD, st));
-            if (k + ncp < pl.nseg) SSD_TRY(cudaEventRecord(side->big_done[cp], st));
+            {
+                cudaStream_t st = ys;
+                SSD_LAUNCH(KIND_SCAN_FWD, launch_scan_tc(sp, mk[cp], SC_FWD, st));
+                if (k + ncp < pl.nseg) SSD_TRY(cudaEventRecord(side->big_done[cp], st));
+                if ((k & 1) && k + 2 >= pl.nseg) SSD_TRY(cudaEventRecord(side->join, st));
+            }
         }
+        SSD_TRY(cudaStreamWaitEvent(st, side->join, 0));        // the last one on the helper stream
         return SSD_OK;
     }
     sp.chain_heads = chain_heads(pl, false);
