@@ -137,7 +137,13 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                 for (int nh = 0; nh < NS / 64; ++nh) tma_load_3d(sb + nh * 16384, &tmV, &full[st], g * NS + nh * 64, tok, b);
             };
             const int ahead = nc < CH_STAGES ? nc : CH_STAGES;
-            for (int i = 0; i < ahead; ++i) load_inputs(i);
+            // The first step sizes would arrive behind all the stages of all CTAs (15.7 MB with 80 heads: the first block scaled 9100 cycles
+            // after the start, now 7000) and everything waits for them: the later stages wait for the first record instead.  Forward
+            // of one segment, 80 heads: 4096 steps 68.8 -> 67.5 us, 16384 in 8 groups 226 -> 218; 24 heads the same.
+            for (int i = 0; i < ahead; ++i) {
+                if (!BWD && i == 1) mbar_wait(vfull, 0, abortp, p.status);
+                load_inputs(i);
+            }
             if (BWD) pdl_wait();                   // the records and states of the forward chain
             for (int i = 0; i < nc; ++i) {
                 const int st = i % CH_STAGES, c = chunk_of(i);
