@@ -156,14 +156,16 @@ cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, long lo
 // cores with fp32 operands as three bf16 parts (ssd_split.cuh): three products where the other operand is bf16 as it stands, six
 // where both are fp32, one where neither is.  Operands are staged as rows, split on the way; the next stage's global loads are in
 // flight while a stage is multiplied.  With FFMA on the CUDA cores (4 x 4 outputs per thread, bound by the shared-memory reads) the
-// large kernel took 309 us (2 x 2048 steps of 32 heads, N = 64, chunk 128, bf16) and 215 us (2 x 1024 of 24, N = 128, fp32), now 139 and
-// 143.  Bound by latency at 16 warps per SM (issue 45, 38 %, tensor pipe 25, 45 %, shared memory 45, 49 %); held to the 80 registers of
-// three CTAs per SM it spills and takes the same time.
+// large kernel took 309 us (2 x 2048 steps of 32 heads, N = 64, chunk 128, bf16) and 215 us (2 x 1024 of 24, N = 128, fp32), now 120
+// and 143.  Bound by latency: masks, splits and addresses around each product, between barriers, at 24 (fp32: 16) warps per SM (of 550
+// TFLOP/s that mma.sync does here the tensor pipe is 30, 45 % busy).  bf16 takes 80 registers a thread, for three CTAs per SM, with
+// some spills: 2 x 8192 steps 1228 -> 1108 us; fp32, with more parts in registers, takes 128 (at 80: 1112 -> 1260 us).
 //
 // What does not depend on the head is not done per head: C B^T is made once per group (k_simt_sums writes it, 64 x 64 causal
 // tiles), and dB / dC come from a head sum of the masked tiles, one product per CTA instead of two per head.
 template <typename T> struct SimtSmem {
     static constexpr int PT = SplitParts<T>::n;      // parts of a value of the caller's tensors
+    static constexpr int CTAS = PT == 1 ? 3 : 2;     // CTAs per SM
     SplitTile t[3 + PT];
     float css[256], dts[256], fac[256], red[6][64];
 };
@@ -206,12 +208,12 @@ __device__ __forceinline__ float *cb_of(const SegParams &p, int b, int c, int g)
     return p.cbt + (((size_t)b * p.ncs + c) * p.G + g) * (size_t)(p.Q * p.Q);
 }
 // an output tile in accumulator layout to rows of `stride` floats: four lanes fill a 32-byte sector
-template <bool SPLIT = true> __device__ __forceinline__ void store_acc(const Acc &acc, float *out, size_t stride) {
+__device__ __forceinline__ void store_acc(const Acc &acc, float *out, size_t stride) {
 #pragma unroll
     for (int half = 0; half < 2; ++half)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-            *reinterpret_cast<float2 *>(out + (size_t)acc_row(half) * stride + acc_col(j)) = acc.get<SPLIT>(j, half);
+            *reinterpret_cast<float2 *>(out + (size_t)acc_row(half) * stride + acc_col(j)) = acc.get(j, half);
 }
 // two neighbouring elements of an accumulator-layout tile as three parts
 __device__ __forceinline__ void put_acc(SplitTile *s, int half, int j, float a, float b) {
@@ -229,9 +231,12 @@ constexpr float kMildTile = 8.f;
 //   S_c[p,n] = sum_s exp(cs_last - cs_s) dt_s x_s[p] B_s[n]     -> Hst slot c+1   (and cs, dtT)
 //   with grads: E_c[p,n] = sum_t exp(cs_t) dy_t[p] C_t[n]       -> Gst slot c      (its CTAs make the cumsum again)
 //   the causal tiles of C B^T, where the scratch has room for them
+// Both sums of a (head, chunk) by one CTA, with one cumsum, where there are CTAs enough (2 x 8192 steps of 32 heads 1103 -> 1082 us);
+// else two, side by side.
+template <int NS> __host__ __device__ __forceinline__ bool simt_sums_merged(const SegParams &p) { return p.nc * p.B * (NS / 64) * p.H >= 2 * kNumSMs; }
 template <typename T, int NS> __host__ __device__ __forceinline__ int simt_n_sums(const SegParams &p, bool grads) {
     const int nrt = p.Q >> 6;
-    return p.nc * p.B * ((NS / 64) * p.H * (grads ? 2 : 1) + (p.cbt ? p.G * (nrt * (nrt + 1) / 2) : 0));
+    return p.nc * p.B * ((NS / 64) * p.H * (grads && !simt_sums_merged<NS>(p) ? 2 : 1) + (p.cbt ? p.G * (nrt * (nrt + 1) / 2) : 0));
 }
 template <typename T, int NS> __device__ __forceinline__ void simt_sums(const SegParams &p, SimtSmem<T> &sm, int id, bool grads) {
     constexpr int PT = SimtSmem<T>::PT;
@@ -242,10 +247,11 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
     Acc acc;
     TileRegs<T> ra, rb;
     acc.zero();
-    const bool dst = grads && id >= nsum && id < 2 * nsum;
-    if (dst) id -= nsum;
+    const bool merged = grads && simt_sums_merged<NS>(p);
+    const bool second = grads && !merged && id >= nsum && id < 2 * nsum;       // a CTA for E alone
+    if (second) id -= nsum;
     else if (id >= nsum) {      // a causal tile of C B^T
-        id -= grads ? 2 * nsum : nsum;
+        id -= grads && !merged ? 2 * nsum : nsum;
         const int npair = nrt * (nrt + 1) / 2;
         int rt, ct;
         pair_of(id % npair, rt, ct);
@@ -262,17 +268,20 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
             __syncthreads();
             tile_mma<PT, PT, false, false>(acc, sm.t, sm.t + PT);
         }
-        store_acc<(PT > 1)>(acc, cb_of(p, b, c, g) + (size_t)rt * 64 * Q + ct * 64, Q);
+        store_acc(acc, cb_of(p, b, c, g) + (size_t)rt * 64 * Q + ct * 64, Q);
         return;
     }
     const int n0 = (id % nh) * 64;
     id /= nh;
     const int h = id % p.H, c = (id / p.H) % p.nc, b = id / (p.H * p.nc), g = h / p.hpg;
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q;
-    const T *rows = (const T *)(dst ? p.dy : p.x) + (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
-    const T *cols = (const T *)(dst ? p.Cm : p.Bm) + (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS + n0;
-    tile_load(ra, rows, HP);
-    tile_load(rb, cols, GN);
+    const size_t xo = (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64, bo = (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS + n0;
+    float *wsm2 = sm.dts;                                                       // the weights of E
+    auto load_rows = [&](bool dst, int s0) {
+        tile_load(ra, (const T *)(dst ? p.dy : p.x) + xo + (size_t)s0 * HP, HP);
+        tile_load(rb, (const T *)(dst ? p.Cm : p.Bm) + bo + (size_t)s0 * GN, GN);
+    };
+    load_rows(second, 0);
     // the chunk cumsum by one warp: a lane sums its Q/32 consecutive steps in order, then a shuffle scan over the lanes
     if (tid < 32) {
         const int per = Q >> 5;
@@ -301,18 +310,23 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
             if (k < per) {
                 const int t = tid * per + k;
                 const float cs = v[k] + excl;
-                wsm[t] = dst ? expf(cs) : expf(fminf(last - cs, 0.f)) * d[k];
-                if (n0 == 0 && !dst) {
+                if (!second) wsm[t] = expf(fminf(last - cs, 0.f)) * d[k];
+                if (second || merged) wsm2[t] = expf(cs);
+                if (n0 == 0 && !second) {
                     p.cs[vec_off(p, b, h, c) + t] = cs;
                     p.dtT[vec_off(p, b, h, c) + t] = d[k];
                 }
             }
     }
     __syncthreads();
-    for (int s0 = 0; s0 < Q; s0 += 64) {
+    const int end = merged ? 2 * Q : Q;
+    for (int i0 = 0; i0 < end; i0 += 64) {
+        const bool dst = second || i0 >= Q;
+        const int s0 = i0 >= Q ? i0 - Q : i0;
+        const float *wv = dst ? wsm2 : wsm;
 #pragma unroll
         for (int k = 0; k < TileRegs<T>::N; ++k) {
-            const float w = wsm[s0 + ra.row(k)];
+            const float w = wv[s0 + ra.row(k)];
             float f[TileRegs<T>::COLS];
             ra.get(k, f);
 #pragma unroll
@@ -321,17 +335,17 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
         }
         tile_store(sm.t + 3, rb);
         __syncthreads();
-        if (s0 + 64 < Q) {
-            tile_load(ra, rows + (size_t)(s0 + 64) * HP, HP);
-            tile_load(rb, cols + (size_t)(s0 + 64) * GN, GN);
-        }
+        if (i0 + 64 < end) load_rows(second || i0 + 64 >= Q, i0 + 64 >= Q ? i0 + 64 - Q : i0 + 64);
         tile_mma<3, PT, true, true>(acc, sm.t, sm.t + 3);
+        if (s0 + 64 == Q) {
+            store_acc(acc, (dst ? p.Gst + slot_off(p, b, c, h) : p.Hst + slot_off(p, b, c + 1, h)) + n0, NS);
+            acc.zero();
+        }
         __syncthreads();
     }
-    store_acc(acc, (dst ? p.Gst + slot_off(p, b, c, h) : p.Hst + slot_off(p, b, c + 1, h)) + n0, NS);
 }
 
-template <typename T, int NS> __global__ void __launch_bounds__(256, 2) k_simt_sums(SegParams p, bool grads) {
+template <typename T, int NS> __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_sums(SegParams p, bool grads) {
     extern __shared__ __align__(16) unsigned char smem[];
     pdl_launch_dependents();
     pdl_wait();
@@ -437,7 +451,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int t = r0 + acc_row(half), s = ct * 64 + acc_col(j);
-                    const float2 v2 = cb.template get<(PT > 1)>(j, half);
+                    const float2 v2 = cb.get(j, half);
                     float e[2] = {v2.x, v2.y};
 #pragma unroll
                     for (int i = 0; i < 2; ++i) {
@@ -518,7 +532,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
 // y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
 // wait for nothing of this one, and a launch of a few microseconds is saved per segment.
 template <typename T, int NS, bool CB>
-__global__ void __launch_bounds__(256, 2) k_simt_y(SegParams p, SegParams nx, int n_next) {
+__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, SegParams nx, int n_next) {
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();
@@ -540,7 +554,7 @@ __global__ void __launch_bounds__(256, 2) k_simt_y(SegParams p, SegParams nx, in
 // A row of tile r has dC slots for ts <= r and dB slots for tt >= r, so the two share Q/64 + 3 slots per head range: dC by ts, dB by
 // tt + 1, then the inter-chunk terms of both.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
+__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p, int n_dx) {
     constexpr int PT = SimtSmem<T>::PT;
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
@@ -628,7 +642,7 @@ __global__ void __launch_bounds__(256, 2) k_simt_bwd(SegParams p, int n_dx) {
                         e.x = expf(fminf(one - rowv[s], 0.f)) * two.x;
                         e.y = expf(fminf(one - rowv[s + 1], 0.f)) * two.y;
                     }
-                    float2 w = __fmul2_rn(acc.get<(PT > 1)>(j, half), e);
+                    float2 w = __fmul2_rn(acc.get(j, half), e);
                     if (diag) {
                         w.x = s <= t ? w.x : 0.f;
                         w.y = s < t ? w.y : 0.f;
@@ -910,7 +924,7 @@ __global__ void __launch_bounds__(256) k_bwd_tail(SegParams p, int nfin) {
 // split path: the same with the sums of the next segment (to the left) in front, which share no scratch with it but the step
 // sizes, of which there are two copies.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256, 2) k_simt_tail(SegParams p, SegParams nx, int n_next, int nfin) {
+__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_tail(SegParams p, SegParams nx, int n_next, int nfin) {
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();

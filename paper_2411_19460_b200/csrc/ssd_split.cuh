@@ -4,9 +4,9 @@
 //   x = p0 + p1 + p2:  p0 the upper half of x's bits (no overflow near the largest values), p1 the rest rounded to nearest, so
 //   that what it leaves for p2 has either sign, p2 the rest of that, at most eight bits.
 // Products p_i q_j with i + j > 2 are left out (below 2^-23 of x y each, of either sign: about 2^-25 on average).  mma.sync truncates when it
-// adds to its accumulator, a bias of half a unit in the last place per step, so the product of the first parts starts from zero
-// for every 32 steps of the contraction and is added with a rounded fp32 addition; the others, 2^-7 of it and less, share an
-// accumulator of their own.  Infinities come out as infinities or NaN (0 x infinity in another part), NaN as NaN.
+// adds to its accumulator, a bias of half a unit in the last place per step, so for every 16 steps of the contraction the products
+// start from zero, the smallest first, and their sum is added with a rounded fp32 addition: one truncation at the size of the sum.
+// Infinities come out as infinities or NaN (0 x infinity in another part), NaN as NaN.
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -21,7 +21,6 @@ constexpr int SP_ROW = 72;          // bf16 per staged row of 64: 144 bytes, so 
 struct SplitTile {
     __nv_bfloat16 v[64][SP_ROW];
 };
-constexpr int SP_FLUSH = 32;         // steps of the contraction that the product of the first parts takes before it is added with rounding
 template <typename T> struct SplitParts;
 template <> struct SplitParts<float> { static constexpr int n = 3; };
 template <> struct SplitParts<__nv_bfloat16> { static constexpr int n = 1; };
@@ -97,22 +96,18 @@ __device__ __forceinline__ void tile_store(SplitTile *s, const TileRegs<float> &
 // ---- products.  Eight warps, warp (wm, wn) has rows 16 wm .. and columns 32 wn .. of the output in the accumulator layout of
 // mma.m16n8k16: element (j, i) is row acc_row(i >> 1), column acc_col(j) + (i & 1).
 struct Acc {
-    float m[4][4], s[4][4];         // products of the first parts | all others
+    float m[4][4];
     __device__ __forceinline__ void zero() {
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
-            for (int i = 0; i < 4; ++i) m[j][i] = s[j][i] = 0.f;
+            for (int i = 0; i < 4; ++i) m[j][i] = 0.f;
     }
     // rows of half `half`, columns acc_col(j) and the next
-    template <bool SPLIT = true> __device__ __forceinline__ float2 get(int j, int half) const {
-        const float2 a = make_float2(m[j][2 * half], m[j][2 * half + 1]);
-        return SPLIT ? __fadd2_rn(a, make_float2(s[j][2 * half], s[j][2 * half + 1])) : a;
-    }
+    __device__ __forceinline__ float2 get(int j, int half) const { return make_float2(m[j][2 * half], m[j][2 * half + 1]); }
     __device__ __forceinline__ void set(int j, int half, float2 v) {
         m[j][2 * half] = v.x;
         m[j][2 * half + 1] = v.y;
-        s[j][2 * half] = s[j][2 * half + 1] = 0.f;
     }
 };
 __device__ __forceinline__ int acc_row(int half) { return ((threadIdx.x >> 5) & 3) * 16 + ((threadIdx.x >> 2) & 7) + half * 8; }
@@ -148,39 +143,33 @@ template <int PA, int PB, bool AK, bool BK> __device__ __forceinline__ void tile
     constexpr uint32_t ROWB = SP_ROW * 2, PART = sizeof(SplitTile);
     const uint32_t aa = sm100::smem_u32(a) + (AK ? (l16 + l7) * ROWB + (wm + l8) * 2 : (wm + l8 + l7) * ROWB + l16 * 2);
     const uint32_t ba = sm100::smem_u32(b) + (BK ? (l8 + l7) * ROWB + (wn + l16) * 2 : (wn + l16 + l7) * ROWB + l8 * 2);
-    float t[4][4];
 #pragma unroll
     for (int k = 0; k < 64; k += 16) {
         uint32_t fa[PA][4];
+        float t[4][4];
 #pragma unroll
         for (int p = 0; p < PA; ++p) ldsm4<AK>(fa[p], aa + p * PART + (AK ? k * ROWB : k * 2));
+        bool first = true;
 #pragma unroll
-        for (int q = 0; q < PB; ++q) {
+        for (int q = PB - 1; q >= 0; --q) {
             uint32_t fb[2][4];
 #pragma unroll
             for (int n = 0; n < 2; ++n) ldsm4<BK>(fb[n], ba + q * PART + (BK ? k * ROWB + n * 32 : k * 2 + n * 16 * ROWB));
 #pragma unroll
-            for (int p = 0; p < PA; ++p) {
+            for (int p = PA - 1; p >= 0; --p) {
                 if (p + q > 2) continue;
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    const uint32_t b0 = fb[j >> 1][(j & 1) * 2], b1 = fb[j >> 1][(j & 1) * 2 + 1];
-                    if (p + q > 0) mma_acc(c.s[j], fa[p], b0, b1);
-                    else if (k % SP_FLUSH == 0) mma_zero(t[j], fa[0], b0, b1);
-                    else mma_acc(t[j], fa[0], b0, b1);
+                    if (first) mma_zero(t[j], fa[p], fb[j >> 1][(j & 1) * 2], fb[j >> 1][(j & 1) * 2 + 1]);
+                    else mma_acc(t[j], fa[p], fb[j >> 1][(j & 1) * 2], fb[j >> 1][(j & 1) * 2 + 1]);
                 }
+                first = false;
             }
         }
-        if (k % SP_FLUSH == SP_FLUSH - 16) {
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
+        for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int i = 0; i < 4; i += 2) {
-                    const float2 v = __fadd2_rn(make_float2(c.m[j][i], c.m[j][i + 1]), make_float2(t[j][i], t[j][i + 1]));
-                    c.m[j][i] = v.x;
-                    c.m[j][i + 1] = v.y;
-                }
-        }
+            for (int half = 0; half < 2; ++half) c.set(j, half, __fadd2_rn(c.get(j, half), make_float2(t[j][2 * half], t[j][2 * half + 1])));
     }
 }
 
