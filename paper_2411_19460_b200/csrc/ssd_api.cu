@@ -156,6 +156,15 @@ static bool simt_overlap(const Plan &pl, bool bwd) {
     return pl.nseg > 1 && (bwd || copy <= (size_t)64 << 20);
 }
 
+// split path: whether the readers of a state make it from the sums of the segment's other chunks.  That saves a launch per segment and
+// direction, some 6 us, and reads 16 KB tiles that a state pass would have added up.  Forward + backward, us, with passes and without,
+// by the number of those tiles a launch of y: 24 (1024 steps of 4 heads) 146 and 129, 288 (4096 of 24 heads) 526 and 453, 768 (2 x 4096 of
+// 8, N = 128) 550 and 540, 896 316 and 282, 1344 (8192 of 24 heads) 1287 and 1387, 2304 1112 and 1133.
+static bool simt_readers(const Plan &pl) {
+    const long long tiles = (long long)pl.ncs * (pl.ncs - 1) / 2 * (pl.Q / 64) * pl.B * pl.H * (pl.N / 64);
+    return !pl.use_tc && pl.ncs <= kReaderChunks && tiles <= 1024;
+}
+
 // Copies of what the forward chain leaves, and of what the gradient chain and the large kernels leave (tensor-core path).  A copy comes
 // back when its segment's tail is done: chain, dB/dC beside dx, tail and the hand-overs take 77 us of 24 heads and 2048 steps, so with
 // two copies a segment can start every 38 us, while the gradient chain alone takes 28; the recompute likewise with three.  Where
@@ -464,6 +473,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     }
     sp.chain_heads = chain_heads(pl, false);
     const bool overlap = beside && simt_overlap(pl, false);
+    const bool readers = beside && simt_readers(pl) && (overlap || pl.nseg == 1);       // a segment's exit state needs the next one's copy
     SegParams next;
     for (int k = 0; k < pl.nseg; ++k) {
         set_segment(pl, k, sp);
@@ -475,15 +485,23 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
             continue;
         }
         select_copy(lo, ws, 0, k & 1, sp);
-        if (k == 0 || !overlap) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, pl.dtype, SIMT_SUMS, st));
-        SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN, fin, st));
+        if (k == 0 || !overlap) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, nullptr, pl.dtype, SIMT_SUMS, st));
+        StatePass pass = {bnd, nullptr, fin, (int64_t)pl.nseg * pl.H * PN, 0};
+        if (readers) {
+            sp.hinit = k == 0 ? h0 : sp.Hst;
+            sp.hinit_bs = k == 0 ? pl.H * PN : (pl.ncs + 1) * pl.H * PN;
+        } else {
+            SSD_LAUNCH(KIND_STATE_PASS_FWD, launch_state_pass_fwd(sp, init, (long long)pl.H * PN, bnd, (long long)pl.nseg * pl.H * PN, fin, st));
+        }
         const bool ahead = overlap && k + 1 < pl.nseg;      // the next segment's sums in the launch of y
         if (ahead) {
             next = sp;
             set_segment(pl, k + 1, next);
             select_copy(lo, ws, 0, (k + 1) & 1, next);
+            pass.leave = next.Hst;                          // slot 0 of the next segment's copy
+            pass.leave_bs = (pl.ncs + 1) * pl.H * PN;
         }
-        SSD_LAUNCH(KIND_SCAN_FWD, launch_simt(sp, ahead ? &next : nullptr, pl.dtype, SIMT_Y, st));
+        SSD_LAUNCH(KIND_SCAN_FWD, launch_simt(sp, ahead ? &next : nullptr, readers ? &pass : nullptr, pl.dtype, SIMT_Y, st));
     }
     return SSD_OK;
 }
@@ -718,14 +736,29 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
                 }
             } else {
                 select_copy(lo, ws, 0, k & 1, sp);
-                if (k == pl.nseg - 1 || pl.serial) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, pl.dtype, SIMT_SUMS_GRAD, st));
-                SSD_LAUNCH(KIND_STATE_PASS_BWD, launch_state_pass_bwd(sp, hin, (long long)pl.nseg * pl.H * PN, ginit, gleft, st));
-                SSD_LAUNCH(KIND_BWD_DX, launch_simt(sp, nullptr, pl.dtype, SIMT_BWD, st));
+                if (k == pl.nseg - 1 || pl.serial) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, nullptr, pl.dtype, SIMT_SUMS_GRAD, st));
+                if (!pl.serial && simt_readers(pl)) {
+                    // the gradient handed left is written while the one from the right is read: in gcarry and the last slot of Gst in turn
+                    const int64_t own = pl.H * PN, slots = (pl.ncs + 1) * pl.H * PN;
+                    float *const turn[2] = {sp.gcarry, sp.Gst + (size_t)pl.ncs * pl.H * PN};
+                    const int i = pl.nseg - 1 - k;
+                    sp.hinit = hin;
+                    sp.hinit_bs = pl.nseg * pl.H * PN;
+                    sp.ginit = i == 0 ? dh_final : turn[i & 1];
+                    sp.ginit_bs = i == 0 || !(i & 1) ? own : slots;
+                    StatePass pass = {};
+                    pass.leave = k == 0 && dh0 ? dh0 : turn[(i + 1) & 1];
+                    pass.leave_bs = (k == 0 && dh0) || !((i + 1) & 1) ? own : slots;
+                    SSD_LAUNCH(KIND_BWD_DX, launch_simt(sp, nullptr, &pass, pl.dtype, SIMT_BWD, st));
+                } else {
+                    SSD_LAUNCH(KIND_STATE_PASS_BWD, launch_state_pass_bwd(sp, hin, (long long)pl.nseg * pl.H * PN, ginit, gleft, st));
+                    SSD_LAUNCH(KIND_BWD_DX, launch_simt(sp, nullptr, nullptr, pl.dtype, SIMT_BWD, st));
+                }
                 if (k > 0 && !pl.serial) {
                     SegParams next = sp;
                     set_segment(pl, k - 1, next);
                     select_copy(lo, ws, 0, (k - 1) & 1, next);
-                    SSD_LAUNCH(KIND_BWD_FINISH, launch_simt(sp, &next, pl.dtype, SIMT_TAIL, st));
+                    SSD_LAUNCH(KIND_BWD_FINISH, launch_simt(sp, &next, nullptr, pl.dtype, SIMT_TAIL, st));
                     continue;
                 }
             }

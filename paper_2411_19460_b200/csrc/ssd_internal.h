@@ -104,6 +104,8 @@ struct SegParams {
     float *Gst;            // split path: [B,ncs+1,H,P,N] slot c+1 = dLoss/d(state leaving chunk c)
     __nv_bfloat16 *Hbf;    // tensor-core path: [B,ncs,H,N,P] (transposed) state entering block c
     __nv_bfloat16 *Gbf;    // tensor-core path: [B,ncs,H,N,P] dLoss/d(state leaving block c)
+    const float *hinit, *ginit;     // split path, states made by their readers: state (gradient) entering the segment from the left
+    int64_t hinit_bs, ginit_bs;     // (right), null = zeros, and their batch strides
     float *hcarry;         // [B,H,P,N]     state handed from segment to segment (forward; null in the backward, which does not)
     float *gcarry;         // [B,H,P,N]     state gradient handed right-to-left (backward)
     float *ghdot;          // [B,H,ncs,16]  partial sums of exp(cs_last) <Gout_c, H_in,c>
@@ -124,8 +126,15 @@ static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; 
 // ssd_simt.cu : kernels of the split path (fp32 operands as bf16 parts), any I/O dtype
 // SIMT_SUMS: chunk sums, cumsum and C B^T | SIMT_SUMS_GRAD: also the state-gradient sums | SIMT_Y: y, and the sums of segment
 // `next` if given | SIMT_BWD: dx, slices of dB and dC | SIMT_TAIL: finishing steps and the sums (with gradients) of segment `next`
+// Short segments need no state pass: with `pass`, whoever reads a state in SIMT_Y or SIMT_BWD makes it from the chunk sums (which stay),
+// and CTAs of the same launch make what the pass hands on.
+constexpr int kReaderChunks = 8;       // chunks of such a segment, at most
+struct StatePass {
+    float *boundary, *leave, *fin;     // state entering the segment (null: not stored) | state (backward: gradient) leaving it | h_final (or null)
+    int64_t boundary_bs, leave_bs;
+};
 enum { SIMT_SUMS = 0, SIMT_SUMS_GRAD, SIMT_Y, SIMT_BWD, SIMT_TAIL };
-cudaError_t launch_simt(const SegParams &p, const SegParams *next, int dtype, int what, cudaStream_t st);
+cudaError_t launch_simt(const SegParams &p, const SegParams *next, const StatePass *pass, int dtype, int what, cudaStream_t st);
 // init: state entering the segment (NULL = zeros), batch stride init_bs elements;
 // boundary_out (nullable): where to store that state, batch stride bnd_bs; final_out nullable.
 cudaError_t launch_state_pass_fwd(const SegParams &p, const float *init, long long init_bs,

@@ -352,13 +352,109 @@ template <typename T, int NS> __global__ void __launch_bounds__(256, SimtSmem<T>
     simt_sums<T, NS>(p, *reinterpret_cast<SimtSmem<T> *>(smem), blockIdx.x, grads);
 }
 
+template <int NS> __device__ __forceinline__ size_t slot_of(const SegParams &p, int b, int slot, int h) {
+    return (((size_t)b * (p.ncs + 1) + slot) * p.H + h) * (size_t)(64 * NS);
+}
+// Columns k0 .. k0 + 63 of the state entering chunk c (GRAD: of the gradient leaving it): from the slot that a state pass filled, or
+// (READER) made here from the sums of the chunks on that side, with the pass's operations in its order, so with the same bits.
+template <int NS, bool GRAD, bool READER>
+__device__ __forceinline__ void load_state(TileRegs<float> &r, const SegParams &p, int b, int h, int c, int k0) {
+    const float *slots = GRAD ? p.Gst : p.Hst;
+    if constexpr (!READER) {
+        tile_load<true>(r, slots + slot_of<NS>(p, b, GRAD ? c + 1 : c, h) + k0, NS);
+    } else {
+        const float *init = GRAD ? p.ginit : p.hinit, *csl = p.cs + vec_off(p, b, h, 0) + (p.Q - 1);
+        if (init) {
+            tile_load<true>(r, init + (size_t)b * (GRAD ? p.ginit_bs : p.hinit_bs) + (size_t)h * 64 * NS + k0, NS);
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) r.v[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        const int n = GRAD ? p.nc - 1 - c : c;
+        for (int i = 0; i < n; ++i) {
+            const int j = GRAD ? p.nc - 1 - i : i;
+            TileRegs<float> s;
+            tile_load<true>(s, slots + slot_of<NS>(p, b, GRAD ? j : j + 1, h) + k0, NS);
+            const float decay = expf(csl[(size_t)j * p.Q]);
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                r.v[k].x = fmaf(decay, r.v[k].x, s.v[k].x);
+                r.v[k].y = fmaf(decay, r.v[k].y, s.v[k].y);
+                r.v[k].z = fmaf(decay, r.v[k].z, s.v[k].z);
+                r.v[k].w = fmaf(decay, r.v[k].w, s.v[k].w);
+            }
+        }
+    }
+}
+
+// What is left of a state pass where the readers make the states: the state (BWD: the gradient) handed on, the boundary state, and
+// (BWD) the partial sums of <Gout, H_in>.  1024 elements per CTA, kReaderChunks chunks at most, all loads in flight.
+template <bool BWD> __device__ __forceinline__ void pass_along(const SegParams &p, const StatePass &a, float *red, int id) {
+    const int PN = p.P * p.N, nblk = PN / 1024, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int blk = id % nblk, h = (id / nblk) % p.H, b = id / (nblk * p.H), e = blk * 1024 + tid * 4;
+    const size_t he = (size_t)h * PN + e;
+    const float *csl = p.cs + vec_off(p, b, h, 0) + (p.Q - 1);
+    auto at = [](const float *q) { return *reinterpret_cast<const float4 *>(q); };
+    auto step = [](float4 &c, float decay, const float4 &s) {
+        c.x = fmaf(decay, c.x, s.x);
+        c.y = fmaf(decay, c.y, s.y);
+        c.z = fmaf(decay, c.z, s.z);
+        c.w = fmaf(decay, c.w, s.w);
+    };
+    float4 carry = make_float4(0.f, 0.f, 0.f, 0.f), sv[kReaderChunks];
+    float dec[kReaderChunks];
+    if (p.hinit) carry = at(p.hinit + (size_t)b * p.hinit_bs + he);
+#pragma unroll
+    for (int c = 0; c < kReaderChunks; ++c)
+        if (c < p.nc) {
+            sv[c] = at(p.Hst + slot_off(p, b, c + 1, h) + e);
+            dec[c] = expf(csl[(size_t)c * p.Q]);
+        }
+    if (!BWD && a.boundary) *reinterpret_cast<float4 *>(a.boundary + (size_t)b * a.boundary_bs + he) = carry;
+#pragma unroll
+    for (int c = 0; c < kReaderChunks; ++c)
+        if (c < p.nc) {
+            const float4 in = carry;
+            step(carry, dec[c], sv[c]);
+            if (BWD) sv[c] = in;            // the state entering chunk c
+        }
+    if (!BWD) {
+        if (a.leave) *reinterpret_cast<float4 *>(a.leave + (size_t)b * a.leave_bs + he) = carry;
+        if (a.fin) *reinterpret_cast<float4 *>(a.fin + (size_t)b * p.H * PN + he) = carry;
+        return;
+    }
+    carry = p.ginit ? at(p.ginit + (size_t)b * p.ginit_bs + he) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int c = kReaderChunks - 1; c >= 0; --c)
+        if (c < p.nc) {
+            const float4 ev = at(p.Gst + slot_off(p, b, c, h) + e);
+            float part = carry.x * sv[c].x;
+            part = fmaf(carry.y, sv[c].y, part);
+            part = fmaf(carry.z, sv[c].z, part);
+            part = fmaf(carry.w, sv[c].w, part);
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) part += __shfl_xor_sync(0xffffffffu, part, off);
+            if (lane == 0) red[c * 8 + warp] = dec[c] * part;
+            step(carry, dec[c], ev);
+        }
+    *reinterpret_cast<float4 *>(a.leave + (size_t)b * a.leave_bs + he) = carry;
+    __syncthreads();
+    if (tid < 2 * p.nc) {                   // two partial sums of 512 elements, as the pass has them
+        const float *r = red + (tid >> 1) * 8 + (tid & 1) * 4;
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 4; ++w) s += r[w];
+        p.ghdot[((((size_t)b * p.H + h) * p.ncs + (tid >> 1)) << 4) + blk * 2 + (tid & 1)] = s;
+    }
+}
+
 // One 64-row tile of y (DX = false) or of dx (DX = true) of one head:
 //   y_t  = sum_{s<=t} CB[t,s] e^{cs_t-cs_s} dt_s x_s + e^{cs_t} C_t H_in + D x_t
 //   u_s  = sum_{t>=s} CB[t,s] e^{cs_t-cs_s} dy_t     + e^{cs_last-cs_s} B_s Gout ;  dx_s = D dy_s + dt_s u_s ,
 //   ddt_direct_s = x_s . u_s , psi2_s = dt_s e^{cs_last-cs_s} x_s . (Gout B_s) , dD partial = sum dy.x
 // CB false (y only): the tiles of C B^T are not in the scratch and are made here, per head, with the same operations in the same
 // order, so with the same bits.
-template <typename T, int NS, bool DX, bool CB>
+template <typename T, int NS, bool DX, bool CB, bool READER>
 __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &sm, int c, int rt, int h, int b) {
     constexpr int PT = SimtSmem<T>::PT;
     float *css = sm.css, *dts = sm.dts, *fac = sm.fac, *facd = sm.red[5];
@@ -367,13 +463,13 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
     const size_t xo = (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64;
     const T *vals = (const T *)(DX ? p.dy : p.x) + xo;
     const T *rowv = (const T *)(DX ? p.Bm : p.Cm) + (size_t)b * p.bc_bs + (tok0 + r0) * GN + (size_t)g * NS;
-    const float *St = DX ? p.Gst + slot_off(p, b, c + 1, h) : p.Hst + slot_off(p, b, c, h), *cbt = cb_of(p, b, c, g);
+    const float *cbt = cb_of(p, b, c, g);
     TileRegs<T> rv;
     TileRegs<float> rf;
     Acc acc;
     acc.zero();
     tile_load(rv, rowv, GN);
-    tile_load<true>(rf, St, NS);
+    load_state<NS, DX, READER>(rf, p, b, h, c, 0);
     for (int t = tid; t < Q; t += 256) {
         css[t] = p.cs[vec_off(p, b, h, c) + t];
         dts[t] = p.dtT[vec_off(p, b, h, c) + t];
@@ -390,7 +486,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
         __syncthreads();
         if (k0 + 64 < NS) {
             tile_load(rv, rowv + k0 + 64, GN);
-            tile_load<true>(rf, St + k0 + 64, NS);
+            load_state<NS, DX, READER>(rf, p, b, h, c, k0 + 64);
         } else if (CB) {
             load_vals(ct0);
         }
@@ -530,9 +626,10 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
 }
 
 // y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
-// wait for nothing of this one, and a launch of a few microseconds is saved per segment.
-template <typename T, int NS, bool CB>
-__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, SegParams nx, int n_next) {
+// wait for nothing of this one, and a launch of a few microseconds is saved per segment.  READER: no state pass has run; n_pass
+// CTAs make what it hands on.
+template <typename T, int NS, bool CB, bool READER>
+__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, SegParams nx, int n_next, StatePass pass, int n_pass) {
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();
@@ -543,8 +640,12 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, 
         simt_sums<T, NS>(nx, sm, id - ny, false);
         return;
     }
+    if (READER && id >= ny - n_pass) {
+        pass_along<false>(p, pass, sm.red[0], id - (ny - n_pass));
+        return;
+    }
     const int rt = id % nrt, c = (id / nrt) % p.nc, h = (id / (nrt * p.nc)) % p.H, b = id / (nrt * p.nc * p.H);
-    simt_row_tile<T, NS, false, CB>(p, sm, c, rt, h, b);
+    simt_row_tile<T, NS, false, CB, READER>(p, sm, c, rt, h, b);
 }
 
 // The large kernel of the backward: tiles of dx, and the partial slices of dB and dC.  Per (chunk, head range):
@@ -553,8 +654,8 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, 
 //   inter dC, tile tt : sum_h e^{cs_t} dy_t H_in (and rho2 per head);  inter dB, tile ts : sum_h dt_s e^{cs_last-cs_s} x_s Gout
 // A row of tile r has dC slots for ts <= r and dB slots for tt >= r, so the two share Q/64 + 3 slots per head range: dC by ts, dB by
 // tt + 1, then the inter-chunk terms of both.
-template <typename T, int NS>
-__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p, int n_dx) {
+template <typename T, int NS, bool READER>
+__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p, int n_dx, StatePass pass, int n_pass) {
     constexpr int PT = SimtSmem<T>::PT;
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
@@ -562,10 +663,15 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
     pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, Q = p.Q, nrt = Q >> 6, npair = nrt * (nrt + 1) / 2;
     int id = blockIdx.x;
-    if (id >= (int)gridDim.x - n_dx) {
-        id -= (int)gridDim.x - n_dx;
+    const int n_bc = (int)gridDim.x - n_dx - n_pass;
+    if (READER && id >= n_bc + n_dx) {
+        pass_along<true>(p, pass, sm.red[0], id - n_bc - n_dx);
+        return;
+    }
+    if (id >= n_bc) {
+        id -= n_bc;
         const int rt = id % nrt, h = (id / nrt) % p.H, c = (id / (nrt * p.H)) % p.nc, b = id / (nrt * p.H * p.nc);
-        simt_row_tile<T, NS, true, true>(p, sm, c, rt, h, b);
+        simt_row_tile<T, NS, true, true, READER>(p, sm, c, rt, h, b);
         return;
     }
     const int per = npair + 2 * nrt, role = id % per;
@@ -710,10 +816,13 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
     for (int m = 0; m < NS / 64; ++m)
 #pragma unroll
         for (int j = 0; j < 4; ++j) tot[m][0][j] = tot[m][1][j] = make_float2(0.f, 0.f);
-    auto state = [&](int h) { return isC ? p.Hst + slot_off(p, b, c, h) : p.Gst + slot_off(p, b, c + 1, h); };
+    auto state = [&](int h, int k0) {
+        if (isC) load_state<NS, false, READER>(rf, p, b, h, c, k0);
+        else load_state<NS, true, READER>(rf, p, b, h, c, k0);
+    };
     const T *rows = (isC ? dyb : xb) + (size_t)rt * 64 * HP;
     tile_load(ra, rows + (size_t)h0 * 64, HP);
-    tile_load<true>(rf, state(h0), NS);
+    state(h0, 0);
     for (int h = h0; h < h1; ++h) {
         const size_t vo = vec_off(p, b, h, c);
         const float cl = p.cs[vo + Q - 1];
@@ -729,10 +838,10 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
             tile_store(sm.t + PT, rf);
             __syncthreads();
             if (m + 1 < NS / 64) {
-                tile_load<true>(rf, state(h) + 64 * (m + 1), NS);
+                state(h, 64 * (m + 1));
             } else if (h + 1 < h1) {
                 tile_load(ra, rows + (size_t)(h + 1) * 64, HP);
-                tile_load<true>(rf, state(h + 1), NS);
+                state(h + 1, 0);
             }
             acc.zero();
             tile_mma<PT, 3, false, true>(acc, sm.t, sm.t + PT);
@@ -951,8 +1060,9 @@ template <auto K, typename T, typename... Args> static cudaError_t simt_start(in
     return launch_pdl(K, dim3(ctas), dim3(256), sizeof(SimtSmem<T>), st, args...);
 }
 template <typename T, int NS>
-static cudaError_t simt_launch(const SegParams &p, const SegParams *next, int what, cudaStream_t st) {
-    const int nrt = p.Q / 64, npair = nrt * (nrt + 1) / 2;
+static cudaError_t simt_launch(const SegParams &p, const SegParams *next, const StatePass *pass, int what, cudaStream_t st) {
+    const int nrt = p.Q / 64, npair = nrt * (nrt + 1) / 2, n_pass = pass ? p.P * p.N / 1024 * p.H * p.B : 0;
+    const StatePass none = {};
     switch (what) {
         case SIMT_SUMS:
         case SIMT_SUMS_GRAD: {
@@ -960,9 +1070,10 @@ static cudaError_t simt_launch(const SegParams &p, const SegParams *next, int wh
             return simt_start<k_simt_sums<T, NS>, T>(simt_n_sums<T, NS>(p, grads), st, p, grads);
         }
         case SIMT_Y: {
-            const int n_next = next ? simt_n_sums<T, NS>(*next, false) : 0, n = p.nc * nrt * p.H * p.B + n_next;
-            if (!p.cbt) return simt_start<k_simt_y<T, NS, false>, T>(n, st, p, p, 0);      // never with `next`
-            return simt_start<k_simt_y<T, NS, true>, T>(n, st, p, next ? *next : p, n_next);
+            const int n_next = next ? simt_n_sums<T, NS>(*next, false) : 0, n = p.nc * nrt * p.H * p.B + n_next + n_pass;
+            if (!p.cbt) return simt_start<k_simt_y<T, NS, false, false>, T>(n, st, p, p, 0, none, 0);      // never with `next` or `pass`
+            if (pass) return simt_start<k_simt_y<T, NS, true, true>, T>(n, st, p, next ? *next : p, n_next, *pass, n_pass);
+            return simt_start<k_simt_y<T, NS, true, false>, T>(n, st, p, next ? *next : p, n_next, none, 0);
         }
         case SIMT_TAIL: {
             const int nfin = tail_finish_ctas(p), n_next = simt_n_sums<T, NS>(*next, true);
@@ -970,13 +1081,14 @@ static cudaError_t simt_launch(const SegParams &p, const SegParams *next, int wh
         }
         default: {
             const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 3)) * p.G * p.B;
-            return simt_start<k_simt_bwd<T, NS>, T>(n_bc + n_dx, st, p, n_dx);
+            if (pass) return simt_start<k_simt_bwd<T, NS, true>, T>(n_bc + n_dx + n_pass, st, p, n_dx, *pass, n_pass);
+            return simt_start<k_simt_bwd<T, NS, false>, T>(n_bc + n_dx, st, p, n_dx, none, 0);
         }
     }
 }
-cudaError_t launch_simt(const SegParams &p, const SegParams *next, int dtype, int what, cudaStream_t st) {
-    if (dtype == SSD_DTYPE_F32) return p.N == 64 ? simt_launch<float, 64>(p, next, what, st) : simt_launch<float, 128>(p, next, what, st);
-    return p.N == 64 ? simt_launch<__nv_bfloat16, 64>(p, next, what, st) : simt_launch<__nv_bfloat16, 128>(p, next, what, st);
+cudaError_t launch_simt(const SegParams &p, const SegParams *next, const StatePass *pass, int dtype, int what, cudaStream_t st) {
+    if (dtype == SSD_DTYPE_F32) return p.N == 64 ? simt_launch<float, 64>(p, next, pass, what, st) : simt_launch<float, 128>(p, next, pass, what, st);
+    return p.N == 64 ? simt_launch<__nv_bfloat16, 64>(p, next, pass, what, st) : simt_launch<__nv_bfloat16, 128>(p, next, pass, what, st);
 }
 
 // ------------------------------------------------------------------ dA, dD over (batch, chunks)
