@@ -425,7 +425,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     SegParams sp;
     fill_params(pl, lo, ws, sp);
     sp.x = x; sp.dt = dt; sp.A = A; sp.Bm = Bm; sp.Cm = Cm; sp.D = D; sp.y = y;
-    SSD_TRY(cudaMemsetAsync(sp.status, 0, 256, st));
+    sp.first = 1;       // the status word is cleared by the first launch
     TcMaps maps;
     if (pl.use_tc && !tc_make_maps(sp, maps)) return SSD_ECUDA;
     const long long PN = (long long)pl.P * pl.N;
@@ -445,6 +445,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
         for (int k = 0; k < pl.nseg; ++k) {
             const int cp = k % ncp;
             set_segment(pl, k, sp);
+            sp.first = k == 0;
             select_copy(lo, ws, cp, 0, sp);
             if (k >= ncp) SSD_TRY(cudaStreamWaitEvent(chain, side->big_done[cp], 0));   // y of segment k - ncp has read this copy
             {
@@ -477,6 +478,7 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     SegParams next;
     for (int k = 0; k < pl.nseg; ++k) {
         set_segment(pl, k, sp);
+        sp.first = k == 0;
         const float *init = (k == 0) ? h0 : sp.hcarry;
         float *bnd = boundary ? boundary + (size_t)k * pl.H * PN : nullptr, *fin = (k == pl.nseg - 1) ? h_final : nullptr;
         if (pl.use_tc) {
@@ -631,7 +633,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
     sp.x = x; sp.dt = dt; sp.A = A; sp.Bm = Bm; sp.Cm = Cm; sp.D = D; sp.dy = dy;
     sp.dx = dx; sp.ddt = ddt; sp.dB = dB; sp.dC = dC;
     sp.dx_skip = (shape->flags & SSD_FLAG_SKIP_GRAD) ? 1.f : 0.f;
-    SSD_TRY(cudaMemsetAsync(sp.status, 0, 256, st));
+    sp.first = 1;       // the status word is cleared by the first launch
     TcMaps maps;
     if (pl.use_tc && !tc_make_maps(sp, maps)) return SSD_ECUDA;
     const long long PN = (long long)pl.P * pl.N;
@@ -663,6 +665,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         for (int k = pl.nseg - 1; k >= 0; --k) {
             const int i = pl.nseg - 1 - k, par = i % npar, cp = i % ncp;
             set_segment(pl, k, sp);
+            sp.first = i == 0;
             select_copy(lo, ws, cp, par, sp);
             TcMaps mk = cmaps[cp];
             mk.G = gmaps[par].G;
@@ -720,6 +723,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         sp.chain_heads = chain_heads(pl, false);
         for (int k = pl.nseg - 1; k >= 0; --k) {
             set_segment(pl, k, sp);
+            sp.first = k == pl.nseg - 1;
             // Recompute_Forward: chunk-entry states of segment k from the stored boundary state; then backward through the
             // segment: dh enters from the right, leaves to the left
             const float *hin = boundary + (size_t)k * pl.H * PN, *ginit = (k == pl.nseg - 1) ? dh_final : sp.gcarry;

@@ -21,7 +21,7 @@ namespace ssd {
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 template <typename... KArgs, typename... Args>
-inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+inline cudaError_t launch_as(bool dependent, void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
     cfg.blockDim = block;
@@ -31,8 +31,12 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = dependent ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kernel, KArgs(args)...);
+}
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+    return launch_as(true, kernel, grid, block, smem, st, args...);
 }
 // Lets kernel K use `bytes` of dynamic shared memory; the attribute is set once per device.
 template <auto K> inline cudaError_t allow_smem(int bytes) {
@@ -85,6 +89,8 @@ struct SegParams {
     int chain_heads; // heads per CTA of the forward chain, 1 or 2 (no effect on results)
     int ngh;       // partial sums of <G,H> per (head, chunk) (<= 16)
     int tiles;     // split path: 64-step tiles per chunk (rho, psi and the slices come per tile); tensor-core path: 0
+    int first;        // the call's first launch: an ordinary one, so that nothing of the call starts before what is older than it has ended;
+                   // it clears the status word (as a launch of its own: 2 us a call)
     float dx_skip;    // 1 when dx also takes dy (a skip connection around the layer), else 0
     int64_t x_bs, dt_bs, bc_bs;  // batch strides, elements
 

@@ -1,3 +1,6 @@
+// Every role of the split path's large kernels loads its first tiles of the caller's tensors before it waits for the launch before it:
+// they are older than the call (its first launch is an ordinary one).
+//
 // The split path: the kernels of fp32 calls (1e-4 parity rules out operands rounded to 16 bits or TF32), of bf16 calls whose
 // intermediates stay in fp32, and a cross-check of the tensor-core kernels.  fp32 operands go to the tensor cores as three bf16
 // parts (ssd_split.cuh).  Also here: inter-chunk state passing of that path, and the backward's finishing scans and reductions of
@@ -263,6 +266,7 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
             tile_load(ra, C + k0, GN);
             tile_load(rb, Bp + k0, GN);
             if (k0) __syncthreads();
+            else pdl_wait();
             tile_store(sm.t, ra);
             tile_store(sm.t + PT, rb);
             __syncthreads();
@@ -290,6 +294,7 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
 #pragma unroll
         for (int k = 0; k < 8; ++k)
             if (k < per) d[k] = __ldg(p.dt + (size_t)b * p.dt_bs + (tok0 + tid * per + k) * p.H + h);
+        pdl_wait();
 #pragma unroll
         for (int k = 0; k < 8; ++k)
             if (k < per) {
@@ -317,6 +322,8 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
                     p.dtT[vec_off(p, b, h, c) + t] = d[k];
                 }
             }
+    } else {
+        pdl_wait();
     }
     __syncthreads();
     const int end = merged ? 2 * Q : Q;
@@ -348,7 +355,7 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
 template <typename T, int NS> __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_sums(SegParams p, bool grads) {
     extern __shared__ __align__(16) unsigned char smem[];
     pdl_launch_dependents();
-    pdl_wait();
+    if (p.first && blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
     simt_sums<T, NS>(p, *reinterpret_cast<SimtSmem<T> *>(smem), blockIdx.x, grads);
 }
 
@@ -469,6 +476,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
     Acc acc;
     acc.zero();
     tile_load(rv, rowv, GN);
+    pdl_wait();
     load_state<NS, DX, READER>(rf, p, b, h, c, 0);
     for (int t = tid; t < Q; t += 256) {
         css[t] = p.cs[vec_off(p, b, h, c) + t];
@@ -633,7 +641,6 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, 
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();
-    pdl_wait();
     const int nrt = p.Q >> 6, ny = (int)gridDim.x - n_next;
     int id = blockIdx.x;
     if (id >= ny) {
@@ -641,6 +648,7 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, 
         return;
     }
     if (READER && id >= ny - n_pass) {
+        pdl_wait();
         pass_along<false>(p, pass, sm.red[0], id - (ny - n_pass));
         return;
     }
@@ -660,11 +668,11 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();
-    pdl_wait();
     const int tid = threadIdx.x, lane = tid & 31, Q = p.Q, nrt = Q >> 6, npair = nrt * (nrt + 1) / 2;
     int id = blockIdx.x;
     const int n_bc = (int)gridDim.x - n_dx - n_pass;
     if (READER && id >= n_bc + n_dx) {
+        pdl_wait();
         pass_along<true>(p, pass, sm.red[0], id - n_bc - n_dx);
         return;
     }
@@ -692,6 +700,12 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
         pair_of(role, tt, ts);
         TileRegs<T> ra, rb;
         float2 cb[2][4], ws[2][4];
+        auto load_rows = [&](int h) {
+            tile_load(ra, dyb + (size_t)tt * 64 * HP + (size_t)h * 64, HP);
+            tile_load(rb, xb + (size_t)ts * 64 * HP + (size_t)h * 64, HP);
+        };
+        load_rows(h0);
+        pdl_wait();
 #pragma unroll
         for (int half = 0; half < 2; ++half)
 #pragma unroll
@@ -704,9 +718,7 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
         float *rowv = sm.fac, *colv = sm.fac + 64;
         const bool diag = tt == ts;
         float va = 0.f, vb = 0.f, vref, vlast;
-        auto load_head = [&](int h) {
-            tile_load(ra, dyb + (size_t)tt * 64 * HP + (size_t)h * 64, HP);
-            tile_load(rb, xb + (size_t)ts * 64 * HP + (size_t)h * 64, HP);
+        auto load_vec = [&](int h) {
             const size_t vo = vec_off(p, b, h, c);
             if (tid < 128) {
                 const size_t o = vo + (tid < 64 ? tt : ts) * 64 + (tid & 63);
@@ -716,7 +728,7 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
             vref = p.cs[vo + tt * 64];
             vlast = p.cs[vo + tt * 64 + 63];
         };
-        load_head(h0);
+        load_vec(h0);
         for (int h = h0; h < h1; ++h) {
             tile_store(sm.t, ra);
             tile_store(sm.t + PT, rb);
@@ -726,7 +738,10 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
                 sm.fac[tid] = factors ? (tid < 64 ? e : e * vb) : (tid < 64 ? va : vb);
             }
             __syncthreads();
-            if (h + 1 < h1) load_head(h + 1);
+            if (h + 1 < h1) {
+                load_rows(h + 1);
+                load_vec(h + 1);
+            }
             acc.zero();
             tile_mma<PT, PT, false, false>(acc, sm.t, sm.t + PT);
             float2 row[2], col[4];
@@ -822,6 +837,7 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
     };
     const T *rows = (isC ? dyb : xb) + (size_t)rt * 64 * HP;
     tile_load(ra, rows + (size_t)h0 * 64, HP);
+    pdl_wait();
     state(h0, 0);
     for (int h = h0; h < h1; ++h) {
         const size_t vo = vec_off(p, b, h, c);
@@ -1037,10 +1053,13 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_tail(SegParams 
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
     pdl_launch_dependents();
-    pdl_wait();
     const int id = (int)blockIdx.x - n_next;
-    if (id < 0) simt_sums<T, NS>(nx, sm, blockIdx.x, true);
-    else if (id < nfin) bwd_finish<false>(p, reinterpret_cast<float *>(sm.t), id);
+    if (id < 0) {
+        simt_sums<T, NS>(nx, sm, blockIdx.x, true);
+        return;
+    }
+    pdl_wait();
+    if (id < nfin) bwd_finish<false>(p, reinterpret_cast<float *>(sm.t), id);
     else reduce_dbdc<T, false>(p, id - nfin);
 }
 
@@ -1054,10 +1073,10 @@ cudaError_t launch_bwd_tail(const SegParams &p, int dtype, cudaStream_t st) {
     return launch_pdl(k_bwd_tail<__nv_bfloat16, true>, grid, dim3(256), 0, st, p, nfin);
 }
 
-template <auto K, typename T, typename... Args> static cudaError_t simt_start(int ctas, cudaStream_t st, Args &&...args) {
+template <auto K, typename T, typename... Args> static cudaError_t simt_start(bool first, int ctas, cudaStream_t st, const SegParams &p, Args &&...args) {
     const cudaError_t e = allow_smem<K>((int)sizeof(SimtSmem<T>));
     if (e != cudaSuccess) return e;
-    return launch_pdl(K, dim3(ctas), dim3(256), sizeof(SimtSmem<T>), st, args...);
+    return launch_as(!first, K, dim3(ctas), dim3(256), sizeof(SimtSmem<T>), st, p, args...);
 }
 template <typename T, int NS>
 static cudaError_t simt_launch(const SegParams &p, const SegParams *next, const StatePass *pass, int what, cudaStream_t st) {
@@ -1067,22 +1086,22 @@ static cudaError_t simt_launch(const SegParams &p, const SegParams *next, const 
         case SIMT_SUMS:
         case SIMT_SUMS_GRAD: {
             const bool grads = what == SIMT_SUMS_GRAD;
-            return simt_start<k_simt_sums<T, NS>, T>(simt_n_sums<T, NS>(p, grads), st, p, grads);
+            return simt_start<k_simt_sums<T, NS>, T>(p.first, simt_n_sums<T, NS>(p, grads), st, p, grads);
         }
         case SIMT_Y: {
             const int n_next = next ? simt_n_sums<T, NS>(*next, false) : 0, n = p.nc * nrt * p.H * p.B + n_next + n_pass;
-            if (!p.cbt) return simt_start<k_simt_y<T, NS, false, false>, T>(n, st, p, p, 0, none, 0);      // never with `next` or `pass`
-            if (pass) return simt_start<k_simt_y<T, NS, true, true>, T>(n, st, p, next ? *next : p, n_next, *pass, n_pass);
-            return simt_start<k_simt_y<T, NS, true, false>, T>(n, st, p, next ? *next : p, n_next, none, 0);
+            if (!p.cbt) return simt_start<k_simt_y<T, NS, false, false>, T>(false, n, st, p, p, 0, none, 0);      // never with `next` or `pass`
+            if (pass) return simt_start<k_simt_y<T, NS, true, true>, T>(false, n, st, p, next ? *next : p, n_next, *pass, n_pass);
+            return simt_start<k_simt_y<T, NS, true, false>, T>(false, n, st, p, next ? *next : p, n_next, none, 0);
         }
         case SIMT_TAIL: {
             const int nfin = tail_finish_ctas(p), n_next = simt_n_sums<T, NS>(*next, true);
-            return simt_start<k_simt_tail<T, NS>, T>(n_next + nfin + tail_reduce_ctas(p), st, p, *next, n_next, nfin);
+            return simt_start<k_simt_tail<T, NS>, T>(false, n_next + nfin + tail_reduce_ctas(p), st, p, *next, n_next, nfin);
         }
         default: {
             const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 3)) * p.G * p.B;
-            if (pass) return simt_start<k_simt_bwd<T, NS, true>, T>(n_bc + n_dx + n_pass, st, p, n_dx, *pass, n_pass);
-            return simt_start<k_simt_bwd<T, NS, false>, T>(n_bc + n_dx, st, p, n_dx, none, 0);
+            if (pass) return simt_start<k_simt_bwd<T, NS, true>, T>(false, n_bc + n_dx + n_pass, st, p, n_dx, *pass, n_pass);
+            return simt_start<k_simt_bwd<T, NS, false>, T>(false, n_bc + n_dx, st, p, n_dx, none, 0);
         }
     }
 }

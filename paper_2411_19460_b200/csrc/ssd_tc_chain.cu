@@ -96,6 +96,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
 
     const int h0 = blockIdx.x * HEADS, b = blockIdx.y, g = h0 / p.hpg, nc = p.nc;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    if (!BWD && p.first && blockIdx.x == 0 && b == 0 && tid < 64) p.status[tid] = 0u;
     auto chunk_of = [&](int i) { return BWD ? nc - 1 - i : i; };
     if (tid == 0) {
         for (int i = 0; i < CH_STAGES; ++i) {
@@ -120,7 +121,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     __syncthreads();
     tc_fence_after_sync();
     // What the kernel before this one in the stream may still write, or still read where this one writes, is waited for in the
-    // roles that touch it; x, dt, B, C and dy are older than that kernel, so the first blocks are loaded and scaled under its end.
+    // roles that touch it; x, dt, B, C and dy are older than the call, whose first launch is an ordinary one, so the first blocks are loaded and scaled under its end.
     const uint32_t tm = words[0];
     volatile uint32_t *abortp = &words[1];
 
@@ -467,7 +468,7 @@ static cudaError_t launch_chain(const SegParams &p, const TcMaps &m, const float
     const cudaError_t e = allow_smem<k_chain_tc<MODE, HEADS>>((int)smem);
     if (e != cudaSuccess) return e;
     const bool bwd = MODE == CHAIN_BWD;
-    return launch_pdl(k_chain_tc<MODE, HEADS>, dim3(p.H / HEADS, p.B), dim3(ch_threads(MODE, HEADS)), (size_t)smem, st, p, init, init_bs, bnd_out,
+    return launch_as(bwd || !p.first, k_chain_tc<MODE, HEADS>, dim3(p.H / HEADS, p.B), dim3(ch_threads(MODE, HEADS)), (size_t)smem, st, p, init, init_bs, bnd_out,
                       bnd_bs, carry_out, final_out, bwd ? m.dy : m.x, bwd ? m.Cm : m.Bm, m.H, bwd ? m.Gst : m.Hst);
 }
 
