@@ -83,7 +83,6 @@ __global__ void __launch_bounds__(CV_RING_THREADS) k_conv_fwd(const T *u, long l
     __shared__ unsigned int status_dummy;
     T *ring = reinterpret_cast<T *>(cv_smem);                     // [stage][CV_STG_TOK][512]
     pdl_launch_dependents();
-    pdl_wait();       // the previous kernel of the stream (a neighbouring segment's) has finished
     const int cbase = blockIdx.x * 512, nch = min(512, C - cbase);
     const int b = blockIdx.z;
     const int r_begin = blockIdx.y * RL, ntok = min(RL, L - r_begin), nst = (ntok + CV_STG_TOK - 1) / CV_STG_TOK;
@@ -100,6 +99,7 @@ __global__ void __launch_bounds__(CV_RING_THREADS) k_conv_fwd(const T *u, long l
         fence_barrier_init();
     }
     __syncthreads();
+    pdl_wait();       // the previous kernel of the stream (a neighbouring segment's) has finished
     if (warp == CV_THREADS / 32) {
         if (elect_one()) {
             const uint32_t row_bytes = (uint32_t)nch * sizeof(T);
@@ -202,7 +202,6 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
     __shared__ unsigned int status_dummy;
     T *ring = reinterpret_cast<T *>(cv_smem);                     // [stage][u rows | dout rows][512]
     pdl_launch_dependents();
-    pdl_wait();
     const int cbase = blockIdx.x * 512, nch = min(512, C - cbase);
     const int b = blockIdx.z;
     const long long r_begin = (long long)blockIdx.y * RL, r_end = min(r_begin + (long long)RL, (long long)L);
@@ -221,15 +220,18 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
         fence_barrier_init();
     }
     __syncthreads();
+    pdl_wait();
+    // the tokens behind the range, which complete its last du's, are a stage of their own
+    const int nbehind = (int)min(3ll, (long long)L - r_end);
     if (warp == CV_THREADS / 32) {
         // ---- producer
         if (elect_one()) {
             const uint32_t row_bytes = (uint32_t)nch * sizeof(T);
-            for (int i = 0; i < nst; ++i) {
+            for (int i = 0; i < nst + (nbehind > 0 ? 1 : 0); ++i) {
                 const int slot = i % CV_STAGES;
                 if (i >= CV_STAGES) mbar_wait(&empty[slot], ((i / CV_STAGES) - 1) & 1, &abort_flag, &status_dummy);
-                const long long t0 = r_begin + (long long)i * CV_STG_TOK;
-                const int n = (int)min((long long)CV_STG_TOK, r_end - t0);
+                const long long t0 = i < nst ? r_begin + (long long)i * CV_STG_TOK : r_end;
+                const int n = i < nst ? (int)min((long long)CV_STG_TOK, r_end - t0) : nbehind;
                 mbar_arrive_expect_tx(&full[slot], 2u * (uint32_t)n * row_bytes);
                 T *su = ring + (size_t)slot * (2 * CV_STG_TOK * 512), *sg = su + CV_STG_TOK * 512;
                 for (int j = 0; j < n; ++j) {
@@ -379,16 +381,19 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
         if (lane == 0) mbar_arrive(&empty[slot]);      // this warp has read the stage
     }
     if (!active) return;
-    // the three tokens behind the range complete its last du's (plain loads: 16 bytes per thread and token)
+    // the three tokens behind the range complete its last du's
+    const int last = nst % CV_STAGES;
+    if (nbehind > 0) mbar_wait(&full[last], (nst / CV_STAGES) & 1, &abort_flag, &status_dummy);
+    const T *spu = ring + (size_t)last * (2 * CV_STG_TOK * 512) + threadIdx.x * CV_CH, *spg = spu + CV_STG_TOK * 512;
+#pragma unroll 1
     for (int k = 0; k < 3; ++k) {
-        const long long s = r_end + k;
         float2 g[NP] = {zero2, zero2};
-        const bool formed = s < (long long)L;
+        const bool formed = k < nbehind;
         if (formed) {
-            ld2x2(ub + (size_t)s * C + c0, x3[0], x3[1]);
-            ld2x2(gb + (size_t)s * C + c0, g[0], g[1]);
+            ld2x2(spu + (size_t)k * 512, x3[0], x3[1]);
+            ld2x2(spg + (size_t)k * 512, g[0], g[1]);
         }
-        token(s, g, false, formed, false);
+        token(r_end + k, g, false, formed, false);
     }
     // partial weight / bias gradients of this range: part[b][range][5][C]
     {
