@@ -10,7 +10,7 @@
 // up to 1 KB), so that many kilobytes per SM are in flight without holding registers, and results go straight to
 // global memory (8 or 16 bytes per thread, coalesced over the channels).  A CTA walks a range of tokens, streamed through a ring
 // of 8-token stages.
-// Weight and bias gradients: one partial per backward CTA, then a fixed-order sum (no atomics).
+// Weight and bias gradients: partials of 64 tokens (short ranges: of a backward CTA), then a fixed-order sum (no atomics).
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
 
@@ -187,15 +187,19 @@ __global__ void __launch_bounds__(CV_RING_THREADS) k_conv_fwd(const T *u, long l
 // tokens behind it (for its own last du's; past the end of the segment they are not formed: their effect arrives
 // as `dtail`).  The rows of u and dout stream through a ring of 8-token stages filled by a producer warp with one
 // bulk copy per row, so the loads of later stages are in flight while a stage is being consumed.
-// dw, dbias: one partial per range, the range's own tokens.
-// 4096 tokens of 5376 channels: 43 us where the bytes take 20; issue 42 %, FMA 36 %, MUFU 28 %, DRAM 30 %, so neither arithmetic nor
-// memory but latency: a CTA lives for ten stages and starts and ends with loads that nothing covers.
-constexpr int CV_STAGES = 3;
+// dw, dbias: partials of the range's own tokens.
+// Neither arithmetic nor memory bounds a call of 4096 tokens (5376 channels: 20 us of bytes; issue 42 %, FMA 36 %, MUFU 28 %, DRAM 30 % with
+// ranges of ten stages) but the start and end of a range, which loads cover only in part.
+// Long ranges (64 tokens and more) take three CTAs per SM with four stages in place of four with three: the longer range covers its start
+// and end better (eight segments of 4096 tokens, forward + backward: 515 -> 490 us, of which the
+// sums after 64 tokens cost 14; five CTAs with two stages 762, two waves of shorter
+// ranges 520).  The fp32 sums of dw and dbias end after 64 tokens, whatever the range.
+constexpr int CV_SUM_STAGES = 8, CV_LONG = CV_SUM_STAGES * CV_STG_TOK;
 
-template <typename T>
-__global__ void __launch_bounds__(CV_RING_THREADS, 4)
+template <typename T, int CV_STAGES, int CTAS>
+__global__ void __launch_bounds__(CV_RING_THREADS, CTAS)
 k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const T *state_in, const T *dout,
-           const float *dtail, T *du, float *dstate, float *part, int L, int C, int RL) {
+           const float *dtail, T *du, float *dstate, float *part, int L, int C, int RL, int parts) {
     extern __shared__ __align__(128) unsigned char cv_smem[];
     __shared__ uint64_t full[CV_STAGES], empty[CV_STAGES];
     __shared__ uint32_t abort_flag;
@@ -351,10 +355,26 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
         }
         dup += C;
     };
+    // partial weight / bias gradients, a slot per 64 tokens: part[b][slot][5][C]
+    const int slots = (RL + CV_LONG - 1) / CV_LONG;
+    auto leave_sums = [&](int k64) {
+        float *pp = part + (((size_t)b * parts + (size_t)blockIdx.y * slots + k64) * 5) * C + c0;
+        float col[CV_CH];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+#pragma unroll
+            for (int i = 0; i < NP; ++i) { col[2 * i] = aw[i][k].x; col[2 * i + 1] = aw[i][k].y; aw[i][k] = zero2; }
+            st4(pp + (size_t)k * C, col);
+        }
+#pragma unroll
+        for (int i = 0; i < NP; ++i) { col[2 * i] = ab[i].x; col[2 * i + 1] = ab[i].y; ab[i] = zero2; }
+        st4(pp + (size_t)4 * C, col);
+    };
     for (int i = 0; i < nst; ++i) {
         const int slot = i % CV_STAGES;
         mbar_wait(&full[slot], (i / CV_STAGES) & 1, &abort_flag, &status_dummy);
         if (active) {
+            if (i && i % CV_SUM_STAGES == 0) leave_sums(i / CV_SUM_STAGES - 1);
             const T *spu = ring + (size_t)slot * (2 * CV_STG_TOK * 512) + threadIdx.x * CV_CH, *spg = spu + CV_STG_TOK * 512;
             const long long t0 = r_begin + (long long)i * CV_STG_TOK;
             const int n = (int)min((long long)CV_STG_TOK, r_end - t0);
@@ -395,20 +415,7 @@ k_conv_bwd(const T *u, long long u_bs, const float *w, const float *bias, const 
         }
         token(r_end + k, g, false, formed, false);
     }
-    // partial weight / bias gradients of this range: part[b][range][5][C]
-    {
-        float *pp = part + (((size_t)b * gridDim.y + blockIdx.y) * 5) * C + c0;
-        float col[CV_CH];
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-#pragma unroll
-            for (int i = 0; i < NP; ++i) { col[2 * i] = aw[i][k].x; col[2 * i + 1] = aw[i][k].y; }
-            st4(pp + (size_t)k * C, col);
-        }
-#pragma unroll
-        for (int i = 0; i < NP; ++i) { col[2 * i] = ab[i].x; col[2 * i + 1] = ab[i].y; }
-        st4(pp + (size_t)4 * C, col);
-    }
+    leave_sums((nst - 1) / CV_SUM_STAGES);
 }
 
 // dw[c][k], dbias[c] from the partials of the ranges, in fp64 and in a fixed order: a CTA owns 32 adjacent channels of one of the
@@ -468,15 +475,26 @@ cudaError_t conv_fwd_t(const T *u, long long u_bs, const float *w, const float *
     return launch_pdl(k_conv_fwd<T>, grid, dim3(CV_RING_THREADS), (size_t)smem, st, u, u_bs, w, bias, state_in, out, state_out, L, C, RL);
 }
 
+// `parts`: partial sums per sequence that the launch leaves
 template <typename T>
 cudaError_t conv_bwd_t(const T *u, long long u_bs, const float *w, const float *bias, const T *state_in, const T *dout,
-                       const float *dtail, T *du, float *dstate, float *part, int B, int L, int C, int RL, cudaStream_t st) {
-    const int smem = CV_STAGES * 2 * CV_STG_TOK * 512 * (int)sizeof(T);
-    const cudaError_t e = allow_smem<k_conv_bwd<T>>(smem);
-    if (e != cudaSuccess) return e;
-    dim3 grid((C + 511) / 512, (L + RL - 1) / RL, B);
-    return launch_pdl(k_conv_bwd<T>, grid, dim3(CV_RING_THREADS), (size_t)smem, st, u, u_bs, w, bias, state_in, dout, dtail, du, dstate,
-                      part, L, C, RL);
+                       const float *dtail, T *du, float *dstate, float *part, int B, int L, int C, int &parts, cudaStream_t st) {
+    auto launch = [&](auto kernel, int stages, int RL) {
+        const int ranges = (L + RL - 1) / RL, last = L - (ranges - 1) * RL;
+        parts = (ranges - 1) * ((RL + CV_LONG - 1) / CV_LONG) + (last + CV_LONG - 1) / CV_LONG;      // at most conv_tiles(L)
+        return launch_pdl(kernel, dim3((C + 511) / 512, ranges, B), dim3(CV_RING_THREADS), (size_t)stages * 2 * CV_STG_TOK * 512 * sizeof(T), st, u, u_bs, w,
+                          bias, state_in, dout, dtail, du, dstate, part, L, C, RL, parts);
+    };
+    constexpr int row = 2 * CV_STG_TOK * 512 * (int)sizeof(T);
+    const int RL = conv_range_len(B, L, C, 4, 32);
+    if constexpr (sizeof(T) == 2) {
+        if (RL >= CV_LONG) {
+            const cudaError_t e = allow_smem<k_conv_bwd<T, 4, 3>>(4 * row);
+            return e != cudaSuccess ? e : launch(k_conv_bwd<T, 4, 3>, 4, conv_range_len(B, L, C, 3, 32));
+        }
+    }
+    const cudaError_t e = allow_smem<k_conv_bwd<T, 3, 4>>(3 * row);
+    return e != cudaSuccess ? e : launch(k_conv_bwd<T, 3, 4>, 3, RL);
 }
 
 }  // namespace
@@ -495,17 +513,17 @@ cudaError_t launch_conv_fwd(int dtype, const void *u, long long u_bs, const floa
 cudaError_t launch_conv_bwd(int dtype, const void *u, long long u_bs, const float *w, const float *bias,
                             const void *state_in, const void *dout, const float *dtail, void *du, float *dstate,
                             float *dw, float *dbias, int accumulate, float *part, int B, int L, int C, cudaStream_t st) {
-    const int RL = conv_range_len(B, L, C, 4, 32);      // never more ranges than conv_tiles() promises scratch for
     cudaError_t e;
+    int parts = 0;
     if (dtype == SSD_DTYPE_F32)
         e = conv_bwd_t<float>((const float *)u, u_bs, w, bias, (const float *)state_in, (const float *)dout, dtail, (float *)du,
-                              dstate, part, B, L, C, RL, st);
+                              dstate, part, B, L, C, parts, st);
     else
         e = conv_bwd_t<__nv_bfloat16>((const __nv_bfloat16 *)u, u_bs, w, bias, (const __nv_bfloat16 *)state_in,
-                                      (const __nv_bfloat16 *)dout, dtail, (__nv_bfloat16 *)du, dstate, part, B, L, C, RL, st);
+                                      (const __nv_bfloat16 *)dout, dtail, (__nv_bfloat16 *)du, dstate, part, B, L, C, parts, st);
     if (e != cudaSuccess) return e;
     return launch_pdl(k_conv_reduce, dim3(5 * ((C + 31) / 32)), dim3(CV_RED_WARPS * 32), (size_t)0, st, (const float *)part, dw, dbias, C,
-                      (L + RL - 1) / RL * B, accumulate);
+                      parts * B, accumulate);
 }
 
 }  // namespace ssd
