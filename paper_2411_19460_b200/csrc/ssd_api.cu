@@ -341,6 +341,7 @@ static void select_copy(const Layout &lo, void *ws, int kc, int k, SegParams &sp
 static void fill_params(const Plan &pl, const Layout &lo, void *ws, SegParams &sp) {
     memset(&sp, 0, sizeof(sp));
     sp.B = pl.B; sp.L = pl.L; sp.H = pl.H; sp.P = pl.P; sp.N = pl.N; sp.G = pl.G; sp.Q = pl.Q;
+    sp.inv_H = inverse_of(pl.H);
     sp.hpg = pl.hpg; sp.ncs = pl.ncs; sp.nct = pl.nct; sp.nsl = pl.nsl;
     sp.ndd = pl.use_tc ? 4 : pl.Q / 64;
     sp.scan_ctas = kNumSMs;
@@ -362,6 +363,7 @@ static void set_segment(const Plan &pl, int k, SegParams &sp) {
     sp.t0 = k * pl.seg;
     const int len = (pl.L - sp.t0 < pl.seg) ? pl.L - sp.t0 : pl.seg;
     sp.nc = len / pl.Q;
+    sp.inv_nc = inverse_of(sp.nc);
     sp.c0 = sp.t0 / pl.Q;
 }
 

@@ -81,6 +81,7 @@ struct SegParams {
     int t0;        // first token of the segment
     int nc;        // chunks in this segment
     int c0;        // global index of the segment's first chunk
+    uint32_t inv_nc, inv_H;  // divide_by() of nc and H
     int ncs;       // chunk capacity of the workspace (chunks of a full segment)
     int nct;       // chunks in the whole sequence (L / Q)
     int nsl;       // slices per group in the dB/dC partial buffers: head ranges, or slots of all ranges (split path)
@@ -125,6 +126,15 @@ struct SegParams {
     float *dAp;            // [B,H,nct]     per-chunk partial of dA
     float *dDp;            // [B,H,nct,4]   partials of dD, the first ndd of each group in use
 };
+
+// n / d by a multiplication and one correction, for n below 2^31: kernels that take a tile per CTA divide its number several times
+static inline uint32_t inverse_of(int d) { return d > 1 ? (uint32_t)((1ull << 32) / (unsigned)d) : 0xffffffffu; }
+#ifdef __CUDACC__
+__device__ __forceinline__ int divide_by(int n, int d, uint32_t inv) {
+    const int q = (int)__umulhi((unsigned)n, inv);      // n / d or one less
+    return n - q * d >= d ? q + 1 : q;
+}
+#endif
 
 static inline size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 

@@ -277,7 +277,7 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
     }
     const int n0 = (id % nh) * 64;
     id /= nh;
-    const int h = id % p.H, c = (id / p.H) % p.nc, b = id / (p.H * p.nc), g = h / p.hpg;
+    const int bc = divide_by(id, p.H, p.inv_H), h = id - bc * p.H, b = divide_by(bc, p.nc, p.inv_nc), c = bc - b * p.nc, g = h / p.hpg;
     const size_t tok0 = (size_t)p.t0 + (size_t)c * Q;
     const size_t xo = (size_t)b * p.x_bs + tok0 * HP + (size_t)h * 64, bo = (size_t)b * p.bc_bs + tok0 * GN + (size_t)g * NS + n0;
     float *wsm2 = sm.dts;                                                       // the weights of E
@@ -652,7 +652,8 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, 
         pass_along<false>(p, pass, sm.red[0], id - (ny - n_pass));
         return;
     }
-    const int rt = id % nrt, c = (id / nrt) % p.nc, h = (id / (nrt * p.nc)) % p.H, b = id / (nrt * p.nc * p.H);
+    const int rt = id & (nrt - 1), bhc = id >> (nrt >> 1), bh = divide_by(bhc, p.nc, p.inv_nc), c = bhc - bh * p.nc, b = divide_by(bh, p.H, p.inv_H),
+              h = bh - b * p.H;       // nrt is 1, 2 or 4
     simt_row_tile<T, NS, false, CB, READER>(p, sm, c, rt, h, b);
 }
 
@@ -678,7 +679,8 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p
     }
     if (id >= n_bc) {
         id -= n_bc;
-        const int rt = id % nrt, h = (id / nrt) % p.H, c = (id / (nrt * p.H)) % p.nc, b = id / (nrt * p.H * p.nc);
+        const int rt = id & (nrt - 1), bch = id >> (nrt >> 1), bc = divide_by(bch, p.H, p.inv_H), h = bch - bc * p.H,
+                  b = divide_by(bc, p.nc, p.inv_nc), c = bc - b * p.nc;
         simt_row_tile<T, NS, true, true, READER>(p, sm, c, rt, h, b);
         return;
     }
