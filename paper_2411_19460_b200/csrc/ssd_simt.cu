@@ -159,10 +159,10 @@ cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, long lo
 // cores with fp32 operands as three bf16 parts (ssd_split.cuh): three products where the other operand is bf16 as it stands, six
 // where both are fp32, one where neither is.  Operands are staged as rows, split on the way; the next stage's global loads are in
 // flight while a stage is multiplied.  With FFMA on the CUDA cores (4 x 4 outputs per thread, bound by the shared-memory reads) the
-// large kernel took 309 us (2 x 2048 steps of 32 heads, N = 64, chunk 128, bf16) and 215 us (2 x 1024 of 24, N = 128, fp32), now 120
-// and 143.  Bound by latency: masks, splits and addresses around each product, between barriers, at 24 (fp32: 16) warps per SM (of 550
-// TFLOP/s that mma.sync does here the tensor pipe is 30, 45 % busy).  bf16 takes 80 registers a thread, for three CTAs per SM, with
-// some spills: 2 x 8192 steps 1228 -> 1108 us; fp32, with more parts in registers, takes 128 (at 80: 1112 -> 1260 us).
+// large kernel took 309 us (2 x 2048 steps of 32 heads, N = 64, chunk 128, bf16) and 215 us (2 x 1024 of 24, N = 128, fp32), now 143
+// and 147, y 119 and 92 us, now 49 and 56.  Bound by latency: masks, splits and addresses around each product, between barriers, at 24
+// (fp32: 16) warps per SM (of 550 TFLOP/s that mma.sync does here the tensor pipe is 25 to 45 % busy).  bf16 takes 80 registers a thread, for
+// three CTAs per SM, with some spills; fp32, with more parts in registers, takes 128 (2 x 4096 steps: 1112 us, at 80: 1260).
 //
 // What does not depend on the head is not done per head: C B^T is made once per group (k_simt_sums writes it, 64 x 64 causal
 // tiles), and dB / dC come from a head sum of the masked tiles, one product per CTA instead of two per head.
@@ -663,8 +663,10 @@ __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, 
 //   inter dC, tile tt : sum_h e^{cs_t} dy_t H_in (and rho2 per head);  inter dB, tile ts : sum_h dt_s e^{cs_last-cs_s} x_s Gout
 // A row of tile r has dC slots for ts <= r and dB slots for tt >= r, so the two share Q/64 + 3 slots per head range: dC by ts, dB by
 // tt + 1, then the inter-chunk terms of both.
+// Three CTAs per SM only for bf16 with N = 64 and state passes (2 x 8192 steps of 32 heads: two 0.6 % slower); elsewhere 80 registers spill too
+// much (4096 steps of 24 heads, N = 128, chunks of 64: 612 us at three, 521 at two; N = 64, states made in their readers, 385 and 352).
 template <typename T, int NS, bool READER>
-__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_bwd(SegParams p, int n_dx, StatePass pass, int n_pass) {
+__global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !READER ? 3 : 2) k_simt_bwd(SegParams p, int n_dx, StatePass pass, int n_pass) {
     constexpr int PT = SimtSmem<T>::PT;
     extern __shared__ __align__(16) unsigned char smem[];
     SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
