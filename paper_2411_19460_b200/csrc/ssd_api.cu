@@ -95,14 +95,23 @@ static int bc_head_split(int blocks, int groups, int hpg) {
     return best;
 }
 
-// The same for the kernel of the split path, whose ranges have Q/64 + 3 slots each: ranges of four heads, of two where there are few, so
-// that a short sequence has CTAs enough (8 heads, 256-step chunks, backward: 2048 steps 265 us, with half the ranges 320; 4096
-// steps 353 and 341).  Long ones (64 chunks and more, counted per group) have them anyway, and the slots cost time and memory:
-// there no more of them than two per head, what a slice for each head would take (2 x 8192 steps of 8 heads 999 -> 918 us, 8192 of
-// 80 heads in 8 groups 3976 -> 3373 us and 985 -> 381 MB of scratch).
+// The same for the kernel of the split path, whose ranges have Q/64 + 3 slots each and as many CTAs as the chunk has tile pairs and
+// twice its tiles.  A range costs its CTAs the last products and the slices, some four heads' worth, so ranges of eight heads where
+// 1024 steps (the choice may not depend on the segments) then have 200 CTAs, of four or two below that, of one where two leave next to
+// none.  Backward, us, with ranges of one, two, four, eight heads (CTAs of 1024 steps with eight):
+//   fp32, 2 x 4096 steps of 24 heads, chunk 256 (432)       -  934  813  752       4096 of 24, chunk 256 (216)    -  537  468  444
+//   bf16, 2 x 8192 of 32 heads, chunk 128 (448)             -  842  800  750       4096 of 24, chunk 128, segments of 512 (168)  -  245  238  300
+//   4096 of 8 heads, chunk 256, one segment (72)          230  185  165    -       1024 of 4, chunk 64 (48)      70   78   98    -
+// Long sequences (64 chunks and more, counted per group): no more slots than two per head, what a slice for each head would take (2 x
+// 8192 steps of 8 heads 711 -> 618 us, 8192 of 80 heads in 8 groups 2852 -> 2332 us and 985 -> 381 MB of scratch).
 static int simt_head_ranges(const Plan &pl) {
-    const int per_range = pl.hpg >= 16 ? 4 : 2, slots = pl.Q / 64 + 3;
-    int n = (pl.hpg + per_range - 1) / per_range;
+    const int nrt = pl.Q / 64, slots = nrt + 3, roles = nrt * (nrt + 1) / 2 + 2 * nrt;
+    const int chunks = pl.nct < 1024 / pl.Q ? pl.nct : 1024 / pl.Q;
+    auto ctas = [&](int per) { return (long long)pl.B * chunks * pl.G * roles * ((pl.hpg + per - 1) / per); };
+    int per = 8;
+    while (per > 2 && ctas(per) < 200) per /= 2;
+    if (per == 2 && ctas(2) < 150) per = 1;
+    int n = (pl.hpg + per - 1) / per;
     if (pl.B * pl.nct * pl.G >= 64 && n * slots > 2 * pl.hpg) n = 2 * pl.hpg >= slots ? 2 * pl.hpg / slots : 1;
     const int hps = (pl.hpg + n - 1) / n;
     return (pl.hpg + hps - 1) / hps;                    // no empty range
@@ -149,8 +158,8 @@ static int make_plan(const ssd_shape_t *s, Plan &pl) {
 }
 
 // split path: whether the sums of a segment ride in a launch of its neighbour.  In the forward that takes second copies of states
-// and C B^T, up to 64 MiB of them: 17 MiB are worth 7 % (24 heads, 2048-step segments, 868 -> 803 us), 20 MiB 10 % (80 heads,
-// 1024 steps, 1544 -> 1391), 38 MiB 6 %, 74 MiB 2 % (80 heads, 4096 steps, 1351 -> 1326).
+// and C B^T, up to 64 MiB of them: in four segments, fp32, N = 128, chunk 256, they are worth 12 % at 8 MiB (24 heads, 2048 steps, 324 ->
+// 286 us), 6 % at 24 MiB (80 heads, 2048 steps, 854 -> 800), 4 % at 46 MiB (4096 steps, 1628 -> 1558).
 static bool simt_overlap(const Plan &pl, bool bwd) {
     const size_t copy = ((size_t)pl.B * pl.H * (pl.ncs + 1) * pl.P * pl.N + (size_t)pl.B * pl.ncs * pl.G * pl.Q * pl.Q) * sizeof(float);
     return pl.nseg > 1 && (bwd || copy <= (size_t)64 << 20);
