@@ -328,7 +328,7 @@ static SideStreams *side_streams() {
 static void select_copy(const Layout &lo, void *ws, int kc, int k, SegParams &sp) {
     char *w = (char *)ws;
     auto at = [&](size_t r) { return r ? (float *)(w + r) : nullptr; };
-    auto f = [&](const auto &r) { return at(r[k]); };
+    auto f = [&](const auto &r) { return at(r[k < (int)(sizeof(r) / sizeof(r[0])) ? k : 0]); };
     sp.rec = at(lo.rec[kc]);
     sp.cs = f(lo.cs);
     sp.dtT = sp.rec ? sp.rec + REC_DT : f(lo.dtT);

@@ -160,6 +160,19 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
         return r;
     };
 
+    // The load of pass `use` over a slot is complete.  A role that takes alternate heads does not see every pass: with nothing but the
+    // parity it would take a load two passes back for this one while the one between is still on its way.  So it first waits until
+    // the slot has been given back for this pass, as the producer did; that wait cannot be two passes early, since the head that the
+    // role had before this one was loaded after the pass before that had been given back.
+    auto wait_full = [&](int slot, uint32_t use) {
+        if (use) mbar_wait(&empty[slot], (use - 1) & 1, abortp, p.status);
+        mbar_wait(&full[slot], use & 1, abortp, p.status);
+    };
+    auto wait_x = [&](uint32_t slot, uint32_t use) {
+        if (use) mbar_wait(&xrempty[slot], (use - 1) & 1, abortp, p.status);
+        mbar_wait(&xrfull[slot], use & 1, abortp, p.status);
+    };
+
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (elect_one()) {
@@ -211,8 +224,8 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
             for (int u = u_begin; u < u_end; ++nrun) {
                 const Run r = run_at(u);
                 if (mine == 0) {
-                    mbar_wait(&full[v.slot], v.use & 1, abortp, p.status);
-                    mbar_wait(&full[NV + t.slot], t.use & 1, abortp, p.status);
+                    wait_full(v.slot, v.use);
+                    wait_full(NV + t.slot, t.use);
                     if (nrun) mbar_wait(&sfree, (nrun - 1) & 1, abortp, p.status);
                     tc_fence_after_sync();
                     const uint32_t lo0 = loC0 + v.slot * 1024, lo1 = loC1 + t.slot * (SC_STB / 16);
@@ -239,7 +252,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                     const uint32_t acc1 = tm + TM_ACC + bf * 128, acc2 = acc1 + 64, mA = tm + TM_M + bf * 64;
                     const uint32_t loV = loV0 + v.slot * 1024, loS = loS0 + t.slot * (SC_STB / 16);
                     if (hc >= 2) mbar_wait(&accempty[bf], par ^ 1u, abortp, p.status);
-                    mbar_wait(&full[NV + t.slot], t.use & 1, abortp, p.status);
+                    wait_full(NV + t.slot, t.use);
                     tc_fence_after_sync();
 #pragma unroll
                     for (int kk = 0; kk < KB; ++kk) {      // Rows (K = n) x state^T rows n (MN-major over p)
@@ -248,7 +261,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                         else umma_bf16_fixed<true>(acc2, ad, bd, id64);
                     }
                     umma_commit(&empty[NV + t.slot]);
-                    mbar_wait(&full[v.slot], v.use & 1, abortp, p.status);
+                    wait_full(v.slot, v.use);
                     mbar_wait(&mfull[bf], par, abortp, p.status);
                     tc_fence_after_sync();
 #pragma unroll
@@ -314,7 +327,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                     const uint32_t turn = hc >> 1;
                     const float *rec = reinterpret_cast<const float *>(smem + OFF_REC + vt.slot * 2048) - REC0;
                     const float *cs2 = rec + REC_CS;
-                    mbar_wait(&full[vt.slot], vt.use & 1, abortp, p.status);
+                    wait_full(vt.slot, vt.use);
                     const float csr = cs2[r], cs_lo = cs2[q * 32], cs_hi = cs2[q * 32 + 31];
                     const float rowf = FWD ? ex2f(csr - cs_lo) : ex2f(cs_hi - csr);      // off the diagonal, <= 1
                     bool waited = turn == 0;
@@ -404,7 +417,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                 if ((int)(hc & 1) != eg) continue;
                 const int h = rn.h0 + k;
                 const float *rec = reinterpret_cast<const float *>(smem + OFF_REC + vt.slot * 2048) - REC0;
-                mbar_wait(&full[vt.slot], vt.use & 1, abortp, p.status);
+                wait_full(vt.slot, vt.use);
                 const float csr = rec[REC_CS + r];
                 const float offs = FWD ? ex2f(csr) : ex2f(rec[REC_CS + 127] - csr);
                 const float dtr = rec[REC_DT + r];
@@ -413,7 +426,7 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
                 unsigned char *vrow = smem + OFF_VAL + vt.slot * 16384 + r * 128;       // x row (SC_FWD) / dy row (SC_DX), then output
                 const uint32_t xs = hc % SC_XR;
                 const unsigned char *xrow = smem + OFF_XR + xs * 16384 + r * 128;      // SC_DX: x row
-                if (!FWD) mbar_wait(&xrfull[xs], (hc / SC_XR) & 1, abortp, p.status);
+                if (!FWD) wait_x(xs, hc / SC_XR);
                 mbar_wait(&accfull[eg], (hc >> 1) & 1, abortp, p.status);
                 __syncwarp();
                 tc_fence_after_sync();
