@@ -178,7 +178,8 @@ static bool simt_readers(const Plan &pl) {
 // back when its segment's tail is done: chain, dB/dC beside dx, tail and the hand-overs take 77 us of 24 heads and 2048 steps, so with
 // two copies a segment can start every 38 us, while the gradient chain alone takes 28; the recompute likewise with three.  Where
 // the copies are small that latency is the bound, and there is one more of each: backward of 8 segments of that size 352 -> 316 us,
-// 16 of 1024 steps 513 -> 437 us (64 heads: 915 -> 716, 80: 1055 -> 820); 64 heads, 8 of 2048 (16 MiB) 602 -> 527 us; with 80 heads and 4096 steps, where SM time is the bound, 8 segments take the same with and without.
+// 16 of 1024 steps 513 -> 437 us (64 heads: 915 -> 716, 80: 1055 -> 820); 64 heads, 8 of 2048 (16 MiB) 602 -> 527 us;
+// with 80 heads and 4096 steps, where SM time is the bound, 8 segments take the same with and without.
 static const size_t kSmallStates = (size_t)16 << 20;
 static bool small_states(const Plan &pl) { return (size_t)pl.B * pl.H * pl.ncs * pl.P * pl.N * 2 <= kSmallStates; }
 static int chain_copies(const Plan &pl, bool bwd) {

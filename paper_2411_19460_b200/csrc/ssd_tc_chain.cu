@@ -121,7 +121,8 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     __syncthreads();
     tc_fence_after_sync();
     // What the kernel before this one in the stream may still write, or still read where this one writes, is waited for in the
-    // roles that touch it; x, dt, B, C and dy are older than the call, whose first launch is an ordinary one, so the first blocks are loaded and scaled under its end.
+    // roles that touch it; x, dt, B, C and dy are older than the call, whose first launch is an ordinary one, so the
+    // first blocks are loaded and scaled under its end.
     const uint32_t tm = words[0];
     volatile uint32_t *abortp = &words[1];
 
