@@ -33,6 +33,9 @@
  *  - Return value: SSD_OK (0) or a negative SSD_E* code.  On error nothing has been enqueued,
  *    except SSD_ECUDA, which reports a failed launch part-way (ssd_last_cuda_error() gives the
  *    CUDA code).
+ *  - Same buffers: h_final may be h0, and dh0 may be dh_final or, where B or nseg is 1, boundary (its first
+ *    state is replaced); the result is that of separate buffers.  boundary may start at h0 where B or nseg is 1.
+ *    No other output may overlap an input or another output, unless the call says so.
  *  - Deterministic: the same inputs give the same bits run to run, and the gradients of
  *    ssd_bwd_segmented do not depend on `seg` (seg == L is the unsegmented backward).
  *  - Gradient outputs are overwritten, not accumulated into (dA, dD: unless SSD_FLAG_ACCUM_PARAM_GRADS).

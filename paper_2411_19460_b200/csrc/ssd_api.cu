@@ -251,6 +251,9 @@ static void make_static_layout(Plan &pl, Layout &lo) {
     make_layout(pl, SSD_OP_FWD, lo, false);
 }
 
+// Whether two buffers of n and m floats (null: none) have a byte in common
+static bool overlap_of(const float *a, size_t n, const float *b, size_t m) { return a && b && a < b + m && b < a + n; }
+
 static bool misaligned(const void *p) { return ((uintptr_t)p & 15u) != 0; }
 
 static int check_device() {
@@ -486,7 +489,11 @@ static int forward_impl(const ssd_shape_t *shape, const void *x, const float *dt
     }
     sp.chain_heads = chain_heads(pl, false);
     const bool overlap = beside && simt_overlap(pl, false);
-    const bool readers = beside && simt_readers(pl) && (overlap || pl.nseg == 1);       // a segment's exit state needs the next one's copy
+    // Readers only where a segment's exit state has the next one's copy to go to, and not where it or the boundary state goes to h0 itself:
+    // its CTAs would store what the tiles of y in the same launch still read.  (A state pass reads and stores an element in one thread.)
+    const size_t nh = (size_t)pl.B * pl.H * PN;
+    const bool in_place = (pl.nseg == 1 && overlap_of(h0, nh, h_final, nh)) || overlap_of(h0, nh, boundary, nh * pl.nseg);
+    const bool readers = beside && simt_readers(pl) && (overlap || pl.nseg == 1) && !in_place;
     SegParams next;
     for (int k = 0; k < pl.nseg; ++k) {
         set_segment(pl, k, sp);
@@ -733,6 +740,10 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
         SSD_TRY(cudaStreamWaitEvent(st, side->tail_done[(pl.nseg - 1) % kChainCopies], 0));   // the finishing stream is in order: this covers every segment
     } else {
         sp.chain_heads = chain_heads(pl, false);
+        // no readers where dh0 goes to what they read beside it: the first segment's state, or the gradient that enters the only segment
+        const size_t nh = (size_t)pl.B * pl.H * PN;
+        const bool in_place = (pl.nseg == 1 && overlap_of(dh0, nh, dh_final, nh)) || overlap_of(dh0, nh, boundary, nh * pl.nseg);
+        const bool readers = !pl.serial && simt_readers(pl) && !in_place;
         for (int k = pl.nseg - 1; k >= 0; --k) {
             set_segment(pl, k, sp);
             sp.first = k == pl.nseg - 1;
@@ -753,7 +764,7 @@ int ssd_bwd_segmented(const ssd_shape_t *shape, const void *x, const float *dt, 
             } else {
                 select_copy(lo, ws, 0, k & 1, sp);
                 if (k == pl.nseg - 1 || pl.serial) SSD_LAUNCH(KIND_CHUNK_STATE, launch_simt(sp, nullptr, nullptr, pl.dtype, SIMT_SUMS_GRAD, st));
-                if (!pl.serial && simt_readers(pl)) {
+                if (readers) {
                     // the gradient handed left is written while the one from the right is read: in gcarry and the last slot of Gst in turn
                     const int64_t own = pl.H * PN, slots = (pl.ncs + 1) * pl.H * PN;
                     float *const turn[2] = {sp.gcarry, sp.Gst + (size_t)pl.ncs * pl.H * PN};
