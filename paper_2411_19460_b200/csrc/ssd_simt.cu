@@ -171,11 +171,20 @@ template <typename T> struct SimtSmem {
     static constexpr int CTAS = PT == 1 ? 3 : 2;     // CTAs per SM
     SplitTile t[3 + PT];
     float css[256], dts[256], fac[256], red[6][64];
+    int again;                                       // a product of this CTA came out as NaN
 };
 constexpr int ST_LD = 72;                            // floats per row of an output tile staged in t[0], t[1]
 static_assert(64 * ST_LD * sizeof(float) <= 2 * sizeof(SplitTile), "an fp32 output tile in the place of two parts");
 static_assert(FIN_TILE * sizeof(float) <= 2 * sizeof(SplitTile), "the finishing step's tile");
 
+template <typename T> __device__ __forceinline__ SimtSmem<T> &simt_smem() {
+    extern __shared__ __align__(16) unsigned char smem[];
+    return *reinterpret_cast<SimtSmem<T> *>(smem);
+}
+// A CTA some of whose sums are NaN (`again` in its shared memory; its body returns true) runs once more with AGAIN, for infinities (see
+// tile_mma), and writes its outputs a second time.  That costs a check of its last accumulators and, in effect, what a second body does to
+// registers and code.  In line: 2 x 4096 steps of 24 heads, fp32, 1029 -> 1027 us, 2 x 8192 of 32, bf16, 1013 -> 1019, 1024 of 4, fp32, 106.7 as
+// before; with a function of its own 1031, 1029 and 109; with one body and a flag 1089, 1099 and 113.
 template <typename T> __device__ __forceinline__ float4 ld4f(const T *p);
 template <> __device__ __forceinline__ float4 ld4f<float>(const float *p) { return __ldg(reinterpret_cast<const float4 *>(p)); }
 template <> __device__ __forceinline__ float4 ld4f<__nv_bfloat16>(const __nv_bfloat16 *p) {
@@ -241,7 +250,7 @@ template <typename T, int NS> __host__ __device__ __forceinline__ int simt_n_sum
     const int nrt = p.Q >> 6;
     return p.nc * p.B * ((NS / 64) * p.H * (grads && !simt_sums_merged<NS>(p) ? 2 : 1) + (p.cbt ? p.G * (nrt * (nrt + 1) / 2) : 0));
 }
-template <typename T, int NS> __device__ __forceinline__ void simt_sums(const SegParams &p, SimtSmem<T> &sm, int id, bool grads) {
+template <typename T, int NS, bool AGAIN> __device__ __forceinline__ bool simt_sums(const SegParams &p, SimtSmem<T> &sm, int id, bool grads) {
     constexpr int PT = SimtSmem<T>::PT;
     const int tid = threadIdx.x, Q = p.Q, nrt = Q >> 6, nh = NS / 64;
     const size_t HP = (size_t)p.H * 64, GN = (size_t)p.G * NS;
@@ -270,10 +279,10 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
             tile_store(sm.t, ra);
             tile_store(sm.t + PT, rb);
             __syncthreads();
-            tile_mma<PT, PT, false, false>(acc, sm.t, sm.t + PT);
+            tile_mma<PT, PT, false, false, AGAIN>(acc, sm.t, sm.t + PT);
         }
         store_acc(acc, cb_of(p, b, c, g) + (size_t)rt * 64 * Q + ct * 64, Q);
-        return;
+        return PT > 1 && !AGAIN && __syncthreads_or(acc.nan());
     }
     const int n0 = (id % nh) * 64;
     id /= nh;
@@ -327,6 +336,7 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
     }
     __syncthreads();
     const int end = merged ? 2 * Q : Q;
+    if (!AGAIN && tid == 0) sm.again = 0;
     for (int i0 = 0; i0 < end; i0 += 64) {
         const bool dst = second || i0 >= Q;
         const int s0 = i0 >= Q ? i0 - Q : i0;
@@ -343,20 +353,21 @@ template <typename T, int NS> __device__ __forceinline__ void simt_sums(const Se
         tile_store(sm.t + 3, rb);
         __syncthreads();
         if (i0 + 64 < end) load_rows(second || i0 + 64 >= Q, i0 + 64 >= Q ? i0 + 64 - Q : i0 + 64);
-        tile_mma<3, PT, true, true>(acc, sm.t, sm.t + 3);
+        tile_mma<3, PT, true, true, AGAIN>(acc, sm.t, sm.t + 3);
         if (s0 + 64 == Q) {
+            if (!AGAIN && acc.nan()) sm.again = 1;
             store_acc(acc, (dst ? p.Gst + slot_off(p, b, c, h) : p.Hst + slot_off(p, b, c + 1, h)) + n0, NS);
             acc.zero();
         }
         __syncthreads();
     }
+    return !AGAIN && sm.again;
 }
 
-template <typename T, int NS> __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_sums(SegParams p, bool grads) {
-    extern __shared__ __align__(16) unsigned char smem[];
+template <typename T, int NS> __global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_sums(const __grid_constant__ SegParams p, bool grads) {
     pdl_launch_dependents();
     if (p.first && blockIdx.x == 0 && threadIdx.x < 64) p.status[threadIdx.x] = 0u;
-    simt_sums<T, NS>(p, *reinterpret_cast<SimtSmem<T> *>(smem), blockIdx.x, grads);
+    if (simt_sums<T, NS, false>(p, simt_smem<T>(), blockIdx.x, grads)) simt_sums<T, NS, true>(p, simt_smem<T>(), blockIdx.x, grads);
 }
 
 template <int NS> __device__ __forceinline__ size_t slot_of(const SegParams &p, int b, int slot, int h) {
@@ -461,8 +472,8 @@ template <bool BWD> __device__ __forceinline__ void pass_along(const SegParams &
 //   ddt_direct_s = x_s . u_s , psi2_s = dt_s e^{cs_last-cs_s} x_s . (Gout B_s) , dD partial = sum dy.x
 // CB false (y only): the tiles of C B^T are not in the scratch and are made here, per head, with the same operations in the same
 // order, so with the same bits.
-template <typename T, int NS, bool DX, bool CB, bool READER>
-__device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &sm, int c, int rt, int h, int b) {
+template <typename T, int NS, bool DX, bool CB, bool READER, bool AGAIN>
+__device__ __forceinline__ bool simt_row_tile(const SegParams &p, SimtSmem<T> &sm, int c, int rt, int h, int b) {
     constexpr int PT = SimtSmem<T>::PT;
     float *css = sm.css, *dts = sm.dts, *fac = sm.fac, *facd = sm.red[5];
     const int tid = threadIdx.x, Q = p.Q, nrt = Q >> 6, g = h / p.hpg, r0 = rt * 64;
@@ -475,6 +486,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
     TileRegs<float> rf;
     Acc acc;
     acc.zero();
+    if (!AGAIN && tid == 0) sm.again = 0;
     tile_load(rv, rowv, GN);
     pdl_wait();
     load_state<NS, DX, READER>(rf, p, b, h, c, 0);
@@ -498,7 +510,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
         } else if (CB) {
             load_vals(ct0);
         }
-        tile_mma<PT, 3, false, false>(acc, sm.t, sm.t + PT);
+        tile_mma<PT, 3, false, false, AGAIN>(acc, sm.t, sm.t + PT);
         __syncthreads();
     }
     // Off the diagonal tile the mask factors at the tile's edge m (its first row; dx: last), where both factors are <= 1:
@@ -546,7 +558,7 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
                 tile_store(sm.t, rv);
                 tile_store(sm.t + PT, rc);
                 __syncthreads();
-                tile_mma<PT, PT, false, false>(cb, sm.t, sm.t + PT);
+                tile_mma<PT, PT, false, false, AGAIN>(cb, sm.t, sm.t + PT);
                 __syncthreads();
             }
             load_vals(ct);
@@ -590,13 +602,15 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
         tile_store(sm.t + 3, rv);
         __syncthreads();
         if (CB && ct + 1 < ct1) load_vals(ct + 1);
-        tile_mma<3, PT, DX, true>(acc, sm.t, sm.t + 3);
+        tile_mma<3, PT, DX, true, AGAIN>(acc, sm.t, sm.t + 3);
         __syncthreads();
     }
     // through shared memory, so that the caller's rows are read and written in whole sectors
     float *stg = reinterpret_cast<float *>(sm.t);
     store_acc(acc, stg, ST_LD);
+    if (!AGAIN && acc.nan()) sm.again = 1;
     __syncthreads();
+    if (!AGAIN && sm.again) return true;
     const float Dh = __ldg(p.D + h) + (DX ? p.dx_skip : 0.f);      // dx: D dy, plus dy itself under a skip connection
     float dsum = 0.f, dprev = 0.f;
 #pragma unroll
@@ -631,63 +645,41 @@ __device__ __forceinline__ void simt_row_tile(const SegParams &p, SimtSmem<T> &s
             p.dDp[((((size_t)b * p.H + h) * p.nct + p.c0 + c) << 2) + rt] = s;
         }
     }
+    return false;
 }
 
 // y of a segment and, in the same launch where the scratch has a second copy, the sums of the next segment (n_next CTAs): they
 // wait for nothing of this one, and a launch of a few microseconds is saved per segment.  READER: no state pass has run; n_pass
 // CTAs make what it hands on.
-template <typename T, int NS, bool CB, bool READER>
-__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_y(SegParams p, SegParams nx, int n_next, StatePass pass, int n_pass) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
-    pdl_launch_dependents();
+template <typename T, int NS, bool CB, bool READER, bool AGAIN>
+__device__ __forceinline__ bool simt_y(const SegParams &p, const SegParams &nx, int n_next, const StatePass &pass, int n_pass) {
+    SimtSmem<T> &sm = simt_smem<T>();
     const int nrt = p.Q >> 6, ny = (int)gridDim.x - n_next;
     int id = blockIdx.x;
-    if (id >= ny) {
-        simt_sums<T, NS>(nx, sm, id - ny, false);
-        return;
-    }
+    if (id >= ny) return simt_sums<T, NS, AGAIN>(nx, sm, id - ny, false);
     if (READER && id >= ny - n_pass) {
         pdl_wait();
         pass_along<false>(p, pass, sm.red[0], id - (ny - n_pass));
-        return;
+        return false;
     }
     const int rt = id & (nrt - 1), bhc = id >> (nrt >> 1), bh = divide_by(bhc, p.nc, p.inv_nc), c = bhc - bh * p.nc, b = divide_by(bh, p.H, p.inv_H),
               h = bh - b * p.H;       // nrt is 1, 2 or 4
-    simt_row_tile<T, NS, false, CB, READER>(p, sm, c, rt, h, b);
+    return simt_row_tile<T, NS, false, CB, READER, AGAIN>(p, sm, c, rt, h, b);
+}
+template <typename T, int NS, bool CB, bool READER>
+__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS)
+k_simt_y(const __grid_constant__ SegParams p, const __grid_constant__ SegParams nx, int n_next, const __grid_constant__ StatePass pass, int n_pass) {
+    pdl_launch_dependents();
+    if (simt_y<T, NS, CB, READER, false>(p, nx, n_next, pass, n_pass)) simt_y<T, NS, CB, READER, true>(p, nx, n_next, pass, n_pass);
 }
 
-// The large kernel of the backward: tiles of dx, and the partial slices of dB and dC.  Per (chunk, head range):
-//   causal tile pair (tt, ts): W_h = (dy_tt x_ts^T) o mask per head, rho / psi partial sums of W_h o CB, head sum of W_h; then
-//                  slices dC[tt] = Wsum B_ts and dB[ts] = Wsum^T C_tt
-//   inter dC, tile tt : sum_h e^{cs_t} dy_t H_in (and rho2 per head);  inter dB, tile ts : sum_h dt_s e^{cs_last-cs_s} x_s Gout
-// A row of tile r has dC slots for ts <= r and dB slots for tt >= r, so the two share Q/64 + 3 slots per head range: dC by ts, dB by
-// tt + 1, then the inter-chunk terms of both.
-// Three CTAs per SM only for bf16 with N = 64 and state passes (2 x 8192 steps of 32 heads: two 0.6 % slower); elsewhere 80 registers spill too
-// much (4096 steps of 24 heads, N = 128, chunks of 64: 612 us at three, 521 at two; N = 64, states made in their readers, 385 and 352).
-template <typename T, int NS, bool READER>
-__global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !READER ? 3 : 2) k_simt_bwd(SegParams p, int n_dx, StatePass pass, int n_pass) {
+// A CTA's part of dB and dC (the roles below)
+template <typename T, int NS, bool READER, bool AGAIN> __device__ __forceinline__ bool simt_dbdc(const SegParams &p, SimtSmem<T> &sm, int id) {
     constexpr int PT = SimtSmem<T>::PT;
-    extern __shared__ __align__(16) unsigned char smem[];
-    SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
-    pdl_launch_dependents();
     const int tid = threadIdx.x, lane = tid & 31, Q = p.Q, nrt = Q >> 6, npair = nrt * (nrt + 1) / 2;
-    int id = blockIdx.x;
-    const int n_bc = (int)gridDim.x - n_dx - n_pass;
-    if (READER && id >= n_bc + n_dx) {
-        pdl_wait();
-        pass_along<true>(p, pass, sm.red[0], id - n_bc - n_dx);
-        return;
-    }
-    if (id >= n_bc) {
-        id -= n_bc;
-        const int rt = id & (nrt - 1), bch = id >> (nrt >> 1), bc = divide_by(bch, p.H, p.inv_H), h = bch - bc * p.H,
-                  b = divide_by(bc, p.nc, p.inv_nc), c = bc - b * p.nc;
-        simt_row_tile<T, NS, true, true, READER>(p, sm, c, rt, h, b);
-        return;
-    }
     const int per = npair + 2 * nrt, role = id % per;
     id /= per;
+    if (!AGAIN && tid == 0) sm.again = 0;
     const int rng = p.nsl / (nrt + 3);                         // head ranges per group
     const int sl = id % rng, g = (id / rng) % p.G, c = (id / (rng * p.G)) % p.nc, b = id / (rng * p.G * p.nc);
     const int hps = (p.hpg + rng - 1) / rng, h0 = g * p.hpg + sl * hps, h1 = min(h0 + hps, (g + 1) * p.hpg);
@@ -747,7 +739,7 @@ __global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !REA
                 load_vec(h + 1);
             }
             acc.zero();
-            tile_mma<PT, PT, false, false>(acc, sm.t, sm.t + PT);
+            tile_mma<PT, PT, false, false, AGAIN>(acc, sm.t, sm.t + PT);
             float2 row[2], col[4];
 #pragma unroll
             for (int j = 0; j < 4; ++j) col[j] = make_float2(0.f, 0.f);
@@ -818,12 +810,13 @@ __global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !REA
             __syncthreads();
             if (n0 + 64 < 2 * NS) tile_load(rb, n0 + 64 >= NS ? Cb + (size_t)tt * 64 * GN + n0 + 64 - NS : Bb + (size_t)ts * 64 * GN + n0 + 64, GN);
             acc.zero();
-            if (isB) tile_mma<3, PT, true, true>(acc, sm.t, sm.t + 3);
-            else tile_mma<3, PT, false, true>(acc, sm.t, sm.t + 3);
+            if (isB) tile_mma<3, PT, true, true, AGAIN>(acc, sm.t, sm.t + 3);
+            else tile_mma<3, PT, false, true, AGAIN>(acc, sm.t, sm.t + 3);
+            if (!AGAIN && acc.nan()) sm.again = 1;         // (a NaN of the head sum is in its whole row of the product)
             store_acc(acc, isB ? slice(ts * 64, tt + 1, n) : slice(tt * 64, ts, n), slice_stride);
             __syncthreads();
         }
-        return;
+        return !AGAIN && sm.again;
     }
     // inter-chunk terms of one row tile: the head's rows times the chunk state (rows p), the products scaled per row
     const bool isC = role - npair < nrt;
@@ -864,7 +857,7 @@ __global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !REA
                 state(h + 1, 0);
             }
             acc.zero();
-            tile_mma<PT, 3, false, true>(acc, sm.t, sm.t + PT);
+            tile_mma<PT, 3, false, true, AGAIN>(acc, sm.t, sm.t + PT);
 #pragma unroll
             for (int half = 0; half < 2; ++half)
 #pragma unroll
@@ -883,6 +876,12 @@ __global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !REA
                     if ((lane & 3) == 0) sm.red[tid >> 7][acc_row(half)] = v;
                 }
             }
+            if (!AGAIN && h + 1 == h1) {
+                bool nan = false;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) nan |= isnan(tot[m][0][j].x) || isnan(tot[m][0][j].y) || isnan(tot[m][1][j].x) || isnan(tot[m][1][j].y);
+                if (nan) sm.again = 1;
+            }
             __syncthreads();
         }
         if (isC && tid < 64) p.rho2[vo + rt * 64 + tid] = sm.red[0][tid] + sm.red[1][tid];
@@ -896,6 +895,38 @@ __global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !REA
             for (int j = 0; j < 4; ++j)
                 *reinterpret_cast<float2 *>(out + (size_t)acc_row(half) * slice_stride + acc_col(j)) = tot[m][half][j];
     }
+    return !AGAIN && sm.again;
+}
+
+// The large kernel of the backward: tiles of dx, and the partial slices of dB and dC.  Per (chunk, head range):
+//   causal tile pair (tt, ts): W_h = (dy_tt x_ts^T) o mask per head, rho / psi partial sums of W_h o CB, head sum of W_h; then
+//                  slices dC[tt] = Wsum B_ts and dB[ts] = Wsum^T C_tt
+//   inter dC, tile tt : sum_h e^{cs_t} dy_t H_in (and rho2 per head);  inter dB, tile ts : sum_h dt_s e^{cs_last-cs_s} x_s Gout
+// A row of tile r has dC slots for ts <= r and dB slots for tt >= r, so the two share Q/64 + 3 slots per head range: dC by ts, dB by
+// tt + 1, then the inter-chunk terms of both.
+// Three CTAs per SM only for bf16 with N = 64 and state passes (2 x 8192 steps of 32 heads: two 0.6 % slower); elsewhere 80 registers spill too
+// much (4096 steps of 24 heads, N = 128, chunks of 64: 612 us at three, 521 at two; N = 64, states made in their readers, 385 and 352).
+template <typename T, int NS, bool READER, bool AGAIN>
+__device__ __forceinline__ bool simt_bwd(const SegParams &p, int n_dx, const StatePass &pass, int n_pass) {
+    SimtSmem<T> &sm = simt_smem<T>();
+    const int nrt = p.Q >> 6, n_bc = (int)gridDim.x - n_dx - n_pass;
+    int id = blockIdx.x;
+    if (READER && id >= n_bc + n_dx) {
+        pdl_wait();
+        pass_along<true>(p, pass, sm.red[0], id - n_bc - n_dx);
+        return false;
+    }
+    if (id < n_bc) return simt_dbdc<T, NS, READER, AGAIN>(p, sm, id);
+    id -= n_bc;
+    const int rt = id & (nrt - 1), bch = id >> (nrt >> 1), bc = divide_by(bch, p.H, p.inv_H), h = bch - bc * p.H,
+              b = divide_by(bc, p.nc, p.inv_nc), c = bc - b * p.nc;
+    return simt_row_tile<T, NS, true, true, READER, AGAIN>(p, sm, c, rt, h, b);
+}
+template <typename T, int NS, bool READER>
+__global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !READER ? 3 : 2)
+k_simt_bwd(const __grid_constant__ SegParams p, int n_dx, const __grid_constant__ StatePass pass, int n_pass) {
+    pdl_launch_dependents();
+    if (simt_bwd<T, NS, READER, false>(p, n_dx, pass, n_pass)) simt_bwd<T, NS, READER, true>(p, n_dx, pass, n_pass);
 }
 
 // ------------------------------------------------------------------ da, ddt, dA partial
@@ -1050,16 +1081,24 @@ __global__ void __launch_bounds__(256) k_bwd_tail(SegParams p, int nfin) {
     if ((int)blockIdx.x < nfin) bwd_finish<TC>(p, tile, blockIdx.x);
     else reduce_dbdc<T, TC>(p, blockIdx.x - nfin);
 }
+// The second pass over the next segment's sums as a function: fp32, where the launch takes 211 us a pass instead of 194 with it in line
+// (2 x 4096 steps of 24 heads); bf16 has it in line (159 us, as a function 173; 2 x 8192 steps of 32 heads)
+template <typename T, int NS> __device__ __noinline__ void simt_sums_call(const SegParams &p) {
+    simt_sums<T, NS, true>(p, simt_smem<T>(), blockIdx.x, true);
+}
 // split path: the same with the sums of the next segment (to the left) in front, which share no scratch with it but the step
 // sizes, of which there are two copies.
 template <typename T, int NS>
-__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS) k_simt_tail(SegParams p, SegParams nx, int n_next, int nfin) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    SimtSmem<T> &sm = *reinterpret_cast<SimtSmem<T> *>(smem);
+__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS)
+k_simt_tail(const __grid_constant__ SegParams p, const __grid_constant__ SegParams nx, int n_next, int nfin) {
+    SimtSmem<T> &sm = simt_smem<T>();
     pdl_launch_dependents();
     const int id = (int)blockIdx.x - n_next;
     if (id < 0) {
-        simt_sums<T, NS>(nx, sm, blockIdx.x, true);
+        if (simt_sums<T, NS, false>(nx, sm, blockIdx.x, true)) {
+            if constexpr (SplitParts<T>::n > 1) simt_sums_call<T, NS>(nx);
+            else simt_sums<T, NS, true>(nx, sm, blockIdx.x, true);
+        }
         return;
     }
     pdl_wait();

@@ -1,12 +1,16 @@
-// 64 x 64 x 64 tile products with fp32 operands on the tensor cores: an fp32 value is the exact sum of three bf16 parts, a bf16
-// value is its own single part, and the products of parts are exact in the fp32 accumulators of mma.sync.
+// 64 x 64 x 64 tile products with fp32 operands on the tensor cores: an fp32 value is the sum of three bf16 parts, a bf16 value is its own
+// single part, and the products of parts are exact in the fp32 accumulators of mma.sync.
 //
 //   x = p0 + p1 + p2:  p0 the upper half of x's bits (no overflow near the largest values), p1 the rest rounded to nearest, so
 //   that what it leaves for p2 has either sign, p2 the rest of that, at most eight bits.
+// The sum is x exactly from 2^-110 up.  Of a smaller x it misses what lies below bf16's smallest number, less than 2^-133: values of 2^-120 are
+// held to 13 bits, those of 2^-126, the smallest normal fp32 number, to seven.
 // Products p_i q_j with i + j > 2 are left out (below 2^-23 of x y each, of either sign: about 2^-25 on average).  mma.sync truncates when it
 // adds to its accumulator, a bias of half a unit in the last place per step, so for every 16 steps of the contraction the products
 // start from zero, the smallest first, and their sum is added with a rounded fp32 addition: one truncation at the size of the sum.
-// Infinities come out as infinities or NaN (0 x infinity in another part), NaN as NaN.
+// Infinities: p1 and p2 of an infinite x are NaN, and p0 = x times parts of either sign or zero would be NaN too, where x y is infinite.  So
+// a NaN among the sums of 16 is taken again with whole values, in a second pass over a tile that has one (AGAIN): infinities and NaN come
+// out as fp32 arithmetic has them.  (A signalling NaN whose payload is all in its lower half may come out as an infinity.)
 #pragma once
 #include <cuda_bf16.h>
 #include <stdint.h>
@@ -103,6 +107,14 @@ struct Acc {
 #pragma unroll
             for (int i = 0; i < 4; ++i) m[j][i] = 0.f;
     }
+    __device__ __forceinline__ bool nan() const {
+        bool r = false;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) r |= isnan(m[j][i]);
+        return r;
+    }
     // rows of half `half`, columns acc_col(j) and the next
     __device__ __forceinline__ float2 get(int j, int half) const { return make_float2(m[j][2 * half], m[j][2 * half + 1]); }
     __device__ __forceinline__ void set(int j, int half, float2 v) {
@@ -135,16 +147,22 @@ __device__ __forceinline__ void mma_zero(float (&c)[4], const uint32_t (&a)[4], 
         : "=f"(c[0]), "=f"(c[1]), "=f"(c[2]), "=f"(c[3])
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
+// Element (row, col) of a tile from its PARTS parts: the first alone where it is infinite, because the others are NaN then
+template <int PARTS> __device__ __forceinline__ float joined(const SplitTile *s, int row, int col) {
+    const float p0 = __bfloat162float(s[0].v[row][col]);
+    if constexpr (PARTS == 1) return p0;
+    const float v = p0 + (__bfloat162float(s[1].v[row][col]) + __bfloat162float(s[2].v[row][col]));
+    return isinf(p0) ? p0 : v;
+}
 // c += A B over 64 steps of the contraction, A of PA parts and B of PB.  AK, BK: the staged rows of that operand run along the
-// contraction (else along the output's rows, columns).
-template <int PA, int PB, bool AK, bool BK> __device__ __forceinline__ void tile_mma(Acc &c, const SplitTile *a, const SplitTile *b) {
+// contraction (else along the output's rows, columns).  AGAIN: sums of 16 products that come out as NaN are taken again, of whole values.
+template <int PA, int PB, bool AK, bool BK, bool AGAIN> __device__ __forceinline__ void tile_mma(Acc &c, const SplitTile *a, const SplitTile *b) {
     const int lane = threadIdx.x & 31, wm = ((threadIdx.x >> 5) & 3) * 16, wn = (threadIdx.x >> 7) * 32;
     const int l7 = lane & 7, l8 = ((lane >> 3) & 1) * 8, l16 = (lane >> 4) * 8;
     constexpr uint32_t ROWB = SP_ROW * 2, PART = sizeof(SplitTile);
     const uint32_t aa = sm100::smem_u32(a) + (AK ? (l16 + l7) * ROWB + (wm + l8) * 2 : (wm + l8 + l7) * ROWB + l16 * 2);
     const uint32_t ba = sm100::smem_u32(b) + (BK ? (l8 + l7) * ROWB + (wn + l16) * 2 : (wn + l16 + l7) * ROWB + l8 * 2);
-#pragma unroll
-    for (int k = 0; k < 64; k += 16) {
+    auto steps = [&](int k) {
         uint32_t fa[PA][4];
         float t[4][4];
 #pragma unroll
@@ -166,10 +184,34 @@ template <int PA, int PB, bool AK, bool BK> __device__ __forceinline__ void tile
                 first = false;
             }
         }
+        if constexpr (AGAIN && PA + PB > 2) {
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                if (!(isnan(t[j][0]) || isnan(t[j][1]) || isnan(t[j][2]) || isnan(t[j][3]))) continue;
+                float f[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 1
+                for (int i = k; i < k + 16; ++i)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int r = acc_row(e >> 1), n = acc_col(j) + (e & 1);
+                        f[e] = fmaf(AK ? joined<PA>(a, i, r) : joined<PA>(a, r, i), BK ? joined<PB>(b, i, n) : joined<PB>(b, n, i), f[e]);
+                    }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) t[j][e] = isnan(t[j][e]) ? f[e] : t[j][e];
+            }
+            __syncwarp();
+        }
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
             for (int half = 0; half < 2; ++half) c.set(j, half, __fadd2_rn(c.get(j, half), make_float2(t[j][2 * half], t[j][2 * half + 1])));
+    };
+    if constexpr (AGAIN) {
+#pragma unroll 1
+        for (int k = 0; k < 64; k += 16) steps(k);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 64; k += 16) steps(k);
     }
 }
 

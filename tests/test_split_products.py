@@ -34,6 +34,16 @@ def test_parts_are_exact_and_what_is_left_out_is_small(exponent):
     assert left < 2.0 ** -16 / math.sqrt(len(x)) * 4
 
 
+@pytest.mark.parametrize("exponent", [-110, -111, -120, -126, -135, -148])
+def test_parts_of_the_smallest_values(exponent):
+    """Exact from 2^-110 up, where the last bit of an fp32 value is bf16's smallest number; below, what lies under that is missing."""
+    g = torch.Generator().manual_seed(exponent + 1000)
+    x = ((1 + torch.rand(1 << 14, generator=g).double()) * 2.0 ** exponent).float()
+    x[::2] *= -1
+    off = (sum(v.double() for v in parts(x)) - x.double()).abs().max().item()
+    assert off < 2.0 ** -133 and (off == 0) == (exponent >= -110)
+
+
 def config(dtype, L, H, N, G, chunk, seg, **extra):
     return CONFIGS[0].scaled(**dict(dict(name="split", dtype=dtype, B=1, L=L, H=H, P=64, N=N, G=G, chunk=chunk, seg=seg, h0_std=0.1,
                                          dh_std=0.1), **extra))
@@ -93,3 +103,101 @@ def test_values_that_are_not_finite_stay_so_and_do_not_go_back_in_time(value):
     got = pu.run_gpu(cfg, inp, want=("fwd",))
     assert not torch.isfinite(got["y"][0, 200:, 1, 7]).any() and not torch.isfinite(got["h_final"][0, 1, 7]).any()
     assert torch.equal(got["y"][0, :128], base["y"][0, :128]) and torch.equal(got["y"][:, :, 0], base["y"][:, :, 0])
+
+
+INFINITE = [("fp32", 64, 128), ("fp32", 128, 256), ("bf16", 64, 128), ("bf16", 128, 64)]
+
+
+def same(a, b):
+    return torch.equal(a.float().view(torch.int32), b.float().view(torch.int32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dtype,N,chunk", INFINITE)
+@pytest.mark.parametrize("sign", [1.0, -1.0])
+def test_infinities_come_out_as_infinities(dtype, N, chunk, sign):
+    """An infinite operand times the parts of either sign of the other is NaN; the recurrence has an infinity there, whose sign the
+    inputs say.  Whatever the infinity does not reach keeps its bits, in the same tile too."""
+    cfg = config(dtype, 512, 2, N, 1, chunk, 256)
+    inp = make_inputs(cfg, "cuda", seed=6)
+    base = pu.run_gpu(cfg, inp)
+    inf = sign * float("inf")
+    t, h, p, n = 200, 1, 7, 9
+    c0, c1 = t // chunk * chunk, (t // chunk + 1) * chunk               # its chunk
+    B, C = inp["Bm"][0, :, 0].double(), inp["Cm"][0, :, 0].double()
+    others = [i for i in range(64) if i != p]
+
+    def run(name, at):
+        i = dict(inp, **{name: inp[name].clone()})
+        i[name][at] = inf
+        got = pu.run_gpu(cfg, i)
+        for k, v in pu.run_gpu(cfg, i, flags=libssd.SSD_FLAG_SERIAL).items():
+            assert same(v, got[k]), (name, k)
+        return got
+
+    def expect(got, signs, what):
+        assert torch.equal(got.double(), (torch.sign(signs) * inf).expand_as(got).double()), what
+
+    got = run("x", (0, t, h, p))
+    expect(got["y"][0, t + 1:c1, h, p], C[t + 1:c1] @ B[t], "x -> y")
+    expect(got["h_final"][0, h, p], B[t], "x -> h_final")
+    expect(got["boundary"][0, 1, h, p], B[t], "x -> boundary")
+    assert same(got["y"][0, :, h, others], base["y"][0, :, h, others]) and same(got["y"][:, :, 0], base["y"][:, :, 0])
+    assert same(got["y"][0, :t // 64 * 64], base["y"][0, :t // 64 * 64]) and same(got["h_final"][0, h, others], base["h_final"][0, h, others])
+    dy = inp["dy"][0, :, h].double()
+    rows = slice(t + 1, c1)
+    if c1 > t + 1:                     # W_ts = (dy_t . x_s) e dt: one infinite column, added up over the heads into dC = W B
+        expect(got["dC"][0, rows, 0], torch.sign(dy[rows, p])[:, None] * torch.sign(B[t])[None], "x -> dC")
+
+    got = run("h0", (0, h, p, n))
+    expect(got["y"][0, :, h, p], C[:, n], "h0 -> y")
+    expect(got["dC"][0, :, 0, n], dy[:, p], "h0 -> dC")
+    assert got["h_final"][0, h, p, n] == inf and same(got["y"][0, :, h, others], base["y"][0, :, h, others])
+    keep = [i for i in range(N) if i != n]
+    assert same(got["h_final"][0, h, p, keep], base["h_final"][0, h, p, keep]) and same(got["dC"][0, :, 0, keep], base["dC"][0, :, 0, keep])
+
+    got = run("dy", (0, t, h, p))
+    expect(got["dx"][0, c0:t, h, p], B[c0:t] @ C[t], "dy -> dx")
+    expect(got["dh0"][0, h, p], C[t], "dy -> dh0")
+    assert same(got["dx"][0, :, h, others], base["dx"][0, :, h, others]) and same(got["dh0"][0, h, others], base["dh0"][0, h, others])
+    assert same(got["dx"][0, (t // 64 + 1) * 64:], base["dx"][0, (t // 64 + 1) * 64:])
+
+    got = run("Bm", (0, t, 0, n))
+    x = inp["x"][0, t].double()                                          # [H, P]
+    expect(got["h_final"][0, :, :, n], x, "B -> h_final")
+    expect(got["y"][0, t + 1:c1], torch.sign(C[t + 1:c1, n])[:, None, None] * torch.sign(x)[None], "B -> y")
+    assert same(got["h_final"][0, :, :, keep], base["h_final"][0, :, :, keep])
+
+
+@pytest.mark.gpu
+def test_infinities_where_every_tile_of_y_makes_its_own_products():
+    """24 heads in 8 groups, segments of 1024 steps: the built-in scratch has no room for C B^T."""
+    cfg = config("fp32", 2048, 24, 64, 8, 64, 1024)
+    inp = make_inputs(cfg, "cuda", seed=8)
+    inp["x"][0, 300, 3, 5] = float("inf")
+    inp["Cm"][0, 700, 2, 11] = float("-inf")
+    kw = dict(chunk=cfg.chunk, seg=cfg.seg)
+    ins = [inp[k] for k in ("x", "dt", "A", "Bm", "Cm", "D", "h0")]
+    y, hf = libssd.ssd_fwd(*ins, **kw)
+    ys, hs = libssd.ssd_fwd_static_ws(*ins, y=torch.empty_like(y), h_final=torch.empty_like(hf), **kw)
+    assert torch.isinf(y).any() and same(y, ys) and same(hf, hs)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("up", [-112, -118])
+def test_values_below_the_exact_range_miss_only_bf16s_smallest_number(up):
+    """x and h0 scaled to where their last bits lie below 2^-133: y is off by no more than what all its operands of that size miss."""
+    cfg = config("fp32", 512, 3, 128, 1, 128, 256)
+    inp = make_inputs(cfg, "cuda", seed=5)
+    base, s = pu.run_gpu(cfg, inp, want=("fwd",)), 2.0 ** up
+    got = pu.run_gpu(cfg, dict(inp, x=inp["x"] * s, h0=inp["h0"] * s), want=("fwd",))
+    B, C, dt = (inp[k].double() for k in ("Bm", "Cm", "dt"))
+    B, C, dt, Q = B[0, :, 0].abs(), C[0, :, 0].abs(), dt[0], cfg.chunk
+    # every operand of that size misses less than 2^-133: x in the masked products of a chunk, the weighted x in the sums of all chunks
+    # before, the state in C H
+    cb = (inp["Cm"][0, :, 0].double() @ inp["Bm"][0, :, 0].double().T).abs()
+    rows = max((cb[c:c + Q, c:c + Q] @ dt[c:c + Q]).max().item() for c in range(0, cfg.L, Q))
+    states = (C @ (1 + B.sum(0))).max().item()
+    bound = 2.0 ** -133 * (rows + states) + 2.0 ** -23 * base["y"].abs().max().item() * s
+    off = (got["y"].double() - base["y"].double() * s).abs().max().item()
+    assert off <= bound, (off, bound)
