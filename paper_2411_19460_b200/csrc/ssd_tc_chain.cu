@@ -89,10 +89,11 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
     }
     uint64_t *const full = reinterpret_cast<uint64_t *>(smem + OFF_BAR), *const scaled = full + CH_STAGES, *const empty = scaled + CH_STAGES;
     uint64_t *const mdone = empty + CH_STAGES, *const dempty = mdone + 2, *const vfull = dempty + 2, *const vempty = vfull + HEADS * CH_VEC;
-    uint32_t *const words = reinterpret_cast<uint32_t *>(vempty + HEADS * CH_VEC);
+    uint64_t *const vfirst = vempty + HEADS * CH_VEC;        // CHAIN_FWD: the first record is made; completed once and never again
+    uint32_t *const words = reinterpret_cast<uint32_t *>(vfirst + 1);
     // CHAIN_BWD has no vector buffers; in their barriers' place: H_in C made, read; the stage's rows read for rho2
     uint64_t *const ydone = vfull, *const yempty = vfull + 2, *const rowread = vempty;
-    static_assert((3 * CH_STAGES + 4 + 2 * HEADS * CH_VEC) * 8 + 8 <= 256, "barriers");
+    static_assert((3 * CH_STAGES + 5 + 2 * HEADS * CH_VEC) * 8 + 8 <= 256, "barriers");
 
     const int h0 = blockIdx.x * HEADS, b = blockIdx.y, g = h0 / p.hpg, nc = p.nc;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -112,6 +113,7 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
             mbar_init(&vfull[i], BWD && i >= 2 ? 4 : 1);
             mbar_init(&vempty[i], BWD ? 4 : 8);    // the carry warps, which read the decay last
         }
+        mbar_init(vfirst, 1);
         words[1] = 0;
         fence_barrier_init();
     }
@@ -141,9 +143,10 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
             const int ahead = nc < CH_STAGES ? nc : CH_STAGES;
             // The first step sizes would arrive behind all the stages of all CTAs (15.7 MB with 80 heads: the first block scaled 9100 cycles
             // after the start, now 7000) and everything waits for them: the later stages wait for the first record instead.  Forward
-            // of one segment, 80 heads: 4096 steps 68.8 -> 67.5 us, 16384 in 8 groups 226 -> 218; 24 heads the same.
+            // of one segment, 80 heads: 4096 steps 68.8 -> 67.5 us, 16384 in 8 groups 226 -> 218; 24 heads the same.  (Not vfull[0]: nothing
+            // holds its next phase back until this thread has looked, and the one after that needs blocks that this thread loads.)
             for (int i = 0; i < ahead; ++i) {
-                if (!BWD && i == 1) mbar_wait(vfull, 0, abortp, p.status);
+                if (!BWD && i == 1) mbar_wait(vfirst, 0, abortp, p.status);
                 load_inputs(i);
             }
             if (BWD) pdl_wait();                   // the records and states of the forward chain
@@ -270,7 +273,10 @@ k_chain_tc(SegParams p, const float *init, long long init_bs, float *bnd_out, lo
                     put_scales(v, ob);
                 if (lane == 0) v[DECAY_AT] = decay;
                 __syncwarp();
-                if (lane == 0) mbar_arrive(&vfull[vbar]);
+                if (lane == 0) {
+                    mbar_arrive(&vfull[vbar]);
+                    if (i == 0 && hl == 0) mbar_arrive(vfirst);
+                }
                 if (i == first) pdl_wait();        // the earlier kernels have read what this copy of the records held
                 const float lo = __shfl_sync(0xffffffffu, cs[3], lane | 7), hi = __shfl_sync(0xffffffffu, cs[0], lane & ~7);
                 const float bi = __shfl_sync(0xffffffffu, cs[0], ((lane >> 2) & 3) * 8), bj = __shfl_sync(0xffffffffu, cs[3], (lane & 3) * 8 + 7);
