@@ -904,8 +904,9 @@ template <typename T, int NS, bool READER, bool AGAIN> __device__ __forceinline_
 //   inter dC, tile tt : sum_h e^{cs_t} dy_t H_in (and rho2 per head);  inter dB, tile ts : sum_h dt_s e^{cs_last-cs_s} x_s Gout
 // A row of tile r has dC slots for ts <= r and dB slots for tt >= r, so the two share Q/64 + 3 slots per head range: dC by ts, dB by
 // tt + 1, then the inter-chunk terms of both.
-// Three CTAs per SM only for bf16 with N = 64 and state passes (2 x 8192 steps of 32 heads: two 0.6 % slower); elsewhere 80 registers spill too
-// much (4096 steps of 24 heads, N = 128, chunks of 64: 612 us at three, 521 at two; N = 64, states made in their readers, 385 and 352).
+// Two CTAs per SM: at three, 80 registers spill too much (bf16, 4096 steps of 24 heads, N = 128, chunks of 64, forward + backward: 612 us at three,
+// 521 at two; N = 64, states made in their readers, 385 and 352; with state passes, the backward: 2 x 8192 steps of 32 heads 758 and 750, 16384 of
+// 24, chunks of 256, 682 and 670, 4 x 8192 of 32 1528 and 1503; at most 0.5 % the other way, 16384 of 24, chunks of 128).
 template <typename T, int NS, bool READER, bool AGAIN>
 __device__ __forceinline__ bool simt_bwd(const SegParams &p, int n_dx, const StatePass &pass, int n_pass) {
     SimtSmem<T> &sm = simt_smem<T>();
@@ -923,7 +924,7 @@ __device__ __forceinline__ bool simt_bwd(const SegParams &p, int n_dx, const Sta
     return simt_row_tile<T, NS, true, true, READER, AGAIN>(p, sm, c, rt, h, b);
 }
 template <typename T, int NS, bool READER>
-__global__ void __launch_bounds__(256, SplitParts<T>::n == 1 && NS == 64 && !READER ? 3 : 2)
+__global__ void __launch_bounds__(256, 2)
 k_simt_bwd(const __grid_constant__ SegParams p, int n_dx, const __grid_constant__ StatePass pass, int n_pass) {
     pdl_launch_dependents();
     if (simt_bwd<T, NS, READER, false>(p, n_dx, pass, n_pass)) simt_bwd<T, NS, READER, true>(p, n_dx, pass, n_pass);
