@@ -191,9 +191,12 @@ __global__ void __launch_bounds__(CV_RING_THREADS) k_conv_fwd(const T *u, long l
 // Neither arithmetic nor memory bounds a call of 4096 tokens (5376 channels: 20 us of bytes; issue 42 %, FMA 36 %, MUFU 28 %, DRAM 30 % with
 // ranges of ten stages) but the start and end of a range, which loads cover only in part.
 // Long ranges (64 tokens and more) take three CTAs per SM with four stages in place of four with three: the longer range covers its start
-// and end better (eight segments of 4096 tokens, forward + backward: 515 -> 490 us, of which the
-// sums after 64 tokens cost 14; five CTAs with two stages 762, two waves of shorter
-// ranges 520).  The fp32 sums of dw and dbias end after 64 tokens, whatever the range.
+// and end better (eight segments of 4096 tokens, forward + backward: 515 -> 490 us, of which the sums after 64 tokens cost 14; five CTAs with
+// two stages 762, two waves of shorter ranges 520).  The fp32 sums of dw and dbias end after 64 tokens, whatever the range.
+// A call's backward, us, with four CTAs and with three, by the range that four have (fp32: 131 KB of ring, so one CTA on an SM; it counts as three):
+//   5376 channels, tokens      2048 (40)   4096 (80)   8192 (160)   16384 (312)   32768 (624)     1792 channels: 8192 (56)   16384 (112)
+//     bf16                      29  28      49  45      78  72       135 123       252 226                      37  36        62  58
+//     fp32                      41  41      64  62      105 102      192 183       370 351                      50  53        80  79
 constexpr int CV_SUM_STAGES = 8, CV_LONG = CV_SUM_STAGES * CV_STG_TOK;
 
 template <typename T, int CV_STAGES, int CTAS>
@@ -487,11 +490,9 @@ cudaError_t conv_bwd_t(const T *u, long long u_bs, const float *w, const float *
     };
     constexpr int row = 2 * CV_STG_TOK * 512 * (int)sizeof(T);
     const int RL = conv_range_len(B, L, C, 4, 32);
-    if constexpr (sizeof(T) == 2) {
-        if (RL >= CV_LONG) {
-            const cudaError_t e = allow_smem<k_conv_bwd<T, 4, 3>>(4 * row);
-            return e != cudaSuccess ? e : launch(k_conv_bwd<T, 4, 3>, 4, conv_range_len(B, L, C, 3, 32));
-        }
+    if (RL >= CV_LONG) {
+        const cudaError_t e = allow_smem<k_conv_bwd<T, 4, 3>>(4 * row);
+        return e != cudaSuccess ? e : launch(k_conv_bwd<T, 4, 3>, 4, conv_range_len(B, L, C, 3, 32));
     }
     const cudaError_t e = allow_smem<k_conv_bwd<T, 3, 4>>(3 * row);
     return e != cudaSuccess ? e : launch(k_conv_bwd<T, 3, 4>, 3, RL);
