@@ -163,7 +163,9 @@ k_scan_tc(SegParams p, const __grid_constant__ CUtensorMap tmRow, const __grid_c
     // The load of pass `use` over a slot is complete.  A role that takes alternate heads does not see every pass: with nothing but the
     // parity it would take a load two passes back for this one while the one between is still on its way.  So it first waits until
     // the slot has been given back for this pass, as the producer did; that wait cannot be two passes early, since the head that the
-    // role had before this one was loaded after the pass before that had been given back.
+    // role had before this one was loaded after the pass before that had been given back: it was at most three turns ago, because heads
+    // per group are even, so that only a CTA's first and last run can be of one head and no two columns operands lie between a role's heads.
+    static_assert(NV >= 3 && NST >= 3 && SC_XR >= 2, "a role's turn before the last use of a slot");
     auto wait_full = [&](int slot, uint32_t use) {
         if (use) mbar_wait(&empty[slot], (use - 1) & 1, abortp, p.status);
         mbar_wait(&full[slot], use & 1, abortp, p.status);
