@@ -1095,17 +1095,26 @@ k_simt_tail(const __grid_constant__ SegParams p, const __grid_constant__ SegPara
     SimtSmem<T> &sm = simt_smem<T>();
     pdl_launch_dependents();
     const int id = (int)blockIdx.x - n_next;
-    // The finishing steps first in the code: behind the two bodies of the sums their loads came out one after the other (bf16, N = 64, 7936
-    // steps of 8 heads in 8 groups: 36 us a launch, 26 without the second body; the backward 355 -> 348 us, 16384 steps of 24 heads 670 -> 640)
-    if (id >= 0) {
+    // bf16: the finishing steps first in the code.  Behind the two bodies of the sums they took longer (N = 64, 7936 steps of 8 heads in 8 groups:
+    // 36 us a launch, 26 without the second body; the backward 355 -> 347 us, 16384 steps of 24 heads 670 -> 640).  fp32, whose second body is
+    // a function, has them last (2 x 4096 steps of 24 heads 443 -> 440, 1024 of 4, forward + backward, 106.2 -> 105.5).
+    auto finish = [&]() {
         pdl_wait();
         if (id < nfin) bwd_finish<false>(p, reinterpret_cast<float *>(sm.t), id);
         else reduce_dbdc<T, false>(p, id - nfin);
-        return;
-    }
-    if (simt_sums<T, NS, false>(nx, sm, blockIdx.x, true)) {
-        if constexpr (SplitParts<T>::n > 1) simt_sums_call<T, NS>(nx);
-        else simt_sums<T, NS, true>(nx, sm, blockIdx.x, true);
+    };
+    if constexpr (SplitParts<T>::n > 1) {
+        if (id < 0) {
+            if (simt_sums<T, NS, false>(nx, sm, blockIdx.x, true)) simt_sums_call<T, NS>(nx);
+            return;
+        }
+        finish();
+    } else {
+        if (id >= 0) {
+            finish();
+            return;
+        }
+        if (simt_sums<T, NS, false>(nx, sm, blockIdx.x, true)) simt_sums<T, NS, true>(nx, sm, blockIdx.x, true);
     }
 }
 
