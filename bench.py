@@ -36,6 +36,7 @@ METRIC = "ssd_fwd_bwd_segmented_tokens_per_s"
 HEADLINE_CONFIG = 4
 ALSO_CONFIGS = (2, 0)
 UNIT = "tokens/s"
+SPLIT_PRODUCTS = 6      # bf16 products on the tensor cores for one of fp32 operands (three parts each, without the three smallest of nine)
 
 
 # ----------------------------------------------------------------------------- analytic model
@@ -369,12 +370,11 @@ def measure_layer(args, rep, dev, cfg, full=True):
         step_roof = dict(flops_per_token=fl, bytes_per_token=by, roofline_ms=t_roof * 1e3,
                          frac=t_roof * 1e3 / ms_per_step, peaks="bf16 tensor (burst) and HBM copy, " + peaks["source"])
     else:
-        # fp32 operands go to the tensor cores as three bf16 parts (TF32 cannot hold 1e-4); the roof stays the plain FFMA rate, measured here
-        ffma = measure_ffma_tflops(dev)
-        t_roof = max(fl * tokens / (ffma * 1e12), by * tokens / (peaks["hbm_gbs"] * 1e9))
+        # fp32 operands go to the tensor cores as three bf16 parts (TF32 cannot hold 1e-4)
+        t_roof = max(fl * tokens * SPLIT_PRODUCTS / (peaks["bf16_tflops"] * 1e12), by * tokens / (peaks["hbm_gbs"] * 1e9))
         step_roof = dict(flops_per_token=fl, bytes_per_token=by, roofline_ms=t_roof * 1e3,
-                         frac=t_roof * 1e3 / ms_per_step, ffma_tflops=ffma,
-                         peaks="fp32 FFMA rate measured by an fp32 matrix product with TF32 off, and HBM copy",
+                         frac=t_roof * 1e3 / ms_per_step, products=SPLIT_PRODUCTS,
+                         peaks="bf16 tensor (burst), %d bf16 products for each fp32 one, and HBM copy, " % SPLIT_PRODUCTS + peaks["source"],
                          note="%d tokens: the roofline time is a few microseconds, below the cost of launching the "
                               "step's kernels; the configuration is launch-bound" % tokens)
     if not full:
@@ -471,12 +471,11 @@ def measure_layer(args, rep, dev, cfg, full=True):
     avg_s = dom_ms * 1e-3 / max(dom_n, 1)
     peak_kind = "HBM copy"
     if bound == "tensor" and cfg.dtype != "bf16":
-        # fp32 contractions (three bf16 parts per operand on the tensor cores) against the measured FFMA rate
-        bound = "alu"
+        # fp32 contractions: three bf16 parts per operand on the tensor cores
         achieved = fl_tok * tok_per_launch / avg_s / 1e12
-        peak = measure_ffma_tflops(dev)
+        peak = peaks["bf16_tflops"] / SPLIT_PRODUCTS
         unit = "TFLOP/s"
-        peak_kind = "fp32 FFMA (fp32 matrix product, TF32 off)"
+        peak_kind = "bf16 matmul, burst, over the %d bf16 products of an fp32 one" % SPLIT_PRODUCTS
     elif bound == "tensor":
         achieved = fl_tok * tok_per_launch / avg_s / 1e12
         peak = peaks["bf16_tflops"]        # a launch timed by itself with CUDA events: the burst figure
@@ -486,7 +485,7 @@ def measure_layer(args, rep, dev, cfg, full=True):
         achieved = by_tok * tok_per_launch / avg_s / 1e9
         peak = peaks["hbm_gbs"]
         unit = "GB/s"
-    roofline = dict(kernel=dom, bound=bound if bound in ("tensor", "alu") else "hbm", achieved=achieved, peak=peak,
+    roofline = dict(kernel=dom, bound="tensor" if bound == "tensor" else "hbm", achieved=achieved, peak=peak,
                     unit=unit, frac=achieved / peak, traffic=ncu_traffic(dom, tok_per_launch, H),
                     peak_source=peaks["source"],
                     peak_kind=peak_kind,
@@ -518,33 +517,6 @@ def measure_layer(args, rep, dev, cfg, full=True):
         "cpu_baseline": cpu,
     }
     return line
-
-
-_FFMA = {}
-
-
-def measure_ffma_tflops(dev):
-    """fp32 multiply-add rate of the CUDA cores: the best of five 4096^3 fp32 matrix products with TF32 disabled."""
-    if dev in _FFMA:
-        return _FFMA[dev]
-    old = torch.backends.cuda.matmul.allow_tf32
-    torch.backends.cuda.matmul.allow_tf32 = False
-    try:
-        n = 4096
-        a = torch.randn(n, n, device=dev)
-        b = torch.randn(n, n, device=dev)
-        best = float("inf")
-        for _ in range(6):
-            e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-            e0.record()
-            torch.matmul(a, b)
-            e1.record()
-            torch.cuda.synchronize()
-            best = min(best, e0.elapsed_time(e1))
-        _FFMA[dev] = 2.0 * n ** 3 / (best * 1e-3) / 1e12
-    finally:
-        torch.backends.cuda.matmul.allow_tf32 = old
-    return _FFMA[dev]
 
 
 # ----------------------------------------------------------------------------- the stacked configuration
