@@ -66,12 +66,13 @@ enum {
                                       score tiles themselves, instead of the one that masks them once for both (a
                                       cross-check; the same values up to the order of the fp32 head sums) */
     SSD_FLAG_SERIAL = 4            /* ssd_fwd / ssd_fwd_segmented / ssd_bwd_segmented: launch every kernel on `stream`
-                                      itself, in order.  By default the tensor-core path, when there is more than one
-                                      segment, runs a segment's state chain (chunk sums, recurrence) up to three segments
-                                      ahead of the large kernels, and the backward's dB/dC and finishing kernels beside
-                                      dx, on library-owned helper streams forked off `stream` and joined back into it
-                                      before the call's last kernel; results are the same bits.  ssd_fwd_static_ws
-                                      always runs in order on `stream` */
+                                      itself, in order.  By default the tensor-core path, with more than one segment (the
+                                      forward: with four or more), runs a segment's state chain (chunk sums, recurrence)
+                                      up to three segments ahead of the large kernels, in the forward y of every second
+                                      segment, and the backward's dB/dC and finishing kernels beside dx, on library-owned
+                                      helper streams forked off `stream`; whatever `stream` gets after the call waits for
+                                      all of them; results are the same bits.  ssd_fwd_static_ws always runs in order on
+                                      `stream` */
 };
 
 /* `op` of ssd_workspace_bytes */

@@ -15,8 +15,10 @@ namespace ssd {
 // Programmatic dependent launch: a kernel launched through launch_pdl() may be scheduled while its predecessor
 // in the stream is still running (its CTAs take the SMs the predecessor's last wave leaves idle, and set up
 // their barriers / tensor memory there); pdl_wait() returns once the predecessor has completed and its writes
-// are visible, and must precede the kernel's first global-memory access.  pdl_launch_dependents() lets the
-// successor be scheduled from this point on.
+// are visible.  It must precede every access to what is written within the call, and every store.  The caller's inputs may be read
+// ahead of it where the call's first launch is an ordinary one (`first` below): they are complete then.  Where every launch
+// is a dependent one (convolution, norm, decode, glue) it precedes the first global-memory access.
+// pdl_launch_dependents() lets the successor be scheduled from this point on.
 #ifdef __CUDACC__
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
