@@ -159,10 +159,11 @@ cudaError_t launch_state_pass_bwd(const SegParams &p, const float *init, long lo
 // cores with fp32 operands as three bf16 parts (ssd_split.cuh): three products where the other operand is bf16 as it stands, six
 // where both are fp32, one where neither is.  Operands are staged as rows, split on the way; the next stage's global loads are in
 // flight while a stage is multiplied.  With FFMA on the CUDA cores (4 x 4 outputs per thread, bound by the shared-memory reads) the
-// large kernel took 309 us (2 x 2048 steps of 32 heads, N = 64, chunk 128, bf16) and 215 us (2 x 1024 of 24, N = 128, fp32), now 143
-// and 147, y 119 and 92 us, now 49 and 56.  Bound by latency: masks, splits and addresses around each product, between barriers, at 24
-// (fp32: 16) warps per SM (of 550 TFLOP/s that mma.sync does here the tensor pipe is 25 to 45 % busy).  bf16 takes 80 registers a thread, for
-// three CTAs per SM, with some spills; fp32, with more parts in registers, takes 128 (2 x 4096 steps: 1112 us, at 80: 1260).
+// large kernel took 309 us (2 x 2048 steps of 32 heads, N = 64, chunk 128, bf16) and 215 us (2 x 1024 of 24, N = 128, fp32), now 130
+// and 134, y 119 and 92 us, now 50 and 55.  Bound by latency: masks, splits and addresses around each product, between barriers, at 24
+// (fp32: 16) warps per SM (of 550 TFLOP/s that mma.sync does here the tensor pipe is 27 to 50 % busy).  bf16 takes 80 registers a thread, for
+// three CTAs per SM, with some spills (the backward's large kernel 128, for two); fp32, with more parts in registers, takes 128 (2 x 4096
+// steps: 1112 us, at 80: 1260).
 //
 // What does not depend on the head is not done per head: C B^T is made once per group (k_simt_sums writes it, 64 x 64 causal
 // tiles), and dB / dC come from a head sum of the masked tiles, one product per CTA instead of two per head.
@@ -243,10 +244,12 @@ constexpr float kMildTile = 8.f;
 //   S_c[p,n] = sum_s exp(cs_last - cs_s) dt_s x_s[p] B_s[n]     -> Hst slot c+1   (and cs, dtT)
 //   with grads: E_c[p,n] = sum_t exp(cs_t) dy_t[p] C_t[n]       -> Gst slot c      (its CTAs make the cumsum again)
 //   the causal tiles of C B^T, where the scratch has room for them
-// Both sums of a (head, chunk) by one CTA, with one cumsum, where there are CTAs enough (2 x 8192 steps of 32 heads 1103 -> 1082 us);
-// else two, side by side.
+// Both sums of a (head, chunk) by one CTA, with one cumsum, where there are CTAs enough; else two, side by side.  Backward, us, with two and
+// with one, by the CTAs of one: 192 (bf16, N = 64, 8192 steps of 24 heads) 404 and 438, (fp32, N = 128, 4096 of 24) 441 and 429; 256 (fp32, N = 64,
+// 4096 of 8, chunks of 64) 133 and 132; 384 (fp32, 2 x 4096 of 24) 756 and 750; 512 (bf16, N = 64, 2 x 8192 of 32) 853 and 817, (fp32, 2 x 8192
+// of 8, chunks of 64) 405 and 382; 768 (bf16, N = 128, 8192 of 24) 517 and 494.
 template <int NS> __host__ __device__ __forceinline__ bool simt_sums_merged(const SegParams &p) { return p.nc * p.B * (NS / 64) * p.H >= 2 * kNumSMs; }
-template <typename T, int NS> __host__ __device__ __forceinline__ int simt_n_sums(const SegParams &p, bool grads) {
+template <int NS> __host__ __device__ __forceinline__ int simt_n_sums(const SegParams &p, bool grads) {
     const int nrt = p.Q >> 6;
     return p.nc * p.B * ((NS / 64) * p.H * (grads && !simt_sums_merged<NS>(p) ? 2 : 1) + (p.cbt ? p.G * (nrt * (nrt + 1) / 2) : 0));
 }
@@ -1097,7 +1100,7 @@ k_simt_tail(const __grid_constant__ SegParams p, const __grid_constant__ SegPara
     const int id = (int)blockIdx.x - n_next;
     // bf16: the finishing steps first in the code.  Behind the two bodies of the sums they took longer (N = 64, 7936 steps of 8 heads in 8 groups:
     // 36 us a launch, 26 without the second body; the backward 355 -> 347 us, 16384 steps of 24 heads 670 -> 640).  fp32, whose second body is
-    // a function, has them last (2 x 4096 steps of 24 heads 443 -> 440, 1024 of 4, forward + backward, 106.2 -> 105.5).
+    // a function, has them last (4096 steps of 24 heads, N = 128, 442 -> 440; 1024 of 4, forward + backward, -0.9 %).
     auto finish = [&]() {
         pdl_wait();
         if (id < nfin) bwd_finish<false>(p, reinterpret_cast<float *>(sm.t), id);
@@ -1141,16 +1144,16 @@ static cudaError_t simt_launch(const SegParams &p, const SegParams *next, const 
         case SIMT_SUMS:
         case SIMT_SUMS_GRAD: {
             const bool grads = what == SIMT_SUMS_GRAD;
-            return simt_start<k_simt_sums<T, NS>, T>(p.first, simt_n_sums<T, NS>(p, grads), st, p, grads);
+            return simt_start<k_simt_sums<T, NS>, T>(p.first, simt_n_sums<NS>(p, grads), st, p, grads);
         }
         case SIMT_Y: {
-            const int n_next = next ? simt_n_sums<T, NS>(*next, false) : 0, n = p.nc * nrt * p.H * p.B + n_next + n_pass;
+            const int n_next = next ? simt_n_sums<NS>(*next, false) : 0, n = p.nc * nrt * p.H * p.B + n_next + n_pass;
             if (!p.cbt) return simt_start<k_simt_y<T, NS, false, false>, T>(false, n, st, p, p, 0, none, 0);      // never with `next` or `pass`
             if (pass) return simt_start<k_simt_y<T, NS, true, true>, T>(false, n, st, p, next ? *next : p, n_next, *pass, n_pass);
             return simt_start<k_simt_y<T, NS, true, false>, T>(false, n, st, p, next ? *next : p, n_next, none, 0);
         }
         case SIMT_TAIL: {
-            const int nfin = tail_finish_ctas(p), n_next = simt_n_sums<T, NS>(*next, true);
+            const int nfin = tail_finish_ctas(p), n_next = simt_n_sums<NS>(*next, true);
             return simt_start<k_simt_tail<T, NS>, T>(false, n_next + nfin + tail_reduce_ctas(p), st, p, *next, n_next, nfin);
         }
         default: {

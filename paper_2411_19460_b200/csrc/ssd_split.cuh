@@ -4,7 +4,7 @@
 //   x = p0 + p1 + p2:  p0 the upper half of x's bits (no overflow near the largest values), p1 the rest rounded to nearest, so
 //   that what it leaves for p2 has either sign, p2 the rest of that, at most eight bits.
 // The sum is x exactly from 2^-110 up.  Of a smaller x it misses what lies below bf16's smallest number, less than 2^-133: values of 2^-120 are
-// held to 13 bits, those of 2^-126, the smallest normal fp32 number, to seven.
+// held to 13 bits, those of 2^-126, the smallest normal fp32 number, to seven, and what is below 2^-134 is zero (against an infinity: NaN).
 // Products p_i q_j with i + j > 2 are left out (below 2^-23 of x y each, of either sign: about 2^-25 on average).  mma.sync truncates when it
 // adds to its accumulator, a bias of half a unit in the last place per step, so for every 16 steps of the contraction the products
 // start from zero, the smallest first, and their sum is added with a rounded fp32 addition: one truncation at the size of the sum.

@@ -45,7 +45,7 @@ static bool make_map3(CUtensorMap *m, const void *ptr, uint64_t dim0, uint64_t d
 // The tensor-core kernels round decayed rows, masked tiles and states to bf16, so that a call's fp32 outputs (states, ddt, dA)
 // are within 2e-3 of the exact ones; the split-path kernels keep all of it in fp32 (1e-6).  Which bf16 calls take which is
 // therefore part of what a caller gets: N = 64, chunks below 256 and odd numbers of heads per group have fp32 intermediates.
-// On these kernels, which could run them, 2 x 8192 steps of 32 heads with N = 64 took 378 us instead of 1014 (with FFMA 2250), and
+// On these kernels, which could run them, 2 x 8192 steps of 32 heads with N = 64 took 378 us instead of 1015 (with FFMA 2250), and
 // h_final was off by 1.7e-3 instead of 9e-7, ddt by 2.1e-3 instead of 2e-7 (4096 of these steps).
 bool tc_supported(int dtype, int flags, int P, int N, int chunk, int heads_per_group) {
     return dtype == SSD_DTYPE_BF16 && !(flags & SSD_FLAG_FORCE_SIMT) && P == 64 && N == kTcState && chunk == 2 * kTcBlock &&

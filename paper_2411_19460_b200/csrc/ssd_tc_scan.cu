@@ -36,7 +36,7 @@
 // a head's hand-overs (168 MB in 30 us; issue 43 % of the slots, shared memory 188 KB a head of 385 KB in that time).  28 warps of 72
 // registers spill (76 bytes stored in y, 152 in dx).  Beside the chain, dB/dC and the next segment, which hold the other SMs, what
 // counts is the time per head; split rings took the forward of 9472 x 3 steps of 64 heads from 279 to 273 us and 131072 steps of 80 heads,
-// forward and backward, from 6.15 to 6.05 ms.
+// forward and backward, from 6.15 to 6.05 ms (plain calls, both sides in turn on one machine; others are up to 8 % slower).
 #include "ssd_internal.h"
 #include "ssd_sm100.cuh"
 
