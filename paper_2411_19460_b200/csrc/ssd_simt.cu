@@ -1098,27 +1098,36 @@ k_simt_tail(const __grid_constant__ SegParams p, const __grid_constant__ SegPara
     SimtSmem<T> &sm = simt_smem<T>();
     pdl_launch_dependents();
     const int id = (int)blockIdx.x - n_next;
-    // bf16: the finishing steps first in the code.  Behind the two bodies of the sums they took longer (N = 64, 7936 steps of 8 heads in 8 groups:
-    // 36 us a launch, 26 without the second body; the backward 355 -> 347 us, 16384 steps of 24 heads 670 -> 640).  fp32, whose second body is
-    // a function, has them last (4096 steps of 24 heads, N = 128, 442 -> 440; 1024 of 4, forward + backward, -0.9 %).
-    auto finish = [&]() {
+    if (id < 0) {
+        if (simt_sums<T, NS, false>(nx, sm, blockIdx.x, true)) {
+            if constexpr (SplitParts<T>::n > 1) simt_sums_call<T, NS>(nx);
+            else simt_sums<T, NS, true>(nx, sm, blockIdx.x, true);
+        }
+        return;
+    }
+    pdl_wait();
+    if (id < nfin) bwd_finish<false>(p, reinterpret_cast<float *>(sm.t), id);
+    else reduce_dbdc<T, false>(p, id - nfin);
+}
+// The same with the finishing steps first in the code, for bf16 with N = 64 and chunks of 128 and 256: behind the two bodies of the sums, which
+// leave the registers short, they take longer (36 us a launch of 7936 steps of 8 heads in 8 groups, 26 behind one body), and ahead of them
+// the sums do, the larger part where chunks are short.  Backward, us, finishing steps first and last: chunks of 256 (16384 steps of 24 heads) 638
+// and 671, (8192 of 32) 484 and 500, (7936 of 8 in 8 groups) 347 and 354; of 128 (16384 of 24) 656 and 678; of 64 (8192 of 32 in 4 groups) 474 and
+// 449, (11456 of 24 in 8) 580 and 562.  N = 128: chunks of 128 (16384 of 24 in 4 groups) 980 and 988, (of 32) 1147 and 1142, of 64 (5632 of 32) 500
+// and 487.  fp32, where the second body is a function: 442 and 440 (4096 of 24, N = 128).
+template <typename T, int NS>
+__global__ void __launch_bounds__(256, SimtSmem<T>::CTAS)
+k_simt_tail_ahead(const __grid_constant__ SegParams p, const __grid_constant__ SegParams nx, int n_next, int nfin) {
+    SimtSmem<T> &sm = simt_smem<T>();
+    pdl_launch_dependents();
+    const int id = (int)blockIdx.x - n_next;
+    if (id >= 0) {
         pdl_wait();
         if (id < nfin) bwd_finish<false>(p, reinterpret_cast<float *>(sm.t), id);
         else reduce_dbdc<T, false>(p, id - nfin);
-    };
-    if constexpr (SplitParts<T>::n > 1) {
-        if (id < 0) {
-            if (simt_sums<T, NS, false>(nx, sm, blockIdx.x, true)) simt_sums_call<T, NS>(nx);
-            return;
-        }
-        finish();
-    } else {
-        if (id >= 0) {
-            finish();
-            return;
-        }
-        if (simt_sums<T, NS, false>(nx, sm, blockIdx.x, true)) simt_sums<T, NS, true>(nx, sm, blockIdx.x, true);
+        return;
     }
+    if (simt_sums<T, NS, false>(nx, sm, blockIdx.x, true)) simt_sums<T, NS, true>(nx, sm, blockIdx.x, true);
 }
 
 static int tail_finish_ctas(const SegParams &p) { return p.nc * ((p.H + FIN_HB - 1) / FIN_HB) * p.B; }
@@ -1154,7 +1163,10 @@ static cudaError_t simt_launch(const SegParams &p, const SegParams *next, const 
         }
         case SIMT_TAIL: {
             const int nfin = tail_finish_ctas(p), n_next = simt_n_sums<NS>(*next, true);
-            return simt_start<k_simt_tail<T, NS>, T>(false, n_next + nfin + tail_reduce_ctas(p), st, p, *next, n_next, nfin);
+            const int n = n_next + nfin + tail_reduce_ctas(p);
+            if constexpr (SplitParts<T>::n == 1 && NS == 64)
+                if (p.Q > 64) return simt_start<k_simt_tail_ahead<T, NS>, T>(false, n, st, p, *next, n_next, nfin);
+            return simt_start<k_simt_tail<T, NS>, T>(false, n, st, p, *next, n_next, nfin);
         }
         default: {
             const int n_dx = p.nc * nrt * p.H * p.B, n_bc = p.nc * (npair + 2 * nrt) * (p.nsl / (nrt + 3)) * p.G * p.B;
